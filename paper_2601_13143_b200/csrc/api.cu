@@ -150,8 +150,8 @@ Workspace plan_workspace(const fastav_params& p) {
   return w;
 }
 
-__global__ void status_or_kernel(int32_t* device_status, int32_t bits) {
-  pdl_trigger();
+__global__ void status_or_kernel(int32_t* device_status, int32_t bits, ChainHead head) {
+  chain_enter(head);
   pdl_wait();
   atomicOr(device_status, bits);
 }
@@ -180,7 +180,7 @@ cudaError_t launch_score(const Shapes& s, const Workspace& w, const void* q, con
     if (forced == FASTAV_SCORE_PATH_WIDE) return cudaErrorNotSupported;
     // The tensor map could not be encoded: the CUDA-core tiles below are correct but far slower, so say so.
     if (device_status) {
-      const cudaError_t es = launch_chained(status_or_kernel, dim3(1), dim3(1), 0, stream, device_status, (int32_t)FASTAV_DEV_SLOW_PATH);
+      const cudaError_t es = launch_chained(status_or_kernel, dim3(1), dim3(1), 0, stream, device_status, (int32_t)FASTAV_DEV_SLOW_PATH, ChainHead{});
       if (es != cudaSuccess) return es;
       count_launches(1);
     }

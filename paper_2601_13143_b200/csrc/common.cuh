@@ -5,6 +5,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "fastav.h"
 
 namespace fastav {
@@ -20,7 +22,11 @@ struct Shapes {
   long long q_st, q_sh, k_st, k_sh, v_st, v_sh, ko_st, ko_sh, vo_st, vo_sh;
   float scale_log2;  // softmax scale * log2(e): logits are kept in base-2 units
   unsigned flags;
+  int head_wait;     // set at launch (launch_chained): this kernel opens a call and must wait before it reads anything
 };
+
+// For the kernels that take no Shapes: the same mark.
+struct ChainHead { int head_wait = 0; };
 
 // Carved from the caller's workspace by plan_workspace(); all offsets 256-byte aligned.
 struct Workspace {
@@ -118,32 +124,6 @@ __host__ __device__ inline size_t align_up(size_t x, size_t a) { return (x + a -
 // global memory another kernel may still read.  Every block waits before it exits, so completion of a
 // kernel implies completion of all its predecessors.
 #ifdef __CUDACC__
-// Sequence b of a packed batch as the device sees it in a prefix-sum array, cut down to what the host scalars
-// promise: buffers and grids are sized from total_tokens / max_seqlen (total_q / max_qlen), loop bounds come from
-// the device array, and a caller whose two views disagree must get a status bit, not an out-of-bounds access.
-struct Span {
-  int first, count;
-  bool bad;  // the array and the host scalars disagree: the span was clamped (FASTAV_DEV_SHAPE_MISMATCH)
-};
-__device__ __forceinline__ Span checked_span(const int32_t* cu, int b, int total, int max_count) {
-  const int a = cu[b], e = cu[b + 1];
-  Span sp{a, e - a, false};
-  if (a < 0 || a > total) {
-    sp = Span{0, 0, true};
-  } else {
-    const int room = min(max_count, total - a);
-    if (sp.count < 0) { sp.count = 0; sp.bad = true; }
-    else if (sp.count > room) { sp.count = room; sp.bad = true; }
-  }
-  return sp;
-}
-__device__ __forceinline__ Span seq_span(const Shapes& s, const int32_t* cu_seqlens, int b) {
-  return checked_span(cu_seqlens, b, s.total_tokens, s.max_seqlen);
-}
-__device__ __forceinline__ Span row_span(const Shapes& s, const int32_t* cu_qlens, int b) {
-  return checked_span(cu_qlens, b, s.total_q, s.max_qlen);
-}
-
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // A pointer to data the predecessor writes must be passed through this after pdl_wait: the compiler
@@ -161,14 +141,74 @@ __device__ __forceinline__ T chain_load(const T* p) { return __ldcg(p); }
 template <typename T>
 __device__ __forceinline__ T chain_load_cached(const T* p) { return __ldca(p); }
 
-// The FIRST kernel an entry point launches takes an ordinary stream dependency: it starts only when all earlier
-// work on the stream has completed, so that the arrays the kernels read before their wait (cu_seqlens, cu_qlens,
-// q_idx, keep_counts, protect: possibly the output of the call before, e.g. its cu_keep) are final.  Every later
-// kernel of the call is launched programmatically.  Under FASTAV_CHAIN_CALLS the caller vouches for those arrays
-// and the first kernel is launched programmatically as well.  chain_begin() marks the start of a call (per host
-// thread).
+
+// Sequence b of a packed batch as the device sees it in a prefix-sum array, cut down to what the host scalars
+// promise: buffers and grids are sized from total_tokens / max_seqlen (total_q / max_qlen), loop bounds come from
+// the device array, and a caller whose two views disagree must get a status bit, not an out-of-bounds access.
+struct Span {
+  int first, count;
+  bool bad;  // the array and the host scalars disagree: the span was clamped (FASTAV_DEV_SHAPE_MISMATCH)
+};
+__device__ __forceinline__ Span checked_span(const int32_t* cu, int b, int total, int max_count) {
+  const int a = chain_load(cu + b), e = chain_load(cu + b + 1);
+  Span sp{a, e - a, false};
+  if (a < 0 || a > total) {
+    sp = Span{0, 0, true};
+  } else {
+    const int room = min(max_count, total - a);
+    if (sp.count < 0) { sp.count = 0; sp.bad = true; }
+    else if (sp.count > room) { sp.count = room; sp.bad = true; }
+  }
+  return sp;
+}
+__device__ __forceinline__ Span seq_span(const Shapes& s, const int32_t* cu_seqlens, int b) {
+  return checked_span(cu_seqlens, b, s.total_tokens, s.max_seqlen);
+}
+__device__ __forceinline__ Span row_span(const Shapes& s, const int32_t* cu_qlens, int b) {
+  return checked_span(cu_qlens, b, s.total_q, s.max_qlen);
+}
+
+// Kernels read the caller's index arrays (cu_seqlens, cu_qlens, q_idx, keep_counts, protect) before their wait, and
+// those may be what earlier work on the stream wrote (the cu_keep of the call before).  So the FIRST kernel an entry
+// point launches waits at its very first instruction and lets its successor start only after that (chain_enter):
+// whatever any kernel of the call then reads early is final.  It is launched programmatically all the same: its blocks
+// are resident when the earlier work ends, which takes the launch latency out of the call (a positional prune of 8 x
+// 2,230 tokens: 29.9 -> 26.4 us among others of its kind).  Under FASTAV_CHAIN_CALLS the caller vouches for those arrays
+// and the first kernel is like any other.  chain_begin() marks the start of a call (per host thread).  Reads ahead of a
+// kernel's own wait go through L2 (chain_load): a kernel that started while an earlier call was still running may find
+// that call's lines in its L1.
+//
+// The arrays a kernel reads after chain_enter are named in the call: the compiler may otherwise hoist a load through a
+// `const __restrict__` pointer above the wait (see pdl_acquire).
+template <typename P>
+__device__ __forceinline__ void chain_acquire_one(P& p) { pdl_acquire(p); }
+template <typename Head, typename... P>
+__device__ __forceinline__ void chain_enter(const Head& head, P&... arrays) {
+  if (head.head_wait) pdl_wait();
+  (chain_acquire_one(arrays), ...);
+  pdl_trigger();
+}
 inline thread_local bool g_chain_head = true;
 inline void chain_begin(uint32_t flags) { g_chain_head = (flags & FASTAV_CHAIN_CALLS) == 0; }
+
+// Function attributes live in the device's context: `set` runs on the first call for each device (per call site, that is
+// per kernel) and never again.
+template <typename F>
+cudaError_t once_per_device(F set) {
+  static std::atomic<unsigned long long> done{0};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 64 && ((done.load(std::memory_order_acquire) >> dev) & 1ull)) return cudaSuccess;
+  e = set();
+  if (e == cudaSuccess && dev < 64) done.fetch_or(1ull << dev, std::memory_order_release);
+  return e;
+}
+
+template <typename T>
+inline void mark_head(T&, bool) {}
+inline void mark_head(Shapes& s, bool head) { s.head_wait = head ? 1 : 0; }
+inline void mark_head(ChainHead& h, bool head) { h.head_wait = head ? 1 : 0; }
 
 template <typename... KArgs, typename... Args>
 cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args... args) {
@@ -181,7 +221,8 @@ cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = g_chain_head ? 0 : 1;
+  cfg.numAttrs = 1;
+  (mark_head(args, g_chain_head), ...);
   g_chain_head = false;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }

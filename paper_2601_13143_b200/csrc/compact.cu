@@ -48,10 +48,11 @@ __global__ void __launch_bounds__(kThreads) compact_rows_kernel(Shapes s, RowStr
                                                                 const int32_t* __restrict__ cu_keep,
                                                                 const int32_t* __restrict__ cu_seqlens,
                                                                 int32_t* device_status) {
-  pdl_trigger();
+  chain_enter(s);
   pdl_wait();  // keep_idx and cu_keep are the previous kernel's output
   pdl_acquire(keep_idx);
   pdl_acquire(cu_keep);
+  pdl_acquire(cu_seqlens);
   // 16-byte chunks per output row: [hidden | K heads | V heads]
   const int per_head = s.dim >> 3;
   const int n_hidden = t.hidden_in ? (s.hidden >> 3) : 0;
@@ -179,7 +180,7 @@ compact_rows_bulk_kernel(Shapes s, RowStreams t, const int32_t* __restrict__ kee
                          int32_t* device_status) {
   extern __shared__ __align__(128) unsigned char bulk_smem[];
   __shared__ uint64_t full[kBulkMaxWarps][kBulkStages];
-  pdl_trigger();
+  chain_enter(s);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
   const uint32_t ring = ptx::smem_u32(bulk_smem) + (uint32_t)warp * kBulkStages * row_bytes;
   Segment seg{};
@@ -193,6 +194,7 @@ compact_rows_bulk_kernel(Shapes s, RowStreams t, const int32_t* __restrict__ kee
   pdl_wait();  // keep_idx and cu_keep are the previous kernel's output
   pdl_acquire(keep_idx);
   pdl_acquire(cu_keep);
+  pdl_acquire(cu_seqlens);
   int rows = chain_load_cached(cu_keep + s.batch);
   if (rows > s.total_keep) rows = s.total_keep;  // never write past the caller's buffers
   const int first = blockIdx.x * warps + warp, step = gridDim.x * warps;
@@ -276,7 +278,8 @@ cudaError_t launch_compact(const Shapes& s, const int32_t* keep_idx, const int32
     int warps = kBulkSmemBudget / (kBulkStages * row_bytes);
     if (warps > kBulkMaxWarps) warps = kBulkMaxWarps;
     const size_t smem = (size_t)warps * kBulkStages * row_bytes;
-    cudaError_t e = cudaFuncSetAttribute(compact_rows_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e =
+        once_per_device([] { return cudaFuncSetAttribute(compact_rows_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBulkSmemBudget); });
     if (e != cudaSuccess) return e;
     int blocks = (s.total_keep + warps - 1) / warps;
     if (blocks > kNumSMs) blocks = kNumSMs;

@@ -243,9 +243,11 @@ __global__ void __launch_bounds__(256) score_finalize_kernel(Shapes s, const int
   }
 }
 
-__global__ void __launch_bounds__(256) lse_import_kernel(int count, const float* __restrict__ lse_in, float* __restrict__ lse_ws) {
-  pdl_trigger();
+__global__ void __launch_bounds__(256) lse_import_kernel(int count, const float* __restrict__ lse_in, float* __restrict__ lse_ws,
+                                                         ChainHead head) {
+  chain_enter(head);
   pdl_wait();
+  pdl_acquire(lse_in);
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const float v = lse_in[i];
@@ -254,8 +256,9 @@ __global__ void __launch_bounds__(256) lse_import_kernel(int count, const float*
 
 // The way back: log2-sum-exp2 of the workspace -> natural-log log-sum-exp as attention kernels report it
 // (-inf for a row that sees no key).
-__global__ void __launch_bounds__(256) lse_export_kernel(int count, const float* __restrict__ lse_ws, float* __restrict__ lse_out) {
-  pdl_trigger();
+__global__ void __launch_bounds__(256) lse_export_kernel(int count, const float* __restrict__ lse_ws, float* __restrict__ lse_out,
+                                                         ChainHead head) {
+  chain_enter(head);
   pdl_wait();
   pdl_acquire(lse_ws);
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -273,8 +276,11 @@ cudaError_t run(const Shapes& s, const Workspace& w, const uint16_t* q, const in
   float* partial = reinterpret_cast<float*>(ws + w.partial_off);
   const size_t smem = sizeof(TileShared<DIM>);
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(score_tile_stats_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(score_tile_accumulate_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+  e = once_per_device([&] {
+    const cudaError_t f = cudaFuncSetAttribute(score_tile_stats_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return f == cudaSuccess ? cudaFuncSetAttribute(score_tile_accumulate_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : f;
+  });
+  if (e != cudaSuccess) return e;
   if (s.total_q > 0 && s.max_seqlen > 0) {
     const dim3 grid(w.stat_tiles, s.hkv, s.batch);
     if (lse_in) {
@@ -303,14 +309,14 @@ cudaError_t launch_lse_import(const Shapes& s, const float* lse_in, float* lse_w
   const int count = s.total_q * s.hq;
   if (count <= 0) return cudaSuccess;
   count_launches(1);
-  return launch_chained(lse_import_kernel, dim3((count + 255) / 256), dim3(256), 0, stream, count, lse_in, lse_ws);
+  return launch_chained(lse_import_kernel, dim3((count + 255) / 256), dim3(256), 0, stream, count, lse_in, lse_ws, ChainHead{});
 }
 
 cudaError_t launch_lse_export(const Shapes& s, const float* lse_ws, float* lse_out, cudaStream_t stream) {
   const int count = s.total_q * s.hq;
   if (count <= 0) return cudaSuccess;
   count_launches(1);
-  return launch_chained(lse_export_kernel, dim3((count + 255) / 256), dim3(256), 0, stream, count, lse_ws, lse_out);
+  return launch_chained(lse_export_kernel, dim3((count + 255) / 256), dim3(256), 0, stream, count, lse_ws, lse_out, ChainHead{});
 }
 
 cudaError_t launch_score_generic(const Shapes& s, const Workspace& w, const void* q, const int32_t* q_idx,

@@ -55,7 +55,7 @@ score_narrow_logits_kernel(Shapes s, const uint16_t* __restrict__ q, const int32
   __shared__ uint64_t full[kStages], empty[kStages];
   __shared__ int abort_flag;
 
-  pdl_trigger();
+  chain_enter(s, cu_seqlens, cu_qlens, q_idx);
   const int warp = threadIdx.x >> 5;
   const int row_bytes = heads_per_block * DIM * 2;  // bytes of one token in a slot
   const int slot_bytes = kSlotKeys * row_bytes;
@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(256) score_narrow_stats_kernel(Shapes s, const
                                                                  const float* __restrict__ logits, int rq,
                                                                  float* __restrict__ lse) {
   __shared__ float red[8];
-  pdl_trigger();
+  chain_enter(s, cu_qlens, cu_seqlens);
   // the caller's arrays first: these loads overlap the predecessor's tail
   const int b = blockIdx.y, head = blockIdx.x / rq, r = blockIdx.x % rq;
   const Span seq = seq_span(s, cu_seqlens, b), qrows = row_span(s, cu_qlens, b);
@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(kFinalizeThreads) score_narrow_finalize_kernel
                                                                                  const float* __restrict__ lse,
                                                                                  float* __restrict__ scores) {
   extern __shared__ float lse_sh[];  // [Hq][rows], then the term offsets
-  pdl_trigger();
+  chain_enter(s, cu_qlens, cu_seqlens);
   // the caller's arrays first: these loads overlap the predecessor's tail
   const int b = blockIdx.y;
   const Span seq = seq_span(s, cu_seqlens, b), qrows = row_span(s, cu_qlens, b);

@@ -71,6 +71,7 @@ struct Unit {
   int new_q;           // the query tile differs from the previous unit's
 };
 
+constexpr int kKeptSpans = 64;
 struct Control {
   uint64_t full_k[kStages], empty_k[kStages];
   uint64_t q_ready, q_free;
@@ -85,18 +86,22 @@ struct Control {
   alignas(16) float neg_lse[4 * kGroups][64];  // sweep 2, per softmax warp: -lse of its query-row columns (-inf: padding)
   alignas(16) int limit[4 * kGroups][64];      // sweep 2, per softmax warp: last key each column's row may see
   float sums[2][kGroups - 1][kTileKeys];       // sweep 2: per accumulator, the partial sums of warpgroups 1-3
+  Span seqs[kKeptSpans], rows[kKeptSpans];     // of the first sequences: describing a unit needs them again
   Unit units[kMaxUnits];
 };
 static_assert(sizeof(Control) <= kCtrlBytes, "control block must fit its slot");
 
 // Number of work units of sequence b: KV heads x query-row chunks x key chunks (0 for an empty sequence
 // or one without scored rows).
-__device__ __forceinline__ int units_of_sequence(const Shapes& s, const int32_t* cu_seqlens, const int32_t* cu_qlens, int b,
-                                                 int rows_per_chunk, int chunk_keys) {
-  const int n = seq_span(s, cu_seqlens, b).count;
-  const int flat_rows = row_span(s, cu_qlens, b).count * s.group;
+__device__ __forceinline__ int units_of_spans(const Shapes& s, const Span& seq, const Span& rows, int rows_per_chunk, int chunk_keys) {
+  const int n = seq.count, flat_rows = rows.count * s.group;
   if (n <= 0 || flat_rows <= 0) return 0;
   return s.hkv * ((flat_rows + rows_per_chunk - 1) / rows_per_chunk) * ((n + chunk_keys - 1) / chunk_keys);
+}
+
+__device__ __forceinline__ int units_of_sequence(const Shapes& s, const int32_t* cu_seqlens, const int32_t* cu_qlens, int b,
+                                                 int rows_per_chunk, int chunk_keys) {
+  return units_of_spans(s, seq_span(s, cu_seqlens, b), row_span(s, cu_qlens, b), rows_per_chunk, chunk_keys);
 }
 
 // Block-wide sum of one int per thread (all threads get the result).
@@ -121,7 +126,7 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
                   float* __restrict__ logits, int rq, int32_t* device_status) {
   using L = Layout<DIM>;
   extern __shared__ unsigned char smem_raw[];
-  pdl_trigger();
+  chain_enter(s, q_idx, cu_qlens, cu_seqlens);
   const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   unsigned char* base_ptr = smem_raw + (base - ptx::smem_u32(smem_raw));
   Control& ctl = *reinterpret_cast<Control*>(base_ptr + L::kCtrlOff);
@@ -138,7 +143,14 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
   int total_units = 0, my_units = 0, my_excl = 0;
   if (table) {
     const int b = threadIdx.x;
-    my_units = b < s.batch ? units_of_sequence(s, cu_seqlens, cu_qlens, b, rows_per_chunk, chunk_keys) : 0;
+    if (b < s.batch) {
+      const Span seq = seq_span(s, cu_seqlens, b), rows = row_span(s, cu_qlens, b);
+      my_units = units_of_spans(s, seq, rows, rows_per_chunk, chunk_keys);
+      if (b < kKeptSpans) {
+        ctl.seqs[b] = seq;
+        ctl.rows[b] = rows;
+      }
+    }
     int incl = my_units;  // inclusive scan inside the warp, then across warps through shared memory
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -175,7 +187,8 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
   if (threadIdx.x == 0 && u1 - u0 > kMaxUnits && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
   // Unit `target` of the global order -> what to work on.  `b` is its sequence, `off` its index inside it.
   auto describe = [&](int b, int off, Unit& un) {
-    const Span seq = seq_span(s, cu_seqlens, b), rows = row_span(s, cu_qlens, b);
+    const bool kept = table && b < kKeptSpans;
+    const Span seq = kept ? ctl.seqs[b] : seq_span(s, cu_seqlens, b), rows = kept ? ctl.rows[b] : row_span(s, cu_qlens, b);
     if ((seq.bad || rows.bad) && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
     un.tok0 = seq.first;
     un.n = seq.count;
@@ -410,6 +423,7 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
     const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16);
     pdl_wait();  // before the first read of lse (sweep 2) and the first write of stats / partial
     pdl_acquire(lse);
+    pdl_acquire(q_idx);
 
     if constexpr (SWEEP == 1) {
       // Warpgroup (e, h) owns the rows of 128-row tile e and the keys [64 h, 64 h + 64) of every K tile:
@@ -425,7 +439,7 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
         const int f = un.rc * rows_per_chunk + e * 128 + my_lane;
         const bool row_valid = e * 128 + my_lane < un.rows_here;
         const int r = row_valid ? f / s.group : 0;
-        const int last_visible = min(un.n - 1, (causal && row_valid) ? q_idx[un.row0 + r] : INT_MAX);
+        const int last_visible = min(un.n - 1, (causal && row_valid) ? chain_load_cached(q_idx + un.row0 + r) : INT_MAX);
         float zmax = -INFINITY;
         float2 sum2 = make_float2(0.f, 0.f);
         for (int t = 0; t < tiles; ++t, ++uses) {
@@ -468,7 +482,7 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
           const int f = un.rc * rows_per_chunk + wg * 32 + lane;
           const int r = f / s.group;
           slot_of[lane] = (un.g * s.group + f % s.group) * rq + r;
-          limit[lane] = (causal && lane < my_cols) ? q_idx[un.row0 + r] : INT_MAX;
+          limit[lane] = (causal && lane < my_cols) ? chain_load_cached(q_idx + un.row0 + r) : INT_MAX;
           __syncwarp();
         }
         float* out = logits + un.tok0;
@@ -521,7 +535,7 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
             if (c < my_cols) {
               const int r = f / s.group;
               nl = -chain_load(lse + (long long)(un.row0 + r) * s.hq + un.g * s.group + f % s.group);
-              lim = causal ? q_idx[un.row0 + r] : INT_MAX;
+              lim = causal ? chain_load_cached(q_idx + un.row0 + r) : INT_MAX;
               min_limit = min(min_limit, lim);
             }
             neg_lse[c] = nl;
@@ -577,19 +591,20 @@ __global__ void __launch_bounds__(256) score_wide_merge_kernel(Shapes s, const i
                                                                const int32_t* __restrict__ cu_seqlens,
                                                                const float2* __restrict__ stats, int stat_chunks,
                                                                int chunk_keys, float* __restrict__ lse) {
-  pdl_trigger();
+  chain_enter(s, cu_qlens, cu_seqlens);
   // which sequence this warp's row belongs to: from the caller's arrays, so before the wait
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   const bool active = w < s.total_q * s.hq;
   int chunks = 0;
   if (active) {
     const int row = w / s.hq;
-    int lo = 0, hi = s.batch;
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (cu_qlens[mid] <= row) lo = mid; else hi = mid;
+    int n = 0;  // length of the row's sequence, the last one that starts at or before it: the whole warp looks
+    for (int b0 = 0; b0 < s.batch; b0 += 32) {
+      const int b = min(b0 + lane, s.batch - 1);
+      const int first = chain_load(cu_qlens + b), count = seq_span(s, cu_seqlens, b).count;
+      const unsigned not_after = __ballot_sync(0xFFFFFFFFu, b0 + lane < s.batch && first <= row);
+      if (not_after) n = __shfl_sync(0xFFFFFFFFu, count, 31 - __clz(not_after));
     }
-    const int n = seq_span(s, cu_seqlens, lo).count;
     chunks = 2 * ((n + chunk_keys - 1) / chunk_keys);  // one entry per 64-key half of every tile run
   }
   pdl_wait();
@@ -621,7 +636,7 @@ __global__ void __launch_bounds__(kFinalizeThreads) score_wide_finalize_kernel(S
                                                                                const int32_t* __restrict__ cu_qlens, int rc_max,
                                                                                int rows_per_chunk, const float* __restrict__ partial,
                                                                                float* __restrict__ scores) {
-  pdl_trigger();
+  chain_enter(s, cu_seqlens, cu_qlens);
   const int b = blockIdx.y;
   const Span seq = seq_span(s, cu_seqlens, b);
   const int tok0 = seq.first, n = seq.count;
@@ -698,7 +713,8 @@ cudaError_t run_logits(const Shapes& s, const CUtensorMap& k_map, const CUtensor
   int grid, chunk_tiles;
   plan_units(s, 1, &grid, &chunk_tiles);
   const int smem = Layout<DIM>::kTotal;
-  cudaError_t e = cudaFuncSetAttribute(score_wide_kernel<DIM, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e =
+      once_per_device([&] { return cudaFuncSetAttribute(score_wide_kernel<DIM, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
   if (e != cudaSuccess) return e;
   return launch_chained(score_wide_kernel<DIM, 0>, dim3(grid), dim3(kThreads), smem, stream, k_map, q_map, s, q_idx, cu_qlens,
                         cu_seqlens, chunk_tiles, 0, 1, wide_rows_per_chunk(s.group), (float2*)nullptr, (const float*)nullptr,
@@ -720,8 +736,11 @@ cudaError_t run(const Shapes& s, const Workspace& w, const CUtensorMap& k_map, c
   const int stat_chunks = 2 * ((s.max_seqlen + chunk_keys - 1) / chunk_keys);  // (max, sum) entries per (row, head)
   const int smem = Layout<DIM>::kTotal;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(score_wide_kernel<DIM, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(score_wide_kernel<DIM, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
+  e = once_per_device([&] {
+    const cudaError_t f = cudaFuncSetAttribute(score_wide_kernel<DIM, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    return f == cudaSuccess ? cudaFuncSetAttribute(score_wide_kernel<DIM, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) : f;
+  });
+  if (e != cudaSuccess) return e;
   if (lse_in) {
     // The caller already has log-sum-exp per (row, head) (the layer's attention kernel returns it): one sweep.
     if ((e = launch_lse_import(s, lse_in, lse, stream)) != cudaSuccess) return e;

@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(kThreads) select_topk_kernel(Shapes s, const f
   SelectShared& sh = *reinterpret_cast<SelectShared*>(smem_raw);
   unsigned* keys = kKeysInShared ? reinterpret_cast<unsigned*>(smem_raw + sizeof(SelectShared)) : nullptr;
 
-  pdl_trigger();
+  chain_enter(s, cu_seqlens, keep_counts, protect, q_idx, cu_qlens);
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const Span seq = seq_span(s, cu_seqlens, b);  // never beyond what the key storage was sized for
   const int tok0 = seq.first, n = seq.count;
@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(kThreads) select_topk_kernel(Shapes s, const f
       const Span si = seq_span(s, cu_seqlens, i);
       const int ni = si.count;
       mismatch |= si.bad;
-      int ki = keep_counts[i];
+      int ki = chain_load(keep_counts + i);
       if (ki < 0 || ki > ni) { clamped = true; ki = ki < 0 ? 0 : ni; }
       if (i < b) part += ki;
     }
@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(kThreads) select_topk_kernel(Shapes s, const f
     if (clamped && device_status) atomicOr(device_status, FASTAV_DEV_K_CLAMPED);
     if (mismatch && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
   }
-  int k = selecting ? keep_counts[b] : 0;
+  int k = selecting ? chain_load(keep_counts + b) : 0;
   k = k < 0 ? 0 : (k > n ? n : k);
 
   pdl_wait();  // the scores (or logits) are the previous kernel's output
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(kThreads) select_topk_kernel(Shapes s, const f
       fl.scores_out[tok0 + j] = score;
       unsigned key = order_key(lowest ? -score : score);
       if (key == kProtectedKey) key = kProtectedKey - 1;
-      if (protect && protect[tok0 + j]) key = kProtectedKey;
+      if (protect && chain_load(protect + tok0 + j)) key = kProtectedKey;
       keys[slot<kKeysInShared>(j)] = key;
     }
     if (!selecting) return;  // uniform for the block
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kThreads) select_topk_kernel(Shapes s, const f
       if (j < n) {
         unsigned key = order_key(lowest ? -v[u] : v[u]);
         if (key == kProtectedKey) key = kProtectedKey - 1;  // only a NaN pattern lands here
-        if (protect && protect[tok0 + j]) key = kProtectedKey;
+        if (protect && chain_load(protect + tok0 + j)) key = kProtectedKey;
         keys[slot<kKeysInShared>(j)] = key;
       }
     }
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(kThreads) select_topk_kernel(Shapes s, const f
   if (s.flags & FASTAV_PROTECT_QUERY_ROWS) {
     const Span rows = checked_span(cu_qlens, b, s.total_q, s.total_q);
     for (int r = rows.first + tid; r < rows.first + rows.count; r += kThreads) {
-      const int j = q_idx[r];
+      const int j = chain_load(q_idx + r);
       if (j >= 0 && j < n) keys[slot<kKeysInShared>(j)] = kProtectedKey;
     }
     __syncthreads();
@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(kThreads) select_topk_blocked_kernel(Shapes s,
   extern __shared__ __align__(16) unsigned char smem_raw[];
   BlockedShared& shared = *reinterpret_cast<BlockedShared*>(smem_raw);
   float* stage = reinterpret_cast<float*>(smem_raw + sizeof(BlockedShared));
-  pdl_trigger();
+  chain_enter(s, cu_seqlens, keep_counts, protect, q_idx, cu_qlens);
   select_sequence_blocked<kThreads, PER, kDigitBits>(
       shared, stage, s, blockIdx.x, threadIdx.x, scores, cu_seqlens, keep_counts, protect, q_idx, cu_qlens, keep_idx, cu_keep,
       device_status, [] { __syncthreads(); }, [] { pdl_wait(); /* the scores are the previous kernel's output */ });
@@ -404,7 +404,8 @@ cudaError_t launch_blocked(const Shapes& s, const float* scores, const int32_t* 
                            const uint8_t* protect, const int32_t* q_idx, const int32_t* cu_qlens, int32_t* keep_idx, int32_t* cu_keep,
                            int32_t* device_status, cudaStream_t stream) {
   const size_t smem = sizeof(BlockedShared) + ((size_t)s.max_seqlen + s.max_seqlen / 32 + 1) * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(select_topk_blocked_kernel<PER>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 1024);
+  cudaError_t e = once_per_device(
+      [] { return cudaFuncSetAttribute(select_topk_blocked_kernel<PER>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 1024); });
   if (e != cudaSuccess) return e;
   return launch_chained(select_topk_blocked_kernel<PER>, dim3(s.batch), dim3(kThreads), smem, stream, s, scores, cu_seqlens,
                         keep_counts, protect, q_idx, cu_qlens, keep_idx, cu_keep, device_status);
@@ -427,7 +428,7 @@ cudaError_t launch_select(const Shapes& s, const Workspace& w, const float* scor
     else if (s.max_seqlen <= kThreads * 16) e = launch_blocked<16>(s, scores, cu_seqlens, keep_counts, protect, q_idx, cu_qlens, keep_idx, cu_keep, device_status, stream);
     else e = launch_blocked<32>(s, scores, cu_seqlens, keep_counts, protect, q_idx, cu_qlens, keep_idx, cu_keep, device_status, stream);
   } else if (want <= kMaxDynamic) {
-    e = cudaFuncSetAttribute(select_topk_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamic);
+    e = once_per_device([] { return cudaFuncSetAttribute(select_topk_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamic); });
     if (e != cudaSuccess) return e;
     e = launch_chained(select_topk_kernel<true, false>, dim3(s.batch), dim3(kThreads), want, stream, s, scores, cu_seqlens,
                        keep_counts, protect, q_idx, cu_qlens, keep_idx, cu_keep, (unsigned*)nullptr, device_status, FromLogits{});
@@ -455,7 +456,8 @@ cudaError_t launch_narrow_tail(const Shapes& s, const float* logits, int rq, flo
                                int32_t* device_status, cudaStream_t stream) {
   const size_t smem = sizeof(SelectShared) + ((size_t)s.max_seqlen + s.max_seqlen / 32 + 1) * sizeof(unsigned) +
                       (size_t)s.hq * rq * (sizeof(float) + sizeof(int));  // keys, log-sum-exp per term, term offsets
-  cudaError_t e = cudaFuncSetAttribute(select_topk_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  cudaError_t e =
+      once_per_device([] { return cudaFuncSetAttribute(select_topk_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024); });
   if (e != cudaSuccess) return e;
   e = launch_chained(select_topk_kernel<true, true>, dim3(s.batch), dim3(kThreads), smem, stream, s, (const float*)nullptr,
                      cu_seqlens, keep_counts, protect, q_idx, cu_qlens, keep_idx, cu_keep, (unsigned*)nullptr, device_status,
@@ -471,7 +473,7 @@ namespace {
 __global__ void __launch_bounds__(256) mask_count_kernel(Shapes s, const uint8_t* __restrict__ keep_mask,
                                                          const int32_t* __restrict__ cu_seqlens, int32_t* __restrict__ counts) {
   __shared__ int warp_sums[8];
-  pdl_trigger();
+  chain_enter(s, cu_seqlens);
   pdl_wait();
   pdl_acquire(keep_mask);
   const int b = blockIdx.x;
@@ -496,7 +498,7 @@ __global__ void __launch_bounds__(kThreads) mask_emit_kernel(Shapes s, const uin
                                                              int32_t* __restrict__ cu_keep, int32_t* device_status) {
   __shared__ unsigned warp_a[kWarps];
   __shared__ int base_sh;
-  pdl_trigger();
+  chain_enter(s, cu_seqlens);
   pdl_wait();
   pdl_acquire(counts);
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;

@@ -73,7 +73,7 @@ __device__ __forceinline__ void select_sequence_blocked(SelectBlockedShared<THRE
       const Span si = seq_span(s, cu_seqlens, i);
       const int ni = si.count;
       mismatch |= si.bad;
-      int ki = keep_counts[i];
+      int ki = chain_load(keep_counts + i);
       if (ki < 0 || ki > ni) { clamped = true; ki = ki < 0 ? 0 : ni; }
       if (i < b) part += ki;
     }
@@ -84,11 +84,11 @@ __device__ __forceinline__ void select_sequence_blocked(SelectBlockedShared<THRE
   if (by_rows) {
     const Span rows = checked_span(cu_qlens, b, s.total_q, s.total_q);
     for (int r = rows.first + tid; r < rows.first + rows.count; r += THREADS) {
-      const int j = q_idx[r];
+      const int j = chain_load(q_idx + r);
       if (j >= 0 && j < n) atomicOr(&sh.prot_bits[j >> 5], 1u << (j & 31));
     }
   }
-  int k = keep_counts[b];
+  int k = chain_load(keep_counts + b);
   k = k < 0 ? 0 : (k > n ? n : k);
   scores_ready();
   pdl_acquire(scores);
@@ -109,7 +109,7 @@ __device__ __forceinline__ void select_sequence_blocked(SelectBlockedShared<THRE
   if (protect) {
     for (int j0 = warp * 32; j0 < n; j0 += THREADS) {  // a warp covers tokens j0 .. j0 + 31: one word
       const int j = j0 + lane;
-      const unsigned word = __ballot_sync(0xFFFFFFFFu, j < n && protect[tok0 + j] != 0);
+      const unsigned word = __ballot_sync(0xFFFFFFFFu, j < n && chain_load(protect + tok0 + j) != 0);
       if (lane == 0 && word) atomicOr(&sh.prot_bits[j0 >> 5], word);
     }
   }
