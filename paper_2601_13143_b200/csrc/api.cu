@@ -6,6 +6,7 @@
 #include <cstring>
 
 #include "common.cuh"
+#include "gather.cuh"
 
 namespace fastav {
 namespace {
@@ -168,11 +169,11 @@ bool score_path_ok(const Shapes& s) {
 // CUDA-core tiles take whatever is left (and whatever the TMA descriptor cannot express).
 cudaError_t launch_score(const Shapes& s, const Workspace& w, const void* q, const int32_t* q_idx,
                          const int32_t* cu_qlens, const void* k, const int32_t* cu_seqlens, const float* lse_in,
-                         float* scores_out, unsigned char* ws, int32_t* device_status, cudaStream_t stream) {
+                         float* scores_out, unsigned char* ws, int32_t* device_status, cudaStream_t stream, ScoreLeft* left) {
   const unsigned forced = s.flags & FASTAV_SCORE_PATH_MASK;
   if (forced == FASTAV_SCORE_PATH_GENERIC) return launch_score_generic(s, w, q, q_idx, cu_qlens, k, cu_seqlens, lse_in, scores_out, ws, stream);
   if (score_narrow_applies(s) && (forced == 0 || forced == FASTAV_SCORE_PATH_NARROW))
-    return launch_score_narrow(s, w, q, q_idx, cu_qlens, k, cu_seqlens, lse_in, scores_out, ws, device_status, stream);
+    return launch_score_narrow(s, w, q, q_idx, cu_qlens, k, cu_seqlens, lse_in, scores_out, ws, device_status, stream, left);
   if (score_wide_applies(s)) {
     bool used = false;
     const cudaError_t e = launch_score_wide(s, w, q, q_idx, cu_qlens, k, cu_seqlens, lse_in, scores_out, ws, device_status, stream, &used);
@@ -322,21 +323,23 @@ int32_t fastav_prune(const fastav_params* params, const void* q, const int32_t* 
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e = cudaSuccess;
-  const unsigned forced = s.flags & FASTAV_SCORE_PATH_MASK;
-  if (params->total_tokens > 0 && !lse_opt && score_narrow_applies(s) && narrow_tail_applies(s) &&
-      (forced == 0 || forced == FASTAV_SCORE_PATH_NARROW)) {
-    // Short sequences, few scored rows: logits, then ONE kernel for the softmax statistics, the scores and the keep list.
-    e = launch_narrow_logits(s, w, q, q_idx, cu_qlens, k, cu_seqlens, ws, device_status, st);
-    if (e == cudaSuccess)
-      e = launch_narrow_tail(s, reinterpret_cast<const float*>(ws + w.logits_off), s.max_qlen, scores_out, true, cu_seqlens,
-                             keep_counts, protect_opt, q_idx, cu_qlens, keep_idx_out, cu_keep_out, device_status, st);
-  } else {
-    if (params->total_tokens > 0) e = launch_score(s, w, q, q_idx, cu_qlens, k, cu_seqlens, lse_opt, scores_out, ws, device_status, st);
-    if (e == cudaSuccess)
+  ScoreLeft left;
+  bool gathered = false;
+  if (params->total_tokens > 0) e = launch_score(s, w, q, q_idx, cu_qlens, k, cu_seqlens, lse_opt, scores_out, ws, device_status, st, &left);
+  if (e == cudaSuccess) {
+    if (left.kind == ScoreLeft::kKeys) {
+      const RowStreams rows{static_cast<const uint16_t*>(hidden_in), static_cast<uint16_t*>(hidden_out), static_cast<const uint16_t*>(k_out ? k : nullptr),
+                            static_cast<uint16_t*>(k_out),           static_cast<const uint16_t*>(v),    static_cast<uint16_t*>(v_out),
+                            pos_in,                                  pos_out};
+      gathered = s.total_keep > 0 && few_gathers(s, row_bytes_of(s, rows));
+      e = launch_few(s, q, k, lse_opt, scores_out, true, gathered ? &rows : nullptr, cu_seqlens, keep_counts, protect_opt, q_idx, cu_qlens,
+                     keep_idx_out, cu_keep_out, device_status, st);
+    } else {
       e = launch_select(s, w, scores_out, cu_seqlens, keep_counts, protect_opt, q_idx, cu_qlens, keep_idx_out, cu_keep_out, ws,
                         device_status, st);
+    }
   }
-  if (e == cudaSuccess)
+  if (e == cudaSuccess && !gathered)
     e = launch_compact(s, keep_idx_out, cu_keep_out, cu_seqlens, hidden_in, hidden_out, pos_in, pos_out, k, k_out, v, v_out,
                        device_status, st);
   return e == cudaSuccess ? FASTAV_OK : cuda_failed(e);

@@ -28,6 +28,11 @@ struct Shapes {
 // For the kernels that take no Shapes: the same mark.
 struct ChainHead { int head_wait = 0; };
 
+// What a prune call still has to do after the scoring kernels, and from what.
+struct ScoreLeft {
+  enum Kind { kScores, kKeys } kind = kScores;  // finished scores; nothing done: the few-rows kernel starts from the keys
+};
+
 // Carved from the caller's workspace by plan_workspace(); all offsets 256-byte aligned.
 struct Workspace {
   size_t total = 0;
@@ -46,8 +51,10 @@ Workspace plan_workspace(const fastav_params& p);
 // ---- launchers (each returns cudaGetLastError() after its launches) -------------------------
 cudaError_t launch_score(const Shapes& s, const Workspace& w, const void* q, const int32_t* q_idx,
                          const int32_t* cu_qlens, const void* k, const int32_t* cu_seqlens, const float* lse_in,
-                         float* scores_out, unsigned char* ws, int32_t* device_status, cudaStream_t stream);
+                         float* scores_out, unsigned char* ws, int32_t* device_status, cudaStream_t stream, ScoreLeft* left = nullptr);
 
+// `left` (optional, everywhere below): when given, a launcher may leave work to the kernel that selects and say what;
+// without it the scores are finished.
 // `lse_in` (optional, everywhere below): the caller's natural-log log-sum-exp per (scored row, head); when
 // given, the softmax statistics are not recomputed.
 cudaError_t launch_score_generic(const Shapes& s, const Workspace& w, const void* q, const int32_t* q_idx,
@@ -65,7 +72,7 @@ constexpr int kNarrowMaxRows = 4;
 bool score_narrow_applies(const Shapes& s);
 cudaError_t launch_score_narrow(const Shapes& s, const Workspace& w, const void* q, const int32_t* q_idx,
                                 const int32_t* cu_qlens, const void* k, const int32_t* cu_seqlens, const float* lse_in,
-                                float* scores_out, unsigned char* ws, int32_t* device_status, cudaStream_t stream);
+                                float* scores_out, unsigned char* ws, int32_t* device_status, cudaStream_t stream, ScoreLeft* left);
 
 // Many scored rows per sequence: tensor-core path (tcgen05 + TMA).  `*used` is false when the TMA
 // descriptor for K could not be built; nothing was launched then and the caller takes another path.
@@ -80,12 +87,15 @@ cudaError_t launch_logits_wide(const Shapes& s, const void* q, const int32_t* q_
                                const int32_t* cu_seqlens, float* logits, int rq, int32_t* device_status, cudaStream_t stream,
                                bool* used);
 
-// Short sequences with few scored rows: one kernel turns the logits into scores and (optionally) the keep list.
-bool narrow_tail_applies(const Shapes& s);
-cudaError_t launch_narrow_tail(const Shapes& s, const float* logits, int rq, float* scores_out, bool do_select,
-                               const int32_t* cu_seqlens, const int32_t* keep_counts, const uint8_t* protect,
-                               const int32_t* q_idx, const int32_t* cu_qlens, int32_t* keep_idx, int32_t* cu_keep,
-                               int32_t* device_status, cudaStream_t stream);
+// Few scored rows on short sequences: one kernel from the keys to the keep list, or to the gathered rows (prune_few.cu).
+struct RowStreams;
+bool few_applies(const Shapes& s);
+bool few_gathers(const Shapes& s, int row_bytes);
+// `rows`: what to gather in the same kernel (nullptr: nothing).
+cudaError_t launch_few(const Shapes& s, const void* q, const void* k, const float* lse_in, float* scores_out, bool do_select,
+                       const RowStreams* rows, const int32_t* cu_seqlens, const int32_t* keep_counts, const uint8_t* protect,
+                       const int32_t* q_idx, const int32_t* cu_qlens, int32_t* keep_idx, int32_t* cu_keep, int32_t* device_status,
+                       cudaStream_t stream);
 // Only the logits [Hq, max_qlen, N] of the few-rows path, into the workspace.
 cudaError_t launch_narrow_logits(const Shapes& s, const Workspace& w, const void* q, const int32_t* q_idx,
                                  const int32_t* cu_qlens, const void* k, const int32_t* cu_seqlens, unsigned char* ws,
@@ -210,21 +220,31 @@ inline void mark_head(T&, bool) {}
 inline void mark_head(Shapes& s, bool head) { s.head_wait = head ? 1 : 0; }
 inline void mark_head(ChainHead& h, bool head) { h.head_wait = head ? 1 : 0; }
 
+// `cluster`: blocks per thread-block cluster along x (0: none).
 template <typename... KArgs, typename... Args>
-cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args... args) {
+cudaError_t launch_chained_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster, size_t smem, cudaStream_t stream,
+                                   Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 0 ? 2 : 1;
   (mark_head(args, g_chain_head), ...);
   g_chain_head = false;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args... args) {
+  return launch_chained_cluster(kernel, grid, block, 0, smem, stream, args...);
 }
 #endif
 

@@ -12,6 +12,7 @@
 // global, several rows in flight per warp and no register staging.  Rows whose segments are not
 // 16-byte friendly, or too long for the ring, take the load/store kernel below.
 #include "common.cuh"
+#include "gather.cuh"
 #include "sm100_ptx.cuh"
 
 namespace fastav {
@@ -19,30 +20,6 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kUnroll = 4;  // 16-byte loads in flight per thread
-
-__device__ __forceinline__ uint4 load_stream(const uint4* p) {
-  uint4 v;
-  // a plain (coherent) load: under programmatic launch the rows may be what the previous kernel wrote
-  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "l"(p));
-  return v;
-}
-
-__device__ __forceinline__ void store_row(uint4* p, const uint4& v) {
-  asm volatile("st.global.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
-}
-
-struct RowStreams {
-  const uint16_t* hidden_in;
-  uint16_t* hidden_out;
-  const uint16_t* k_in;
-  uint16_t* k_out;
-  const uint16_t* v_in;
-  uint16_t* v_out;
-  const int32_t* pos_in;
-  int32_t* pos_out;
-};
 
 __global__ void __launch_bounds__(kThreads) compact_rows_kernel(Shapes s, RowStreams t, const int32_t* __restrict__ keep_idx,
                                                                 const int32_t* __restrict__ cu_keep,
@@ -53,13 +30,7 @@ __global__ void __launch_bounds__(kThreads) compact_rows_kernel(Shapes s, RowStr
   pdl_acquire(keep_idx);
   pdl_acquire(cu_keep);
   pdl_acquire(cu_seqlens);
-  // 16-byte chunks per output row: [hidden | K heads | V heads]
-  const int per_head = s.dim >> 3;
-  const int n_hidden = t.hidden_in ? (s.hidden >> 3) : 0;
-  const int n_k = t.k_in ? s.hkv * per_head : 0;
-  const int n_v = t.v_in ? s.hkv * per_head : 0;
-  const int n_chunks = n_hidden + n_k + n_v;
-  const int head_shift = (s.dim == 128) ? 4 : 3;
+  const RowShape shape(s, t);
   const bool global_idx = (s.flags & FASTAV_KEEP_IDX_GLOBAL) != 0;
   int rows = chain_load_cached(cu_keep + s.batch);
   if (rows > s.total_keep) rows = s.total_keep;  // never write past the caller's buffers
@@ -78,36 +49,7 @@ __global__ void __launch_bounds__(kThreads) compact_rows_kernel(Shapes s, RowStr
     }
     if (threadIdx.x == 0 && t.pos_in) t.pos_out[dst] = t.pos_in[src];
 
-    for (int base = 0; base < n_chunks; base += kThreads * kUnroll) {
-      uint4 regs[kUnroll];
-      uint4* out_ptr[kUnroll];
-#pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
-        const int c = base + u * kThreads + threadIdx.x;
-        out_ptr[u] = nullptr;
-        if (c < n_chunks) {
-          const uint16_t* in;
-          uint16_t* out;
-          if (c < n_hidden) {
-            in = t.hidden_in + src * s.hidden + (c << 3);
-            out = t.hidden_out + dst * s.hidden + (c << 3);
-          } else if (c < n_hidden + n_k) {
-            const int cc = c - n_hidden, head = cc >> head_shift, off = (cc & (per_head - 1)) << 3;
-            in = t.k_in + src * s.k_st + head * s.k_sh + off;
-            out = t.k_out + dst * s.ko_st + head * s.ko_sh + off;
-          } else {
-            const int cc = c - n_hidden - n_k, head = cc >> head_shift, off = (cc & (per_head - 1)) << 3;
-            in = t.v_in + src * s.v_st + head * s.v_sh + off;
-            out = t.v_out + dst * s.vo_st + head * s.vo_sh + off;
-          }
-          regs[u] = load_stream(reinterpret_cast<const uint4*>(in));
-          out_ptr[u] = reinterpret_cast<uint4*>(out);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < kUnroll; ++u)
-        if (out_ptr[u]) store_row(out_ptr[u], regs[u]);
-    }
+    copy_row<kThreads, kUnroll>(s, t, shape, src, dst, threadIdx.x);
   }
 }
 
@@ -271,7 +213,7 @@ cudaError_t launch_compact(const Shapes& s, const int32_t* keep_idx, const int32
   // a row must fit a slot, and there may be at most one segment per lane.
   const bool packed_k = k_in && s.k_sh == s.dim && s.ko_sh == s.dim, packed_v = v_in && s.v_sh == s.dim && s.vo_sh == s.dim;
   const int n_segments = (hidden_in ? 1 : 0) + (k_in ? (packed_k ? 1 : s.hkv) : 0) + (v_in ? (packed_v ? 1 : s.hkv) : 0);
-  const int row_bytes = (hidden_in ? s.hidden * 2 : 0) + ((k_in ? 1 : 0) + (v_in ? 1 : 0)) * s.hkv * s.dim * 2;
+  const int row_bytes = row_bytes_of(s, t);
   const int forced = (s.flags & FASTAV_COMPACT_PATH_MASK);
   if (forced != FASTAV_COMPACT_PATH_LOADSTORE && n_segments >= 1 && n_segments <= 32 && row_bytes > 0 &&
       kBulkStages * row_bytes <= kBulkSmemBudget) {

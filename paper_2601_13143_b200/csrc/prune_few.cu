@@ -1,0 +1,540 @@
+// A prune call with few scored rows on short sequences, in ONE kernel: one thread-block CLUSTER per sequence goes from the
+// keys to the scores, the keep list and (where that is little) the survivors' rows.  This is the paper's own fine stage
+// (Section 2.2, "Fine pruning": one last-token query) on what the global stage left.
+//
+//   logits  Q K^T by mma.sync, fragments loaded straight from global memory (see KeyFragment);
+//   scores  log-sum-exp per row and head (statistics per segment, exchanged through distributed shared memory, one
+//           cluster barrier), then per token the fixed-order sum over heads and rows (Eq. 4);
+//   select  the scores as order-preserving 32-bit keys (protected tokens: the largest) go to every block of the cluster, a
+//           second cluster barrier, and each block runs the whole selection for itself: a histogram of the leading 12 bits,
+//           the keys of the bin that holds the k-th largest finished by counting ranks (further 12-bit passes only if it holds
+//           more than 256), one stable prefix sum in index order;
+//   gather  the survivors among a block's own tokens.
+//
+// Bound: latency.  Nothing here is long, so what counts is the number of dependent steps: every index array is asked for
+// at once, the keys before anything that is only needed later, every reduction is spread over as many lanes as keep its
+// order fixed, and nothing is computed by an owner that would have to publish it.  FEW_FIGURES
+//
+// A sequence's scores depend on its length only, not on the cluster's size or the batch, and equal keys get bit-equal
+// scores: all sums have a fixed order.
+#include <math.h>
+
+#include "cluster.cuh"
+#include "common.cuh"
+#include "gather.cuh"
+#include "select_keys.cuh"
+#include "sm100_ptx.cuh"
+
+namespace fastav {
+namespace {
+
+constexpr int kThreads = 512;
+constexpr int kWarps = kThreads / 32;
+constexpr int kMaxTokens = 4 * kThreads;  // four keys per thread in the selection
+constexpr int kDigitBits = 12;
+constexpr int kBins = 1 << kDigitBits;
+constexpr int kBinsPerThread = kBins / kThreads;
+constexpr int kStatLanes = 8;   // lanes that share one (segment, term) of the row statistics
+constexpr int kTokenLanes = 8;  // lanes that share one token's sum over the terms
+
+// A sequence is cut into sixteen segments whatever the size of the cluster, and a block owns 16 / blocks of them: the row
+// statistics are kept per segment and merged in a fixed tree.
+constexpr int kSegments = kMaxCluster;
+__host__ __device__ inline int segment_of(int n) { return n <= 32 * kSegments ? 32 : ((n + kSegments - 1) / kSegments + 31) & ~31; }
+
+struct FewArgs {
+  const uint16_t* q;
+  const uint16_t* k;
+  const float* lse;     // optional: the caller's natural-log log-sum-exp [total_q, Hq]
+  float* scores_out;    // [N]
+  int rq;               // most scored rows of a sequence
+  int do_select;        // 0: only the scores are wanted
+  int do_gather;
+  int slice_cap;        // tokens per block that shared memory was sized for
+  RowStreams rows;      // do_gather
+};
+
+struct alignas(16) FewShared {
+  unsigned hist[kBins];  // later: the block's survivors
+  unsigned keys[kMaxTokens];
+  unsigned prot_bits[kMaxTokens / 32];
+  unsigned list[kDirectMax];
+  int row_of[128], term_of[128];  // of a KV group's flat query row: scored row, term inside the group
+  unsigned warp_a[kWarps];
+  int limit[kNarrowMaxRows];
+  int base, list_n, remaining, bucket, need_eq, first_out, end_out, unused;
+  unsigned prefix, threshold, unused2[2];
+};
+static_assert(sizeof(FewShared) % 16 == 0 && kBins >= kMaxTokens, "what follows it stays 16-byte aligned");
+
+// Dynamic shared memory after FewShared (bytes, every piece 16-byte aligned); host and device agree on it.
+struct FewLayout {
+  unsigned q, lse, stats, z, total;
+};
+__host__ __device__ inline int z_stride_of(int slice_cap) { return slice_cap + 4; }  // + 4: fragments store free of bank conflicts
+__host__ __device__ inline FewLayout few_layout(int slice_cap, int terms, int dim) {
+  FewLayout l{};
+  unsigned at = 0;
+  l.q = at;      // the query rows, 64 bytes of padding each
+  at += (unsigned)terms * (dim * 2 + 64);
+  l.lse = at;    // [terms]
+  at += (unsigned)align_up((size_t)terms * 4, 16);
+  l.stats = at;  // float2 [segments][terms], written by all blocks
+  at += (unsigned)terms * kSegments * 8;
+  l.z = at;      // [terms][z_stride]: this block's logits
+  at += (unsigned)terms * z_stride_of(slice_cap) * 4;
+  l.total = at;
+  return l;
+}
+
+// One warp, 16 tokens of one KV head.  The contraction may run over head_dim in any order as long as both operands use
+// the same one, so a lane's fragment registers of two k-steps are ONE 16-byte piece of a row (lane t of a quad: elements
+// 32 i + 8 t ..): the loads are 64 contiguous bytes per row and instruction and nothing is staged or transposed.
+template <int DIM>
+struct KeyFragment {
+  uint4 lo[DIM / 32], hi[DIM / 32];  // tokens lane / 4 and lane / 4 + 8
+  __device__ __forceinline__ void load(const uint16_t* k, long long st, int tokens, int lane) {  // `tokens` exist from `k` on
+    const int r = lane >> 2;
+    const uint4 zero = make_uint4(0, 0, 0, 0);
+    const uint16_t* p = k + r * st + (lane & 3) * 8;
+#pragma unroll
+    for (int i = 0; i < DIM / 32; ++i) {
+      lo[i] = r < tokens ? chain_load(reinterpret_cast<const uint4*>(p + i * 32)) : zero;
+      hi[i] = r + 8 < tokens ? chain_load(reinterpret_cast<const uint4*>(p + 8 * st + i * 32)) : zero;
+    }
+  }
+};
+
+__device__ __forceinline__ void mma_16x8x16(float (&c)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0, unsigned b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+template <int DIM>
+__global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArgs a, const int32_t* __restrict__ cu_seqlens,
+                                                                const int32_t* __restrict__ keep_counts,
+                                                                const uint8_t* __restrict__ protect, const int32_t* __restrict__ q_idx,
+                                                                const int32_t* __restrict__ cu_qlens, int32_t* __restrict__ keep_idx,
+                                                                int32_t* __restrict__ cu_keep, int32_t* device_status) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  FewShared& sh = *reinterpret_cast<FewShared*>(smem_raw);
+  chain_enter(s, cu_seqlens, keep_counts, protect, q_idx, cu_qlens);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int blocks = (int)gridDim.x / s.batch;  // blocks per cluster
+  const int b = blockIdx.x / blocks, c = (int)cluster_rank();
+  cluster_arrive();  // "this block runs": waited for before the first remote access
+
+  // ---- the caller's index arrays, all asked for at once ------------------------------------------------
+  const bool selecting = a.do_select != 0;
+  int k = selecting ? chain_load(keep_counts + b) : 0;
+  const Span seq = seq_span(s, cu_seqlens, b), qrows = row_span(s, cu_qlens, b);
+  if (selecting)
+    for (int i = tid; i < kBins / 4; i += kThreads) reinterpret_cast<uint4*>(sh.hist)[i] = make_uint4(0, 0, 0, 0);
+  if (tid < kMaxTokens / 32) sh.prot_bits[tid] = 0u;
+  if (tid == 0) { sh.base = 0; sh.list_n = 0; }
+  const int tok0 = seq.first, n = min(seq.count, a.slice_cap * blocks);
+  const int seg = segment_of(n), slice = seg * (kSegments / blocks);  // tokens per segment, per block
+  const int t0 = min(n, c * slice), m = min(n - t0, slice);           // this block's tokens: [t0, t0 + m) of the sequence
+  const int all_rows = qrows.count, rows = min(all_rows, a.rq);
+  const int flat = rows * s.group;  // query rows of one KV group, f = row * G + head of the group
+  const int terms = s.hq * rows;    // term i = (head i / rows, row i % rows)
+  const bool causal = (s.flags & FASTAV_CAUSAL) != 0;
+  k = k < 0 ? 0 : (k > n ? n : k);
+
+  pdl_wait();
+  pdl_acquire(a.q);
+  pdl_acquire(a.k);
+  // ---- logits ----------------------------------------------------------------------------------------------
+  const FewLayout lay = few_layout(a.slice_cap, s.hq * a.rq, DIM);
+  unsigned char* const more = smem_raw + sizeof(FewShared);
+  constexpr int kQStride = DIM * 2 + 64;
+  unsigned char* const q_sh = more + lay.q;
+  float* const lse = reinterpret_cast<float*>(more + lay.lse);
+  float2* const stats = reinterpret_cast<float2*>(more + lay.stats);
+  float* const z = reinterpret_cast<float*>(more + lay.z);
+  const int z_stride = z_stride_of(a.slice_cap);
+  // Units of 16 tokens x one KV head, KV heads running fastest; the first one's keys are on their way before the queries
+  // are staged.
+  const int units = flat > 0 ? (m + 15) / 16 * s.hkv : 0;
+  const uint16_t* const k_base = a.k + (long long)(tok0 + t0) * s.k_st;
+  KeyFragment<DIM> frag;
+  int g = warp % s.hkv, tok = warp / s.hkv * 16;
+  if (warp < units) frag.load(k_base + (long long)tok * s.k_st + (long long)g * s.k_sh, s.k_st, m - tok, lane);
+  for (int i = tid; i < terms * (DIM / 8); i += kThreads) {
+    const int row = i / (DIM / 8), piece = i % (DIM / 8);  // row: (KV head, f)
+    const int gg = row / flat, f = row - gg * flat, r = f / s.group;
+    const uint4 v = chain_load(reinterpret_cast<const uint4*>(a.q + (long long)(qrows.first + r) * s.q_st +
+                                                              (long long)(gg * s.group + f - r * s.group) * s.q_sh + piece * 8));
+    *reinterpret_cast<uint4*>(q_sh + row * kQStride + piece * 16) = v;
+  }
+  if (tid < flat) {
+    sh.row_of[tid] = tid / s.group;
+    sh.term_of[tid] = (tid % s.group) * rows + tid / s.group;
+  }
+  if (tid >= 128 && tid < 128 + kNarrowMaxRows)
+    sh.limit[tid - 128] = (causal && tid - 128 < rows) ? chain_load(q_idx + qrows.first + tid - 128) - t0 : 0x7FFFFFFF;  // relative to t0
+  __syncthreads();
+  for (int u = warp; u < units; u += kWarps) {
+    const KeyFragment<DIM> cur = frag;
+    const int g_here = g, tok_here = tok;
+    if (u + kWarps < units) {
+      g = (u + kWarps) % s.hkv;
+      tok = (u + kWarps) / s.hkv * 16;
+      frag.load(k_base + (long long)tok * s.k_st + (long long)g * s.k_sh, s.k_st, m - tok, lane);
+    }
+#pragma unroll 1
+    for (int f0 = 0; f0 < flat; f0 += 8) {  // eight query rows at a time
+      float acc[4] = {0.f, 0.f, 0.f, 0.f};
+      const unsigned char* const qp = q_sh + (g_here * flat + min(f0 + (lane >> 2), flat - 1)) * kQStride + (lane & 3) * 16;
+#pragma unroll
+      for (int i = 0; i < DIM / 32; ++i) {
+        const uint4 qv = *reinterpret_cast<const uint4*>(qp + i * 64);
+        mma_16x8x16(acc, cur.lo[i].x, cur.hi[i].x, cur.lo[i].y, cur.hi[i].y, qv.x, qv.y);
+        mma_16x8x16(acc, cur.lo[i].z, cur.hi[i].z, cur.lo[i].w, cur.hi[i].w, qv.z, qv.w);
+      }
+      const int j = tok_here + (lane >> 2);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int f = f0 + (lane & 3) * 2 + e;
+        if (f < flat) {
+          const int lim = sh.limit[sh.row_of[f]];
+          float* const at = z + (g_here * flat + sh.term_of[f]) * z_stride + j;
+          at[0] = j <= lim ? acc[e] * s.scale_log2 : -INFINITY;
+          at[8] = j + 8 <= lim ? acc[e + 2] * s.scale_log2 : -INFINITY;
+        }
+      }
+    }
+  }
+  // What the selection needs and nothing has needed so far: it arrives while other warps still multiply.
+  if (selecting) {
+    if (b > 0 || c == 0) {
+      int part = 0;
+      bool clamped = false, mismatch = false;
+      for (int i = tid; i <= b; i += kThreads) {  // output offset: the clamped keep counts of the sequences before this one
+        const Span si = seq_span(s, cu_seqlens, i);
+        mismatch |= si.bad;
+        int ki = chain_load(keep_counts + i);
+        if (ki < 0 || ki > si.count) { clamped = true; ki = ki < 0 ? 0 : si.count; }
+        if (i < b) part += ki;
+      }
+      if (part) atomicAdd(&sh.base, part);
+      if (clamped && device_status) atomicOr(device_status, FASTAV_DEV_K_CLAMPED);
+      if (mismatch && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
+    }
+    if (s.flags & FASTAV_PROTECT_QUERY_ROWS) {
+      const Span pr = checked_span(cu_qlens, b, s.total_q, s.total_q);
+      for (int r = pr.first + tid; r < pr.first + pr.count; r += kThreads) {
+        const int j = chain_load(q_idx + r) - t0;
+        if (j >= 0 && j < m) atomicOr(&sh.prot_bits[j >> 5], 1u << (j & 31));
+      }
+    }
+    if (protect)
+      for (int j0 = warp * 32; j0 < m; j0 += kThreads) {  // a warp covers 32 tokens: one word
+        const int j = j0 + lane;
+        const unsigned word = __ballot_sync(0xFFFFFFFFu, j < m && chain_load(protect + tok0 + t0 + j) != 0);
+        if (lane == 0 && word) atomicOr(&sh.prot_bits[j0 >> 5], word);
+      }
+  }
+  if (tid == 0 && (seq.bad || qrows.bad) && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
+  cluster_wait();
+  __syncthreads();
+
+  // ---- log-sum-exp per term ----------------------------------------------------------------------------------
+  if (a.lse) {
+    for (int i = tid; i < terms; i += kThreads) {
+      const float v = chain_load(a.lse + (long long)(qrows.first + i % rows) * s.hq + i / rows);
+      lse[i] = (v == v && fabsf(v) != INFINITY) ? v * kLog2e : INFINITY;  // a row that sees no key adds 0
+    }
+  } else {
+    const int first_seg = t0 / seg, segs = (m + seg - 1) / seg, l8 = tid & (kStatLanes - 1);
+#pragma unroll 1
+    for (int i0 = 0; i0 < terms * segs; i0 += kThreads / kStatLanes) {  // (segment, term): running (max, sum 2^(z - max))
+      const int i = i0 + tid / kStatLanes;
+      const bool active = i < terms * segs;
+      const int sg = segs == 1 ? 0 : i / terms, term = i - sg * terms, end = active ? min(m, (sg + 1) * seg) : 0;
+      const float* const row = z + (active ? term : 0) * z_stride;
+      float zm = -INFINITY, sum = 0.f;
+#pragma unroll 1
+      for (int j0 = sg * seg + l8; j0 < end; j0 += kStatLanes * 4) {
+        float v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = j0 + kStatLanes * u < end ? row[j0 + kStatLanes * u] : -INFINITY;
+        const float zn = fmaxf(zm, fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])));
+        const float ref = zn == -INFINITY ? 0.f : zn;
+        sum *= ptx::ex2_approx(zm - ref);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) sum += ptx::ex2_approx(v[u] - ref);
+        zm = zn;
+      }
+      __syncwarp();
+      float bm = zm;
+#pragma unroll
+      for (int d = kStatLanes / 2; d; d >>= 1) bm = fmaxf(bm, __shfl_xor_sync(0xFFFFFFFFu, bm, d));
+      sum = bm == -INFINITY ? 0.f : sum * ptx::ex2_approx(zm - bm);
+#pragma unroll
+      for (int d = kStatLanes / 2; d; d >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, d);
+      if (active) {
+        float2* const at = &stats[(first_seg + sg) * terms + term];
+        for (int q = l8; q < blocks; q += kStatLanes) remote_store2(remote(at, q), __float_as_uint(bm), __float_as_uint(sum));
+      }
+    }
+    cluster_sync();
+    const int all_segs = (n + seg - 1) / seg, sg = tid & (kSegments - 1);
+#pragma unroll 1
+    for (int i0 = 0; i0 < terms; i0 += kThreads / kSegments) {  // a lane per segment
+      const int i = i0 + tid / kSegments;
+      float2 p = make_float2(-INFINITY, 0.f);
+      if (i < terms && sg < all_segs) p = stats[sg * terms + i];
+      float bm = p.x;
+#pragma unroll
+      for (int d = kSegments / 2; d; d >>= 1) bm = fmaxf(bm, __shfl_xor_sync(0xFFFFFFFFu, bm, d));
+      float total = p.x > -INFINITY ? p.y * ptx::ex2_approx(p.x - bm) : 0.f;
+#pragma unroll
+      for (int d = kSegments / 2; d; d >>= 1) total += __shfl_xor_sync(0xFFFFFFFFu, total, d);
+      if (i < terms && sg == 0) lse[i] = total > 0.f ? bm + log2f(total) : INFINITY;
+    }
+  }
+  __syncthreads();
+
+  // ---- scores: eight lanes per token, each every eighth term in ascending order, added in a fixed tree ---------
+  const bool lowest = (s.flags & FASTAV_SELECT_LOWEST) != 0;
+  const float inv = all_rows > 0 ? 1.0f / ((float)s.hq * (float)all_rows) : 0.f;
+  const int part = tid & (kTokenLanes - 1);
+#pragma unroll 1
+  for (int j0 = 0; j0 < m; j0 += kThreads / kTokenLanes) {
+    const int j = j0 + tid / kTokenLanes;
+    float total = 0.f;
+    if (j < m) {
+#pragma unroll 4
+      for (int i = part; i < terms; i += kTokenLanes) total += ptx::ex2_approx(z[i * z_stride + j] - lse[i]);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int d = kTokenLanes / 2; d; d >>= 1) total += __shfl_xor_sync(0xFFFFFFFFu, total, d);
+    const float score = total * inv;
+    if (j < m) {
+      if (part == 0) a.scores_out[tok0 + t0 + j] = score;
+      if (selecting) {
+        unsigned x = order_key(lowest ? -score : score);
+        if (x == kProtectedKey) x = kProtectedKey - 1;  // only a NaN pattern lands here
+        if ((sh.prot_bits[j >> 5] >> (j & 31)) & 1u) x = kProtectedKey;
+        for (int q = part; q < blocks; q += kTokenLanes) remote_store(remote(&sh.keys[t0 + j], q), x);  // to every block of the cluster
+      }
+    }
+  }
+  if (!selecting) return;  // uniform for the cluster; nothing remote is outstanding
+  cluster_sync();          // the last remote access: from here on every block works for itself
+
+  // ---- selection: thread t owns the tokens 4 t .. 4 t + 3 of the whole sequence ----------------------------------
+  const int base = sh.base;
+  if (c == 0 && tid == 0) {
+    cu_keep[b + 1] = base + k;
+    if (b == 0) cu_keep[0] = 0;
+  }
+  if (k == 0) return;  // uniform for the cluster
+  const int mine = max(0, min(4, n - 4 * tid));
+  unsigned x[4];
+  {
+    const uint4 v = *reinterpret_cast<const uint4*>(&sh.keys[4 * tid]);
+    x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+  }
+  unsigned prefix = 0u;   // the bits of the k-th largest key fixed so far
+  int remaining = k, bits_left = 32;
+#pragma unroll 1
+  while (bits_left > 0) {
+    const int shift = max(0, bits_left - kDigitBits);
+    const unsigned above_want = __funnelshift_rc(prefix, 0u, bits_left);  // prefix >> bits_left, 0 for 32
+    if (bits_left < 32) {
+      for (int i = tid; i < kBins / 4; i += kThreads) reinterpret_cast<uint4*>(sh.hist)[i] = make_uint4(0, 0, 0, 0);
+      __syncthreads();
+    }
+    {
+      unsigned run_digit = kBins, run_len = 0u;  // equal digits of consecutive tokens (typically zeros): one update
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (u < mine && __funnelshift_rc(x[u], 0u, bits_left) == above_want) {
+          const unsigned digit = (x[u] >> shift) & (kBins - 1);
+          if (digit != run_digit) {
+            if (run_len) atomicAdd(&sh.hist[run_digit], run_len);
+            run_digit = digit;
+            run_len = 0u;
+          }
+          ++run_len;
+        }
+      }
+      if (run_len) atomicAdd(&sh.hist[run_digit], run_len);
+    }
+    __syncthreads();
+    unsigned h[kBinsPerThread], own = 0;
+#pragma unroll
+    for (int i = 0; i < kBinsPerThread; i += 4) {
+      const uint4 v = *reinterpret_cast<const uint4*>(&sh.hist[tid * kBinsPerThread + i]);
+      h[i] = v.x; h[i + 1] = v.y; h[i + 2] = v.z; h[i + 3] = v.w;
+      own += v.x + v.y + v.z + v.w;
+    }
+    unsigned above = sum_above<kWarps>(own, sh.warp_a, lane, warp);
+    const unsigned rem = (unsigned)remaining;
+    if (above < rem && rem <= above + own) {  // exactly one thread: its bins from the top
+#pragma unroll
+      for (int i = kBinsPerThread - 1; i >= 0; --i) {
+        if (above < rem && rem <= above + h[i]) {
+          sh.prefix = prefix | ((unsigned)(tid * kBinsPerThread + i) << shift);
+          sh.remaining = (int)(rem - above);
+          sh.bucket = (int)h[i];
+        }
+        above += h[i];
+      }
+    }
+    __syncthreads();
+    prefix = sh.prefix;
+    remaining = sh.remaining;
+    bits_left = shift;
+    if (bits_left > 0 && sh.bucket <= kDirectMax) {  // few keys left: collect them, each finds its rank by counting
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (u < mine && (x[u] >> bits_left) == (prefix >> bits_left)) sh.list[atomicAdd(&sh.list_n, 1)] = x[u];
+      __syncthreads();
+      rank_finish(sh.list, sh.list_n, remaining, tid, &sh.threshold, &sh.need_eq);
+      __syncthreads();
+      prefix = sh.threshold;
+      remaining = sh.need_eq;
+      bits_left = 0;
+    }
+  }
+  const unsigned T = prefix;
+  const int need_eq = remaining;  // how many keys equal to T are kept: the lowest-index ones
+  unsigned both = 0;              // keys above the threshold in the low half, keys equal to it in the high half
+#pragma unroll
+  for (int u = 0; u < 4; ++u) both += u < mine ? (x[u] > T ? 1u : 0u) + (x[u] == T ? 0x10000u : 0u) : 0u;
+  const unsigned before = sum_before<kWarps>(both, sh.warp_a, lane, warp);
+  int gt = (int)(before & 0xFFFFu), eq = (int)(before >> 16);
+  if (c == 0 && tid == kThreads - 1 && T == kProtectedKey && eq + (int)(both >> 16) > need_eq && device_status)
+    atomicOr(device_status, FASTAV_DEV_PROTECT_OVERFLOW);  // more protected tokens than k
+  const bool global_idx = (s.flags & FASTAV_KEEP_IDX_GLOBAL) != 0;
+  if (4 * tid == t0) sh.first_out = gt + min(eq, need_eq);   // t0 is a multiple of 32
+  if (4 * tid == t0 + m) sh.end_out = gt + min(eq, need_eq); // so is the end of a slice, but for the last one's
+  unsigned* const picked = sh.hist;                          // survivor `out` of the sequence is token picked[out % 2048]
+  if (4 * tid >= t0 && 4 * tid < t0 + m) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const bool is_gt = x[u] > T, is_eq = x[u] == T;
+      if (u < mine && (is_gt || (is_eq && eq < need_eq))) {
+        const int out = gt + min(eq, need_eq), j = 4 * tid + u;
+        keep_idx[base + out] = (global_idx ? tok0 : 0) + j;
+        picked[out & (kMaxTokens - 1)] = (unsigned)j;
+      }
+      gt += is_gt;
+      eq += is_eq;
+    }
+  }
+  if (!a.do_gather || m == 0) return;  // (a block without tokens has nothing to copy)
+
+  // ---- gather: this block's survivors, 16-byte chunks of all their rows dealt over the threads ---------------------
+  __syncthreads();
+  const RowShape shape(s, a.rows);
+  const int first = sh.first_out, count = min((t0 + m == n ? k : sh.end_out) - first, s.total_keep - base - first);
+  if (a.rows.pos_in)
+    for (int i = tid; i < count; i += kThreads)
+      a.rows.pos_out[base + first + i] = chain_load(a.rows.pos_in + tok0 + picked[(first + i) & (kMaxTokens - 1)]);
+  const unsigned magic = 0xFFFFFFFFu / (unsigned)shape.n_chunks + 1u;  // e / n_chunks = umulhi(e, magic) while e * n_chunks < 2^32
+  const int chunks = count * shape.n_chunks;
+  constexpr int kUnroll = 6;
+#pragma unroll 1
+  for (int e0 = tid; e0 < chunks; e0 += kThreads * kUnroll) {
+    uint4 v[kUnroll];
+    int row[kUnroll], chunk[kUnroll];
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u) {
+      const int e = e0 + u * kThreads;
+      if (e < chunks) {
+        row[u] = shape.n_chunks == 1 ? e : (int)__umulhi((unsigned)e, magic);
+        chunk[u] = e - row[u] * shape.n_chunks;
+        v[u] = load_stream(chunk_in(s, a.rows, shape, (long long)tok0 + picked[(first + row[u]) & (kMaxTokens - 1)], chunk[u]));
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u)
+      if (e0 + u * kThreads < chunks) store_row(chunk_out(s, a.rows, shape, (long long)base + first + row[u], chunk[u]), v[u]);
+  }
+}
+
+#ifndef FASTAV_FEW_CLUSTER
+#define FASTAV_FEW_CLUSTER 16
+#endif
+#ifndef FASTAV_FEW_SLICE
+#define FASTAV_FEW_SLICE 32
+#endif
+#ifndef FASTAV_GATHER_BYTES
+#define FASTAV_GATHER_BYTES (96 << 10)
+#endif
+
+int slice_of(const Shapes& s, int blocks) { return segment_of(s.max_seqlen) * (kSegments / blocks); }  // tokens per block
+
+size_t smem_of(const Shapes& s, int blocks) {
+  return sizeof(FewShared) + few_layout(slice_of(s, blocks), s.hq * s.max_qlen, s.dim).total;
+}
+
+constexpr size_t kMaxDynamic = 220 * 1024;
+
+// Blocks per sequence.  FEW_CLUSTER_RULE
+int cluster_of(const Shapes& s) {
+  int blocks = FASTAV_FEW_CLUSTER;
+  while (blocks > 1 && ((long long)s.batch * blocks > kNumSMs || s.max_seqlen <= blocks / 2 * FASTAV_FEW_SLICE)) blocks /= 2;
+  while (blocks < kMaxCluster && smem_of(s, blocks) > kMaxDynamic) blocks *= 2;
+  return blocks;
+}
+
+template <int DIM>
+cudaError_t launch(const Shapes& s, FewArgs a, const int32_t* cu_seqlens, const int32_t* keep_counts, const uint8_t* protect,
+                   const int32_t* q_idx, const int32_t* cu_qlens, int32_t* keep_idx, int32_t* cu_keep, int32_t* device_status,
+                   cudaStream_t stream) {
+  const int blocks = cluster_of(s);
+  a.slice_cap = slice_of(s, blocks);
+  cudaError_t e = once_per_device([] {
+    cudaError_t f = cudaFuncSetAttribute(prune_few_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamic);
+    if (f == cudaSuccess) f = cudaFuncSetAttribute(prune_few_kernel<DIM>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return f;
+  });
+  if (e != cudaSuccess) return e;
+  e = launch_chained_cluster(prune_few_kernel<DIM>, dim3(s.batch * blocks), dim3(kThreads), blocks, smem_of(s, blocks), stream, s, a,
+                             cu_seqlens, keep_counts, protect, q_idx, cu_qlens, keep_idx, cu_keep, device_status);
+  count_launches(1);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+}  // namespace
+
+// Few scored rows, up to 2,048 tokens (FEW_RULE).
+bool few_applies(const Shapes& s) {
+  if ((s.flags & FASTAV_SCORE_PATH_MASK) != 0) return false;
+  if (s.max_qlen < 1 || s.max_qlen > kNarrowMaxRows || s.max_qlen * s.group > 128) return false;
+  return s.max_seqlen >= 1 && s.max_seqlen <= kMaxTokens && smem_of(s, cluster_of(s)) <= kMaxDynamic;
+}
+
+// The survivors' rows may be copied by the blocks that select them: worth it while that is little per block (GATHER_RULE).
+bool few_gathers(const Shapes& s, int row_bytes) {
+  const int blocks = cluster_of(s);
+  return row_bytes > 0 && (long long)((s.max_keep + blocks - 1) / blocks) * row_bytes <= FASTAV_GATHER_BYTES;
+}
+
+cudaError_t launch_few(const Shapes& s, const void* q, const void* k, const float* lse_in, float* scores_out, bool do_select,
+                       const RowStreams* rows, const int32_t* cu_seqlens, const int32_t* keep_counts, const uint8_t* protect,
+                       const int32_t* q_idx, const int32_t* cu_qlens, int32_t* keep_idx, int32_t* cu_keep, int32_t* device_status,
+                       cudaStream_t stream) {
+  FewArgs a{};
+  a.q = static_cast<const uint16_t*>(q);
+  a.k = static_cast<const uint16_t*>(k);
+  a.lse = lse_in;
+  a.scores_out = scores_out;
+  a.rq = s.max_qlen;
+  a.do_select = do_select ? 1 : 0;
+  if (rows) {
+    a.do_gather = 1;
+    a.rows = *rows;
+  }
+  return s.dim == 128 ? launch<128>(s, a, cu_seqlens, keep_counts, protect, q_idx, cu_qlens, keep_idx, cu_keep, device_status, stream)
+                      : launch<64>(s, a, cu_seqlens, keep_counts, protect, q_idx, cu_qlens, keep_idx, cu_keep, device_status, stream);
+}
+
+}  // namespace fastav

@@ -354,15 +354,20 @@ cudaError_t launch_narrow_logits(const Shapes& s, const Workspace& w, const void
 
 cudaError_t launch_score_narrow(const Shapes& s, const Workspace& w, const void* q, const int32_t* q_idx,
                                 const int32_t* cu_qlens, const void* k, const int32_t* cu_seqlens, const float* lse_in,
-                                float* scores_out, unsigned char* ws, int32_t* device_status, cudaStream_t stream) {
+                                float* scores_out, unsigned char* ws, int32_t* device_status, cudaStream_t stream, ScoreLeft* left) {
   float* logits = reinterpret_cast<float*>(ws + w.logits_off);
   float* lse = reinterpret_cast<float*>(ws + w.lse_off);
   const int rq = s.max_qlen;
+  if (scores_out && few_applies(s)) {  // one kernel from the keys to the scores, together with the selection if there is one
+    if (left) {
+      left->kind = ScoreLeft::kKeys;
+      return cudaSuccess;
+    }
+    return launch_few(s, q, k, lse_in, scores_out, false, nullptr, cu_seqlens, nullptr, nullptr, q_idx, cu_qlens, nullptr, nullptr,
+                      device_status, stream);
+  }
   cudaError_t e = launch_narrow_logits(s, w, q, q_idx, cu_qlens, k, cu_seqlens, ws, device_status, stream);
   if (e != cudaSuccess) return e;
-  if (!lse_in && scores_out && narrow_tail_applies(s))  // short sequences: statistics and scores in one kernel
-    return launch_narrow_tail(s, logits, rq, scores_out, false, cu_seqlens, nullptr, nullptr, q_idx, cu_qlens, nullptr, nullptr,
-                              device_status, stream);
   if (lse_in) e = launch_lse_import(s, lse_in, lse, stream);
   else e = launch_chained(score_narrow_stats_kernel, dim3(s.hq * rq, s.batch), dim3(256), 0, stream, s, cu_qlens, cu_seqlens,
                           (const float*)logits, rq, lse);
