@@ -205,14 +205,15 @@ __global__ void __launch_bounds__(256) score_narrow_stats_kernel(Shapes s, const
                                                                  const float* __restrict__ logits, int rq,
                                                                  float* __restrict__ lse) {
   __shared__ float red[8];
-  chain_enter(s, cu_qlens, cu_seqlens);
-  // the caller's arrays first: these loads overlap the predecessor's tail
-  const int b = blockIdx.y, head = blockIdx.x / rq, r = blockIdx.x % rq;
-  const Span seq = seq_span(s, cu_seqlens, b), qrows = row_span(s, cu_qlens, b);
-  const int row0 = qrows.first, rows = min(qrows.count, rq);
-  const int tok0 = seq.first, n = seq.count;
+  chain_enter(s);
   pdl_wait();
   pdl_acquire(logits);
+  pdl_acquire(cu_qlens);
+  pdl_acquire(cu_seqlens);
+  const int b = blockIdx.y, head = blockIdx.x / rq, r = blockIdx.x % rq;
+  const Span seq = seq_span<true>(s, cu_seqlens, b), qrows = row_span<true>(s, cu_qlens, b);
+  const int row0 = qrows.first, rows = min(qrows.count, rq);
+  const int tok0 = seq.first, n = seq.count;
   if (r >= rows) return;
   const float* z = logits + ((long long)head * rq + r) * s.total_tokens + tok0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -263,16 +264,17 @@ __global__ void __launch_bounds__(kFinalizeThreads) score_narrow_finalize_kernel
                                                                                  const float* __restrict__ lse,
                                                                                  float* __restrict__ scores) {
   extern __shared__ float lse_sh[];  // [Hq][rows], then the term offsets
-  chain_enter(s, cu_qlens, cu_seqlens);
-  // the caller's arrays first: these loads overlap the predecessor's tail
-  const int b = blockIdx.y;
-  const Span seq = seq_span(s, cu_seqlens, b), qrows = row_span(s, cu_qlens, b);
-  const int tok0 = seq.first, n = seq.count;
-  const int row0 = qrows.first, all_rows = qrows.count, rows = min(all_rows, rq);
-  const int terms = s.hq * rows;
+  chain_enter(s);
   pdl_wait();
   pdl_acquire(logits);
   pdl_acquire(lse);
+  pdl_acquire(cu_qlens);
+  pdl_acquire(cu_seqlens);
+  const int b = blockIdx.y;
+  const Span seq = seq_span<true>(s, cu_seqlens, b), qrows = row_span<true>(s, cu_qlens, b);
+  const int tok0 = seq.first, n = seq.count;
+  const int row0 = qrows.first, all_rows = qrows.count, rows = min(all_rows, rq);
+  const int terms = s.hq * rows;
   if ((int)(blockIdx.x * blockDim.x) >= n) return;
   // where term i's logits start, in units of N floats: worked out once per block (no integer division per logit below)
   int* term_row = reinterpret_cast<int*>(lse_sh + s.hq * rq);

@@ -591,25 +591,22 @@ __global__ void __launch_bounds__(256) score_wide_merge_kernel(Shapes s, const i
                                                                const int32_t* __restrict__ cu_seqlens,
                                                                const float2* __restrict__ stats, int stat_chunks,
                                                                int chunk_keys, float* __restrict__ lse) {
-  chain_enter(s, cu_qlens, cu_seqlens);
-  // which sequence this warp's row belongs to: from the caller's arrays, so before the wait
-  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  const bool active = w < s.total_q * s.hq;
-  int chunks = 0;
-  if (active) {
-    const int row = w / s.hq;
-    int n = 0;  // length of the row's sequence, the last one that starts at or before it: the whole warp looks
-    for (int b0 = 0; b0 < s.batch; b0 += 32) {
-      const int b = min(b0 + lane, s.batch - 1);
-      const int first = chain_load(cu_qlens + b), count = seq_span(s, cu_seqlens, b).count;
-      const unsigned not_after = __ballot_sync(0xFFFFFFFFu, b0 + lane < s.batch && first <= row);
-      if (not_after) n = __shfl_sync(0xFFFFFFFFu, count, 31 - __clz(not_after));
-    }
-    chunks = 2 * ((n + chunk_keys - 1) / chunk_keys);  // one entry per 64-key half of every tile run
-  }
+  chain_enter(s);
   pdl_wait();
   pdl_acquire(stats);
-  if (!active) return;
+  pdl_acquire(cu_qlens);
+  pdl_acquire(cu_seqlens);
+  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (w >= s.total_q * s.hq) return;
+  const int row = w / s.hq;
+  int n = 0;  // length of the row's sequence, the last one that starts at or before it: the whole warp looks
+  for (int b0 = 0; b0 < s.batch; b0 += 32) {
+    const int b = min(b0 + lane, s.batch - 1);
+    const int first = chain_load_cached(cu_qlens + b), count = seq_span<true>(s, cu_seqlens, b).count;
+    const unsigned not_after = __ballot_sync(0xFFFFFFFFu, b0 + lane < s.batch && first <= row);
+    if (not_after) n = __shfl_sync(0xFFFFFFFFu, count, 31 - __clz(not_after));
+  }
+  const int chunks = 2 * ((n + chunk_keys - 1) / chunk_keys);  // one entry per 64-key half of every tile run
   const float2* mine = stats + (long long)w * stat_chunks;
   // the first 32 entries stay in a register (usually all of them); the rest, if any, is read twice
   const float2 first = lane < chunks ? chain_load(mine + lane) : make_float2(-INFINITY, 0.f);
@@ -636,15 +633,17 @@ __global__ void __launch_bounds__(kFinalizeThreads) score_wide_finalize_kernel(S
                                                                                const int32_t* __restrict__ cu_qlens, int rc_max,
                                                                                int rows_per_chunk, const float* __restrict__ partial,
                                                                                float* __restrict__ scores) {
-  chain_enter(s, cu_seqlens, cu_qlens);
-  const int b = blockIdx.y;
-  const Span seq = seq_span(s, cu_seqlens, b);
-  const int tok0 = seq.first, n = seq.count;
-  const int rows = row_span(s, cu_qlens, b).count;
-  const int row_chunks = (rows * s.group + rows_per_chunk - 1) / rows_per_chunk;
-  const float inv = rows > 0 ? 1.0f / ((float)s.hq * (float)rows) : 0.f;
+  chain_enter(s);
   pdl_wait();
   pdl_acquire(partial);
+  pdl_acquire(cu_seqlens);
+  pdl_acquire(cu_qlens);
+  const int b = blockIdx.y;
+  const Span seq = seq_span<true>(s, cu_seqlens, b);
+  const int tok0 = seq.first, n = seq.count;
+  const int rows = row_span<true>(s, cu_qlens, b).count;
+  const int row_chunks = (rows * s.group + rows_per_chunk - 1) / rows_per_chunk;
+  const float inv = rows > 0 ? 1.0f / ((float)s.hq * (float)rows) : 0.f;
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
   // Partial i = (KV head, row chunk) in that order; eight loads in flight, one running sum in fixed order.

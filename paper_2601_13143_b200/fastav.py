@@ -74,6 +74,16 @@ class FastavError(RuntimeError):
 
 
 _lib = None
+_binding = None
+
+
+def _native():
+    """The C module that marshals the hot calls (raises ImportError if it has not been built)."""
+    global _binding
+    if _binding is None:
+        from . import _binding as module
+        _binding = module
+    return _binding
 
 
 def library_path() -> str:
@@ -138,17 +148,34 @@ def library() -> ctypes.CDLL:
     return _lib
 
 
-def _p(t: torch.Tensor | None):
-    """Device pointer of a tensor (None -> NULL)."""
-    if t is None:
-        return None
-    return ctypes.c_void_p(t.data_ptr())
+def _p(t: torch.Tensor | None) -> int | None:
+    """Device pointer of a tensor (None -> NULL); ctypes makes it the pointer the entry point's argtypes ask for."""
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+def _stream(stream) -> int:
+    if stream is not None:
+        return stream.cuda_stream
+    if torch.cuda.is_initialized():  # the current stream's handle without a Stream object around it
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return torch.cuda.current_stream().cuda_stream
+
+
+_addresses: dict[str, int] = {}
+
+
+def _address(name: str) -> int:
+    """Where the library's entry point `name` lies, for the C module that calls it."""
+    found = _addresses.get(name)
+    if found is None:
+        found = _addresses[name] = ctypes.cast(getattr(library(), name), ctypes.c_void_p).value
+    return found
+
+
+def _params(params: fastav_params) -> int:
+    if type(params) is not fastav_params:
+        raise TypeError("expected a fastav_params")
+    return ctypes.addressof(params)
 
 
 def _strides3(t: torch.Tensor | None, heads: int, dim: int) -> tuple[int, int]:
@@ -195,7 +222,7 @@ def fastav_workspace_bytes(params: fastav_params) -> int:
 
 
 def _ws(workspace: torch.Tensor | None):
-    return (_p(workspace), ctypes.c_size_t(0 if workspace is None else workspace.numel() * workspace.element_size()))
+    return (None, 0) if workspace is None else (workspace.data_ptr(), workspace.nbytes)
 
 
 def fastav_score(params, q, q_idx, cu_qlens, k, cu_seqlens, scores_out, workspace, device_status=None, stream=None,
@@ -222,9 +249,9 @@ def fastav_select(params, scores, cu_seqlens, keep_counts, protect_opt, q_idx, c
 
 def fastav_select_mask(params, keep_mask, cu_seqlens, keep_idx_out, cu_keep_out, workspace, device_status=None, stream=None) -> None:
     """Keep list of a rule-given keep mask (the paper's positional global stage)."""
-    ws, ws_bytes = _ws(workspace)
-    _check(library().fastav_select_mask(ctypes.byref(params), _p(keep_mask), _p(cu_seqlens), _p(keep_idx_out), _p(cu_keep_out),
-                                        ws, ws_bytes, _p(device_status), _stream(stream)), "fastav_select_mask")
+    status = _native().select_mask(_address("fastav_select_mask"), _params(params), keep_mask, cu_seqlens, keep_idx_out, cu_keep_out, workspace,
+                                   device_status, _stream(stream))
+    _check(status, "fastav_select_mask")
 
 
 def fastav_selftest_bounded_wait(limit_ms: int, device_status, stream=None) -> None:
@@ -291,19 +318,18 @@ def fastav_select_noalloc(params, scores, cu_seqlens, keep_counts, protect_opt, 
 
 def fastav_compact(params, keep_idx, cu_keep, cu_seqlens, hidden_in=None, hidden_out=None, pos_in=None, pos_out=None,
                    k_in=None, k_out=None, v_in=None, v_out=None, device_status=None, stream=None) -> None:
-    _check(library().fastav_compact(ctypes.byref(params), _p(keep_idx), _p(cu_keep), _p(cu_seqlens), _p(hidden_in),
-                                    _p(hidden_out), _p(pos_in), _p(pos_out), _p(k_in), _p(k_out), _p(v_in), _p(v_out),
-                                    _p(device_status), _stream(stream)), "fastav_compact")
+    status = _native().compact(_address("fastav_compact"), _params(params), keep_idx, cu_keep, cu_seqlens, hidden_in, hidden_out, pos_in, pos_out,
+                               k_in, k_out, v_in, v_out, device_status, _stream(stream))
+    _check(status, "fastav_compact")
 
 
 def fastav_prune(params, q, q_idx, cu_qlens, k, v, cu_seqlens, keep_counts, protect_opt, hidden_in, pos_in, scores_out,
                  keep_idx_out, cu_keep_out, hidden_out, pos_out, k_out, v_out, workspace, device_status=None,
                  stream=None, lse_opt=None) -> None:
-    ws, ws_bytes = _ws(workspace)
-    _check(library().fastav_prune(ctypes.byref(params), _p(q), _p(q_idx), _p(cu_qlens), _p(k), _p(v), _p(cu_seqlens),
-                                  _p(lse_opt), _p(keep_counts), _p(protect_opt), _p(hidden_in), _p(pos_in), _p(scores_out),
-                                  _p(keep_idx_out), _p(cu_keep_out), _p(hidden_out), _p(pos_out), _p(k_out), _p(v_out),
-                                  ws, ws_bytes, _p(device_status), _stream(stream)), "fastav_prune")
+    status = _native().prune(_address("fastav_prune"), _params(params), q, q_idx, cu_qlens, k, v, cu_seqlens, lse_opt, keep_counts, protect_opt,
+                             hidden_in, pos_in, scores_out, keep_idx_out, cu_keep_out, hidden_out, pos_out, k_out, v_out, workspace,
+                             device_status, _stream(stream))
+    _check(status, "fastav_prune")
 
 
 def fastav_kernel_launches() -> int:
