@@ -56,21 +56,6 @@ size_t view_bytes(int64_t rows, int64_t st, int64_t sh, int heads, int dim) {
   return (size_t)(((rows - 1) * st + (int64_t)(heads - 1) * sh + dim) * 2);
 }
 
-Shapes make_shapes(const fastav_params& p) {
-  Shapes s{};
-  s.batch = p.batch; s.total_tokens = p.total_tokens; s.max_seqlen = p.max_seqlen;
-  s.total_q = p.total_q; s.max_qlen = p.max_qlen; s.total_keep = p.total_keep; s.max_keep = p.max_keep;
-  s.hq = p.num_q_heads; s.hkv = p.num_kv_heads; s.group = p.num_q_heads / p.num_kv_heads;
-  s.dim = p.head_dim; s.hidden = p.hidden;
-  s.q_st = p.q_stride_tok; s.q_sh = p.q_stride_head;
-  s.k_st = p.k_stride_tok; s.k_sh = p.k_stride_head; s.v_st = p.v_stride_tok; s.v_sh = p.v_stride_head;
-  s.ko_st = p.ko_stride_tok; s.ko_sh = p.ko_stride_head; s.vo_st = p.vo_stride_tok; s.vo_sh = p.vo_stride_head;
-  const float scale = p.softmax_scale > 0.f ? p.softmax_scale : 1.0f / std::sqrt((float)p.head_dim);
-  s.scale_log2 = scale * kLog2e;
-  s.flags = p.flags;
-  return s;
-}
-
 int32_t check_workspace(const Workspace& w, const void* ws, size_t bytes) {
   if (w.total == 0) return FASTAV_OK;
   if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || bytes < w.total) return FASTAV_ERR_WORKSPACE;
@@ -129,6 +114,21 @@ int32_t check_compact_args(const fastav_params* p, const int32_t* keep_idx, cons
 }
 
 }  // namespace
+
+Shapes make_shapes(const fastav_params& p) {
+  Shapes s{};
+  s.batch = p.batch; s.total_tokens = p.total_tokens; s.max_seqlen = p.max_seqlen;
+  s.total_q = p.total_q; s.max_qlen = p.max_qlen; s.total_keep = p.total_keep; s.max_keep = p.max_keep;
+  s.hq = p.num_q_heads; s.hkv = p.num_kv_heads; s.group = p.num_q_heads / p.num_kv_heads;
+  s.dim = p.head_dim; s.hidden = p.hidden;
+  s.q_st = p.q_stride_tok; s.q_sh = p.q_stride_head;
+  s.k_st = p.k_stride_tok; s.k_sh = p.k_stride_head; s.v_st = p.v_stride_tok; s.v_sh = p.v_stride_head;
+  s.ko_st = p.ko_stride_tok; s.ko_sh = p.ko_stride_head; s.vo_st = p.vo_stride_tok; s.vo_sh = p.vo_stride_head;
+  const float scale = p.softmax_scale > 0.f ? p.softmax_scale : 1.0f / std::sqrt((float)p.head_dim);
+  s.scale_log2 = scale * kLog2e;
+  s.flags = p.flags;
+  return s;
+}
 
 void count_launches(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
@@ -308,6 +308,35 @@ int32_t fastav_compact(const fastav_params* params, const int32_t* keep_idx, con
   return e == cudaSuccess ? FASTAV_OK : cuda_failed(e);
 }
 
+}  // extern "C"
+
+namespace fastav {
+
+// Scores and keep list of a validated prune call.  `rows` (optional): what to gather; *gathered says whether that was done
+// as well (few survivors: the kernel that selects them copies their rows).
+cudaError_t enqueue_selection(const fastav_params& params, const void* q, const int32_t* q_idx, const int32_t* cu_qlens, const void* k,
+                              const int32_t* cu_seqlens, const float* lse_opt, const int32_t* keep_counts, const uint8_t* protect_opt,
+                              const RowStreams* rows, float* scores_out, int32_t* keep_idx_out, int32_t* cu_keep_out, unsigned char* ws,
+                              int32_t* device_status, cudaStream_t st, bool* gathered) {
+  const Workspace w = plan_workspace(params);
+  const Shapes s = make_shapes(params);
+  cudaError_t e = cudaSuccess;
+  ScoreLeft left;
+  *gathered = false;
+  if (s.total_tokens > 0) e = launch_score(s, w, q, q_idx, cu_qlens, k, cu_seqlens, lse_opt, scores_out, ws, device_status, st, &left);
+  if (e != cudaSuccess) return e;
+  if (left.kind == ScoreLeft::kKeys) {
+    *gathered = rows && s.total_keep > 0 && few_gathers(s, row_bytes_of(s, *rows));
+    return launch_few(s, q, k, lse_opt, scores_out, true, *gathered ? rows : nullptr, cu_seqlens, keep_counts, protect_opt, q_idx, cu_qlens,
+                      keep_idx_out, cu_keep_out, device_status, st);
+  }
+  return launch_select(s, w, scores_out, cu_seqlens, keep_counts, protect_opt, q_idx, cu_qlens, keep_idx_out, cu_keep_out, ws, device_status, st);
+}
+
+}  // namespace fastav
+
+extern "C" {
+
 int32_t fastav_prune(const fastav_params* params, const void* q, const int32_t* q_idx, const int32_t* cu_qlens,
                      const void* k, const void* v, const int32_t* cu_seqlens, const float* lse_opt, const int32_t* keep_counts,
                      const uint8_t* protect_opt, const void* hidden_in, const int32_t* pos_in, float* scores_out,
@@ -318,29 +347,15 @@ int32_t fastav_prune(const fastav_params* params, const void* q, const int32_t* 
                               cu_keep_out, hidden_out, pos_out, k_out, v_out, workspace, workspace_bytes);
   if (rc != FASTAV_OK) return rc;
   chain_begin(params->flags);
-  const Workspace w = plan_workspace(*params);
-  const Shapes s = make_shapes(*params);
-  unsigned char* ws = static_cast<unsigned char*>(workspace);
+  const RowStreams rows{static_cast<const uint16_t*>(hidden_in), static_cast<uint16_t*>(hidden_out), static_cast<const uint16_t*>(k_out ? k : nullptr),
+                        static_cast<uint16_t*>(k_out),           static_cast<const uint16_t*>(v),    static_cast<uint16_t*>(v_out),
+                        pos_in,                                  pos_out};
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  cudaError_t e = cudaSuccess;
-  ScoreLeft left;
   bool gathered = false;
-  if (params->total_tokens > 0) e = launch_score(s, w, q, q_idx, cu_qlens, k, cu_seqlens, lse_opt, scores_out, ws, device_status, st, &left);
-  if (e == cudaSuccess) {
-    if (left.kind == ScoreLeft::kKeys) {
-      const RowStreams rows{static_cast<const uint16_t*>(hidden_in), static_cast<uint16_t*>(hidden_out), static_cast<const uint16_t*>(k_out ? k : nullptr),
-                            static_cast<uint16_t*>(k_out),           static_cast<const uint16_t*>(v),    static_cast<uint16_t*>(v_out),
-                            pos_in,                                  pos_out};
-      gathered = s.total_keep > 0 && few_gathers(s, row_bytes_of(s, rows));
-      e = launch_few(s, q, k, lse_opt, scores_out, true, gathered ? &rows : nullptr, cu_seqlens, keep_counts, protect_opt, q_idx, cu_qlens,
-                     keep_idx_out, cu_keep_out, device_status, st);
-    } else {
-      e = launch_select(s, w, scores_out, cu_seqlens, keep_counts, protect_opt, q_idx, cu_qlens, keep_idx_out, cu_keep_out, ws,
-                        device_status, st);
-    }
-  }
+  cudaError_t e = enqueue_selection(*params, q, q_idx, cu_qlens, k, cu_seqlens, lse_opt, keep_counts, protect_opt, &rows, scores_out,
+                                    keep_idx_out, cu_keep_out, static_cast<unsigned char*>(workspace), device_status, st, &gathered);
   if (e == cudaSuccess && !gathered)
-    e = launch_compact(s, keep_idx_out, cu_keep_out, cu_seqlens, hidden_in, hidden_out, pos_in, pos_out, k, k_out, v, v_out,
+    e = launch_compact(make_shapes(*params), keep_idx_out, cu_keep_out, cu_seqlens, hidden_in, hidden_out, pos_in, pos_out, k, k_out, v, v_out,
                        device_status, st);
   return e == cudaSuccess ? FASTAV_OK : cuda_failed(e);
 }

@@ -47,6 +47,7 @@ struct Workspace {
 };
 
 Workspace plan_workspace(const fastav_params& p);
+Shapes make_shapes(const fastav_params& p);
 
 // ---- launchers (each returns cudaGetLastError() after its launches) -------------------------
 cudaError_t launch_score(const Shapes& s, const Workspace& w, const void* q, const int32_t* q_idx,
@@ -116,6 +117,11 @@ int32_t validate_prune(const fastav_params* params, const void* q, const int32_t
                        const int32_t* pos_in, const float* scores_out, const int32_t* keep_idx_out, const int32_t* cu_keep_out,
                        const void* hidden_out, const int32_t* pos_out, const void* k_out, const void* v_out, const void* workspace,
                        size_t workspace_bytes);
+
+cudaError_t enqueue_selection(const fastav_params& params, const void* q, const int32_t* q_idx, const int32_t* cu_qlens, const void* k,
+                              const int32_t* cu_seqlens, const float* lse_opt, const int32_t* keep_counts, const uint8_t* protect_opt,
+                              const RowStreams* rows, float* scores_out, int32_t* keep_idx_out, int32_t* cu_keep_out, unsigned char* ws,
+                              int32_t* device_status, cudaStream_t st, bool* gathered);
 
 // Diagnostic launch counter (fastav_kernel_launches).
 void count_launches(int n);

@@ -1,9 +1,16 @@
-// Host-buffer entry point: the same prune step for callers whose tensors live in host memory
-// (offloaded activations / KV cache).  Copies in, runs fastav_prune, copies out -- all enqueued on
-// the caller's stream, staged through a device arena the caller provides.
+// Host-buffer entry point: the same prune step for callers whose tensors live in host memory (offloaded activations / KV
+// cache), all enqueued on the caller's stream and staged through a device arena the caller provides.
+//
+// Bound by PCIe, about 55 GB/s each way.  Where every buffer is page-locked the GPU can reach them itself, and two things
+// follow.  Only what the method needs crosses the bus: K and the small arrays once, then the SURVIVORS' hidden states and
+// V rows (the others are never uploaded).  And the two directions run at the same time: one kernel reads survivors' rows
+// from host memory and writes them to the host outputs, instead of uploads, kernels and downloads in a row; a handful of
+// copies of a few bytes each (2-4 us apiece) become part of two kernels.  2,048 tokens, half of them kept: HOST_FIGURES.
+// Pageable buffers take the asynchronous copies.
 #include <atomic>
 
 #include "common.cuh"
+#include "gather.cuh"
 
 namespace fastav {
 namespace {
@@ -50,6 +57,121 @@ Arena plan_arena(const fastav_params& p) {
   a.workspace = carve(a.workspace_bytes);
   a.total = off;
   return a;
+}
+
+// ---- the page-locked path ----------------------------------------------------------------------------
+constexpr int kCopyThreads = 256;
+constexpr int kCopyUnroll = 8;                                   // 16-byte loads in flight per thread
+constexpr int kPieceBytes = kCopyThreads * kCopyUnroll * 16;     // what a block copies at a time: 32 KB
+constexpr int kMaxSegments = 12;
+
+struct CopyList {
+  struct {
+    const unsigned char* src;
+    unsigned char* dst;
+    unsigned long long bytes;
+  } seg[kMaxSegments];
+  int count = 0;
+  long long pieces = 0;
+  void add(void* dst, const void* src, size_t bytes) {
+    if (!src || !dst || !bytes) return;
+    seg[count++] = {static_cast<const unsigned char*>(src), static_cast<unsigned char*>(dst), (unsigned long long)bytes};
+    pieces += (long long)((bytes + kPieceBytes - 1) / kPieceBytes);
+  }
+};
+
+// Piece `piece` of the list by one block: 16 bytes at a time where both sides allow it, else single bytes (only the ends of
+// an array, or a small array of odd alignment).
+__device__ __forceinline__ void copy_piece(const CopyList& list, long long piece) {
+  int i = 0;
+  for (; i < list.count; ++i) {
+    const long long here = (long long)((list.seg[i].bytes + kPieceBytes - 1) / kPieceBytes);
+    if (piece < here) break;
+    piece -= here;
+  }
+  if (i == list.count) return;
+  const unsigned char* src = list.seg[i].src + piece * kPieceBytes;
+  unsigned char* dst = list.seg[i].dst + piece * kPieceBytes;
+  const unsigned long long left = list.seg[i].bytes - piece * kPieceBytes;
+  const int bytes = left < (unsigned long long)kPieceBytes ? (int)left : kPieceBytes;
+  int done = 0;
+  if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15u) == 0) {
+    const int quads = bytes / 16;
+    uint4 v[kCopyUnroll];
+#pragma unroll
+    for (int u = 0; u < kCopyUnroll; ++u) {
+      const int q = u * kCopyThreads + threadIdx.x;
+      if (q < quads) v[u] = load_stream(reinterpret_cast<const uint4*>(src) + q);
+    }
+#pragma unroll
+    for (int u = 0; u < kCopyUnroll; ++u) {
+      const int q = u * kCopyThreads + threadIdx.x;
+      if (q < quads) store_row(reinterpret_cast<uint4*>(dst) + q, v[u]);
+    }
+    done = quads * 16;
+  }
+  for (int at = done + threadIdx.x; at < bytes; at += kCopyThreads) dst[at] = chain_load(src + at);
+}
+
+// Host arrays -> arena; the status word starts at zero.
+__global__ void __launch_bounds__(kCopyThreads) host_upload_kernel(CopyList list, int32_t* device_status, ChainHead head) {
+  chain_enter(head);
+  pdl_wait();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *device_status = 0;
+  for (long long piece = blockIdx.x; piece < list.pieces; piece += gridDim.x) copy_piece(list, piece);
+}
+
+// The survivors' rows (hidden states and V straight from host memory, K from the arena) and the small results -> host memory.
+__global__ void __launch_bounds__(kCopyThreads) host_gather_kernel(Shapes s, RowStreams t, CopyList list, const int32_t* __restrict__ keep_idx,
+                                                                   const int32_t* __restrict__ cu_keep,
+                                                                   const int32_t* __restrict__ cu_seqlens) {
+  chain_enter(s);
+  pdl_wait();
+  pdl_acquire(keep_idx);
+  pdl_acquire(cu_keep);
+  pdl_acquire(cu_seqlens);
+  for (long long piece = blockIdx.x; piece < list.pieces; piece += gridDim.x) copy_piece(list, piece);
+  const RowShape shape(s, t);
+  const bool global_idx = (s.flags & FASTAV_KEEP_IDX_GLOBAL) != 0;
+  const int rows = min(chain_load_cached(cu_keep + s.batch), s.total_keep);
+  const int lane = threadIdx.x & 31, step = gridDim.x * (kCopyThreads / 32);
+  for (int row = blockIdx.x * (kCopyThreads / 32) + (threadIdx.x >> 5); row < rows; row += step) {  // a warp per row
+    int lo = 0, hi = s.batch;  // largest b with cu_keep[b] <= row
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (chain_load_cached(cu_keep + mid) <= row) lo = mid; else hi = mid;
+    }
+    const long long src = (global_idx ? 0ll : (long long)chain_load_cached(cu_seqlens + lo)) + chain_load(keep_idx + row);
+    if (src < 0 || src >= s.total_tokens) continue;  // (the selection's own indices: cannot happen)
+    if (lane == 0 && t.pos_in) t.pos_out[row] = chain_load(t.pos_in + src);
+    copy_row<32, kCopyUnroll>(s, t, shape, src, row, lane);
+  }
+}
+
+struct Range {
+  const void* at;
+  size_t bytes;
+  bool overlaps(const Range& o) const {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(at), b = reinterpret_cast<uintptr_t>(o.at);
+    return at && o.at && a < b + o.bytes && b < a + bytes;
+  }
+};
+
+// The address under which the GPU reaches a page-locked host array, or nullptr.  Both ends are looked up: the array has
+// to lie inside one mapping.
+void* mapped(const void* host, size_t bytes) {
+  cudaPointerAttributes first{}, last{};
+  if (cudaPointerGetAttributes(&first, host) != cudaSuccess || first.type != cudaMemoryTypeHost || !first.devicePointer) {
+    (void)cudaGetLastError();
+    return nullptr;
+  }
+  const unsigned char* end = static_cast<const unsigned char*>(host) + (bytes ? bytes - 1 : 0);
+  if (cudaPointerGetAttributes(&last, end) != cudaSuccess || last.type != cudaMemoryTypeHost ||
+      static_cast<unsigned char*>(last.devicePointer) - static_cast<unsigned char*>(first.devicePointer) != (ptrdiff_t)(bytes ? bytes - 1 : 0)) {
+    (void)cudaGetLastError();
+    return nullptr;
+  }
+  return first.devicePointer;
 }
 
 }  // namespace
@@ -100,6 +222,75 @@ int32_t fastav_prune_host(const fastav_params* params, const void* q, const int3
                       (const int32_t*)(base + a.cu_keep), dev(a.hidden_out, hidden_out), (const int32_t*)dev(a.pos_out, pos_out),
                       base + a.k_out, dev(a.v_out, v_out), base + a.workspace, a.workspace_bytes);
   if (rc != FASTAV_OK) return rc;
+  {
+    // Every array page-locked (and the row arrays on 16-byte boundaries): the GPU fetches and delivers them itself.  With
+    // inputs that are also outputs the order matters, which only the copies below keep.
+    const size_t hidden_row = (size_t)p.hidden * 2, q_bytes = R * p.num_q_heads * p.head_dim * 2;
+    const Range ins[] = {{q, q_bytes}, {q_idx, R * 4}, {cu_qlens, (B + 1) * 4}, {k, N * kv_row}, {v, N * kv_row}, {cu_seqlens, (B + 1) * 4},
+                         {lse_opt, R * p.num_q_heads * 4}, {keep_counts, B * 4}, {protect_opt, N}, {hidden_in, N * hidden_row}, {pos_in, N * 4}};
+    const Range outs[] = {{scores_out, N * 4}, {keep_idx_out, K * 4}, {cu_keep_out, (B + 1) * 4}, {hidden_out, K * hidden_row},
+                          {pos_out, K * 4}, {k_out, K * kv_row}, {v_out, K * kv_row}, {status_out, 4}};
+    bool ok = true;
+    for (const Range& i : ins)
+      for (const Range& o : outs) ok = ok && !i.overlaps(o);
+    auto at = [&](const void* host, size_t bytes) -> void* {
+      if (!host || !ok) return nullptr;
+      void* p = mapped(host, bytes);
+      ok = p != nullptr;
+      return p;
+    };
+    auto at16 = [&](const void* host, size_t bytes) -> void* {
+      void* p = at(host, bytes);
+      ok = ok && (reinterpret_cast<uintptr_t>(p) & 15u) == 0;
+      return p;
+    };
+    CopyList up, down;
+    RowStreams rows{};
+    up.add(base + a.k, at16(k, N * kv_row), N * kv_row);
+    rows.hidden_in = static_cast<const uint16_t*>(at16(hidden_in, N * hidden_row));
+    rows.v_in = static_cast<const uint16_t*>(at16(v, N * kv_row));
+    rows.hidden_out = static_cast<uint16_t*>(at16(hidden_out, K * hidden_row));
+    rows.k_out = static_cast<uint16_t*>(at16(k_out, K * kv_row));
+    rows.v_out = static_cast<uint16_t*>(at16(v_out, K * kv_row));
+    rows.pos_out = static_cast<int32_t*>(at(pos_out, K * 4));
+    up.add(base + a.q, at(q, q_bytes), q_bytes);
+    up.add(base + a.q_idx, at(q_idx, R * 4), R * 4);
+    up.add(base + a.cu_qlens, at(cu_qlens, (B + 1) * 4), (B + 1) * 4);
+    up.add(base + a.cu_seqlens, at(cu_seqlens, (B + 1) * 4), (B + 1) * 4);
+    up.add(base + a.lse, at(lse_opt, R * p.num_q_heads * 4), R * p.num_q_heads * 4);
+    up.add(base + a.keep_counts, at(keep_counts, B * 4), B * 4);
+    up.add(base + a.protect, at(protect_opt, N), N);
+    up.add(base + a.pos, at(pos_in, N * 4), N * 4);
+    down.add(at(scores_out, N * 4), base + a.scores, N * 4);
+    down.add(at(keep_idx_out, K * 4), base + a.keep_idx, K * 4);
+    down.add(at(cu_keep_out, (B + 1) * 4), base + a.cu_keep, (B + 1) * 4);
+    down.add(at(status_out, 4), base + a.status, 4);
+    if (ok && K > 0) {
+      rows.k_in = reinterpret_cast<const uint16_t*>(base + a.k);
+      rows.pos_in = pos_in ? reinterpret_cast<const int32_t*>(base + a.pos) : nullptr;
+      int32_t* status = reinterpret_cast<int32_t*>(base + a.status);
+      const int32_t *d_cu_seqlens = reinterpret_cast<const int32_t*>(base + a.cu_seqlens);
+      int32_t *d_keep_idx = reinterpret_cast<int32_t*>(base + a.keep_idx), *d_cu_keep = reinterpret_cast<int32_t*>(base + a.cu_keep);
+      chain_begin(p.flags);
+      const int grid = (int)(up.pieces < 2 * kNumSMs ? (up.pieces > 0 ? up.pieces : 1) : 2 * kNumSMs);
+      cudaError_t e = launch_chained(host_upload_kernel, dim3(grid), dim3(kCopyThreads), 0, st, up, status, ChainHead{});
+      count_launches(1);
+      // The kernels that follow read the arrays this one uploads before their own wait, so the next one waits first too.
+      chain_begin(p.flags);
+      bool gathered = false;
+      if (e == cudaSuccess)
+        e = enqueue_selection(p, base + a.q, (const int32_t*)(base + a.q_idx), (const int32_t*)(base + a.cu_qlens), base + a.k, d_cu_seqlens,
+                              (const float*)dev(a.lse, lse_opt), (const int32_t*)(base + a.keep_counts),
+                              (const uint8_t*)dev(a.protect, protect_opt), nullptr, (float*)(base + a.scores), d_keep_idx, d_cu_keep,
+                              base + a.workspace, status, st, &gathered);
+      if (e == cudaSuccess) {
+        e = launch_chained(host_gather_kernel, dim3(kNumSMs), dim3(kCopyThreads), 0, st, make_shapes(p), rows, down, (const int32_t*)d_keep_idx,
+                           (const int32_t*)d_cu_keep, d_cu_seqlens);
+        count_launches(1);
+      }
+      return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? FASTAV_OK : FASTAV_ERR_CUDA;
+    }
+  }
   cudaError_t e = cudaSuccess;
   auto h2d = [&](size_t off, const void* src, size_t bytes) {
     if (e == cudaSuccess && src && bytes) e = cudaMemcpyAsync(base + off, src, bytes, cudaMemcpyHostToDevice, st);
