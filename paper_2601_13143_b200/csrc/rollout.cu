@@ -16,9 +16,17 @@
 // the causal mask RT is upper and A~ lower triangular: tiles above the diagonal are written as zeros and the
 // K loop of tile (m, n) only covers the blocks m..n.
 //
-// One CTA per 128 x 128 output tile: warp 0 issues the TMA loads, warp 1 the MMAs, warps 2..17 are the epilogue
-// (thread <-> accumulator row, four warps per 32-lane quarter of TMEM, 32 columns each: the epilogue, one
-// exponential per element, is what a tile costs, so it gets four warps per scheduler).  All waits are bounded.
+// All three kernels are PERSISTENT: the work of a layer is one flat list of items (a 128 x 128 tile of one head's logits;
+// 64 of the K range of one tile of the product), cut into as many equal runs as there are SMs.  A kernel with one block
+// per tile leaves half the chip idle at this size: 171 visible tiles of 28 heads are two rounds of blocks on 148 SMs, and
+// the longest chain of the triangular product alone is 15 us.  Where a run ends inside a tile, the tile's parts meet through
+// the workspace: the statistics as a few partial log-sum-exps per row, the sums as fp32 tiles that the block which finishes
+// last adds up in order (no block waits for another).  ROLLOUT_FIGURES
+//
+// Warp 0 issues the TMA loads, warp 1 the MMAs into a ring of accumulators in tensor memory, warps 2..17 are the
+// epilogue (thread <-> accumulator row, four warps per 32-lane quarter of TMEM, 32 columns each).  The epilogue of the
+// attention kernels, one exponential per element, is their bound: 16 per clock and SM from the special-function unit, so
+// two of every eight go through the FMA pipe instead, at the same precision (exp2_pair below).  All waits are bounded.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <limits.h>
@@ -34,15 +42,19 @@ constexpr int kTile = 128;
 constexpr int kThreads = 576;
 constexpr int kEpilogueThreads = 512;
 constexpr int kColGroups = 4;  // epilogue warps per TMEM quarter; each takes 32 of the 128 columns
-constexpr int kTmemCols = 256;  // two 128-column accumulators
-constexpr int kMaxStages = 6;
+constexpr int kTmemCols = 512;
+constexpr int kBuffers = 4;    // accumulators of 128 columns
+constexpr int kMaxStages = 4;
 constexpr int kSubTileBytes = kTile * 128;  // 128 rows of one 64-element (128-byte) column block
+constexpr int kMaxParts = 4;   // blocks that may share one row block's statistics
+constexpr size_t kPartialBytes = (size_t)kTile * kTile * sizeof(float);
 
 struct alignas(16) PipeControl {
-  uint64_t full[kMaxStages], empty[kMaxStages], tmem_full[2], tmem_empty[2];
+  uint64_t full[kMaxStages], empty[kMaxStages], tmem_full[kBuffers], tmem_empty[kBuffers], q_empty[2];
   uint32_t tmem_base;
   int abort;
-  float2 part[kColGroups - 1][kTile];  // statistics kernel: (max, sum) per row of column groups 1..3
+  int last;                               // this block finished the tile's last part
+  float2 part[2][kColGroups - 1][kTile];  // statistics kernel: (max, sum) per row of column groups 1..3
 };
 
 __device__ __forceinline__ void split_bf16(float x, __nv_bfloat16& hi, __nv_bfloat16& lo) {
@@ -62,16 +74,45 @@ __device__ __forceinline__ void store_split_row(const float (&x)[32], __nv_bfloa
   }
 }
 
+// 2^x for a pair of x <= ~0 on the FMA and integer pipes: x = n + f with n the nearest integer (read off the mantissa after
+// adding 1.5 * 2^23), a minimax polynomial of degree 5 for 2^f on [-1/2, 1/2] (Remez exchange on the relative error:
+// 7.5e-8, 2.3e-7 when evaluated in fp32, what the special-function unit has), and n added into the exponent field.
+// Inputs below -126 (including -inf) give about 2^-126.
+__device__ __forceinline__ float2 exp2_pair_fma(float2 x) {
+  const float kMagic = 12582912.f;
+  x.x = fmaxf(x.x, -126.f);
+  x.y = fmaxf(x.y, -126.f);
+  const float2 t = __fadd2_rn(x, make_float2(kMagic, kMagic));
+  const float2 n = __fadd2_rn(t, make_float2(-kMagic, -kMagic));
+  const float2 f = __ffma2_rn(n, make_float2(-1.f, -1.f), x);
+  float2 p = __ffma2_rn(f, make_float2(1.32764725e-3f, 1.32764725e-3f), make_float2(9.67554096e-3f, 9.67554096e-3f));
+  p = __ffma2_rn(p, f, make_float2(0.0555071309f, 0.0555071309f));
+  p = __ffma2_rn(p, f, make_float2(0.240221202f, 0.240221202f));
+  p = __ffma2_rn(p, f, make_float2(0.693146944f, 0.693146944f));
+  p = __ffma2_rn(p, f, make_float2(1.00000012f, 1.00000012f));
+  return make_float2(__int_as_float(__float_as_int(p.x) + (__float_as_int(t.x) << 23)),
+                     __int_as_float(__float_as_int(p.y) + (__float_as_int(t.y) << 23)));
+}
+#ifndef FASTAV_ROLLOUT_FMA
+#define FASTAV_ROLLOUT_FMA 0x88
+#endif
+// Of the 8 column pairs of every 16 columns, those of the mask take the FMA pipe.
+__device__ __forceinline__ float2 exp2_pair(float2 x, int pair) {
+  if ((FASTAV_ROLLOUT_FMA >> (pair & 7)) & 1) return exp2_pair_fma(x);
+  return make_float2(ptx::ex2_approx(x.x), ptx::ex2_approx(x.y));
+}
+
 __device__ __forceinline__ void pipe_setup(PipeControl& ctl, int stages, int warp, const void* map_a, const void* map_b) {
   if (threadIdx.x == 0) {
     for (int i = 0; i < stages; ++i) {
       ptx::mbar_init(ptx::smem_u32(&ctl.full[i]), 1);
       ptx::mbar_init(ptx::smem_u32(&ctl.empty[i]), 1);
     }
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < kBuffers; ++i) {
       ptx::mbar_init(ptx::smem_u32(&ctl.tmem_full[i]), 1);
       ptx::mbar_init(ptx::smem_u32(&ctl.tmem_empty[i]), kEpilogueThreads);
     }
+    for (int i = 0; i < 2; ++i) ptx::mbar_init(ptx::smem_u32(&ctl.q_empty[i]), 1);
     ctl.abort = 0;
     ptx::fence_barrier_init();
     ptx::prefetch_tensormap(map_a);
@@ -104,96 +145,199 @@ __device__ __forceinline__ void drain_loads(PipeControl& ctl, int issued, int st
     ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.full[t % stages]), (t / stages) & 1, &never);
 }
 
+__device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueThreads) : "memory"); }
+
+// ---- the flat list of items and its equal runs -------------------------------------------------------
+__device__ __forceinline__ long long run_begin(long long items, int blocks, int b) { return items * b / blocks; }
+// The block whose run holds item x.
+__device__ __forceinline__ int run_of(long long items, int blocks, long long x) {
+  int b = (int)((x * blocks) / items);
+  while (run_begin(items, blocks, b + 1) <= x) ++b;
+  while (run_begin(items, blocks, b) > x) --b;
+  return b;
+}
+// Largest r with r (r + 1) / 2 <= x.
+__device__ __forceinline__ int triangular_root(long long x) {
+  int r = (int)((sqrtf(8.f * (float)x + 1.f) - 1.f) * 0.5f);
+  while ((long long)(r + 1) * (r + 2) / 2 <= x) ++r;
+  while ((long long)r * (r + 1) / 2 > x) --r;
+  return r;
+}
+
+// A tile's sum is complete in `acc` (32 columns of one row per thread) of the block that gets true back.  The tile's items
+// are [first, end) of the list; a block that holds only part of them leaves its part in the workspace (at most two per
+// block: at the start and at the end of its run), and the last one to finish adds the parts up in the order of the runs.
+__device__ bool meet(PipeControl& ctl, float (&acc)[32], long long items, long long first, long long end, float* partials, int* counter,
+                     bool ok, int ethread) {
+  const int blocks = gridDim.x, me = blockIdx.x;
+  const int b0 = run_of(items, blocks, first), b1 = run_of(items, blocks, end - 1);
+  if (b0 == b1) return ok;
+  auto part_of = [&](int b) { return partials + (size_t)(2 * b + (first <= run_begin(items, blocks, b) ? 0 : 1)) * (kTile * kTile) + ethread; };
+  {
+    float* const mine = part_of(me);
+#pragma unroll
+    for (int c = 0; c < 32; ++c) __stcg(mine + c * kEpilogueThreads, acc[c]);
+  }
+  __threadfence();
+  epilogue_sync();
+  if (ethread == 0) ctl.last = atomicAdd(counter, 1) == b1 - b0 && !ctl.abort;
+  epilogue_sync();
+  const bool last = ctl.last != 0;
+  if (!last || !ok) return false;
+  __threadfence();
+  float total[32];
+#pragma unroll
+  for (int c = 0; c < 32; ++c) total[c] = 0.f;
+#pragma unroll 1
+  for (int b = b0; b <= b1; ++b) {
+    const float* const other = part_of(b);
+#pragma unroll
+    for (int c = 0; c < 32; ++c) total[c] += __ldcg(other + c * kEpilogueThreads);
+  }
+#pragma unroll
+  for (int c = 0; c < 32; ++c) acc[c] = total[c];
+  return true;
+}
+
 // ---- the attention map ---------------------------------------------------------------------------
 template <int DIM, int MODE>
 struct AttnSmem {
   static constexpr int kOperandBytes = (DIM / 64) * kSubTileBytes;
-  static constexpr int kSlots = MODE == 0 ? 1 : 3;
+  static constexpr int kSlots = MODE == 0 ? 2 : 3;
   static constexpr int kStages = 6 - kSlots;  // six tiles in all: 192 KB at head_dim 128
   static constexpr size_t kBytes = (size_t)6 * kOperandBytes + sizeof(PipeControl) + 1024;
 };
 
-// MODE 0: grid (row blocks, heads); the block walks the key blocks its rows may see and leaves, per row, the
-//         log2-sum-exp2 of the scaled logits of head blockIdx.y in lse2_out[head][row].
-// MODE 1: grid (row blocks, key blocks); the block walks the heads and accumulates the softmax weights of its
-//         128 x 128 tile, then applies Eq. 2 and stores the hi / lo planes (and, if asked, A itself in fp32).
+// One item: head, row block, key block.  MODE 0 walks the key blocks of a row block, then the row blocks of a head; MODE 1
+// the heads of a tile, then the tiles (key blocks of a row block).
+template <int MODE>
+struct Item {
+  int head, rb, jb, blocks, hq;
+  bool causal;
+  long long first;  // MODE 1: first item of the tile
+  __device__ Item(long long x, int blocks_, int hq_, bool causal_) : blocks(blocks_), hq(hq_), causal(causal_) {
+    const long long per_head = causal ? (long long)blocks * (blocks + 1) / 2 : (long long)blocks * blocks;
+    long long t;  // visible tile in row order
+    if (MODE == 0) {
+      head = (int)(x / per_head);
+      t = x % per_head;
+      first = 0;
+    } else {
+      t = x / hq;
+      head = (int)(x % hq);
+      first = t * hq;
+    }
+    rb = causal ? triangular_root(t) : (int)(t / blocks);
+    jb = (int)(t - (causal ? (long long)rb * (rb + 1) / 2 : (long long)rb * blocks));
+  }
+  __device__ __forceinline__ int last_jb() const { return causal ? rb : blocks - 1; }
+  __device__ __forceinline__ bool unit_ends() const { return MODE == 0 ? jb == last_jb() : head == hq - 1; }
+  __device__ __forceinline__ void advance() {
+    if (MODE == 1) {
+      if (++head < hq) return;
+      head = 0;
+      first += hq;
+    }
+    if (jb < last_jb()) {
+      ++jb;
+      return;
+    }
+    jb = 0;
+    if (++rb == blocks) {
+      rb = 0;
+      ++head;  // MODE 0 only: the list of MODE 1 ends here
+    }
+  }
+};
+
+struct AttnArgs {
+  int n, n_pad, hq, group;
+  float scale_log2;
+  int causal;
+  long long items;
+  float4* lse_parts;      // [hq][n_pad]: log2-sum-exp2 of up to four runs of a row's keys (-inf: no such run); MODE 0 writes, MODE 1 reads
+  int* counters;          // MODE 0 clears them: one per tile of the map and of the product
+  int n_counters;
+  const float* lse_opt;   // MODE 1, instead of lse_parts: the caller's natural logarithms [n][hq]
+  float alpha;
+  __nv_bfloat16 *a_hi, *a_lo;
+  float* map_out;
+  float* partials;
+  int32_t* device_status;
+};
+
+// MODE 0: per row and head, the log2-sum-exp2 of the scaled logits.
+// MODE 1: per 128 x 128 tile, the sum over the heads of the softmax weights; then Eq. 2, stored as hi / lo planes (and, if
+//         asked, A itself in fp32).
 template <int DIM, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
-rollout_attn_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map, int n, int n_pad,
-                    int hq, int group, float scale_log2, int causal, float* __restrict__ lse2_out,
-                    const float* __restrict__ lse, long long lse_row, long long lse_head, float lse_mult, float alpha,
-                    __nv_bfloat16* __restrict__ a_hi, __nv_bfloat16* __restrict__ a_lo, float* __restrict__ map_out,
-                    int32_t* device_status) {
-  // Shared memory: a ring of tiles of the operand that changes every iteration (MODE 0: the K tile of the key
-  // block; MODE 1: the Q tile of the head) and a few slots for the one that changes rarely (MODE 0: the Q tile,
-  // loaded once; MODE 1: the K tile, loaded once per KV head and shared by the G heads of its group -- three
-  // slots used in turn, so that a slot is overwritten no sooner than three iterations after its last use,
-  // which is the distance the ring's own barriers already guarantee).
+rollout_attn_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map, AttnArgs a, ChainHead head) {
+  // Shared memory: a ring of tiles of the operand that changes every item (MODE 0: K; MODE 1: Q) and a few slots for the
+  // one that changes rarely (MODE 0: Q, per row block, freed by the last MMA that reads it; MODE 1: K, per KV head and
+  // shared by the G heads of its group -- three slots used in turn, so that a slot is overwritten no sooner than three
+  // items after its last use, which is the distance the ring's own barriers already guarantee).
   using Cfg = AttnSmem<DIM, MODE>;
   constexpr int kStages = Cfg::kStages, kSlots = Cfg::kSlots;
   constexpr int kSubTiles = DIM / 64;
   constexpr int kOperandBytes = Cfg::kOperandBytes;  // one 128 x DIM tile
   extern __shared__ unsigned char smem_raw[];
+  chain_enter(head);
   const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t slots = base + kStages * kOperandBytes;
   PipeControl& ctl = *reinterpret_cast<PipeControl*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + (kStages + kSlots) * kOperandBytes);
   volatile int* abort = &ctl.abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int blocks = n_pad / kTile;
-  // Under the causal mask the last row block has the most key blocks to walk: the statistics kernel starts those first.
-  const int rb = (MODE == 0 && causal) ? blocks - 1 - (int)blockIdx.x : (int)blockIdx.x;
-
-  if (MODE == 1 && causal && (int)blockIdx.y > rb) {
-    // a tile no row may see: zeros (uniform for the block, before anything is set up)
-    for (int i = threadIdx.x; i < kTile * (kTile / 8); i += kThreads) {
-      const int r = i / (kTile / 8), c = (i % (kTile / 8)) * 8;
-      const long long at = (long long)(rb * kTile + r) * n_pad + blockIdx.y * kTile + c;
-      *reinterpret_cast<uint4*>(a_hi + at) = make_uint4(0, 0, 0, 0);
-      *reinterpret_cast<uint4*>(a_lo + at) = make_uint4(0, 0, 0, 0);
-    }
-    if (map_out)
-      for (int i = threadIdx.x; i < kTile * kTile; i += kThreads) {
-        const int r = rb * kTile + i / kTile, c = blockIdx.y * kTile + i % kTile;
-        if (r < n && c < n) map_out[(long long)r * n + c] = 0.f;
-      }
-    return;
-  }
-  const int iters = MODE == 0 ? (causal ? rb + 1 : blocks) : hq;
+  const int blocks = a.n_pad / kTile, group = a.group;
+  const long long begin = run_begin(a.items, gridDim.x, blockIdx.x), end = run_begin(a.items, gridDim.x, blockIdx.x + 1);
+  const int count = (int)(end - begin);
 
   pipe_setup(ctl, kStages, warp, &q_map, &k_map);
   const uint32_t tmem = ctl.tmem_base;
 
   if (warp == 0) {
     if (lane == 0) {
-      int it = 0;
-      for (; it < iters; ++it) {
+      pdl_wait();  // q and k may be what earlier work wrote
+      Item<MODE> x(begin, blocks, a.hq, a.causal != 0);
+      int it = 0, loads = 0;  // items, tiles of the operand that changes rarely
+      for (; it < count; ++it) {
         const int stage = it % kStages;
         if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.empty[stage]), ((it / kStages) & 1) ^ 1u, abort)) break;
-        const int head = MODE == 0 ? (int)blockIdx.y : it, jb = MODE == 0 ? it : (int)blockIdx.y;
+        const bool load_slot = it == 0 || (MODE == 0 ? x.jb == 0 : x.head % group == 0);
+        const uint32_t slot = slots + (loads % kSlots) * kOperandBytes;
+        if (MODE == 0 && load_slot &&
+            !ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.q_empty[loads & 1]), ((loads >> 1) & 1) ^ 1u, abort))
+          break;
         const uint32_t bar = ptx::smem_u32(&ctl.full[stage]);
-        const bool load_q = MODE == 1 || it == 0, load_k = MODE == 0 || it % group == 0;
         const uint32_t ring = base + stage * kOperandBytes;
-        const uint32_t q_dst = MODE == 0 ? slots : ring;
-        const uint32_t k_dst = MODE == 0 ? ring : slots + ((it / group) % kSlots) * kOperandBytes;
-        ptx::mbar_arrive_expect_tx(bar, (load_q ? kOperandBytes : 0) + (load_k ? kOperandBytes : 0));
+        ptx::mbar_arrive_expect_tx(bar, kOperandBytes + (load_slot ? kOperandBytes : 0));
 #pragma unroll
         for (int sub = 0; sub < kSubTiles; ++sub) {
-          if (load_q) ptx::tma_load_3d(q_dst + sub * kSubTileBytes, &q_map, sub * 64, head, rb * kTile, bar);
-          if (load_k) ptx::tma_load_3d(k_dst + sub * kSubTileBytes, &k_map, sub * 64, head / group, jb * kTile, bar);
+          const uint32_t at = sub * kSubTileBytes;
+          if (MODE == 0) {
+            if (load_slot) ptx::tma_load_3d(slot + at, &q_map, sub * 64, x.head, x.rb * kTile, bar);
+            ptx::tma_load_3d(ring + at, &k_map, sub * 64, x.head / group, x.jb * kTile, bar);
+          } else {
+            if (load_slot) ptx::tma_load_3d(slot + at, &k_map, sub * 64, x.head / group, x.jb * kTile, bar);
+            ptx::tma_load_3d(ring + at, &q_map, sub * 64, x.head, x.rb * kTile, bar);
+          }
         }
+        loads += load_slot;
+        x.advance();
       }
       if (*abort) drain_loads(ctl, it, kStages);
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      for (int it = 0; it < iters; ++it) {
-        const int stage = it % kStages, buf = it & 1;
+      Item<MODE> x(begin, blocks, a.hq, a.causal != 0);
+      int loads = 0;
+      for (int it = 0; it < count; ++it) {
+        const int stage = it % kStages, buf = it % kBuffers;
         if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort)) break;
-        if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_empty[buf]), ((it >> 1) & 1) ^ 1u, abort)) break;
+        if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_empty[buf]), ((it / kBuffers) & 1) ^ 1u, abort)) break;
         ptx::tc_fence_after_sync();
-        const uint32_t ring = base + stage * kOperandBytes;
-        const uint32_t q_tile = MODE == 0 ? slots : ring;
-        const uint32_t k_tile = MODE == 0 ? ring : slots + ((it / group) % kSlots) * kOperandBytes;
+        loads += it == 0 || (MODE == 0 ? x.jb == 0 : x.head % group == 0);
+        const uint32_t ring = base + stage * kOperandBytes, slot = slots + ((loads - 1) % kSlots) * kOperandBytes;
+        const uint32_t q_tile = MODE == 0 ? slot : ring, k_tile = MODE == 0 ? ring : slot;
 #pragma unroll
         for (int ks = 0; ks < DIM / 16; ++ks) {
           const uint32_t sub = ks / 4, off = (ks % 4) * 32;
@@ -202,174 +346,266 @@ rollout_attn_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
         }
         ptx::umma_commit(ptx::smem_u32(&ctl.empty[stage]));
         ptx::umma_commit(ptx::smem_u32(&ctl.tmem_full[buf]));
+        if (MODE == 0 && x.unit_ends()) ptx::umma_commit(ptx::smem_u32(&ctl.q_empty[(loads - 1) & 1]));
+        x.advance();
       }
     }
   } else {
     const int quarter = warp & 3, cg = (warp - 2) >> 2;  // TMEM lanes 32 quarter .., columns 32 cg ..
-    const int row_in = quarter * 32 + lane, row = rb * kTile + row_in;
-    const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16);
-    const int last_visible = min(n - 1, causal ? row : INT_MAX);
-    float zmax = -INFINITY, sum = 0.f;  // MODE 0, in scaled log2 units
-    float acc[32];                      // MODE 1
+    const int row_in = quarter * 32 + lane, ethread = cg * kTile + row_in;
+    const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16) + cg * 32;
+    pdl_wait();
+    float4* lse_parts = a.lse_parts;
+    const float* lse_opt = a.lse_opt;
+    pdl_acquire(lse_parts);
+    pdl_acquire(lse_opt);
+    if (MODE == 0)
+      for (int i = blockIdx.x * kEpilogueThreads + ethread; i < a.n_counters; i += gridDim.x * kEpilogueThreads) a.counters[i] = 0;
+    Item<MODE> x(begin, blocks, a.hq, a.causal != 0);
+    float zmax = -INFINITY;                             // MODE 0, unscaled
+    float2 sum2 = make_float2(0.f, 0.f);
+    float2 acc2[16];                                    // MODE 1
 #pragma unroll
-    for (int c = 0; c < 32; ++c) acc[c] = 0.f;
+    for (int c = 0; c < 16; ++c) acc2[c] = make_float2(0.f, 0.f);
+    const float scale = a.scale_log2;
+    const float2 sc = make_float2(scale, scale);
+    // MODE 1: a row's statistic of one head; the NEXT item's is fetched while this one is worked on.
+    auto fetch = [&](const Item<MODE>& at) -> float4 {
+      const int row = at.rb * kTile + row_in;
+      if (lse_opt) return make_float4(row < a.n ? __ldcg(lse_opt + (long long)row * a.hq + at.head) * kLog2e : 0.f, -INFINITY, -INFINITY, -INFINITY);
+      return __ldcg(lse_parts + (long long)at.head * a.n_pad + row);
+    };
+    float4 stat_next = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (MODE == 1 && count > 0) stat_next = fetch(x);
+    int turn = 0;  // MODE 0: which half of the exchange buffer
     bool ok = true;
-    // MODE 1: the row's statistic of the NEXT head is fetched while this head's tile is worked on
-    float lse_next = (MODE == 1 && row < n) ? lse[row * lse_row] : 0.f;
-    for (int it = 0; it < iters; ++it) {
-      const int buf = it & 1;
-      const float lse_here = lse_next;
-      if (MODE == 1 && row < n && it + 1 < iters) lse_next = lse[row * lse_row + (it + 1) * lse_head];
-      ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_full[buf]), (it >> 1) & 1, abort);
-      if (!ok) break;
-      ptx::tc_fence_after_sync();
-      const int jb = MODE == 0 ? it : (int)blockIdx.y;
-      uint32_t v[32];
-      ptx::tmem_ld32(lane_addr + buf * kTile + cg * 32, v);
-      ptx::tmem_ld_wait_for(v);
-      ptx::tc_fence_before_sync();
-      ptx::mbar_arrive(ptx::smem_u32(&ctl.tmem_empty[buf]));  // the accumulator may be overwritten
-      const int limit = last_visible - (jb * kTile + cg * 32);  // columns 0..limit of this group are visible
-      if (limit < 0) continue;
-      const bool whole = limit >= 31;  // the usual case; only tiles on the diagonal or at the end of the sequence are cut
-      if constexpr (MODE == 0) {
-        float tile_max = -INFINITY;
-        if (whole) {
-#pragma unroll
-          for (int c = 0; c < 32; ++c) tile_max = fmaxf(tile_max, __uint_as_float(v[c]));
-        } else {
-#pragma unroll
-          for (int c = 0; c < 32; ++c)
-            if (c <= limit) tile_max = fmaxf(tile_max, __uint_as_float(v[c]));
+#pragma unroll 1
+    for (int it = 0; it < count; ++it) {
+      const int buf = it % kBuffers;
+      const Item<MODE> here = x;
+      x.advance();
+      float neg_lse2 = 0.f;
+      if (MODE == 1) {
+        const float4 st = stat_next;
+        if (it + 1 < count) stat_next = fetch(x);
+        float lse2 = st.x;
+        if (__any_sync(0xFFFFFFFFu, st.y > -INFINITY)) {  // the row block's statistics come from several runs
+          const float m = fmaxf(fmaxf(st.x, st.y), fmaxf(st.z, st.w));
+          const float t = ptx::ex2_approx(st.x - m) + ptx::ex2_approx(st.y - m) + ptx::ex2_approx(st.z - m) + ptx::ex2_approx(st.w - m);
+          lse2 = m > -INFINITY ? m + log2f(t) : -INFINITY;
         }
-        const float new_max = fmaxf(zmax, tile_max * scale_log2);
-        float add0 = 0.f, add1 = 0.f;
-        if (whole) {
+        neg_lse2 = lse2 > -INFINITY ? -lse2 : -INFINITY;  // a row that sees nothing adds 0
+      }
+      if (ok) ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_full[buf]), (it / kBuffers) & 1, abort);
+      if (ok) {
+        ptx::tc_fence_after_sync();
+        uint32_t v[32];
+        ptx::tmem_ld32(lane_addr + buf * kTile, v);
+        ptx::tmem_ld_wait_for(v);
+        ptx::tc_fence_before_sync();
+        ptx::mbar_arrive(ptx::smem_u32(&ctl.tmem_empty[buf]));  // the accumulator may be overwritten
+        const int row = here.rb * kTile + row_in;
+        const int last_visible = min(a.n - 1, a.causal ? row : INT_MAX);
+        const int limit = last_visible - (here.jb * kTile + cg * 32);  // columns 0..limit of this group are visible
+        const bool whole = limit >= 31;  // the usual case; only tiles on the diagonal or at the end of the sequence are cut
+        if constexpr (MODE == 0) {
+          if (limit >= 0) {
+            if (!whole) {
 #pragma unroll
-          for (int c = 0; c < 32; c += 2) {
-            add0 += ptx::ex2_approx(fmaf(__uint_as_float(v[c]), scale_log2, -new_max));
-            add1 += ptx::ex2_approx(fmaf(__uint_as_float(v[c + 1]), scale_log2, -new_max));
+              for (int c = 0; c < 32; ++c)
+                if (c > limit) v[c] = 0xFF800000u;  // -inf
+            }
+            float m = zmax;
+#pragma unroll
+            for (int c = 0; c < 32; c += 2) m = fmaxf(m, fmaxf(__uint_as_float(v[c]), __uint_as_float(v[c + 1])));
+            const float corr = ptx::ex2_approx((zmax - m) * scale);  // 0 the first time
+            sum2.x *= corr;
+            sum2.y *= corr;
+            zmax = m;
+            const float shift = -m * scale;
+            const float2 sh = make_float2(shift, shift);
+#pragma unroll
+            for (int c = 0; c < 32; c += 2)
+              sum2 = __fadd2_rn(sum2, exp2_pair(__ffma2_rn(make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc, sh), c / 2));
           }
+          __syncwarp();  // the rows of a warp differ in `limit`; the tcgen05 instructions that follow need the whole warp
         } else {
+          const float2 nl = make_float2(neg_lse2, neg_lse2);
+          if (whole) {
 #pragma unroll
-          for (int c = 0; c < 32; ++c)
-            if (c <= limit) add0 += ptx::ex2_approx(fmaf(__uint_as_float(v[c]), scale_log2, -new_max));
+            for (int c = 0; c < 32; c += 2)
+              acc2[c / 2] = __fadd2_rn(acc2[c / 2], exp2_pair(__ffma2_rn(make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc, nl), c / 2));
+          } else if (limit >= 0) {
+#pragma unroll
+            for (int c = 0; c < 32; c += 2) {
+              const float2 p = exp2_pair(__ffma2_rn(make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc, nl), c / 2);
+              acc2[c / 2].x += c <= limit ? p.x : 0.f;
+              acc2[c / 2].y += c + 1 <= limit ? p.y : 0.f;
+            }
+          }
+          __syncwarp();
         }
-        sum = sum * ptx::ex2_approx(zmax - new_max) + (add0 + add1);  // zmax = -inf the first time: the factor is 0
-        zmax = new_max;
+      }
+      const bool unit_ends = here.unit_ends();
+      if (!unit_ends && it + 1 < count) continue;
+      // ---- the end of a row block's keys (MODE 0) or of a tile's heads (MODE 1), or of this block's run ------------
+      if constexpr (MODE == 0) {
+        if (cg > 0) ctl.part[turn][cg - 1][row_in] = make_float2(zmax, sum2.x + sum2.y);
+        epilogue_sync();
+        if (cg == 0 && ok) {
+          float m = zmax;
+#pragma unroll
+          for (int g = 0; g < kColGroups - 1; ++g) m = fmaxf(m, ctl.part[turn][g][row_in].x);
+          float total = zmax > -INFINITY ? (sum2.x + sum2.y) * ptx::ex2_approx((zmax - m) * scale) : 0.f;
+#pragma unroll
+          for (int g = 0; g < kColGroups - 1; ++g) {
+            const float2 other = ctl.part[turn][g][row_in];
+            if (other.x > -INFINITY) total += other.y * ptx::ex2_approx((other.x - m) * scale);
+          }
+          const float value = total > 0.f ? m * scale + log2f(total) : -INFINITY;
+          // which of the row block's runs this is: the one after those of the blocks before
+          const long long first_item = begin + it - here.jb;
+          const int part = blockIdx.x - run_of(a.items, gridDim.x, first_item);
+          float* const out = reinterpret_cast<float*>(lse_parts + (long long)here.head * a.n_pad + here.rb * kTile + row_in);
+          if (part < kMaxParts) out[part] = value;
+          if (unit_ends)
+            for (int p = part + 1; p < kMaxParts; ++p) out[p] = -INFINITY;
+        }
+        turn ^= 1;
+        zmax = -INFINITY;
+        sum2 = make_float2(0.f, 0.f);
       } else {
-        const float neg_lse2 = -lse_here * lse_mult;
-        if (whole) {
+        float acc[32];
 #pragma unroll
-          for (int c = 0; c < 32; ++c) acc[c] += ptx::ex2_approx(fmaf(__uint_as_float(v[c]), scale_log2, neg_lse2));
-        } else {
+        for (int c = 0; c < 16; ++c) {
+          acc[2 * c] = acc2[c].x;
+          acc[2 * c + 1] = acc2[c].y;
+          acc2[c] = make_float2(0.f, 0.f);
+        }
+        if (meet(ctl, acc, a.items, here.first, here.first + a.hq, a.partials, a.counters + here.rb * blocks + here.jb, ok, ethread)) {
+          const int row = here.rb * kTile + row_in, col0 = here.jb * kTile + cg * 32;
+          const float inv_heads = 1.0f / (float)a.hq;
 #pragma unroll
-          for (int c = 0; c < 32; ++c)
-            if (c <= limit) acc[c] += ptx::ex2_approx(fmaf(__uint_as_float(v[c]), scale_log2, neg_lse2));
+          for (int c = 0; c < 32; ++c) {
+            const float weight = row < a.n ? acc[c] * inv_heads : 0.f;
+            if (a.map_out && row < a.n && col0 + c < a.n) a.map_out[(long long)row * a.n + col0 + c] = weight;
+            acc[c] = a.alpha * weight + ((row < a.n && col0 + c == row) ? 1.0f - a.alpha : 0.f);  // Eq. 2
+          }
+          const long long at = (long long)row * a.n_pad + col0;
+          store_split_row(acc, a.a_hi + at, a.a_lo + at);
         }
       }
     }
-    if constexpr (MODE == 0) {
-      // the four column groups of a row meet in shared memory; group 0 writes the result
-      if (cg > 0) ctl.part[cg - 1][row_in] = make_float2(zmax, sum);
-      asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueThreads) : "memory");
-      if (cg == 0 && ok && !*abort) {
-        float m = zmax;
-#pragma unroll
-        for (int g = 0; g < kColGroups - 1; ++g) m = fmaxf(m, ctl.part[g][row_in].x);
-        float total = zmax > -INFINITY ? sum * ptx::ex2_approx(zmax - m) : 0.f;
-#pragma unroll
-        for (int g = 0; g < kColGroups - 1; ++g) {
-          const float2 other = ctl.part[g][row_in];
-          if (other.x > -INFINITY) total += other.y * ptx::ex2_approx(other.x - m);
+    if (MODE == 1 && a.map_out && a.causal) {  // tiles no row may see (of the planes the product reads only the others)
+      for (int t = blockIdx.x; t < blocks * blocks; t += gridDim.x) {
+        const int rb = t / blocks, jb = t % blocks;
+        if (jb <= rb) continue;
+        for (int i = ethread; i < kTile * kTile; i += kEpilogueThreads) {
+          const int r = rb * kTile + i / kTile, c = jb * kTile + i % kTile;
+          if (r < a.n && c < a.n) a.map_out[(long long)r * a.n + c] = 0.f;
         }
-        lse2_out[(long long)blockIdx.y * n_pad + row] = total > 0.f ? m + log2f(total) : INFINITY;  // a row that sees nothing adds 0
       }
-    } else if (ok) {
-      const int col0 = blockIdx.y * kTile + cg * 32;
-      const float inv_heads = 1.0f / (float)hq;
-      float x[32];
-#pragma unroll
-      for (int c = 0; c < 32; ++c) {
-        const float a = row < n ? acc[c] * inv_heads : 0.f;
-        if (map_out && row < n && col0 + c < n) map_out[(long long)row * n + col0 + c] = a;
-        x[c] = alpha * a + ((row < n && col0 + c == row) ? 1.0f - alpha : 0.f);  // Eq. 2
-      }
-      const long long at = (long long)row * n_pad + col0;
-      store_split_row(x, a_hi + at, a_lo + at);
     }
   }
-  pipe_teardown(ctl, warp, device_status);
+  pipe_teardown(ctl, warp, a.device_status);
 }
 
 // ---- Eq. 3: RT_new = RT_old * A~^T ------------------------------------------------------------------
-// Grid (n_pad / 128, n_pad / 128): one block per 128 x 128 tile of RT_new.  Per 64-wide K block the four
-// operand tiles (RT hi, RT lo, A~ hi, A~ lo) are loaded once and used for the three products
-// RT hi * A~ hi, RT lo * A~ hi, RT hi * A~ lo, all accumulated into the same TMEM tile.
+// One item: a 64-wide K block of one 128 x 128 tile of RT_new.  Its four operand tiles (RT hi, RT lo, A~ hi, A~ lo) are
+// loaded once and used for the three products RT hi * A~ hi, RT lo * A~ hi, RT hi * A~ lo, all accumulated into the same
+// TMEM tile.  Under the causal mask RT is upper and A~ lower triangular: tile (m, nn) has the K blocks m .. nn only.
+struct GemmItem {
+  int mb, nb, kb, blocks;  // kb: 64-wide K block
+  bool causal;
+  long long first;         // first item of the tile
+  __device__ GemmItem(long long x, int blocks_, bool causal_) : blocks(blocks_), causal(causal_) {
+    mb = 0;
+    first = 0;
+    if (causal) {
+      for (;;) {  // row mb holds 2 (1 + 2 + ... + (blocks - mb)) items
+        const long long row = (long long)(blocks - mb) * (blocks - mb + 1);
+        if (x < first + row) break;
+        first += row;
+        ++mb;
+      }
+      const long long r = (x - first) / 2;
+      const int d = triangular_root(r);
+      first += (long long)d * (d + 1);
+      nb = mb + d;
+      kb = 2 * mb + (int)(x - first);
+    } else {
+      const long long tile = x / (2 * blocks);
+      mb = (int)(tile / blocks);
+      nb = (int)(tile % blocks);
+      first = tile * 2 * blocks;
+      kb = (int)(x - first);
+    }
+  }
+  __device__ __forceinline__ int kb_first() const { return causal ? 2 * mb : 0; }
+  __device__ __forceinline__ int kb_last() const { return causal ? 2 * nb + 1 : 2 * blocks - 1; }
+  __device__ __forceinline__ long long tile_end() const { return first + kb_last() - kb_first() + 1; }
+  __device__ __forceinline__ void advance() {
+    if (kb < kb_last()) {
+      ++kb;
+      return;
+    }
+    first = tile_end();
+    if (++nb == blocks) {
+      ++mb;
+      nb = causal ? mb : 0;
+    }
+    kb = kb_first();
+  }
+};
+
 __global__ void __launch_bounds__(kThreads, 1)
 rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_constant__ CUtensorMap rt_lo_map,
                     const __grid_constant__ CUtensorMap a_hi_map, const __grid_constant__ CUtensorMap a_lo_map, int n_pad,
-                    int causal, __nv_bfloat16* __restrict__ out_hi, __nv_bfloat16* __restrict__ out_lo, int32_t* device_status) {
+                    int causal, long long items, int clear, __nv_bfloat16* __restrict__ out_hi, __nv_bfloat16* __restrict__ out_lo,
+                    float* partials, int* counters, int32_t* device_status, ChainHead head) {
   constexpr int kStages = 3;
   constexpr int kStageBytes = 4 * kSubTileBytes;  // 128 x 64 each of RT hi, RT lo, A~ hi, A~ lo
   extern __shared__ unsigned char smem_raw[];
+  chain_enter(head);
   const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   PipeControl& ctl = *reinterpret_cast<PipeControl*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + kStages * kStageBytes);
   volatile int* abort = &ctl.abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // Tile of this block.  Under the causal mask tile (m, nn) has a K loop of nn - m + 1 blocks: the blocks are handed
-  // out by decreasing nn - m (longest first, so that the short ones fill the tail), the all-zero tiles last.
-  int mb = blockIdx.x, nb = blockIdx.y;
-  if (causal) {
-    const int blocks = gridDim.x;
-    int id = blockIdx.y * blocks + blockIdx.x, diag = blocks - 1;  // diag = nn - m, from blocks - 1 down to -(blocks - 1)
-    while (id >= blocks - abs(diag)) {
-      id -= blocks - abs(diag);
-      --diag;
-    }
-    mb = diag >= 0 ? id : id - diag;
-    nb = mb + diag;
-  }
-
-  if (causal && mb > nb) {  // RT is upper triangular: nothing but zeros here
-    for (int i = threadIdx.x; i < kTile * (kTile / 8); i += kThreads) {
-      const int r = i / (kTile / 8), c = (i % (kTile / 8)) * 8;
-      const long long at = (long long)(mb * kTile + r) * n_pad + nb * kTile + c;
-      *reinterpret_cast<uint4*>(out_hi + at) = make_uint4(0, 0, 0, 0);
-      *reinterpret_cast<uint4*>(out_lo + at) = make_uint4(0, 0, 0, 0);
-    }
-    return;
-  }
-  // 64-wide K blocks: RT[m][k] is zero for k < m, A~[nn][k] for k > nn
-  const int kb_lo = causal ? mb * 2 : 0, kb_hi = causal ? (nb + 1) * 2 : n_pad / 64;
-  const int iters = kb_hi - kb_lo;
+  const int blocks = n_pad / kTile;
+  const long long begin = run_begin(items, gridDim.x, blockIdx.x), end = run_begin(items, gridDim.x, blockIdx.x + 1);
+  const int count = (int)(end - begin);
 
   pipe_setup(ctl, kStages, warp, &rt_hi_map, &a_hi_map);
   const uint32_t tmem = ctl.tmem_base;
 
   if (warp == 0) {
     if (lane == 0) {
+      pdl_wait();
+      GemmItem x(begin, blocks, causal != 0);
       int it = 0;
-      for (; it < iters; ++it) {
+      for (; it < count; ++it) {
         const int stage = it % kStages;
         if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.empty[stage]), ((it / kStages) & 1) ^ 1u, abort)) break;
-        const int kb = kb_lo + it;
         const uint32_t bar = ptx::smem_u32(&ctl.full[stage]);
         const uint32_t dst = base + stage * kStageBytes;
         ptx::mbar_arrive_expect_tx(bar, kStageBytes);
-        ptx::tma_load_2d(dst, &rt_hi_map, kb * 64, mb * kTile, bar);
-        ptx::tma_load_2d(dst + kSubTileBytes, &rt_lo_map, kb * 64, mb * kTile, bar);
-        ptx::tma_load_2d(dst + 2 * kSubTileBytes, &a_hi_map, kb * 64, nb * kTile, bar);
-        ptx::tma_load_2d(dst + 3 * kSubTileBytes, &a_lo_map, kb * 64, nb * kTile, bar);
+        ptx::tma_load_2d(dst, &rt_hi_map, x.kb * 64, x.mb * kTile, bar);
+        ptx::tma_load_2d(dst + kSubTileBytes, &rt_lo_map, x.kb * 64, x.mb * kTile, bar);
+        ptx::tma_load_2d(dst + 2 * kSubTileBytes, &a_hi_map, x.kb * 64, x.nb * kTile, bar);
+        ptx::tma_load_2d(dst + 3 * kSubTileBytes, &a_lo_map, x.kb * 64, x.nb * kTile, bar);
+        x.advance();
       }
       if (*abort) drain_loads(ctl, it, kStages);
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      bool ok = true;
-      for (int it = 0; it < iters && ok; ++it) {
-        const int stage = it % kStages;
-        ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort);
+      GemmItem x(begin, blocks, causal != 0);
+      int tile = 0;  // tiles (or parts of one) begun by this block
+      bool fresh = true, ok = true;
+      for (int it = 0; it < count && ok; ++it) {
+        const int stage = it % kStages, buf = tile % kBuffers;
+        if (fresh) ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_empty[buf]), ((tile / kBuffers) & 1) ^ 1u, abort);
+        if (ok) ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort);
         if (!ok) break;
         ptx::tc_fence_after_sync();
         const uint32_t rt_hi = base + stage * kStageBytes, rt_lo = rt_hi + kSubTileBytes, a_hi = rt_hi + 2 * kSubTileBytes,
@@ -379,27 +615,64 @@ rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_
           const uint32_t rt_tile = term == 1 ? rt_lo : rt_hi, a_tile = term == 2 ? a_lo : a_hi;
 #pragma unroll
           for (int ks = 0; ks < 4; ++ks)
-            ptx::umma_bf16(tmem, ptx::umma_desc_sw128(rt_tile, ks * 32), ptx::umma_desc_sw128(a_tile, ks * 32),
-                           ptx::umma_idesc_bf16(kTile, kTile), (it > 0 || term > 0 || ks > 0) ? 1u : 0u);
+            ptx::umma_bf16(tmem + buf * kTile, ptx::umma_desc_sw128(rt_tile, ks * 32), ptx::umma_desc_sw128(a_tile, ks * 32),
+                           ptx::umma_idesc_bf16(kTile, kTile), (!fresh || term > 0 || ks > 0) ? 1u : 0u);
         }
         ptx::umma_commit(ptx::smem_u32(&ctl.empty[stage]));
+        fresh = x.kb == x.kb_last() || it + 1 == count;
+        if (fresh) {
+          ptx::umma_commit(ptx::smem_u32(&ctl.tmem_full[buf]));
+          ++tile;
+        }
+        x.advance();
       }
-      if (ok) ptx::umma_commit(ptx::smem_u32(&ctl.tmem_full[0]));
     }
   } else {
     const int quarter = warp & 3, cg = (warp - 2) >> 2;
-    const int row = mb * kTile + quarter * 32 + lane;
-    if (ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_full[0]), 0, abort)) {
-      ptx::tc_fence_after_sync();
-      uint32_t v[32];
-      ptx::tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + cg * 32, v);
-      ptx::tmem_ld_wait_for(v);
-      float x[32];
+    const int row_in = quarter * 32 + lane, ethread = cg * kTile + row_in;
+    pdl_wait();
+    bool ok = true;
+    GemmItem x(begin, blocks, causal != 0);
+    int tile = 0;
+#pragma unroll 1
+    for (long long at = begin; at < end; ++tile) {
+      const long long tile_end = x.tile_end();
+      const int buf = tile % kBuffers;
+      if (ok) ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_full[buf]), (tile / kBuffers) & 1, abort);
+      float acc[32];
+      if (ok) {
+        ptx::tc_fence_after_sync();
+        uint32_t v[32];
+        ptx::tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + buf * kTile + cg * 32, v);
+        ptx::tmem_ld_wait_for(v);
+        ptx::tc_fence_before_sync();
+        ptx::mbar_arrive(ptx::smem_u32(&ctl.tmem_empty[buf]));
 #pragma unroll
-      for (int c = 0; c < 32; ++c) x[c] = __uint_as_float(v[c]);
-      const long long at = (long long)row * n_pad + nb * kTile + cg * 32;
-      store_split_row(x, out_hi + at, out_lo + at);
+        for (int c = 0; c < 32; ++c) acc[c] = __uint_as_float(v[c]);
+      } else {
+#pragma unroll
+        for (int c = 0; c < 32; ++c) acc[c] = 0.f;
+      }
+      if (meet(ctl, acc, items, x.first, tile_end, partials, counters + x.mb * blocks + x.nb, ok, ethread)) {
+        const long long out = (long long)(x.mb * kTile + row_in) * n_pad + x.nb * kTile + cg * 32;
+        store_split_row(acc, out_hi + out, out_lo + out);
+      }
+      __syncwarp();
+      at = tile_end;
+      x.kb = x.kb_last();
+      x.advance();
     }
+    if (clear)  // RT is upper triangular: nothing but zeros below (later layers leave them as they are)
+      for (int t = blockIdx.x; t < blocks * blocks; t += gridDim.x) {
+        const int mb = t / blocks, nb = t % blocks;
+        if (mb <= nb) continue;
+        for (int i = ethread; i < kTile * (kTile / 8); i += kEpilogueThreads) {
+          const int r = i / (kTile / 8), c = (i % (kTile / 8)) * 8;
+          const long long out = (long long)(mb * kTile + r) * n_pad + nb * kTile + c;
+          *reinterpret_cast<uint4*>(out_hi + out) = make_uint4(0, 0, 0, 0);
+          *reinterpret_cast<uint4*>(out_lo + out) = make_uint4(0, 0, 0, 0);
+        }
+      }
   }
   pipe_teardown(ctl, warp, device_status);
 }
@@ -508,36 +781,89 @@ __nv_bfloat16* state_plane(void* state, int n, int copy, int lo) {
   return reinterpret_cast<__nv_bfloat16*>(static_cast<unsigned char*>(state) + (size_t)(copy * 2 + lo) * plane_bytes(n));
 }
 
+// ---- runs and workspace: the same on both sides ----------------------------------------------------------
+long long visible_tiles(int blocks, bool causal) { return causal ? (long long)blocks * (blocks + 1) / 2 : (long long)blocks * blocks; }
+long long attn_items(int blocks, int hq, bool causal) { return visible_tiles(blocks, causal) * hq; }
+long long gemm_items(int blocks, bool causal) {  // causal: sum over the rows of 2 (1 + ... + (blocks - mb))
+  return causal ? (long long)blocks * (blocks + 1) * (blocks + 2) / 3 : 2ll * blocks * blocks * blocks;
+}
+// Blocks: one per SM unless the runs would get too short.  A row block's statistics may come from at most kMaxParts runs
+// (a run of at least a third of the longest row block); a tile's sum from any number, but each part costs an exchange of
+// 64 KB, so a run has at least six tiles of logits or four K blocks.
+int grid_for(long long items, long long shortest_run) {
+  const long long g = items / shortest_run;
+  return (int)(g < 1 ? 1 : g > kNumSMs ? kNumSMs : g);
+}
+int stats_grid(int blocks, int hq, bool causal) { return grid_for(attn_items(blocks, hq, causal), (blocks + 2) / 3); }
+int map_grid(int blocks, int hq, bool causal) { return grid_for(attn_items(blocks, hq, causal), 6); }
+int gemm_grid(int blocks, bool causal) { return grid_for(gemm_items(blocks, causal), 4); }
+
+struct RolloutWorkspace {
+  size_t a_hi, a_lo, lse_parts, partials, counters, total;
+  int n_counters;
+};
+RolloutWorkspace plan_rollout(int n, int hq) {
+  RolloutWorkspace w{};
+  const int blocks = pad_of(n) / kTile;
+  int grid = 0;  // over both masks
+  for (int causal = 0; causal < 2; ++causal) {
+    const int m = map_grid(blocks, hq, causal != 0), g = gemm_grid(blocks, causal != 0);
+    grid = m > grid ? m : grid;
+    grid = g > grid ? g : grid;
+  }
+  size_t off = 0;
+  auto carve = [&](size_t bytes) { const size_t at = off; off = align_up(off + bytes, 256); return at; };
+  w.a_hi = carve(plane_bytes(n));
+  w.a_lo = carve(plane_bytes(n));
+  w.lse_parts = carve((size_t)hq * pad_of(n) * sizeof(float4));
+  w.partials = carve((size_t)2 * grid * kPartialBytes);
+  w.n_counters = 2 * blocks * blocks;  // the map's tiles, then the product's
+  w.counters = carve((size_t)w.n_counters * sizeof(int));
+  w.total = off;
+  return w;
+}
+
 template <int DIM>
-cudaError_t run_layer(const fastav_params& p, const CUtensorMap& q_map, const CUtensorMap& k_map, const float* lse_opt,
-                      float alpha, float* lse2, __nv_bfloat16* a_hi, __nv_bfloat16* a_lo, float* map_out,
-                      int32_t* device_status, cudaStream_t stream) {
+cudaError_t run_layer(const fastav_params& p, const CUtensorMap& q_map, const CUtensorMap& k_map, const float* lse_opt, float alpha,
+                      const RolloutWorkspace& w, unsigned char* ws, float* map_out, int32_t* device_status, cudaStream_t stream) {
   constexpr size_t smem = AttnSmem<DIM, 0>::kBytes;
   static_assert(AttnSmem<DIM, 0>::kBytes == AttnSmem<DIM, 1>::kBytes, "both kernels are launched with the same size");
-  const int n = p.total_tokens, n_pad = pad_of(n), blocks = n_pad / kTile;
-  const int causal = (p.flags & FASTAV_CAUSAL) ? 1 : 0;
+  const bool causal = (p.flags & FASTAV_CAUSAL) != 0;
   const float scale = p.softmax_scale > 0.f ? p.softmax_scale : 1.0f / sqrtf((float)p.head_dim);
-  const float scale_log2 = scale * kLog2e;
-  const int group = p.num_q_heads / p.num_kv_heads;
-  cudaError_t e;
-  if (!lse_opt) {
-    e = cudaFuncSetAttribute(rollout_attn_kernel<DIM, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    rollout_attn_kernel<DIM, 0><<<dim3(blocks, p.num_q_heads), kThreads, smem, stream>>>(
-        q_map, k_map, n, n_pad, p.num_q_heads, group, scale_log2, causal, lse2, nullptr, 0, 0, 0.f, 0.f, nullptr, nullptr,
-        nullptr, device_status);
+  AttnArgs a{};
+  a.n = p.total_tokens;
+  a.n_pad = pad_of(a.n);
+  a.hq = p.num_q_heads;
+  a.group = p.num_q_heads / p.num_kv_heads;
+  a.scale_log2 = scale * kLog2e;
+  a.causal = causal ? 1 : 0;
+  const int blocks = a.n_pad / kTile;
+  a.items = attn_items(blocks, a.hq, causal);
+  a.lse_parts = reinterpret_cast<float4*>(ws + w.lse_parts);
+  a.counters = reinterpret_cast<int*>(ws + w.counters);
+  a.n_counters = w.n_counters;
+  a.lse_opt = lse_opt;
+  a.alpha = alpha;
+  a.a_hi = reinterpret_cast<__nv_bfloat16*>(ws + w.a_hi);
+  a.a_lo = reinterpret_cast<__nv_bfloat16*>(ws + w.a_lo);
+  a.map_out = map_out;
+  a.partials = reinterpret_cast<float*>(ws + w.partials);
+  a.device_status = device_status;
+  cudaError_t e = once_per_device([&] {
+    const cudaError_t f = cudaFuncSetAttribute(rollout_attn_kernel<DIM, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return f == cudaSuccess ? cudaFuncSetAttribute(rollout_attn_kernel<DIM, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : f;
+  });
+  if (e != cudaSuccess) return e;
+  if (lse_opt) {
+    e = cudaMemsetAsync(a.counters, 0, (size_t)w.n_counters * sizeof(int), stream);
+  } else {
+    e = launch_chained(rollout_attn_kernel<DIM, 0>, dim3(stats_grid(blocks, a.hq, causal)), dim3(kThreads), smem, stream, q_map, k_map, a, ChainHead{});
     count_launches(1);
   }
-  e = cudaFuncSetAttribute(rollout_attn_kernel<DIM, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  // statistics: ours are [head][row] in log2 units; the caller's are [row][head] natural logarithms
-  const float* lse = lse_opt ? lse_opt : lse2;
-  const long long lse_row = lse_opt ? p.num_q_heads : 1, lse_head = lse_opt ? 1 : n_pad;
-  rollout_attn_kernel<DIM, 1><<<dim3(blocks, blocks), kThreads, smem, stream>>>(
-      q_map, k_map, n, n_pad, p.num_q_heads, group, scale_log2, causal, nullptr, lse, lse_row, lse_head,
-      lse_opt ? kLog2e : 1.0f, alpha, a_hi, a_lo, map_out, device_status);
+  e = launch_chained(rollout_attn_kernel<DIM, 1>, dim3(map_grid(blocks, a.hq, causal)), dim3(kThreads), smem, stream, q_map, k_map, a, ChainHead{});
   count_launches(1);
-  return cudaGetLastError();
+  return e;
 }
 
 bool aligned256(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 255u) == 0; }
@@ -557,7 +883,7 @@ extern "C" int32_t fastav_rollout_state_bytes(int32_t n, size_t* out_bytes) {
 extern "C" int32_t fastav_rollout_workspace_bytes(const fastav_params* p, size_t* out_bytes) {
   if (!p || !out_bytes || p->total_tokens < 1 || p->num_q_heads < 1) return FASTAV_ERR_INVALID_ARG;
   if (p->total_tokens > FASTAV_ROLLOUT_MAX_TOKENS) return FASTAV_ERR_UNSUPPORTED;
-  *out_bytes = 2 * plane_bytes(p->total_tokens) + align_up((size_t)p->num_q_heads * pad_of(p->total_tokens) * sizeof(float), 256);
+  *out_bytes = plan_rollout(p->total_tokens, p->num_q_heads).total;
   return FASTAV_OK;
 }
 
@@ -597,29 +923,30 @@ extern "C" int32_t fastav_rollout_layer(const fastav_params* p, const void* q, c
 
   const int n_pad = pad_of(n);
   unsigned char* ws = static_cast<unsigned char*>(workspace);
-  __nv_bfloat16* a_hi = reinterpret_cast<__nv_bfloat16*>(ws);
-  __nv_bfloat16* a_lo = reinterpret_cast<__nv_bfloat16*>(ws + plane_bytes(n));
-  float* lse2 = reinterpret_cast<float*>(ws + 2 * plane_bytes(n));
+  const RolloutWorkspace w = plan_rollout(n, p->num_q_heads);
   const int src = layer_index & 1, dst = src ^ 1;
   CUtensorMap q_map, k_map, rt_hi_map, rt_lo_map, a_hi_map, a_lo_map;
   if (!qk_map(q, p->head_dim, p->num_q_heads, n, p->q_stride_tok, p->q_stride_head, &q_map) ||
       !qk_map(k, p->head_dim, p->num_kv_heads, n, p->k_stride_tok, p->k_stride_head, &k_map) ||
       !plane_map(state_plane(state, n, src, 0), n_pad, &rt_hi_map) || !plane_map(state_plane(state, n, src, 1), n_pad, &rt_lo_map) ||
-      !plane_map(a_hi, n_pad, &a_hi_map) || !plane_map(a_lo, n_pad, &a_lo_map))
+      !plane_map(ws + w.a_hi, n_pad, &a_hi_map) || !plane_map(ws + w.a_lo, n_pad, &a_lo_map))
     return FASTAV_ERR_UNSUPPORTED;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  cudaError_t e = p->head_dim == 128
-                      ? run_layer<128>(*p, q_map, k_map, lse_opt, alpha, lse2, a_hi, a_lo, map_out_opt, device_status, st)
-                      : run_layer<64>(*p, q_map, k_map, lse_opt, alpha, lse2, a_hi, a_lo, map_out_opt, device_status, st);
+  chain_begin(0);
+  cudaError_t e = p->head_dim == 128 ? run_layer<128>(*p, q_map, k_map, lse_opt, alpha, w, ws, map_out_opt, device_status, st)
+                                     : run_layer<64>(*p, q_map, k_map, lse_opt, alpha, w, ws, map_out_opt, device_status, st);
   if (e != cudaSuccess) return FASTAV_ERR_CUDA;
   constexpr size_t gemm_smem = 3 * 4 * kSubTileBytes + sizeof(PipeControl) + 1024;
-  e = cudaFuncSetAttribute(rollout_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem);
+  e = once_per_device([] { return cudaFuncSetAttribute(rollout_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem); });
   if (e != cudaSuccess) return FASTAV_ERR_CUDA;
-  rollout_gemm_kernel<<<dim3(n_pad / kTile, n_pad / kTile), kThreads, gemm_smem, st>>>(
-      rt_hi_map, rt_lo_map, a_hi_map, a_lo_map, n_pad, (p->flags & FASTAV_CAUSAL) ? 1 : 0, state_plane(state, n, dst, 0),
-      state_plane(state, n, dst, 1), device_status);
+  const bool causal = (p->flags & FASTAV_CAUSAL) != 0;
+  const int blocks = n_pad / kTile;
+  e = launch_chained(rollout_gemm_kernel, dim3(gemm_grid(blocks, causal)), dim3(kThreads), gemm_smem, st, rt_hi_map, rt_lo_map, a_hi_map, a_lo_map,
+                     n_pad, causal ? 1 : 0, gemm_items(blocks, causal), causal ? 1 : 0, state_plane(state, n, dst, 0),
+                     state_plane(state, n, dst, 1), reinterpret_cast<float*>(ws + w.partials),
+                     reinterpret_cast<int*>(ws + w.counters) + blocks * blocks, device_status, ChainHead{});
   count_launches(1);
-  return cudaGetLastError() == cudaSuccess ? FASTAV_OK : FASTAV_ERR_CUDA;
+  return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? FASTAV_OK : FASTAV_ERR_CUDA;
 }
 
 extern "C" int32_t fastav_rollout_read(int32_t n, int32_t layers_applied, const void* state, size_t state_bytes,
