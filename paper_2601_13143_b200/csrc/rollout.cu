@@ -16,17 +16,19 @@
 // the causal mask RT is upper and A~ lower triangular: tiles above the diagonal are written as zeros and the
 // K loop of tile (m, n) only covers the blocks m..n.
 //
-// All three kernels are PERSISTENT: the work of a layer is one flat list of items (a 128 x 128 tile of one head's logits;
-// 64 of the K range of one tile of the product), cut into as many equal runs as there are SMs.  A kernel with one block
-// per tile leaves half the chip idle at this size: 171 visible tiles of 28 heads are two rounds of blocks on 148 SMs, and
-// the longest chain of the triangular product alone is 15 us.  Where a run ends inside a tile, the tile's parts meet through
-// the workspace: the statistics as a few partial log-sum-exps per row, the sums as fp32 tiles that the block which finishes
-// last adds up in order (no block waits for another).  ROLLOUT_FIGURES
+// Sharing out the work.  At the paper's prompt size a layer is 171 visible 128 x 128 tiles on 148 SMs, so one block per tile
+// and head, or per tile, leaves much of the chip idle in a second round, and the longest K loop of the triangular product
+// alone is 36 blocks of 64.  The statistics kernel is PERSISTENT: its (head, row block, key block) items are cut into equal
+// runs, one per SM, and a row block that several runs share leaves up to four partial log-sum-exps per row, which the map
+// kernel merges when it reads them.  The map kernel gives every SM whole tiles and cuts the tiles that are left over into
+// slices of 64 or 32 columns.  The product cuts the K loops that are longer than an SM's fair share into parts, whose
+// fp32 tiles meet in the workspace: the part that finishes last adds them up in order (no block waits for another).
+// ROLLOUT_FIGURES
 //
-// Warp 0 issues the TMA loads, warp 1 the MMAs into a ring of accumulators in tensor memory, warps 2..17 are the
-// epilogue (thread <-> accumulator row, four warps per 32-lane quarter of TMEM, 32 columns each).  The epilogue of the
-// attention kernels, one exponential per element, is their bound: 16 per clock and SM from the special-function unit, so
-// two of every eight go through the FMA pipe instead, at the same precision (exp2_pair below).  All waits are bounded.
+// Warp 0 issues the TMA loads, warp 1 the MMAs into accumulators in tensor memory, warps 2..17 are the epilogue
+// (thread <-> accumulator row, four warps per 32-lane quarter of TMEM, a quarter of the columns each).  The epilogue of
+// the attention kernels, one exponential per element, is their bound: 16 per clock and SM from the special-function unit,
+// so two of every eight go through the FMA pipe instead, at the same precision (exp2_pair below).  All waits are bounded.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <limits.h>
@@ -47,14 +49,16 @@ constexpr int kBuffers = 4;    // accumulators of 128 columns
 constexpr int kMaxStages = 4;
 constexpr int kSubTileBytes = kTile * 128;  // 128 rows of one 64-element (128-byte) column block
 constexpr int kMaxParts = 4;   // blocks that may share one row block's statistics
+constexpr int kHeadChunk = 32;
 constexpr size_t kPartialBytes = (size_t)kTile * kTile * sizeof(float);
 
 struct alignas(16) PipeControl {
   uint64_t full[kMaxStages], empty[kMaxStages], tmem_full[kBuffers], tmem_empty[kBuffers], q_empty[2];
   uint32_t tmem_base;
   int abort;
-  int last;                               // this block finished the tile's last part
-  float2 part[2][kColGroups - 1][kTile];  // statistics kernel: (max, sum) per row of column groups 1..3
+  int last;                               // product: this block finished the tile's last part
+  float2 part[2][kColGroups - 1][kTile];  // statistics: (max, sum) per row of column groups 1..3
+  float neg_lse[kHeadChunk][kTile];       // map: minus the log2-sum-exp2 of this tile's rows, some heads at a time
 };
 
 __device__ __forceinline__ void split_bf16(float x, __nv_bfloat16& hi, __nv_bfloat16& lo) {
@@ -164,131 +168,68 @@ __device__ __forceinline__ int triangular_root(long long x) {
   return r;
 }
 
-// A tile's sum is complete in `acc` (32 columns of one row per thread) of the block that gets true back.  The tile's items
-// are [first, end) of the list; a block that holds only part of them leaves its part in the workspace (at most two per
-// block: at the start and at the end of its run), and the last one to finish adds the parts up in the order of the runs.
-__device__ bool meet(PipeControl& ctl, float (&acc)[32], long long items, long long first, long long end, float* partials, int* counter,
-                     bool ok, int ethread) {
-  const int blocks = gridDim.x, me = blockIdx.x;
-  const int b0 = run_of(items, blocks, first), b1 = run_of(items, blocks, end - 1);
-  if (b0 == b1) return ok;
-  auto part_of = [&](int b) { return partials + (size_t)(2 * b + (first <= run_begin(items, blocks, b) ? 0 : 1)) * (kTile * kTile) + ethread; };
-  {
-    float* const mine = part_of(me);
-#pragma unroll
-    for (int c = 0; c < 32; ++c) __stcg(mine + c * kEpilogueThreads, acc[c]);
-  }
-  __threadfence();
-  epilogue_sync();
-  if (ethread == 0) ctl.last = atomicAdd(counter, 1) == b1 - b0 && !ctl.abort;
-  epilogue_sync();
-  const bool last = ctl.last != 0;
-  if (!last || !ok) return false;
-  __threadfence();
-  float total[32];
-#pragma unroll
-  for (int c = 0; c < 32; ++c) total[c] = 0.f;
-#pragma unroll 1
-  for (int b = b0; b <= b1; ++b) {
-    const float* const other = part_of(b);
-#pragma unroll
-    for (int c = 0; c < 32; ++c) total[c] += __ldcg(other + c * kEpilogueThreads);
-  }
-#pragma unroll
-  for (int c = 0; c < 32; ++c) acc[c] = total[c];
-  return true;
-}
-
 // ---- the attention map ---------------------------------------------------------------------------
-template <int DIM, int MODE>
+// Shared memory of both kernels: six tiles of 128 x DIM (192 KB at head_dim 128).
+template <int DIM, int SLOTS>
 struct AttnSmem {
-  static constexpr int kOperandBytes = (DIM / 64) * kSubTileBytes;
-  static constexpr int kSlots = MODE == 0 ? 2 : 3;
-  static constexpr int kStages = 6 - kSlots;  // six tiles in all: 192 KB at head_dim 128
+  static constexpr int kSubTiles = DIM / 64;
+  static constexpr int kOperandBytes = kSubTiles * kSubTileBytes;
+  static constexpr int kSlots = SLOTS;          // for the operand that changes rarely
+  static constexpr int kStages = 6 - kSlots;    // the ring of the operand that changes every iteration
   static constexpr size_t kBytes = (size_t)6 * kOperandBytes + sizeof(PipeControl) + 1024;
-};
-
-// One item: head, row block, key block.  MODE 0 walks the key blocks of a row block, then the row blocks of a head; MODE 1
-// the heads of a tile, then the tiles (key blocks of a row block).
-template <int MODE>
-struct Item {
-  int head, rb, jb, blocks, hq;
-  bool causal;
-  long long first;  // MODE 1: first item of the tile
-  __device__ Item(long long x, int blocks_, int hq_, bool causal_) : blocks(blocks_), hq(hq_), causal(causal_) {
-    const long long per_head = causal ? (long long)blocks * (blocks + 1) / 2 : (long long)blocks * blocks;
-    long long t;  // visible tile in row order
-    if (MODE == 0) {
-      head = (int)(x / per_head);
-      t = x % per_head;
-      first = 0;
-    } else {
-      t = x / hq;
-      head = (int)(x % hq);
-      first = t * hq;
-    }
-    rb = causal ? triangular_root(t) : (int)(t / blocks);
-    jb = (int)(t - (causal ? (long long)rb * (rb + 1) / 2 : (long long)rb * blocks));
-  }
-  __device__ __forceinline__ int last_jb() const { return causal ? rb : blocks - 1; }
-  __device__ __forceinline__ bool unit_ends() const { return MODE == 0 ? jb == last_jb() : head == hq - 1; }
-  __device__ __forceinline__ void advance() {
-    if (MODE == 1) {
-      if (++head < hq) return;
-      head = 0;
-      first += hq;
-    }
-    if (jb < last_jb()) {
-      ++jb;
-      return;
-    }
-    jb = 0;
-    if (++rb == blocks) {
-      rb = 0;
-      ++head;  // MODE 0 only: the list of MODE 1 ends here
-    }
-  }
 };
 
 struct AttnArgs {
   int n, n_pad, hq, group;
   float scale_log2;
   int causal;
-  long long items;
-  float4* lse_parts;      // [hq][n_pad]: log2-sum-exp2 of up to four runs of a row's keys (-inf: no such run); MODE 0 writes, MODE 1 reads
-  int* counters;          // MODE 0 clears them: one per tile of the map and of the product
-  int n_counters;
-  const float* lse_opt;   // MODE 1, instead of lse_parts: the caller's natural logarithms [n][hq]
-  float alpha;
-  __nv_bfloat16 *a_hi, *a_lo;
-  float* map_out;
-  float* partials;
+  float4* lse_parts;      // [hq][n_pad]: log2-sum-exp2 of up to four runs of a row's keys (-inf: no such run)
   int32_t* device_status;
 };
 
-// MODE 0: per row and head, the log2-sum-exp2 of the scaled logits.
-// MODE 1: per 128 x 128 tile, the sum over the heads of the softmax weights; then Eq. 2, stored as hi / lo planes (and, if
-//         asked, A itself in fp32).
-template <int DIM, int MODE>
+// One item of the statistics: head, row block, key block, in that order.
+struct StatItem {
+  int head, rb, jb, blocks;
+  bool causal;
+  __device__ StatItem(long long x, int blocks_, bool causal_) : blocks(blocks_), causal(causal_) {
+    const long long per_head = causal ? (long long)blocks * (blocks + 1) / 2 : (long long)blocks * blocks;
+    head = (int)(x / per_head);
+    const long long t = x % per_head;
+    rb = causal ? triangular_root(t) : (int)(t / blocks);
+    jb = (int)(t - (causal ? (long long)rb * (rb + 1) / 2 : (long long)rb * blocks));
+  }
+  __device__ __forceinline__ bool row_ends() const { return jb == (causal ? rb : blocks - 1); }
+  __device__ __forceinline__ void advance() {
+    if (!row_ends()) {
+      ++jb;
+      return;
+    }
+    jb = 0;
+    if (++rb == blocks) {
+      rb = 0;
+      ++head;
+    }
+  }
+};
+
+// Per row and head, the log2-sum-exp2 of the scaled logits.
+template <int DIM>
 __global__ void __launch_bounds__(kThreads, 1)
-rollout_attn_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map, AttnArgs a, ChainHead head) {
-  // Shared memory: a ring of tiles of the operand that changes every item (MODE 0: K; MODE 1: Q) and a few slots for the
-  // one that changes rarely (MODE 0: Q, per row block, freed by the last MMA that reads it; MODE 1: K, per KV head and
-  // shared by the G heads of its group -- three slots used in turn, so that a slot is overwritten no sooner than three
-  // items after its last use, which is the distance the ring's own barriers already guarantee).
-  using Cfg = AttnSmem<DIM, MODE>;
-  constexpr int kStages = Cfg::kStages, kSlots = Cfg::kSlots;
-  constexpr int kSubTiles = DIM / 64;
-  constexpr int kOperandBytes = Cfg::kOperandBytes;  // one 128 x DIM tile
+rollout_stats_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map, AttnArgs a, long long items,
+                     int* counters, int n_counters, ChainHead chain_head) {
+  // The ring holds K tiles; a Q tile's slot is freed by the last MMA that reads it.
+  using Cfg = AttnSmem<DIM, 2>;
+  constexpr int kStages = Cfg::kStages, kOperandBytes = Cfg::kOperandBytes;
   extern __shared__ unsigned char smem_raw[];
-  chain_enter(head);
+  chain_enter(chain_head);
   const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t slots = base + kStages * kOperandBytes;
-  PipeControl& ctl = *reinterpret_cast<PipeControl*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + (kStages + kSlots) * kOperandBytes);
+  PipeControl& ctl = *reinterpret_cast<PipeControl*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + 6 * kOperandBytes);
   volatile int* abort = &ctl.abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int blocks = a.n_pad / kTile, group = a.group;
-  const long long begin = run_begin(a.items, gridDim.x, blockIdx.x), end = run_begin(a.items, gridDim.x, blockIdx.x + 1);
+  const int blocks = a.n_pad / kTile;
+  const bool causal = a.causal != 0;
+  const long long begin = run_begin(items, gridDim.x, blockIdx.x), end = run_begin(items, gridDim.x, blockIdx.x + 1);
   const int count = (int)(end - begin);
 
   pipe_setup(ctl, kStages, warp, &q_map, &k_map);
@@ -297,47 +238,37 @@ rollout_attn_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
   if (warp == 0) {
     if (lane == 0) {
       pdl_wait();  // q and k may be what earlier work wrote
-      Item<MODE> x(begin, blocks, a.hq, a.causal != 0);
-      int it = 0, loads = 0;  // items, tiles of the operand that changes rarely
+      StatItem x(begin, blocks, causal);
+      int it = 0, loads = 0;  // items, Q tiles
       for (; it < count; ++it) {
         const int stage = it % kStages;
         if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.empty[stage]), ((it / kStages) & 1) ^ 1u, abort)) break;
-        const bool load_slot = it == 0 || (MODE == 0 ? x.jb == 0 : x.head % group == 0);
-        const uint32_t slot = slots + (loads % kSlots) * kOperandBytes;
-        if (MODE == 0 && load_slot &&
-            !ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.q_empty[loads & 1]), ((loads >> 1) & 1) ^ 1u, abort))
-          break;
+        const bool load_q = it == 0 || x.jb == 0;
+        if (load_q && !ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.q_empty[loads & 1]), ((loads >> 1) & 1) ^ 1u, abort)) break;
         const uint32_t bar = ptx::smem_u32(&ctl.full[stage]);
-        const uint32_t ring = base + stage * kOperandBytes;
-        ptx::mbar_arrive_expect_tx(bar, kOperandBytes + (load_slot ? kOperandBytes : 0));
+        const uint32_t ring = base + stage * kOperandBytes, slot = slots + (loads & 1) * kOperandBytes;
+        ptx::mbar_arrive_expect_tx(bar, kOperandBytes + (load_q ? kOperandBytes : 0));
 #pragma unroll
-        for (int sub = 0; sub < kSubTiles; ++sub) {
-          const uint32_t at = sub * kSubTileBytes;
-          if (MODE == 0) {
-            if (load_slot) ptx::tma_load_3d(slot + at, &q_map, sub * 64, x.head, x.rb * kTile, bar);
-            ptx::tma_load_3d(ring + at, &k_map, sub * 64, x.head / group, x.jb * kTile, bar);
-          } else {
-            if (load_slot) ptx::tma_load_3d(slot + at, &k_map, sub * 64, x.head / group, x.jb * kTile, bar);
-            ptx::tma_load_3d(ring + at, &q_map, sub * 64, x.head, x.rb * kTile, bar);
-          }
+        for (int sub = 0; sub < Cfg::kSubTiles; ++sub) {
+          if (load_q) ptx::tma_load_3d(slot + sub * kSubTileBytes, &q_map, sub * 64, x.head, x.rb * kTile, bar);
+          ptx::tma_load_3d(ring + sub * kSubTileBytes, &k_map, sub * 64, x.head / a.group, x.jb * kTile, bar);
         }
-        loads += load_slot;
+        loads += load_q;
         x.advance();
       }
       if (*abort) drain_loads(ctl, it, kStages);
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      Item<MODE> x(begin, blocks, a.hq, a.causal != 0);
+      StatItem x(begin, blocks, causal);
       int loads = 0;
       for (int it = 0; it < count; ++it) {
         const int stage = it % kStages, buf = it % kBuffers;
         if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort)) break;
         if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_empty[buf]), ((it / kBuffers) & 1) ^ 1u, abort)) break;
         ptx::tc_fence_after_sync();
-        loads += it == 0 || (MODE == 0 ? x.jb == 0 : x.head % group == 0);
-        const uint32_t ring = base + stage * kOperandBytes, slot = slots + ((loads - 1) % kSlots) * kOperandBytes;
-        const uint32_t q_tile = MODE == 0 ? slot : ring, k_tile = MODE == 0 ? ring : slot;
+        loads += it == 0 || x.jb == 0;
+        const uint32_t k_tile = base + stage * kOperandBytes, q_tile = slots + ((loads - 1) & 1) * kOperandBytes;
 #pragma unroll
         for (int ks = 0; ks < DIM / 16; ++ks) {
           const uint32_t sub = ks / 4, off = (ks % 4) * 32;
@@ -346,7 +277,7 @@ rollout_attn_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
         }
         ptx::umma_commit(ptx::smem_u32(&ctl.empty[stage]));
         ptx::umma_commit(ptx::smem_u32(&ctl.tmem_full[buf]));
-        if (MODE == 0 && x.unit_ends()) ptx::umma_commit(ptx::smem_u32(&ctl.q_empty[(loads - 1) & 1]));
+        if (x.row_ends()) ptx::umma_commit(ptx::smem_u32(&ctl.q_empty[(loads - 1) & 1]));
         x.advance();
       }
     }
@@ -355,47 +286,19 @@ rollout_attn_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
     const int row_in = quarter * 32 + lane, ethread = cg * kTile + row_in;
     const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16) + cg * 32;
     pdl_wait();
-    float4* lse_parts = a.lse_parts;
-    const float* lse_opt = a.lse_opt;
-    pdl_acquire(lse_parts);
-    pdl_acquire(lse_opt);
-    if (MODE == 0)
-      for (int i = blockIdx.x * kEpilogueThreads + ethread; i < a.n_counters; i += gridDim.x * kEpilogueThreads) a.counters[i] = 0;
-    Item<MODE> x(begin, blocks, a.hq, a.causal != 0);
-    float zmax = -INFINITY;                             // MODE 0, unscaled
-    float2 sum2 = make_float2(0.f, 0.f);
-    float2 acc2[16];                                    // MODE 1
-#pragma unroll
-    for (int c = 0; c < 16; ++c) acc2[c] = make_float2(0.f, 0.f);
+    for (int i = blockIdx.x * kEpilogueThreads + ethread; i < n_counters; i += gridDim.x * kEpilogueThreads) counters[i] = 0;
+    StatItem x(begin, blocks, causal);
+    // which of its row block's runs this block's first one is; every later row block starts here
+    int part = blockIdx.x - run_of(items, gridDim.x, begin - x.jb);
     const float scale = a.scale_log2;
     const float2 sc = make_float2(scale, scale);
-    // MODE 1: a row's statistic of one head; the NEXT item's is fetched while this one is worked on.
-    auto fetch = [&](const Item<MODE>& at) -> float4 {
-      const int row = at.rb * kTile + row_in;
-      if (lse_opt) return make_float4(row < a.n ? __ldcg(lse_opt + (long long)row * a.hq + at.head) * kLog2e : 0.f, -INFINITY, -INFINITY, -INFINITY);
-      return __ldcg(lse_parts + (long long)at.head * a.n_pad + row);
-    };
-    float4 stat_next = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (MODE == 1 && count > 0) stat_next = fetch(x);
-    int turn = 0;  // MODE 0: which half of the exchange buffer
+    float zmax = -INFINITY;  // unscaled
+    float2 sum2 = make_float2(0.f, 0.f);
+    int turn = 0;            // which half of the exchange buffer
     bool ok = true;
 #pragma unroll 1
-    for (int it = 0; it < count; ++it) {
+    for (int it = 0; it < count; ++it, x.advance()) {
       const int buf = it % kBuffers;
-      const Item<MODE> here = x;
-      x.advance();
-      float neg_lse2 = 0.f;
-      if (MODE == 1) {
-        const float4 st = stat_next;
-        if (it + 1 < count) stat_next = fetch(x);
-        float lse2 = st.x;
-        if (__any_sync(0xFFFFFFFFu, st.y > -INFINITY)) {  // the row block's statistics come from several runs
-          const float m = fmaxf(fmaxf(st.x, st.y), fmaxf(st.z, st.w));
-          const float t = ptx::ex2_approx(st.x - m) + ptx::ex2_approx(st.y - m) + ptx::ex2_approx(st.z - m) + ptx::ex2_approx(st.w - m);
-          lse2 = m > -INFINITY ? m + log2f(t) : -INFINITY;
-        }
-        neg_lse2 = lse2 > -INFINITY ? -lse2 : -INFINITY;  // a row that sees nothing adds 0
-      }
       if (ok) ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_full[buf]), (it / kBuffers) & 1, abort);
       if (ok) {
         ptx::tc_fence_after_sync();
@@ -404,106 +307,238 @@ rollout_attn_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
         ptx::tmem_ld_wait_for(v);
         ptx::tc_fence_before_sync();
         ptx::mbar_arrive(ptx::smem_u32(&ctl.tmem_empty[buf]));  // the accumulator may be overwritten
-        const int row = here.rb * kTile + row_in;
-        const int last_visible = min(a.n - 1, a.causal ? row : INT_MAX);
-        const int limit = last_visible - (here.jb * kTile + cg * 32);  // columns 0..limit of this group are visible
-        const bool whole = limit >= 31;  // the usual case; only tiles on the diagonal or at the end of the sequence are cut
-        if constexpr (MODE == 0) {
-          if (limit >= 0) {
-            if (!whole) {
+        const int last_visible = min(a.n - 1, causal ? x.rb * kTile + row_in : INT_MAX);
+        const int limit = last_visible - (x.jb * kTile + cg * 32);  // columns 0..limit of this group are visible
+        if (limit < 31) {  // only tiles on the diagonal or at the end of the sequence
 #pragma unroll
-              for (int c = 0; c < 32; ++c)
-                if (c > limit) v[c] = 0xFF800000u;  // -inf
-            }
-            float m = zmax;
-#pragma unroll
-            for (int c = 0; c < 32; c += 2) m = fmaxf(m, fmaxf(__uint_as_float(v[c]), __uint_as_float(v[c + 1])));
-            const float corr = ptx::ex2_approx((zmax - m) * scale);  // 0 the first time
-            sum2.x *= corr;
-            sum2.y *= corr;
-            zmax = m;
-            const float shift = -m * scale;
-            const float2 sh = make_float2(shift, shift);
-#pragma unroll
-            for (int c = 0; c < 32; c += 2)
-              sum2 = __fadd2_rn(sum2, exp2_pair(__ffma2_rn(make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc, sh), c / 2));
-          }
-          __syncwarp();  // the rows of a warp differ in `limit`; the tcgen05 instructions that follow need the whole warp
-        } else {
-          const float2 nl = make_float2(neg_lse2, neg_lse2);
-          if (whole) {
-#pragma unroll
-            for (int c = 0; c < 32; c += 2)
-              acc2[c / 2] = __fadd2_rn(acc2[c / 2], exp2_pair(__ffma2_rn(make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc, nl), c / 2));
-          } else if (limit >= 0) {
-#pragma unroll
-            for (int c = 0; c < 32; c += 2) {
-              const float2 p = exp2_pair(__ffma2_rn(make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc, nl), c / 2);
-              acc2[c / 2].x += c <= limit ? p.x : 0.f;
-              acc2[c / 2].y += c + 1 <= limit ? p.y : 0.f;
-            }
-          }
-          __syncwarp();
+          for (int c = 0; c < 32; ++c)
+            if (c > limit) v[c] = 0xFF800000u;  // -inf
         }
-      }
-      const bool unit_ends = here.unit_ends();
-      if (!unit_ends && it + 1 < count) continue;
-      // ---- the end of a row block's keys (MODE 0) or of a tile's heads (MODE 1), or of this block's run ------------
-      if constexpr (MODE == 0) {
-        if (cg > 0) ctl.part[turn][cg - 1][row_in] = make_float2(zmax, sum2.x + sum2.y);
-        epilogue_sync();
-        if (cg == 0 && ok) {
+        if (limit >= 0) {
           float m = zmax;
 #pragma unroll
-          for (int g = 0; g < kColGroups - 1; ++g) m = fmaxf(m, ctl.part[turn][g][row_in].x);
-          float total = zmax > -INFINITY ? (sum2.x + sum2.y) * ptx::ex2_approx((zmax - m) * scale) : 0.f;
+          for (int c = 0; c < 32; c += 2) m = fmaxf(m, fmaxf(__uint_as_float(v[c]), __uint_as_float(v[c + 1])));
+          const float corr = ptx::ex2_approx((zmax - m) * scale);  // 0 the first time
+          sum2.x *= corr;
+          sum2.y *= corr;
+          zmax = m;
+          const float shift = -m * scale;
+          const float2 sh = make_float2(shift, shift);
 #pragma unroll
-          for (int g = 0; g < kColGroups - 1; ++g) {
-            const float2 other = ctl.part[turn][g][row_in];
-            if (other.x > -INFINITY) total += other.y * ptx::ex2_approx((other.x - m) * scale);
-          }
-          const float value = total > 0.f ? m * scale + log2f(total) : -INFINITY;
-          // which of the row block's runs this is: the one after those of the blocks before
-          const long long first_item = begin + it - here.jb;
-          const int part = blockIdx.x - run_of(a.items, gridDim.x, first_item);
-          float* const out = reinterpret_cast<float*>(lse_parts + (long long)here.head * a.n_pad + here.rb * kTile + row_in);
-          if (part < kMaxParts) out[part] = value;
-          if (unit_ends)
-            for (int p = part + 1; p < kMaxParts; ++p) out[p] = -INFINITY;
+          for (int c = 0; c < 32; c += 2)
+            sum2 = __fadd2_rn(sum2, exp2_pair(__ffma2_rn(make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc, sh), c / 2));
         }
-        turn ^= 1;
-        zmax = -INFINITY;
-        sum2 = make_float2(0.f, 0.f);
+        __syncwarp();  // the rows of a warp differ in `limit`; the tcgen05 instructions that follow need the whole warp
+      }
+      const bool row_ends = x.row_ends();
+      if (!row_ends && it + 1 < count) continue;
+      // the four column groups of a row meet in shared memory; group 0 writes the result
+      if (cg > 0) ctl.part[turn][cg - 1][row_in] = make_float2(zmax, sum2.x + sum2.y);
+      epilogue_sync();
+      if (cg == 0 && ok) {
+        float m = zmax;
+#pragma unroll
+        for (int g = 0; g < kColGroups - 1; ++g) m = fmaxf(m, ctl.part[turn][g][row_in].x);
+        float total = zmax > -INFINITY ? (sum2.x + sum2.y) * ptx::ex2_approx((zmax - m) * scale) : 0.f;
+#pragma unroll
+        for (int g = 0; g < kColGroups - 1; ++g) {
+          const float2 other = ctl.part[turn][g][row_in];
+          if (other.x > -INFINITY) total += other.y * ptx::ex2_approx((other.x - m) * scale);
+        }
+        float* const out = reinterpret_cast<float*>(a.lse_parts + (long long)x.head * a.n_pad + x.rb * kTile + row_in);
+        if (part < kMaxParts) out[part] = total > 0.f ? m * scale + log2f(total) : -INFINITY;
+        if (row_ends)
+          for (int p = part + 1; p < kMaxParts; ++p) out[p] = -INFINITY;
+      }
+      part = 0;
+      turn ^= 1;
+      zmax = -INFINITY;
+      sum2 = make_float2(0.f, 0.f);
+    }
+  }
+  pipe_teardown(ctl, warp, a.device_status);
+}
+
+// Per 128 x 128 tile, or slice of its columns: the sum over the heads of the softmax weights, then Eq. 2, stored as hi / lo
+// planes (and, if asked, A itself in fp32).  Blocks 0 .. whole - 1 take whole tiles, the others slices of 128 / slices
+// columns of the tiles that are left; tiles no row may see (which the product never reads) only if the map is wanted.
+template <int DIM>
+__global__ void __launch_bounds__(kThreads, 1)
+rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map, AttnArgs a,
+                   const float* __restrict__ lse_opt, float alpha, int whole, int slices, int blocks_of_work,
+                   __nv_bfloat16* __restrict__ a_hi, __nv_bfloat16* __restrict__ a_lo, float* __restrict__ map_out, ChainHead chain_head) {
+  // The ring holds Q tiles, one per head; a K tile is loaded once per KV head and shared by the G heads of its group -- three
+  // slots used in turn, so that a slot is overwritten no sooner than three iterations after its last use, which is the
+  // distance the ring's own barriers already guarantee.
+  using Cfg = AttnSmem<DIM, 3>;
+  constexpr int kStages = Cfg::kStages, kSlots = Cfg::kSlots, kOperandBytes = Cfg::kOperandBytes;
+  extern __shared__ unsigned char smem_raw[];
+  chain_enter(chain_head);
+  const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
+  const uint32_t slots = base + kStages * kOperandBytes;
+  PipeControl& ctl = *reinterpret_cast<PipeControl*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + 6 * kOperandBytes);
+  volatile int* abort = &ctl.abort;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int blocks = a.n_pad / kTile, hq = a.hq, group = a.group;
+  const bool causal = a.causal != 0;
+
+  if ((int)blockIdx.x >= blocks_of_work) {  // a tile no row may see, and the map is wanted: zeros (uniform for the block)
+    pdl_wait();
+    const int t = blockIdx.x - blocks_of_work;        // (jb, rb) with jb > rb, in the order of the transposed triangle
+    const int jb = triangular_root(t) + 1, rb = t - (jb - 1) * jb / 2;
+    for (int i = threadIdx.x; i < kTile * kTile; i += kThreads) {
+      const int r = rb * kTile + i / kTile, c = jb * kTile + i % kTile;
+      if (r < a.n && c < a.n) map_out[(long long)r * a.n + c] = 0.f;
+    }
+    return;
+  }
+  const bool sliced = (int)blockIdx.x >= whole;
+  const int tile = sliced ? whole + ((int)blockIdx.x - whole) / slices : (int)blockIdx.x;
+  const int width = sliced ? kTile / slices : kTile;                       // columns of this block
+  const int col_first = sliced ? ((int)blockIdx.x - whole) % slices * width : 0;
+  const int rb = causal ? triangular_root(tile) : tile / blocks;
+  const int jb = tile - (causal ? rb * (rb + 1) / 2 : rb * blocks);
+
+  pipe_setup(ctl, kStages, warp, &q_map, &k_map);
+  const uint32_t tmem = ctl.tmem_base;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      pdl_wait();
+      int it = 0;
+      for (; it < hq; ++it) {
+        const int stage = it % kStages;
+        if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.empty[stage]), ((it / kStages) & 1) ^ 1u, abort)) break;
+        const uint32_t bar = ptx::smem_u32(&ctl.full[stage]);
+        const bool load_k = it % group == 0;
+        const uint32_t ring = base + stage * kOperandBytes, slot = slots + ((it / group) % kSlots) * kOperandBytes;
+        ptx::mbar_arrive_expect_tx(bar, kOperandBytes + (load_k ? kOperandBytes : 0));
+#pragma unroll
+        for (int sub = 0; sub < Cfg::kSubTiles; ++sub) {
+          ptx::tma_load_3d(ring + sub * kSubTileBytes, &q_map, sub * 64, it, rb * kTile, bar);
+          if (load_k) ptx::tma_load_3d(slot + sub * kSubTileBytes, &k_map, sub * 64, it / group, jb * kTile, bar);
+        }
+      }
+      if (*abort) drain_loads(ctl, it, kStages);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      const uint32_t idesc = ptx::umma_idesc_bf16(kTile, width);
+      for (int it = 0; it < hq; ++it) {
+        const int stage = it % kStages, buf = it % kBuffers;
+        if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort)) break;
+        if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_empty[buf]), ((it / kBuffers) & 1) ^ 1u, abort)) break;
+        ptx::tc_fence_after_sync();
+        const uint32_t q_tile = base + stage * kOperandBytes;
+        const uint32_t k_tile = slots + ((it / group) % kSlots) * kOperandBytes + col_first * 128;  // a multiple of 32 rows of 128 bytes
+#pragma unroll
+        for (int ks = 0; ks < DIM / 16; ++ks) {
+          const uint32_t sub = ks / 4, off = (ks % 4) * 32;
+          ptx::umma_bf16(tmem + buf * kTile, ptx::umma_desc_sw128(q_tile + sub * kSubTileBytes, off),
+                         ptx::umma_desc_sw128(k_tile + sub * kSubTileBytes, off), idesc, ks > 0);
+        }
+        ptx::umma_commit(ptx::smem_u32(&ctl.empty[stage]));
+        ptx::umma_commit(ptx::smem_u32(&ctl.tmem_full[buf]));
+      }
+    }
+  } else {
+    const int quarter = warp & 3, cg = (warp - 2) >> 2;  // TMEM lanes 32 quarter .., columns width / 4 * cg ..
+    const int row_in = quarter * 32 + lane, ethread = cg * kTile + row_in, row = rb * kTile + row_in;
+    const int cols = width / 4, pieces = cols / 8, col0 = jb * kTile + col_first + cg * cols;
+    const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16) + cg * cols;
+    pdl_wait();
+    float4* lse_parts = a.lse_parts;
+    pdl_acquire(lse_parts);
+    pdl_acquire(lse_opt);
+    const int last_visible = min(a.n - 1, causal ? row : INT_MAX);
+    const int limit = last_visible - col0;  // columns 0..limit of this group are visible
+    const bool whole_visible = __all_sync(0xFFFFFFFFu, limit >= cols - 1);
+    const float2 sc = make_float2(a.scale_log2, a.scale_log2);
+    float2 acc2[16];
+#pragma unroll
+    for (int c = 0; c < 16; ++c) acc2[c] = make_float2(0.f, 0.f);
+    bool ok = true;
+#pragma unroll 1
+    for (int it = 0; it < hq; ++it) {
+      const int buf = it % kBuffers;
+      if (it % kHeadChunk == 0) {  // the rows' statistics of the next heads
+        if (it > 0) epilogue_sync();
+        for (int e = ethread; e < min(kHeadChunk, hq - it) * kTile; e += kEpilogueThreads) {
+          const int h = it + e / kTile, r = rb * kTile + e % kTile;
+          float lse2;
+          if (lse_opt) {
+            lse2 = r < a.n ? chain_load(lse_opt + (long long)r * hq + h) * kLog2e : 0.f;
+          } else {
+            const float4 st = chain_load(lse_parts + (long long)h * a.n_pad + r);
+            lse2 = st.x;
+            if (st.y > -INFINITY) {  // several runs of the row's keys
+              const float m = fmaxf(fmaxf(st.x, st.y), fmaxf(st.z, st.w));
+              lse2 = m + log2f(ptx::ex2_approx(st.x - m) + ptx::ex2_approx(st.y - m) + ptx::ex2_approx(st.z - m) + ptx::ex2_approx(st.w - m));
+            }
+          }
+          ctl.neg_lse[e / kTile][e % kTile] = fabsf(lse2) < INFINITY ? -lse2 : -INFINITY;  // a row that sees nothing adds 0
+        }
+        epilogue_sync();
+      }
+      if (!ok) continue;
+      ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_full[buf]), (it / kBuffers) & 1, abort);
+      if (!ok) continue;
+      ptx::tc_fence_after_sync();
+      const float neg_lse2 = ctl.neg_lse[it % kHeadChunk][row_in];
+      const float2 nl = make_float2(neg_lse2, neg_lse2);
+      uint32_t v[32];
+      if (pieces == 4) {
+        ptx::tmem_ld32(lane_addr + buf * kTile, v);
+        ptx::tmem_ld_wait_for(v);
       } else {
-        float acc[32];
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          acc[2 * c] = acc2[c].x;
-          acc[2 * c + 1] = acc2[c].y;
-          acc2[c] = make_float2(0.f, 0.f);
+        ptx::tmem_ld8(lane_addr + buf * kTile, v);
+        if (pieces == 2) ptx::tmem_ld8(lane_addr + buf * kTile + 8, v + 8);
+        ptx::tmem_ld_wait_for16(v);
+      }
+      ptx::tc_fence_before_sync();
+      ptx::mbar_arrive(ptx::smem_u32(&ctl.tmem_empty[buf]));  // the accumulator may be overwritten
+      auto add = [&](int c) {  // columns c, c + 1
+        float2 p = exp2_pair(__ffma2_rn(make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc, nl), c / 2);
+        if (!whole_visible) {
+          p.x = c <= limit ? p.x : 0.f;
+          p.y = c + 1 <= limit ? p.y : 0.f;
         }
-        if (meet(ctl, acc, a.items, here.first, here.first + a.hq, a.partials, a.counters + here.rb * blocks + here.jb, ok, ethread)) {
-          const int row = here.rb * kTile + row_in, col0 = here.jb * kTile + cg * 32;
-          const float inv_heads = 1.0f / (float)a.hq;
+        acc2[c / 2] = __fadd2_rn(acc2[c / 2], p);
+      };
+      if (pieces == 4) {
+        if (whole_visible) {
 #pragma unroll
-          for (int c = 0; c < 32; ++c) {
-            const float weight = row < a.n ? acc[c] * inv_heads : 0.f;
-            if (a.map_out && row < a.n && col0 + c < a.n) a.map_out[(long long)row * a.n + col0 + c] = weight;
-            acc[c] = a.alpha * weight + ((row < a.n && col0 + c == row) ? 1.0f - a.alpha : 0.f);  // Eq. 2
-          }
-          const long long at = (long long)row * a.n_pad + col0;
-          store_split_row(acc, a.a_hi + at, a.a_lo + at);
+          for (int c = 0; c < 32; c += 2)
+            acc2[c / 2] = __fadd2_rn(acc2[c / 2], exp2_pair(__ffma2_rn(make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc, nl), c / 2));
+        } else {
+#pragma unroll
+          for (int c = 0; c < 32; c += 2) add(c);
+        }
+      } else {
+#pragma unroll
+        for (int c = 0; c < 8; c += 2) add(c);
+        if (pieces == 2) {
+#pragma unroll
+          for (int c = 8; c < 16; c += 2) add(c);
         }
       }
     }
-    if (MODE == 1 && a.map_out && a.causal) {  // tiles no row may see (of the planes the product reads only the others)
-      for (int t = blockIdx.x; t < blocks * blocks; t += gridDim.x) {
-        const int rb = t / blocks, jb = t % blocks;
-        if (jb <= rb) continue;
-        for (int i = ethread; i < kTile * kTile; i += kEpilogueThreads) {
-          const int r = rb * kTile + i / kTile, c = jb * kTile + i % kTile;
-          if (r < a.n && c < a.n) a.map_out[(long long)r * a.n + c] = 0.f;
+    if (ok) {
+      const float inv_heads = 1.0f / (float)hq;
+      const long long at = (long long)row * a.n_pad + col0;
+#pragma unroll
+      for (int c0 = 0; c0 < 32; c0 += 8) {
+        if (c0 >= cols) break;
+        alignas(16) __nv_bfloat16 hi[8], lo[8];
+#pragma unroll
+        for (int c = c0; c < c0 + 8; ++c) {
+          const float sum = (c & 1) ? acc2[c / 2].y : acc2[c / 2].x;
+          const float weight = row < a.n ? sum * inv_heads : 0.f;
+          if (map_out && row < a.n && col0 + c < a.n) map_out[(long long)row * a.n + col0 + c] = weight;
+          split_bf16(alpha * weight + ((row < a.n && col0 + c == row) ? 1.0f - alpha : 0.f), hi[c - c0], lo[c - c0]);  // Eq. 2
         }
+        *reinterpret_cast<uint4*>(a_hi + at + c0) = *reinterpret_cast<const uint4*>(hi);
+        *reinterpret_cast<uint4*>(a_lo + at + c0) = *reinterpret_cast<const uint4*>(lo);
       }
     }
   }
@@ -511,69 +546,73 @@ rollout_attn_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
 }
 
 // ---- Eq. 3: RT_new = RT_old * A~^T ------------------------------------------------------------------
-// One item: a 64-wide K block of one 128 x 128 tile of RT_new.  Its four operand tiles (RT hi, RT lo, A~ hi, A~ lo) are
-// loaded once and used for the three products RT hi * A~ hi, RT lo * A~ hi, RT hi * A~ lo, all accumulated into the same
-// TMEM tile.  Under the causal mask RT is upper and A~ lower triangular: tile (m, nn) has the K blocks m .. nn only.
-struct GemmItem {
-  int mb, nb, kb, blocks;  // kb: 64-wide K block
-  bool causal;
-  long long first;         // first item of the tile
-  __device__ GemmItem(long long x, int blocks_, bool causal_) : blocks(blocks_), causal(causal_) {
-    mb = 0;
-    first = 0;
+// One block per part of a 128 x 128 tile of RT_new.  Per 64-wide K block the four operand tiles (RT hi, RT lo, A~ hi, A~ lo)
+// are loaded once and used for the three products RT hi * A~ hi, RT lo * A~ hi, RT hi * A~ lo, all accumulated into the same
+// TMEM tile.  Under the causal mask RT is upper and A~ lower triangular: tile (m, nn) has the K blocks m .. nn only, so
+// that the tiles of one diagonal nn - m = d have 2 (d + 1) of them.  A tile is cut into ceil(its K blocks / share) equal
+// parts; the blocks are handed out by decreasing d (the longest loops first, the short ones fill the tail), so the parts of
+// cut tiles come first and a part's place in the workspace is its block's number.
+struct GemmUnit {
+  int mb, nb, kb0, kb1;  // tile; 64-wide K blocks [kb0, kb1)
+  int part, parts;
+  bool exists;
+  __device__ GemmUnit(int u, int blocks, bool causal, int share) {
+    exists = true;
     if (causal) {
-      for (;;) {  // row mb holds 2 (1 + 2 + ... + (blocks - mb)) items
-        const long long row = (long long)(blocks - mb) * (blocks - mb + 1);
-        if (x < first + row) break;
-        first += row;
-        ++mb;
+      int d = blocks - 1;
+      for (;; --d) {
+        if (d < 0) {
+          exists = false;
+          return;
+        }
+        parts = (2 * (d + 1) + share - 1) / share;
+        if (u < (blocks - d) * parts) break;
+        u -= (blocks - d) * parts;
       }
-      const long long r = (x - first) / 2;
-      const int d = triangular_root(r);
-      first += (long long)d * (d + 1);
+      mb = u / parts;
       nb = mb + d;
-      kb = 2 * mb + (int)(x - first);
     } else {
-      const long long tile = x / (2 * blocks);
-      mb = (int)(tile / blocks);
-      nb = (int)(tile % blocks);
-      first = tile * 2 * blocks;
-      kb = (int)(x - first);
+      parts = (2 * blocks + share - 1) / share;
+      mb = u / parts / blocks;
+      nb = u / parts % blocks;
+      exists = mb < blocks;
     }
-  }
-  __device__ __forceinline__ int kb_first() const { return causal ? 2 * mb : 0; }
-  __device__ __forceinline__ int kb_last() const { return causal ? 2 * nb + 1 : 2 * blocks - 1; }
-  __device__ __forceinline__ long long tile_end() const { return first + kb_last() - kb_first() + 1; }
-  __device__ __forceinline__ void advance() {
-    if (kb < kb_last()) {
-      ++kb;
-      return;
-    }
-    first = tile_end();
-    if (++nb == blocks) {
-      ++mb;
-      nb = causal ? mb : 0;
-    }
-    kb = kb_first();
+    part = u % parts;
+    const int first = causal ? 2 * mb : 0, count = causal ? 2 * (nb - mb + 1) : 2 * blocks;
+    kb0 = first + count * part / parts;
+    kb1 = first + count * (part + 1) / parts;
   }
 };
 
 __global__ void __launch_bounds__(kThreads, 1)
 rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_constant__ CUtensorMap rt_lo_map,
                     const __grid_constant__ CUtensorMap a_hi_map, const __grid_constant__ CUtensorMap a_lo_map, int n_pad,
-                    int causal, long long items, int clear, __nv_bfloat16* __restrict__ out_hi, __nv_bfloat16* __restrict__ out_lo,
-                    float* partials, int* counters, int32_t* device_status, ChainHead head) {
+                    int causal, int share, int units, __nv_bfloat16* __restrict__ out_hi, __nv_bfloat16* __restrict__ out_lo,
+                    float* partials, int* counters, int32_t* device_status, ChainHead chain_head) {
   constexpr int kStages = 3;
   constexpr int kStageBytes = 4 * kSubTileBytes;  // 128 x 64 each of RT hi, RT lo, A~ hi, A~ lo
   extern __shared__ unsigned char smem_raw[];
-  chain_enter(head);
+  chain_enter(chain_head);
   const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   PipeControl& ctl = *reinterpret_cast<PipeControl*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + kStages * kStageBytes);
   volatile int* abort = &ctl.abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int blocks = n_pad / kTile;
-  const long long begin = run_begin(items, gridDim.x, blockIdx.x), end = run_begin(items, gridDim.x, blockIdx.x + 1);
-  const int count = (int)(end - begin);
+
+  if ((int)blockIdx.x >= units) {  // the first causal layer: nothing but zeros below the diagonal (later layers leave them)
+    pdl_wait();
+    const int t = blockIdx.x - units;  // (mb, nb) with mb > nb
+    const int mb = triangular_root(t) + 1, nb = t - (mb - 1) * mb / 2;
+    for (int i = threadIdx.x; i < kTile * (kTile / 8); i += kThreads) {
+      const int r = i / (kTile / 8), c = (i % (kTile / 8)) * 8;
+      const long long at = (long long)(mb * kTile + r) * n_pad + nb * kTile + c;
+      *reinterpret_cast<uint4*>(out_hi + at) = make_uint4(0, 0, 0, 0);
+      *reinterpret_cast<uint4*>(out_lo + at) = make_uint4(0, 0, 0, 0);
+    }
+    return;
+  }
+  const GemmUnit unit(blockIdx.x, blocks, causal != 0, share);
+  const int iters = unit.exists ? unit.kb1 - unit.kb0 : 0;  // (the host counts the units as the device does: always exists)
 
   pipe_setup(ctl, kStages, warp, &rt_hi_map, &a_hi_map);
   const uint32_t tmem = ctl.tmem_base;
@@ -581,31 +620,27 @@ rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_
   if (warp == 0) {
     if (lane == 0) {
       pdl_wait();
-      GemmItem x(begin, blocks, causal != 0);
       int it = 0;
-      for (; it < count; ++it) {
+      for (; it < iters; ++it) {
         const int stage = it % kStages;
         if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.empty[stage]), ((it / kStages) & 1) ^ 1u, abort)) break;
+        const int kb = unit.kb0 + it;
         const uint32_t bar = ptx::smem_u32(&ctl.full[stage]);
         const uint32_t dst = base + stage * kStageBytes;
         ptx::mbar_arrive_expect_tx(bar, kStageBytes);
-        ptx::tma_load_2d(dst, &rt_hi_map, x.kb * 64, x.mb * kTile, bar);
-        ptx::tma_load_2d(dst + kSubTileBytes, &rt_lo_map, x.kb * 64, x.mb * kTile, bar);
-        ptx::tma_load_2d(dst + 2 * kSubTileBytes, &a_hi_map, x.kb * 64, x.nb * kTile, bar);
-        ptx::tma_load_2d(dst + 3 * kSubTileBytes, &a_lo_map, x.kb * 64, x.nb * kTile, bar);
-        x.advance();
+        ptx::tma_load_2d(dst, &rt_hi_map, kb * 64, unit.mb * kTile, bar);
+        ptx::tma_load_2d(dst + kSubTileBytes, &rt_lo_map, kb * 64, unit.mb * kTile, bar);
+        ptx::tma_load_2d(dst + 2 * kSubTileBytes, &a_hi_map, kb * 64, unit.nb * kTile, bar);
+        ptx::tma_load_2d(dst + 3 * kSubTileBytes, &a_lo_map, kb * 64, unit.nb * kTile, bar);
       }
       if (*abort) drain_loads(ctl, it, kStages);
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      GemmItem x(begin, blocks, causal != 0);
-      int tile = 0;  // tiles (or parts of one) begun by this block
-      bool fresh = true, ok = true;
-      for (int it = 0; it < count && ok; ++it) {
-        const int stage = it % kStages, buf = tile % kBuffers;
-        if (fresh) ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_empty[buf]), ((tile / kBuffers) & 1) ^ 1u, abort);
-        if (ok) ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort);
+      bool ok = true;
+      for (int it = 0; it < iters && ok; ++it) {
+        const int stage = it % kStages;
+        ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort);
         if (!ok) break;
         ptx::tc_fence_after_sync();
         const uint32_t rt_hi = base + stage * kStageBytes, rt_lo = rt_hi + kSubTileBytes, a_hi = rt_hi + 2 * kSubTileBytes,
@@ -615,64 +650,57 @@ rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_
           const uint32_t rt_tile = term == 1 ? rt_lo : rt_hi, a_tile = term == 2 ? a_lo : a_hi;
 #pragma unroll
           for (int ks = 0; ks < 4; ++ks)
-            ptx::umma_bf16(tmem + buf * kTile, ptx::umma_desc_sw128(rt_tile, ks * 32), ptx::umma_desc_sw128(a_tile, ks * 32),
-                           ptx::umma_idesc_bf16(kTile, kTile), (!fresh || term > 0 || ks > 0) ? 1u : 0u);
+            ptx::umma_bf16(tmem, ptx::umma_desc_sw128(rt_tile, ks * 32), ptx::umma_desc_sw128(a_tile, ks * 32),
+                           ptx::umma_idesc_bf16(kTile, kTile), (it > 0 || term > 0 || ks > 0) ? 1u : 0u);
         }
         ptx::umma_commit(ptx::smem_u32(&ctl.empty[stage]));
-        fresh = x.kb == x.kb_last() || it + 1 == count;
-        if (fresh) {
-          ptx::umma_commit(ptx::smem_u32(&ctl.tmem_full[buf]));
-          ++tile;
-        }
-        x.advance();
       }
+      if (ok) ptx::umma_commit(ptx::smem_u32(&ctl.tmem_full[0]));
     }
   } else {
     const int quarter = warp & 3, cg = (warp - 2) >> 2;
     const int row_in = quarter * 32 + lane, ethread = cg * kTile + row_in;
     pdl_wait();
-    bool ok = true;
-    GemmItem x(begin, blocks, causal != 0);
-    int tile = 0;
-#pragma unroll 1
-    for (long long at = begin; at < end; ++tile) {
-      const long long tile_end = x.tile_end();
-      const int buf = tile % kBuffers;
-      if (ok) ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_full[buf]), (tile / kBuffers) & 1, abort);
-      float acc[32];
-      if (ok) {
-        ptx::tc_fence_after_sync();
-        uint32_t v[32];
-        ptx::tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + buf * kTile + cg * 32, v);
-        ptx::tmem_ld_wait_for(v);
-        ptx::tc_fence_before_sync();
-        ptx::mbar_arrive(ptx::smem_u32(&ctl.tmem_empty[buf]));
+    const bool ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_full[0]), 0, abort);
+    float x[32];
+    if (ok) {
+      ptx::tc_fence_after_sync();
+      uint32_t v[32];
+      ptx::tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + cg * 32, v);
+      ptx::tmem_ld_wait_for(v);
 #pragma unroll
-        for (int c = 0; c < 32; ++c) acc[c] = __uint_as_float(v[c]);
-      } else {
+      for (int c = 0; c < 32; ++c) x[c] = __uint_as_float(v[c]);
+    } else {
 #pragma unroll
-        for (int c = 0; c < 32; ++c) acc[c] = 0.f;
-      }
-      if (meet(ctl, acc, items, x.first, tile_end, partials, counters + x.mb * blocks + x.nb, ok, ethread)) {
-        const long long out = (long long)(x.mb * kTile + row_in) * n_pad + x.nb * kTile + cg * 32;
-        store_split_row(acc, out_hi + out, out_lo + out);
-      }
-      __syncwarp();
-      at = tile_end;
-      x.kb = x.kb_last();
-      x.advance();
+      for (int c = 0; c < 32; ++c) x[c] = 0.f;
     }
-    if (clear)  // RT is upper triangular: nothing but zeros below (later layers leave them as they are)
-      for (int t = blockIdx.x; t < blocks * blocks; t += gridDim.x) {
-        const int mb = t / blocks, nb = t % blocks;
-        if (mb <= nb) continue;
-        for (int i = ethread; i < kTile * (kTile / 8); i += kEpilogueThreads) {
-          const int r = i / (kTile / 8), c = (i % (kTile / 8)) * 8;
-          const long long out = (long long)(mb * kTile + r) * n_pad + nb * kTile + c;
-          *reinterpret_cast<uint4*>(out_hi + out) = make_uint4(0, 0, 0, 0);
-          *reinterpret_cast<uint4*>(out_lo + out) = make_uint4(0, 0, 0, 0);
+    bool mine = ok;  // this block writes the tile
+    if (unit.parts > 1) {
+      constexpr int kFloats = kTile * kTile;
+      float* const here = partials + (size_t)blockIdx.x * kFloats + ethread;
+#pragma unroll
+      for (int c = 0; c < 32; ++c) __stcg(here + c * kEpilogueThreads, x[c]);
+      __threadfence();
+      epilogue_sync();
+      if (ethread == 0) ctl.last = atomicAdd(counters + unit.mb * blocks + unit.nb, 1) == unit.parts - 1 && !ctl.abort;
+      epilogue_sync();
+      mine = ok && ctl.last != 0;
+      if (mine) {  // the last part to finish: add the parts up in order
+        __threadfence();
+        const float* p = partials + (size_t)(blockIdx.x - unit.part) * kFloats + ethread;
+#pragma unroll
+        for (int c = 0; c < 32; ++c) x[c] = 0.f;
+#pragma unroll 1
+        for (int i = 0; i < unit.parts; ++i, p += kFloats) {
+#pragma unroll
+          for (int c = 0; c < 32; ++c) x[c] += __ldcg(p + c * kEpilogueThreads);
         }
       }
+    }
+    if (mine) {
+      const long long at = (long long)(unit.mb * kTile + row_in) * n_pad + unit.nb * kTile + cg * 32;
+      store_split_row(x, out_hi + at, out_lo + at);
+    }
   }
   pipe_teardown(ctl, warp, device_status);
 }
@@ -781,22 +809,41 @@ __nv_bfloat16* state_plane(void* state, int n, int copy, int lo) {
   return reinterpret_cast<__nv_bfloat16*>(static_cast<unsigned char*>(state) + (size_t)(copy * 2 + lo) * plane_bytes(n));
 }
 
-// ---- runs and workspace: the same on both sides ----------------------------------------------------------
+// ---- how a layer's work is shared out ------------------------------------------------------------------
 long long visible_tiles(int blocks, bool causal) { return causal ? (long long)blocks * (blocks + 1) / 2 : (long long)blocks * blocks; }
-long long attn_items(int blocks, int hq, bool causal) { return visible_tiles(blocks, causal) * hq; }
-long long gemm_items(int blocks, bool causal) {  // causal: sum over the rows of 2 (1 + ... + (blocks - mb))
-  return causal ? (long long)blocks * (blocks + 1) * (blocks + 2) / 3 : 2ll * blocks * blocks * blocks;
-}
-// Blocks: one per SM unless the runs would get too short.  A row block's statistics may come from at most kMaxParts runs
-// (a run of at least a third of the longest row block); a tile's sum from any number, but each part costs an exchange of
-// 64 KB, so a run has at least six tiles of logits or four K blocks.
-int grid_for(long long items, long long shortest_run) {
-  const long long g = items / shortest_run;
+long long hidden_tiles(int blocks) { return (long long)blocks * (blocks - 1) / 2; }
+
+// Statistics: one run per SM unless the runs would get too short; a run of at least a third of the longest row block keeps
+// the number of runs that share one within kMaxParts.
+int stats_grid(int blocks, int hq, bool causal) {
+  const long long g = visible_tiles(blocks, causal) * hq / ((blocks + 2) / 3);
   return (int)(g < 1 ? 1 : g > kNumSMs ? kNumSMs : g);
 }
-int stats_grid(int blocks, int hq, bool causal) { return grid_for(attn_items(blocks, hq, causal), (blocks + 2) / 3); }
-int map_grid(int blocks, int hq, bool causal) { return grid_for(attn_items(blocks, hq, causal), 6); }
-int gemm_grid(int blocks, bool causal) { return grid_for(gemm_items(blocks, causal), 4); }
+
+// Map: whole tiles as long as they fill rounds of all SMs, the rest in as many slices of at least 32 columns as still
+// make one round.
+void map_shares(int blocks, bool causal, int* whole, int* slices) {
+  const long long tiles = visible_tiles(blocks, causal);
+  const int rest = (int)(tiles % kNumSMs);
+  *slices = rest * 4 <= kNumSMs ? 4 : rest * 2 <= kNumSMs ? 2 : 1;
+  *whole = (int)(tiles - rest);
+}
+
+// Product: no K loop longer than an SM's share of all K blocks (at least eight: a part costs an exchange of 64 KB).
+int gemm_share(int blocks, bool causal) {
+  const long long items = causal ? (long long)blocks * (blocks + 1) * (blocks + 2) / 3 : 2ll * blocks * blocks * blocks;
+  const long long share = (items + kNumSMs - 1) / kNumSMs;
+  return (int)(share < 8 ? 8 : share);
+}
+// Parts in all, and those of tiles that are cut (they come first).
+void gemm_units(int blocks, bool causal, int share, int* units, int* cut) {
+  *units = *cut = 0;
+  for (int d = blocks - 1; d >= 0; --d) {
+    const int count = causal ? 2 * (d + 1) : 2 * blocks, tiles = causal ? blocks - d : blocks, parts = (count + share - 1) / share;
+    *units += tiles * parts;
+    if (parts > 1) *cut += tiles * parts;
+  }
+}
 
 struct RolloutWorkspace {
   size_t a_hi, a_lo, lse_parts, partials, counters, total;
@@ -805,29 +852,29 @@ struct RolloutWorkspace {
 RolloutWorkspace plan_rollout(int n, int hq) {
   RolloutWorkspace w{};
   const int blocks = pad_of(n) / kTile;
-  int grid = 0;  // over both masks
+  int most = 0;  // parts that need a place, over both masks
   for (int causal = 0; causal < 2; ++causal) {
-    const int m = map_grid(blocks, hq, causal != 0), g = gemm_grid(blocks, causal != 0);
-    grid = m > grid ? m : grid;
-    grid = g > grid ? g : grid;
+    int units, cut;
+    gemm_units(blocks, causal != 0, gemm_share(blocks, causal != 0), &units, &cut);
+    most = cut > most ? cut : most;
   }
   size_t off = 0;
   auto carve = [&](size_t bytes) { const size_t at = off; off = align_up(off + bytes, 256); return at; };
   w.a_hi = carve(plane_bytes(n));
   w.a_lo = carve(plane_bytes(n));
   w.lse_parts = carve((size_t)hq * pad_of(n) * sizeof(float4));
-  w.partials = carve((size_t)2 * grid * kPartialBytes);
-  w.n_counters = 2 * blocks * blocks;  // the map's tiles, then the product's
+  w.partials = carve((size_t)most * kPartialBytes);
+  w.n_counters = blocks * blocks;  // one per tile of the product
   w.counters = carve((size_t)w.n_counters * sizeof(int));
   w.total = off;
   return w;
 }
 
 template <int DIM>
-cudaError_t run_layer(const fastav_params& p, const CUtensorMap& q_map, const CUtensorMap& k_map, const float* lse_opt, float alpha,
-                      const RolloutWorkspace& w, unsigned char* ws, float* map_out, int32_t* device_status, cudaStream_t stream) {
-  constexpr size_t smem = AttnSmem<DIM, 0>::kBytes;
-  static_assert(AttnSmem<DIM, 0>::kBytes == AttnSmem<DIM, 1>::kBytes, "both kernels are launched with the same size");
+cudaError_t run_attention(const fastav_params& p, const CUtensorMap& q_map, const CUtensorMap& k_map, const float* lse_opt, float alpha,
+                          const RolloutWorkspace& w, unsigned char* ws, float* map_out, int32_t* device_status, cudaStream_t stream) {
+  constexpr size_t smem = AttnSmem<DIM, 2>::kBytes;
+  static_assert(AttnSmem<DIM, 2>::kBytes == AttnSmem<DIM, 3>::kBytes, "both kernels are launched with the same size");
   const bool causal = (p.flags & FASTAV_CAUSAL) != 0;
   const float scale = p.softmax_scale > 0.f ? p.softmax_scale : 1.0f / sqrtf((float)p.head_dim);
   AttnArgs a{};
@@ -837,31 +884,29 @@ cudaError_t run_layer(const fastav_params& p, const CUtensorMap& q_map, const CU
   a.group = p.num_q_heads / p.num_kv_heads;
   a.scale_log2 = scale * kLog2e;
   a.causal = causal ? 1 : 0;
-  const int blocks = a.n_pad / kTile;
-  a.items = attn_items(blocks, a.hq, causal);
   a.lse_parts = reinterpret_cast<float4*>(ws + w.lse_parts);
-  a.counters = reinterpret_cast<int*>(ws + w.counters);
-  a.n_counters = w.n_counters;
-  a.lse_opt = lse_opt;
-  a.alpha = alpha;
-  a.a_hi = reinterpret_cast<__nv_bfloat16*>(ws + w.a_hi);
-  a.a_lo = reinterpret_cast<__nv_bfloat16*>(ws + w.a_lo);
-  a.map_out = map_out;
-  a.partials = reinterpret_cast<float*>(ws + w.partials);
   a.device_status = device_status;
+  const int blocks = a.n_pad / kTile;
+  int* counters = reinterpret_cast<int*>(ws + w.counters);
   cudaError_t e = once_per_device([&] {
-    const cudaError_t f = cudaFuncSetAttribute(rollout_attn_kernel<DIM, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    return f == cudaSuccess ? cudaFuncSetAttribute(rollout_attn_kernel<DIM, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : f;
+    const cudaError_t f = cudaFuncSetAttribute(rollout_stats_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return f == cudaSuccess ? cudaFuncSetAttribute(rollout_map_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : f;
   });
   if (e != cudaSuccess) return e;
   if (lse_opt) {
-    e = cudaMemsetAsync(a.counters, 0, (size_t)w.n_counters * sizeof(int), stream);
+    e = cudaMemsetAsync(counters, 0, (size_t)w.n_counters * sizeof(int), stream);
   } else {
-    e = launch_chained(rollout_attn_kernel<DIM, 0>, dim3(stats_grid(blocks, a.hq, causal)), dim3(kThreads), smem, stream, q_map, k_map, a, ChainHead{});
+    e = launch_chained(rollout_stats_kernel<DIM>, dim3(stats_grid(blocks, a.hq, causal)), dim3(kThreads), smem, stream, q_map, k_map, a,
+                       visible_tiles(blocks, causal) * a.hq, counters, w.n_counters, ChainHead{});
     count_launches(1);
   }
   if (e != cudaSuccess) return e;
-  e = launch_chained(rollout_attn_kernel<DIM, 1>, dim3(map_grid(blocks, a.hq, causal)), dim3(kThreads), smem, stream, q_map, k_map, a, ChainHead{});
+  int whole, slices;
+  map_shares(blocks, causal, &whole, &slices);
+  const int work = whole + (int)(visible_tiles(blocks, causal) - whole) * slices;
+  const int zeros = map_out && causal ? (int)hidden_tiles(blocks) : 0;
+  e = launch_chained(rollout_map_kernel<DIM>, dim3(work + zeros), dim3(kThreads), smem, stream, q_map, k_map, a, lse_opt, alpha, whole, slices, work,
+                     reinterpret_cast<__nv_bfloat16*>(ws + w.a_hi), reinterpret_cast<__nv_bfloat16*>(ws + w.a_lo), map_out, ChainHead{});
   count_launches(1);
   return e;
 }
@@ -933,18 +978,20 @@ extern "C" int32_t fastav_rollout_layer(const fastav_params* p, const void* q, c
     return FASTAV_ERR_UNSUPPORTED;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   chain_begin(0);
-  cudaError_t e = p->head_dim == 128 ? run_layer<128>(*p, q_map, k_map, lse_opt, alpha, w, ws, map_out_opt, device_status, st)
-                                     : run_layer<64>(*p, q_map, k_map, lse_opt, alpha, w, ws, map_out_opt, device_status, st);
+  cudaError_t e = p->head_dim == 128 ? run_attention<128>(*p, q_map, k_map, lse_opt, alpha, w, ws, map_out_opt, device_status, st)
+                                     : run_attention<64>(*p, q_map, k_map, lse_opt, alpha, w, ws, map_out_opt, device_status, st);
   if (e != cudaSuccess) return FASTAV_ERR_CUDA;
   constexpr size_t gemm_smem = 3 * 4 * kSubTileBytes + sizeof(PipeControl) + 1024;
   e = once_per_device([] { return cudaFuncSetAttribute(rollout_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem); });
   if (e != cudaSuccess) return FASTAV_ERR_CUDA;
   const bool causal = (p->flags & FASTAV_CAUSAL) != 0;
-  const int blocks = n_pad / kTile;
-  e = launch_chained(rollout_gemm_kernel, dim3(gemm_grid(blocks, causal)), dim3(kThreads), gemm_smem, st, rt_hi_map, rt_lo_map, a_hi_map, a_lo_map,
-                     n_pad, causal ? 1 : 0, gemm_items(blocks, causal), causal ? 1 : 0, state_plane(state, n, dst, 0),
-                     state_plane(state, n, dst, 1), reinterpret_cast<float*>(ws + w.partials),
-                     reinterpret_cast<int*>(ws + w.counters) + blocks * blocks, device_status, ChainHead{});
+  const int blocks = n_pad / kTile, share = gemm_share(blocks, causal);
+  int units, cut;
+  gemm_units(blocks, causal, share, &units, &cut);
+  const int zeros = causal && layer_index == 0 ? (int)hidden_tiles(blocks) : 0;
+  e = launch_chained(rollout_gemm_kernel, dim3(units + zeros), dim3(kThreads), gemm_smem, st, rt_hi_map, rt_lo_map, a_hi_map, a_lo_map, n_pad,
+                     causal ? 1 : 0, share, units, state_plane(state, n, dst, 0), state_plane(state, n, dst, 1),
+                     reinterpret_cast<float*>(ws + w.partials), reinterpret_cast<int*>(ws + w.counters), device_status, ChainHead{});
   count_launches(1);
   return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? FASTAV_OK : FASTAV_ERR_CUDA;
 }
