@@ -114,7 +114,7 @@ __device__ __forceinline__ void pipe_setup(PipeControl& ctl, int stages, int war
     }
     for (int i = 0; i < kBuffers; ++i) {
       ptx::mbar_init(ptx::smem_u32(&ctl.tmem_full[i]), 1);
-      ptx::mbar_init(ptx::smem_u32(&ctl.tmem_empty[i]), kEpilogueThreads);
+      ptx::mbar_init(ptx::smem_u32(&ctl.tmem_empty[i]), kEpilogueThreads / 32);
     }
     for (int i = 0; i < 2; ++i) ptx::mbar_init(ptx::smem_u32(&ctl.q_empty[i]), 1);
     ctl.abort = 0;
@@ -259,7 +259,7 @@ rollout_stats_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
       if (*abort) drain_loads(ctl, it, kStages);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
       StatItem x(begin, blocks, causal);
       int loads = 0;
       for (int it = 0; it < count; ++it) {
@@ -269,12 +269,8 @@ rollout_stats_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
         ptx::tc_fence_after_sync();
         loads += it == 0 || x.jb == 0;
         const uint32_t k_tile = base + stage * kOperandBytes, q_tile = slots + ((loads - 1) & 1) * kOperandBytes;
-#pragma unroll
-        for (int ks = 0; ks < DIM / 16; ++ks) {
-          const uint32_t sub = ks / 4, off = (ks % 4) * 32;
-          ptx::umma_bf16(tmem + buf * kTile, ptx::umma_desc_sw128(q_tile + sub * kSubTileBytes, off),
-                         ptx::umma_desc_sw128(k_tile + sub * kSubTileBytes, off), ptx::umma_idesc_bf16(kTile, kTile), ks > 0);
-        }
+        ptx::umma_bf16_steps<DIM / 16, kSubTileBytes, kSubTileBytes>(tmem + buf * kTile, ptx::umma_desc_sw128(q_tile, 0),
+                                                                     ptx::umma_desc_sw128(k_tile, 0), ptx::umma_idesc_bf16(kTile, kTile), false);
         ptx::umma_commit(ptx::smem_u32(&ctl.empty[stage]));
         ptx::umma_commit(ptx::smem_u32(&ctl.tmem_full[buf]));
         if (x.row_ends()) ptx::umma_commit(ptx::smem_u32(&ctl.q_empty[(loads - 1) & 1]));
@@ -306,7 +302,7 @@ rollout_stats_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
         ptx::tmem_ld32(lane_addr + buf * kTile, v);
         ptx::tmem_ld_wait_for(v);
         ptx::tc_fence_before_sync();
-        ptx::mbar_arrive(ptx::smem_u32(&ctl.tmem_empty[buf]));  // the accumulator may be overwritten
+        ptx::mbar_arrive_warp(ptx::smem_u32(&ctl.tmem_empty[buf]), lane);  // the accumulator may be overwritten
         const int last_visible = min(a.n - 1, causal ? x.rb * kTile + row_in : INT_MAX);
         const int limit = last_visible - (x.jb * kTile + cg * 32);  // columns 0..limit of this group are visible
         if (limit < 31) {  // only tiles on the diagonal or at the end of the sequence
@@ -422,7 +418,7 @@ rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       if (*abort) drain_loads(ctl, it, kStages);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
       const uint32_t idesc = ptx::umma_idesc_bf16(kTile, width);
       for (int it = 0; it < hq; ++it) {
         const int stage = it % kStages, buf = it % kBuffers;
@@ -431,12 +427,8 @@ rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         ptx::tc_fence_after_sync();
         const uint32_t q_tile = base + stage * kOperandBytes;
         const uint32_t k_tile = slots + ((it / group) % kSlots) * kOperandBytes + col_first * 128;  // a multiple of 32 rows of 128 bytes
-#pragma unroll
-        for (int ks = 0; ks < DIM / 16; ++ks) {
-          const uint32_t sub = ks / 4, off = (ks % 4) * 32;
-          ptx::umma_bf16(tmem + buf * kTile, ptx::umma_desc_sw128(q_tile + sub * kSubTileBytes, off),
-                         ptx::umma_desc_sw128(k_tile + sub * kSubTileBytes, off), idesc, ks > 0);
-        }
+        ptx::umma_bf16_steps<DIM / 16, kSubTileBytes, kSubTileBytes>(tmem + buf * kTile, ptx::umma_desc_sw128(q_tile, 0),
+                                                                     ptx::umma_desc_sw128(k_tile, 0), idesc, false);
         ptx::umma_commit(ptx::smem_u32(&ctl.empty[stage]));
         ptx::umma_commit(ptx::smem_u32(&ctl.tmem_full[buf]));
       }
@@ -496,7 +488,7 @@ rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         ptx::tmem_ld_wait_for16(v);
       }
       ptx::tc_fence_before_sync();
-      ptx::mbar_arrive(ptx::smem_u32(&ctl.tmem_empty[buf]));  // the accumulator may be overwritten
+      ptx::mbar_arrive_warp(ptx::smem_u32(&ctl.tmem_empty[buf]), lane);  // the accumulator may be overwritten
       auto add = [&](int c) {  // columns c, c + 1
         float2 p = exp2_pair(__ffma2_rn(make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc, nl), c / 2);
         if (!whole_visible) {
@@ -636,7 +628,7 @@ rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_
       if (*abort) drain_loads(ctl, it, kStages);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
       bool ok = true;
       for (int it = 0; it < iters && ok; ++it) {
         const int stage = it % kStages;
@@ -645,14 +637,12 @@ rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_
         ptx::tc_fence_after_sync();
         const uint32_t rt_hi = base + stage * kStageBytes, rt_lo = rt_hi + kSubTileBytes, a_hi = rt_hi + 2 * kSubTileBytes,
                        a_lo = rt_hi + 3 * kSubTileBytes;
-#pragma unroll
-        for (int term = 0; term < 3; ++term) {
-          const uint32_t rt_tile = term == 1 ? rt_lo : rt_hi, a_tile = term == 2 ? a_lo : a_hi;
-#pragma unroll
-          for (int ks = 0; ks < 4; ++ks)
-            ptx::umma_bf16(tmem, ptx::umma_desc_sw128(rt_tile, ks * 32), ptx::umma_desc_sw128(a_tile, ks * 32),
-                           ptx::umma_idesc_bf16(kTile, kTile), (it > 0 || term > 0 || ks > 0) ? 1u : 0u);
-        }
+        const uint64_t rt_hi_desc = ptx::umma_desc_sw128(rt_hi, 0), rt_lo_desc = ptx::umma_desc_sw128(rt_lo, 0),
+                       a_hi_desc = ptx::umma_desc_sw128(a_hi, 0), a_lo_desc = ptx::umma_desc_sw128(a_lo, 0);
+        constexpr uint32_t idesc = ptx::umma_idesc_bf16(kTile, kTile);
+        ptx::umma_bf16_steps<4, 0, 0>(tmem, rt_hi_desc, a_hi_desc, idesc, it > 0);
+        ptx::umma_bf16_steps<4, 0, 0>(tmem, rt_lo_desc, a_hi_desc, idesc, true);
+        ptx::umma_bf16_steps<4, 0, 0>(tmem, rt_hi_desc, a_lo_desc, idesc, true);
         ptx::umma_commit(ptx::smem_u32(&ctl.empty[stage]));
       }
       if (ok) ptx::umma_commit(ptx::smem_u32(&ctl.tmem_full[0]));

@@ -81,6 +81,13 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
   }
 }
 
+// One arrival for a whole warp: 32 single ones queue at the barrier's word like atomics (an epilogue of 512 threads spends
+// more on them than on reading its accumulators).  Orders the warp's earlier shared-memory accesses before the arrival.
+__device__ __forceinline__ void mbar_arrive_warp(uint32_t bar, int lane) {
+  __syncwarp();
+  if (lane == 0) mbar_arrive(bar);
+}
+
 // ---- proxies and fences ------------------------------------------------------------------------
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -179,19 +186,30 @@ __host__ __device__ constexpr uint32_t umma_idesc_bf16(int m, int n) {
          | ((uint32_t)(m >> 4) << 24); // M / 16
 }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, issued by ONE thread.
+// D[tmem] (+)= A[smem] * B[smem]^T.  Called by a whole converged warp; one elected lane issues.  (A loop that one lane runs
+// alone keeps the descriptors in per-thread registers and issues at half the pace: eight MMAs 700 cycles instead of 420.)
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n\t"
-      ".reg .pred p;\n\t"
+      ".reg .pred p, q;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
+      "elect.sync _|q, 0xFFFFFFFF;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
       "}\n" ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// Makes `bar` receive one arrival when every MMA issued so far by this thread has finished.
+// The same over a K range of 16 STEPS elements: the 16-element slices of one 128-byte row lie 32 bytes apart, the next 64
+// elements `a_sub` / `b_sub` bytes further on.  The descriptors are made once and stepped by constants.
+template <int STEPS, int A_SUB, int B_SUB>
+__device__ __forceinline__ void umma_bf16_steps(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate) {
+#pragma unroll
+  for (int ks = 0; ks < STEPS; ++ks)
+    umma_bf16(d_tmem, a_desc + (uint64_t)((ks / 4) * (A_SUB >> 4) + (ks % 4) * 2), b_desc + (uint64_t)((ks / 4) * (B_SUB >> 4) + (ks % 4) * 2), idesc,
+              ks > 0 || accumulate ? 1u : 0u);
+}
+// Makes `bar` receive one arrival when every MMA issued so far has finished (whole warp, the same elected lane).
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xFFFFFFFF;\n\t@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar) : "memory");
 }
 
 __device__ __forceinline__ float ex2_approx(float x) {
