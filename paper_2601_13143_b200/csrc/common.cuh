@@ -165,11 +165,7 @@ struct Span {
   int first, count;
   bool bad;  // the array and the host scalars disagree: the span was clamped (FASTAV_DEV_SHAPE_MISMATCH)
 };
-// CACHED: the loads may stay in L1.  Only after the kernel's own wait (see below), and then worth it where thousands of
-// blocks read the same few words: through L2 alone they queue at one slice (32 sequences, 28,672 warps: 22 us instead of 11).
-template <bool CACHED = false>
-__device__ __forceinline__ Span checked_span(const int32_t* cu, int b, int total, int max_count) {
-  const int a = CACHED ? chain_load_cached(cu + b) : chain_load(cu + b), e = CACHED ? chain_load_cached(cu + b + 1) : chain_load(cu + b + 1);
+__device__ __forceinline__ Span checked_words(int a, int e, int total, int max_count) {  // of two consecutive prefix sums
   Span sp{a, e - a, false};
   if (a < 0 || a > total) {
     sp = Span{0, 0, true};
@@ -179,6 +175,13 @@ __device__ __forceinline__ Span checked_span(const int32_t* cu, int b, int total
     else if (sp.count > room) { sp.count = room; sp.bad = true; }
   }
   return sp;
+}
+// CACHED: the loads may stay in L1.  Only after the kernel's own wait (see below), and then worth it where thousands of
+// blocks read the same few words: through L2 alone they queue at one slice (32 sequences, 28,672 warps: 22 us instead of 11).
+template <bool CACHED = false>
+__device__ __forceinline__ Span checked_span(const int32_t* cu, int b, int total, int max_count) {
+  return checked_words(CACHED ? chain_load_cached(cu + b) : chain_load(cu + b), CACHED ? chain_load_cached(cu + b + 1) : chain_load(cu + b + 1),
+                       total, max_count);
 }
 template <bool CACHED = false>
 __device__ __forceinline__ Span seq_span(const Shapes& s, const int32_t* cu_seqlens, int b) {

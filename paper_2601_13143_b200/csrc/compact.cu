@@ -118,13 +118,13 @@ __device__ __forceinline__ bool make_segment(const Shapes& s, const RowStreams& 
 
 __global__ void __launch_bounds__(kBulkMaxWarps * 32, 1)
 compact_rows_bulk_kernel(Shapes s, RowStreams t, const int32_t* __restrict__ keep_idx, const int32_t* __restrict__ cu_keep,
-                         const int32_t* __restrict__ cu_seqlens, int n_segments, int packed_k, int packed_v, int row_bytes,
+                         const int32_t* __restrict__ cu_seqlens, int n_segments, int packed_k, int packed_v, int row_bytes, int slots,
                          int32_t* device_status) {
   extern __shared__ __align__(128) unsigned char bulk_smem[];
   __shared__ uint64_t full[kBulkMaxWarps][kBulkStages];
   chain_enter(s);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
-  const uint32_t ring = ptx::smem_u32(bulk_smem) + (uint32_t)warp * kBulkStages * row_bytes;
+  const uint32_t ring = ptx::smem_u32(bulk_smem) + (uint32_t)warp * slots * row_bytes;  // a warp with fewer rows than stages has that many slots
   Segment seg{};
   const bool active = lane < n_segments && make_segment(s, t, lane, packed_k != 0, packed_v != 0, seg);
   if (lane == 0) {
@@ -219,14 +219,17 @@ cudaError_t launch_compact(const Shapes& s, const int32_t* keep_idx, const int32
       kBulkStages * row_bytes <= kBulkSmemBudget) {
     int warps = kBulkSmemBudget / (kBulkStages * row_bytes);
     if (warps > kBulkMaxWarps) warps = kBulkMaxWarps;
-    const size_t smem = (size_t)warps * kBulkStages * row_bytes;
     cudaError_t e =
         once_per_device([] { return cudaFuncSetAttribute(compact_rows_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBulkSmemBudget); });
     if (e != cudaSuccess) return e;
     int blocks = (s.total_keep + warps - 1) / warps;
     if (blocks > kNumSMs) blocks = kNumSMs;
+    // No deeper rings than a warp has rows: the next call's first kernel then fits beside this one on the same SMs.
+    const int rows_per_warp = (s.total_keep + blocks * warps - 1) / (blocks * warps);
+    const int slots = rows_per_warp < kBulkStages ? rows_per_warp : kBulkStages;
+    const size_t smem = (size_t)warps * slots * row_bytes;
     e = launch_chained(compact_rows_bulk_kernel, dim3(blocks), dim3(warps * 32), smem, stream, s, t, keep_idx, cu_keep, cu_seqlens,
-                       n_segments, (int)packed_k, (int)packed_v, row_bytes, device_status);
+                       n_segments, (int)packed_k, (int)packed_v, row_bytes, slots, device_status);
     count_launches(1);
     return e != cudaSuccess ? e : cudaGetLastError();
   }
