@@ -142,8 +142,9 @@ Workspace plan_workspace(const fastav_params& p) {
   const size_t stat_entries = (size_t)2 * ((p.max_seqlen + 127) / 128);
   w.stats_off = carve(rows_heads * (stat_entries > (size_t)w.stat_tiles ? stat_entries : (size_t)w.stat_tiles) * sizeof(float2));
   w.lse_off = carve(rows_heads * sizeof(float));
-  w.partial_off = carve((size_t)p.num_kv_heads * wide_row_chunks(p.max_qlen, p.num_q_heads / p.num_kv_heads) *
-                        p.total_tokens * sizeof(float));
+  const int group = p.num_q_heads / p.num_kv_heads, wide_chunks = wide_row_chunks(p.max_qlen, group);
+  const int once_chunks = p.max_seqlen <= kOnceMaxTokens ? once_row_tiles(p.max_qlen, group) : 0;
+  w.partial_off = carve((size_t)p.num_kv_heads * (wide_chunks > once_chunks ? wide_chunks : once_chunks) * p.total_tokens * sizeof(float));
   const bool narrow = p.max_qlen >= 1 && p.max_qlen <= kNarrowMaxRows;
   w.logits_off = carve(narrow ? (size_t)p.num_q_heads * p.max_qlen * p.total_tokens * sizeof(float) : 0);
   w.keys_off = carve((size_t)p.total_tokens * sizeof(uint32_t));
@@ -176,7 +177,7 @@ cudaError_t launch_score(const Shapes& s, const Workspace& w, const void* q, con
     return launch_score_narrow(s, w, q, q_idx, cu_qlens, k, cu_seqlens, lse_in, scores_out, ws, device_status, stream, left);
   if (score_wide_applies(s)) {
     bool used = false;
-    const cudaError_t e = launch_score_wide(s, w, q, q_idx, cu_qlens, k, cu_seqlens, lse_in, scores_out, ws, device_status, stream, &used);
+    const cudaError_t e = launch_score_wide(s, w, q, q_idx, cu_qlens, k, cu_seqlens, lse_in, scores_out, ws, device_status, stream, &used, left);
     if (used || e != cudaSuccess) return e;
     if (forced == FASTAV_SCORE_PATH_WIDE) return cudaErrorNotSupported;
     // The tensor map could not be encoded: the CUDA-core tiles below are correct but far slower, so say so.
@@ -325,10 +326,15 @@ cudaError_t enqueue_selection(const fastav_params& params, const void* q, const 
   *gathered = false;
   if (s.total_tokens > 0) e = launch_score(s, w, q, q_idx, cu_qlens, k, cu_seqlens, lse_opt, scores_out, ws, device_status, st, &left);
   if (e != cudaSuccess) return e;
+  const SelectArgs t{cu_seqlens, keep_counts, protect_opt, q_idx, cu_qlens, keep_idx_out, cu_keep_out, device_status};
+  const int row_bytes = rows && s.total_keep > 0 ? row_bytes_of(s, *rows) : 0;
   if (left.kind == ScoreLeft::kKeys) {
-    *gathered = rows && s.total_keep > 0 && few_gathers(s, row_bytes_of(s, *rows));
-    return launch_few(s, q, k, lse_opt, scores_out, true, *gathered ? rows : nullptr, cu_seqlens, keep_counts, protect_opt, q_idx, cu_qlens,
-                      keep_idx_out, cu_keep_out, device_status, st);
+    *gathered = row_bytes > 0 && few_gathers(s, row_bytes);
+    return launch_few(s, q, k, lse_opt, scores_out, true, *gathered ? rows : nullptr, t, st);
+  }
+  if (left.kind == ScoreLeft::kPartials) {
+    *gathered = row_bytes > 0 && cluster_select_gathers(s, row_bytes);
+    return launch_select_partials(s, reinterpret_cast<const float*>(ws + w.partial_off), left, scores_out, *gathered ? rows : nullptr, t, st);
   }
   return launch_select(s, w, scores_out, cu_seqlens, keep_counts, protect_opt, q_idx, cu_qlens, keep_idx_out, cu_keep_out, ws, device_status, st);
 }

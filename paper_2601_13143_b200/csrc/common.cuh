@@ -30,7 +30,9 @@ struct ChainHead { int head_wait = 0; };
 
 // What a prune call still has to do after the scoring kernels, and from what.
 struct ScoreLeft {
-  enum Kind { kScores, kKeys } kind = kScores;  // finished scores; nothing done: the few-rows kernel starts from the keys
+  enum Kind { kScores, kKeys, kPartials } kind = kScores;  // finished scores; nothing done: the kernel that selects starts from
+                                                            // the keys; sums per (KV head, chunk of query rows) and token
+  int row_chunks = 0, rows_per_chunk = 0;                   // kPartials: most chunks of a KV head, query rows of a chunk
 };
 
 // Carved from the caller's workspace by plan_workspace(); all offsets 256-byte aligned.
@@ -82,21 +84,42 @@ int wide_row_chunks(int max_qlen, int group);
 bool score_wide_applies(const Shapes& s);
 cudaError_t launch_score_wide(const Shapes& s, const Workspace& w, const void* q, const int32_t* q_idx,
                               const int32_t* cu_qlens, const void* k, const int32_t* cu_seqlens, const float* lse_in,
-                              float* scores_out, unsigned char* ws, int32_t* device_status, cudaStream_t stream, bool* used);
+                              float* scores_out, unsigned char* ws, int32_t* device_status, cudaStream_t stream, bool* used, ScoreLeft* left);
 
 cudaError_t launch_logits_wide(const Shapes& s, const void* q, const int32_t* q_idx, const int32_t* cu_qlens, const void* k,
                                const int32_t* cu_seqlens, float* logits, int rq, int32_t* device_status, cudaStream_t stream,
                                bool* used);
 
-// Few scored rows on short sequences: one kernel from the keys to the keep list, or to the gathered rows (prune_few.cu).
+// The kernel that selects, a thread-block cluster per sequence (prune_few.cu): from the keys themselves (few scored rows, short
+// sequences), from partial sums or from finished scores, to the keep list, or to the gathered rows.
 struct RowStreams;
-bool few_applies(const Shapes& s);
+struct SelectArgs {
+  const int32_t *cu_seqlens, *keep_counts;
+  const uint8_t* protect;
+  const int32_t *q_idx, *cu_qlens;
+  int32_t *keep_idx, *cu_keep, *device_status;
+};
+bool few_applies(const Shapes& s);              // from the keys
+bool cluster_select_applies(const Shapes& s);   // from partial sums or scores
 bool few_gathers(const Shapes& s, int row_bytes);
+bool cluster_select_gathers(const Shapes& s, int row_bytes);
 // `rows`: what to gather in the same kernel (nullptr: nothing).
 cudaError_t launch_few(const Shapes& s, const void* q, const void* k, const float* lse_in, float* scores_out, bool do_select,
-                       const RowStreams* rows, const int32_t* cu_seqlens, const int32_t* keep_counts, const uint8_t* protect,
-                       const int32_t* q_idx, const int32_t* cu_qlens, int32_t* keep_idx, int32_t* cu_keep, int32_t* device_status,
-                       cudaStream_t stream);
+                       const RowStreams* rows, const SelectArgs& t, cudaStream_t stream);
+cudaError_t launch_select_partials(const Shapes& s, const float* partial, const ScoreLeft& left, float* scores_out, const RowStreams* rows,
+                                   const SelectArgs& t, cudaStream_t stream);
+cudaError_t launch_select_scores(const Shapes& s, const float* scores, const SelectArgs& t, cudaStream_t stream);
+
+// Many scored rows on short sequences: one pass over K (score_once.cu).
+struct OncePlan {
+  int rows_per_tile, row_tiles, blocks, tiles_per_block;
+};
+constexpr int kOnceMaxTokens = 4096;
+int once_row_tiles(int max_qlen, int group);
+bool once_plan(const Shapes& s, OncePlan* plan);
+cudaError_t launch_score_once(const Shapes& s, const void* k_map, const void* q_map, const int32_t* q_idx, const int32_t* cu_qlens,
+                              const int32_t* cu_seqlens, const float* lse_in, const OncePlan& plan, float* partial, int32_t* device_status,
+                              cudaStream_t stream);
 // Only the logits [Hq, max_qlen, N] of the few-rows path, into the workspace.
 cudaError_t launch_narrow_logits(const Shapes& s, const Workspace& w, const void* q, const int32_t* q_idx,
                                  const int32_t* cu_qlens, const void* k, const int32_t* cu_seqlens, unsigned char* ws,

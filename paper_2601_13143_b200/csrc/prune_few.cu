@@ -1,12 +1,14 @@
-// A prune call with few scored rows on short sequences, in ONE kernel: one thread-block CLUSTER per sequence goes from the
-// keys to the scores, the keep list and (where that is little) the survivors' rows.  This is the paper's own fine stage
-// (Section 2.2, "Fine pruning": one last-token query) on what the global stage left.
+// The kernel that selects: one thread-block CLUSTER per sequence goes from what scoring left to the keep list and (where that is
+// little) the survivors' rows.
 //
-//   logits  Q K^T by mma.sync, fragments loaded straight from global memory (see KeyFragment);
-//   scores  log-sum-exp per row and head (statistics per segment, exchanged through distributed shared memory, one
-//           cluster barrier), then per token the fixed-order sum over heads and rows (Eq. 4);
+//   front   kKeys: few scored rows on a short sequence, nothing done yet -- the paper's own fine stage (Section 2.2, "Fine
+//           pruning": one last-token query) on what the global stage left.  Q K^T by mma.sync, fragments loaded straight
+//           from global memory (see KeyFragment); log-sum-exp per row and head (statistics per segment, exchanged through
+//           distributed shared memory, one cluster barrier); then per token the fixed-order sum over heads and rows (Eq. 4).
+//           kPartials: the tensor-core kernels' sums per (KV head, chunk of query rows) and token are added up.
+//           kScores: finished scores (fastav_select).
 //   select  the scores as order-preserving 32-bit keys (protected tokens: the largest) go to every block of the cluster, a
-//           second cluster barrier, and each block runs the whole selection for itself: a histogram of the leading 12 bits,
+//           cluster barrier, and each block runs the whole selection for itself: a histogram of the leading 12 bits,
 //           the keys of the bin that holds the k-th largest finished by counting ranks (further 12-bit passes only if it holds
 //           more than 256), one stable prefix sum in index order;
 //   gather  the survivors among a block's own tokens.
@@ -30,7 +32,11 @@ namespace {
 
 constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
-constexpr int kMaxTokens = 4 * kThreads;  // four keys per thread in the selection
+constexpr int kKeysTokens = 4 * kThreads;     // kKeys: up to four keys per thread in the selection
+constexpr int kSelectTokens = 16 * kThreads;  // the other fronts: up to sixteen
+
+enum Front { kKeys, kPartials, kScores };
+
 constexpr int kDigitBits = 12;
 constexpr int kBins = 1 << kDigitBits;
 constexpr int kBinsPerThread = kBins / kThreads;
@@ -43,18 +49,22 @@ constexpr int kSegments = kMaxCluster;
 __host__ __device__ inline int segment_of(int n) { return n <= 32 * kSegments ? 32 : ((n + kSegments - 1) / kSegments + 31) & ~31; }
 
 struct FewArgs {
-  const uint16_t* q;
+  const uint16_t* q;    // kKeys
   const uint16_t* k;
-  const float* lse;     // optional: the caller's natural-log log-sum-exp [total_q, Hq]
-  float* scores_out;    // [N]
-  int rq;               // most scored rows of a sequence
+  const float* lse;     // kKeys, optional: the caller's natural-log log-sum-exp [total_q, Hq]
+  int rq;               // kKeys: most scored rows of a sequence
+  const float* in;      // kPartials [Hkv * row_chunks][N]; kScores [N]
+  int row_chunks, rows_per_chunk;  // kPartials
+  float* scores_out;    // [N] (not used by kScores)
   int do_select;        // 0: only the scores are wanted
   int do_gather;
   int slice_cap;        // tokens per block that shared memory was sized for
   RowStreams rows;      // do_gather
 };
 
+template <int PER>  // keys per thread in the selection
 struct alignas(16) FewShared {
+  static constexpr int kMaxTokens = PER * kThreads;
   unsigned hist[kBins];  // later: the block's survivors
   unsigned keys[kMaxTokens];
   unsigned prot_bits[kMaxTokens / 32];
@@ -66,7 +76,7 @@ struct alignas(16) FewShared {
   int base, list_n, remaining, bucket, need_eq, first_out, end_out, unused;
   unsigned prefix, threshold, unused2[2];
 };
-static_assert(sizeof(FewShared) % 16 == 0 && kBins >= kMaxTokens, "what follows it stays 16-byte aligned");
+static_assert(sizeof(FewShared<4>) % 16 == 0 && sizeof(FewShared<16>) % 16 == 0, "what follows it stays 16-byte aligned");
 
 // Dynamic shared memory after FewShared (bytes, every piece 16-byte aligned); host and device agree on it.
 struct FewLayout {
@@ -112,14 +122,16 @@ __device__ __forceinline__ void mma_16x8x16(float (&c)[4], unsigned a0, unsigned
                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-template <int DIM>
+template <Front FRONT, int DIM, int PER>
 __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArgs a, const int32_t* __restrict__ cu_seqlens,
                                                                 const int32_t* __restrict__ keep_counts,
                                                                 const uint8_t* __restrict__ protect, const int32_t* __restrict__ q_idx,
                                                                 const int32_t* __restrict__ cu_qlens, int32_t* __restrict__ keep_idx,
                                                                 int32_t* __restrict__ cu_keep, int32_t* device_status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  FewShared& sh = *reinterpret_cast<FewShared*>(smem_raw);
+  using Shared = FewShared<PER>;
+  constexpr int kMaxTokens = Shared::kMaxTokens;
+  Shared& sh = *reinterpret_cast<Shared*>(smem_raw);
   chain_enter(s, cu_seqlens, keep_counts, protect, q_idx, cu_qlens);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int blocks = (int)gridDim.x / s.batch;  // blocks per cluster
@@ -131,17 +143,18 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   const bool selecting = a.do_select != 0;
   if (warp == 0) {
     const int32_t* word = lane < 2 ? cu_seqlens + b + lane : lane < 4 ? cu_qlens + b + lane - 2 : keep_counts + b;
-    const int v = lane < 4 || (lane == 4 && selecting) ? chain_load(word) : 0;
+    const bool there = lane < 2 || (lane < 4 ? cu_qlens != nullptr : lane == 4 && selecting);
+    const int v = there ? chain_load(word) : 0;
     if (lane < 5) sh.index[lane] = v;
   } else {
     if (selecting)
       for (int i = tid - 32; i < kBins / 4; i += kThreads - 32) reinterpret_cast<uint4*>(sh.hist)[i] = make_uint4(0, 0, 0, 0);
-    if (tid - 32 < kMaxTokens / 32) sh.prot_bits[tid - 32] = 0u;
+    for (int i = tid - 32; i < kMaxTokens / 32; i += kThreads - 32) sh.prot_bits[i] = 0u;
     if (tid == 32) { sh.base = 0; sh.list_n = 0; }
   }
   __syncthreads();
   const Span seq = checked_words(sh.index[0], sh.index[1], s.total_tokens, s.max_seqlen);
-  const Span qrows = checked_words(sh.index[2], sh.index[3], s.total_q, s.max_qlen);
+  const Span qrows = checked_words(sh.index[2], sh.index[3], s.total_q, FRONT == kScores ? s.total_q : s.max_qlen);
   int k = sh.index[4];
   const bool k_clamped = k < 0 || k > seq.count;
   const int tok0 = seq.first, n = min(seq.count, a.slice_cap * blocks);
@@ -154,11 +167,47 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   k = k < 0 ? 0 : (k > n ? n : k);
 
   pdl_wait();
+  // The scored rows' tokens survive (kKeys also needs them as the rows' limits).
+  auto protect_rows = [&](int first_thread, int threads) {
+    if (selecting && (s.flags & FASTAV_PROTECT_QUERY_ROWS))
+      for (int r = tid - first_thread; r < all_rows; r += threads) {
+        const int j = chain_load(q_idx + qrows.first + r) - t0;  // relative to this block's first token
+        if (j >= 0 && j < m) atomicOr(&sh.prot_bits[j >> 5], 1u << (j & 31));
+      }
+  };
+  // What the selection needs and nothing has needed so far.
+  auto selection_inputs = [&] {
+    if (!selecting) return;
+    if (b > 0 && warp == kWarps - 1) {  // output offset: the clamped keep counts of the sequences before this one
+      int part = 0;
+      for (int i = lane; i < b; i += 32) {
+        const int ni = seq_span(s, cu_seqlens, i).count, ki = chain_load(keep_counts + i);
+        part += ki < 0 ? 0 : min(ki, ni);
+      }
+      part = __reduce_add_sync(0xFFFFFFFFu, part);
+      if (lane == 0) sh.base = part;
+    }
+    if (protect)
+      for (int j0 = warp * 32; j0 < m; j0 += kThreads) {  // a warp covers 32 tokens: one word
+        const int j = j0 + lane;
+        const unsigned word = __ballot_sync(0xFFFFFFFFu, j < m && chain_load(protect + tok0 + t0 + j) != 0);
+        if (lane == 0 && word) atomicOr(&sh.prot_bits[j0 >> 5], word);
+      }
+    if (tid == 0 && c == 0 && k_clamped && device_status) atomicOr(device_status, FASTAV_DEV_K_CLAMPED);
+  };
+  if (tid == 0 && (seq.bad || qrows.bad) && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
+  const bool lowest = (s.flags & FASTAV_SELECT_LOWEST) != 0;
+  auto key_of = [&](int j, float score) -> unsigned {  // token t0 + j of the sequence
+    unsigned x = order_key(lowest ? -score : score);
+    if (x == kProtectedKey) x = kProtectedKey - 1;  // only a NaN pattern lands here
+    return ((sh.prot_bits[j >> 5] >> (j & 31)) & 1u) ? kProtectedKey : x;
+  };
+  if constexpr (FRONT == kKeys) {
   pdl_acquire(a.q);
   pdl_acquire(a.k);
   // ---- logits ----------------------------------------------------------------------------------------------
   const FewLayout lay = few_layout(a.slice_cap, s.hq * a.rq, DIM);
-  unsigned char* const more = smem_raw + sizeof(FewShared);
+  unsigned char* const more = smem_raw + sizeof(Shared);
   constexpr int kQStride = DIM * 2 + 64;
   unsigned char* const q_sh = more + lay.q;
   float* const lse = reinterpret_cast<float*>(more + lay.lse);
@@ -184,12 +233,9 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
     sh.term_of[tid] = (tid % s.group) * rows + tid / s.group;
   }
   if (warp == 0) {
-    // The scored rows' tokens: what each row may see, and (protected) that they survive.
-    for (int r = lane; r < max(kNarrowMaxRows, all_rows); r += 32) {
-      const int j = r < all_rows ? chain_load(q_idx + qrows.first + r) - t0 : 0x7FFFFFFF;  // relative to this block's first token
-      if (r < kNarrowMaxRows) sh.limit[r] = causal && r < rows ? j : 0x7FFFFFFF;
-      if (selecting && (s.flags & FASTAV_PROTECT_QUERY_ROWS) && j >= 0 && j < m) atomicOr(&sh.prot_bits[j >> 5], 1u << (j & 31));
-    }
+    // what each scored row may see, relative to this block's first token
+    if (lane < kNarrowMaxRows) sh.limit[lane] = causal && lane < rows ? chain_load(q_idx + qrows.first + lane) - t0 : 0x7FFFFFFF;
+    protect_rows(0, 32);
   }
   __syncthreads();
   for (int u = warp; u < units; u += kWarps) {
@@ -223,25 +269,7 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
       }
     }
   }
-  if (selecting) {
-    if (b > 0 && warp == kWarps - 1) {  // output offset: the clamped keep counts of the sequences before this one
-      int part = 0;
-      for (int i = lane; i < b; i += 32) {
-        const int ni = seq_span(s, cu_seqlens, i).count, ki = chain_load(keep_counts + i);
-        part += ki < 0 ? 0 : min(ki, ni);
-      }
-      part = __reduce_add_sync(0xFFFFFFFFu, part);
-      if (lane == 0) sh.base = part;
-    }
-    if (protect)
-      for (int j0 = warp * 32; j0 < m; j0 += kThreads) {  // a warp covers 32 tokens: one word
-        const int j = j0 + lane;
-        const unsigned word = __ballot_sync(0xFFFFFFFFu, j < m && chain_load(protect + tok0 + t0 + j) != 0);
-        if (lane == 0 && word) atomicOr(&sh.prot_bits[j0 >> 5], word);
-      }
-    if (tid == 0 && c == 0 && k_clamped && device_status) atomicOr(device_status, FASTAV_DEV_K_CLAMPED);
-  }
-  if (tid == 0 && (seq.bad || qrows.bad) && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
+  selection_inputs();  // arrives while other warps still multiply
   cluster_wait();
   __syncthreads();
 
@@ -303,7 +331,6 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   __syncthreads();
 
   // ---- scores: eight lanes per token, each every eighth term in ascending order, added in a fixed tree ---------
-  const bool lowest = (s.flags & FASTAV_SELECT_LOWEST) != 0;
   const float inv = all_rows > 0 ? 1.0f / ((float)s.hq * (float)all_rows) : 0.f;
   const int part = tid & (kTokenLanes - 1);
 #pragma unroll 1
@@ -321,28 +348,69 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
     if (j < m) {
       if (part == 0) a.scores_out[tok0 + t0 + j] = score;
       if (selecting) {
-        unsigned x = order_key(lowest ? -score : score);
-        if (x == kProtectedKey) x = kProtectedKey - 1;  // only a NaN pattern lands here
-        if ((sh.prot_bits[j >> 5] >> (j & 31)) & 1u) x = kProtectedKey;
+        const unsigned x = key_of(j, score);
         for (int q = part; q < blocks; q += kTokenLanes) remote_store(remote(&sh.keys[t0 + j], q), x);  // to every block of the cluster
       }
+    }
+  }
+  } else {
+    // ---- scores from partial sums, or as they are --------------------------------------------------------------------
+    const float* in = a.in;
+    pdl_acquire(in);
+    protect_rows(0, kThreads);
+    selection_inputs();
+    cluster_wait();
+    __syncthreads();
+    const float* const col = in + tok0 + t0;
+    if constexpr (FRONT == kPartials) {
+      const int row_chunks = (all_rows * s.group + a.rows_per_chunk - 1) / a.rows_per_chunk, terms = s.hkv * row_chunks;
+      const float inv = all_rows > 0 ? 1.0f / ((float)s.hq * (float)all_rows) : 0.f;
+      for (int j = tid; j < m; j += kThreads) {
+        // Partial i = (KV head, row chunk) in that order; sixteen loads in flight, one running sum in fixed order.
+        float total = 0.f;
+        int g = 0, rc = 0;  // (KV head, row chunk) of the next term, stepped along instead of divided out
+        for (int i0 = 0; i0 < terms; i0 += 16) {
+          float v[16];
+#pragma unroll
+          for (int u = 0; u < 16; ++u) {
+            v[u] = i0 + u < terms ? chain_load(col + (long long)(g * a.row_chunks + rc) * s.total_tokens + j) : 0.f;
+            if (++rc == row_chunks) { rc = 0; ++g; }
+          }
+#pragma unroll
+          for (int u = 0; u < 16; ++u) total += v[u];
+        }
+        const float score = total * inv;
+        a.scores_out[tok0 + t0 + j] = score;
+        sh.keys[t0 + j] = key_of(j, score);
+      }
+    } else {
+#pragma unroll 4
+      for (int j = tid; j < m; j += kThreads) sh.keys[t0 + j] = key_of(j, chain_load(col + j));
+    }
+    __syncthreads();
+    // This block's keys to everybody else, 16 bytes at a time (what lies past the last token is never read).
+    const int quads = (m + 3) / 4;
+    for (int q = 0; q < blocks; ++q) {
+      if (q == c) continue;
+      for (int i = tid; i < quads; i += kThreads) remote_store4(remote(&sh.keys[t0 + 4 * i], q), *reinterpret_cast<const uint4*>(&sh.keys[t0 + 4 * i]));
     }
   }
   if (!selecting) return;  // uniform for the cluster; nothing remote is outstanding
   cluster_sync();          // the last remote access: from here on every block works for itself
 
-  // ---- selection: thread t owns the tokens 4 t .. 4 t + 3 of the whole sequence ----------------------------------
+  // ---- selection: thread t owns the tokens PER t .. PER t + PER - 1 of the whole sequence ----------------------------------
   const int base = sh.base;
   if (c == 0 && tid == 0) {
     cu_keep[b + 1] = base + k;
     if (b == 0) cu_keep[0] = 0;
   }
   if (k == 0) return;  // uniform for the cluster
-  const int mine = max(0, min(4, n - 4 * tid));
-  unsigned x[4];
-  {
-    const uint4 v = *reinterpret_cast<const uint4*>(&sh.keys[4 * tid]);
-    x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+  const int mine = max(0, min(PER, n - PER * tid));
+  unsigned x[PER];
+#pragma unroll
+  for (int u = 0; u < PER; u += 4) {
+    const uint4 v = *reinterpret_cast<const uint4*>(&sh.keys[PER * tid + u]);
+    x[u] = v.x; x[u + 1] = v.y; x[u + 2] = v.z; x[u + 3] = v.w;
   }
   unsigned prefix = 0u;   // the bits of the k-th largest key fixed so far
   int remaining = k, bits_left = 32;
@@ -357,7 +425,7 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
     {
       unsigned run_digit = kBins, run_len = 0u;  // equal digits of consecutive tokens (typically zeros): one update
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < PER; ++u) {
         if (u < mine && __funnelshift_rc(x[u], 0u, bits_left) == above_want) {
           const unsigned digit = (x[u] >> shift) & (kBins - 1);
           if (digit != run_digit) {
@@ -397,7 +465,7 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
     bits_left = shift;
     if (bits_left > 0 && sh.bucket <= kDirectMax) {  // few keys left: collect them, each finds its rank by counting
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+      for (int u = 0; u < PER; ++u)
         if (u < mine && (x[u] >> bits_left) == (prefix >> bits_left)) sh.list[atomicAdd(&sh.list_n, 1)] = x[u];
       __syncthreads();
       rank_finish(sh.list, sh.list_n, remaining, tid, &sh.threshold, &sh.need_eq);
@@ -411,23 +479,23 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   const int need_eq = remaining;  // how many keys equal to T are kept: the lowest-index ones
   unsigned both = 0;              // keys above the threshold in the low half, keys equal to it in the high half
 #pragma unroll
-  for (int u = 0; u < 4; ++u) both += u < mine ? (x[u] > T ? 1u : 0u) + (x[u] == T ? 0x10000u : 0u) : 0u;
+  for (int u = 0; u < PER; ++u) both += u < mine ? (x[u] > T ? 1u : 0u) + (x[u] == T ? 0x10000u : 0u) : 0u;
   const unsigned before = sum_before<kWarps>(both, sh.warp_a, lane, warp);
   int gt = (int)(before & 0xFFFFu), eq = (int)(before >> 16);
   if (c == 0 && tid == kThreads - 1 && T == kProtectedKey && eq + (int)(both >> 16) > need_eq && device_status)
     atomicOr(device_status, FASTAV_DEV_PROTECT_OVERFLOW);  // more protected tokens than k
   const bool global_idx = (s.flags & FASTAV_KEEP_IDX_GLOBAL) != 0;
-  if (4 * tid == t0) sh.first_out = gt + min(eq, need_eq);   // t0 is a multiple of 32
-  if (4 * tid == t0 + m) sh.end_out = gt + min(eq, need_eq); // so is the end of a slice, but for the last one's
-  unsigned* const picked = sh.hist;                          // survivor `out` of the sequence is token picked[out % 2048]
-  if (4 * tid >= t0 && 4 * tid < t0 + m) {
+  if (PER * tid == t0) sh.first_out = gt + min(eq, need_eq);   // t0 is a multiple of 32
+  if (PER * tid == t0 + m) sh.end_out = gt + min(eq, need_eq); // so is the end of a slice, but for the last one's
+  unsigned* const picked = sh.hist;                          // survivor `out` of the sequence is token picked[out % 4096]
+  if (PER * tid >= t0 && PER * tid < t0 + m) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < PER; ++u) {
       const bool is_gt = x[u] > T, is_eq = x[u] == T;
       if (u < mine && (is_gt || (is_eq && eq < need_eq))) {
-        const int out = gt + min(eq, need_eq), j = 4 * tid + u;
+        const int out = gt + min(eq, need_eq), j = PER * tid + u;
         keep_idx[base + out] = (global_idx ? tok0 : 0) + j;
-        picked[out & (kMaxTokens - 1)] = (unsigned)j;
+        picked[out & (kBins - 1)] = (unsigned)j;
       }
       gt += is_gt;
       eq += is_eq;
@@ -441,7 +509,7 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   const int first = sh.first_out, count = min((t0 + m == n ? k : sh.end_out) - first, s.total_keep - base - first);
   if (a.rows.pos_in)
     for (int i = tid; i < count; i += kThreads)
-      a.rows.pos_out[base + first + i] = chain_load(a.rows.pos_in + tok0 + picked[(first + i) & (kMaxTokens - 1)]);
+      a.rows.pos_out[base + first + i] = chain_load(a.rows.pos_in + tok0 + picked[(first + i) & (kBins - 1)]);
   const unsigned magic = 0xFFFFFFFFu / (unsigned)shape.n_chunks + 1u;  // e / n_chunks = umulhi(e, magic) while e * n_chunks < 2^32
   const int chunks = count * shape.n_chunks;
   constexpr int kUnroll = 6;
@@ -455,7 +523,7 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
       if (e < chunks) {
         row[u] = shape.n_chunks == 1 ? e : (int)__umulhi((unsigned)e, magic);
         chunk[u] = e - row[u] * shape.n_chunks;
-        v[u] = load_stream(chunk_in(s, a.rows, shape, (long long)tok0 + picked[(first + row[u]) & (kMaxTokens - 1)], chunk[u]));
+        v[u] = load_stream(chunk_in(s, a.rows, shape, (long long)tok0 + picked[(first + row[u]) & (kBins - 1)], chunk[u]));
       }
     }
 #pragma unroll
@@ -476,36 +544,61 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
 
 int slice_of(const Shapes& s, int blocks) { return segment_of(s.max_seqlen) * (kSegments / blocks); }  // tokens per block
 
-size_t smem_of(const Shapes& s, int blocks) {
-  return sizeof(FewShared) + few_layout(slice_of(s, blocks), s.hq * s.max_qlen, s.dim).total;
+size_t smem_keys(const Shapes& s, int blocks) {
+  return sizeof(FewShared<4>) + few_layout(slice_of(s, blocks), s.hq * s.max_qlen, s.dim).total;
 }
 
 constexpr size_t kMaxDynamic = 220 * 1024;
 
+#ifndef FASTAV_SELECT_SLICE
+#define FASTAV_SELECT_SLICE 128
+#endif
 // Blocks per sequence.  FEW_CLUSTER_RULE
-int cluster_of(const Shapes& s) {
+int cluster_for(const Shapes& s, int slice) {
   int blocks = FASTAV_FEW_CLUSTER;
-  while (blocks > 1 && ((long long)s.batch * blocks > kNumSMs || s.max_seqlen <= blocks / 2 * FASTAV_FEW_SLICE)) blocks /= 2;
-  while (blocks < kMaxCluster && smem_of(s, blocks) > kMaxDynamic) blocks *= 2;
+  while (blocks > 1 && ((long long)s.batch * blocks > kNumSMs || s.max_seqlen <= blocks / 2 * slice)) blocks /= 2;
+  return blocks;
+}
+int cluster_keys(const Shapes& s) {
+  int blocks = cluster_for(s, FASTAV_FEW_SLICE);
+  while (blocks < kMaxCluster && smem_keys(s, blocks) > kMaxDynamic) blocks *= 2;
+  return blocks;
+}
+int cluster_select(const Shapes& s) {
+  int blocks = cluster_for(s, FASTAV_SELECT_SLICE);
+  while (slice_of(s, blocks) > kBins) blocks *= 2;  // a block's survivors have to fit the histogram's place
   return blocks;
 }
 
-template <int DIM>
-cudaError_t launch(const Shapes& s, FewArgs a, const int32_t* cu_seqlens, const int32_t* keep_counts, const uint8_t* protect,
-                   const int32_t* q_idx, const int32_t* cu_qlens, int32_t* keep_idx, int32_t* cu_keep, int32_t* device_status,
-                   cudaStream_t stream) {
-  const int blocks = cluster_of(s);
+template <Front FRONT, int DIM, int PER>
+cudaError_t launch(const Shapes& s, FewArgs a, int blocks, size_t smem, const RowStreams* rows, const SelectArgs& t, cudaStream_t stream) {
   a.slice_cap = slice_of(s, blocks);
-  cudaError_t e = once_per_device([] {
-    cudaError_t f = cudaFuncSetAttribute(prune_few_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamic);
-    if (f == cudaSuccess) f = cudaFuncSetAttribute(prune_few_kernel<DIM>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (rows) {
+    a.do_gather = 1;
+    a.rows = *rows;
+  }
+  const auto kernel = prune_few_kernel<FRONT, DIM, PER>;
+  cudaError_t e = once_per_device([&] {
+    cudaError_t f = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamic);
+    if (f == cudaSuccess) f = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return f;
   });
   if (e != cudaSuccess) return e;
-  e = launch_chained_cluster(prune_few_kernel<DIM>, dim3(s.batch * blocks), dim3(kThreads), blocks, smem_of(s, blocks), stream, s, a,
-                             cu_seqlens, keep_counts, protect, q_idx, cu_qlens, keep_idx, cu_keep, device_status);
+  e = launch_chained_cluster(kernel, dim3(s.batch * blocks), dim3(kThreads), blocks, smem, stream, s, a, t.cu_seqlens, t.keep_counts,
+                             t.protect, t.q_idx, t.cu_qlens, t.keep_idx, t.cu_keep, t.device_status);
   count_launches(1);
   return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <Front FRONT>
+cudaError_t launch_from(const Shapes& s, const FewArgs& a, const RowStreams* rows, const SelectArgs& t, cudaStream_t stream) {
+  const int blocks = cluster_select(s);
+  return s.max_seqlen <= kKeysTokens ? launch<FRONT, 128, 4>(s, a, blocks, sizeof(FewShared<4>), rows, t, stream)
+                                     : launch<FRONT, 128, 16>(s, a, blocks, sizeof(FewShared<16>), rows, t, stream);
+}
+
+bool little(const Shapes& s, int blocks, int row_bytes) {
+  return row_bytes > 0 && (long long)((s.max_keep + blocks - 1) / blocks) * row_bytes <= FASTAV_GATHER_BYTES;
 }
 
 }  // namespace
@@ -514,19 +607,16 @@ cudaError_t launch(const Shapes& s, FewArgs a, const int32_t* cu_seqlens, const 
 bool few_applies(const Shapes& s) {
   if ((s.flags & FASTAV_SCORE_PATH_MASK) != 0) return false;
   if (s.max_qlen < 1 || s.max_qlen > kNarrowMaxRows || s.max_qlen * s.group > 128) return false;
-  return s.max_seqlen >= 1 && s.max_seqlen <= kMaxTokens && smem_of(s, cluster_of(s)) <= kMaxDynamic;
+  return s.max_seqlen >= 1 && s.max_seqlen <= kKeysTokens && smem_keys(s, cluster_keys(s)) <= kMaxDynamic;
 }
+bool cluster_select_applies(const Shapes& s) { return s.max_seqlen <= kSelectTokens; }
 
 // The survivors' rows may be copied by the blocks that select them: worth it while that is little per block (GATHER_RULE).
-bool few_gathers(const Shapes& s, int row_bytes) {
-  const int blocks = cluster_of(s);
-  return row_bytes > 0 && (long long)((s.max_keep + blocks - 1) / blocks) * row_bytes <= FASTAV_GATHER_BYTES;
-}
+bool few_gathers(const Shapes& s, int row_bytes) { return little(s, cluster_keys(s), row_bytes); }
+bool cluster_select_gathers(const Shapes& s, int row_bytes) { return little(s, cluster_select(s), row_bytes); }
 
 cudaError_t launch_few(const Shapes& s, const void* q, const void* k, const float* lse_in, float* scores_out, bool do_select,
-                       const RowStreams* rows, const int32_t* cu_seqlens, const int32_t* keep_counts, const uint8_t* protect,
-                       const int32_t* q_idx, const int32_t* cu_qlens, int32_t* keep_idx, int32_t* cu_keep, int32_t* device_status,
-                       cudaStream_t stream) {
+                       const RowStreams* rows, const SelectArgs& t, cudaStream_t stream) {
   FewArgs a{};
   a.q = static_cast<const uint16_t*>(q);
   a.k = static_cast<const uint16_t*>(k);
@@ -534,12 +624,27 @@ cudaError_t launch_few(const Shapes& s, const void* q, const void* k, const floa
   a.scores_out = scores_out;
   a.rq = s.max_qlen;
   a.do_select = do_select ? 1 : 0;
-  if (rows) {
-    a.do_gather = 1;
-    a.rows = *rows;
-  }
-  return s.dim == 128 ? launch<128>(s, a, cu_seqlens, keep_counts, protect, q_idx, cu_qlens, keep_idx, cu_keep, device_status, stream)
-                      : launch<64>(s, a, cu_seqlens, keep_counts, protect, q_idx, cu_qlens, keep_idx, cu_keep, device_status, stream);
+  const int blocks = cluster_keys(s);
+  return s.dim == 128 ? launch<kKeys, 128, 4>(s, a, blocks, smem_keys(s, blocks), rows, t, stream)
+                      : launch<kKeys, 64, 4>(s, a, blocks, smem_keys(s, blocks), rows, t, stream);
+}
+
+cudaError_t launch_select_partials(const Shapes& s, const float* partial, const ScoreLeft& left, float* scores_out, const RowStreams* rows,
+                                   const SelectArgs& t, cudaStream_t stream) {
+  FewArgs a{};
+  a.in = partial;
+  a.row_chunks = left.row_chunks;
+  a.rows_per_chunk = left.rows_per_chunk;
+  a.scores_out = scores_out;
+  a.do_select = 1;
+  return launch_from<kPartials>(s, a, rows, t, stream);
+}
+
+cudaError_t launch_select_scores(const Shapes& s, const float* scores, const SelectArgs& t, cudaStream_t stream) {
+  FewArgs a{};
+  a.in = scores;
+  a.do_select = 1;
+  return launch_from<kScores>(s, a, nullptr, t, stream);
 }
 
 }  // namespace fastav

@@ -365,8 +365,8 @@ cudaError_t launch_score_narrow(const Shapes& s, const Workspace& w, const void*
       left->kind = ScoreLeft::kKeys;
       return cudaSuccess;
     }
-    return launch_few(s, q, k, lse_in, scores_out, false, nullptr, cu_seqlens, nullptr, nullptr, q_idx, cu_qlens, nullptr, nullptr,
-                      device_status, stream);
+    return launch_few(s, q, k, lse_in, scores_out, false, nullptr, SelectArgs{cu_seqlens, nullptr, nullptr, q_idx, cu_qlens, nullptr, nullptr, device_status},
+                      stream);
   }
   cudaError_t e = launch_narrow_logits(s, w, q, q_idx, cu_qlens, k, cu_seqlens, ws, device_status, stream);
   if (e != cudaSuccess) return e;

@@ -1,0 +1,368 @@
+// Importance score, Eq. 4 (Section 2.2), for many scored rows on SHORT sequences: one pass over K.
+//
+// The long-sequence path (score_wide.cu) sweeps K twice because its logits fit nowhere.  Here they do: a thread-block cluster
+// owns one tile of 128 query rows of one KV head, its blocks share out the keys, and a block's logits -- 128 rows x up to 512
+// keys in fp32 -- stay in its 256 KB of tensor memory.  So
+//
+//   S = Q K^T per key tile (tcgen05.mma, operands by TMA), read once for (max, sum 2^(z - max)) per row and key tile; the
+//   blocks exchange those through distributed shared memory (one cluster barrier); each block then works out its rows'
+//   log2-sum-exp2 and reads S again: 2^(z - lse), summed over the 128 rows of every key by a butterfly that leaves one
+//   key per lane -> partial[KV head, row tile][token], which the selecting kernel (prune_few.cu) adds up.
+//
+// Two kernels (this and the selection) replace five (two sweeps, merge, per-token sums, selection).  Bound: latency, the
+// chip is far from full.  ONCE_FIGURES
+//
+// A key's sums do not depend on its position (every column goes through the same arithmetic and the same tree), and a
+// row's statistics are kept per key tile and folded in tile order, so that equal keys get bit-equal scores and a sequence's
+// scores do not depend on the cluster's size.  All waits are bounded.
+#include <cuda.h>
+#include <limits.h>
+
+#include "cluster.cuh"
+#include "common.cuh"
+#include "sm100_ptx.cuh"
+
+namespace fastav {
+namespace {
+
+constexpr int kTile = 128;                 // query rows of a tile; keys of a key tile
+constexpr int kThreads = 576;              // warp 0: TMA, warp 1: MMA, warps 2-17: epilogue
+constexpr int kEpilogueThreads = 512;
+constexpr int kBlockTiles = 4;             // key tiles of a block: 512 columns of tensor memory
+constexpr int kMaxTiles = kOnceMaxTokens / kTile;  // key tiles of a sequence
+constexpr int kTmemCols = 512;
+constexpr int kSubTileBytes = kTile * 128;
+
+struct alignas(16) Control {
+  uint64_t q_full, k_full[kBlockTiles], s_full[kBlockTiles];
+  uint32_t tmem_base;
+  int abort;
+  int index[4];
+  int limit[kTile];                            // last key each row may see (-1: no such row)
+  float neg_lse[kTile];
+  float2 part[4][kBlockTiles][kTile];          // (max, sum) per column group, key tile, row
+  float2 stats[kMaxTiles][kTile];              // per key tile of the sequence: written by all blocks of the cluster
+  float colsum[kBlockTiles][4][kTile];         // per key tile and 32-row quarter, the sums of every key
+};
+
+template <int DIM>
+struct Layout {
+  static constexpr int kOperandBytes = (DIM / 64) * kSubTileBytes;
+  static constexpr size_t kBytes = (size_t)(1 + kBlockTiles) * kOperandBytes + sizeof(Control) + 1024;
+};
+
+__device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueThreads) : "memory"); }
+
+// Lane j gets the sum over the warp's lanes of v[j]: at each step a lane gives away the half its partner keeps.
+__device__ __forceinline__ float transpose_sum(float (&v)[32], int lane) {
+#pragma unroll
+  for (int half = 16; half >= 1; half >>= 1) {
+    const bool upper = (lane & half) != 0;
+#pragma unroll
+    for (int i = 0; i < half; ++i) {
+      const float send = upper ? v[i] : v[i + half];
+      const float keep = upper ? v[i + half] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, half);
+    }
+  }
+  return v[0];
+}
+
+template <int DIM>
+__global__ void __launch_bounds__(kThreads, 1)
+score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap q_map, Shapes s,
+                  const int32_t* __restrict__ q_idx, const int32_t* __restrict__ cu_qlens, const int32_t* __restrict__ cu_seqlens,
+                  const float* lse_in, int blocks, int rows_per_tile, int row_tiles, int tiles_per_block, float* __restrict__ partial,
+                  int32_t* device_status) {
+  using L = Layout<DIM>;
+  constexpr int kSubTiles = DIM / 64;
+  extern __shared__ unsigned char smem_raw[];
+  chain_enter(s, q_idx, cu_qlens, cu_seqlens);
+  cluster_arrive();  // "this block runs": waited for before the first remote access
+  const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
+  const uint32_t q_smem = base, k_smem = base + L::kOperandBytes;
+  Control& ctl = *reinterpret_cast<Control*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + (1 + kBlockTiles) * L::kOperandBytes);
+  volatile int* abort = &ctl.abort;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int c = (int)cluster_rank(), id = (int)blockIdx.x / blocks;
+  const int rt = id % row_tiles, g = id / row_tiles % s.hkv, b = id / row_tiles / s.hkv;
+
+  if (warp == 0) {  // the sequence's bounds, asked for by one warp
+    const int32_t* word = lane < 2 ? cu_seqlens + b + lane : cu_qlens + b + (lane & 1);
+    if (lane < 4) ctl.index[lane] = chain_load(word);
+  } else if (warp == 1) {
+    if (lane == 0) {
+      ptx::mbar_init(ptx::smem_u32(&ctl.q_full), 1);
+      for (int i = 0; i < kBlockTiles; ++i) {
+        ptx::mbar_init(ptx::smem_u32(&ctl.k_full[i]), 1);
+        ptx::mbar_init(ptx::smem_u32(&ctl.s_full[i]), 1);
+      }
+      ctl.abort = 0;
+      ptx::fence_barrier_init();
+      ptx::prefetch_tensormap(&k_map);
+      ptx::prefetch_tensormap(&q_map);
+    }
+    __syncwarp();
+    ptx::tmem_alloc(ptx::smem_u32(&ctl.tmem_base), kTmemCols);
+    ptx::tmem_relinquish();
+  } else {
+    // The query tile starts as zeros: rows no copy ever fills are then harmless operands.
+    for (int i = threadIdx.x - 64; i < L::kOperandBytes / 16; i += kEpilogueThreads)
+      asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(q_smem + i * 16), "r"(0) : "memory");
+    ptx::fence_proxy_async_smem();  // ordered before the TMA writes that follow the barrier
+  }
+  ptx::tc_fence_before_sync();
+  __syncthreads();
+  ptx::tc_fence_after_sync();
+  const uint32_t tmem = ctl.tmem_base;
+  const Span seq = checked_words(ctl.index[0], ctl.index[1], s.total_tokens, s.max_seqlen);
+  const Span rows = checked_words(ctl.index[2], ctl.index[3], s.total_q, s.max_qlen);
+  if (threadIdx.x == 0 && (seq.bad || rows.bad) && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
+  const int n = min(seq.count, blocks * tiles_per_block * kTile);
+  const int rows_here = min(rows_per_tile, rows.count * s.group - rt * rows_per_tile);  // of this row tile (a multiple of G)
+  const int tiles = rows_here > 0 ? (n + kTile - 1) / kTile : 0;                         // key tiles of the sequence
+  const int t0 = min(tiles, c * tiles_per_block), mine = min(tiles - t0, tiles_per_block);
+  const bool causal = (s.flags & FASTAV_CAUSAL) != 0;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      pdl_wait();  // q and k may be what earlier work wrote
+      if (mine > 0) {
+        // Boxes of 8 scored rows x G heads x 64 columns land as 8 G consecutive 128-byte rows: the flat (scored row, head)
+        // order of the tile, a whole number of 1024-byte swizzle groups.
+        const int boxes = (rows_here / s.group + 7) / 8;
+        const uint32_t box_bytes = 8u * s.group * 128u, bar = ptx::smem_u32(&ctl.q_full);
+        ptx::mbar_arrive_expect_tx(bar, boxes * box_bytes * kSubTiles);
+        for (int t = 0; t < mine; ++t) ptx::mbar_arrive_expect_tx(ptx::smem_u32(&ctl.k_full[t]), L::kOperandBytes);
+        for (int sub = 0; sub < kSubTiles; ++sub)
+          ptx::tma_load_3d(k_smem + sub * kSubTileBytes, &k_map, sub * 64, g, seq.first + t0 * kTile, ptx::smem_u32(&ctl.k_full[0]));
+        for (int sub = 0; sub < kSubTiles; ++sub)
+          for (int i = 0; i < boxes; ++i)
+            ptx::tma_load_3d(q_smem + sub * kSubTileBytes + i * box_bytes, &q_map, sub * 64, g * s.group,
+                             rows.first + rt * (rows_per_tile / s.group) + 8 * i, bar);
+        for (int t = 1; t < mine; ++t)
+          for (int sub = 0; sub < kSubTiles; ++sub)
+            ptx::tma_load_3d(k_smem + t * L::kOperandBytes + sub * kSubTileBytes, &k_map, sub * 64, g, seq.first + (t0 + t) * kTile,
+                             ptx::smem_u32(&ctl.k_full[t]));
+        // The copies write into this block's shared memory: they have to be waited for before it may exit.
+        int never = 0;
+        ptx::mbar_wait_bounded(bar, 0, &never);
+        for (int t = 0; t < mine; ++t) ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.k_full[t]), 0, &never);
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    bool ok = mine <= 0 || ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.q_full), 0, abort);
+    for (int t = 0; t < mine && ok; ++t) {
+      ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.k_full[t]), 0, abort);
+      if (!ok) break;
+      ptx::tc_fence_after_sync();
+      ptx::umma_bf16_steps<DIM / 16, kSubTileBytes, kSubTileBytes>(tmem + t * kTile, ptx::umma_desc_sw128(q_smem, 0),
+                                                                   ptx::umma_desc_sw128(k_smem + t * L::kOperandBytes, 0),
+                                                                   ptx::umma_idesc_bf16(kTile, kTile), false);
+      ptx::umma_commit(ptx::smem_u32(&ctl.s_full[t]));
+    }
+    __syncwarp();
+  }
+  const int quarter = warp & 3, cg = (warp - 2) >> 2;  // epilogue: TMEM lanes 32 quarter .., columns 32 cg .. of every key tile
+  const int row_in = quarter * 32 + lane, ethread = cg * kTile + row_in;
+  const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16) + cg * 32;
+  const float scale = s.scale_log2;
+  const float2 sc = make_float2(scale, scale);
+  bool ok = true;
+  int limit = -1;
+  if (warp >= 2) {
+    pdl_wait();
+    pdl_acquire(lse_in);
+    if (cg == 0) {  // one column group asks, all four need it
+      const int f = rt * rows_per_tile + row_in;
+      int last = -1;
+      float nl = -INFINITY;
+      if (row_in < rows_here) {
+        const int r = rows.first + f / s.group;
+        last = min(n - 1, causal ? chain_load(q_idx + r) : INT_MAX);
+        if (lse_in) {
+          const float v = chain_load(lse_in + (long long)r * s.hq + g * s.group + f % s.group);
+          nl = v == v && fabsf(v) != INFINITY ? -v * kLog2e : -INFINITY;  // a row that sees no key adds 0
+        }
+      }
+      ctl.limit[row_in] = last;
+      ctl.neg_lse[row_in] = nl;
+    }
+    epilogue_sync();
+    limit = ctl.limit[row_in];
+    if (!lse_in) {
+      for (int t = 0; t < mine; ++t) {
+        if (ok) ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.s_full[t]), 0, abort);
+        if (!ok) break;
+        ptx::tc_fence_after_sync();
+        uint32_t v[32];
+        ptx::tmem_ld32(lane_addr + t * kTile, v);
+        ptx::tmem_ld_wait_for(v);
+        const int bound = limit - ((t0 + t) * kTile + cg * 32);  // columns 0..bound are visible
+        if (bound < 31) {
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            if (j > bound) v[j] = 0xFF800000u;  // -inf
+        }
+        float m0 = -INFINITY, m1 = -INFINITY;
+#pragma unroll
+        for (int j = 0; j < 32; j += 4) {
+          m0 = fmaxf(m0, fmaxf(__uint_as_float(v[j]), __uint_as_float(v[j + 1])));
+          m1 = fmaxf(m1, fmaxf(__uint_as_float(v[j + 2]), __uint_as_float(v[j + 3])));
+        }
+        const float m = fmaxf(m0, m1), shift = m == -INFINITY ? 0.f : -m * scale;
+        float2 sum = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int j = 0; j < 32; j += 2) {
+          const float2 z = __ffma2_rn(make_float2(__uint_as_float(v[j]), __uint_as_float(v[j + 1])), sc, make_float2(shift, shift));
+          sum = __fadd2_rn(sum, make_float2(ptx::ex2_approx(z.x), ptx::ex2_approx(z.y)));
+        }
+        ctl.part[cg][t][row_in] = make_float2(m * scale, sum.x + sum.y);
+        __syncwarp();  // rows differ in `bound`; the tcgen05 instructions that follow need the whole warp
+      }
+    }
+  }
+  __syncwarp();
+  cluster_wait();  // every block of the cluster runs
+  if (!lse_in) {
+    if (warp >= 2) {
+      epilogue_sync();
+      const int t = ethread >> 7, row = ethread & (kTile - 1);
+      if (ok && t < mine) {  // one thread per (key tile, row): the four column groups, and off to every block
+        float m = -INFINITY, l = 0.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) m = fmaxf(m, ctl.part[i][t][row].x);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float2 p = ctl.part[i][t][row];
+          if (p.x > -INFINITY) l += p.y * ptx::ex2_approx(p.x - m);
+        }
+        for (int q = 0; q < blocks; ++q) remote_store2(remote(&ctl.stats[t0 + t][row], q), __float_as_uint(m), __float_as_uint(l));
+      }
+    }
+    cluster_sync();  // the last remote access
+  }
+
+  if (warp >= 2) {
+    if (!lse_in) {
+      // Each row's key tiles in four interleaved runs, in order, then the four.
+      const int j = ethread >> 7, row = ethread & (kTile - 1);
+      float m = -INFINITY, l = 0.f;
+      for (int t = j; t < tiles; t += 4) m = fmaxf(m, ctl.stats[t][row].x);
+      for (int t = j; t < tiles; t += 4) {
+        const float2 p = ctl.stats[t][row];
+        if (p.x > -INFINITY) l += p.y * ptx::ex2_approx(p.x - m);
+      }
+      ctl.part[j][0][row] = make_float2(m, l);
+      epilogue_sync();
+      if (ethread < kTile) {
+        float mm = -INFINITY, total = 0.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) mm = fmaxf(mm, ctl.part[i][0][ethread].x);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float2 p = ctl.part[i][0][ethread];
+          if (p.x > -INFINITY) total += p.y * ptx::ex2_approx(p.x - mm);
+        }
+        ctl.neg_lse[ethread] = total > 0.f && ethread < rows_here ? -(mm + __log2f(total)) : -INFINITY;
+      }
+      epilogue_sync();
+    }
+    const float nl = ctl.neg_lse[row_in];
+    const float2 nl2 = make_float2(nl, nl);
+    for (int t = 0; t < mine; ++t) {
+      if (ok) ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.s_full[t]), 0, abort);
+      if (!ok) break;
+      ptx::tc_fence_after_sync();
+      uint32_t v[32];
+      ptx::tmem_ld32(lane_addr + t * kTile, v);
+      ptx::tmem_ld_wait_for(v);
+      const int bound = limit - ((t0 + t) * kTile + cg * 32);
+      float p[32];
+#pragma unroll
+      for (int j = 0; j < 32; j += 2) {
+        const float2 z = __ffma2_rn(make_float2(__uint_as_float(v[j]), __uint_as_float(v[j + 1])), sc, nl2);
+        p[j] = ptx::ex2_approx(z.x);
+        p[j + 1] = ptx::ex2_approx(z.y);
+      }
+      if (bound < 31) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+          if (j > bound) p[j] = 0.f;
+      }
+      __syncwarp();
+      ctl.colsum[t][quarter][cg * 32 + lane] = transpose_sum(p, lane);
+    }
+    epilogue_sync();
+    const int t = ethread >> 7, col = ethread & (kTile - 1), key = (t0 + t) * kTile + col;
+    if (ok && t < mine && key < n)
+      partial[(long long)(g * row_tiles + rt) * s.total_tokens + seq.first + key] =
+          (ctl.colsum[t][0][col] + ctl.colsum[t][1][col]) + (ctl.colsum[t][2][col] + ctl.colsum[t][3][col]);
+  }
+
+  // ---- teardown: everybody meets here, whatever happened above ------------------------------------
+  ptx::tc_fence_before_sync();
+  __syncthreads();
+  if (warp == 1) {
+    ptx::tc_fence_after_sync();
+    ptx::tmem_dealloc(tmem, kTmemCols);
+  }
+  if (threadIdx.x == 0 && ctl.abort && device_status) atomicOr(device_status, FASTAV_DEV_WAIT_EXPIRED);
+}
+
+template <int DIM>
+cudaError_t launch(const Shapes& s, const CUtensorMap& k_map, const CUtensorMap& q_map, const int32_t* q_idx, const int32_t* cu_qlens,
+                   const int32_t* cu_seqlens, const float* lse_in, const OncePlan& plan, float* partial, int32_t* device_status, cudaStream_t stream) {
+  const size_t smem = Layout<DIM>::kBytes;
+  cudaError_t e = once_per_device([&] {
+    cudaError_t f = cudaFuncSetAttribute(score_once_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (f == cudaSuccess) f = cudaFuncSetAttribute(score_once_kernel<DIM>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return f;
+  });
+  if (e != cudaSuccess) return e;
+  e = launch_chained_cluster(score_once_kernel<DIM>, dim3(s.batch * s.hkv * plan.row_tiles * plan.blocks), dim3(kThreads), plan.blocks, smem, stream,
+                             k_map, q_map, s, q_idx, cu_qlens, cu_seqlens, lse_in, plan.blocks, plan.rows_per_tile, plan.row_tiles,
+                             plan.tiles_per_block, partial, device_status);
+  count_launches(1);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+}  // namespace
+
+// Query rows of a tile: whole TMA boxes of 8 scored rows x G heads (0: no box fits).
+int once_rows_per_tile(int group) { return group >= 1 && group <= 16 ? kTile / (8 * group) * (8 * group) : 0; }
+int once_row_tiles(int max_qlen, int group) {
+  const int per = once_rows_per_tile(group);
+  return per == 0 ? 0 : (max_qlen * group + per - 1) / per;
+}
+
+#ifndef FASTAV_ONCE_WAVES
+#define FASTAV_ONCE_WAVES 1
+#endif
+bool once_plan(const Shapes& s, OncePlan* plan) {
+  plan->rows_per_tile = once_rows_per_tile(s.group);
+  if (plan->rows_per_tile == 0 || s.max_seqlen < 1 || s.max_qlen < 1) return false;
+  plan->row_tiles = once_row_tiles(s.max_qlen, s.group);
+  const int tiles = (s.max_seqlen + kTile - 1) / kTile;
+  if (tiles > kMaxTiles) return false;
+  const long long clusters = (long long)s.batch * s.hkv * plan->row_tiles;
+  // One key tile per block as long as all blocks run at once, up to four otherwise (ONCE_RULE).
+  int blocks = 1;
+  while (blocks < tiles && blocks < kMaxCluster) blocks *= 2;
+  while (blocks > 1 && clusters * blocks > (long long)FASTAV_ONCE_WAVES * kNumSMs && tiles <= blocks / 2 * kBlockTiles) blocks /= 2;
+  plan->blocks = blocks;
+  plan->tiles_per_block = (tiles + blocks - 1) / blocks;
+  return plan->tiles_per_block <= kBlockTiles && clusters * blocks <= (long long)FASTAV_ONCE_WAVES * kNumSMs;
+}
+
+cudaError_t launch_score_once(const Shapes& s, const void* k_map, const void* q_map, const int32_t* q_idx, const int32_t* cu_qlens,
+                              const int32_t* cu_seqlens, const float* lse_in, const OncePlan& plan, float* partial, int32_t* device_status,
+                              cudaStream_t stream) {
+  const CUtensorMap& km = *static_cast<const CUtensorMap*>(k_map);
+  const CUtensorMap& qm = *static_cast<const CUtensorMap*>(q_map);
+  return s.dim == 128 ? launch<128>(s, km, qm, q_idx, cu_qlens, cu_seqlens, lse_in, plan, partial, device_status, stream)
+                      : launch<64>(s, km, qm, q_idx, cu_qlens, cu_seqlens, lse_in, plan, partial, device_status, stream);
+}
+
+}  // namespace fastav

@@ -714,10 +714,27 @@ cudaError_t run_logits(const Shapes& s, const CUtensorMap& k_map, const CUtensor
 template <int DIM>
 cudaError_t run(const Shapes& s, const Workspace& w, const CUtensorMap& k_map, const CUtensorMap& q_map, const int32_t* q_idx,
                 const int32_t* cu_qlens, const int32_t* cu_seqlens, const float* lse_in, float* scores_out, unsigned char* ws,
-                int32_t* device_status, cudaStream_t stream) {
+                int32_t* device_status, cudaStream_t stream, ScoreLeft* left) {
   float2* stats = reinterpret_cast<float2*>(ws + w.stats_off);
   float* lse = reinterpret_cast<float*>(ws + w.lse_off);
   float* partial = reinterpret_cast<float*>(ws + w.partial_off);
+  // Partial sums per (KV head, chunk of query rows) -> scores: by the kernel that selects, or here.
+  auto finish = [&](int row_chunks, int chunk) -> cudaError_t {
+    if (left && cluster_select_applies(s)) {
+      left->kind = ScoreLeft::kPartials;
+      left->row_chunks = row_chunks;
+      left->rows_per_chunk = chunk;
+      return cudaSuccess;
+    }
+    count_launches(1);
+    return launch_chained(score_wide_finalize_kernel, dim3((s.max_seqlen + kFinalizeThreads - 1) / kFinalizeThreads, s.batch),
+                          dim3(kFinalizeThreads), 0, stream, s, cu_seqlens, cu_qlens, row_chunks, chunk, (const float*)partial, scores_out);
+  };
+  OncePlan once;
+  if (scores_out && (s.flags & FASTAV_SCORE_PATH_MASK) == 0 && once_plan(s, &once)) {
+    const cudaError_t f = launch_score_once(s, &k_map, &q_map, q_idx, cu_qlens, cu_seqlens, lse_in, once, partial, device_status, stream);
+    return f != cudaSuccess ? f : finish(once.row_tiles, once.rows_per_tile);
+  }
   const int rows_per_chunk = wide_rows_per_chunk(s.group);
   const int rc_max = wide_row_chunks(s.max_qlen, s.group);
   int grid, chunk_tiles;
@@ -750,11 +767,8 @@ cudaError_t run(const Shapes& s, const Workspace& w, const CUtensorMap& k_map, c
                           cu_seqlens, chunk_tiles, stat_chunks, rc_max, rows_per_chunk, (float2*)nullptr, (const float*)lse,
                           partial, (float*)nullptr, 0, device_status)) != cudaSuccess)
     return e;
-  if ((e = launch_chained(score_wide_finalize_kernel, dim3((s.max_seqlen + kFinalizeThreads - 1) / kFinalizeThreads, s.batch),
-                          dim3(kFinalizeThreads), 0, stream, s,
-                          cu_seqlens, cu_qlens, rc_max, rows_per_chunk, (const float*)partial, scores_out)) != cudaSuccess)
-    return e;
-  count_launches(2);
+  count_launches(1);
+  if ((e = finish(rc_max, rows_per_chunk)) != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
@@ -803,13 +817,14 @@ cudaError_t launch_logits_wide(const Shapes& s, const void* q, const int32_t* q_
 
 cudaError_t launch_score_wide(const Shapes& s, const Workspace& w, const void* q, const int32_t* q_idx,
                               const int32_t* cu_qlens, const void* k, const int32_t* cu_seqlens, const float* lse_in,
-                              float* scores_out, unsigned char* ws, int32_t* device_status, cudaStream_t stream, bool* used) {
+                              float* scores_out, unsigned char* ws, int32_t* device_status, cudaStream_t stream, bool* used,
+                              ScoreLeft* left) {
   CUtensorMap k_map, q_map;
   *used = make_map(k, s.dim, s.hkv, s.total_tokens, s.k_st, s.k_sh, 1, kTileKeys, &k_map) &&
           make_map(q, s.dim, s.hq, s.total_q, s.q_st, s.q_sh, s.group, 8, &q_map);
   if (!*used) return cudaSuccess;  // the caller falls back to the CUDA-core path
-  if (s.dim == 128) return run<128>(s, w, k_map, q_map, q_idx, cu_qlens, cu_seqlens, lse_in, scores_out, ws, device_status, stream);
-  return run<64>(s, w, k_map, q_map, q_idx, cu_qlens, cu_seqlens, lse_in, scores_out, ws, device_status, stream);
+  if (s.dim == 128) return run<128>(s, w, k_map, q_map, q_idx, cu_qlens, cu_seqlens, lse_in, scores_out, ws, device_status, stream, left);
+  return run<64>(s, w, k_map, q_map, q_idx, cu_qlens, cu_seqlens, lse_in, scores_out, ws, device_status, stream, left);
 }
 
 }  // namespace fastav

@@ -350,6 +350,8 @@ cudaError_t launch_select(const Shapes& s, const Workspace& w, const float* scor
   const size_t want = fixed + ((size_t)s.max_seqlen + s.max_seqlen / 32 + 1) * sizeof(unsigned);
   constexpr size_t kMaxDynamic = 227 * 1024 - 1024;
   cudaError_t e;
+  if (cluster_select_applies(s))
+    return launch_select_scores(s, scores, SelectArgs{cu_seqlens, keep_counts, protect, q_idx, cu_qlens, keep_idx, cu_keep, device_status}, stream);
   if (s.max_seqlen > kBlockedMinKeys && s.max_seqlen <= kBlockedMaxKeys) {
     // the fewest tokens per thread that cover the longest sequence: all 1024 threads share the work
     if (s.max_seqlen <= kThreads * 4) e = launch_blocked<4>(s, scores, cu_seqlens, keep_counts, protect, q_idx, cu_qlens, keep_idx, cu_keep, device_status, stream);
