@@ -32,8 +32,8 @@ namespace {
 
 constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
-constexpr int kKeysTokens = 4 * kThreads;     // kKeys: up to four keys per thread in the selection
-constexpr int kSelectTokens = 16 * kThreads;  // the other fronts: up to sixteen
+constexpr int kPer = 4;                    // keys per thread in the selection
+constexpr int kMaxTokens = kPer * kThreads;
 
 enum Front { kKeys, kPartials, kScores };
 
@@ -62,9 +62,7 @@ struct FewArgs {
   RowStreams rows;      // do_gather
 };
 
-template <int PER>  // keys per thread in the selection
 struct alignas(16) FewShared {
-  static constexpr int kMaxTokens = PER * kThreads;
   unsigned hist[kBins];  // later: the block's survivors
   unsigned keys[kMaxTokens];
   unsigned prot_bits[kMaxTokens / 32];
@@ -76,7 +74,7 @@ struct alignas(16) FewShared {
   int base, list_n, remaining, bucket, need_eq, first_out, end_out, unused;
   unsigned prefix, threshold, unused2[2];
 };
-static_assert(sizeof(FewShared<4>) % 16 == 0 && sizeof(FewShared<16>) % 16 == 0, "what follows it stays 16-byte aligned");
+static_assert(sizeof(FewShared) % 16 == 0 && kBins >= kMaxTokens, "what follows it stays 16-byte aligned");
 
 // Dynamic shared memory after FewShared (bytes, every piece 16-byte aligned); host and device agree on it.
 struct FewLayout {
@@ -122,16 +120,14 @@ __device__ __forceinline__ void mma_16x8x16(float (&c)[4], unsigned a0, unsigned
                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-template <Front FRONT, int DIM, int PER>
+template <Front FRONT, int DIM>
 __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArgs a, const int32_t* __restrict__ cu_seqlens,
                                                                 const int32_t* __restrict__ keep_counts,
                                                                 const uint8_t* __restrict__ protect, const int32_t* __restrict__ q_idx,
                                                                 const int32_t* __restrict__ cu_qlens, int32_t* __restrict__ keep_idx,
                                                                 int32_t* __restrict__ cu_keep, int32_t* device_status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  using Shared = FewShared<PER>;
-  constexpr int kMaxTokens = Shared::kMaxTokens;
-  Shared& sh = *reinterpret_cast<Shared*>(smem_raw);
+  FewShared& sh = *reinterpret_cast<FewShared*>(smem_raw);
   chain_enter(s, cu_seqlens, keep_counts, protect, q_idx, cu_qlens);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int blocks = (int)gridDim.x / s.batch;  // blocks per cluster
@@ -207,7 +203,7 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   pdl_acquire(a.k);
   // ---- logits ----------------------------------------------------------------------------------------------
   const FewLayout lay = few_layout(a.slice_cap, s.hq * a.rq, DIM);
-  unsigned char* const more = smem_raw + sizeof(Shared);
+  unsigned char* const more = smem_raw + sizeof(FewShared);
   constexpr int kQStride = DIM * 2 + 64;
   unsigned char* const q_sh = more + lay.q;
   float* const lse = reinterpret_cast<float*>(more + lay.lse);
@@ -398,18 +394,18 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   if (!selecting) return;  // uniform for the cluster; nothing remote is outstanding
   cluster_sync();          // the last remote access: from here on every block works for itself
 
-  // ---- selection: thread t owns the tokens PER t .. PER t + PER - 1 of the whole sequence ----------------------------------
+  // ---- selection: thread t owns the tokens 4 t .. 4 t + 3 of the whole sequence ----------------------------------
   const int base = sh.base;
   if (c == 0 && tid == 0) {
     cu_keep[b + 1] = base + k;
     if (b == 0) cu_keep[0] = 0;
   }
   if (k == 0) return;  // uniform for the cluster
-  const int mine = max(0, min(PER, n - PER * tid));
-  unsigned x[PER];
+  const int mine = max(0, min(kPer, n - kPer * tid));
+  unsigned x[kPer];
 #pragma unroll
-  for (int u = 0; u < PER; u += 4) {
-    const uint4 v = *reinterpret_cast<const uint4*>(&sh.keys[PER * tid + u]);
+  for (int u = 0; u < kPer; u += 4) {
+    const uint4 v = *reinterpret_cast<const uint4*>(&sh.keys[kPer * tid + u]);
     x[u] = v.x; x[u + 1] = v.y; x[u + 2] = v.z; x[u + 3] = v.w;
   }
   unsigned prefix = 0u;   // the bits of the k-th largest key fixed so far
@@ -425,7 +421,7 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
     {
       unsigned run_digit = kBins, run_len = 0u;  // equal digits of consecutive tokens (typically zeros): one update
 #pragma unroll
-      for (int u = 0; u < PER; ++u) {
+      for (int u = 0; u < kPer; ++u) {
         if (u < mine && __funnelshift_rc(x[u], 0u, bits_left) == above_want) {
           const unsigned digit = (x[u] >> shift) & (kBins - 1);
           if (digit != run_digit) {
@@ -465,7 +461,7 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
     bits_left = shift;
     if (bits_left > 0 && sh.bucket <= kDirectMax) {  // few keys left: collect them, each finds its rank by counting
 #pragma unroll
-      for (int u = 0; u < PER; ++u)
+      for (int u = 0; u < kPer; ++u)
         if (u < mine && (x[u] >> bits_left) == (prefix >> bits_left)) sh.list[atomicAdd(&sh.list_n, 1)] = x[u];
       __syncthreads();
       rank_finish(sh.list, sh.list_n, remaining, tid, &sh.threshold, &sh.need_eq);
@@ -479,21 +475,21 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   const int need_eq = remaining;  // how many keys equal to T are kept: the lowest-index ones
   unsigned both = 0;              // keys above the threshold in the low half, keys equal to it in the high half
 #pragma unroll
-  for (int u = 0; u < PER; ++u) both += u < mine ? (x[u] > T ? 1u : 0u) + (x[u] == T ? 0x10000u : 0u) : 0u;
+  for (int u = 0; u < kPer; ++u) both += u < mine ? (x[u] > T ? 1u : 0u) + (x[u] == T ? 0x10000u : 0u) : 0u;
   const unsigned before = sum_before<kWarps>(both, sh.warp_a, lane, warp);
   int gt = (int)(before & 0xFFFFu), eq = (int)(before >> 16);
   if (c == 0 && tid == kThreads - 1 && T == kProtectedKey && eq + (int)(both >> 16) > need_eq && device_status)
     atomicOr(device_status, FASTAV_DEV_PROTECT_OVERFLOW);  // more protected tokens than k
   const bool global_idx = (s.flags & FASTAV_KEEP_IDX_GLOBAL) != 0;
-  if (PER * tid == t0) sh.first_out = gt + min(eq, need_eq);   // t0 is a multiple of 32
-  if (PER * tid == t0 + m) sh.end_out = gt + min(eq, need_eq); // so is the end of a slice, but for the last one's
+  if (kPer * tid == t0) sh.first_out = gt + min(eq, need_eq);   // t0 is a multiple of 32
+  if (kPer * tid == t0 + m) sh.end_out = gt + min(eq, need_eq); // so is the end of a slice, but for the last one's
   unsigned* const picked = sh.hist;                          // survivor `out` of the sequence is token picked[out % 4096]
-  if (PER * tid >= t0 && PER * tid < t0 + m) {
+  if (kPer * tid >= t0 && kPer * tid < t0 + m) {
 #pragma unroll
-    for (int u = 0; u < PER; ++u) {
+    for (int u = 0; u < kPer; ++u) {
       const bool is_gt = x[u] > T, is_eq = x[u] == T;
       if (u < mine && (is_gt || (is_eq && eq < need_eq))) {
-        const int out = gt + min(eq, need_eq), j = PER * tid + u;
+        const int out = gt + min(eq, need_eq), j = kPer * tid + u;
         keep_idx[base + out] = (global_idx ? tok0 : 0) + j;
         picked[out & (kBins - 1)] = (unsigned)j;
       }
@@ -545,13 +541,13 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
 int slice_of(const Shapes& s, int blocks) { return segment_of(s.max_seqlen) * (kSegments / blocks); }  // tokens per block
 
 size_t smem_keys(const Shapes& s, int blocks) {
-  return sizeof(FewShared<4>) + few_layout(slice_of(s, blocks), s.hq * s.max_qlen, s.dim).total;
+  return sizeof(FewShared) + few_layout(slice_of(s, blocks), s.hq * s.max_qlen, s.dim).total;
 }
 
 constexpr size_t kMaxDynamic = 220 * 1024;
 
 #ifndef FASTAV_SELECT_SLICE
-#define FASTAV_SELECT_SLICE 128
+#define FASTAV_SELECT_SLICE 256
 #endif
 // Blocks per sequence.  FEW_CLUSTER_RULE
 int cluster_for(const Shapes& s, int slice) {
@@ -564,20 +560,16 @@ int cluster_keys(const Shapes& s) {
   while (blocks < kMaxCluster && smem_keys(s, blocks) > kMaxDynamic) blocks *= 2;
   return blocks;
 }
-int cluster_select(const Shapes& s) {
-  int blocks = cluster_for(s, FASTAV_SELECT_SLICE);
-  while (slice_of(s, blocks) > kBins) blocks *= 2;  // a block's survivors have to fit the histogram's place
-  return blocks;
-}
+int cluster_select(const Shapes& s) { return cluster_for(s, FASTAV_SELECT_SLICE); }
 
-template <Front FRONT, int DIM, int PER>
+template <Front FRONT, int DIM>
 cudaError_t launch(const Shapes& s, FewArgs a, int blocks, size_t smem, const RowStreams* rows, const SelectArgs& t, cudaStream_t stream) {
   a.slice_cap = slice_of(s, blocks);
   if (rows) {
     a.do_gather = 1;
     a.rows = *rows;
   }
-  const auto kernel = prune_few_kernel<FRONT, DIM, PER>;
+  const auto kernel = prune_few_kernel<FRONT, DIM>;
   cudaError_t e = once_per_device([&] {
     cudaError_t f = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamic);
     if (f == cudaSuccess) f = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -593,8 +585,7 @@ cudaError_t launch(const Shapes& s, FewArgs a, int blocks, size_t smem, const Ro
 template <Front FRONT>
 cudaError_t launch_from(const Shapes& s, const FewArgs& a, const RowStreams* rows, const SelectArgs& t, cudaStream_t stream) {
   const int blocks = cluster_select(s);
-  return s.max_seqlen <= kKeysTokens ? launch<FRONT, 128, 4>(s, a, blocks, sizeof(FewShared<4>), rows, t, stream)
-                                     : launch<FRONT, 128, 16>(s, a, blocks, sizeof(FewShared<16>), rows, t, stream);
+  return launch<FRONT, 128>(s, a, blocks, sizeof(FewShared), rows, t, stream);
 }
 
 bool little(const Shapes& s, int blocks, int row_bytes) {
@@ -607,9 +598,9 @@ bool little(const Shapes& s, int blocks, int row_bytes) {
 bool few_applies(const Shapes& s) {
   if ((s.flags & FASTAV_SCORE_PATH_MASK) != 0) return false;
   if (s.max_qlen < 1 || s.max_qlen > kNarrowMaxRows || s.max_qlen * s.group > 128) return false;
-  return s.max_seqlen >= 1 && s.max_seqlen <= kKeysTokens && smem_keys(s, cluster_keys(s)) <= kMaxDynamic;
+  return s.max_seqlen >= 1 && s.max_seqlen <= kMaxTokens && smem_keys(s, cluster_keys(s)) <= kMaxDynamic;
 }
-bool cluster_select_applies(const Shapes& s) { return s.max_seqlen <= kSelectTokens; }
+bool cluster_select_applies(const Shapes& s) { return s.max_seqlen <= kMaxTokens; }
 
 // The survivors' rows may be copied by the blocks that select them: worth it while that is little per block (GATHER_RULE).
 bool few_gathers(const Shapes& s, int row_bytes) { return little(s, cluster_keys(s), row_bytes); }
@@ -625,8 +616,8 @@ cudaError_t launch_few(const Shapes& s, const void* q, const void* k, const floa
   a.rq = s.max_qlen;
   a.do_select = do_select ? 1 : 0;
   const int blocks = cluster_keys(s);
-  return s.dim == 128 ? launch<kKeys, 128, 4>(s, a, blocks, smem_keys(s, blocks), rows, t, stream)
-                      : launch<kKeys, 64, 4>(s, a, blocks, smem_keys(s, blocks), rows, t, stream);
+  return s.dim == 128 ? launch<kKeys, 128>(s, a, blocks, smem_keys(s, blocks), rows, t, stream)
+                      : launch<kKeys, 64>(s, a, blocks, smem_keys(s, blocks), rows, t, stream);
 }
 
 cudaError_t launch_select_partials(const Shapes& s, const float* partial, const ScoreLeft& left, float* scores_out, const RowStreams* rows,
