@@ -552,7 +552,7 @@ constexpr size_t kMaxDynamic = 220 * 1024;
 // Blocks per sequence.  FEW_CLUSTER_RULE
 int cluster_for(const Shapes& s, int slice) {
   int blocks = FASTAV_FEW_CLUSTER;
-  while (blocks > 1 && ((long long)s.batch * blocks > kNumSMs || s.max_seqlen <= blocks / 2 * slice)) blocks /= 2;
+  while (blocks > 1 && (s.batch > kAtOnce[blocks] || s.max_seqlen <= blocks / 2 * slice)) blocks /= 2;
   return blocks;
 }
 int cluster_keys(const Shapes& s) {

@@ -48,7 +48,7 @@ struct alignas(16) Control {
 template <int DIM>
 struct Layout {
   static constexpr int kOperandBytes = (DIM / 64) * kSubTileBytes;
-  static constexpr size_t kBytes = (size_t)(1 + kBlockTiles) * kOperandBytes + sizeof(Control) + 1024;
+  static constexpr size_t bytes(int tiles) { return (size_t)(1 + tiles) * kOperandBytes + sizeof(Control) + 1024; }
 };
 
 __device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueThreads) : "memory"); }
@@ -77,20 +77,17 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
   using L = Layout<DIM>;
   constexpr int kSubTiles = DIM / 64;
   extern __shared__ unsigned char smem_raw[];
-  chain_enter(s, q_idx, cu_qlens, cu_seqlens);
   cluster_arrive();  // "this block runs": waited for before the first remote access
   const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t q_smem = base, k_smem = base + L::kOperandBytes;
-  Control& ctl = *reinterpret_cast<Control*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + (1 + kBlockTiles) * L::kOperandBytes);
+  Control& ctl = *reinterpret_cast<Control*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + (1 + tiles_per_block) * L::kOperandBytes);
   volatile int* abort = &ctl.abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int c = (int)cluster_rank(), id = (int)blockIdx.x / blocks;
   const int rt = id % row_tiles, g = id / row_tiles % s.hkv, b = id / row_tiles / s.hkv;
 
-  if (warp == 0) {  // the sequence's bounds, asked for by one warp
-    const int32_t* word = lane < 2 ? cu_seqlens + b + lane : cu_qlens + b + (lane & 1);
-    if (lane < 4) ctl.index[lane] = chain_load(word);
-  } else if (warp == 1) {
+  // Everything that touches no global memory comes before the wait of a call's first kernel.
+  if (warp == 1) {
     if (lane == 0) {
       ptx::mbar_init(ptx::smem_u32(&ctl.q_full), 1);
       for (int i = 0; i < kBlockTiles; ++i) {
@@ -105,11 +102,16 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
     __syncwarp();
     ptx::tmem_alloc(ptx::smem_u32(&ctl.tmem_base), kTmemCols);
     ptx::tmem_relinquish();
-  } else {
+  } else if (warp >= 2) {
     // The query tile starts as zeros: rows no copy ever fills are then harmless operands.
     for (int i = threadIdx.x - 64; i < L::kOperandBytes / 16; i += kEpilogueThreads)
       asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(q_smem + i * 16), "r"(0) : "memory");
     ptx::fence_proxy_async_smem();  // ordered before the TMA writes that follow the barrier
+  }
+  chain_enter(s, q_idx, cu_qlens, cu_seqlens);
+  if (warp == 0) {  // the sequence's bounds, asked for by one warp
+    const int32_t* word = lane < 2 ? cu_seqlens + b + lane : cu_qlens + b + (lane & 1);
+    if (lane < 4) ctl.index[lane] = chain_load(word);
   }
   ptx::tc_fence_before_sync();
   __syncthreads();
@@ -125,30 +127,29 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
   const bool causal = (s.flags & FASTAV_CAUSAL) != 0;
 
   if (warp == 0) {
-    if (lane == 0) {
-      pdl_wait();  // q and k may be what earlier work wrote
-      if (mine > 0) {
-        // Boxes of 8 scored rows x G heads x 64 columns land as 8 G consecutive 128-byte rows: the flat (scored row, head)
-        // order of the tile, a whole number of 1024-byte swizzle groups.
-        const int boxes = (rows_here / s.group + 7) / 8;
-        const uint32_t box_bytes = 8u * s.group * 128u, bar = ptx::smem_u32(&ctl.q_full);
-        ptx::mbar_arrive_expect_tx(bar, boxes * box_bytes * kSubTiles);
-        for (int t = 0; t < mine; ++t) ptx::mbar_arrive_expect_tx(ptx::smem_u32(&ctl.k_full[t]), L::kOperandBytes);
+    pdl_wait();  // q and k may be what earlier work wrote
+    if (mine > 0) {
+      // Boxes of 8 scored rows x G heads x 64 columns land as 8 G consecutive 128-byte rows: the flat (scored row, head)
+      // order of the tile, a whole number of 1024-byte swizzle groups.
+      const int boxes = (rows_here / s.group + 7) / 8;
+      const uint32_t box_bytes = 8u * s.group * 128u, bar = ptx::smem_u32(&ctl.q_full);
+      ptx::mbar_expect_tx_warp(bar, boxes * box_bytes * kSubTiles);
+      for (int i = 0; i < boxes; ++i)
+#pragma unroll
         for (int sub = 0; sub < kSubTiles; ++sub)
-          ptx::tma_load_3d(k_smem + sub * kSubTileBytes, &k_map, sub * 64, g, seq.first + t0 * kTile, ptx::smem_u32(&ctl.k_full[0]));
+          ptx::tma_load_3d_warp(q_smem + sub * kSubTileBytes + i * box_bytes, &q_map, sub * 64, g * s.group,
+                                rows.first + rt * (rows_per_tile / s.group) + 8 * i, bar);
+      for (int t = 0; t < mine; ++t) {
+        const uint32_t k_bar = ptx::smem_u32(&ctl.k_full[t]);
+        ptx::mbar_expect_tx_warp(k_bar, L::kOperandBytes);
+#pragma unroll
         for (int sub = 0; sub < kSubTiles; ++sub)
-          for (int i = 0; i < boxes; ++i)
-            ptx::tma_load_3d(q_smem + sub * kSubTileBytes + i * box_bytes, &q_map, sub * 64, g * s.group,
-                             rows.first + rt * (rows_per_tile / s.group) + 8 * i, bar);
-        for (int t = 1; t < mine; ++t)
-          for (int sub = 0; sub < kSubTiles; ++sub)
-            ptx::tma_load_3d(k_smem + t * L::kOperandBytes + sub * kSubTileBytes, &k_map, sub * 64, g, seq.first + (t0 + t) * kTile,
-                             ptx::smem_u32(&ctl.k_full[t]));
-        // The copies write into this block's shared memory: they have to be waited for before it may exit.
-        int never = 0;
-        ptx::mbar_wait_bounded(bar, 0, &never);
-        for (int t = 0; t < mine; ++t) ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.k_full[t]), 0, &never);
+          ptx::tma_load_3d_warp(k_smem + t * L::kOperandBytes + sub * kSubTileBytes, &k_map, sub * 64, g, seq.first + (t0 + t) * kTile, k_bar);
       }
+      // The copies write into this block's shared memory: they have to be waited for before it may exit.
+      int never = 0;
+      ptx::mbar_wait_bounded(bar, 0, &never);
+      for (int t = 0; t < mine; ++t) ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.k_full[t]), 0, &never);
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -314,9 +315,9 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
 template <int DIM>
 cudaError_t launch(const Shapes& s, const CUtensorMap& k_map, const CUtensorMap& q_map, const int32_t* q_idx, const int32_t* cu_qlens,
                    const int32_t* cu_seqlens, const float* lse_in, const OncePlan& plan, float* partial, int32_t* device_status, cudaStream_t stream) {
-  const size_t smem = Layout<DIM>::kBytes;
+  const size_t smem = Layout<DIM>::bytes(plan.tiles_per_block);
   cudaError_t e = once_per_device([&] {
-    cudaError_t f = cudaFuncSetAttribute(score_once_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t f = cudaFuncSetAttribute(score_once_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Layout<DIM>::bytes(kBlockTiles));
     if (f == cudaSuccess) f = cudaFuncSetAttribute(score_once_kernel<DIM>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return f;
   });
@@ -337,9 +338,6 @@ int once_row_tiles(int max_qlen, int group) {
   return per == 0 ? 0 : (max_qlen * group + per - 1) / per;
 }
 
-#ifndef FASTAV_ONCE_WAVES
-#define FASTAV_ONCE_WAVES 1
-#endif
 bool once_plan(const Shapes& s, OncePlan* plan) {
   plan->rows_per_tile = once_rows_per_tile(s.group);
   if (plan->rows_per_tile == 0 || s.max_seqlen < 1 || s.max_qlen < 1) return false;
@@ -347,13 +345,15 @@ bool once_plan(const Shapes& s, OncePlan* plan) {
   const int tiles = (s.max_seqlen + kTile - 1) / kTile;
   if (tiles > kMaxTiles) return false;
   const long long clusters = (long long)s.batch * s.hkv * plan->row_tiles;
-  // One key tile per block as long as all blocks run at once, up to four otherwise (ONCE_RULE).
-  int blocks = 1;
-  while (blocks < tiles && blocks < kMaxCluster) blocks *= 2;
-  while (blocks > 1 && clusters * blocks > (long long)FASTAV_ONCE_WAVES * kNumSMs && tiles <= blocks / 2 * kBlockTiles) blocks /= 2;
-  plan->blocks = blocks;
-  plan->tiles_per_block = (tiles + blocks - 1) / blocks;
-  return plan->tiles_per_block <= kBlockTiles && clusters * blocks <= (long long)FASTAV_ONCE_WAVES * kNumSMs;
+  // The fewest key tiles per block with which all clusters run at once (ONCE_RULE).
+  for (int per = 1; per <= kBlockTiles; ++per) {
+    const int blocks = (tiles + per - 1) / per;
+    if (blocks > kMaxCluster || clusters > kAtOnce[blocks]) continue;
+    plan->blocks = blocks;
+    plan->tiles_per_block = per;
+    return true;
+  }
+  return false;
 }
 
 cudaError_t launch_score_once(const Shapes& s, const void* k_map, const void* q_map, const int32_t* q_idx, const int32_t* cu_qlens,
