@@ -235,6 +235,19 @@ __device__ __forceinline__ void chain_enter(const Head& head, P&... arrays) {
   (chain_acquire_one(arrays), ...);
   pdl_trigger();
 }
+// The same in two halves, for kernels with set-up work that touches no global memory: a call's first kernel does that work
+// ahead of its wait, the others let their successor start before anything else (a set-up of 0.2 us ahead of the trigger
+// shows as 0.2 us per launch in a chain of small calls).
+template <typename Head>
+__device__ __forceinline__ void chain_begin_setup(const Head& head) {
+  if (!head.head_wait) pdl_trigger();
+}
+template <typename Head, typename... P>
+__device__ __forceinline__ void chain_end_setup(const Head& head, P&... arrays) {
+  if (head.head_wait) pdl_wait();
+  (chain_acquire_one(arrays), ...);
+  if (head.head_wait) pdl_trigger();
+}
 inline thread_local bool g_chain_head = true;
 inline void chain_begin(uint32_t flags) { g_chain_head = (flags & FASTAV_CHAIN_CALLS) == 0; }
 

@@ -128,25 +128,26 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
                                                                 int32_t* __restrict__ cu_keep, int32_t* device_status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   FewShared& sh = *reinterpret_cast<FewShared*>(smem_raw);
-  chain_enter(s, cu_seqlens, keep_counts, protect, q_idx, cu_qlens);
+  chain_begin_setup(s);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int blocks = (int)gridDim.x / s.batch;  // blocks per cluster
   const int b = blockIdx.x / blocks, c = (int)cluster_rank();
   cluster_arrive();  // "this block runs": waited for before the first remote access
 
+  // Whatever touches no global memory comes before the wait of a call's first kernel.
+  const bool selecting = a.do_select != 0;
+  if (selecting)
+    for (int i = tid; i < kBins / 4; i += kThreads) reinterpret_cast<uint4*>(sh.hist)[i] = make_uint4(0, 0, 0, 0);
+  if (tid < kMaxTokens / 32) sh.prot_bits[tid] = 0u;
+  if (tid == 32) { sh.base = 0; sh.list_n = 0; }
+  chain_end_setup(s, cu_seqlens, keep_counts, protect, q_idx, cu_qlens);
   // ---- the caller's index arrays: one warp asks for all of them at once (sixteen warps of sixteen blocks asking for the
   //      same words queue at one L2 slice: 2,500 cycles instead of 900) ----------------------------------------------------
-  const bool selecting = a.do_select != 0;
   if (warp == 0) {
     const int32_t* word = lane < 2 ? cu_seqlens + b + lane : lane < 4 ? cu_qlens + b + lane - 2 : keep_counts + b;
     const bool there = lane < 2 || (lane < 4 ? cu_qlens != nullptr : lane == 4 && selecting);
     const int v = there ? chain_load(word) : 0;
     if (lane < 5) sh.index[lane] = v;
-  } else {
-    if (selecting)
-      for (int i = tid - 32; i < kBins / 4; i += kThreads - 32) reinterpret_cast<uint4*>(sh.hist)[i] = make_uint4(0, 0, 0, 0);
-    for (int i = tid - 32; i < kMaxTokens / 32; i += kThreads - 32) sh.prot_bits[i] = 0u;
-    if (tid == 32) { sh.base = 0; sh.list_n = 0; }
   }
   __syncthreads();
   const Span seq = checked_words(sh.index[0], sh.index[1], s.total_tokens, s.max_seqlen);
@@ -199,156 +200,159 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
     return ((sh.prot_bits[j >> 5] >> (j & 31)) & 1u) ? kProtectedKey : x;
   };
   if constexpr (FRONT == kKeys) {
-  pdl_acquire(a.q);
-  pdl_acquire(a.k);
-  // ---- logits ----------------------------------------------------------------------------------------------
-  const FewLayout lay = few_layout(a.slice_cap, s.hq * a.rq, DIM);
-  unsigned char* const more = smem_raw + sizeof(FewShared);
-  constexpr int kQStride = DIM * 2 + 64;
-  unsigned char* const q_sh = more + lay.q;
-  float* const lse = reinterpret_cast<float*>(more + lay.lse);
-  float2* const stats = reinterpret_cast<float2*>(more + lay.stats);
-  float* const z = reinterpret_cast<float*>(more + lay.z);
-  const int z_stride = z_stride_of(a.slice_cap);
-  // Units of 16 tokens x one KV head, KV heads running fastest; the first one's keys are on their way before the queries
-  // are staged.
-  const int units = flat > 0 ? (m + 15) / 16 * s.hkv : 0;
-  const uint16_t* const k_base = a.k + (long long)(tok0 + t0) * s.k_st;
-  KeyFragment<DIM> frag;
-  int g = warp % s.hkv, tok = warp / s.hkv * 16;
-  if (warp < units) frag.load(k_base + (long long)tok * s.k_st + (long long)g * s.k_sh, s.k_st, m - tok, lane);
-  for (int i = tid; i < terms * (DIM / 8); i += kThreads) {
-    const int row = i / (DIM / 8), piece = i % (DIM / 8);  // row: (KV head, f)
-    const int gg = row / flat, f = row - gg * flat, r = f / s.group;
-    const uint4 v = chain_load(reinterpret_cast<const uint4*>(a.q + (long long)(qrows.first + r) * s.q_st +
-                                                              (long long)(gg * s.group + f - r * s.group) * s.q_sh + piece * 8));
-    *reinterpret_cast<uint4*>(q_sh + row * kQStride + piece * 16) = v;
-  }
-  if (tid < flat) {
-    sh.row_of[tid] = tid / s.group;
-    sh.term_of[tid] = (tid % s.group) * rows + tid / s.group;
-  }
-  if (warp == 0) {
-    // what each scored row may see, relative to this block's first token
-    if (lane < kNarrowMaxRows) sh.limit[lane] = causal && lane < rows ? chain_load(q_idx + qrows.first + lane) - t0 : 0x7FFFFFFF;
-    protect_rows(0, 32);
-  }
-  __syncthreads();
-  for (int u = warp; u < units; u += kWarps) {
-    const KeyFragment<DIM> cur = frag;
-    const int g_here = g, tok_here = tok;
-    if (u + kWarps < units) {
-      g = (u + kWarps) % s.hkv;
-      tok = (u + kWarps) / s.hkv * 16;
-      frag.load(k_base + (long long)tok * s.k_st + (long long)g * s.k_sh, s.k_st, m - tok, lane);
+    pdl_acquire(a.q);
+    pdl_acquire(a.k);
+    // ---- logits ----------------------------------------------------------------------------------------------
+    const FewLayout lay = few_layout(a.slice_cap, s.hq * a.rq, DIM);
+    unsigned char* const more = smem_raw + sizeof(FewShared);
+    constexpr int kQStride = DIM * 2 + 64;
+    unsigned char* const q_sh = more + lay.q;
+    float* const lse = reinterpret_cast<float*>(more + lay.lse);
+    float2* const stats = reinterpret_cast<float2*>(more + lay.stats);
+    float* const z = reinterpret_cast<float*>(more + lay.z);
+    const int z_stride = z_stride_of(a.slice_cap);
+    // Units of 16 tokens x one KV head, KV heads running fastest; the first one's keys are on their way before the queries
+    // are staged.
+    const int units = flat > 0 ? (m + 15) / 16 * s.hkv : 0;
+    const uint16_t* const k_base = a.k + (long long)(tok0 + t0) * s.k_st;
+    // Two fragments take turns: while one is multiplied the other is on its way.
+    KeyFragment<DIM> even, odd;
+    auto fetch = [&](KeyFragment<DIM>& frag, int u) {
+      const int g = u % s.hkv, tok = u / s.hkv * 16;
+      if (u < units) frag.load(k_base + (long long)tok * s.k_st + (long long)g * s.k_sh, s.k_st, m - tok, lane);
+    };
+    fetch(even, warp);
+    fetch(odd, warp + kWarps);
+    for (int i = tid; i < terms * (DIM / 8); i += kThreads) {
+      const int row = i / (DIM / 8), piece = i % (DIM / 8);  // row: (KV head, f)
+      const int gg = row / flat, f = row - gg * flat, r = f / s.group;
+      const uint4 v = chain_load(reinterpret_cast<const uint4*>(a.q + (long long)(qrows.first + r) * s.q_st +
+                                                                (long long)(gg * s.group + f - r * s.group) * s.q_sh + piece * 8));
+      *reinterpret_cast<uint4*>(q_sh + row * kQStride + piece * 16) = v;
     }
+    if (tid < flat) {
+      sh.row_of[tid] = tid / s.group;
+      sh.term_of[tid] = (tid % s.group) * rows + tid / s.group;
+    }
+    // what each scored row may see, relative to this block's first token (asked for beside the queries: both are one L2 latency)
+    if (tid < kNarrowMaxRows) sh.limit[tid] = causal && tid < rows ? chain_load(q_idx + qrows.first + tid) - t0 : 0x7FFFFFFF;
+    if (warp == 1) protect_rows(32, 32);
+    __syncthreads();
+    auto multiply = [&](const KeyFragment<DIM>& frag, int u) {
+      const int g = u % s.hkv, j = u / s.hkv * 16 + (lane >> 2);
 #pragma unroll 1
-    for (int f0 = 0; f0 < flat; f0 += 8) {  // eight query rows at a time
-      float acc[4] = {0.f, 0.f, 0.f, 0.f};
-      const unsigned char* const qp = q_sh + (g_here * flat + min(f0 + (lane >> 2), flat - 1)) * kQStride + (lane & 3) * 16;
+      for (int f0 = 0; f0 < flat; f0 += 8) {  // eight query rows at a time
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        const unsigned char* const qp = q_sh + (g * flat + min(f0 + (lane >> 2), flat - 1)) * kQStride + (lane & 3) * 16;
 #pragma unroll
-      for (int i = 0; i < DIM / 32; ++i) {
-        const uint4 qv = *reinterpret_cast<const uint4*>(qp + i * 64);
-        mma_16x8x16(acc, cur.lo[i].x, cur.hi[i].x, cur.lo[i].y, cur.hi[i].y, qv.x, qv.y);
-        mma_16x8x16(acc, cur.lo[i].z, cur.hi[i].z, cur.lo[i].w, cur.hi[i].w, qv.z, qv.w);
+        for (int i = 0; i < DIM / 32; ++i) {
+          const uint4 qv = *reinterpret_cast<const uint4*>(qp + i * 64);
+          mma_16x8x16(acc, frag.lo[i].x, frag.hi[i].x, frag.lo[i].y, frag.hi[i].y, qv.x, qv.y);
+          mma_16x8x16(acc, frag.lo[i].z, frag.hi[i].z, frag.lo[i].w, frag.hi[i].w, qv.z, qv.w);
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int f = f0 + (lane & 3) * 2 + e;
+          if (f < flat) {
+            const int lim = sh.limit[sh.row_of[f]];
+            float* const at = z + (g * flat + sh.term_of[f]) * z_stride + j;
+            at[0] = j <= lim ? acc[e] * s.scale_log2 : -INFINITY;
+            at[8] = j + 8 <= lim ? acc[e + 2] * s.scale_log2 : -INFINITY;
+          }
+        }
+        __syncwarp();
       }
-      const int j = tok_here + (lane >> 2);
+    };
+    for (int u = warp; u < units; u += 2 * kWarps) {
+      multiply(even, u);
+      fetch(even, u + 2 * kWarps);
+      if (u + kWarps < units) multiply(odd, u + kWarps);
+      fetch(odd, u + 3 * kWarps);
+    }
+    selection_inputs();  // arrives while other warps still multiply
+    cluster_wait();
+    __syncthreads();
+
+    // ---- log-sum-exp per term ----------------------------------------------------------------------------------
+    if (a.lse) {
+      for (int i = tid; i < terms; i += kThreads) {
+        const float v = chain_load(a.lse + (long long)(qrows.first + i % rows) * s.hq + i / rows);
+        lse[i] = (v == v && fabsf(v) != INFINITY) ? v * kLog2e : INFINITY;  // a row that sees no key adds 0
+      }
+    } else {
+      const int first_seg = t0 / seg, segs = (m + seg - 1) / seg, l8 = tid & (kStatLanes - 1);
+#pragma unroll 1
+      for (int i0 = 0; i0 < terms * segs; i0 += kThreads / kStatLanes) {  // (segment, term): running (max, sum 2^(z - max))
+        const int i = i0 + tid / kStatLanes;
+        const bool active = i < terms * segs;
+        const int sg = segs == 1 ? 0 : i / terms, term = i - sg * terms, end = active ? min(m, (sg + 1) * seg) : 0;
+        const float* const row = z + (active ? term : 0) * z_stride;
+        float zm = -INFINITY, sum = 0.f;
+#pragma unroll 1
+        for (int j0 = sg * seg + l8; j0 < end; j0 += kStatLanes * 4) {
+          float v[4];
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int f = f0 + (lane & 3) * 2 + e;
-        if (f < flat) {
-          const int lim = sh.limit[sh.row_of[f]];
-          float* const at = z + (g_here * flat + sh.term_of[f]) * z_stride + j;
-          at[0] = j <= lim ? acc[e] * s.scale_log2 : -INFINITY;
-          at[8] = j + 8 <= lim ? acc[e + 2] * s.scale_log2 : -INFINITY;
+          for (int u = 0; u < 4; ++u) v[u] = j0 + kStatLanes * u < end ? row[j0 + kStatLanes * u] : -INFINITY;
+          const float zn = fmaxf(zm, fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])));
+          const float ref = zn == -INFINITY ? 0.f : zn;
+          sum *= ptx::ex2_approx(zm - ref);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) sum += ptx::ex2_approx(v[u] - ref);
+          zm = zn;
+        }
+        __syncwarp();
+        float bm = zm;
+#pragma unroll
+        for (int d = kStatLanes / 2; d; d >>= 1) bm = fmaxf(bm, __shfl_xor_sync(0xFFFFFFFFu, bm, d));
+        sum = bm == -INFINITY ? 0.f : sum * ptx::ex2_approx(zm - bm);
+#pragma unroll
+        for (int d = kStatLanes / 2; d; d >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, d);
+        if (active) {
+          float2* const at = &stats[(first_seg + sg) * terms + term];
+          for (int q = l8; q < blocks; q += kStatLanes) remote_store2(remote(at, q), __float_as_uint(bm), __float_as_uint(sum));
+        }
+      }
+      cluster_sync();
+      const int all_segs = (n + seg - 1) / seg, sg = tid & (kSegments - 1);
+#pragma unroll 1
+      for (int i0 = 0; i0 < terms; i0 += kThreads / kSegments) {  // a lane per segment
+        const int i = i0 + tid / kSegments;
+        float2 p = make_float2(-INFINITY, 0.f);
+        if (i < terms && sg < all_segs) p = stats[sg * terms + i];
+        float bm = p.x;
+#pragma unroll
+        for (int d = kSegments / 2; d; d >>= 1) bm = fmaxf(bm, __shfl_xor_sync(0xFFFFFFFFu, bm, d));
+        float total = p.x > -INFINITY ? p.y * ptx::ex2_approx(p.x - bm) : 0.f;
+#pragma unroll
+        for (int d = kSegments / 2; d; d >>= 1) total += __shfl_xor_sync(0xFFFFFFFFu, total, d);
+        if (i < terms && sg == 0) lse[i] = total > 0.f ? bm + __log2f(total) : INFINITY;
+      }
+    }
+    __syncthreads();
+
+    // ---- scores: eight lanes per token, each every eighth term in ascending order, added in a fixed tree ---------
+    const float inv = all_rows > 0 ? 1.0f / ((float)s.hq * (float)all_rows) : 0.f;
+    const int part = tid & (kTokenLanes - 1);
+#pragma unroll 1
+    for (int j0 = 0; j0 < m; j0 += kThreads / kTokenLanes) {
+      const int j = j0 + tid / kTokenLanes;
+      float total = 0.f;
+      if (j < m) {
+#pragma unroll 4
+        for (int i = part; i < terms; i += kTokenLanes) total += ptx::ex2_approx(z[i * z_stride + j] - lse[i]);
+      }
+      __syncwarp();
+#pragma unroll
+      for (int d = kTokenLanes / 2; d; d >>= 1) total += __shfl_xor_sync(0xFFFFFFFFu, total, d);
+      const float score = total * inv;
+      if (j < m) {
+        if (part == 0) a.scores_out[tok0 + t0 + j] = score;
+        if (selecting) {
+          const unsigned x = key_of(j, score);
+          for (int q = part; q < blocks; q += kTokenLanes) remote_store(remote(&sh.keys[t0 + j], q), x);  // to every block of the cluster
         }
       }
     }
-  }
-  selection_inputs();  // arrives while other warps still multiply
-  cluster_wait();
-  __syncthreads();
-
-  // ---- log-sum-exp per term ----------------------------------------------------------------------------------
-  if (a.lse) {
-    for (int i = tid; i < terms; i += kThreads) {
-      const float v = chain_load(a.lse + (long long)(qrows.first + i % rows) * s.hq + i / rows);
-      lse[i] = (v == v && fabsf(v) != INFINITY) ? v * kLog2e : INFINITY;  // a row that sees no key adds 0
-    }
-  } else {
-    const int first_seg = t0 / seg, segs = (m + seg - 1) / seg, l8 = tid & (kStatLanes - 1);
-#pragma unroll 1
-    for (int i0 = 0; i0 < terms * segs; i0 += kThreads / kStatLanes) {  // (segment, term): running (max, sum 2^(z - max))
-      const int i = i0 + tid / kStatLanes;
-      const bool active = i < terms * segs;
-      const int sg = segs == 1 ? 0 : i / terms, term = i - sg * terms, end = active ? min(m, (sg + 1) * seg) : 0;
-      const float* const row = z + (active ? term : 0) * z_stride;
-      float zm = -INFINITY, sum = 0.f;
-#pragma unroll 1
-      for (int j0 = sg * seg + l8; j0 < end; j0 += kStatLanes * 4) {
-        float v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = j0 + kStatLanes * u < end ? row[j0 + kStatLanes * u] : -INFINITY;
-        const float zn = fmaxf(zm, fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])));
-        const float ref = zn == -INFINITY ? 0.f : zn;
-        sum *= ptx::ex2_approx(zm - ref);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) sum += ptx::ex2_approx(v[u] - ref);
-        zm = zn;
-      }
-      __syncwarp();
-      float bm = zm;
-#pragma unroll
-      for (int d = kStatLanes / 2; d; d >>= 1) bm = fmaxf(bm, __shfl_xor_sync(0xFFFFFFFFu, bm, d));
-      sum = bm == -INFINITY ? 0.f : sum * ptx::ex2_approx(zm - bm);
-#pragma unroll
-      for (int d = kStatLanes / 2; d; d >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, d);
-      if (active) {
-        float2* const at = &stats[(first_seg + sg) * terms + term];
-        for (int q = l8; q < blocks; q += kStatLanes) remote_store2(remote(at, q), __float_as_uint(bm), __float_as_uint(sum));
-      }
-    }
-    cluster_sync();
-    const int all_segs = (n + seg - 1) / seg, sg = tid & (kSegments - 1);
-#pragma unroll 1
-    for (int i0 = 0; i0 < terms; i0 += kThreads / kSegments) {  // a lane per segment
-      const int i = i0 + tid / kSegments;
-      float2 p = make_float2(-INFINITY, 0.f);
-      if (i < terms && sg < all_segs) p = stats[sg * terms + i];
-      float bm = p.x;
-#pragma unroll
-      for (int d = kSegments / 2; d; d >>= 1) bm = fmaxf(bm, __shfl_xor_sync(0xFFFFFFFFu, bm, d));
-      float total = p.x > -INFINITY ? p.y * ptx::ex2_approx(p.x - bm) : 0.f;
-#pragma unroll
-      for (int d = kSegments / 2; d; d >>= 1) total += __shfl_xor_sync(0xFFFFFFFFu, total, d);
-      if (i < terms && sg == 0) lse[i] = total > 0.f ? bm + __log2f(total) : INFINITY;
-    }
-  }
-  __syncthreads();
-
-  // ---- scores: eight lanes per token, each every eighth term in ascending order, added in a fixed tree ---------
-  const float inv = all_rows > 0 ? 1.0f / ((float)s.hq * (float)all_rows) : 0.f;
-  const int part = tid & (kTokenLanes - 1);
-#pragma unroll 1
-  for (int j0 = 0; j0 < m; j0 += kThreads / kTokenLanes) {
-    const int j = j0 + tid / kTokenLanes;
-    float total = 0.f;
-    if (j < m) {
-#pragma unroll 4
-      for (int i = part; i < terms; i += kTokenLanes) total += ptx::ex2_approx(z[i * z_stride + j] - lse[i]);
-    }
-    __syncwarp();
-#pragma unroll
-    for (int d = kTokenLanes / 2; d; d >>= 1) total += __shfl_xor_sync(0xFFFFFFFFu, total, d);
-    const float score = total * inv;
-    if (j < m) {
-      if (part == 0) a.scores_out[tok0 + t0 + j] = score;
-      if (selecting) {
-        const unsigned x = key_of(j, score);
-        for (int q = part; q < blocks; q += kTokenLanes) remote_store(remote(&sh.keys[t0 + j], q), x);  // to every block of the cluster
-      }
-    }
-  }
   } else {
     // ---- scores from partial sums, or as they are --------------------------------------------------------------------
     const float* in = a.in;

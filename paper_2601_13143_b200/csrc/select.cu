@@ -375,60 +375,71 @@ cudaError_t launch_select(const Shapes& s, const Workspace& w, const float* scor
 // ---- keep set given as a mask (the paper's positional global rule) ---------------------------------
 namespace {
 
-// counts[b] = number of kept tokens of sequence b.
-__global__ void __launch_bounds__(256) mask_count_kernel(Shapes s, const uint8_t* __restrict__ keep_mask,
-                                                         const int32_t* __restrict__ cu_seqlens, int32_t* __restrict__ counts) {
-  __shared__ int warp_sums[8];
+// Non-zero bytes of mask[0, count), per thread; 16 bytes at a time between the ends.
+__device__ __forceinline__ int count_nonzero(const uint8_t* mask, int count, int tid) {
+  const int head = min(count, (int)(-reinterpret_cast<uintptr_t>(mask) & 15u)), quads = (count - head) / 16;
+  int c = 0;
+  for (int j = tid; j < head; j += kThreads) c += mask[j] != 0;
+  const uint4* q = reinterpret_cast<const uint4*>(mask + head);
+  for (int j = tid; j < quads; j += kThreads) {
+    const uint4 v = q[j];
+    const unsigned w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) c += __popc((((w[i] & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | w[i]) & 0x80808080u);
+  }
+  for (int j = head + quads * 16 + tid; j < count; j += kThreads) c += mask[j] != 0;
+  return c;
+}
+
+// counts[b] = number of kept tokens of sequence b (large batches only; see mask_emit_kernel).
+__global__ void __launch_bounds__(kThreads) mask_count_kernel(Shapes s, const uint8_t* __restrict__ keep_mask,
+                                                              const int32_t* __restrict__ cu_seqlens, int32_t* __restrict__ counts) {
+  __shared__ int total;
   chain_enter(s, cu_seqlens);
+  if (threadIdx.x == 0) total = 0;
   pdl_wait();
   pdl_acquire(keep_mask);
   const int b = blockIdx.x;
   const Span seq = checked_span(cu_seqlens, b, s.total_tokens, s.total_tokens);
-  const int tok0 = seq.first, n = seq.count;
-  int c = 0;
-  for (int j = threadIdx.x; j < n; j += 256) c += keep_mask[tok0 + j] != 0;
-  c = __reduce_add_sync(0xFFFFFFFFu, c);
-  if ((threadIdx.x & 31) == 0) warp_sums[threadIdx.x >> 5] = c;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int total = 0;
-    for (int w = 0; w < 8; ++w) total += warp_sums[w];
-    counts[b] = total;
-  }
+  const int c = __reduce_add_sync(0xFFFFFFFFu, count_nonzero(keep_mask + seq.first, seq.count, threadIdx.x));
+  if ((threadIdx.x & 31) == 0 && c) atomicAdd(&total, c);
+  __syncthreads();
+  if (threadIdx.x == 0) counts[b] = total;
 }
 
-// Survivors of sequence b in ascending order, after those of the sequences before it.
+// Survivors of sequence b in ascending order, after those of the sequences before it: their number is read from `counts`, or,
+// without it, counted here from the mask itself (one kernel less).
 __global__ void __launch_bounds__(kThreads) mask_emit_kernel(Shapes s, const uint8_t* __restrict__ keep_mask,
                                                              const int32_t* __restrict__ cu_seqlens,
                                                              const int32_t* __restrict__ counts, int32_t* __restrict__ keep_idx,
                                                              int32_t* __restrict__ cu_keep, int32_t* device_status) {
   __shared__ unsigned warp_a[kWarps];
-  __shared__ int base_sh;
+  __shared__ int base_sh, mine_sh;
   chain_enter(s, cu_seqlens);
-  pdl_wait();
-  pdl_acquire(counts);
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const Span seq = checked_span(cu_seqlens, b, s.total_tokens, s.total_tokens);
   const int tok0 = seq.first, n = seq.count;
   if (tid == 0 && seq.bad && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
   if (tid == 0) base_sh = 0;
+  pdl_wait();
+  pdl_acquire(keep_mask);
+  pdl_acquire(counts);
   __syncthreads();
   int part = 0;
-  for (int i = tid; i < b; i += kThreads) part += chain_load(counts + i);
-  if (part) atomicAdd(&base_sh, part);
-  __syncthreads();
-  const int base = base_sh;
-  if (tid == 0) {
-    const int mine = chain_load(counts + b);
-    cu_keep[b + 1] = min(base + mine, s.total_keep);
-    if (b == 0) cu_keep[0] = 0;
-    if (base + mine > s.total_keep && device_status) atomicOr(device_status, FASTAV_DEV_K_CLAMPED);
+  if (counts) {
+    for (int i = tid; i < b; i += kThreads) part += chain_load(counts + i);
+  } else {
+    part = count_nonzero(keep_mask, tok0, tid);  // the sequences before this one lie before it in the packed batch
   }
+  part = __reduce_add_sync(0xFFFFFFFFu, part);
+  if (lane == 0 && part) atomicAdd(&base_sh, part);
   const bool global_idx = (s.flags & FASTAV_KEEP_IDX_GLOBAL) != 0;
   const int per = (n + kThreads - 1) / kThreads;
   const int j0 = min(n, tid * per), j1 = min(n, j0 + per);
   unsigned mine = 0;
   for (int j = j0; j < j1; ++j) mine += keep_mask[tok0 + j] != 0;
+  __syncwarp();
   unsigned incl = mine;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
@@ -439,11 +450,19 @@ __global__ void __launch_bounds__(kThreads) mask_emit_kernel(Shapes s, const uin
   __syncthreads();
   unsigned before = incl - mine;
   for (int w = 0; w < warp; ++w) before += warp_a[w];
+  const int base = base_sh;
+  if (tid == kThreads - 1) mine_sh = (int)(before + mine);
   for (int j = j0; j < j1; ++j)
     if (keep_mask[tok0 + j]) {
       const int out = base + (int)before++;
       if (out < s.total_keep) keep_idx[out] = global_idx ? tok0 + j : j;  // never past the caller's buffer
     }
+  __syncthreads();
+  if (tid == 0) {
+    cu_keep[b + 1] = min(base + mine_sh, s.total_keep);
+    if (b == 0) cu_keep[0] = 0;
+    if (base + mine_sh > s.total_keep && device_status) atomicOr(device_status, FASTAV_DEV_K_CLAMPED);
+  }
 }
 
 }  // namespace
@@ -464,11 +483,16 @@ extern "C" int32_t fastav_select_mask(const fastav_params* p, const uint8_t* kee
   s.flags = p->flags;
   int32_t* counts = static_cast<int32_t*>(workspace);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  cudaError_t e = launch_chained(mask_count_kernel, dim3(s.batch), dim3(256), 0, st, s, keep_mask, cu_seqlens, counts);
+  // Each block counts the whole batch before its sequence; beyond a quarter of a million tokens a kernel that counts every
+  // sequence once is the shorter way.
+  constexpr int kCountHere = 1 << 18;
+  const bool count_first = s.total_tokens > kCountHere;
+  cudaError_t e = cudaSuccess;
+  if (count_first) e = launch_chained(mask_count_kernel, dim3(s.batch), dim3(kThreads), 0, st, s, keep_mask, cu_seqlens, counts);
   if (e == cudaSuccess)
-    e = launch_chained(mask_emit_kernel, dim3(s.batch), dim3(kThreads), 0, st, s, keep_mask, cu_seqlens, (const int32_t*)counts,
-                       keep_idx_out, cu_keep_out, device_status);
-  count_launches(2);
+    e = launch_chained(mask_emit_kernel, dim3(s.batch), dim3(kThreads), 0, st, s, keep_mask, cu_seqlens,
+                       count_first ? (const int32_t*)counts : (const int32_t*)nullptr, keep_idx_out, cu_keep_out, device_status);
+  count_launches(count_first ? 2 : 1);
   return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? FASTAV_OK : FASTAV_ERR_CUDA;
 }
 
