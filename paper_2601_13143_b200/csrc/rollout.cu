@@ -20,9 +20,9 @@
 // and head, or per tile, leaves much of the chip idle in a second round, and the longest K loop of the triangular product
 // alone is 36 blocks of 64.  The statistics kernel is PERSISTENT: its (head, row block, key block) items are cut into equal
 // runs, one per SM, and a row block that several runs share leaves up to four partial log-sum-exps per row, which the map
-// kernel merges when it reads them.  The map kernel gives every SM whole tiles and cuts the tiles that are left over into
-// slices of 64 or 32 columns.  The product cuts the K loops that are longer than an SM's fair share into parts, whose
-// fp32 tiles meet in the workspace: the part that finishes last adds them up in order (no block waits for another).
+// kernel merges when it reads them.  The map kernel cuts every row block into STRIPS of at most 32 .. 160 columns, the width
+// that makes the fewest, fullest rounds.  The product cuts the K loops that are longer than an SM's fair share into parts,
+// whose fp32 tiles meet in the workspace: the part that finishes last adds them up in order (no block waits for another).
 // ROLLOUT_FIGURES
 //
 // Warp 0 issues the TMA loads, warp 1 the MMAs into accumulators in tensor memory, warps 2..17 are the epilogue
@@ -46,6 +46,8 @@ constexpr int kEpilogueThreads = 512;
 constexpr int kColGroups = 4;  // epilogue warps per TMEM quarter; each takes 32 of the 128 columns
 constexpr int kTmemCols = 512;
 constexpr int kBuffers = 4;    // accumulators of 128 columns
+constexpr int kMaxStripUnits = 5;  // the map's strips: up to 160 columns
+constexpr int kMapBuffers = 3;     // accumulators of 160 columns
 constexpr int kMaxStages = 4;
 constexpr int kSubTileBytes = kTile * 128;  // 128 rows of one 64-element (128-byte) column block
 constexpr int kMaxParts = 4;   // blocks that may share one row block's statistics
@@ -57,8 +59,10 @@ struct alignas(16) PipeControl {
   uint32_t tmem_base;
   int abort;
   int last;                               // product: this block finished the tile's last part
-  float2 part[2][kColGroups - 1][kTile];  // statistics: (max, sum) per row of column groups 1..3
-  float neg_lse[kHeadChunk][kTile];       // map: minus the log2-sum-exp2 of this tile's rows, some heads at a time
+  union {
+    float2 part[2][kColGroups - 1][kTile];  // statistics: (max, sum) per row of column groups 1..3
+    float neg_lse[kHeadChunk][kTile];       // map: minus the log2-sum-exp2 of this strip's rows, some heads at a time
+  };
 };
 
 __device__ __forceinline__ void split_bf16(float x, __nv_bfloat16& hi, __nv_bfloat16& lo) {
@@ -169,13 +173,12 @@ __device__ __forceinline__ int triangular_root(long long x) {
 }
 
 // ---- the attention map ---------------------------------------------------------------------------
-// Shared memory of both kernels: six tiles of 128 x DIM (192 KB at head_dim 128).
-template <int DIM, int SLOTS>
-struct AttnSmem {
+// Shared memory of the statistics kernel: six tiles of 128 x DIM (192 KB at head_dim 128).
+template <int DIM>
+struct StatSmem {
   static constexpr int kSubTiles = DIM / 64;
   static constexpr int kOperandBytes = kSubTiles * kSubTileBytes;
-  static constexpr int kSlots = SLOTS;          // for the operand that changes rarely
-  static constexpr int kStages = 6 - kSlots;    // the ring of the operand that changes every iteration
+  static constexpr int kStages = 4;  // the ring of K tiles; two more slots for Q tiles
   static constexpr size_t kBytes = (size_t)6 * kOperandBytes + sizeof(PipeControl) + 1024;
 };
 
@@ -218,7 +221,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 rollout_stats_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map, AttnArgs a, long long items,
                      int* counters, int n_counters, ChainHead chain_head) {
   // The ring holds K tiles; a Q tile's slot is freed by the last MMA that reads it.
-  using Cfg = AttnSmem<DIM, 2>;
+  using Cfg = StatSmem<DIM>;
   constexpr int kStages = Cfg::kStages, kOperandBytes = Cfg::kOperandBytes;
   extern __shared__ unsigned char smem_raw[];
   chain_enter(chain_head);
@@ -355,32 +358,58 @@ rollout_stats_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
   pipe_teardown(ctl, warp, a.device_status);
 }
 
-// Per 128 x 128 tile, or slice of its columns: the sum over the heads of the softmax weights, then Eq. 2, stored as hi / lo
-// planes (and, if asked, A itself in fp32).  Blocks 0 .. whole - 1 take whole tiles, the others slices of 128 / slices
-// columns of the tiles that are left; tiles no row may see (which the product never reads) only if the map is wanted.
+// One block per strip: 128 rows of the map by 32 .. 160 of its columns.  `units` of 32 columns is the widest strip; a row block
+// of U units that any row may see has ceil(U / units) strips of nearly equal width, long row blocks first.
+struct MapStrip {
+  int rb, unit, width;  // row block; first unit; units
+  __device__ MapStrip(int t, int blocks, bool causal, int units) {
+    for (rb = blocks - 1;; --rb) {
+      const int all = 4 * (causal ? rb + 1 : blocks), strips = (all + units - 1) / units;
+      if (t < strips || rb == 0) {
+        unit = all * t / strips;
+        width = all * (t + 1) / strips - unit;
+        return;
+      }
+      t -= strips;
+    }
+  }
+};
+
+// Shared memory of the map kernel: a ring of Q tiles, one per head, and two slots for a strip of K, which is loaded once per
+// KV head and shared by the G heads of its group (208 KB at head_dim 128).
+template <int DIM>
+struct MapSmem {
+  static constexpr int kSubTiles = DIM / 64, kStages = 4, kSlots = 2;
+  static constexpr int kOperandBytes = kSubTiles * kSubTileBytes;
+  static constexpr int kStripSubBytes = 32 * kMaxStripUnits * 128;  // one 64-element column block of the widest strip
+  static constexpr int kStripBytes = kSubTiles * kStripSubBytes;
+  static constexpr size_t kBytes = (size_t)kStages * kOperandBytes + kSlots * kStripBytes + sizeof(PipeControl) + 1024;
+  static_assert(kBytes <= 227 * 1024);
+};
+
+// Per strip: the sum over the heads of the softmax weights, then Eq. 2, stored as hi / lo planes (and, if asked, A itself in
+// fp32).  Tiles no row may see, which the product never reads, are written only if the map is wanted.
 template <int DIM>
 __global__ void __launch_bounds__(kThreads, 1)
-rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map, AttnArgs a,
-                   const float* __restrict__ lse_opt, float alpha, int whole, int slices, int blocks_of_work,
+rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_strip_map, AttnArgs a,
+                   const float* __restrict__ lse_opt, float alpha, int units, int strips,
                    __nv_bfloat16* __restrict__ a_hi, __nv_bfloat16* __restrict__ a_lo, float* __restrict__ map_out, ChainHead chain_head) {
-  // The ring holds Q tiles, one per head; a K tile is loaded once per KV head and shared by the G heads of its group -- three
-  // slots used in turn, so that a slot is overwritten no sooner than three iterations after its last use, which is the
-  // distance the ring's own barriers already guarantee.
-  using Cfg = AttnSmem<DIM, 3>;
-  constexpr int kStages = Cfg::kStages, kSlots = Cfg::kSlots, kOperandBytes = Cfg::kOperandBytes;
+  using Cfg = MapSmem<DIM>;
+  constexpr int kStages = Cfg::kStages, kOperandBytes = Cfg::kOperandBytes;
+  constexpr int kStripCols = 32 * kMaxStripUnits;
   extern __shared__ unsigned char smem_raw[];
   chain_enter(chain_head);
   const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t slots = base + kStages * kOperandBytes;
-  PipeControl& ctl = *reinterpret_cast<PipeControl*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + 6 * kOperandBytes);
+  PipeControl& ctl = *reinterpret_cast<PipeControl*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + kStages * kOperandBytes + Cfg::kSlots * Cfg::kStripBytes);
   volatile int* abort = &ctl.abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int blocks = a.n_pad / kTile, hq = a.hq, group = a.group;
   const bool causal = a.causal != 0;
 
-  if ((int)blockIdx.x >= blocks_of_work) {  // a tile no row may see, and the map is wanted: zeros (uniform for the block)
+  if ((int)blockIdx.x >= strips) {  // a tile no row may see, and the map is wanted: zeros (uniform for the block)
     pdl_wait();
-    const int t = blockIdx.x - blocks_of_work;        // (jb, rb) with jb > rb, in the order of the transposed triangle
+    const int t = blockIdx.x - strips;                // (jb, rb) with jb > rb, in the order of the transposed triangle
     const int jb = triangular_root(t) + 1, rb = t - (jb - 1) * jb / 2;
     for (int i = threadIdx.x; i < kTile * kTile; i += kThreads) {
       const int r = rb * kTile + i / kTile, c = jb * kTile + i % kTile;
@@ -388,14 +417,10 @@ rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     }
     return;
   }
-  const bool sliced = (int)blockIdx.x >= whole;
-  const int tile = sliced ? whole + ((int)blockIdx.x - whole) / slices : (int)blockIdx.x;
-  const int width = sliced ? kTile / slices : kTile;                       // columns of this block
-  const int col_first = sliced ? ((int)blockIdx.x - whole) % slices * width : 0;
-  const int rb = causal ? triangular_root(tile) : tile / blocks;
-  const int jb = tile - (causal ? rb * (rb + 1) / 2 : rb * blocks);
+  const MapStrip strip(blockIdx.x, blocks, causal, units);
+  const int rb = strip.rb;
 
-  pipe_setup(ctl, kStages, warp, &q_map, &k_map);
+  pipe_setup(ctl, kStages, warp, &q_map, &k_strip_map);
   const uint32_t tmem = ctl.tmem_base;
 
   if (warp == 0) {
@@ -407,36 +432,42 @@ rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.empty[stage]), ((it / kStages) & 1) ^ 1u, abort)) break;
         const uint32_t bar = ptx::smem_u32(&ctl.full[stage]);
         const bool load_k = it % group == 0;
-        const uint32_t ring = base + stage * kOperandBytes, slot = slots + ((it / group) % kSlots) * kOperandBytes;
-        ptx::mbar_arrive_expect_tx(bar, kOperandBytes + (load_k ? kOperandBytes : 0));
+        // the slot's last reader, two KV heads ago, if the wait above does not cover it
+        const int reader = it - group - 1;
+        if (load_k && reader >= 0 && reader > it - kStages &&
+            !ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.empty[reader % kStages]), (reader / kStages) & 1, abort))
+          break;
+        const uint32_t ring = base + stage * kOperandBytes, slot = slots + ((it / group) & 1) * Cfg::kStripBytes;
+        ptx::mbar_arrive_expect_tx(bar, kOperandBytes + (load_k ? Cfg::kSubTiles * strip.width * 4096 : 0));
 #pragma unroll
         for (int sub = 0; sub < Cfg::kSubTiles; ++sub) {
           ptx::tma_load_3d(ring + sub * kSubTileBytes, &q_map, sub * 64, it, rb * kTile, bar);
-          if (load_k) ptx::tma_load_3d(slot + sub * kSubTileBytes, &k_map, sub * 64, it / group, jb * kTile, bar);
+          if (load_k)
+            for (int u = 0; u < strip.width; ++u)
+              ptx::tma_load_3d(slot + sub * Cfg::kStripSubBytes + u * 4096, &k_strip_map, sub * 64, it / group, (strip.unit + u) * 32, bar);
         }
       }
       if (*abort) drain_loads(ctl, it, kStages);
     }
   } else if (warp == 1) {
     {
-      const uint32_t idesc = ptx::umma_idesc_bf16(kTile, width);
+      const uint32_t idesc = ptx::umma_idesc_bf16(kTile, 32 * strip.width);
       for (int it = 0; it < hq; ++it) {
-        const int stage = it % kStages, buf = it % kBuffers;
+        const int stage = it % kStages, buf = it % kMapBuffers;
         if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort)) break;
-        if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_empty[buf]), ((it / kBuffers) & 1) ^ 1u, abort)) break;
+        if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_empty[buf]), ((it / kMapBuffers) & 1) ^ 1u, abort)) break;
         ptx::tc_fence_after_sync();
-        const uint32_t q_tile = base + stage * kOperandBytes;
-        const uint32_t k_tile = slots + ((it / group) % kSlots) * kOperandBytes + col_first * 128;  // a multiple of 32 rows of 128 bytes
-        ptx::umma_bf16_steps<DIM / 16, kSubTileBytes, kSubTileBytes>(tmem + buf * kTile, ptx::umma_desc_sw128(q_tile, 0),
-                                                                     ptx::umma_desc_sw128(k_tile, 0), idesc, false);
+        const uint32_t q_tile = base + stage * kOperandBytes, k_tile = slots + ((it / group) & 1) * Cfg::kStripBytes;
+        ptx::umma_bf16_steps<DIM / 16, kSubTileBytes, Cfg::kStripSubBytes>(tmem + buf * kStripCols, ptx::umma_desc_sw128(q_tile, 0),
+                                                                           ptx::umma_desc_sw128(k_tile, 0), idesc, false);
         ptx::umma_commit(ptx::smem_u32(&ctl.empty[stage]));
         ptx::umma_commit(ptx::smem_u32(&ctl.tmem_full[buf]));
       }
     }
   } else {
-    const int quarter = warp & 3, cg = (warp - 2) >> 2;  // TMEM lanes 32 quarter .., columns width / 4 * cg ..
+    const int quarter = warp & 3, cg = (warp - 2) >> 2;  // TMEM lanes 32 quarter .., columns cols * cg ..
     const int row_in = quarter * 32 + lane, ethread = cg * kTile + row_in, row = rb * kTile + row_in;
-    const int cols = width / 4, pieces = cols / 8, col0 = jb * kTile + col_first + cg * cols;
+    const int pieces = strip.width, cols = 8 * pieces, col0 = strip.unit * 32 + cg * cols;
     const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16) + cg * cols;
     pdl_wait();
     float4* lse_parts = a.lse_parts;
@@ -446,13 +477,13 @@ rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     const int limit = last_visible - col0;  // columns 0..limit of this group are visible
     const bool whole_visible = __all_sync(0xFFFFFFFFu, limit >= cols - 1);
     const float2 sc = make_float2(a.scale_log2, a.scale_log2);
-    float2 acc2[16];
+    float2 acc2[4 * kMaxStripUnits];
 #pragma unroll
-    for (int c = 0; c < 16; ++c) acc2[c] = make_float2(0.f, 0.f);
+    for (int c = 0; c < 4 * kMaxStripUnits; ++c) acc2[c] = make_float2(0.f, 0.f);
     bool ok = true;
 #pragma unroll 1
     for (int it = 0; it < hq; ++it) {
-      const int buf = it % kBuffers;
+      const int buf = it % kMapBuffers;
       if (it % kHeadChunk == 0) {  // the rows' statistics of the next heads
         if (it > 0) epilogue_sync();
         for (int e = ethread; e < min(kHeadChunk, hq - it) * kTile; e += kEpilogueThreads) {
@@ -473,45 +504,46 @@ rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         epilogue_sync();
       }
       if (!ok) continue;
-      ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_full[buf]), (it / kBuffers) & 1, abort);
+      ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_full[buf]), (it / kMapBuffers) & 1, abort);
       if (!ok) continue;
       ptx::tc_fence_after_sync();
       const float neg_lse2 = ctl.neg_lse[it % kHeadChunk][row_in];
       const float2 nl = make_float2(neg_lse2, neg_lse2);
-      uint32_t v[32];
-      if (pieces == 4) {
-        ptx::tmem_ld32(lane_addr + buf * kTile, v);
-        ptx::tmem_ld_wait_for(v);
+      uint32_t v[32], v4[8];  // the fifth piece by itself
+      const uint32_t from = lane_addr + buf * kStripCols;
+      if (pieces >= 4) {
+        ptx::tmem_ld32(from, v);
+        if (pieces == 5) ptx::tmem_ld8(from + 32, v4);
       } else {
-        ptx::tmem_ld8(lane_addr + buf * kTile, v);
-        if (pieces == 2) ptx::tmem_ld8(lane_addr + buf * kTile + 8, v + 8);
-        ptx::tmem_ld_wait_for16(v);
+        ptx::tmem_ld8(from, v);
+        if (pieces >= 2) ptx::tmem_ld8(from + 8, v + 8);
+        if (pieces >= 3) ptx::tmem_ld8(from + 16, v + 16);
       }
+      ptx::tmem_ld_wait_for(v, v4);
       ptx::tc_fence_before_sync();
       ptx::mbar_arrive_warp(ptx::smem_u32(&ctl.tmem_empty[buf]), lane);  // the accumulator may be overwritten
-      auto add = [&](int c) {  // columns c, c + 1
-        float2 p = exp2_pair(__ffma2_rn(make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc, nl), c / 2);
-        if (!whole_visible) {
-          p.x = c <= limit ? p.x : 0.f;
-          p.y = c + 1 <= limit ? p.y : 0.f;
-        }
-        acc2[c / 2] = __fadd2_rn(acc2[c / 2], p);
+      auto weights = [&](const uint32_t* x, int c) {
+        return exp2_pair(__ffma2_rn(make_float2(__uint_as_float(x[0]), __uint_as_float(x[1])), sc, nl), c / 2);
       };
-      if (pieces == 4) {
-        if (whole_visible) {
+      if (pieces >= 4 && whole_visible) {
 #pragma unroll
-          for (int c = 0; c < 32; c += 2)
-            acc2[c / 2] = __fadd2_rn(acc2[c / 2], exp2_pair(__ffma2_rn(make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc, nl), c / 2));
-        } else {
+        for (int c = 0; c < 32; c += 2) acc2[c / 2] = __fadd2_rn(acc2[c / 2], weights(v + c, c));
+        if (pieces == 5) {
 #pragma unroll
-          for (int c = 0; c < 32; c += 2) add(c);
+          for (int c = 0; c < 8; c += 2) acc2[16 + c / 2] = __fadd2_rn(acc2[16 + c / 2], weights(v4 + c, c));
         }
       } else {
 #pragma unroll
-        for (int c = 0; c < 8; c += 2) add(c);
-        if (pieces == 2) {
+        for (int p = 0; p < kMaxStripUnits; ++p) {
+          if (p < pieces) {
 #pragma unroll
-          for (int c = 8; c < 16; c += 2) add(c);
+            for (int c = 8 * p; c < 8 * p + 8; c += 2) {
+              float2 w = weights(p < 4 ? v + c : v4 + c - 32, c);
+              w.x = c <= limit ? w.x : 0.f;
+              w.y = c + 1 <= limit ? w.y : 0.f;
+              acc2[c / 2] = __fadd2_rn(acc2[c / 2], w);
+            }
+          }
         }
       }
     }
@@ -519,7 +551,7 @@ rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       const float inv_heads = 1.0f / (float)hq;
       const long long at = (long long)row * a.n_pad + col0;
 #pragma unroll
-      for (int c0 = 0; c0 < 32; c0 += 8) {
+      for (int c0 = 0; c0 < 8 * kMaxStripUnits; c0 += 8) {
         if (c0 >= cols) break;
         alignas(16) __nv_bfloat16 hi[8], lo[8];
 #pragma unroll
@@ -777,14 +809,14 @@ bool plane_map(const void* ptr, int n_pad, CUtensorMap* map) {
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// [tokens, heads, d] bf16 with element strides (st, sh, 1) as (d, heads, tokens); a box is 128 tokens of one
+// [tokens, heads, d] bf16 with element strides (st, sh, 1) as (d, heads, tokens); a box is 128 tokens, or `rows`, of one
 // head's 64-element column block.  Tokens past the end read as zeros.
-bool qk_map(const void* ptr, int dim, int heads, int tokens, long long st, long long sh, CUtensorMap* map) {
+bool qk_map(const void* ptr, int dim, int heads, int tokens, long long st, long long sh, CUtensorMap* map, int rows = kTile) {
   auto encode = reinterpret_cast<EncodeTiledFn>(tensor_map_encode_entry());
   if (!encode) return false;
   const cuuint64_t dims[3] = {(cuuint64_t)dim, (cuuint64_t)heads, (cuuint64_t)tokens};
   const cuuint64_t strides[2] = {(cuuint64_t)sh * 2, (cuuint64_t)st * 2};
-  const cuuint32_t box[3] = {64, 1, kTile};
+  const cuuint32_t box[3] = {64, 1, (cuuint32_t)rows};
   const cuuint32_t elem[3] = {1, 1, 1};
   return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, elem,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -810,13 +842,27 @@ int stats_grid(int blocks, int hq, bool causal) {
   return (int)(g < 1 ? 1 : g > kNumSMs ? kNumSMs : g);
 }
 
-// Map: whole tiles as long as they fill rounds of all SMs, the rest in as many slices of at least 32 columns as still
-// make one round.
-void map_shares(int blocks, bool causal, int* whole, int* slices) {
-  const long long tiles = visible_tiles(blocks, causal);
-  const int rest = (int)(tiles % kNumSMs);
-  *slices = rest * 4 <= kNumSMs ? 4 : rest * 2 <= kNumSMs ? 2 : 1;
-  *whole = (int)(tiles - rest);
+// Map: strips of at most `units` units of 32 columns.  Per head, a strip of u units takes some 350 + 270 u cycles (tiles of 128
+// columns measured 1,430, strips of 160 1,700), and a block 6,000 before and after its heads; the width with the least
+// rounds x cycles wins.  2,230 tokens, 28 heads: 144 strips of up to 160 columns are one round of 40.3 us, where 148 whole
+// tiles and the other 23 in column slices of 32 were two of 51 us.
+long long map_strips(int blocks, bool causal, int units) {
+  long long strips = 0;
+  for (int rb = 0; rb < blocks; ++rb) strips += (4 * (causal ? rb + 1 : blocks) + units - 1) / units;
+  return strips;
+}
+int map_units(int blocks, bool causal, int hq) {
+  int best = 1;
+  long long least = LLONG_MAX;
+  for (int units = 1; units <= kMaxStripUnits; ++units) {
+    const long long rounds = (map_strips(blocks, causal, units) + kNumSMs - 1) / kNumSMs;
+    const long long cycles = rounds * ((long long)hq * (350 + 270 * units) + 6000);
+    if (cycles < least) {
+      least = cycles;
+      best = units;
+    }
+  }
+  return best;
 }
 
 // Product: no K loop longer than an SM's share of all K blocks (at least eight: a part costs an exchange of 64 KB).
@@ -861,10 +907,8 @@ RolloutWorkspace plan_rollout(int n, int hq) {
 }
 
 template <int DIM>
-cudaError_t run_attention(const fastav_params& p, const CUtensorMap& q_map, const CUtensorMap& k_map, const float* lse_opt, float alpha,
+cudaError_t run_attention(const fastav_params& p, const CUtensorMap& q_map, const CUtensorMap& k_map, const CUtensorMap& k_strip_map, const float* lse_opt, float alpha,
                           const RolloutWorkspace& w, unsigned char* ws, float* map_out, int32_t* device_status, cudaStream_t stream) {
-  constexpr size_t smem = AttnSmem<DIM, 2>::kBytes;
-  static_assert(AttnSmem<DIM, 2>::kBytes == AttnSmem<DIM, 3>::kBytes, "both kernels are launched with the same size");
   const bool causal = (p.flags & FASTAV_CAUSAL) != 0;
   const float scale = p.softmax_scale > 0.f ? p.softmax_scale : 1.0f / sqrtf((float)p.head_dim);
   AttnArgs a{};
@@ -879,23 +923,21 @@ cudaError_t run_attention(const fastav_params& p, const CUtensorMap& q_map, cons
   const int blocks = a.n_pad / kTile;
   int* counters = reinterpret_cast<int*>(ws + w.counters);
   cudaError_t e = once_per_device([&] {
-    const cudaError_t f = cudaFuncSetAttribute(rollout_stats_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    return f == cudaSuccess ? cudaFuncSetAttribute(rollout_map_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : f;
+    const cudaError_t f = cudaFuncSetAttribute(rollout_stats_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)StatSmem<DIM>::kBytes);
+    return f == cudaSuccess ? cudaFuncSetAttribute(rollout_map_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MapSmem<DIM>::kBytes) : f;
   });
   if (e != cudaSuccess) return e;
   if (lse_opt) {
     e = cudaMemsetAsync(counters, 0, (size_t)w.n_counters * sizeof(int), stream);
   } else {
-    e = launch_chained(rollout_stats_kernel<DIM>, dim3(stats_grid(blocks, a.hq, causal)), dim3(kThreads), smem, stream, q_map, k_map, a,
+    e = launch_chained(rollout_stats_kernel<DIM>, dim3(stats_grid(blocks, a.hq, causal)), dim3(kThreads), StatSmem<DIM>::kBytes, stream, q_map, k_map, a,
                        visible_tiles(blocks, causal) * a.hq, counters, w.n_counters, ChainHead{});
     count_launches(1);
   }
   if (e != cudaSuccess) return e;
-  int whole, slices;
-  map_shares(blocks, causal, &whole, &slices);
-  const int work = whole + (int)(visible_tiles(blocks, causal) - whole) * slices;
+  const int units = map_units(blocks, causal, a.hq), strips = (int)map_strips(blocks, causal, units);
   const int zeros = map_out && causal ? (int)hidden_tiles(blocks) : 0;
-  e = launch_chained(rollout_map_kernel<DIM>, dim3(work + zeros), dim3(kThreads), smem, stream, q_map, k_map, a, lse_opt, alpha, whole, slices, work,
+  e = launch_chained(rollout_map_kernel<DIM>, dim3(strips + zeros), dim3(kThreads), MapSmem<DIM>::kBytes, stream, q_map, k_strip_map, a, lse_opt, alpha, units, strips,
                      reinterpret_cast<__nv_bfloat16*>(ws + w.a_hi), reinterpret_cast<__nv_bfloat16*>(ws + w.a_lo), map_out, ChainHead{});
   count_launches(1);
   return e;
@@ -960,16 +1002,17 @@ extern "C" int32_t fastav_rollout_layer(const fastav_params* p, const void* q, c
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   const RolloutWorkspace w = plan_rollout(n, p->num_q_heads);
   const int src = layer_index & 1, dst = src ^ 1;
-  CUtensorMap q_map, k_map, rt_hi_map, rt_lo_map, a_hi_map, a_lo_map;
+  CUtensorMap q_map, k_map, k_strip_map, rt_hi_map, rt_lo_map, a_hi_map, a_lo_map;
   if (!qk_map(q, p->head_dim, p->num_q_heads, n, p->q_stride_tok, p->q_stride_head, &q_map) ||
       !qk_map(k, p->head_dim, p->num_kv_heads, n, p->k_stride_tok, p->k_stride_head, &k_map) ||
+      !qk_map(k, p->head_dim, p->num_kv_heads, n, p->k_stride_tok, p->k_stride_head, &k_strip_map, 32) ||
       !plane_map(state_plane(state, n, src, 0), n_pad, &rt_hi_map) || !plane_map(state_plane(state, n, src, 1), n_pad, &rt_lo_map) ||
       !plane_map(ws + w.a_hi, n_pad, &a_hi_map) || !plane_map(ws + w.a_lo, n_pad, &a_lo_map))
     return FASTAV_ERR_UNSUPPORTED;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   chain_begin(0);
-  cudaError_t e = p->head_dim == 128 ? run_attention<128>(*p, q_map, k_map, lse_opt, alpha, w, ws, map_out_opt, device_status, st)
-                                     : run_attention<64>(*p, q_map, k_map, lse_opt, alpha, w, ws, map_out_opt, device_status, st);
+  cudaError_t e = p->head_dim == 128 ? run_attention<128>(*p, q_map, k_map, k_strip_map, lse_opt, alpha, w, ws, map_out_opt, device_status, st)
+                                     : run_attention<64>(*p, q_map, k_map, k_strip_map, lse_opt, alpha, w, ws, map_out_opt, device_status, st);
   if (e != cudaSuccess) return FASTAV_ERR_CUDA;
   constexpr size_t gemm_smem = 3 * 4 * kSubTileBytes + sizeof(PipeControl) + 1024;
   e = once_per_device([] { return cudaFuncSetAttribute(rollout_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem); });
