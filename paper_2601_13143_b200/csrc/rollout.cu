@@ -21,7 +21,7 @@
 // alone is 36 blocks of 64.  The statistics kernel is PERSISTENT: its (head, row block, key block) items are cut into equal
 // runs, one per SM, and a row block that several runs share leaves up to four partial log-sum-exps per row, which the map
 // kernel merges when it reads them.  The map kernel cuts every row block into STRIPS of at most 32 .. 160 columns, the width
-// that makes the fewest, fullest rounds.  The product cuts the K loops that are longer than an SM's fair share into parts,
+// that makes the fewest, fullest rounds.  The product cuts the K loops that are much longer than an SM's fair share into parts,
 // whose fp32 tiles meet in the workspace: the part that finishes last adds them up in order (no block waits for another).
 // ROLLOUT_FIGURES
 //
@@ -64,6 +64,8 @@ struct alignas(16) PipeControl {
   uint32_t tmem_base;
   int abort;
   int last;                               // product: this block finished the tile's last part
+};
+struct AttnControl : PipeControl {
   union {
     float2 part[2][kColGroups - 1][kTile];  // statistics: (max, sum) per row of column groups 1..3
     float neg_lse[kHeadChunk][kTile];       // map: minus the log2-sum-exp2 of this strip's rows, some heads at a time
@@ -75,17 +77,11 @@ __device__ __forceinline__ void split_bf16(float x, __nv_bfloat16& hi, __nv_bflo
   lo = __float2bfloat16_rn(x - __bfloat162float(hi));
 }
 
-// A tile leaves through shared memory (the operand ring, which is idle by then): a thread holds columns of ONE row, and 32
+// A tile leaves through shared memory (the map's in the operand ring, which is idle by then): a thread holds columns of ONE row, and 32
 // lanes that each store 16 bytes to another row fill half sectors of 32 rows at a time.  The accumulators are put down as
 // they are, and a loop finishes 8 columns at a time, whole rows side by side.  Rows are an odd number of 16-byte pieces
 // apart, so that the 8 rows of a quarter warp fall on different banks.  Product at 2,230 tokens: 28.3 -> 24.8 us.
 constexpr int kStageStride = 32 * kMaxStripUnits + 4;  // floats
-template <int N>
-__device__ __forceinline__ void put_row(float* at, const float (&x)[N], int used) {
-#pragma unroll
-  for (int c = 0; c < N; c += 4)
-    if (c < used) *reinterpret_cast<float4*>(at + c) = make_float4(x[c], x[c + 1], x[c + 2], x[c + 3]);
-}
 __device__ __forceinline__ void store_split(const float (&x)[8], __nv_bfloat16* hi, __nv_bfloat16* lo) {
   alignas(16) __nv_bfloat16 h[8], l[8];
 #pragma unroll
@@ -195,7 +191,7 @@ struct StatSmem {
   static constexpr int kSubTiles = DIM / 64;
   static constexpr int kOperandBytes = kSubTiles * kSubTileBytes;
   static constexpr int kStages = 4;  // the ring of K tiles; two more slots for Q tiles
-  static constexpr size_t kBytes = (size_t)6 * kOperandBytes + sizeof(PipeControl) + 1024;
+  static constexpr size_t kBytes = (size_t)6 * kOperandBytes + sizeof(AttnControl) + 1024;
 };
 
 struct AttnArgs {
@@ -243,7 +239,7 @@ rollout_stats_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
   chain_enter(chain_head);
   const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t slots = base + kStages * kOperandBytes;
-  PipeControl& ctl = *reinterpret_cast<PipeControl*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + 6 * kOperandBytes);
+  AttnControl& ctl = *reinterpret_cast<AttnControl*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + 6 * kOperandBytes);
   volatile int* abort = &ctl.abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int blocks = a.n_pad / kTile;
@@ -399,7 +395,7 @@ struct MapSmem {
   static constexpr int kOperandBytes = kSubTiles * kSubTileBytes;
   static constexpr int kStripSubBytes = 32 * kMaxStripUnits * 128;  // one 64-element column block of the widest strip
   static constexpr int kStripBytes = kSubTiles * kStripSubBytes;
-  static constexpr size_t kBytes = (size_t)kStages * kOperandBytes + kSlots * kStripBytes + sizeof(PipeControl) + 1024;
+  static constexpr size_t kBytes = (size_t)kStages * kOperandBytes + kSlots * kStripBytes + sizeof(AttnControl) + 1024;
   static_assert(kBytes <= 227 * 1024);
 };
 
@@ -417,7 +413,8 @@ rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
   chain_enter(chain_head);
   const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t slots = base + kStages * kOperandBytes;
-  PipeControl& ctl = *reinterpret_cast<PipeControl*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + kStages * kOperandBytes + Cfg::kSlots * Cfg::kStripBytes);
+  AttnControl& ctl =
+      *reinterpret_cast<AttnControl*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + kStages * kOperandBytes + Cfg::kSlots * Cfg::kStripBytes);
   volatile int* abort = &ctl.abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int blocks = a.n_pad / kTile, hq = a.hq, group = a.group;
@@ -607,12 +604,18 @@ rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
 }
 
 // ---- Eq. 3: RT_new = RT_old * A~^T ------------------------------------------------------------------
-// One block per part of a 128 x 128 tile of RT_new.  Per 64-wide K block the four operand tiles (RT hi, RT lo, A~ hi, A~ lo)
+// A unit is a part of a 128 x 128 tile of RT_new.  Per 64-wide K block the four operand tiles (RT hi, RT lo, A~ hi, A~ lo)
 // are loaded once and used for the three products RT hi * A~ hi, RT lo * A~ hi, RT hi * A~ lo, all accumulated into the same
 // TMEM tile.  Under the causal mask RT is upper and A~ lower triangular: tile (m, nn) has the K blocks m .. nn only, so
 // that the tiles of one diagonal nn - m = d have 2 (d + 1) of them.  A tile is cut into ceil(its K blocks / share) equal
-// parts; the blocks are handed out by decreasing d (the longest loops first, the short ones fill the tail), so the parts of
-// cut tiles come first and a part's place in the workspace is its block's number.
+// parts; the parts are listed by decreasing d (the longest loops first, the short ones fill the tail), so the parts of
+// cut tiles come first and a part's place in the workspace is its number.
+// The kernel is persistent, one block per SM, and takes the list back and forth (block b: units b, 2 G - 1 - b, 2 G + b, ..):
+// a unit's tile is stored while the next one's K loop runs on the other accumulator (24.8 -> 21.1 us at 2,230 tokens, with
+// the limit of gemm_share; twelve MMAs of 64 cycles per K block are 6.2 us of it).
+constexpr int kGemmStages = 3;
+constexpr int kGemmStageBytes = 4 * kSubTileBytes;  // 128 x 64 each of RT hi, RT lo, A~ hi, A~ lo
+constexpr int kGemmStageOut = 64 * kTile * sizeof(float);  // half a tile on its way out
 struct GemmUnit {
   int mb, nb, kb0, kb1;  // tile; 64-wide K blocks [kb0, kb1)
   int part, parts;
@@ -648,21 +651,20 @@ struct GemmUnit {
 __global__ void __launch_bounds__(kThreads, 1)
 rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_constant__ CUtensorMap rt_lo_map,
                     const __grid_constant__ CUtensorMap a_hi_map, const __grid_constant__ CUtensorMap a_lo_map, int n_pad,
-                    int causal, int share, int units, __nv_bfloat16* __restrict__ out_hi, __nv_bfloat16* __restrict__ out_lo,
+                    int causal, int share, int units, int grid, __nv_bfloat16* __restrict__ out_hi, __nv_bfloat16* __restrict__ out_lo,
                     float* partials, int* counters, int32_t* device_status, ChainHead chain_head) {
-  constexpr int kStages = 3;
-  constexpr int kStageBytes = 4 * kSubTileBytes;  // 128 x 64 each of RT hi, RT lo, A~ hi, A~ lo
+  constexpr int kStages = kGemmStages, kStageBytes = kGemmStageBytes;
   extern __shared__ unsigned char smem_raw[];
   chain_enter(chain_head);
   const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
-  PipeControl& ctl = *reinterpret_cast<PipeControl*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + kStages * kStageBytes);
+  PipeControl& ctl = *reinterpret_cast<PipeControl*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + kStages * kStageBytes + kGemmStageOut);
   volatile int* abort = &ctl.abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int blocks = n_pad / kTile;
 
-  if ((int)blockIdx.x >= units) {  // the first causal layer: nothing but zeros below the diagonal (later layers leave them)
+  if ((int)blockIdx.x >= grid) {  // the first causal layer: nothing but zeros below the diagonal (later layers leave them)
     pdl_wait();
-    const int t = blockIdx.x - units;  // (mb, nb) with mb > nb
+    const int t = blockIdx.x - grid;  // (mb, nb) with mb > nb
     const int mb = triangular_root(t) + 1, nb = t - (mb - 1) * mb / 2;
     for (int i = threadIdx.x; i < kTile * (kTile / 8); i += kThreads) {
       const int r = i / (kTile / 8), c = (i % (kTile / 8)) * 8;
@@ -672,8 +674,7 @@ rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_
     }
     return;
   }
-  const GemmUnit unit(blockIdx.x, blocks, causal != 0, share);
-  const int iters = unit.exists ? unit.kb1 - unit.kb0 : 0;  // (the host counts the units as the device does: always exists)
+  auto unit_of = [&](int round) { return (round & 1) ? (round + 1) * grid - 1 - (int)blockIdx.x : round * grid + (int)blockIdx.x; };
 
   pipe_setup(ctl, kStages, warp, &rt_hi_map, &a_hi_map);
   const uint32_t tmem = ctl.tmem_base;
@@ -682,91 +683,121 @@ rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_
     if (lane == 0) {
       pdl_wait();
       int it = 0;
-      for (; it < iters; ++it) {
-        const int stage = it % kStages;
-        if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.empty[stage]), ((it / kStages) & 1) ^ 1u, abort)) break;
-        const int kb = unit.kb0 + it;
-        const uint32_t bar = ptx::smem_u32(&ctl.full[stage]);
-        const uint32_t dst = base + stage * kStageBytes;
-        ptx::mbar_arrive_expect_tx(bar, kStageBytes);
-        ptx::tma_load_2d(dst, &rt_hi_map, kb * 64, unit.mb * kTile, bar);
-        ptx::tma_load_2d(dst + kSubTileBytes, &rt_lo_map, kb * 64, unit.mb * kTile, bar);
-        ptx::tma_load_2d(dst + 2 * kSubTileBytes, &a_hi_map, kb * 64, unit.nb * kTile, bar);
-        ptx::tma_load_2d(dst + 3 * kSubTileBytes, &a_lo_map, kb * 64, unit.nb * kTile, bar);
+      bool ok = true;
+      for (int round = 0; ok && unit_of(round) < units; ++round) {
+        const GemmUnit unit(unit_of(round), blocks, causal != 0, share);
+        for (int kb = unit.kb0; kb < unit.kb1; ++kb, ++it) {
+          const int stage = it % kStages;
+          ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.empty[stage]), ((it / kStages) & 1) ^ 1u, abort);
+          if (!ok) break;
+          const uint32_t bar = ptx::smem_u32(&ctl.full[stage]);
+          const uint32_t dst = base + stage * kStageBytes;
+          ptx::mbar_arrive_expect_tx(bar, kStageBytes);
+          ptx::tma_load_2d(dst, &rt_hi_map, kb * 64, unit.mb * kTile, bar);
+          ptx::tma_load_2d(dst + kSubTileBytes, &rt_lo_map, kb * 64, unit.mb * kTile, bar);
+          ptx::tma_load_2d(dst + 2 * kSubTileBytes, &a_hi_map, kb * 64, unit.nb * kTile, bar);
+          ptx::tma_load_2d(dst + 3 * kSubTileBytes, &a_lo_map, kb * 64, unit.nb * kTile, bar);
+        }
       }
       if (*abort) drain_loads(ctl, it, kStages);
     }
   } else if (warp == 1) {
     {
+      int it = 0;
       bool ok = true;
-      for (int it = 0; it < iters && ok; ++it) {
-        const int stage = it % kStages;
-        ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort);
-        if (!ok) break;
-        ptx::tc_fence_after_sync();
-        const uint32_t rt_hi = base + stage * kStageBytes, rt_lo = rt_hi + kSubTileBytes, a_hi = rt_hi + 2 * kSubTileBytes,
-                       a_lo = rt_hi + 3 * kSubTileBytes;
-        const uint64_t rt_hi_desc = ptx::umma_desc_sw128(rt_hi, 0), rt_lo_desc = ptx::umma_desc_sw128(rt_lo, 0),
-                       a_hi_desc = ptx::umma_desc_sw128(a_hi, 0), a_lo_desc = ptx::umma_desc_sw128(a_lo, 0);
-        constexpr uint32_t idesc = ptx::umma_idesc_bf16(kTile, kTile);
-        ptx::umma_bf16_steps<4, 0, 0>(tmem, rt_hi_desc, a_hi_desc, idesc, it > 0);
-        ptx::umma_bf16_steps<4, 0, 0>(tmem, rt_lo_desc, a_hi_desc, idesc, true);
-        ptx::umma_bf16_steps<4, 0, 0>(tmem, rt_hi_desc, a_lo_desc, idesc, true);
-        ptx::umma_commit(ptx::smem_u32(&ctl.empty[stage]));
+      for (int round = 0; ok && unit_of(round) < units; ++round) {
+        const GemmUnit unit(unit_of(round), blocks, causal != 0, share);
+        const int buf = round & 1;
+        ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_empty[buf]), ((round >> 1) & 1) ^ 1u, abort);
+        for (int kb = unit.kb0; kb < unit.kb1 && ok; ++kb, ++it) {
+          const int stage = it % kStages;
+          ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort);
+          if (!ok) break;
+          ptx::tc_fence_after_sync();
+          const uint32_t rt_hi = base + stage * kStageBytes, rt_lo = rt_hi + kSubTileBytes, a_hi = rt_hi + 2 * kSubTileBytes,
+                         a_lo = rt_hi + 3 * kSubTileBytes;
+          const uint64_t rt_hi_desc = ptx::umma_desc_sw128(rt_hi, 0), rt_lo_desc = ptx::umma_desc_sw128(rt_lo, 0),
+                         a_hi_desc = ptx::umma_desc_sw128(a_hi, 0), a_lo_desc = ptx::umma_desc_sw128(a_lo, 0);
+          constexpr uint32_t idesc = ptx::umma_idesc_bf16(kTile, kTile);
+          const uint32_t d = tmem + buf * kTile;
+          ptx::umma_bf16_steps<4, 0, 0>(d, rt_hi_desc, a_hi_desc, idesc, kb > unit.kb0);
+          ptx::umma_bf16_steps<4, 0, 0>(d, rt_lo_desc, a_hi_desc, idesc, true);
+          ptx::umma_bf16_steps<4, 0, 0>(d, rt_hi_desc, a_lo_desc, idesc, true);
+          ptx::umma_commit(ptx::smem_u32(&ctl.empty[stage]));
+        }
+        if (ok) ptx::umma_commit(ptx::smem_u32(&ctl.tmem_full[buf]));
       }
-      if (ok) ptx::umma_commit(ptx::smem_u32(&ctl.tmem_full[0]));
     }
   } else {
     const int quarter = warp & 3, cg = (warp - 2) >> 2;
     const int row_in = quarter * 32 + lane, ethread = cg * kTile + row_in;
     pdl_wait();
-    const bool ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_full[0]), 0, abort);
-    float x[32];
-    if (ok) {
-      ptx::tc_fence_after_sync();
-      uint32_t v[32];
-      ptx::tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + cg * 32, v);
-      ptx::tmem_ld_wait_for(v);
+    bool ok = true;
+#pragma unroll 1
+    for (int round = 0; unit_of(round) < units; ++round) {
+      const int u = unit_of(round), buf = round & 1;
+      const GemmUnit unit(u, blocks, causal != 0, share);
+      if (ok) ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_full[buf]), (round >> 1) & 1, abort);
+      float x[32];
+      if (ok) {
+        ptx::tc_fence_after_sync();
+        uint32_t v[32];
+        ptx::tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + buf * kTile + cg * 32, v);
+        ptx::tmem_ld_wait_for(v);
+        ptx::tc_fence_before_sync();
+        ptx::mbar_arrive_warp(ptx::smem_u32(&ctl.tmem_empty[buf]), lane);  // the accumulator may be overwritten
 #pragma unroll
-      for (int c = 0; c < 32; ++c) x[c] = __uint_as_float(v[c]);
-    } else {
-#pragma unroll
-      for (int c = 0; c < 32; ++c) x[c] = 0.f;
-    }
-    bool mine = ok;  // this block writes the tile
-    if (unit.parts > 1) {
-      constexpr int kFloats = kTile * kTile;
-      float* const here = partials + (size_t)blockIdx.x * kFloats + ethread;
-#pragma unroll
-      for (int c = 0; c < 32; ++c) __stcg(here + c * kEpilogueThreads, x[c]);
-      __threadfence();
-      epilogue_sync();
-      if (ethread == 0) ctl.last = atomicAdd(counters + unit.mb * blocks + unit.nb, 1) == unit.parts - 1 && !ctl.abort;
-      epilogue_sync();
-      mine = ok && ctl.last != 0;
-      if (mine) {  // the last part to finish: add the parts up in order
-        __threadfence();
-        const float* p = partials + (size_t)(blockIdx.x - unit.part) * kFloats + ethread;
+        for (int c = 0; c < 32; ++c) x[c] = __uint_as_float(v[c]);
+      } else {
 #pragma unroll
         for (int c = 0; c < 32; ++c) x[c] = 0.f;
-#pragma unroll 1
-        for (int i = 0; i < unit.parts; ++i, p += kFloats) {
-#pragma unroll
-          for (int c = 0; c < 32; ++c) x[c] += __ldcg(p + c * kEpilogueThreads);
-        }
       }
-    }
-    float* const stage = reinterpret_cast<float*>(smem_raw + (base - ptx::smem_u32(smem_raw)));
-    if (mine) put_row(stage + row_in * kStageStride + cg * 32, x, 32);
-    epilogue_sync();
-    if (mine) {
+      bool mine = ok;  // this block writes the tile
+      if (unit.parts > 1) {
+        constexpr int kFloats = kTile * kTile;
+        float* const here = partials + (size_t)u * kFloats + ethread;
+#pragma unroll
+        for (int c = 0; c < 32; ++c) __stcg(here + c * kEpilogueThreads, x[c]);
+        __threadfence();
+        epilogue_sync();
+        if (ethread == 0) ctl.last = atomicAdd(counters + unit.mb * blocks + unit.nb, 1) == unit.parts - 1 && !ctl.abort;
+        epilogue_sync();
+        mine = ok && ctl.last != 0;
+        if (mine) {  // the last part to finish: add the parts up in order
+          __threadfence();
+          const float* p = partials + (size_t)(u - unit.part) * kFloats + ethread;
+#pragma unroll
+          for (int c = 0; c < 32; ++c) x[c] = 0.f;
 #pragma unroll 1
-      for (int e = ethread; e < kTile * kTile / 8; e += kEpilogueThreads) {
-        const int r_in = e / (kTile / 8), c_in = e % (kTile / 8) * 8;
-        float y[8];
-        get8(stage + r_in * kStageStride + c_in, y);
-        const long long at = (long long)(unit.mb * kTile + r_in) * n_pad + unit.nb * kTile + c_in;
-        store_split(y, out_hi + at, out_lo + at);
+          for (int i = 0; i < unit.parts; ++i, p += kFloats) {
+#pragma unroll
+            for (int c = 0; c < 32; ++c) x[c] += __ldcg(p + c * kEpilogueThreads);
+          }
+        }
+        if (!ctl.last) continue;  // (uniform for the epilogue)
+      }
+      // 64 rows at a time; a row's 16-byte pieces are permuted by its number, so that 8 rows fall on different banks
+      float4* const stage = reinterpret_cast<float4*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + kStages * kStageBytes);
+#pragma unroll 1
+      for (int half = 0; half < 2; ++half) {
+        if (quarter >> 1 == half) {
+          const int r = row_in & 63;
+#pragma unroll
+          for (int c = 0; c < 32; c += 4)
+            stage[r * 32 + ((cg * 8 + c / 4) ^ (r & 7))] = make_float4(x[c], x[c + 1], x[c + 2], x[c + 3]);
+        }
+        epilogue_sync();
+        if (mine) {
+#pragma unroll
+          for (int i = 0; i < 64 * 16 / kEpilogueThreads; ++i) {
+            const int e = ethread + i * kEpilogueThreads, r = e >> 4, c = e & 15;
+            const float4 p = stage[r * 32 + ((2 * c) ^ (r & 7))], q = stage[r * 32 + ((2 * c + 1) ^ (r & 7))];
+            const float y[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+            const long long at = (long long)(unit.mb * kTile + half * 64 + r) * n_pad + unit.nb * kTile + c * 8;
+            store_split(y, out_hi + at, out_lo + at);
+          }
+        }
+        epilogue_sync();
       }
     }
   }
@@ -918,11 +949,13 @@ int map_units(int blocks, bool causal, int hq) {
   return best;
 }
 
-// Product: no K loop longer than an SM's share of all K blocks (at least eight: a part costs an exchange of 64 KB).
+// Product: no K loop longer than one and a half times an SM's share of all K blocks, and at least twelve: a part costs an
+// exchange of 64 KB, 4,000 to 8,000 cycles, the time of five to ten K blocks.  2,230 tokens (fair share 16): limits of
+// 16 / 18 / 20 / 22 / 24 / 28 and none (36) took 23.9 / 23.0 / 22.1 / 21.1 / 21.1 / 22.3 / 25.6 us.
 int gemm_share(int blocks, bool causal) {
   const long long items = causal ? (long long)blocks * (blocks + 1) * (blocks + 2) / 3 : 2ll * blocks * blocks * blocks;
-  const long long share = (items + kNumSMs - 1) / kNumSMs;
-  return (int)(share < 8 ? 8 : share);
+  const long long share = (3 * items / 2 + kNumSMs - 1) / kNumSMs;
+  return (int)(share < 12 ? 12 : share);
 }
 // Parts in all, and those of tiles that are cut (they come first).
 void gemm_units(int blocks, bool causal, int share, int* units, int* cut) {
@@ -1067,16 +1100,18 @@ extern "C" int32_t fastav_rollout_layer(const fastav_params* p, const void* q, c
   cudaError_t e = p->head_dim == 128 ? run_attention<128>(*p, q_map, k_map, k_strip_map, lse_opt, alpha, w, ws, map_out_opt, device_status, st)
                                      : run_attention<64>(*p, q_map, k_map, k_strip_map, lse_opt, alpha, w, ws, map_out_opt, device_status, st);
   if (e != cudaSuccess) return FASTAV_ERR_CUDA;
-  constexpr size_t gemm_smem = 3 * 4 * kSubTileBytes + sizeof(PipeControl) + 1024;
+  constexpr size_t gemm_smem = kGemmStages * kGemmStageBytes + kGemmStageOut + sizeof(PipeControl) + 1024;
+  static_assert(gemm_smem <= 227 * 1024);
   e = once_per_device([] { return cudaFuncSetAttribute(rollout_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem); });
   if (e != cudaSuccess) return FASTAV_ERR_CUDA;
   const bool causal = (p->flags & FASTAV_CAUSAL) != 0;
   const int blocks = n_pad / kTile, share = gemm_share(blocks, causal);
   int units, cut;
   gemm_units(blocks, causal, share, &units, &cut);
+  const int grid = units < kNumSMs ? units : kNumSMs;
   const int zeros = causal && layer_index == 0 ? (int)hidden_tiles(blocks) : 0;
-  e = launch_chained(rollout_gemm_kernel, dim3(units + zeros), dim3(kThreads), gemm_smem, st, rt_hi_map, rt_lo_map, a_hi_map, a_lo_map, n_pad,
-                     causal ? 1 : 0, share, units, state_plane(state, n, dst, 0), state_plane(state, n, dst, 1),
+  e = launch_chained(rollout_gemm_kernel, dim3(grid + zeros), dim3(kThreads), gemm_smem, st, rt_hi_map, rt_lo_map, a_hi_map, a_lo_map, n_pad,
+                     causal ? 1 : 0, share, units, grid, state_plane(state, n, dst, 0), state_plane(state, n, dst, 1),
                      reinterpret_cast<float*>(ws + w.partials), reinterpret_cast<int*>(ws + w.counters), device_status, ChainHead{});
   count_launches(1);
   return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? FASTAV_OK : FASTAV_ERR_CUDA;
