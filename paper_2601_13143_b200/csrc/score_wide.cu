@@ -277,9 +277,9 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
     for (int i = 0; i < 4; ++i) {
       ptx::mbar_init(ptx::smem_u32(&ctl.tmem_full[i]), 1);
       // sweep 1: accumulator (e, i) is read by the two warpgroups of row tile e; sweep 2: accumulator i by all four
-      ptx::mbar_init(ptx::smem_u32(&ctl.tmem_empty[i]), SWEEP == 1 ? 8 : 4 * kGroups);  // one arrival per warp
+      ptx::mbar_init(ptx::smem_u32(&ctl.tmem_empty[i]), SWEEP == 1 ? 256 : 128 * kGroups);
     }
-    for (int i = 0; i < 2; ++i) ptx::mbar_init(ptx::smem_u32(&ctl.sums_ready[i]), 4 * (kGroups - 1));
+    for (int i = 0; i < 2; ++i) ptx::mbar_init(ptx::smem_u32(&ctl.sums_ready[i]), 128 * (kGroups - 1));
     ctl.abort = 0;
     ptx::fence_barrier_init();
     ptx::prefetch_tensormap(&k_map);
@@ -350,8 +350,11 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
       }
     }
   } else if (warp == 1) {
-    // ---- MMA issuer: one elected lane -------------------------------------------------------------
-    {
+    // ---- MMA issuer: one lane.  Issue by an elected lane of the whole warp is quicker, and so is one arrival per warp at the
+    // accumulators' barriers, but these sweeps wait for their softmax warps, and both made them slower: 4 x 16,384 tokens, 128
+    // rows, sweep 1 / 2: 86.3 / 80.0 us as it is, 87.0 / 80.9 with warp arrivals, 88.1 / 81.5 with elected issue, 90.0 / 82.0
+    // with both.
+    if (lane == 0) {
       int tile_no = 0, q_gen = 0;
       int uses0 = 0, uses1 = 0;  // sweep 1: how often the accumulators of 128-row tile e have been used
       bool ok = true;
@@ -382,13 +385,13 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
               ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_empty[i * 2 + e]), ((uses >> 1) & 1) ^ 1u, abort);
               if (!ok) break;
               ptx::tc_fence_after_sync();
-              ptx::umma_bf16_steps<DIM / 16, L::kQSubBytes, L::kKSubBytes>(tmem + i * 256 + e * 128, ptx::umma_desc_sw128(q_smem + e * 128 * 128, 0),
+              ptx::umma_bf16_steps<DIM / 16, L::kQSubBytes, L::kKSubBytes, false>(tmem + i * 256 + e * 128, ptx::umma_desc_sw128(q_smem + e * 128 * 128, 0),
                                                                            ptx::umma_desc_sw128(k_tile, 0), ptx::umma_idesc_bf16(128, kTileKeys), false);
-              ptx::umma_commit(ptx::smem_u32(&ctl.tmem_full[i * 2 + e]));
+              ptx::umma_commit<false>(ptx::smem_u32(&ctl.tmem_full[i * 2 + e]));
               if (e == 0) ++uses0; else ++uses1;
             }
             if (!ok) break;
-            ptx::umma_commit(ptx::smem_u32(&ctl.empty_k[stage]));
+            ptx::umma_commit<false>(ptx::smem_u32(&ctl.empty_k[stage]));
           } else {
             // S^T = K Q^T: A = 128 keys, B = n_cols query rows; accumulator i at columns i*256.
             const int i = tile_no & 1;
@@ -396,14 +399,14 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
             if (!ok) break;
             ptx::tc_fence_after_sync();
             const uint32_t idesc = ptx::umma_idesc_bf16(kTileKeys, n_cols);
-            ptx::umma_bf16_steps<DIM / 16, L::kKSubBytes, L::kQSubBytes>(tmem + i * 256, ptx::umma_desc_sw128(k_tile, 0), ptx::umma_desc_sw128(q_smem, 0),
+            ptx::umma_bf16_steps<DIM / 16, L::kKSubBytes, L::kQSubBytes, false>(tmem + i * 256, ptx::umma_desc_sw128(k_tile, 0), ptx::umma_desc_sw128(q_smem, 0),
                                                                          idesc, false);
-            ptx::umma_commit(ptx::smem_u32(&ctl.empty_k[stage]));
-            ptx::umma_commit(ptx::smem_u32(&ctl.tmem_full[i]));
+            ptx::umma_commit<false>(ptx::smem_u32(&ctl.empty_k[stage]));
+            ptx::umma_commit<false>(ptx::smem_u32(&ctl.tmem_full[i]));
           }
         }
         // Once the MMAs issued so far are done, the query tile may be replaced.
-        if (ok && u + 1 < n_units && ctl.units[u + 1].new_q) ptx::umma_commit(ptx::smem_u32(&ctl.q_free));
+        if (ok && u + 1 < n_units && ctl.units[u + 1].new_q) ptx::umma_commit<false>(ptx::smem_u32(&ctl.q_free));
       }
     }
   } else {
@@ -447,7 +450,7 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
           fold_row_piece_any(va, bound, s.scale_log2, zmax, sum2);
           tmem_ld_wait_for(vb);
           ptx::tc_fence_before_sync();
-          ptx::mbar_arrive_warp(ptx::smem_u32(&ctl.tmem_empty[i * 2 + e]), lane);  // the accumulator may be overwritten
+          ptx::mbar_arrive(ptx::smem_u32(&ctl.tmem_empty[i * 2 + e]));  // the accumulator may be overwritten
           fold_row_piece_any(vb, bound - 32, s.scale_log2, zmax, sum2);
         }
         if (ok && row_valid) {
@@ -488,7 +491,7 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
             ptx::tmem_ld32(lane_addr + i * 256 + wg * 32, v);
             tmem_ld_wait_for(v);
             ptx::tc_fence_before_sync();
-            ptx::mbar_arrive_warp(ptx::smem_u32(&ctl.tmem_empty[i]), lane);
+            ptx::mbar_arrive(ptx::smem_u32(&ctl.tmem_empty[i]));
             if (key < un.n) {
 #pragma unroll
               for (int c = 0; c < 32; ++c)
@@ -497,7 +500,7 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
             }
           } else {
             ptx::tc_fence_before_sync();
-            ptx::mbar_arrive_warp(ptx::smem_u32(&ctl.tmem_empty[i]), lane);
+            ptx::mbar_arrive(ptx::smem_u32(&ctl.tmem_empty[i]));
           }
         }
       }
@@ -552,7 +555,7 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
           if (wg > 0) {
             // sums[i] is free again: warpgroup 0 read it before it released accumulator i two tiles ago
             ctl.sums[i][wg - 1][my_lane] = sum;
-            ptx::mbar_arrive_warp(ptx::smem_u32(&ctl.sums_ready[i]), lane);
+            ptx::mbar_arrive(ptx::smem_u32(&ctl.sums_ready[i]));
           } else {
             ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.sums_ready[i]), parity, abort);
             if (!ok) break;
@@ -561,7 +564,7 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
             if (key < un.n) out[key] = sum;
           }
           ptx::tc_fence_before_sync();
-          ptx::mbar_arrive_warp(ptx::smem_u32(&ctl.tmem_empty[i]), lane);
+          ptx::mbar_arrive(ptx::smem_u32(&ctl.tmem_empty[i]));
         }
       }
     }

@@ -81,8 +81,7 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
   }
 }
 
-// One arrival for a whole warp: 32 single ones queue at the barrier's word like atomics (an epilogue of 512 threads spends
-// more on them than on reading its accumulators).  Orders the warp's earlier shared-memory accesses before the arrival.
+// One arrival for a whole warp; orders the warp's earlier shared-memory accesses before the arrival.
 __device__ __forceinline__ void mbar_arrive_warp(uint32_t bar, int lane) {
   __syncwarp();
   if (lane == 0) mbar_arrive(bar);
@@ -203,30 +202,45 @@ __host__ __device__ constexpr uint32_t umma_idesc_bf16(int m, int n) {
          | ((uint32_t)(m >> 4) << 24); // M / 16
 }
 
-// D[tmem] (+)= A[smem] * B[smem]^T.  Called by a whole converged warp; one elected lane issues.  (A loop that one lane runs
-// alone keeps the descriptors in per-thread registers and issues at half the pace: eight MMAs 700 cycles instead of 420.)
+// D[tmem] (+)= A[smem] * B[smem]^T.  ELECT: called by a whole converged warp, one elected lane issues; else called by one
+// thread.  (A loop that one lane runs alone keeps the descriptors in per-thread registers and issues at half the pace, eight
+// MMAs 700 cycles instead of 420; the two-sweep score, which waits for its epilogue, is the faster for it.)
+template <bool ELECT = true>
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t"
-      ".reg .pred p, q;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "elect.sync _|q, 0xFFFFFFFF;\n\t"
-      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
-      "}\n" ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
+  if constexpr (ELECT)
+    asm volatile(
+        "{\n\t"
+        ".reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "elect.sync _|q, 0xFFFFFFFF;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
+        "}\n" ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+  else
+    asm volatile(
+        "{\n\t"
+        ".reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
+        "}\n" ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
 }
 // The same over a K range of 16 STEPS elements: the 16-element slices of one 128-byte row lie 32 bytes apart, the next 64
 // elements `a_sub` / `b_sub` bytes further on.  The descriptors are made once and stepped by constants.
-template <int STEPS, int A_SUB, int B_SUB>
+template <int STEPS, int A_SUB, int B_SUB, bool ELECT = true>
 __device__ __forceinline__ void umma_bf16_steps(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate) {
 #pragma unroll
   for (int ks = 0; ks < STEPS; ++ks)
-    umma_bf16(d_tmem, a_desc + (uint64_t)((ks / 4) * (A_SUB >> 4) + (ks % 4) * 2), b_desc + (uint64_t)((ks / 4) * (B_SUB >> 4) + (ks % 4) * 2), idesc,
-              ks > 0 || accumulate ? 1u : 0u);
+    umma_bf16<ELECT>(d_tmem, a_desc + (uint64_t)((ks / 4) * (A_SUB >> 4) + (ks % 4) * 2), b_desc + (uint64_t)((ks / 4) * (B_SUB >> 4) + (ks % 4) * 2),
+                     idesc, ks > 0 || accumulate ? 1u : 0u);
 }
-// Makes `bar` receive one arrival when every MMA issued so far has finished (whole warp, the same elected lane).
+// Makes `bar` receive one arrival when every MMA issued so far by the same lane has finished.
+template <bool ELECT = true>
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xFFFFFFFF;\n\t@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar) : "memory");
+  if constexpr (ELECT)
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xFFFFFFFF;\n\t@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar) : "memory");
+  else
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
 __device__ __forceinline__ float ex2_approx(float x) {
