@@ -112,11 +112,11 @@ cudaError_t launch_select_scores(const Shapes& s, const float* scores, const Sel
 
 // Many scored rows on short sequences: one pass over K (score_once.cu).
 struct OncePlan {
-  int rows_per_tile, row_tiles, blocks, tiles_per_block;
+  int rows_per_tile, row_tiles, blocks, tiles_per_block, rounds;
 };
 constexpr int kOnceMaxTokens = 4096;
 int once_row_tiles(int max_qlen, int group);
-bool once_plan(const Shapes& s, OncePlan* plan);
+bool once_plan(const Shapes& s, bool lse_given, OncePlan* plan);
 cudaError_t launch_score_once(const Shapes& s, const void* k_map, const void* q_map, const int32_t* q_idx, const int32_t* cu_qlens,
                               const int32_t* cu_seqlens, const float* lse_in, const OncePlan& plan, float* partial, int32_t* device_status,
                               cudaStream_t stream);

@@ -10,7 +10,9 @@
 //   key per lane -> partial[KV head, row tile][token], which the selecting kernel (prune_few.cu) adds up.
 //
 // Two kernels (this and the selection) replace five (two sweeps, merge, per-token sums, selection).  Bound: latency, the
-// chip is far from full.  ONCE_FIGURES
+// chip is far from full.  Prune calls against the two-sweep path (28 / 4 heads, half the tokens kept): 32 rows on 1 x 1,024
+// tokens 16.9 us instead of 28.9, 1 x 2,048 20.7 / 31.0, 4 x 2,048 36.3 / 50.1, 1 x 4,096 28.9 / 32.9; 128 rows on 1 x 2,048
+// 25.9 / 37.7.
 //
 // A key's sums do not depend on its position (every column goes through the same arithmetic and the same tree), and a
 // row's statistics are kept per key tile and folded in tile order, so that equal keys get bit-equal scores and a sequence's
@@ -339,22 +341,41 @@ int once_row_tiles(int max_qlen, int group) {
   return per == 0 ? 0 : (max_qlen * group + per - 1) / per;
 }
 
-bool once_plan(const Shapes& s, OncePlan* plan) {
+bool once_plan(const Shapes& s, bool lse_given, OncePlan* plan) {
   plan->rows_per_tile = once_rows_per_tile(s.group);
   if (plan->rows_per_tile == 0 || s.max_seqlen < 1 || s.max_qlen < 1) return false;
   plan->row_tiles = once_row_tiles(s.max_qlen, s.group);
   const int tiles = (s.max_seqlen + kTile - 1) / kTile;
   if (tiles > kMaxTiles) return false;
   const long long clusters = (long long)s.batch * s.hkv * plan->row_tiles;
-  // The fewest key tiles per block with which all clusters run at once (ONCE_RULE).
+  // Key tiles per block: the least time of all rounds (in quarters of a microsecond): a round of clusters that run at once takes
+  // some 6 us and 3.75 us per key tile of a block.  One round is always the better way (1 x 2,048 tokens, 32 rows, 28 / 4 heads:
+  // 20.7 us with 2 key tiles per block in one round, 26.5 with 1 in two; the two sweeps 31.0).  Several rounds are compared with
+  // the two sweeps: about 19 us, and per SM and key tile 2.25 us for every 128 rows of the first and 128 columns of the second.
+  // Prune of 32 x 512 tokens, 32 rows: 60.0 against 71.1 us (32 / 8 heads: 66.8 against 83.4), 15 x 1,024: 57.9 / 64.5, but
+  // 2 x 4,096 tokens, 32 / 8 heads: 57.9 / 52.8, 16 x 2,048, 8 rows, 32 / 8 heads: 127 / 116.
+  long long least = LLONG_MAX;
   for (int per = 1; per <= kBlockTiles; ++per) {
     const int blocks = (tiles + per - 1) / per;
-    if (blocks > kMaxCluster || clusters > kAtOnce[blocks]) continue;
+    if (blocks > kMaxCluster) continue;
+    const long long rounds = (clusters + kAtOnce[blocks] - 1) / kAtOnce[blocks], cost = rounds * (24 + 15 * per);
+    if (cost >= least) continue;
+    least = cost;
     plan->blocks = blocks;
     plan->tiles_per_block = per;
-    return true;
+    plan->rounds = (int)(rounds < 100 ? rounds : 100);
   }
-  return false;
+  if (least == LLONG_MAX) return false;
+  if (plan->rounds == 1 || lse_given) return plan->rounds == 1;
+  const long long key_tiles = s.total_tokens / kTile + (s.batch + 1) / 2;
+  const int flat = s.max_qlen * s.group, chunk = wide_rows_per_chunk(s.group);
+  long long per_tile = 0;  // of the first sweep in steps of 128 rows, of the second in rows
+  for (int f = 0; f < flat; f += chunk) {
+    const int rows = flat - f < chunk ? flat - f : chunk;
+    per_tile += 9 * ((rows + 127) / 128) + 9 * (rows > 64 ? rows : 64) / 128;
+  }
+  const long long sweeps = 75 + key_tiles * s.hkv * per_tile / kNumSMs;
+  return least + least / 32 < sweeps;
 }
 
 cudaError_t launch_score_once(const Shapes& s, const void* k_map, const void* q_map, const int32_t* q_idx, const int32_t* cu_qlens,

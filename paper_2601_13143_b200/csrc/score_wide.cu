@@ -734,7 +734,7 @@ cudaError_t run(const Shapes& s, const Workspace& w, const CUtensorMap& k_map, c
                           dim3(kFinalizeThreads), 0, stream, s, cu_seqlens, cu_qlens, row_chunks, chunk, (const float*)partial, scores_out);
   };
   OncePlan once;
-  if (scores_out && (s.flags & FASTAV_SCORE_PATH_MASK) == 0 && once_plan(s, &once)) {
+  if (scores_out && (s.flags & FASTAV_SCORE_PATH_MASK) == 0 && once_plan(s, lse_in != nullptr, &once)) {
     const cudaError_t f = launch_score_once(s, &k_map, &q_map, q_idx, cu_qlens, cu_seqlens, lse_in, once, partial, device_status, stream);
     return f != cudaSuccess ? f : finish(once.row_tiles, once.rows_per_tile);
   }
