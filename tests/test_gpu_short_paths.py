@@ -1,0 +1,75 @@
+"""The prune call's paths for short sequences and their borders: the few-rows cluster kernel (up to 4 scored rows, 2,048 tokens),
+the one-pass score in tensor memory (up to 4,096 tokens; one round of clusters or several), the cluster selection from partial
+sums and from finished scores, rows gathered by the selecting blocks or by the compaction, the mask's emission with one kernel
+or two.  Against the oracle; keep sets as parity.py judges them (scores within its bound, equal keys bit-equal)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import parity
+from paper_2601_13143_b200 import fastav, workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(lens, rows, hq, hkv, d, hid=64, keep=0.5, **more):
+    p = W.random_problem(seed=sum(lens) + hq + rows, lens=lens, rows=[min(rows, n) for n in lens], keeps=[max(min(1, n), int(n * keep)) for n in lens],
+                         num_q_heads=hq, num_kv_heads=hkv, head_dim=d, hidden=hid, duplicate_keys=2, **more)
+    p.protect_rows = rows % 2 == 1
+    protect = (torch.arange(p.total_tokens) % 29 == 3).to(torch.uint8) if hq % 8 == 0 else None
+    buf = parity.to_device(p, protect=protect)
+    buf.prune()
+    torch.cuda.synchronize()
+    stats = parity.check_fused_against_oracle(p, buf, parity.oracle_prune(p, protect=protect), protect=protect, what=f"{lens} x {rows}")
+    assert stats["device_status"] & ~fastav.FASTAV_DEV_PROTECT_OVERFLOW == 0
+
+
+# Few rows: ends of fragments (8, 16), segments (32) and of the token range; 1-4 rows; groups of 1, 2, 4, 7; clusters of 16 down to 1
+# (more sequences than clusters that run at once), and batches beyond the number of SMs on either side of 512 tokens.
+@pytest.mark.parametrize("lens,rows,hq,hkv,d", [
+    ([1], 1, 2, 1, 64), ([15, 33, 8], 2, 4, 4, 64), ([511, 512, 513], 3, 8, 2, 128), ([2047], 4, 28, 4, 128), ([2048], 1, 28, 4, 128),
+    ([2049], 1, 28, 4, 128), ([1025, 0, 31] * 4, 1, 8, 4, 64), ([200, 64] * 20, 2, 4, 2, 64), ([70] * 149, 1, 4, 1, 64), ([512] * 2 + [9] * 150, 1, 4, 2, 64),
+    ([513] + [9] * 150, 1, 4, 2, 64),
+])
+def test_few_rows(lens, rows, hq, hkv, d):
+    _check(lens, rows, hq, hkv, d)
+
+
+# Many rows, one pass: ends of key tiles (128) and of the range, row tiles that are not full, groups of 1 to 16, one round of
+# clusters and several, and the two-sweep path next to it (4,097 tokens; a group of 17).
+@pytest.mark.parametrize("lens,rows,hq,hkv,d", [
+    ([5], 5, 2, 2, 64), ([127, 128, 129], 9, 8, 8, 64), ([1000, 3], 33, 28, 4, 128), ([4095], 8, 8, 2, 128), ([4096], 17, 16, 1, 64), ([4097], 8, 8, 2, 128),
+    ([2048, 100], 130, 4, 2, 64), ([300], 12, 17, 1, 64), ([512] * 40, 32, 28, 4, 128), ([1024, 640, 999] * 5, 32, 8, 8, 64), ([256] * 24, 128, 16, 4, 64),
+])
+@pytest.mark.parametrize("trailing", [True, False])
+def test_many_rows(lens, rows, hq, hkv, d, trailing):
+    _check(lens, rows, hq, hkv, d, trailing_rows=trailing)
+
+
+# Rows gathered by the selecting blocks (little per block) or by the compaction (more), and rows per warp around the ring's depth.
+@pytest.mark.parametrize("n,keep,hid", [(64, 1.0, 8), (512, 0.9, 512), (1500, 0.7, 64), (1500, 0.9, 2048), (2048, 0.1, 3584), (2048, 1.0, 1024)])
+@pytest.mark.parametrize("rows", [1, 8])
+def test_gather_by_either_kernel(n, keep, hid, rows):
+    _check([n, n // 3], rows, 8, 2, 64, hid=hid, keep=keep)
+
+
+@pytest.mark.parametrize("total,batch", [(1, 1), (4095, 3), (4097, 1), ((1 << 18), 7), ((1 << 18) + 1, 7), (300_000, 513)])
+@pytest.mark.parametrize("offset", [0, 1])  # masks that are not 16-byte aligned
+def test_mask_emission(total, batch, offset):
+    rng = np.random.default_rng(total + offset)
+    cu = np.concatenate([[0], np.sort(rng.integers(0, total + 1, batch - 1)), [total]]).astype(np.int32)
+    mask = (rng.random(total) < 0.6).astype(np.uint8)
+    ref_idx, ref_cu = oracle.select_mask(mask, cu)
+    kept = int(ref_cu[-1])
+    params = fastav.make_params(batch=batch, total_tokens=total, max_seqlen=int(np.diff(cu).max()), total_q=0, max_qlen=0, total_keep=kept,
+                                max_keep=kept, num_q_heads=4, num_kv_heads=2, head_dim=64, hidden=64)
+    held = torch.zeros(total + 16, dtype=torch.uint8, device="cuda")
+    held[offset:offset + total] = torch.from_numpy(mask).cuda()
+    idx = torch.full((kept + 8,), -7, dtype=torch.int32, device="cuda")
+    cu_keep, status = torch.empty(batch + 1, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(max(256, fastav.fastav_workspace_bytes(params)), dtype=torch.uint8, device="cuda")
+    fastav.fastav_select_mask(params, held[offset:offset + total], torch.from_numpy(cu).cuda(), idx, cu_keep, ws, status)
+    torch.cuda.synchronize()
+    assert int(status) == 0 and cu_keep.cpu().tolist() == ref_cu.tolist()
+    assert np.array_equal(idx.cpu().numpy(), np.concatenate([ref_idx, np.full(8, -7)]))
