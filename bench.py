@@ -188,7 +188,9 @@ def host_chain(w: W.Workload, device):
              "arena": torch.empty(fastav.fastav_host_arena_bytes(params), dtype=torch.uint8, device=device)}
         ins = ("q", "q_idx", "cu_qlens", "k", "v", "cu_seqlens", "keep_counts", "hidden", "pos")
         outs = ("scores", "keep_idx", "cu_keep", "hidden_out", "pos_out", "k_out", "v_out", "status")
-        h["h2d"] = sum(h[x].numel() * h[x].element_size() for x in ins)
+        # of the hidden states and V only the survivors' rows are read
+        sent = [h[{"v": "v_out", "hidden": "hidden_out"}.get(x, x)] for x in ins]
+        h["h2d"] = sum(t.numel() * t.element_size() for t in sent)
         h["d2h"] = sum(h[x].numel() * h[x].element_size() for x in outs)
         out.append(h)
         prev = h
