@@ -24,7 +24,7 @@
 // that makes the fewest, fullest rounds.  The product cuts the K loops that are much longer than an SM's fair share into parts,
 // whose fp32 tiles meet in the workspace: the part that finishes last adds them up in order (no block waits for another).
 // 2,230 tokens, 28 / 4 heads of 128, per layer: statistics 34, map 37.4, product 21.1 us; 14 layers with their
-// read-out 1,168 us (1,924 with a block per tile and head, or per tile).
+// read-out 1,164 us (1,924 with a block per tile and head, or per tile).
 //
 // Warp 0 issues the TMA loads, warp 1 the MMAs into accumulators in tensor memory, warps 2..17 are the epilogue
 // (thread <-> accumulator row, four warps per 32-lane quarter of TMEM, a quarter of the columns each).  The epilogue of
@@ -837,20 +837,35 @@ __global__ void __launch_bounds__(256) rollout_importance_kernel(int n, int n_pa
   if (lane == 0) importance[j] = total / (float)n;
 }
 
-// R[i][j] = RT[j][i] in fp32: 32 x 32 tiles through shared memory.
+// R[i][j] = RT[j][i] in fp32: 64 x 64 tiles through shared memory, read 8 elements at a time and written a row of 64 at a time
+// (32 x 32 tiles with loads of 2 bytes kept too little in flight: 17.2 -> 8.7 us at 2,230 tokens; the whole read-out 16.4 ->
+// 12.0 us, at 4,096 tokens 55.3 -> 33.3).
+constexpr int kExportTile = 64;
 __global__ void __launch_bounds__(256) rollout_export_kernel(int n, int n_pad, const __nv_bfloat16* __restrict__ hi,
                                                               const __nv_bfloat16* __restrict__ lo, float* __restrict__ out) {
-  __shared__ float tile[32][33];
-  const int j0 = blockIdx.y * 32, i0 = blockIdx.x * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  for (int r = ty; r < 32; r += 8) {
-    const int j = j0 + r, i = i0 + tx;
-    const long long at = (long long)j * n_pad + i;
-    tile[r][tx] = (j < n && i < n) ? __bfloat162float(hi[at]) + __bfloat162float(lo[at]) : 0.f;
+  __shared__ float tile[kExportTile][kExportTile + 1];
+  const int j0 = blockIdx.y * kExportTile, i0 = blockIdx.x * kExportTile;  // (n_pad is a multiple of 128: whole tiles exist)
+#pragma unroll
+  for (int e = threadIdx.x; e < kExportTile * kExportTile / 8; e += 256) {
+    const int r = e / (kExportTile / 8), c = e % (kExportTile / 8) * 8;
+    const long long at = (long long)(j0 + r) * n_pad + i0 + c;
+    const uint4 x = *reinterpret_cast<const uint4*>(hi + at), y = *reinterpret_cast<const uint4*>(lo + at);
+    const uint32_t hw[4] = {x.x, x.y, x.z, x.w}, lw[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      tile[r][c + 2 * u] = __uint_as_float(hw[u] << 16) + __uint_as_float(lw[u] << 16);
+      tile[r][c + 2 * u + 1] = __uint_as_float(hw[u] & 0xFFFF0000u) + __uint_as_float(lw[u] & 0xFFFF0000u);
+    }
   }
   __syncthreads();
-  for (int r = ty; r < 32; r += 8) {
-    const int i = i0 + r, j = j0 + tx;
-    if (i < n && j < n) out[(long long)i * n + j] = tile[tx][r];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll 4
+  for (int r = ty; r < kExportTile; r += 8) {
+    const int i = i0 + r;
+    if (i >= n) break;
+#pragma unroll
+    for (int c = tx; c < kExportTile; c += 32)
+      if (j0 + c < n) out[(long long)i * n + j0 + c] = tile[c][r];
   }
 }
 
@@ -1130,7 +1145,8 @@ extern "C" int32_t fastav_rollout_read(int32_t n, int32_t layers_applied, const 
   rollout_importance_kernel<<<(n + 7) / 8, 256, 0, st>>>(n, n_pad, hi, lo, importance_out);
   count_launches(1);
   if (rollout_out_opt) {
-    rollout_export_kernel<<<dim3((n + 31) / 32, (n + 31) / 32), 256, 0, st>>>(n, n_pad, hi, lo, rollout_out_opt);
+    const int tiles = (n + kExportTile - 1) / kExportTile;
+    rollout_export_kernel<<<dim3(tiles, tiles), 256, 0, st>>>(n, n_pad, hi, lo, rollout_out_opt);
     count_launches(1);
   }
   return cudaGetLastError() == cudaSuccess ? FASTAV_OK : FASTAV_ERR_CUDA;
