@@ -147,7 +147,9 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   //      same words queue at one L2 slice: 2,500 cycles instead of 900) ----------------------------------------------------
   if (warp == 0) {
     const int32_t* word = lane < 2 ? cu_seqlens + b + lane : lane < 4 ? cu_qlens + b + lane - 2 : keep_counts + b;
-    const bool there = lane < 2 || (lane < 4 ? cu_qlens != nullptr : lane == 4 && selecting);
+    // finished scores need the scored rows only where those survive by flag; without it the array may say anything
+    const bool wants_rows = FRONT != kScores || (s.flags & FASTAV_PROTECT_QUERY_ROWS);
+    const bool there = lane < 2 || (lane < 4 ? wants_rows : lane == 4 && selecting);
     const int v = there ? chain_load(word) : 0;
     if (lane < 5) sh.index[lane] = v;
   }

@@ -1,0 +1,35 @@
+"""What the header promises of every call, checked where a size decides which kernel serves it."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2601_13143_b200 import fastav
+
+pytestmark = pytest.mark.gpu
+
+
+def select(lens, keeps, scores, protect=None, q_idx=None, cu_qlens=None, total_q=0, flags=0):
+    """fastav_select on host arrays: (keep_idx, cu_keep, status)."""
+    dev = lambda a, dt: None if a is None else torch.as_tensor(np.asarray(a), dtype=dt).cuda()
+    n, kept = sum(lens), sum(keeps)
+    params = fastav.make_params(batch=len(lens), total_tokens=n, max_seqlen=max(lens), total_q=total_q, max_qlen=total_q, total_keep=kept,
+                                max_keep=max(keeps), num_q_heads=4, num_kv_heads=2, head_dim=64, hidden=64, flags=flags)
+    ws = torch.empty(max(256, fastav.fastav_workspace_bytes(params)), dtype=torch.uint8, device="cuda")
+    idx = torch.full((kept + 1,), -7, dtype=torch.int32, device="cuda")
+    cu_keep, status = torch.empty(len(lens) + 1, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    fastav.fastav_select(params, dev(scores, torch.float32), dev(np.concatenate([[0], np.cumsum(lens)]), torch.int32), dev(keeps, torch.int32),
+                         dev(protect, torch.uint8), dev(q_idx, torch.int32), dev(cu_qlens, torch.int32), idx, cu_keep, ws, status)
+    torch.cuda.synchronize()
+    return idx.cpu().numpy()[:kept], cu_keep.cpu().numpy(), int(status)
+
+
+@pytest.mark.parametrize("longest", [2048, 2049])
+def test_select_reads_the_scored_rows_only_under_their_flag(longest):
+    """Without FASTAV_PROTECT_QUERY_ROWS the arrays may say anything, here rows that total_q = 0 denies."""
+    lens, keeps = [longest, 100], [700, 33]
+    scores = np.random.default_rng(longest).random(sum(lens)).astype(np.float32)
+    idx, cu_keep, status = select(lens, keeps, scores, q_idx=[5, 6, 7], cu_qlens=[0, 2, 3])
+    want_idx, want_cu = oracle.select(scores, np.concatenate([[0], np.cumsum(lens)]), np.asarray(keeps))
+    assert status == 0
+    assert np.array_equal(idx, want_idx) and np.array_equal(cu_keep, want_cu)
