@@ -408,7 +408,12 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
     cu_keep[b + 1] = base + k;
     if (b == 0) cu_keep[0] = 0;
   }
-  if (k == 0) return;  // uniform for the cluster
+  if (k == 0) {  // nothing is kept, protected or not (uniform for the cluster)
+    if (c == 0 && device_status)
+      for (int j = tid; j < n; j += kThreads)
+        if (sh.keys[j] == kProtectedKey) atomicOr(device_status, FASTAV_DEV_PROTECT_OVERFLOW);
+    return;
+  }
   const int mine = max(0, min(kPer, n - kPer * tid));
   unsigned x[kPer];
 #pragma unroll

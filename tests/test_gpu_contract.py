@@ -33,3 +33,20 @@ def test_select_reads_the_scored_rows_only_under_their_flag(longest):
     want_idx, want_cu = oracle.select(scores, np.concatenate([[0], np.cumsum(lens)]), np.asarray(keeps))
     assert status == 0
     assert np.array_equal(idx, want_idx) and np.array_equal(cu_keep, want_cu)
+
+
+@pytest.mark.parametrize("longest", [2048, 2049])
+@pytest.mark.parametrize("keep", [0, 1, 2, 3])
+@pytest.mark.parametrize("by_rows", [False, True])
+def test_more_protected_tokens_than_are_kept_is_reported(longest, keep, by_rows):
+    """Two protected tokens in the first sequence: the bit is set exactly when fewer are kept, none included."""
+    lens, keeps = [longest, 64], [keep, 10]
+    scores = np.random.default_rng(7).random(sum(lens)).astype(np.float32)
+    protect = np.zeros(sum(lens), dtype=np.uint8)
+    rows = dict(q_idx=[40, longest - 1], cu_qlens=[0, 2, 2], total_q=2, flags=fastav.FASTAV_PROTECT_QUERY_ROWS)
+    if not by_rows:
+        protect[[40, longest - 1]] = 1
+        rows = {}
+    idx, cu_keep, status = select(lens, keeps, scores, protect, **rows)
+    assert status == (fastav.FASTAV_DEV_PROTECT_OVERFLOW if keep < 2 else 0)
+    assert cu_keep.tolist() == [0, keep, keep + 10] and {40, longest - 1} & set(idx[:keep]) == ({40, longest - 1} if keep >= 2 else {40} if keep else set())
