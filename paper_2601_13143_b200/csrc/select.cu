@@ -422,15 +422,24 @@ __global__ void __launch_bounds__(kThreads) mask_emit_kernel(Shapes s, const uin
   const int tok0 = seq.first, n = seq.count;
   if (tid == 0 && seq.bad && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
   if (tid == 0) base_sh = 0;
+  int cut = 0;  // a span before this one was cut down
+  if (!counts)
+    for (int i = tid; i < b; i += kThreads) cut |= checked_span(cu_seqlens, i, s.total_tokens, s.total_tokens).bad;
+  const int start = b > 0 ? chain_load(cu_seqlens) : tok0;
   pdl_wait();
   pdl_acquire(keep_mask);
   pdl_acquire(counts);
-  __syncthreads();
+  cut = __syncthreads_or(cut);
   int part = 0;
   if (counts) {
     for (int i = tid; i < b; i += kThreads) part += chain_load(counts + i);
+  } else if (!cut) {
+    part = count_nonzero(keep_mask + start, tok0 - start, tid);  // the sequences before this one, one after the other
   } else {
-    part = count_nonzero(keep_mask, tok0, tid);  // the sequences before this one lie before it in the packed batch
+    for (int i = 0; i < b; ++i) {
+      const Span before = checked_span(cu_seqlens, i, s.total_tokens, s.total_tokens);
+      part += count_nonzero(keep_mask + before.first, before.count, tid);
+    }
   }
   part = __reduce_add_sync(0xFFFFFFFFu, part);
   if (lane == 0 && part) atomicAdd(&base_sh, part);

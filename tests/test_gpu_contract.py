@@ -50,3 +50,36 @@ def test_more_protected_tokens_than_are_kept_is_reported(longest, keep, by_rows)
     idx, cu_keep, status = select(lens, keeps, scores, protect, **rows)
     assert status == (fastav.FASTAV_DEV_PROTECT_OVERFLOW if keep < 2 else 0)
     assert cu_keep.tolist() == [0, keep, keep + 10] and {40, longest - 1} & set(idx[:keep]) == ({40, longest - 1} if keep >= 2 else {40} if keep else set())
+
+
+def mask_call(mask, cu, total_keep):
+    params = fastav.make_params(batch=len(cu) - 1, total_tokens=len(mask), max_seqlen=len(mask), total_q=0, max_qlen=0, total_keep=total_keep,
+                                max_keep=total_keep, num_q_heads=4, num_kv_heads=2, head_dim=64, hidden=64)
+    idx = torch.full((total_keep,), -7, dtype=torch.int32, device="cuda")
+    cu_keep, status = torch.empty(len(cu), dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(max(256, 4 * len(cu) + 256), dtype=torch.uint8, device="cuda")
+    fastav.fastav_select_mask(params, torch.as_tensor(mask).cuda(), torch.as_tensor(np.asarray(cu), dtype=torch.int32).cuda(), idx, cu_keep, ws, status)
+    torch.cuda.synchronize()
+    return idx.cpu().numpy(), cu_keep.cpu().numpy(), int(status)
+
+
+@pytest.mark.parametrize("total", [5000, (1 << 18) + 77])
+def test_mask_counts_the_tokens_of_the_sequences_only(total):
+    """Marked tokens before the first sequence belong to none."""
+    mask = (np.random.default_rng(total).random(total) < 0.5).astype(np.uint8)
+    mask[:900] = 1
+    cu = np.array([900, 900, 1700, total - 3], dtype=np.int32)
+    want_idx, want_cu = oracle.select_mask(mask, cu)
+    idx, cu_keep, status = mask_call(mask, cu, int(want_cu[-1]))
+    assert status == 0 and np.array_equal(cu_keep, want_cu) and np.array_equal(idx, want_idx)
+
+
+@pytest.mark.parametrize("total", [5000, (1 << 18) + 77])
+def test_mask_cuts_impossible_spans_down(total):
+    """Bounds beyond the batch are cut down and reported; the survivors' prefix sums never fall back."""
+    mask = np.ones(total, dtype=np.uint8)
+    cu = [0, 100, total + 50, total + 60, 40, 300]  # 100 tokens; the rest of the batch; none; none (backwards); 260 tokens
+    idx, cu_keep, status = mask_call(mask, cu, total)
+    assert status == fastav.FASTAV_DEV_SHAPE_MISMATCH | fastav.FASTAV_DEV_K_CLAMPED
+    assert cu_keep.tolist() == [0, 100, total, total, total, total]
+    assert np.array_equal(idx, np.concatenate([np.arange(100), np.arange(total - 100)]))
