@@ -314,6 +314,8 @@ int32_t fastav_selftest_bounded_wait(int32_t limit_ms, int32_t* device_status, v
  *                          params, post-RoPE as the layer's attention uses them), applies Eq. 2 and multiplies
  *                          it onto R from the left (Eq. 3).  `layer_index` counts the layers applied so far
  *                          (0 for the first call after begin); it selects which copy of the state is read.
+ *                          Under FASTAV_CAUSAL R is taken to be lower triangular: no layer before may have
+ *                          been applied without the flag.
  *                          lse_opt: NULL, or [n, Hq] fp32 natural-log row sums exp as an attention kernel
  *                          returns them for this layer (then the statistics pass is skipped).
  *                          map_out_opt: NULL, or [n, n] fp32 row-major, receives A^l itself (the "raw

@@ -13,8 +13,8 @@
 // Layout.  R is kept TRANSPOSED, RT[j][i] = R[i][j], row-major with the rows padded to n_pad = ceil(n / 128) *
 // 128: then RT_new = RT_old * A~^T has both operands K-major (RT_old rows as the M side, A~ rows as the N
 // side), which is what TMA tiles with the 128-byte swizzle feed to tcgen05.mma without any transpose.  Under
-// the causal mask RT is upper and A~ lower triangular: tiles above the diagonal are written as zeros and the
-// K loop of tile (m, n) only covers the blocks m..n.
+// the causal mask RT is upper and A~ lower triangular: RT's tiles below the diagonal stay the zeros that begin
+// wrote, A~'s above it are neither written nor read, and the K loop of tile (m, n) only covers the blocks m..n.
 //
 // Sharing out the work.  At the paper's prompt size a layer is 171 visible 128 x 128 tiles on 148 SMs, so one block per tile
 // and head, or per tile, leaves much of the chip idle in a second round, and the longest K loop of the triangular product
@@ -650,7 +650,7 @@ struct GemmUnit {
 __global__ void __launch_bounds__(kThreads, 1)
 rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_constant__ CUtensorMap rt_lo_map,
                     const __grid_constant__ CUtensorMap a_hi_map, const __grid_constant__ CUtensorMap a_lo_map, int n_pad,
-                    int causal, int share, int units, int grid, __nv_bfloat16* __restrict__ out_hi, __nv_bfloat16* __restrict__ out_lo,
+                    int causal, int share, int units, __nv_bfloat16* __restrict__ out_hi, __nv_bfloat16* __restrict__ out_lo,
                     float* partials, int* counters, int32_t* device_status, ChainHead chain_head) {
   constexpr int kStages = kGemmStages, kStageBytes = kGemmStageBytes;
   extern __shared__ unsigned char smem_raw[];
@@ -659,20 +659,7 @@ rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_
   PipeControl& ctl = *reinterpret_cast<PipeControl*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + kStages * kStageBytes + kGemmStageOut);
   volatile int* abort = &ctl.abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int blocks = n_pad / kTile;
-
-  if ((int)blockIdx.x >= grid) {  // the first causal layer: nothing but zeros below the diagonal (later layers leave them)
-    pdl_wait();
-    const int t = blockIdx.x - grid;  // (mb, nb) with mb > nb
-    const int mb = triangular_root(t) + 1, nb = t - (mb - 1) * mb / 2;
-    for (int i = threadIdx.x; i < kTile * (kTile / 8); i += kThreads) {
-      const int r = i / (kTile / 8), c = (i % (kTile / 8)) * 8;
-      const long long at = (long long)(mb * kTile + r) * n_pad + nb * kTile + c;
-      *reinterpret_cast<uint4*>(out_hi + at) = make_uint4(0, 0, 0, 0);
-      *reinterpret_cast<uint4*>(out_lo + at) = make_uint4(0, 0, 0, 0);
-    }
-    return;
-  }
+  const int blocks = n_pad / kTile, grid = gridDim.x;
   auto unit_of = [&](int round) { return (round & 1) ? (round + 1) * grid - 1 - (int)blockIdx.x : round * grid + (int)blockIdx.x; };
 
   pipe_setup(ctl, kStages, warp, &rt_hi_map, &a_hi_map);
@@ -804,8 +791,10 @@ rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_
 }
 
 // ---- small kernels ----------------------------------------------------------------------------------
-// RT <- I on the first n rows (the padding stays zero): 8 elements per thread.
-__global__ void rollout_identity_kernel(int n, int n_pad, __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
+// RT <- I on the first n rows (the padding stays zero): 8 elements per thread.  The other copy's tiles below the diagonal become
+// zeros: a causal layer writes none of them.
+__global__ void rollout_identity_kernel(int n, int n_pad, __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
+                                        __nv_bfloat16* __restrict__ other_hi, __nv_bfloat16* __restrict__ other_lo) {
   const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 8;
   if (i >= (long long)n_pad * n_pad) return;
   const int r = (int)(i / n_pad), c = (int)(i % n_pad);
@@ -814,6 +803,10 @@ __global__ void rollout_identity_kernel(int n, int n_pad, __nv_bfloat16* __restr
   for (int u = 0; u < 8; ++u) h[u] = __float2bfloat16_rn((r < n && c + u == r) ? 1.f : 0.f);
   *reinterpret_cast<uint4*>(hi + i) = *reinterpret_cast<const uint4*>(h);
   *reinterpret_cast<uint4*>(lo + i) = make_uint4(0, 0, 0, 0);
+  if (r / kTile > c / kTile) {
+    *reinterpret_cast<uint4*>(other_hi + i) = make_uint4(0, 0, 0, 0);
+    *reinterpret_cast<uint4*>(other_lo + i) = make_uint4(0, 0, 0, 0);
+  }
 }
 
 // importance[j] = (1 / n) sum_i R[i][j] = mean of row j of RT: one warp per row, a fixed summation order.
@@ -1072,7 +1065,7 @@ extern "C" int32_t fastav_rollout_begin(int32_t n, void* state, size_t state_byt
   const int n_pad = pad_of(n);
   const long long threads = (long long)n_pad * n_pad / 8;
   rollout_identity_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-      n, n_pad, state_plane(state, n, 0, 0), state_plane(state, n, 0, 1));
+      n, n_pad, state_plane(state, n, 0, 0), state_plane(state, n, 0, 1), state_plane(state, n, 1, 0), state_plane(state, n, 1, 1));
   count_launches(1);
   return cudaGetLastError() == cudaSuccess ? FASTAV_OK : FASTAV_ERR_CUDA;
 }
@@ -1123,9 +1116,8 @@ extern "C" int32_t fastav_rollout_layer(const fastav_params* p, const void* q, c
   int units, cut;
   gemm_units(blocks, causal, share, &units, &cut);
   const int grid = units < kNumSMs ? units : kNumSMs;
-  const int zeros = causal && layer_index == 0 ? (int)hidden_tiles(blocks) : 0;
-  e = launch_chained(rollout_gemm_kernel, dim3(grid + zeros), dim3(kThreads), gemm_smem, st, rt_hi_map, rt_lo_map, a_hi_map, a_lo_map, n_pad,
-                     causal ? 1 : 0, share, units, grid, state_plane(state, n, dst, 0), state_plane(state, n, dst, 1),
+  e = launch_chained(rollout_gemm_kernel, dim3(grid), dim3(kThreads), gemm_smem, st, rt_hi_map, rt_lo_map, a_hi_map, a_lo_map, n_pad,
+                     causal ? 1 : 0, share, units, state_plane(state, n, dst, 0), state_plane(state, n, dst, 1),
                      reinterpret_cast<float*>(ws + w.partials), reinterpret_cast<int*>(ws + w.counters), device_status, ChainHead{});
   count_launches(1);
   return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? FASTAV_OK : FASTAV_ERR_CUDA;

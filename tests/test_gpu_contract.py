@@ -83,3 +83,25 @@ def test_mask_cuts_impossible_spans_down(total):
     assert status == fastav.FASTAV_DEV_SHAPE_MISMATCH | fastav.FASTAV_DEV_K_CLAMPED
     assert cu_keep.tolist() == [0, 100, total, total, total, total]
     assert np.array_equal(idx, np.concatenate([np.arange(100), np.arange(total - 100)]))
+
+
+@pytest.mark.parametrize("first", [2, 6])
+def test_a_rollout_may_start_at_any_even_layer_number(first):
+    """`layer_index` chooses which copy of the state is read; nothing else depends on where the
+    count starts (begin leaves the identity where an even layer reads)."""
+    from test_gpu_rollout import _layers, _params
+
+    n, hq, hkv, d, layers = 300, 4, 2, 64, 3
+    qk = [(q.cuda(), k.cuda()) for q, k in _layers(3, n, hq, hkv, d, layers)]
+    p = _params(n, hq, hkv, d, *qk[0], d**-0.5, True)
+    ws = torch.empty(fastav.fastav_rollout_workspace_bytes(p), dtype=torch.uint8, device="cuda")
+    got = []
+    for start in (0, first):
+        state = torch.full((fastav.fastav_rollout_state_bytes(n),), 255, dtype=torch.uint8, device="cuda")
+        fastav.fastav_rollout_begin(n, state)
+        for i, (q, k) in enumerate(qk):
+            fastav.fastav_rollout_layer(p, q, k, 0.5, start + i, state, ws)
+        imp, r = torch.empty(n, device="cuda"), torch.empty(n, n, device="cuda")
+        fastav.fastav_rollout_read(n, start + layers, state, imp, r)
+        got.append((imp, r))
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
