@@ -375,70 +375,86 @@ cudaError_t launch_select(const Shapes& s, const Workspace& w, const float* scor
 // ---- keep set given as a mask (the paper's positional global rule) ---------------------------------
 namespace {
 
-// Non-zero bytes of mask[0, count), per thread; 16 bytes at a time between the ends.
+// Non-zero bytes of mask[0, count), per thread of THREADS; 16 bytes at a time between the ends.
+template <int THREADS>
 __device__ __forceinline__ int count_nonzero(const uint8_t* mask, int count, int tid) {
   const int head = min(count, (int)(-reinterpret_cast<uintptr_t>(mask) & 15u)), quads = (count - head) / 16;
   int c = 0;
-  for (int j = tid; j < head; j += kThreads) c += mask[j] != 0;
+  for (int j = tid; j < head; j += THREADS) c += mask[j] != 0;
   const uint4* q = reinterpret_cast<const uint4*>(mask + head);
-  for (int j = tid; j < quads; j += kThreads) {
+  for (int j = tid; j < quads; j += THREADS) {
     const uint4 v = q[j];
     const unsigned w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
     for (int i = 0; i < 4; ++i) c += __popc((((w[i] & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | w[i]) & 0x80808080u);
   }
-  for (int j = head + quads * 16 + tid; j < count; j += kThreads) c += mask[j] != 0;
+  for (int j = head + quads * 16 + tid; j < count; j += THREADS) c += mask[j] != 0;
   return c;
 }
 
-// counts[b] = number of kept tokens of sequence b (large batches only; see mask_emit_kernel).
-__global__ void __launch_bounds__(kThreads) mask_count_kernel(Shapes s, const uint8_t* __restrict__ keep_mask,
+// counts[b] = number of kept tokens of sequence b.
+constexpr int kCountThreads = 256;
+__global__ void __launch_bounds__(kCountThreads) mask_count_kernel(Shapes s, const uint8_t* __restrict__ keep_mask,
                                                               const int32_t* __restrict__ cu_seqlens, int32_t* __restrict__ counts) {
   __shared__ int total;
   chain_enter(s, cu_seqlens);
   if (threadIdx.x == 0) total = 0;
   pdl_wait();
   pdl_acquire(keep_mask);
+  pdl_acquire(cu_seqlens);
   const int b = blockIdx.x;
-  const Span seq = checked_span(cu_seqlens, b, s.total_tokens, s.total_tokens);
+  const Span seq = checked_span<true>(cu_seqlens, b, s.total_tokens, s.total_tokens);
   __syncthreads();
-  const int c = __reduce_add_sync(0xFFFFFFFFu, count_nonzero(keep_mask + seq.first, seq.count, threadIdx.x));
+  const int c = __reduce_add_sync(0xFFFFFFFFu, count_nonzero<kCountThreads>(keep_mask + seq.first, seq.count, threadIdx.x));
   if ((threadIdx.x & 31) == 0 && c) atomicAdd(&total, c);
   __syncthreads();
   if (threadIdx.x == 0) counts[b] = total;
 }
 
 // Survivors of sequence b in ascending order, after those of the sequences before it: their number is read from `counts`, or,
-// without it, counted here from the mask itself (one kernel less).
-__global__ void __launch_bounds__(kThreads) mask_emit_kernel(Shapes s, const uint8_t* __restrict__ keep_mask,
+// COUNT_HERE, counted from the mask itself (one kernel less).  A large batch needs two blocks per SM (256 x 512 tokens: 7.8 us
+// with one) and the bounds through L1 (7.2 us without, 5.2 with).
+template <bool COUNT_HERE>
+__global__ void __launch_bounds__(kThreads, COUNT_HERE ? 1 : 2) mask_emit_kernel(Shapes s, const uint8_t* __restrict__ keep_mask,
                                                              const int32_t* __restrict__ cu_seqlens,
                                                              const int32_t* __restrict__ counts, int32_t* __restrict__ keep_idx,
                                                              int32_t* __restrict__ cu_keep, int32_t* device_status) {
   __shared__ unsigned warp_a[kWarps];
-  __shared__ int base_sh, mine_sh;
+  __shared__ int base_sh, mine_sh, start_sh;
   chain_enter(s, cu_seqlens);
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const Span seq = checked_span(cu_seqlens, b, s.total_tokens, s.total_tokens);
+  if (!COUNT_HERE) {  // a large batch: through L1, after the wait (see checked_span)
+    pdl_wait();
+    pdl_acquire(cu_seqlens);
+  }
+  // this sequence's bounds, and a predecessor's (one memory latency for both)
+  const bool looks = COUNT_HERE && tid < b;
+  const int first = COUNT_HERE ? chain_load(cu_seqlens + b) : chain_load_cached(cu_seqlens + b);
+  const int next = COUNT_HERE ? chain_load(cu_seqlens + b + 1) : chain_load_cached(cu_seqlens + b + 1);
+  const int other = looks ? chain_load(cu_seqlens + tid) : 0, other_next = looks ? chain_load(cu_seqlens + tid + 1) : 0;
+  const Span seq = checked_words(first, next, s.total_tokens, s.total_tokens);
   const int tok0 = seq.first, n = seq.count;
+  if (tid == 0) {
+    base_sh = 0;
+    start_sh = b > 0 ? other : tok0;
+  }
+  int cut = checked_words(other, other_next, s.total_tokens, s.total_tokens).bad;  // a span before this one was cut down
+  if (COUNT_HERE)
+    for (int i = tid + kThreads; i < b; i += kThreads) cut |= checked_span(cu_seqlens, i, s.total_tokens, s.total_tokens).bad;
   if (tid == 0 && seq.bad && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
-  if (tid == 0) base_sh = 0;
-  int cut = 0;  // a span before this one was cut down
-  if (!counts)
-    for (int i = tid; i < b; i += kThreads) cut |= checked_span(cu_seqlens, i, s.total_tokens, s.total_tokens).bad;
-  const int start = b > 0 ? chain_load(cu_seqlens) : tok0;
   pdl_wait();
   pdl_acquire(keep_mask);
   pdl_acquire(counts);
   cut = __syncthreads_or(cut);
   int part = 0;
-  if (counts) {
-    for (int i = tid; i < b; i += kThreads) part += chain_load(counts + i);
+  if (!COUNT_HERE) {
+    for (int i = tid; i < b; i += kThreads) part += chain_load_cached(counts + i);
   } else if (!cut) {
-    part = count_nonzero(keep_mask + start, tok0 - start, tid);  // the sequences before this one, one after the other
+    part = count_nonzero<kThreads>(keep_mask + start_sh, tok0 - start_sh, tid);  // the sequences before this one, one after the other
   } else {
     for (int i = 0; i < b; ++i) {
       const Span before = checked_span(cu_seqlens, i, s.total_tokens, s.total_tokens);
-      part += count_nonzero(keep_mask + before.first, before.count, tid);
+      part += count_nonzero<kThreads>(keep_mask + before.first, before.count, tid);
     }
   }
   part = __reduce_add_sync(0xFFFFFFFFu, part);
@@ -492,15 +508,17 @@ extern "C" int32_t fastav_select_mask(const fastav_params* p, const uint8_t* kee
   s.flags = p->flags;
   int32_t* counts = static_cast<int32_t*>(workspace);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // Each block counts the whole batch before its sequence; beyond a quarter of a million tokens a kernel that counts every
-  // sequence once is the shorter way.
-  constexpr int kCountHere = 1 << 18;
-  const bool count_first = s.total_tokens > kCountHere;
+  // One kernel in which each block counts all tokens before its sequence, or one that counts every sequence once and one that
+  // emits.  The first reads batch x tokens, the second costs a launch.  Kernel times, one / two: 32 x 1,000 tokens 3.8 / 4.2 us,
+  // 32 x 2,230 4.5 / 4.6, 128 x 1,024 5.3 / 5.3, 64 x 4,000 6.7 / 4.5; more sequences than SMs 200 x 100 5.7 / 4.8, 2,048 x
+  // 128 38 / 21.
+  constexpr int kCountHere = 1 << 17, kCountHereBatch = kNumSMs;
+  const bool count_first = s.total_tokens > kCountHere || s.batch > kCountHereBatch;
   cudaError_t e = cudaSuccess;
-  if (count_first) e = launch_chained(mask_count_kernel, dim3(s.batch), dim3(kThreads), 0, st, s, keep_mask, cu_seqlens, counts);
+  if (count_first) e = launch_chained(mask_count_kernel, dim3(s.batch), dim3(kCountThreads), 0, st, s, keep_mask, cu_seqlens, counts);
   if (e == cudaSuccess)
-    e = launch_chained(mask_emit_kernel, dim3(s.batch), dim3(kThreads), 0, st, s, keep_mask, cu_seqlens,
-                       count_first ? (const int32_t*)counts : (const int32_t*)nullptr, keep_idx_out, cu_keep_out, device_status);
+    e = launch_chained(count_first ? mask_emit_kernel<false> : mask_emit_kernel<true>, dim3(s.batch), dim3(kThreads), 0, st, s, keep_mask, cu_seqlens,
+                       (const int32_t*)counts, keep_idx_out, cu_keep_out, device_status);
   count_launches(count_first ? 2 : 1);
   return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? FASTAV_OK : FASTAV_ERR_CUDA;
 }

@@ -63,7 +63,7 @@ def mask_call(mask, cu, total_keep):
     return idx.cpu().numpy(), cu_keep.cpu().numpy(), int(status)
 
 
-@pytest.mark.parametrize("total", [5000, (1 << 18) + 77])
+@pytest.mark.parametrize("total", [5000, (1 << 17) + 77])
 def test_mask_counts_the_tokens_of_the_sequences_only(total):
     """Marked tokens before the first sequence belong to none."""
     mask = (np.random.default_rng(total).random(total) < 0.5).astype(np.uint8)
@@ -74,7 +74,7 @@ def test_mask_counts_the_tokens_of_the_sequences_only(total):
     assert status == 0 and np.array_equal(cu_keep, want_cu) and np.array_equal(idx, want_idx)
 
 
-@pytest.mark.parametrize("total", [5000, (1 << 18) + 77])
+@pytest.mark.parametrize("total", [5000, (1 << 17) + 77])
 def test_mask_cuts_impossible_spans_down(total):
     """Bounds beyond the batch are cut down and reported; the survivors' prefix sums never fall back."""
     mask = np.ones(total, dtype=np.uint8)

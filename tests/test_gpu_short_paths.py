@@ -56,7 +56,7 @@ def test_gather_by_either_kernel(n, keep, hid, rows):
     _check([n, n // 3], rows, 8, 2, 64, hid=hid, keep=keep)
 
 
-@pytest.mark.parametrize("total,batch", [(1, 1), (4095, 3), (4097, 1), ((1 << 18), 7), ((1 << 18) + 1, 7), (300_000, 513)])
+@pytest.mark.parametrize("total,batch", [(1, 1), (4095, 3), (4097, 1), ((1 << 18), 7), ((1 << 18) + 1, 7), ((1 << 17), 7), ((1 << 17) + 1, 7), (3000, 148), (3000, 149), (300_000, 513)])
 @pytest.mark.parametrize("offset", [0, 1])  # masks that are not 16-byte aligned
 def test_mask_emission(total, batch, offset):
     rng = np.random.default_rng(total + offset)
