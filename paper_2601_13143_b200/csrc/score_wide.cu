@@ -685,17 +685,19 @@ bool make_map(const void* ptr, int dim, int heads, long long rows, long long st,
 }
 
 // Persistent grid and key chunk: one block per SM; chunks sized so that a block gets about a dozen units (fine
-// enough to balance, and never more than its table holds).
+// enough to balance, and never more than its table holds).  Batches of so many sequences that no chunk does that take more
+// blocks.
 void plan_units(const Shapes& s, int rc_max, int* grid_out, int* chunk_tiles_out) {
   const long long tiles_upper = (long long)s.total_tokens / kTileKeys + s.batch;  // >= sum over sequences of ceil(n / 128)
   const long long tile_units = tiles_upper * s.hkv * rc_max;
-  const int grid = (int)(tile_units < kNumSMs ? tile_units : kNumSMs);
-  long long chunk_tiles = (tile_units + (long long)grid * kUnitsPerBlock - 1) / ((long long)grid * kUnitsPerBlock);
+  long long grid = tile_units < kNumSMs ? tile_units : kNumSMs;
+  long long chunk_tiles = (tile_units + grid * kUnitsPerBlock - 1) / (grid * kUnitsPerBlock);
   if (chunk_tiles < 1) chunk_tiles = 1;
   // units <= hkv * rc_max * (tokens / chunk + batch); keep the per-block share within the table
-  while (((long long)s.hkv * rc_max * (s.total_tokens / (chunk_tiles * kTileKeys) + s.batch) + grid - 1) / grid + 1 > kMaxUnits)
-    ++chunk_tiles;
-  *grid_out = grid;
+  auto units = [&] { return (long long)s.hkv * rc_max * (s.total_tokens / (chunk_tiles * kTileKeys) + s.batch); };
+  while ((units() + grid - 1) / grid + 1 > kMaxUnits && chunk_tiles * kTileKeys <= s.total_tokens) ++chunk_tiles;
+  if ((units() + grid - 1) / grid + 1 > kMaxUnits) grid = (units() + kMaxUnits - 2) / (kMaxUnits - 1);
+  *grid_out = (int)grid;
   *chunk_tiles_out = (int)chunk_tiles;
 }
 

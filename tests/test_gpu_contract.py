@@ -4,7 +4,8 @@ import pytest
 import torch
 
 import oracle
-from paper_2601_13143_b200 import fastav
+import parity
+from paper_2601_13143_b200 import fastav, workloads as W
 
 pytestmark = pytest.mark.gpu
 
@@ -105,3 +106,16 @@ def test_a_rollout_may_start_at_any_even_layer_number(first):
         fastav.fastav_rollout_read(n, start + layers, state, imp, r)
         got.append((imp, r))
     assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+
+
+@pytest.mark.parametrize("longest,rows", [(6, 5), (600, 1)])
+def test_batches_of_thousands(longest, rows):
+    """More (sequence, KV head) pairs than the tensor-core kernels' blocks, one per SM, can list: on its sweeps (forced, the one-pass
+    score would take them) and on its logits for few rows."""
+    lens = [longest] + [6] * 3599
+    p = W.random_problem(3, lens, [rows] * 3600, [2] * 3600, 4, 2, 64, 16)
+    buf = parity.to_device(p, extra_flags=fastav.FASTAV_SCORE_PATH_WIDE if rows > 4 else 0)
+    buf.prune()
+    torch.cuda.synchronize()
+    stats = parity.check_fused_against_oracle(p, buf, parity.oracle_prune(p))
+    assert stats["device_status"] & ~fastav.FASTAV_DEV_PROTECT_OVERFLOW == 0
