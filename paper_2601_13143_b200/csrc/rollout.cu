@@ -278,8 +278,8 @@ rollout_stats_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
       int loads = 0;
       for (int it = 0; it < count; ++it) {
         const int stage = it % kStages, buf = it % kBuffers;
-        if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort)) break;
-        if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_empty[buf]), ((it / kBuffers) & 1) ^ 1u, abort)) break;
+        if (!ptx::mbar_wait_warp(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort)) break;
+        if (!ptx::mbar_wait_warp(ptx::smem_u32(&ctl.tmem_empty[buf]), ((it / kBuffers) & 1) ^ 1u, abort)) break;
         ptx::tc_fence_after_sync();
         loads += it == 0 || x.jb == 0;
         const uint32_t k_tile = base + stage * kOperandBytes, q_tile = slots + ((loads - 1) & 1) * kOperandBytes;
@@ -309,7 +309,7 @@ rollout_stats_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
 #pragma unroll 1
     for (int it = 0; it < count; ++it, x.advance()) {
       const int buf = it % kBuffers;
-      if (ok) ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_full[buf]), (it / kBuffers) & 1, abort);
+      if (ok) ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.tmem_full[buf]), (it / kBuffers) & 1, abort);
       if (ok) {
         ptx::tc_fence_after_sync();
         uint32_t v[32];
@@ -466,8 +466,8 @@ rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       const uint32_t idesc = ptx::umma_idesc_bf16(kTile, 32 * strip.width);
       for (int it = 0; it < hq; ++it) {
         const int stage = it % kStages, buf = it % kMapBuffers;
-        if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort)) break;
-        if (!ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_empty[buf]), ((it / kMapBuffers) & 1) ^ 1u, abort)) break;
+        if (!ptx::mbar_wait_warp(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort)) break;
+        if (!ptx::mbar_wait_warp(ptx::smem_u32(&ctl.tmem_empty[buf]), ((it / kMapBuffers) & 1) ^ 1u, abort)) break;
         ptx::tc_fence_after_sync();
         const uint32_t q_tile = base + stage * kOperandBytes, k_tile = slots + ((it / group) & 1) * Cfg::kStripBytes;
         ptx::umma_bf16_steps<DIM / 16, kSubTileBytes, Cfg::kStripSubBytes>(tmem + buf * kStripCols, ptx::umma_desc_sw128(q_tile, 0),
@@ -530,7 +530,7 @@ rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         epilogue_sync();
       }
       if (!ok) continue;
-      ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_full[buf]), (it / kMapBuffers) & 1, abort);
+      ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.tmem_full[buf]), (it / kMapBuffers) & 1, abort);
       if (!ok) continue;
       ptx::tc_fence_after_sync();
       const float neg_lse2 = ctl.neg_lse[it % kHeadChunk][row_in];
@@ -694,10 +694,10 @@ rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_
       for (int round = 0; ok && unit_of(round) < units; ++round) {
         const GemmUnit unit(unit_of(round), blocks, causal != 0, share);
         const int buf = round & 1;
-        ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_empty[buf]), ((round >> 1) & 1) ^ 1u, abort);
+        ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.tmem_empty[buf]), ((round >> 1) & 1) ^ 1u, abort);
         for (int kb = unit.kb0; kb < unit.kb1 && ok; ++kb, ++it) {
           const int stage = it % kStages;
-          ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort);
+          ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort);
           if (!ok) break;
           ptx::tc_fence_after_sync();
           const uint32_t rt_hi = base + stage * kStageBytes, rt_lo = rt_hi + kSubTileBytes, a_hi = rt_hi + 2 * kSubTileBytes,
@@ -723,7 +723,7 @@ rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_
     for (int round = 0; unit_of(round) < units; ++round) {
       const int u = unit_of(round), buf = round & 1;
       const GemmUnit unit(u, blocks, causal != 0, share);
-      if (ok) ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_full[buf]), (round >> 1) & 1, abort);
+      if (ok) ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.tmem_full[buf]), (round >> 1) & 1, abort);
       float x[32];
       if (ok) {
         ptx::tc_fence_after_sync();

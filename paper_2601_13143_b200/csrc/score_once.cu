@@ -156,9 +156,9 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
     }
     __syncwarp();
   } else if (warp == 1) {
-    bool ok = mine <= 0 || ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.q_full), 0, abort);
+    bool ok = mine <= 0 || ptx::mbar_wait_warp(ptx::smem_u32(&ctl.q_full), 0, abort);
     for (int t = 0; t < mine && ok; ++t) {
-      ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.k_full[t]), 0, abort);
+      ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.k_full[t]), 0, abort);
       if (!ok) break;
       ptx::tc_fence_after_sync();
       ptx::umma_bf16_steps<DIM / 16, kSubTileBytes, kSubTileBytes>(tmem + t * kTile, ptx::umma_desc_sw128(q_smem, 0),
@@ -197,7 +197,7 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
     limit = ctl.limit[row_in];
     if (!lse_in) {
       for (int t = 0; t < mine; ++t) {
-        if (ok) ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.s_full[t]), 0, abort);
+        if (ok) ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.s_full[t]), 0, abort);
         if (!ok) break;
         ptx::tc_fence_after_sync();
         uint32_t v[32];
@@ -276,7 +276,7 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
     const float nl = ctl.neg_lse[row_in];
     const float2 nl2 = make_float2(nl, nl);
     for (int t = 0; t < mine; ++t) {
-      if (ok) ok = ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.s_full[t]), 0, abort);
+      if (ok) ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.s_full[t]), 0, abort);
       if (!ok) break;
       ptx::tc_fence_after_sync();
       uint32_t v[32];

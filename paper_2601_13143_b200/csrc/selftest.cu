@@ -15,8 +15,8 @@ __global__ void __launch_bounds__(64) bounded_wait_selftest_kernel(unsigned long
     ptx::fence_barrier_init();
   }
   __syncthreads();
-  // Phase 0 of `bar` never completes: every thread's wait has to give up (the first one to time out tells the rest).
-  const bool completed = ptx::mbar_wait_bounded(ptx::smem_u32(&bar), 0, &abort_flag, limit_ns);
+  // Phase 0 of `bar` never completes: every warp's wait has to give up (the first one to time out tells the rest).
+  const bool completed = ptx::mbar_wait_warp(ptx::smem_u32(&bar), 0, &abort_flag, limit_ns);
   if (!completed && threadIdx.x == 0 && device_status) atomicOr(device_status, FASTAV_DEV_WAIT_EXPIRED);
 }
 

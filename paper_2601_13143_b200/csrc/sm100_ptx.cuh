@@ -81,6 +81,13 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
   }
 }
 
+// The same for a whole converged warp, with one answer: a lane may see the phase complete just as another gives up, and what
+// follows a wait (elect.sync, tcgen05.ld, a warp's arrival) needs all lanes or none.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort, uint64_t limit_ns = kWaitLimitNs) {
+  if (__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) return true;
+  return __all_sync(0xFFFFFFFFu, mbar_wait_bounded(bar, parity, abort, limit_ns)) != 0;
+}
+
 // One arrival for a whole warp; orders the warp's earlier shared-memory accesses before the arrival.
 __device__ __forceinline__ void mbar_arrive_warp(uint32_t bar, int lane) {
   __syncwarp();
