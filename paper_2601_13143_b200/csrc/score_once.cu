@@ -16,7 +16,8 @@
 //
 // A key's sums do not depend on its position (every column goes through the same arithmetic and the same tree), and a
 // row's statistics are kept per key tile and folded in tile order, so that equal keys get bit-equal scores and a sequence's
-// scores do not depend on the cluster's size.  All waits are bounded.
+// scores do not depend on the cluster's size.  All waits are bounded but the cluster's own barriers, which end because its blocks
+// all run and every one of them arrives whatever happened before.
 #include <cuda.h>
 #include <limits.h>
 
@@ -36,7 +37,7 @@ constexpr int kTmemCols = 512;
 constexpr int kSubTileBytes = kTile * 128;
 
 struct alignas(16) Control {
-  uint64_t q_full, k_full[kBlockTiles], s_full[kBlockTiles];
+  uint64_t q_full, tmem_ready, k_full[kBlockTiles], s_full[kBlockTiles];
   uint32_t tmem_base;
   int abort;
   int index[4];
@@ -47,10 +48,18 @@ struct alignas(16) Control {
   float colsum[kBlockTiles][4][kTile];         // per key tile and 32-row quarter, the sums of every key
 };
 
+// Every block takes all of an SM's tensor memory, and the blocks of a cluster wait for one another: two clusters that met on
+// two SMs could each hold one and want the other.  So no SM may hold two blocks, and what rules that out is shared memory
+// (228 KB per SM, 1 KB of it per block not ours).
+constexpr size_t kOneBlockBytes = 114 * 1024;
+static_assert(2 * (kOneBlockBytes + 1024) > 228 * 1024, "two blocks would fit on an SM");
 template <int DIM>
 struct Layout {
   static constexpr int kOperandBytes = (DIM / 64) * kSubTileBytes;
-  static constexpr size_t bytes(int tiles) { return (size_t)(1 + tiles) * kOperandBytes + sizeof(Control) + 1024; }
+  static constexpr size_t bytes(int tiles) {
+    const size_t used = (size_t)(1 + tiles) * kOperandBytes + sizeof(Control) + 1024;
+    return used > kOneBlockBytes ? used : kOneBlockBytes;
+  }
 };
 
 __device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueThreads) : "memory"); }
@@ -93,6 +102,7 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
   if (warp == 1) {
     if (lane == 0) {
       ptx::mbar_init(ptx::smem_u32(&ctl.q_full), 1);
+      ptx::mbar_init(ptx::smem_u32(&ctl.tmem_ready), 1);
       for (int i = 0; i < kBlockTiles; ++i) {
         ptx::mbar_init(ptx::smem_u32(&ctl.k_full[i]), 1);
         ptx::mbar_init(ptx::smem_u32(&ctl.s_full[i]), 1);
@@ -102,9 +112,6 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
       ptx::prefetch_tensormap(&k_map);
       ptx::prefetch_tensormap(&q_map);
     }
-    __syncwarp();
-    ptx::tmem_alloc(ptx::smem_u32(&ctl.tmem_base), kTmemCols);
-    ptx::tmem_relinquish();
   } else if (warp >= 2) {
     // The query tile starts as zeros: rows no copy ever fills are then harmless operands.
     for (int i = threadIdx.x - 64; i < L::kOperandBytes / 16; i += kEpilogueThreads)
@@ -116,10 +123,7 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
     const int32_t* word = lane < 2 ? cu_seqlens + b + lane : cu_qlens + b + (lane & 1);
     if (lane < 4) ctl.index[lane] = chain_load(word);
   }
-  ptx::tc_fence_before_sync();
   __syncthreads();
-  ptx::tc_fence_after_sync();
-  const uint32_t tmem = ctl.tmem_base;
   const Span seq = checked_words(ctl.index[0], ctl.index[1], s.total_tokens, s.max_seqlen);
   const Span rows = checked_words(ctl.index[2], ctl.index[3], s.total_q, s.max_qlen);
   if (threadIdx.x == 0 && (seq.bad || rows.bad) && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
@@ -156,6 +160,16 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
     }
     __syncwarp();
   } else if (warp == 1) {
+    // Tensor memory is taken when all earlier work has ended, never before: a block of an earlier kernel that starts its
+    // successors first and allocates second would wait for this one's columns while this one waits for it.  The loads are on
+    // their way meanwhile.
+    pdl_wait();
+    __syncwarp();
+    ptx::tmem_alloc(ptx::smem_u32(&ctl.tmem_base), kTmemCols);
+    ptx::tmem_relinquish();
+    ptx::tc_fence_before_sync();
+    ptx::mbar_arrive_warp(ptx::smem_u32(&ctl.tmem_ready), lane);
+    const uint32_t tmem = ctl.tmem_base;
     bool ok = mine <= 0 || ptx::mbar_wait_warp(ptx::smem_u32(&ctl.q_full), 0, abort);
     for (int t = 0; t < mine && ok; ++t) {
       ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.k_full[t]), 0, abort);
@@ -170,7 +184,7 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
   }
   const int quarter = warp & 3, cg = (warp - 2) >> 2;  // epilogue: TMEM lanes 32 quarter .., columns 32 cg .. of every key tile
   const int row_in = quarter * 32 + lane, ethread = cg * kTile + row_in;
-  const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16) + cg * 32;
+  uint32_t lane_addr = 0;
   const float scale = s.scale_log2;
   const float2 sc = make_float2(scale, scale);
   bool ok = true;
@@ -195,6 +209,9 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
     }
     epilogue_sync();
     limit = ctl.limit[row_in];
+    ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.tmem_ready), 0, abort);
+    ptx::tc_fence_after_sync();
+    lane_addr = ctl.tmem_base + ((uint32_t)(quarter * 32) << 16) + cg * 32;
     if (!lse_in) {
       for (int t = 0; t < mine; ++t) {
         if (ok) ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.s_full[t]), 0, abort);
@@ -276,7 +293,7 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
     const float nl = ctl.neg_lse[row_in];
     const float2 nl2 = make_float2(nl, nl);
     for (int t = 0; t < mine; ++t) {
-      if (ok) ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.s_full[t]), 0, abort);
+      if (ok && lse_in) ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.s_full[t]), 0, abort);  // (else waited for above)
       if (!ok) break;
       ptx::tc_fence_after_sync();
       uint32_t v[32];
@@ -310,7 +327,7 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
   __syncthreads();
   if (warp == 1) {
     ptx::tc_fence_after_sync();
-    ptx::tmem_dealloc(tmem, kTmemCols);
+    ptx::tmem_dealloc(ctl.tmem_base, kTmemCols);
   }
   if (threadIdx.x == 0 && ctl.abort && device_status) atomicOr(device_status, FASTAV_DEV_WAIT_EXPIRED);
 }
