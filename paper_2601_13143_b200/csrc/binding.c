@@ -2,7 +2,8 @@
  *
  * A prune call takes about twenty pointers.  Through ctypes that is 6.5 us a call, more than a small call's kernels take to
  * launch; a tensor's data_ptr() called from C is 60 ns.  The library itself stays free of Python: the functions come in
- * as addresses of the ctypes handle that loaded it. */
+ * as addresses of the ctypes handle that loaded it.  As through ctypes, other threads run during a call: a launch waits while
+ * the stream's queue is full, and what empties the queue may be a Python callback. */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
@@ -60,8 +61,12 @@ static PyObject* prune(PyObject* self, PyObject* const* a, Py_ssize_t n) {
     return NULL;
   stream = address(a[22]);
   if (PyErr_Occurred()) return NULL;
-  return PyLong_FromLong(((__typeof__(&fastav_prune))f)(p, t[0], t[1], t[2], t[3], t[4], t[5], t[6], t[7], t[8], t[9], t[10], t[11], t[12],
-                                                        t[13], t[14], t[15], t[16], t[17], ws, bytes, status, stream));
+  int32_t rc;
+  Py_BEGIN_ALLOW_THREADS
+  rc = ((__typeof__(&fastav_prune))f)(p, t[0], t[1], t[2], t[3], t[4], t[5], t[6], t[7], t[8], t[9], t[10], t[11], t[12], t[13], t[14], t[15],
+                                      t[16], t[17], ws, bytes, status, stream);
+  Py_END_ALLOW_THREADS
+  return PyLong_FromLong(rc);
 }
 
 /* (function, params, keep_mask, cu_seqlens, keep_idx_out, cu_keep_out, workspace, device_status, stream) */
@@ -73,7 +78,11 @@ static PyObject* select_mask(PyObject* self, PyObject* const* a, Py_ssize_t n) {
     return NULL;
   stream = address(a[8]);
   if (PyErr_Occurred()) return NULL;
-  return PyLong_FromLong(((__typeof__(&fastav_select_mask))f)(p, t[0], t[1], t[2], t[3], ws, bytes, status, stream));
+  int32_t rc;
+  Py_BEGIN_ALLOW_THREADS
+  rc = ((__typeof__(&fastav_select_mask))f)(p, t[0], t[1], t[2], t[3], ws, bytes, status, stream);
+  Py_END_ALLOW_THREADS
+  return PyLong_FromLong(rc);
 }
 
 /* (function, params, keep_idx, cu_keep, cu_seqlens, hidden in/out, pos in/out, k in/out, v in/out, device_status, stream) */
@@ -82,8 +91,11 @@ static PyObject* compact(PyObject* self, PyObject* const* a, Py_ssize_t n) {
   if (expect("compact", n, 15) || ((f = address(a[0])) == NULL) || ((p = address(a[1])) == NULL) || pointers(a + 2, 12, t)) return NULL;
   stream = address(a[14]);
   if (PyErr_Occurred()) return NULL;
-  return PyLong_FromLong(
-      ((__typeof__(&fastav_compact))f)(p, t[0], t[1], t[2], t[3], t[4], t[5], t[6], t[7], t[8], t[9], t[10], t[11], stream));
+  int32_t rc;
+  Py_BEGIN_ALLOW_THREADS
+  rc = ((__typeof__(&fastav_compact))f)(p, t[0], t[1], t[2], t[3], t[4], t[5], t[6], t[7], t[8], t[9], t[10], t[11], stream);
+  Py_END_ALLOW_THREADS
+  return PyLong_FromLong(rc);
 }
 
 static PyMethodDef methods[] = {
