@@ -173,7 +173,7 @@ def _address(name: str) -> int:
 
 
 def _params(params: fastav_params) -> int:
-    if type(params) is not fastav_params:
+    if not isinstance(params, fastav_params):
         raise TypeError("expected a fastav_params")
     return ctypes.addressof(params)
 

@@ -38,3 +38,13 @@ def test_other_threads_run_during_a_call(native, name, count):
         other.join()
     assert end - start > 0.25
     assert sum(start + 0.05 < t < end - 0.05 for t in steps) >= 5
+
+
+def test_params_may_be_of_a_derived_type():
+    class Named(fastav.fastav_params):
+        pass
+
+    params = Named()
+    assert fastav._params(params) == ctypes.addressof(params)
+    with pytest.raises(TypeError):
+        fastav._params(None)
