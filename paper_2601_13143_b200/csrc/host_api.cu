@@ -8,10 +8,11 @@
 // copies of a few bytes each (2-4 us apiece) become part of two kernels.  2,048 tokens, half of them kept: 323 us
 // instead of 636.
 // Pageable buffers take the asynchronous copies.
-#include <atomic>
+#include <cuda.h>
 
 #include "common.cuh"
 #include "gather.cuh"
+#include "host_rules.h"
 
 namespace fastav {
 namespace {
@@ -161,20 +162,32 @@ struct Range {
   }
 };
 
-// The address under which the GPU reaches a page-locked host array, or nullptr.  Both ends are looked up: the array has
-// to lie inside one mapping.
+// The address under which the GPU reaches a page-locked host array, or nullptr.  The whole array has to lie inside the one
+// page-locked allocation or registration that its first byte belongs to: an array whose two ends are page-locked may
+// still have a gap between them that the GPU must not touch.
+using PointerAttributeFn = CUresult (*)(void*, CUpointer_attribute, CUdeviceptr);
+PointerAttributeFn pointer_attribute_fn() {
+  static void* entry = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult res;
+    if (cudaGetDriverEntryPoint("cuPointerGetAttribute", &p, cudaEnableDefault, &res) != cudaSuccess || res != cudaDriverEntryPointSuccess) p = nullptr;
+    return p;
+  }();
+  return reinterpret_cast<PointerAttributeFn>(entry);
+}
 void* mapped(const void* host, size_t bytes) {
-  cudaPointerAttributes first{}, last{};
+  cudaPointerAttributes first{};
   if (cudaPointerGetAttributes(&first, host) != cudaSuccess || first.type != cudaMemoryTypeHost || !first.devicePointer) {
     (void)cudaGetLastError();
     return nullptr;
   }
-  const unsigned char* end = static_cast<const unsigned char*>(host) + (bytes ? bytes - 1 : 0);
-  if (cudaPointerGetAttributes(&last, end) != cudaSuccess || last.type != cudaMemoryTypeHost ||
-      static_cast<unsigned char*>(last.devicePointer) - static_cast<unsigned char*>(first.devicePointer) != (ptrdiff_t)(bytes ? bytes - 1 : 0)) {
-    (void)cudaGetLastError();
+  const PointerAttributeFn attribute = pointer_attribute_fn();
+  const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(first.devicePointer);
+  CUdeviceptr start = 0;
+  size_t size = 0;
+  if (!attribute || attribute(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, at) != CUDA_SUCCESS ||
+      attribute(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, at) != CUDA_SUCCESS || !inside_range(at, bytes, start, size))
     return nullptr;
-  }
   return first.devicePointer;
 }
 
