@@ -240,7 +240,7 @@ int32_t fastav_prune_host(const fastav_params* params, const void* q, const int3
                       base + a.k_out, dev(a.v_out, v_out), base + a.workspace, a.workspace_bytes);
   if (rc != FASTAV_OK) return rc;
   {
-    // Every array page-locked (and the row arrays on 16-byte boundaries): the GPU fetches and delivers them itself.  With
+    // Every array page-locked (the row arrays on 16-byte boundaries, the positions on 4-byte ones): the GPU fetches and delivers them itself.  With
     // inputs that are also outputs the order matters, which only the copies below keep.
     const size_t hidden_row = (size_t)p.hidden * 2, q_bytes = R * p.num_q_heads * p.head_dim * 2;
     const Range ins[] = {{q, q_bytes}, {q_idx, R * 4}, {cu_qlens, (B + 1) * 4}, {k, N * kv_row}, {v, N * kv_row}, {cu_seqlens, (B + 1) * 4},
@@ -256,11 +256,12 @@ int32_t fastav_prune_host(const fastav_params* params, const void* q, const int3
       ok = p != nullptr;
       return p;
     };
-    auto at16 = [&](const void* host, size_t bytes) -> void* {
+    auto aligned_at = [&](const void* host, size_t bytes, uintptr_t alignment) -> void* {
       void* p = at(host, bytes);
-      ok = ok && (reinterpret_cast<uintptr_t>(p) & 15u) == 0;
+      ok = ok && (reinterpret_cast<uintptr_t>(p) & (alignment - 1)) == 0;
       return p;
     };
+    auto at16 = [&](const void* host, size_t bytes) { return aligned_at(host, bytes, 16); };
     CopyList up, down;
     RowStreams rows{};
     up.add(base + a.k, at16(k, N * kv_row), N * kv_row);
@@ -269,7 +270,7 @@ int32_t fastav_prune_host(const fastav_params* params, const void* q, const int3
     rows.hidden_out = static_cast<uint16_t*>(at16(hidden_out, K * hidden_row));
     rows.k_out = static_cast<uint16_t*>(at16(k_out, K * kv_row));
     rows.v_out = static_cast<uint16_t*>(at16(v_out, K * kv_row));
-    rows.pos_out = static_cast<int32_t*>(at(pos_out, K * 4));
+    rows.pos_out = static_cast<int32_t*>(aligned_at(pos_out, K * 4, 4));
     up.add(base + a.q, at(q, q_bytes), q_bytes);
     up.add(base + a.q_idx, at(q_idx, R * 4), R * 4);
     up.add(base + a.cu_qlens, at(cu_qlens, (B + 1) * 4), (B + 1) * 4);

@@ -56,3 +56,37 @@ def test_host_buffers_give_what_the_device_call_gives(how, lens, rows, keeps):
         if n == "keep_idx":
             want, out[n] = want[:kept], out[n][:kept]
         parity.assert_bits_equal(out[n], want, f"{how}: {n}")
+
+
+class At:
+    """A host array at any byte address, as far as fastav_prune_host looks at it."""
+    is_cuda = False
+
+    def __init__(self, address):
+        self.address = address
+
+    def data_ptr(self):
+        return self.address
+
+    def is_contiguous(self):
+        return True
+
+
+@pytest.mark.parametrize("shift", [1, 2, 3])
+def test_small_arrays_may_start_at_any_byte(shift):
+    """The small arrays are copied as bytes; positions, which a kernel would store as words, then take the copies too."""
+    p = W.random_problem(4, [300, 90], [1, 1], [120, 40], 8, 2, 64, 136)
+    buf = parity.to_device(p)
+    buf.prune()
+    torch.cuda.synchronize()
+    host = {n: getattr(p, n).pin_memory() for n in NAMES}
+    out = {n: torch.zeros_like(getattr(buf, n), device="cpu").pin_memory() for n in OUTS}
+    small = {n: torch.zeros(out[n].nbytes + 8, dtype=torch.uint8).pin_memory() for n in ("scores", "keep_idx", "cu_keep", "pos_out")}
+    arena = torch.empty(fastav.fastav_host_arena_bytes(buf.params), dtype=torch.uint8, device="cuda")
+    fastav.fastav_prune_host(buf.params, *(host[n] for n in NAMES[:7]), None, host["hidden"], host["pos"],
+                             *(At(small[n].data_ptr() + shift) if n in small else out[n] for n in OUTS), None, arena)
+    torch.cuda.synchronize()
+    for n in OUTS:
+        got = small[n][shift:shift + out[n].nbytes].clone().view(out[n].dtype) if n in small else out[n]
+        parity.assert_bits_equal(got, getattr(buf, n).cpu(), n)
+        assert n not in small or (small[n][:shift].eq(0).all() and small[n][shift + out[n].nbytes:].eq(0).all())
