@@ -521,6 +521,7 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
       a.rows.pos_out[base + first + i] = chain_load(a.rows.pos_in + tok0 + picked[(first + i) & (kBins - 1)]);
   const unsigned magic = 0xFFFFFFFFu / (unsigned)shape.n_chunks + 1u;  // e / n_chunks = umulhi(e, magic) while e * n_chunks < 2^32
   const int chunks = count * shape.n_chunks;
+  const bool by_magic = shape.n_chunks > 1 && (long long)chunks * shape.n_chunks < 1ll << 32;  // (always, if max_keep holds: see little)
   constexpr int kUnroll = 6;
 #pragma unroll 1
   for (int e0 = tid; e0 < chunks; e0 += kThreads * kUnroll) {
@@ -530,7 +531,7 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
     for (int u = 0; u < kUnroll; ++u) {
       const int e = e0 + u * kThreads;
       if (e < chunks) {
-        row[u] = shape.n_chunks == 1 ? e : (int)__umulhi((unsigned)e, magic);
+        row[u] = by_magic ? (int)__umulhi((unsigned)e, magic) : e / shape.n_chunks;
         chunk[u] = e - row[u] * shape.n_chunks;
         v[u] = load_stream(chunk_in(s, a.rows, shape, (long long)tok0 + picked[(first + row[u]) & (kBins - 1)], chunk[u]));
       }

@@ -119,3 +119,16 @@ def test_batches_of_thousands(longest, rows):
     torch.cuda.synchronize()
     stats = parity.check_fused_against_oracle(p, buf, parity.oracle_prune(p))
     assert stats["device_status"] & ~fastav.FASTAV_DEV_PROTECT_OVERFLOW == 0
+
+
+def test_rows_are_right_where_max_keep_says_too_little():
+    """2,048 survivors of 1,458 pieces each in one block, where max_keep promises one: rows are found by a division that is a
+    multiplication only for what max_keep allows."""
+    lens = [2048] + [1] * 74
+    p = W.random_problem(8, lens, [1] * 75, lens, 2, 1, 64, 11536)
+    buf = parity.to_device(p)
+    buf.params.max_keep = 1
+    buf.prune()
+    torch.cuda.synchronize()
+    for name, source in (("hidden_out", p.hidden), ("pos_out", p.pos), ("k_out", p.k), ("v_out", p.v)):
+        parity.assert_bits_equal(getattr(buf, name), source, name)
