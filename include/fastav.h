@@ -347,8 +347,9 @@ int32_t fastav_rollout_threshold(int32_t n, const float* importance, float thres
                                  uint8_t* keep_mask_out, int32_t* cut_out, void* stream);
 
 /*
- * Number of kernels this library has launched in this process so far (a diagnostic counter; the
- * only process-wide state the library has).  Benchmarks read it before and after a timed region.
+ * Number of kernels this library has launched in this process so far (a diagnostic counter).
+ * Benchmarks read it before and after a timed region.  Beside it the library keeps, process-wide, only
+ * what never changes a result: addresses it has looked up and the contexts it has set kernel attributes in.
  */
 int64_t fastav_kernel_launches(void);
 

@@ -5,6 +5,8 @@
 #include <cstdio>
 #include <cstring>
 
+#include <cuda.h>
+
 #include "common.cuh"
 #include "gather.cuh"
 
@@ -128,6 +130,19 @@ Shapes make_shapes(const fastav_params& p) {
   s.scale_log2 = scale * kLog2e;
   s.flags = p.flags;
   return s;
+}
+
+unsigned long long current_context() {
+  using GetIdFn = CUresult (*)(CUcontext, unsigned long long*);
+  static void* entry = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult res;
+    if (cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &res) != cudaSuccess || res != cudaDriverEntryPointSuccess) p = nullptr;
+    return p;
+  }();
+  unsigned long long id = 0;
+  if (!entry || reinterpret_cast<GetIdFn>(entry)(nullptr, &id) != CUDA_SUCCESS) return 0;
+  return id + 1;
 }
 
 void count_launches(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }

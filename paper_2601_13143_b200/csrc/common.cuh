@@ -152,6 +152,9 @@ void count_launches(int n);
 // The driver's tensor-map encoder (cuTensorMapEncodeTiled), looked up once through the runtime; nullptr if absent.
 void* tensor_map_encode_entry();
 
+// A number for the calling thread's current context, never given to another one in this process; 0 if there is none (yet).
+unsigned long long current_context();
+
 __host__ __device__ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // ---- programmatic dependent launch ----------------------------------------------------------------
@@ -251,17 +254,19 @@ __device__ __forceinline__ void chain_end_setup(const Head& head, P&... arrays) 
 inline thread_local bool g_chain_head = true;
 inline void chain_begin(uint32_t flags) { g_chain_head = (flags & FASTAV_CHAIN_CALLS) == 0; }
 
-// Function attributes live in the device's context: `set` runs on the first call for each device (per call site, that is
-// per kernel) and never again.
+// Function attributes live in a context: `set` runs on the first call in each (per call site, that is per kernel).  The eight
+// latest are remembered, by the number the driver gives every context once; where it gives none, `set` runs each time.
 template <typename F>
-cudaError_t once_per_device(F set) {
-  static std::atomic<unsigned long long> done{0};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 64 && ((done.load(std::memory_order_acquire) >> dev) & 1ull)) return cudaSuccess;
-  e = set();
-  if (e == cudaSuccess && dev < 64) done.fetch_or(1ull << dev, std::memory_order_release);
+cudaError_t once_per_context(F set) {
+  constexpr int kKept = 8;
+  static std::atomic<unsigned long long> done[kKept];
+  static std::atomic<unsigned> next{0};
+  const unsigned long long context = current_context();
+  if (context)
+    for (const auto& d : done)
+      if (d.load(std::memory_order_acquire) == context) return cudaSuccess;
+  const cudaError_t e = set();
+  if (e == cudaSuccess && context) done[next.fetch_add(1, std::memory_order_relaxed) % kKept].store(context, std::memory_order_release);
   return e;
 }
 

@@ -220,7 +220,7 @@ cudaError_t launch_compact(const Shapes& s, const int32_t* keep_idx, const int32
     int warps = kBulkSmemBudget / (kBulkStages * row_bytes);
     if (warps > kBulkMaxWarps) warps = kBulkMaxWarps;
     cudaError_t e =
-        once_per_device([] { return cudaFuncSetAttribute(compact_rows_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBulkSmemBudget); });
+        once_per_context([] { return cudaFuncSetAttribute(compact_rows_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBulkSmemBudget); });
     if (e != cudaSuccess) return e;
     int blocks = (s.total_keep + warps - 1) / warps;
     if (blocks > kNumSMs) blocks = kNumSMs;

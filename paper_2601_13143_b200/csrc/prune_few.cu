@@ -577,7 +577,7 @@ cudaError_t launch(const Shapes& s, FewArgs a, int blocks, size_t smem, const Ro
     a.rows = *rows;
   }
   const auto kernel = prune_few_kernel<FRONT, DIM>;
-  cudaError_t e = once_per_device([&] {
+  cudaError_t e = once_per_context([&] {
     cudaError_t f = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamic);
     if (f == cudaSuccess) f = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return f;

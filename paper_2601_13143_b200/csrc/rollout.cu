@@ -1015,7 +1015,7 @@ cudaError_t run_attention(const fastav_params& p, const CUtensorMap& q_map, cons
   a.device_status = device_status;
   const int blocks = a.n_pad / kTile;
   int* counters = reinterpret_cast<int*>(ws + w.counters);
-  cudaError_t e = once_per_device([&] {
+  cudaError_t e = once_per_context([&] {
     const cudaError_t f = cudaFuncSetAttribute(rollout_stats_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)StatSmem<DIM>::kBytes);
     return f == cudaSuccess ? cudaFuncSetAttribute(rollout_map_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MapSmem<DIM>::kBytes) : f;
   });
@@ -1109,7 +1109,7 @@ extern "C" int32_t fastav_rollout_layer(const fastav_params* p, const void* q, c
   if (e != cudaSuccess) return FASTAV_ERR_CUDA;
   constexpr size_t gemm_smem = kGemmStages * kGemmStageBytes + kGemmStageOut + sizeof(PipeControl) + 1024;
   static_assert(gemm_smem <= 227 * 1024);
-  e = once_per_device([] { return cudaFuncSetAttribute(rollout_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem); });
+  e = once_per_context([] { return cudaFuncSetAttribute(rollout_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem); });
   if (e != cudaSuccess) return FASTAV_ERR_CUDA;
   const bool causal = (p->flags & FASTAV_CAUSAL) != 0;
   const int blocks = n_pad / kTile, share = gemm_share(blocks, causal);

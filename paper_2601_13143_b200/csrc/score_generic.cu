@@ -276,7 +276,7 @@ cudaError_t run(const Shapes& s, const Workspace& w, const uint16_t* q, const in
   float* partial = reinterpret_cast<float*>(ws + w.partial_off);
   const size_t smem = sizeof(TileShared<DIM>);
   cudaError_t e;
-  e = once_per_device([&] {
+  e = once_per_context([&] {
     const cudaError_t f = cudaFuncSetAttribute(score_tile_stats_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     return f == cudaSuccess ? cudaFuncSetAttribute(score_tile_accumulate_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : f;
   });

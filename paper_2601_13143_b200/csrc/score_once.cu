@@ -336,7 +336,7 @@ template <int DIM>
 cudaError_t launch(const Shapes& s, const CUtensorMap& k_map, const CUtensorMap& q_map, const int32_t* q_idx, const int32_t* cu_qlens,
                    const int32_t* cu_seqlens, const float* lse_in, const OncePlan& plan, float* partial, int32_t* device_status, cudaStream_t stream) {
   const size_t smem = Layout<DIM>::bytes(plan.tiles_per_block);
-  cudaError_t e = once_per_device([&] {
+  cudaError_t e = once_per_context([&] {
     cudaError_t f = cudaFuncSetAttribute(score_once_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Layout<DIM>::bytes(kBlockTiles));
     if (f == cudaSuccess) f = cudaFuncSetAttribute(score_once_kernel<DIM>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return f;

@@ -709,7 +709,7 @@ cudaError_t run_logits(const Shapes& s, const CUtensorMap& k_map, const CUtensor
   plan_units(s, 1, &grid, &chunk_tiles);
   const int smem = Layout<DIM>::kTotal;
   cudaError_t e =
-      once_per_device([&] { return cudaFuncSetAttribute(score_wide_kernel<DIM, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
+      once_per_context([&] { return cudaFuncSetAttribute(score_wide_kernel<DIM, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
   if (e != cudaSuccess) return e;
   return launch_chained(score_wide_kernel<DIM, 0>, dim3(grid), dim3(kThreads), smem, stream, k_map, q_map, s, q_idx, cu_qlens,
                         cu_seqlens, chunk_tiles, 0, 1, wide_rows_per_chunk(s.group), (float2*)nullptr, (const float*)nullptr,
@@ -748,7 +748,7 @@ cudaError_t run(const Shapes& s, const Workspace& w, const CUtensorMap& k_map, c
   const int stat_chunks = 2 * ((s.max_seqlen + chunk_keys - 1) / chunk_keys);  // (max, sum) entries per (row, head)
   const int smem = Layout<DIM>::kTotal;
   cudaError_t e;
-  e = once_per_device([&] {
+  e = once_per_context([&] {
     const cudaError_t f = cudaFuncSetAttribute(score_wide_kernel<DIM, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     return f == cudaSuccess ? cudaFuncSetAttribute(score_wide_kernel<DIM, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) : f;
   });

@@ -333,7 +333,7 @@ cudaError_t launch_blocked(const Shapes& s, const float* scores, const int32_t* 
                            const uint8_t* protect, const int32_t* q_idx, const int32_t* cu_qlens, int32_t* keep_idx, int32_t* cu_keep,
                            int32_t* device_status, cudaStream_t stream) {
   const size_t smem = sizeof(BlockedShared) + ((size_t)s.max_seqlen + s.max_seqlen / 32 + 1) * sizeof(float);
-  cudaError_t e = once_per_device(
+  cudaError_t e = once_per_context(
       [] { return cudaFuncSetAttribute(select_topk_blocked_kernel<PER>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 1024); });
   if (e != cudaSuccess) return e;
   return launch_chained(select_topk_blocked_kernel<PER>, dim3(s.batch), dim3(kThreads), smem, stream, s, scores, cu_seqlens,
@@ -359,7 +359,7 @@ cudaError_t launch_select(const Shapes& s, const Workspace& w, const float* scor
     else if (s.max_seqlen <= kThreads * 16) e = launch_blocked<16>(s, scores, cu_seqlens, keep_counts, protect, q_idx, cu_qlens, keep_idx, cu_keep, device_status, stream);
     else e = launch_blocked<32>(s, scores, cu_seqlens, keep_counts, protect, q_idx, cu_qlens, keep_idx, cu_keep, device_status, stream);
   } else if (want <= kMaxDynamic) {
-    e = once_per_device([] { return cudaFuncSetAttribute(select_topk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamic); });
+    e = once_per_context([] { return cudaFuncSetAttribute(select_topk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamic); });
     if (e != cudaSuccess) return e;
     e = launch_chained(select_topk_kernel<true>, dim3(s.batch), dim3(kThreads), want, stream, s, scores, cu_seqlens,
                        keep_counts, protect, q_idx, cu_qlens, keep_idx, cu_keep, (unsigned*)nullptr, device_status);

@@ -1,4 +1,6 @@
 """What the header promises of every call, checked where a size decides which kernel serves it."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -132,3 +134,46 @@ def test_rows_are_right_where_max_keep_says_too_little():
     torch.cuda.synchronize()
     for name, source in (("hidden_out", p.hidden), ("pos_out", p.pos), ("k_out", p.k), ("v_out", p.v)):
         parity.assert_bits_equal(getattr(buf, name), source, name)
+
+
+@pytest.mark.parametrize("rows", [1, 9])
+def test_calls_work_in_a_second_context_of_the_same_device(rows):
+    """Kernel attributes belong to a context: what was set in torch's does not count in another one."""
+    buf = parity.to_device(W.random_problem(5, [700, 300], [rows, rows], [350, 100], 8, 2, 64, 128))
+    buf.prune()
+    torch.cuda.synchronize()
+    names = ("q", "q_idx", "cu_qlens", "k", "v", "cu_seqlens", None, "keep_counts", None, "hidden", "pos", "scores", "keep_idx", "cu_keep",
+             "hidden_out", "pos_out", "k_out", "v_out")
+    host = {n: getattr(buf, n).cpu().contiguous() for n in names if n}
+    cuda = ctypes.CDLL("libcuda.so.1")
+
+    def call(name, *args):
+        assert getattr(cuda, name)(*args) == 0, name
+
+    def allocated(size):
+        at = ctypes.c_uint64()
+        call("cuMemAlloc_v2", ctypes.byref(at), ctypes.c_size_t(size))
+        return at
+
+    before, context = ctypes.c_void_p(), ctypes.c_void_p()
+    call("cuCtxGetCurrent", ctypes.byref(before))
+    call("cuCtxCreate_v2", ctypes.byref(context), 0, torch.cuda.current_device())
+    try:
+        where = {n: allocated(t.nbytes) for n, t in host.items()}
+        for n, t in host.items():
+            call("cuMemcpyHtoD_v2", where[n], ctypes.c_void_p(t.data_ptr()), ctypes.c_size_t(t.nbytes))
+        outputs = names[names.index("scores"):]
+        for n in outputs:
+            call("cuMemsetD8_v2", where[n], ctypes.c_ubyte(0xEE), ctypes.c_size_t(host[n].nbytes))
+        workspace = allocated(buf.workspace.nbytes)
+        rc = fastav.library().fastav_prune(ctypes.byref(buf.params), *(ctypes.c_void_p(where[n].value) if n else None for n in names),
+                                           ctypes.c_void_p(workspace.value), buf.workspace.nbytes, None, None)
+        assert rc == 0, fastav.library().fastav_last_cuda_error()
+        call("cuCtxSynchronize")
+        for n in outputs:
+            got = torch.empty_like(host[n])
+            call("cuMemcpyDtoH_v2", ctypes.c_void_p(got.data_ptr()), where[n], ctypes.c_size_t(got.nbytes))
+            parity.assert_bits_equal(got, host[n], n)
+    finally:
+        call("cuCtxDestroy_v2", context)
+        call("cuCtxSetCurrent", before)
