@@ -129,6 +129,7 @@ Shapes make_shapes(const fastav_params& p) {
   const float scale = p.softmax_scale > 0.f ? p.softmax_scale : 1.0f / std::sqrt((float)p.head_dim);
   s.scale_log2 = scale * kLog2e;
   s.flags = p.flags;
+  s.cluster_limit = cluster_limit();
   return s;
 }
 

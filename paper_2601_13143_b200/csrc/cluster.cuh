@@ -2,16 +2,11 @@
 #pragma once
 
 #include "common.cuh"
+#include "host_rules.h"
 #include "select_keys.cuh"
 #include "sm100_ptx.cuh"
 
 namespace fastav {
-
-constexpr int kMaxCluster = 16;  // beyond the portable 8: allowed per kernel
-
-// Clusters of each size that run at once with one block per SM (cudaOccupancyMaxActiveClusters on a B200): a cluster's
-// blocks share a GPC, and the GPCs hold 16 to 20 SMs.  Sixteen clusters of eight take two rounds, 20 us instead of 10.
-constexpr int kAtOnce[kMaxCluster + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15, 15, 11, 7, 7, 7, 7, 7, 7};
 
 // ---- distributed shared memory ---------------------------------------------------------------------
 __device__ __forceinline__ uint32_t cluster_rank() {

@@ -22,6 +22,7 @@ struct Shapes {
   long long q_st, q_sh, k_st, k_sh, v_st, v_sh, ko_st, ko_sh, vo_st, vo_sh;
   float scale_log2;  // softmax scale * log2(e): logits are kept in base-2 units
   unsigned flags;
+  int cluster_limit; // most blocks of a cluster in the current context (host side)
   int head_wait;     // set at launch (launch_chained): this kernel opens a call and must wait before it reads anything
 };
 
@@ -109,6 +110,9 @@ cudaError_t launch_few(const Shapes& s, const void* q, const void* k, const floa
 cudaError_t launch_select_partials(const Shapes& s, const float* partial, const ScoreLeft& left, float* scores_out, const RowStreams* rows,
                                    const SelectArgs& t, cudaStream_t stream);
 cudaError_t launch_select_scores(const Shapes& s, const float* scores, const SelectArgs& t, cudaStream_t stream);
+
+// Most blocks of a cluster that the current context can place: 16, or the portable 8.
+int cluster_limit();
 
 // Many scored rows on short sequences: one pass over K (score_once.cu).
 struct OncePlan {

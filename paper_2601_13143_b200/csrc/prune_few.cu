@@ -23,6 +23,8 @@
 // scores: all sums have a fixed order.
 #include <math.h>
 
+#include <atomic>
+
 #include "cluster.cuh"
 #include "common.cuh"
 #include "gather.cuh"
@@ -551,23 +553,17 @@ size_t smem_keys(const Shapes& s, int blocks) {
 
 constexpr size_t kMaxDynamic = 220 * 1024;
 
-// Blocks per sequence: as many as have at least `slice` tokens each and still run at once (sixteen clusters of eight take two
-// rounds where sixteen of four take one).  From the keys every token more per block counts: 32 tokens, sixteen blocks against
-// eight, 1 x 512 tokens: 12.0 / 12.6 us, 1 x 2,048: 17.9 / 20.8; slices of 128 instead: 1 x 256 tokens 18.2 us instead of 12.2.
-// From sums or scores there is less to share and the exchange counts: with slices of 256 / 64 / 2,048 tokens the prune of 1 x
+// Tokens per block, at least (see cluster_blocks).  From the keys every token more per block counts: 32 tokens, sixteen blocks
+// against eight, 1 x 512 tokens: 12.0 / 12.6 us, 1 x 2,048: 17.9 / 20.8; slices of 128 instead: 1 x 256 tokens 18.2 us instead of
+// 12.2.  From sums or scores there is less to share and the exchange counts: with slices of 256 / 64 / 2,048 tokens the prune of 1 x
 // 2,048 tokens, 32 rows, takes 20.7 / 22.9 / 23.9 us, 4 x 2,048 36.3 / 37.7 / 39.2.
 constexpr int kKeySlice = 32, kScoreSlice = 256;
-int cluster_for(const Shapes& s, int slice) {
-  int blocks = kMaxCluster;
-  while (blocks > 1 && (s.batch > kAtOnce[blocks] || s.max_seqlen <= blocks / 2 * slice)) blocks /= 2;
-  return blocks;
-}
 int cluster_keys(const Shapes& s) {
-  int blocks = cluster_for(s, kKeySlice);
-  while (blocks < kMaxCluster && smem_keys(s, blocks) > kMaxDynamic) blocks *= 2;
+  int blocks = cluster_blocks(s.batch, s.max_seqlen, kKeySlice, s.cluster_limit);
+  while (blocks < s.cluster_limit && smem_keys(s, blocks) > kMaxDynamic) blocks *= 2;
   return blocks;
 }
-int cluster_select(const Shapes& s) { return cluster_for(s, kScoreSlice); }
+int cluster_select(const Shapes& s) { return cluster_blocks(s.batch, s.max_seqlen, kScoreSlice, s.cluster_limit); }
 
 template <Front FRONT, int DIM>
 cudaError_t launch(const Shapes& s, FewArgs a, int blocks, size_t smem, const RowStreams* rows, const SelectArgs& t, cudaStream_t stream) {
@@ -604,6 +600,40 @@ bool little(const Shapes& s, int blocks, int row_bytes) {
 }
 
 }  // namespace
+
+// Asked of the few-rows kernel with all the shared memory it may take (the one-pass score needs an SM per block too), once per
+// context: a device with fewer SMs per GPC, or a context that was given a part of one, may have no room for sixteen.
+int cluster_limit() {
+  static std::atomic<unsigned long long> known[8];  // context number x 2 + (sixteen can be placed)
+  static std::atomic<unsigned> next{0};
+  const unsigned long long context = current_context();
+  for (const auto& k : known) {
+    const unsigned long long v = k.load(std::memory_order_acquire);
+    if (context && v >> 1 == context) return v & 1 ? kMaxCluster : kPortableCluster;
+  }
+  const auto kernel = prune_few_kernel<kKeys, 128>;
+  int clusters = 0;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamic);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kMaxCluster);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kMaxDynamic;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = kMaxCluster;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    e = cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg);
+  }
+  if (e != cudaSuccess) (void)cudaGetLastError();
+  const bool sixteen = e == cudaSuccess && clusters > 0;
+  if (context && e == cudaSuccess)
+    known[next.fetch_add(1, std::memory_order_relaxed) % 8].store(context << 1 | (sixteen ? 1u : 0u), std::memory_order_release);
+  return sixteen ? kMaxCluster : kPortableCluster;
+}
 
 // Few scored rows, up to 2,048 tokens (kPer keys per thread).  More sequences than SMs take several rounds, one sequence per block:
 // that is still the better way up to 512 tokens (300 x 128: 145 us, 600 x 200: 407; with the scoring kernels of long sequences

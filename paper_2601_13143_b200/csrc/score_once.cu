@@ -374,7 +374,7 @@ bool once_plan(const Shapes& s, bool lse_given, OncePlan* plan) {
   long long least = LLONG_MAX;
   for (int per = 1; per <= kBlockTiles; ++per) {
     const int blocks = (tiles + per - 1) / per;
-    if (blocks > kMaxCluster) continue;
+    if (blocks > s.cluster_limit) continue;
     const long long rounds = (clusters + kAtOnce[blocks] - 1) / kAtOnce[blocks], cost = rounds * (24 + 15 * per);
     if (cost >= least) continue;
     least = cost;

@@ -12,6 +12,7 @@ SOURCE = """
 extern "C" int inside(unsigned long long at, unsigned long long bytes, unsigned long long start, unsigned long long size) {
   return fastav::inside_range(at, bytes, start, size);
 }
+extern "C" int blocks(int batch, int max_seqlen, int slice, int limit) { return fastav::cluster_blocks(batch, max_seqlen, slice, limit); }
 """
 
 
@@ -33,3 +34,12 @@ def test_an_array_is_inside_one_range_or_not(rules, at, bytes_, start, size, ins
     """Two registrations with a gap between them are two ranges: the first byte's range has to hold the last byte too."""
     u64 = ctypes.c_uint64
     assert rules.inside(u64(at), u64(bytes_), u64(start), u64(size)) == inside
+
+
+@pytest.mark.parametrize("batch,tokens,slice_,sixteen,eight", [
+    (1, 2048, 32, 16, 8), (1, 512, 32, 16, 8), (1, 257, 32, 16, 8), (1, 256, 32, 8, 8), (7, 2048, 32, 16, 8), (8, 2048, 32, 8, 8), (16, 2048, 32, 4, 4),
+    (1, 2048, 256, 8, 8), (75, 2048, 32, 1, 1), (149, 100, 32, 1, 1), (1, 0, 32, 1, 1),
+])
+def test_blocks_per_sequence_keep_within_what_can_be_placed(rules, batch, tokens, slice_, sixteen, eight):
+    assert rules.blocks(batch, tokens, slice_, 16) == sixteen
+    assert rules.blocks(batch, tokens, slice_, 8) == eight
