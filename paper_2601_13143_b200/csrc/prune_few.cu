@@ -594,9 +594,17 @@ cudaError_t launch_from(const Shapes& s, const FewArgs& a, const RowStreams* row
 // Survivors' rows are copied by the blocks that select them where that is little per block: it saves a launch (tiny prompt of
 // 512 tokens 10.3 us instead of 11.6), but the rows of one sequence then come through its own blocks only, and the compaction
 // kernel has the whole chip (chain of 13 stages from 744 tokens: 162 us with limits of 0 and 48 KB, 241 with 192 KB).
-constexpr int kGatherBytes = 48 << 10;
+// Survivors may all lie in one block's slice (early tokens are the ones attended to), so that has a limit too, a higher one
+// where many sequences keep the chip busy.  Survivors spread / in one slice / rows by the compaction, from the keys: 1 x 1,024
+// tokens of 1,536 bytes, 30 % kept (98 KB in one slice) 10.6 / 12.0 / 12.0 us, 1 x 2,048, 10 % (196 KB) 11.0 / 15.7 / 12.2, 16 x
+// 2,000, 5 % (154 KB) 16.3 / 19.6 / 18.6.  From partial sums the blocks are fewer and one sequence does not gain: 1 x 512 tokens of
+// 384 bytes, half kept 15.1 / 16.9 / 13.7; 8 x 1,000, 20 % 15.1 / 17.1 / 17.0, 16 x 2,000, 5 % 19.3 / 19.9 / 22.2, 256 x 128 of 640
+// bytes, half kept 54 instead of 84.
+constexpr int kGatherBytes = 48 << 10, kGatherBytesOneSlice = 96 << 10, kGatherBytesOneSliceBusy = 160 << 10;
 bool little(const Shapes& s, int blocks, int row_bytes) {
-  return row_bytes > 0 && (long long)((s.max_keep + blocks - 1) / blocks) * row_bytes <= kGatherBytes;
+  const int slice = slice_of(s, blocks);
+  const long long spread = (s.max_keep + blocks - 1) / blocks, one_slice = s.max_keep < slice ? s.max_keep : slice;
+  return row_bytes > 0 && spread * row_bytes <= kGatherBytes && one_slice * row_bytes <= (s.batch >= 16 ? kGatherBytesOneSliceBusy : kGatherBytesOneSlice);
 }
 
 }  // namespace
@@ -647,7 +655,7 @@ bool few_applies(const Shapes& s) {
 bool cluster_select_applies(const Shapes& s) { return s.max_seqlen <= kMaxTokens; }
 
 bool few_gathers(const Shapes& s, int row_bytes) { return little(s, cluster_keys(s), row_bytes); }
-bool cluster_select_gathers(const Shapes& s, int row_bytes) { return little(s, cluster_select(s), row_bytes); }
+bool cluster_select_gathers(const Shapes& s, int row_bytes) { return s.batch >= 8 && little(s, cluster_select(s), row_bytes); }
 
 cudaError_t launch_few(const Shapes& s, const void* q, const void* k, const float* lse_in, float* scores_out, bool do_select,
                        const RowStreams* rows, const SelectArgs& t, cudaStream_t stream) {

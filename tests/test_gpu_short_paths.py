@@ -75,3 +75,10 @@ def test_mask_emission(total, batch, offset):
     torch.cuda.synchronize()
     assert int(status) == 0 and cu_keep.cpu().tolist() == ref_cu.tolist()
     assert np.array_equal(idx.cpu().numpy(), np.concatenate([ref_idx, np.full(8, -7)]))
+
+
+# Who gathers also depends on how many sequences there are, and on what one block's slice of the tokens can hold.
+@pytest.mark.parametrize("batch,n,keep", [(7, 1000, 0.05), (8, 1000, 0.05), (8, 1000, 0.3), (15, 400, 0.3), (16, 400, 0.3), (150, 120, 0.5)])
+@pytest.mark.parametrize("rows", [1, 8])
+def test_gather_of_batches(batch, n, keep, rows):
+    _check([n] * batch, rows, 8, 2, 64, hid=64, keep=keep)
