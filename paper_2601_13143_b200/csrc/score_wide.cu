@@ -593,11 +593,22 @@ __global__ void __launch_bounds__(256) score_wide_merge_kernel(Shapes s, const i
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (w >= s.total_q * s.hq) return;
   const int row = w / s.hq;
-  int n = 0;  // length of the row's sequence, the last one that starts at or before it: the whole warp looks
-  for (int b0 = 0; b0 < s.batch; b0 += 32) {
-    const int b = min(b0 + lane, s.batch - 1);
+  // The row's sequence is the last one that starts at or before it.  The whole warp looks, 32 starts at a time: at evenly spaced
+  // ones until at most 32 sequences are left, then at those (1,024 sequences: two rounds; one after the other 32 of them made a
+  // score call of 1,024 x 128 tokens 169 us instead of 98).
+  int lo = 0, left = s.batch;
+  while (left > 32) {
+    const int step = (left + 31) / 32, at = lo + lane * step;
+    const unsigned not_after = __ballot_sync(0xFFFFFFFFu, lane * step < left && chain_load_cached(cu_qlens + at) <= row);
+    const int skip = not_after ? (31 - __clz(not_after)) * step : 0;
+    lo += skip;
+    left = min(step, left - skip);
+  }
+  int n = 0;
+  {
+    const int b = min(lo + lane, s.batch - 1);
     const int first = chain_load_cached(cu_qlens + b), count = seq_span<true>(s, cu_seqlens, b).count;
-    const unsigned not_after = __ballot_sync(0xFFFFFFFFu, b0 + lane < s.batch && first <= row);
+    const unsigned not_after = __ballot_sync(0xFFFFFFFFu, lane < left && first <= row);
     if (not_after) n = __shfl_sync(0xFFFFFFFFu, count, 31 - __clz(not_after));
   }
   const int chunks = 2 * ((n + chunk_keys - 1) / chunk_keys);  // one entry per 64-key half of every tile run

@@ -177,3 +177,16 @@ def test_calls_work_in_a_second_context_of_the_same_device(rows):
     finally:
         call("cuCtxDestroy_v2", context)
         call("cuCtxSetCurrent", before)
+
+
+@pytest.mark.parametrize("batch", [31, 32, 33, 64, 65, 1024, 1025, 1057])
+def test_statistics_find_their_sequence_in_any_batch(batch):
+    """The merge of the two sweeps' statistics looks a row's sequence up, 32 at a time; empty sequences and ones without rows among
+    them."""
+    lens = [(37 * i) % 23 + 6 if i % 7 else 0 for i in range(batch)]
+    p = W.random_problem(batch, lens, [0 if n == 0 or n % 5 == 0 else 5 for n in lens], [n // 2 for n in lens], 4, 2, 64, 16)
+    buf = parity.to_device(p, extra_flags=fastav.FASTAV_SCORE_PATH_WIDE)
+    buf.score()
+    torch.cuda.synchronize()
+    parity.assert_scores_close(buf.scores, parity.oracle_scores(p))
+    assert int(buf.device_status) == 0
