@@ -181,14 +181,17 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   // What the selection needs and nothing has needed so far.
   auto selection_inputs = [&] {
     if (!selecting) return;
-    if (b > 0 && warp == kWarps - 1) {  // output offset: the clamped keep counts of the sequences before this one
+    // output offset: the clamped keep counts of the sequences before this one, 32 per warp (up to 32 of them: the last warp)
+    const int w = kWarps - 1 - warp;
+    if (w * 32 < b) {
       int part = 0;
-      for (int i = lane; i < b; i += 32) {
+#pragma unroll 2
+      for (int i = w * 32 + lane; i < b; i += kThreads) {
         const int ni = seq_span(s, cu_seqlens, i).count, ki = chain_load(keep_counts + i);
         part += ki < 0 ? 0 : min(ki, ni);
       }
       part = __reduce_add_sync(0xFFFFFFFFu, part);
-      if (lane == 0) sh.base = part;
+      if (lane == 0 && part) atomicAdd(&sh.base, part);
     }
     if (protect)
       for (int j0 = warp * 32; j0 < m; j0 += kThreads) {  // a warp covers 32 tokens: one word
