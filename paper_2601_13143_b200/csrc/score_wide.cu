@@ -99,9 +99,10 @@ __device__ __forceinline__ int units_of_spans(const Shapes& s, const Span& seq, 
   return s.hkv * ((flat_rows + rows_per_chunk - 1) / rows_per_chunk) * ((n + chunk_keys - 1) / chunk_keys);
 }
 
+// (through L1: for batches beyond the table, whose kernels wait first)
 __device__ __forceinline__ int units_of_sequence(const Shapes& s, const int32_t* cu_seqlens, const int32_t* cu_qlens, int b,
                                                  int rows_per_chunk, int chunk_keys) {
-  return units_of_spans(s, seq_span(s, cu_seqlens, b), row_span(s, cu_qlens, b), rows_per_chunk, chunk_keys);
+  return units_of_spans(s, seq_span<true>(s, cu_seqlens, b), row_span<true>(s, cu_qlens, b), rows_per_chunk, chunk_keys);
 }
 
 // Block-wide sum of one int per thread (all threads get the result).
@@ -169,6 +170,9 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
     ctl.seq_first_unit[b] = my_excl;  // first unit of sequence b in the global order
     if (b == 0) ctl.seq_first_unit[kThreads] = total_units;
   } else {
+    pdl_wait();  // the bounds are read many times, one after the other below: after the wait, through L1
+    pdl_acquire(cu_seqlens);
+    pdl_acquire(cu_qlens);
     for (int b0 = 0; b0 < s.batch; b0 += kThreads) {
       const int b = b0 + threadIdx.x;
       total_units += block_sum(b < s.batch ? units_of_sequence(s, cu_seqlens, cu_qlens, b, rows_per_chunk, chunk_keys) : 0,
@@ -188,7 +192,8 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
   // Unit `target` of the global order -> what to work on.  `b` is its sequence, `off` its index inside it.
   auto describe = [&](int b, int off, Unit& un) {
     const bool kept = table && b < kKeptSpans;
-    const Span seq = kept ? ctl.seqs[b] : seq_span(s, cu_seqlens, b), rows = kept ? ctl.rows[b] : row_span(s, cu_qlens, b);
+    const Span seq = kept ? ctl.seqs[b] : table ? seq_span(s, cu_seqlens, b) : seq_span<true>(s, cu_seqlens, b);
+    const Span rows = kept ? ctl.rows[b] : table ? row_span(s, cu_qlens, b) : row_span<true>(s, cu_qlens, b);
     if ((seq.bad || rows.bad) && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
     un.tok0 = seq.first;
     un.n = seq.count;
