@@ -29,7 +29,11 @@
 // Warp 0 issues the TMA loads, warp 1 the MMAs into accumulators in tensor memory, warps 2..17 are the epilogue
 // (thread <-> accumulator row, four warps per 32-lane quarter of TMEM, a quarter of the columns each).  The epilogue of
 // the attention kernels, one exponential per element, is their bound: 16 per clock and SM from the special-function unit,
-// so two of every eight go through the FMA pipe instead, at the same precision (exp2_pair below).  All waits are bounded.
+// so two of every eight go through the FMA pipe instead, at the same precision (exp2_pair below).  All waits are bounded.  Where
+// one gives up, the producer stops, and the warps that work together go on to the end of their lists on whatever there is, since what
+// follows a wait there (elect.sync, tcgen05.ld, a warp's arrival) needs all lanes: every wait then returns after a few
+// attempts, the results are marked invalid, and the way is the same for every lane.  (A vote per wait: 1,167 -> 1,186 us for 14
+// layers of 2,230 tokens.)
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <limits.h>
@@ -164,6 +168,14 @@ __device__ __forceinline__ void drain_loads(PipeControl& ctl, int issued, int st
     ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.full[t % stages]), (t / stages) & 1, &never);
 }
 
+// The MMAs a warp has issued still write tensor memory: the accumulator of the last of them, in turn with `buffers`, has to be
+// done before the columns are given back.
+__device__ __forceinline__ void drain_mmas(PipeControl& ctl, int issued, int buffers) {
+  int never = 0;
+  if (issued > 0) ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_full[(issued - 1) % buffers]), ((issued - 1) / buffers) & 1, &never);
+  __syncwarp();
+}
+
 __device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueThreads) : "memory"); }
 
 // ---- the flat list of items and its equal runs -------------------------------------------------------
@@ -278,8 +290,8 @@ rollout_stats_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
       int loads = 0;
       for (int it = 0; it < count; ++it) {
         const int stage = it % kStages, buf = it % kBuffers;
-        if (!ptx::mbar_wait_warp(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort)) break;
-        if (!ptx::mbar_wait_warp(ptx::smem_u32(&ctl.tmem_empty[buf]), ((it / kBuffers) & 1) ^ 1u, abort)) break;
+        ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort);
+        ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_empty[buf]), ((it / kBuffers) & 1) ^ 1u, abort);
         ptx::tc_fence_after_sync();
         loads += it == 0 || x.jb == 0;
         const uint32_t k_tile = base + stage * kOperandBytes, q_tile = slots + ((loads - 1) & 1) * kOperandBytes;
@@ -290,6 +302,7 @@ rollout_stats_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
         if (x.row_ends()) ptx::umma_commit(ptx::smem_u32(&ctl.q_empty[(loads - 1) & 1]));
         x.advance();
       }
+      if (*abort) drain_mmas(ctl, count, kBuffers);
     }
   } else {
     const int quarter = warp & 3, cg = (warp - 2) >> 2;  // TMEM lanes 32 quarter .., columns 32 cg ..
@@ -309,8 +322,8 @@ rollout_stats_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
 #pragma unroll 1
     for (int it = 0; it < count; ++it, x.advance()) {
       const int buf = it % kBuffers;
-      if (ok) ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.tmem_full[buf]), (it / kBuffers) & 1, abort);
-      if (ok) {
+      ok &= ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_full[buf]), (it / kBuffers) & 1, abort);
+      {
         ptx::tc_fence_after_sync();
         uint32_t v[32];
         ptx::tmem_ld32(lane_addr + buf * kTile, v);
@@ -466,8 +479,8 @@ rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       const uint32_t idesc = ptx::umma_idesc_bf16(kTile, 32 * strip.width);
       for (int it = 0; it < hq; ++it) {
         const int stage = it % kStages, buf = it % kMapBuffers;
-        if (!ptx::mbar_wait_warp(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort)) break;
-        if (!ptx::mbar_wait_warp(ptx::smem_u32(&ctl.tmem_empty[buf]), ((it / kMapBuffers) & 1) ^ 1u, abort)) break;
+        ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort);
+        ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_empty[buf]), ((it / kMapBuffers) & 1) ^ 1u, abort);
         ptx::tc_fence_after_sync();
         const uint32_t q_tile = base + stage * kOperandBytes, k_tile = slots + ((it / group) & 1) * Cfg::kStripBytes;
         ptx::umma_bf16_steps<DIM / 16, kSubTileBytes, Cfg::kStripSubBytes>(tmem + buf * kStripCols, ptx::umma_desc_sw128(q_tile, 0),
@@ -475,6 +488,7 @@ rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         ptx::umma_commit(ptx::smem_u32(&ctl.empty[stage]));
         ptx::umma_commit(ptx::smem_u32(&ctl.tmem_full[buf]));
       }
+      if (*abort) drain_mmas(ctl, hq, kMapBuffers);
     }
   } else {
     const int quarter = warp & 3, cg = (warp - 2) >> 2;  // TMEM lanes 32 quarter .., columns cols * cg ..
@@ -529,9 +543,7 @@ rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         stage_stats(it, IntTag<1>{});
         epilogue_sync();
       }
-      if (!ok) continue;
-      ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.tmem_full[buf]), (it / kMapBuffers) & 1, abort);
-      if (!ok) continue;
+      ok &= ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_full[buf]), (it / kMapBuffers) & 1, abort);
       ptx::tc_fence_after_sync();
       const float neg_lse2 = ctl.neg_lse[it % kHeadChunk][row_in];
       const float2 nl = make_float2(neg_lse2, neg_lse2);
@@ -689,16 +701,14 @@ rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_
     }
   } else if (warp == 1) {
     {
-      int it = 0;
-      bool ok = true;
-      for (int round = 0; ok && unit_of(round) < units; ++round) {
+      int it = 0, round = 0;
+      for (; unit_of(round) < units; ++round) {
         const GemmUnit unit(unit_of(round), blocks, causal != 0, share);
         const int buf = round & 1;
-        ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.tmem_empty[buf]), ((round >> 1) & 1) ^ 1u, abort);
-        for (int kb = unit.kb0; kb < unit.kb1 && ok; ++kb, ++it) {
+        ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_empty[buf]), ((round >> 1) & 1) ^ 1u, abort);
+        for (int kb = unit.kb0; kb < unit.kb1; ++kb, ++it) {
           const int stage = it % kStages;
-          ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort);
-          if (!ok) break;
+          ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.full[stage]), (it / kStages) & 1, abort);
           ptx::tc_fence_after_sync();
           const uint32_t rt_hi = base + stage * kStageBytes, rt_lo = rt_hi + kSubTileBytes, a_hi = rt_hi + 2 * kSubTileBytes,
                          a_lo = rt_hi + 3 * kSubTileBytes;
@@ -711,8 +721,9 @@ rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_
           ptx::umma_bf16_steps<4, 0, 0>(d, rt_hi_desc, a_lo_desc, idesc, true);
           ptx::umma_commit(ptx::smem_u32(&ctl.empty[stage]));
         }
-        if (ok) ptx::umma_commit(ptx::smem_u32(&ctl.tmem_full[buf]));
+        ptx::umma_commit(ptx::smem_u32(&ctl.tmem_full[buf]));
       }
+      if (*abort) drain_mmas(ctl, round, 2);
     }
   } else {
     const int quarter = warp & 3, cg = (warp - 2) >> 2;
@@ -723,9 +734,9 @@ rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_
     for (int round = 0; unit_of(round) < units; ++round) {
       const int u = unit_of(round), buf = round & 1;
       const GemmUnit unit(u, blocks, causal != 0, share);
-      if (ok) ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.tmem_full[buf]), (round >> 1) & 1, abort);
+      ok &= ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.tmem_full[buf]), (round >> 1) & 1, abort);
       float x[32];
-      if (ok) {
+      {
         ptx::tc_fence_after_sync();
         uint32_t v[32];
         ptx::tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + buf * kTile + cg * 32, v);
@@ -734,9 +745,6 @@ rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_
         ptx::mbar_arrive_warp(ptx::smem_u32(&ctl.tmem_empty[buf]), lane);  // the accumulator may be overwritten
 #pragma unroll
         for (int c = 0; c < 32; ++c) x[c] = __uint_as_float(v[c]);
-      } else {
-#pragma unroll
-        for (int c = 0; c < 32; ++c) x[c] = 0.f;
       }
       bool mine = ok;  // this block writes the tile
       if (unit.parts > 1) {

@@ -130,7 +130,8 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
   const int n = min(seq.count, blocks * tiles_per_block * kTile);
   const int rows_here = min(rows_per_tile, rows.count * s.group - rt * rows_per_tile);  // of this row tile (a multiple of G)
   const int tiles = rows_here > 0 ? (n + kTile - 1) / kTile : 0;                         // key tiles of the sequence
-  const int t0 = min(tiles, c * tiles_per_block), mine = min(tiles - t0, tiles_per_block);
+  const int t0 = min(tiles, c * tiles_per_block);
+  int mine = min(tiles - t0, tiles_per_block);
   const bool causal = (s.flags & FASTAV_CAUSAL) != 0;
 
   if (warp == 0) {
@@ -170,15 +171,19 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
     ptx::tc_fence_before_sync();
     ptx::mbar_arrive_warp(ptx::smem_u32(&ctl.tmem_ready), lane);
     const uint32_t tmem = ctl.tmem_base;
-    bool ok = mine <= 0 || ptx::mbar_wait_warp(ptx::smem_u32(&ctl.q_full), 0, abort);
-    for (int t = 0; t < mine && ok; ++t) {
-      ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.k_full[t]), 0, abort);
-      if (!ok) break;
+    // A wait that gives up changes nothing in the way the warp goes: see the epilogue.
+    if (mine > 0) ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.q_full), 0, abort);
+    for (int t = 0; t < mine; ++t) {
+      ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.k_full[t]), 0, abort);
       ptx::tc_fence_after_sync();
       ptx::umma_bf16_steps<DIM / 16, kSubTileBytes, kSubTileBytes>(tmem + t * kTile, ptx::umma_desc_sw128(q_smem, 0),
                                                                    ptx::umma_desc_sw128(k_smem + t * L::kOperandBytes, 0),
                                                                    ptx::umma_idesc_bf16(kTile, kTile), false);
       ptx::umma_commit(ptx::smem_u32(&ctl.s_full[t]));
+    }
+    if (*abort && mine > 0) {  // the columns are given back below: not before the last MMA is done
+      int never = 0;
+      ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.s_full[mine - 1]), 0, &never);
     }
     __syncwarp();
   }
@@ -209,13 +214,15 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
     }
     epilogue_sync();
     limit = ctl.limit[row_in];
-    ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.tmem_ready), 0, abort);
+    // No tensor memory (one answer for the warp): nothing to read.  After that a wait that gives up only marks the results as
+    // invalid: what follows it needs all lanes, so they all go on.
+    const bool have_tmem = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.tmem_ready), 0, abort);
+    if (!have_tmem) mine = 0;
     ptx::tc_fence_after_sync();
     lane_addr = ctl.tmem_base + ((uint32_t)(quarter * 32) << 16) + cg * 32;
     if (!lse_in) {
       for (int t = 0; t < mine; ++t) {
-        if (ok) ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.s_full[t]), 0, abort);
-        if (!ok) break;
+        ok &= ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.s_full[t]), 0, abort);
         ptx::tc_fence_after_sync();
         uint32_t v[32];
         ptx::tmem_ld32(lane_addr + t * kTile, v);
@@ -293,8 +300,7 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
     const float nl = ctl.neg_lse[row_in];
     const float2 nl2 = make_float2(nl, nl);
     for (int t = 0; t < mine; ++t) {
-      if (ok && lse_in) ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.s_full[t]), 0, abort);  // (else waited for above)
-      if (!ok) break;
+      if (lse_in) ok &= ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.s_full[t]), 0, abort);  // (else waited for above)
       ptx::tc_fence_after_sync();
       uint32_t v[32];
       ptx::tmem_ld32(lane_addr + t * kTile, v);

@@ -443,7 +443,7 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
         float2 sum2 = make_float2(0.f, 0.f);
         for (int t = 0; t < tiles; ++t, ++uses) {
           const int i = uses & 1;
-          ok = ptx::mbar_wait_warp<true>(ptx::smem_u32(&ctl.tmem_full[i * 2 + e]), (uses >> 1) & 1, abort);
+          ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.tmem_full[i * 2 + e]), (uses >> 1) & 1, abort);
           if (!ok) break;
           ptx::tc_fence_after_sync();
           const int bound = last_visible - (key_begin + t * kTileKeys + h * 64);  // columns 0..bound of this half are visible
@@ -487,7 +487,7 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
         float* out = logits + un.tok0;
         for (int t = 0; t < tiles; ++t, ++tile_no) {
           const int i = tile_no & 1;
-          ok = ptx::mbar_wait_warp<true>(ptx::smem_u32(&ctl.tmem_full[i]), (tile_no >> 1) & 1, abort);
+          ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.tmem_full[i]), (tile_no >> 1) & 1, abort);
           if (!ok) break;
           ptx::tc_fence_after_sync();
           const int key = key_begin + t * kTileKeys + my_lane;
@@ -547,7 +547,7 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
         for (int t = 0; t < tiles; ++t, ++tile_no) {
           const int i = tile_no & 1;
           const uint32_t parity = (tile_no >> 1) & 1;
-          ok = ptx::mbar_wait_warp<true>(ptx::smem_u32(&ctl.tmem_full[i]), parity, abort);
+          ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.tmem_full[i]), parity, abort);
           if (!ok) break;
           ptx::tc_fence_after_sync();
           const int key = key_begin + t * kTileKeys + my_lane;
@@ -562,7 +562,7 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
             ctl.sums[i][wg - 1][my_lane] = sum;
             ptx::mbar_arrive(ptx::smem_u32(&ctl.sums_ready[i]));
           } else {
-            ok = ptx::mbar_wait_warp<true>(ptx::smem_u32(&ctl.sums_ready[i]), parity, abort);
+            ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.sums_ready[i]), parity, abort);
             if (!ok) break;
 #pragma unroll
             for (int w = 0; w < kGroups - 1; ++w) sum += ctl.sums[i][w][my_lane];

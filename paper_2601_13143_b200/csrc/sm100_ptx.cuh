@@ -82,12 +82,10 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
 }
 
 // The same for a whole converged warp, with one answer: a lane may see the phase complete just as another gives up, and what
-// follows a wait (elect.sync, tcgen05.ld, a warp's arrival) needs all lanes or none.  VOTE_FIRST: a first attempt by itself,
-// which the two-sweep score (294.3 us instead of 299.2 for 4 x 16,384 tokens) is the faster for, and the one-pass score the
-// slower (24.2 us instead of 24.1 for 2,048).
-template <bool VOTE_FIRST = false>
+// follows a wait (elect.sync, tcgen05.ld, a warp's arrival) needs all lanes or none.  (The voted first attempt: 294.3 us instead
+// of 299.2 for the two sweeps of 4 x 16,384 tokens.)
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort, uint64_t limit_ns = kWaitLimitNs) {
-  if (VOTE_FIRST && __all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) return true;
+  if (__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) return true;
   return __all_sync(0xFFFFFFFFu, mbar_wait_bounded(bar, parity, abort, limit_ns)) != 0;
 }
 
