@@ -28,8 +28,8 @@
 //
 // Warp 0 issues the TMA loads, warp 1 the MMAs into accumulators in tensor memory, warps 2..17 are the epilogue
 // (thread <-> accumulator row, four warps per 32-lane quarter of TMEM, a quarter of the columns each).  The epilogue of
-// the attention kernels, one exponential per element, is their bound: 16 per clock and SM from the special-function unit,
-// so two of every eight go through the FMA pipe instead, at the same precision (exp2_pair below).  All waits are bounded.  Where
+// the attention kernels is their bound: one exponential per element, 16 per clock and SM, and as much again of fixed cost per tile
+// (a quarter of the exponentials on the FMA pipe instead: 0.5 to 1 %, and NaN came out as 2^-126).  All waits are bounded.  Where
 // one gives up, the producer stops, and the warps that work together go on to the end of their lists on whatever there is, since what
 // follows a wait there (elect.sync, tcgen05.ld, a warp's arrival) needs all lanes: every wait then returns after a few
 // attempts, the results are marked invalid, and the way is the same for every lane.  (A vote per wait: 1,167 -> 1,186 us for 14
@@ -99,31 +99,7 @@ __device__ __forceinline__ void get8(const float* at, float (&x)[8]) {
   x[0] = a.x, x[1] = a.y, x[2] = a.z, x[3] = a.w, x[4] = b.x, x[5] = b.y, x[6] = b.z, x[7] = b.w;
 }
 
-// 2^x for a pair of x <= ~0 on the FMA and integer pipes: x = n + f with n the nearest integer (read off the mantissa after
-// adding 1.5 * 2^23), a minimax polynomial of degree 5 for 2^f on [-1/2, 1/2] (Remez exchange on the relative error:
-// 7.5e-8, 2.3e-7 when evaluated in fp32, what the special-function unit has), and n added into the exponent field.
-// Inputs below -126 (including -inf) give about 2^-126.
-__device__ __forceinline__ float2 exp2_pair_fma(float2 x) {
-  const float kMagic = 12582912.f;
-  x.x = fmaxf(x.x, -126.f);
-  x.y = fmaxf(x.y, -126.f);
-  const float2 t = __fadd2_rn(x, make_float2(kMagic, kMagic));
-  const float2 n = __fadd2_rn(t, make_float2(-kMagic, -kMagic));
-  const float2 f = __ffma2_rn(n, make_float2(-1.f, -1.f), x);
-  float2 p = __ffma2_rn(f, make_float2(1.32764725e-3f, 1.32764725e-3f), make_float2(9.67554096e-3f, 9.67554096e-3f));
-  p = __ffma2_rn(p, f, make_float2(0.0555071309f, 0.0555071309f));
-  p = __ffma2_rn(p, f, make_float2(0.240221202f, 0.240221202f));
-  p = __ffma2_rn(p, f, make_float2(0.693146944f, 0.693146944f));
-  p = __ffma2_rn(p, f, make_float2(1.00000012f, 1.00000012f));
-  return make_float2(__int_as_float(__float_as_int(p.x) + (__float_as_int(t.x) << 23)),
-                     __int_as_float(__float_as_int(p.y) + (__float_as_int(t.y) << 23)));
-}
-// Of the 8 column pairs of every 16 columns, those of the mask take the FMA pipe (none, 1, 2, 3 or 4 of 8: within 1-3 %).
-constexpr int kFmaPairs = 0x88;
-__device__ __forceinline__ float2 exp2_pair(float2 x, int pair) {
-  if ((kFmaPairs >> (pair & 7)) & 1) return exp2_pair_fma(x);
-  return make_float2(ptx::ex2_approx(x.x), ptx::ex2_approx(x.y));
-}
+__device__ __forceinline__ float2 exp2_pair(float2 x) { return make_float2(ptx::ex2_approx(x.x), ptx::ex2_approx(x.y)); }
 
 __device__ __forceinline__ void pipe_setup(PipeControl& ctl, int stages, int warp, const void* map_a, const void* map_b) {
   if (threadIdx.x == 0) {
@@ -349,7 +325,7 @@ rollout_stats_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
           const float2 sh = make_float2(shift, shift);
 #pragma unroll
           for (int c = 0; c < 32; c += 2)
-            sum2 = __fadd2_rn(sum2, exp2_pair(__ffma2_rn(make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc, sh), c / 2));
+            sum2 = __fadd2_rn(sum2, exp2_pair(__ffma2_rn(make_float2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc, sh)));
         }
         __syncwarp();  // the rows of a warp differ in `limit`; the tcgen05 instructions that follow need the whole warp
       }
@@ -560,24 +536,24 @@ rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
       ptx::tmem_ld_wait_for(v, v4);
       ptx::tc_fence_before_sync();
       ptx::mbar_arrive_warp(ptx::smem_u32(&ctl.tmem_empty[buf]), lane);  // the accumulator may be overwritten
-      auto weights = [&](const uint32_t* x, int c) {
-        return exp2_pair(__ffma2_rn(make_float2(__uint_as_float(x[0]), __uint_as_float(x[1])), sc, nl), c / 2);
+      auto weights = [&](const uint32_t* x) {
+        return exp2_pair(__ffma2_rn(make_float2(__uint_as_float(x[0]), __uint_as_float(x[1])), sc, nl));
       };
       // Columns that a row may not see are added up too (a column's sum meets no other) and dropped when the tile is stored: with
       // two selects per pair the strips on the diagonal ended last (39.8 -> 37.4 us).
       if (pieces >= 4) {
 #pragma unroll
-        for (int c = 0; c < 32; c += 2) acc2[c / 2] = __fadd2_rn(acc2[c / 2], weights(v + c, c));
+        for (int c = 0; c < 32; c += 2) acc2[c / 2] = __fadd2_rn(acc2[c / 2], weights(v + c));
         if (pieces == 5) {
 #pragma unroll
-          for (int c = 0; c < 8; c += 2) acc2[16 + c / 2] = __fadd2_rn(acc2[16 + c / 2], weights(v4 + c, c));
+          for (int c = 0; c < 8; c += 2) acc2[16 + c / 2] = __fadd2_rn(acc2[16 + c / 2], weights(v4 + c));
         }
       } else {
 #pragma unroll
         for (int p = 0; p < 3; ++p) {
           if (p < pieces) {
 #pragma unroll
-            for (int c = 8 * p; c < 8 * p + 8; c += 2) acc2[c / 2] = __fadd2_rn(acc2[c / 2], weights(v + c, c));
+            for (int c = 8 * p; c < 8 * p + 8; c += 2) acc2[c / 2] = __fadd2_rn(acc2[c / 2], weights(v + c));
           }
         }
       }

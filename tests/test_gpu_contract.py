@@ -190,3 +190,21 @@ def test_statistics_find_their_sequence_in_any_batch(batch):
     torch.cuda.synchronize()
     parity.assert_scores_close(buf.scores, parity.oracle_scores(p))
     assert int(buf.device_status) == 0
+
+
+def test_a_key_that_is_not_a_number_shows_in_the_attention_map():
+    """Whatever column it stands in: every row that sees the key has NaN there."""
+    from test_gpu_rollout import _layers, _params
+
+    n, hq, hkv, d = 160, 2, 1, 64
+    (q, k), = [(q.cuda(), k.cuda()) for q, k in _layers(5, n, hq, hkv, d, 1)]
+    p = _params(n, hq, hkv, d, q, k, d**-0.5, True)
+    ws = torch.empty(fastav.fastav_rollout_workspace_bytes(p), dtype=torch.uint8, device="cuda")
+    state = torch.empty(fastav.fastav_rollout_state_bytes(n), dtype=torch.uint8, device="cuda")
+    for j in range(32, 49):
+        bad = k.clone()
+        bad[j] = float("nan")
+        out = torch.zeros(n, n, device="cuda")
+        fastav.fastav_rollout_begin(n, state)
+        fastav.fastav_rollout_layer(p, q, bad, 0.5, 0, state, ws, map_out_opt=out)
+        assert out[j:, j].isnan().all(), j
