@@ -28,11 +28,6 @@ __device__ __forceinline__ void remote_store2(uint32_t a, unsigned x, unsigned y
 __device__ __forceinline__ void remote_store4(uint32_t a, uint4 v) {  // 16-byte aligned
   asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
-__device__ __forceinline__ unsigned remote_load(uint32_t a) {
-  unsigned v;
-  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
-  return v;
-}
 __device__ __forceinline__ void cluster_arrive() {
   __syncwarp();  // the aligned form needs whole warps
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");

@@ -63,8 +63,10 @@ Arena plan_arena(const fastav_params& p) {
 
 // ---- the page-locked path ----------------------------------------------------------------------------
 constexpr int kCopyThreads = 256;
-// Blocks of the gather through PCIe: a quarter of the SMs keeps enough rows on the way; more only crowd the link (2,048 tokens,
-// half of them kept: 37 / 74 / 148 / 592 blocks take 333 / 341 / 348 / 361 us).
+// Blocks of the gather through PCIe: a quarter of the SMs keeps enough rows on the way; more only crowd the link.  18 / 37 / 74 /
+// 148 blocks, us per call: 2,048 tokens of 9 KB (hidden 3,584), 30 % kept 268 / 229 / 240 / 238, half 348 / 318 / 328 / 340, 90 % 494 / 505 /
+// 516 / 534, 1,200 tokens of 12 KB, 40 % 262 / 231 / 240 / 242, 500 tokens of 9 KB, half 103 / 105 / 105 / 106, 2,048 of 1.5 KB 81 / 81 /
+// 82 / 86, 400 of 1.5 KB 47 / 43 / 43 / 44.
 constexpr int kHostGatherBlocks = kNumSMs / 4;
 constexpr int kCopyUnroll = 8;                                   // 16-byte loads in flight per thread
 constexpr int kPieceBytes = kCopyThreads * kCopyUnroll * 16;     // what a block copies at a time: 32 KB
