@@ -51,6 +51,11 @@ def oracle_prune(p, hidden=None, pos=None, protect=None):
                         protect_rows=p.protect_rows, protect_mask=None if protect is None else protect.numpy())
 
 
+def overflows(protected: np.ndarray, cu, keeps) -> bool:
+    """Some sequence has more protected tokens than it keeps (FASTAV_DEV_PROTECT_OVERFLOW)."""
+    return any(int(protected[a:b].sum()) > min(max(int(k), 0), int(b) - int(a)) for a, b, k in zip(cu, cu[1:], keeps))
+
+
 def assert_scores_close(gpu_scores: torch.Tensor, ref: np.ndarray, what=""):
     got = gpu_scores.detach().cpu().double().numpy()
     assert got.shape == ref.shape
@@ -136,6 +141,8 @@ def assert_bits_equal(gpu_t: torch.Tensor | None, ref, what=""):
 def check_fused_against_oracle(p, buf: fastav.PruneBuffers, ref: dict, hidden=None, pos=None, protect=None, what="") -> dict:
     """Full comparison of one fused prune call.  Returns statistics."""
     status = int(buf.device_status.cpu())
+    overflow = overflows(protected_mask(p, protect), p.cu_seqlens.tolist(), p.keep_counts.tolist())
+    assert bool(status & fastav.FASTAV_DEV_PROTECT_OVERFLOW) == overflow, f"{what}: status {status}"
     max_rel = assert_scores_close(buf.scores, ref["scores"], what)
     total_keep = int(ref["cu_keep"][-1])
     gpu_keep = buf.keep_idx[:total_keep]

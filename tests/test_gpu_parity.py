@@ -226,6 +226,12 @@ def _select_case(lens, keeps, scores, protect=None, rows=None, q_idx=None, globa
     got = keep_idx.cpu().numpy()
     assert got[:len(ref_idx)].tolist() == ref_idx.tolist()
     assert (got[len(ref_idx):] == -7).all()          # nothing written past the end
+    protected = np.zeros(int(cu[-1]), dtype=bool) if protect is None else np.asarray(protect) != 0
+    if protect_rows:
+        for b, n in enumerate(lens):
+            idx = q_idx[cuq[b]:cuq[b + 1]]
+            protected[cu[b] + idx[(idx >= 0) & (idx < n)]] = True
+    assert bool(int(status) & fastav.FASTAV_DEV_PROTECT_OVERFLOW) == parity.overflows(protected, cu, keeps)
     return int(status.cpu())
 
 
