@@ -24,7 +24,7 @@
 // that makes the fewest, fullest rounds.  The product cuts the K loops that are much longer than an SM's fair share into parts,
 // whose fp32 tiles meet in the workspace: the part that finishes last adds them up in order (no block waits for another).
 // 2,230 tokens, 28 / 4 heads of 128, per layer: statistics 34, map 37.4, product 21.1 us; 14 layers with their
-// read-out 1,164 us (1,924 with a block per tile and head, or per tile).
+// read-out 1,146 us (1,924 with a block per tile and head, or per tile).
 //
 // Warp 0 issues the TMA loads, warp 1 the MMAs into accumulators in tensor memory, warps 2..17 are the epilogue
 // (thread <-> accumulator row, four warps per 32-lane quarter of TMEM, a quarter of the columns each).  The epilogue of
