@@ -11,6 +11,8 @@
 // segment issuing cp.async.bulk global -> shared (completion on an mbarrier) and then shared ->
 // global, several rows in flight per warp and no register staging.  Rows whose segments are not
 // 16-byte friendly, or too long for the ring, take the load/store kernel below.
+#include <limits.h>
+
 #include "common.cuh"
 #include "gather.cuh"
 #include "sm100_ptx.cuh"
@@ -55,6 +57,7 @@ __global__ void __launch_bounds__(kThreads) compact_rows_kernel(Shapes s, RowStr
 
 // ---- bulk-copy path ---------------------------------------------------------------------------------
 constexpr int kBulkStages = 4;          // row slots per warp
+constexpr int kAhead = kBulkStages - 2; // rows loaded ahead of the one being stored
 constexpr int kBulkMaxWarps = 8;
 constexpr int kBulkSmemBudget = 200 * 1024;
 
@@ -137,53 +140,95 @@ compact_rows_bulk_kernel(Shapes s, RowStreams t, const int32_t* __restrict__ kee
   pdl_acquire(keep_idx);
   pdl_acquire(cu_keep);
   pdl_acquire(cu_seqlens);
-  int rows = chain_load_cached(cu_keep + s.batch);
-  if (rows > s.total_keep) rows = s.total_keep;  // never write past the caller's buffers
+  // Where this warp's rows come from.  The index words of its first rows are asked for all at once: the bounds of the sequences,
+  // one per lane, and the tokens (one read for a row that does not exist is never used).  One after the other they were four trips to L2
+  // ahead of the first copy, and more where the sequence of a row was searched for: a chain of 13 stages from 744 tokens 171 ->
+  // 164 us, 1 x 2,048 tokens 24.2 -> 23.3, 32 ragged sequences of up to 8,192 tokens 314 -> 308.
   const int first = blockIdx.x * warps + warp, step = gridDim.x * warps;
+  const bool by_lane = s.batch < 32;
+  int keep_at = INT_MAX, seq_at = 0;  // by_lane: cu_keep and cu_seqlens of entry `lane`
+  if (by_lane && lane <= s.batch) {
+    keep_at = chain_load_cached(cu_keep + lane);
+    seq_at = chain_load_cached(cu_seqlens + lane);
+  }
+  auto token_of = [&](int i) -> int {  // keep_idx of this warp's row i
+    const long long row = first + (long long)i * step;
+    return row < s.total_keep ? chain_load(keep_idx + row) : 0;
+  };
+  int token[kAhead];
+#pragma unroll
+  for (int i = 0; i < kAhead; ++i) token[i] = token_of(i);
+  int rows = by_lane ? __shfl_sync(0xFFFFFFFFu, keep_at, s.batch) : chain_load_cached(cu_keep + s.batch);
+  if (rows > s.total_keep) rows = s.total_keep;  // never write past the caller's buffers
   const int my_rows = first < rows ? (rows - first + step - 1) / step : 0;
+  if (!by_lane || lane >= s.batch) keep_at = INT_MAX;
 
-  // Source token of this warp's i-th row, or -1 for an index outside its sequence (row skipped, reported).
-  auto source_of = [&](int i) -> long long {
+  // Source token of row i, whose entry of keep_idx is `idx`, or -1 for an index outside its sequence (row skipped, reported).
+  auto source_of = [&](int i, int idx) -> long long {
     const int row = first + i * step;
-    int lo = 0, hi = s.batch;  // largest b with cu_keep[b] <= row
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (chain_load_cached(cu_keep + mid) <= row) lo = mid; else hi = mid;
+    int from, end;  // of the row's sequence
+    if (by_lane) {
+      const int b = max(0, 31 - __clz(__ballot_sync(0xFFFFFFFFu, keep_at <= row)));  // the last one that starts at or before it
+      from = __shfl_sync(0xFFFFFFFFu, seq_at, b);
+      end = __shfl_sync(0xFFFFFFFFu, seq_at, b + 1);
+    } else {
+      int lo = 0, hi = s.batch;  // largest b with cu_keep[b] <= row
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (chain_load_cached(cu_keep + mid) <= row) lo = mid; else hi = mid;
+      }
+      from = chain_load_cached(cu_seqlens + lo);
+      end = chain_load_cached(cu_seqlens + lo + 1);
     }
-    const long long src = (global_idx ? 0ll : (long long)cu_seqlens[lo]) + chain_load(keep_idx + row);
-    if (src < cu_seqlens[lo] || src >= cu_seqlens[lo + 1]) {
+    const long long src = (global_idx ? 0ll : (long long)from) + idx;
+    if (src < from || src >= end) {
       if (lane == 0 && device_status) atomicOr(device_status, FASTAV_DEV_BAD_INDEX);
       return -1;
     }
     return src;
   };
   // Issue the loads of row i into slot i % stages (all lanes call; one lane per segment copies).
-  auto issue_load = [&](int i) -> bool {
-    const long long src = source_of(i);
+  auto issue_load = [&](int i, long long src) {
+    const uint32_t bar = ptx::smem_u32(&full[warp][i % kBulkStages]);
+    if (!active) return;
     if (src < 0) {  // skipped row: the slot's barrier still completes its phase, so later rows keep their parity
-      if (active) ptx::mbar_arrive(ptx::smem_u32(&full[warp][i % kBulkStages]));
-      return false;
-    }
-    if (active) {
-      const uint32_t bar = ptx::smem_u32(&full[warp][i % kBulkStages]);
+      ptx::mbar_arrive(bar);
+    } else {
       ptx::mbar_arrive_expect_tx(bar, seg.bytes);
       bulk_load(ring + (i % kBulkStages) * row_bytes + seg.slot_off, seg.in + src * seg.in_stride, seg.bytes, bar);
     }
-    if (lane == 0 && t.pos_in) t.pos_out[first + i * step] = t.pos_in[src];
-    return true;
   };
 
   int abort_flag = 0;
   unsigned loaded = 0;  // bit i % 32: row i has loads in flight or done (not skipped)
-  constexpr int kAhead = kBulkStages - 2;  // rows loaded ahead of the one being stored
-  for (int i = 0; i < min(kAhead, my_rows); ++i)
-    if (issue_load(i)) loaded |= 1u << (i & 31);
+  // The first rows' positions, one per lane, are read beside the rows and written after the first of them: where a warp has a row
+  // or two, each read and written in turn would add a trip to memory.
+  long long first_src = -1;
+#pragma unroll
+  for (int i = 0; i < kAhead; ++i)
+    if (i < my_rows) {
+      const long long src = source_of(i, token[i]);
+      issue_load(i, src);
+      if (src >= 0) loaded |= 1u << i;
+      if (lane == i) first_src = src;
+    }
+  const bool has_pos = t.pos_in && first_src >= 0;
+  const int32_t first_pos = has_pos ? t.pos_in[first_src] : 0;
   for (int i = 0; i < my_rows; ++i) {
     // The slot of row i + kAhead last held row i - 2: its store must have finished reading shared memory.
-    if (i + kAhead < my_rows) {
+    const int next = i + kAhead;
+    if (next < my_rows) {
       bulk_wait_read<1>();
-      if (issue_load(i + kAhead)) loaded |= 1u << ((i + kAhead) & 31);
-      else loaded &= ~(1u << ((i + kAhead) & 31));
+      // (the token is read here and not ahead: tokens of 32 rows at a time took the wait out and made the gathers of 4 x 6,554
+      // tokens 109 -> 115 us, 32 sequences of up to 4,096 214 -> 222)
+      const long long src = source_of(next, chain_load(keep_idx + first + (long long)next * step));
+      issue_load(next, src);
+      if (src >= 0) {
+        loaded |= 1u << (next & 31);
+        if (lane == 0 && t.pos_in) t.pos_out[first + (long long)next * step] = t.pos_in[src];
+      } else {
+        loaded &= ~(1u << (next & 31));
+      }
     }
     if (loaded & (1u << (i & 31))) {
       const uint32_t bar = ptx::smem_u32(&full[warp][i % kBulkStages]);
@@ -194,6 +239,7 @@ compact_rows_bulk_kernel(Shapes s, RowStreams t, const int32_t* __restrict__ kee
       if (active) bulk_store(seg.out + (long long)(first + i * step) * seg.out_stride, ring + (i % kBulkStages) * row_bytes + seg.slot_off, seg.bytes);
     }
     bulk_commit();  // one group per row, empty or not, so that the wait above always counts rows
+    if (i == 0 && has_pos) t.pos_out[first + (long long)lane * step] = first_pos;
   }
   bulk_wait_all();  // the slots and the outputs are this kernel's until every store has landed
 }

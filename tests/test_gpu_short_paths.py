@@ -80,3 +80,9 @@ def test_mask_emission(total, batch, offset):
 @pytest.mark.parametrize("rows", [1, 8])
 def test_gather_of_batches(batch, n, keep, rows):
     _check([n] * batch, rows, 8, 2, 64, hid=64, keep=keep)
+
+
+# The compaction keeps the bounds of up to 31 sequences in a warp's lanes; warps with one row, a few, and more than 32.
+@pytest.mark.parametrize("batch,n", [(1, 40), (1, 592), (30, 50), (31, 50), (32, 50), (31, 1000), (33, 1000)])
+def test_gather_bounds_by_lane(batch, n):
+    _check([n if b % 5 else 0 for b in range(1, batch)] + [n], 1, 4, 2, 64, hid=3584, keep=0.8)
