@@ -8,7 +8,8 @@
 //           kPartials: the tensor-core kernels' sums per (KV head, chunk of query rows) and token are added up.
 //           kScores: finished scores (fastav_select).
 //   select  the scores as order-preserving 32-bit keys (protected tokens: the largest) go to every block of the cluster, a
-//           cluster barrier, and each block runs the whole selection for itself: a histogram of the leading 12 bits,
+//           cluster barrier.  Up to 768 tokens (clusters of 16) each block then ranks its own slice by counting and tells the others how
+//           many it keeps.  Beyond, each block runs the whole selection for itself: a histogram of the leading 12 bits,
 //           the keys of the bin that holds the k-th largest finished by counting ranks (further 12-bit passes only if it holds
 //           more than 256), one stable prefix sum in index order;
 //   gather  the survivors among a block's own tokens.
@@ -48,9 +49,10 @@ constexpr int kStatLanes = 8;   // lanes that share one (segment, term) of the r
 constexpr int kTokenLanes = 8;  // lanes that share one token's sum over the terms
 
 // A sequence is cut into sixteen segments whatever the size of the cluster, and a block owns 16 / blocks of them: the row
-// statistics are kept per segment and merged in a fixed tree.
+// statistics are kept per segment and merged in a fixed tree.  Segments are whole fragments of 16 tokens (in steps of 32, 744 tokens
+// kept twelve of sixteen blocks busy).
 constexpr int kSegments = kMaxCluster;
-__host__ __device__ inline int segment_of(int n) { return n <= 32 * kSegments ? 32 : ((n + kSegments - 1) / kSegments + 31) & ~31; }
+__host__ __device__ inline int segment_of(int n) { return n <= 32 * kSegments ? 32 : ((n + kSegments - 1) / kSegments + 15) & ~15; }
 
 struct FewArgs {
   const uint16_t* q;    // kKeys
@@ -66,6 +68,12 @@ struct FewArgs {
   RowStreams rows;      // do_gather
 };
 
+// Short sequences are selected by counting: every block ranks its own slice's keys against all keys of the sequence, at most this
+// many comparisons and tokens per block.  In place of five block-wide steps, one with no barrier inside and another exchange over the
+// cluster; the comparisons grow with the square of the length.  From all keys to the keep list, by digits / by counting (time stamps):
+// 512 tokens 2.3 / 1.9 us, 744 2.3 / 2.1, 820 2.4 / 2.9, 1,024 2.7 / 3.2.
+constexpr int kCountPairs = 36 << 10, kCountSlice = 256;
+
 struct alignas(16) FewShared {
   unsigned hist[kBins];  // later: the block's survivors
   unsigned keys[kMaxTokens];
@@ -75,6 +83,7 @@ struct alignas(16) FewShared {
   unsigned warp_a[kWarps];
   int limit[kNarrowMaxRows];
   int index[8];
+  unsigned kept[kCountSlice / 32], kept_of[kMaxCluster];  // selection by counting: the block's survivors; how many each block has
   int base, list_n, remaining, bucket, need_eq, first_out, end_out, unused;
   unsigned prefix, threshold, unused2[2];
 };
@@ -143,6 +152,7 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   if (selecting)
     for (int i = tid; i < kBins / 4; i += kThreads) reinterpret_cast<uint4*>(sh.hist)[i] = make_uint4(0, 0, 0, 0);
   if (tid < kMaxTokens / 32) sh.prot_bits[tid] = 0u;
+  if (tid < kCountSlice / 32) sh.kept[tid] = 0u;
   if (tid == 32) { sh.base = 0; sh.list_n = 0; }
   chain_end_setup(s, cu_seqlens, keep_counts, protect, q_idx, cu_qlens);
   // ---- the caller's index arrays: one warp asks for all of them at once (sixteen warps of sixteen blocks asking for the
@@ -168,6 +178,20 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   const int terms = s.hq * rows;    // term i = (head i / rows, row i % rows)
   const bool causal = (s.flags & FASTAV_CAUSAL) != 0;
   k = k < 0 ? 0 : (k > n ? n : k);
+
+  // kKeys: the piece of the queries this thread stages first.
+  constexpr int kQStride = DIM * 2 + 64;
+  auto q_piece = [&](int i, int& at) -> const uint4* {  // piece i of the query rows; where it goes
+    const int row = i / (DIM / 8), piece = i % (DIM / 8);  // row: (KV head, f)
+    const int gg = row / flat, f = row - gg * flat, r = f / s.group;
+    at = row * kQStride + piece * 16;
+    return reinterpret_cast<const uint4*>(a.q + (long long)(qrows.first + r) * s.q_st + (long long)(gg * s.group + f - r * s.group) * s.q_sh + piece * 8);
+  };
+  const bool stages = FRONT == kKeys && tid < terms * (DIM / 8);
+  int q_at = 0;
+  const uint4* q_from = nullptr;
+  if (stages) q_from = q_piece(tid, q_at);
+  asm volatile("" : "+l"(q_from), "+r"(q_at));  // worked out ahead of the wait
 
   pdl_wait();
   // The scored rows' tokens survive (kKeys also needs them as the rows' limits).
@@ -214,7 +238,6 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
     // ---- logits ----------------------------------------------------------------------------------------------
     const FewLayout lay = few_layout(a.slice_cap, s.hq * a.rq, DIM);
     unsigned char* const more = smem_raw + sizeof(FewShared);
-    constexpr int kQStride = DIM * 2 + 64;
     unsigned char* const q_sh = more + lay.q;
     float* const lse = reinterpret_cast<float*>(more + lay.lse);
     float2* const stats = reinterpret_cast<float2*>(more + lay.stats);
@@ -230,14 +253,15 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
       const int g = u % s.hkv, tok = u / s.hkv * 16;
       if (u < units) frag.load(k_base + (long long)tok * s.k_st + (long long)g * s.k_sh, s.k_st, m - tok, lane);
     };
+    uint4 q_first = make_uint4(0, 0, 0, 0);
+    if (stages) q_first = chain_load(q_from);  // the queries ahead of the keys: all warps wait for them together
     fetch(even, warp);
     fetch(odd, warp + kWarps);
-    for (int i = tid; i < terms * (DIM / 8); i += kThreads) {
-      const int row = i / (DIM / 8), piece = i % (DIM / 8);  // row: (KV head, f)
-      const int gg = row / flat, f = row - gg * flat, r = f / s.group;
-      const uint4 v = chain_load(reinterpret_cast<const uint4*>(a.q + (long long)(qrows.first + r) * s.q_st +
-                                                                (long long)(gg * s.group + f - r * s.group) * s.q_sh + piece * 8));
-      *reinterpret_cast<uint4*>(q_sh + row * kQStride + piece * 16) = v;
+    if (stages) *reinterpret_cast<uint4*>(q_sh + q_at) = q_first;
+    for (int i = tid + kThreads; i < terms * (DIM / 8); i += kThreads) {
+      int at;
+      const uint4 v = chain_load(q_piece(i, at));
+      *reinterpret_cast<uint4*>(q_sh + at) = v;
     }
     if (tid < flat) {
       sh.row_of[tid] = tid / s.group;
@@ -405,9 +429,8 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
     }
   }
   if (!selecting) return;  // uniform for the cluster; nothing remote is outstanding
-  cluster_sync();          // the last remote access: from here on every block works for itself
+  cluster_sync();          // every block has all keys
 
-  // ---- selection: thread t owns the tokens 4 t .. 4 t + 3 of the whole sequence ----------------------------------
   const int base = sh.base;
   if (c == 0 && tid == 0) {
     cu_keep[b + 1] = base + k;
@@ -419,6 +442,60 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
         if (sh.keys[j] == kProtectedKey) atomicOr(device_status, FASTAV_DEV_PROTECT_OVERFLOW);
     return;
   }
+  const bool global_idx = (s.flags & FASTAV_KEEP_IDX_GLOBAL) != 0;
+  unsigned* const picked = sh.hist;  // survivor `out` of the sequence is token picked[out % 4096]
+  int first = 0, count = 0;          // this block's survivors
+
+  if (slice <= kCountSlice && n * slice <= kCountPairs) {
+    // ---- selection by counting (uniform for the cluster): some lanes per token of the slice, each compares it with every so
+    //      many keys.  A token's rank is the number of keys above its own plus the equal ones of lower index. --------------
+    const int tok_bits = slice <= 32 ? 1 : slice <= 64 ? 2 : slice <= 128 ? 3 : 4;  // tokens per warp; the lanes share them out
+    const int j = (warp << tok_bits) + (lane & ((1 << tok_bits) - 1)), part = lane >> tok_bits, lanes = 32 >> tok_bits, at = t0 + j;
+    const bool active = j < m;
+    const unsigned own = active ? sh.keys[at] : 0xFFFFFFFFu;
+    const uint4* const quads = reinterpret_cast<const uint4*>(sh.keys);
+    int rank = 0;
+    const int below = m > 0 ? t0 / 4 : 0, slice_end = min((t0 + m + 3) / 4, n / 4), whole = m > 0 ? n / 4 : 0;  // t0 is a multiple of 16
+    int i = part;
+#pragma unroll 2
+    for (; i < below; i += lanes) {  // tokens before the slice
+      const uint4 v = quads[i];
+      rank += (v.x >= own) + (v.y >= own) + (v.z >= own) + (v.w >= own);
+    }
+#pragma unroll 1
+    for (; i < slice_end; i += lanes) {
+      const uint4 v = quads[i];
+      const int d = at - 4 * i;  // words 0 .. d - 1 come before the token
+      rank += (v.x > own || (v.x == own && d > 0)) + (v.y > own || (v.y == own && d > 1)) + (v.z > own || (v.z == own && d > 2)) +
+              (v.w > own || (v.w == own && d > 3));
+    }
+#pragma unroll 2
+    for (; i < whole; i += lanes) {  // tokens behind it
+      const uint4 v = quads[i];
+      rank += (v.x > own) + (v.y > own) + (v.z > own) + (v.w > own);
+    }
+    for (i = n / 4 * 4 + part; i < n; i += lanes) rank += sh.keys[i] > own || (sh.keys[i] == own && i < at);  // the last few tokens
+    __syncwarp();
+    for (int d = 16; d >> tok_bits; d >>= 1) rank += __shfl_xor_sync(0xFFFFFFFFu, rank, d);
+    const unsigned bits = __ballot_sync(0xFFFFFFFFu, part == 0 && active && rank < k);
+    if (lane == 0 && bits) atomicOr(&sh.kept[(warp << tok_bits) >> 5], bits << ((warp << tok_bits) & 31));
+    if (part == 0 && active && rank >= k && own == kProtectedKey && device_status)
+      atomicOr(device_status, FASTAV_DEV_PROTECT_OVERFLOW);  // more protected tokens than k
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kCountSlice / 32; ++w) count += __popc(sh.kept[w]);
+    if (tid < blocks) remote_store(remote(&sh.kept_of[c], tid), (unsigned)count);
+    cluster_sync();  // the last remote access
+    first = (int)__reduce_add_sync(0xFFFFFFFFu, lane < c ? sh.kept_of[lane] : 0u);
+    if (tid < m && ((sh.kept[tid >> 5] >> lane) & 1u)) {
+      int out = first + __popc(sh.kept[tid >> 5] & ((1u << lane) - 1u));
+#pragma unroll
+      for (int w = 0; w < kCountSlice / 32; ++w) out += w < (tid >> 5) ? __popc(sh.kept[w]) : 0;
+      keep_idx[base + out] = (global_idx ? tok0 : 0) + t0 + tid;
+      picked[out & (kBins - 1)] = (unsigned)(t0 + tid);
+    }
+  } else {
+  // ---- selection by digits: thread t owns the tokens 4 t .. 4 t + 3 of the whole sequence ------------------------------
   const int mine = max(0, min(kPer, n - kPer * tid));
   unsigned x[kPer];
 #pragma unroll
@@ -498,10 +575,8 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   int gt = (int)(before & 0xFFFFu), eq = (int)(before >> 16);
   if (c == 0 && tid == kThreads - 1 && T == kProtectedKey && eq + (int)(both >> 16) > need_eq && device_status)
     atomicOr(device_status, FASTAV_DEV_PROTECT_OVERFLOW);  // more protected tokens than k
-  const bool global_idx = (s.flags & FASTAV_KEEP_IDX_GLOBAL) != 0;
   if (kPer * tid == t0) sh.first_out = gt + min(eq, need_eq);   // t0 is a multiple of 32
   if (kPer * tid == t0 + m) sh.end_out = gt + min(eq, need_eq); // so is the end of a slice, but for the last one's
-  unsigned* const picked = sh.hist;                          // survivor `out` of the sequence is token picked[out % 4096]
   if (kPer * tid >= t0 && kPer * tid < t0 + m) {
 #pragma unroll
     for (int u = 0; u < kPer; ++u) {
@@ -515,12 +590,18 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
       eq += is_eq;
     }
   }
+  if (a.do_gather && m > 0) {
+    __syncthreads();
+    first = sh.first_out;
+    count = (t0 + m == n ? k : sh.end_out) - first;
+  }
+  }
   if (!a.do_gather || m == 0) return;  // (a block without tokens has nothing to copy)
 
   // ---- gather: this block's survivors, 16-byte chunks of all their rows dealt over the threads ---------------------
   __syncthreads();
   const RowShape shape(s, a.rows);
-  const int first = sh.first_out, count = min((t0 + m == n ? k : sh.end_out) - first, s.total_keep - base - first);
+  count = min(count, s.total_keep - base - first);
   if (a.rows.pos_in)
     for (int i = tid; i < count; i += kThreads)
       a.rows.pos_out[base + first + i] = chain_load(a.rows.pos_in + tok0 + picked[(first + i) & (kBins - 1)]);

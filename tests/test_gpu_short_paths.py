@@ -82,6 +82,23 @@ def test_gather_of_batches(batch, n, keep, rows):
     _check([n] * batch, rows, 8, 2, 64, hid=64, keep=keep)
 
 
+# The few-rows kernel ranks a slice's keys by counting while (tokens x tokens of a slice) is small: both sides of that border for
+# clusters of 16, 8, 4 and 2, lengths that are no multiple of 4, one token, all scores equal (the lower index wins) and not.
+@pytest.mark.parametrize("lens", [[1], [2, 3, 5], [513], [767], [768], [769], [511] * 8, [577] * 8, [288] * 16, [289, 7] * 8, [143] * 34, [145, 0] * 17])
+@pytest.mark.parametrize("equal", [False, True])
+def test_selection_by_counting(lens, equal):
+    p = W.random_problem(seed=sum(lens), lens=lens, rows=[min(1, n) for n in lens], keeps=[(2 * n + 2) // 3 for n in lens], num_q_heads=8, num_kv_heads=2,
+                         head_dim=64, hidden=64, duplicate_keys=2)
+    if equal:
+        p.q.zero_()
+    protect = (torch.arange(p.total_tokens) % 3 != 1).to(torch.uint8) if len(lens) % 3 == 1 else None  # now and then more than are kept
+    buf = parity.to_device(p, protect=protect)
+    buf.prune()
+    torch.cuda.synchronize()
+    stats = parity.check_fused_against_oracle(p, buf, parity.oracle_prune(p, protect=protect), protect=protect, what=f"{lens} equal {equal}")
+    assert stats["device_status"] & ~fastav.FASTAV_DEV_PROTECT_OVERFLOW == 0
+
+
 # The compaction keeps the bounds of up to 31 sequences in a warp's lanes; warps with one row, a few, and more than 32.
 @pytest.mark.parametrize("batch,n", [(1, 40), (1, 592), (30, 50), (31, 50), (32, 50), (31, 1000), (33, 1000)])
 def test_gather_bounds_by_lane(batch, n):
