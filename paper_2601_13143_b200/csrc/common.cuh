@@ -111,6 +111,10 @@ cudaError_t launch_select_partials(const Shapes& s, const float* partial, const 
                                    const SelectArgs& t, cudaStream_t stream);
 cudaError_t launch_select_scores(const Shapes& s, const float* scores, const SelectArgs& t, cudaStream_t stream);
 
+// ... and of longer sequences, a slice of the tokens per block (select_long.cu), from partial sums.
+bool long_select_applies(const Shapes& s);
+cudaError_t launch_long_partials(const Shapes& s, const float* partial, const ScoreLeft& left, float* scores_out, const SelectArgs& t, cudaStream_t stream);
+
 // Most blocks of a cluster that the current context can place: 16, or the portable 8.
 int cluster_limit();
 

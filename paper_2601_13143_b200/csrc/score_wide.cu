@@ -741,7 +741,7 @@ cudaError_t run(const Shapes& s, const Workspace& w, const CUtensorMap& k_map, c
   float* partial = reinterpret_cast<float*>(ws + w.partial_off);
   // Partial sums per (KV head, chunk of query rows) -> scores: by the kernel that selects, or here.
   auto finish = [&](int row_chunks, int chunk) -> cudaError_t {
-    if (left && cluster_select_applies(s)) {
+    if (left && (cluster_select_applies(s) || long_select_applies(s))) {
       left->kind = ScoreLeft::kPartials;
       left->row_chunks = row_chunks;
       left->rows_per_chunk = chunk;

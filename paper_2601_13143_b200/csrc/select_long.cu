@@ -1,0 +1,336 @@
+// What follows the tensor-core sweeps on sequences of more than 2,048 tokens, in one kernel: their sums per (KV head, chunk of query
+// rows) and token become scores, in their fixed order, and the k highest are selected (Section 2.2; ties to the lower index,
+// protected tokens always).  One thread-block cluster per sequence, a slice of at most 2,048 tokens per block.
+//
+// The keys stay where they are.  A pass takes 13 bits: each block counts its slice's digits, adds the bins it has to the block that
+// owns them (distributed shared memory), and after a cluster barrier each reads all totals and finds the bin of the k-th largest
+// for itself.  Where that bin holds at most 512 keys every block fetches them and ranks them by counting, else the next pass
+// follows.  Then the blocks tell one another how many of theirs lie above and on the threshold, and write their survivors.
+//
+// Bound: latency, a chain of a dozen steps of which four are cluster barriers.  It saves the kernel that added the sums up; against
+// that and a selection by one block: 3 x 8,001-9,001 tokens with the log-sum-exp given 74.0 -> 72.5 us, 1 to 3 % of a
+// call on a few thousand tokens, 0.3 % of one on 4 x 16,384.  Clusters of 4, 8 or 16 make no difference.  From finished scores
+// (the few-rows path, fastav_select) nothing is saved and one block stays quicker: 4 x 6,554 tokens, one row 109.8 us against 111.7, 32
+// ragged sequences 217.8 against 219.7.
+#include "cluster.cuh"
+#include "common.cuh"
+#include "select_keys.cuh"
+
+namespace fastav {
+namespace {
+
+constexpr int kThreads = 512;
+constexpr int kWarps = kThreads / 32;
+constexpr int kPer = 4;                      // keys per thread
+constexpr int kSlice = kPer * kThreads;      // most tokens of a block
+constexpr int kDigitBits = 13;
+constexpr int kBins = 1 << kDigitBits;
+constexpr int kBinsPerThread = kBins / kThreads;
+constexpr int kListMax = kThreads;           // keys of a bin that are ranked by counting
+constexpr int kLeastSlice = 256;             // tokens per block worth a block
+
+// Two counts to a word: a slice has at most 2,048 keys, a sequence at most 32,768.  In the 34 KB that the compaction's ring leaves, so that its
+// blocks are resident beside these when the selection ends.
+struct alignas(16) LongShared {
+  union {
+    unsigned hist[kBins / 2];  // of the block's slice
+    unsigned all[kListMax];    // the cluster's list
+  };
+  unsigned prot_bits[kSlice / 32];
+  unsigned list[kListMax];
+  unsigned warp_a[kWarps], warp_b[kWarps];
+  unsigned count_of[kMaxCluster];  // keys in each block's list
+  unsigned kept_of[kMaxCluster];   // keys above the threshold (low half) and on it (high half)
+  int index[8];
+  int base, list_n, remaining, bucket, need_eq;
+  unsigned prefix, threshold, own;
+};
+
+struct LongArgs {
+  const float* partial;            // [Hkv * row_chunks][N]
+  int row_chunks, rows_per_chunk;
+  float* scores_out;
+  int blocks, slice_cap;           // blocks of a cluster; tokens of a block that the longest sequence needs
+};
+
+// After LongShared: the scores of the slice, then the totals of the bins this block owns, of the whole cluster.
+__host__ __device__ inline int owned_words(int blocks) { return kBins / 2 / blocks; }
+inline size_t long_bytes(int blocks, int slice_cap) { return sizeof(LongShared) + (size_t)(slice_cap + owned_words(blocks)) * sizeof(unsigned); }
+__host__ __device__ inline int slice_for(int n, int blocks) { return ((n + blocks - 1) / blocks + 31) & ~31; }
+
+__device__ __forceinline__ void remote_add(uint32_t a, unsigned v) {
+  asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ unsigned remote_load(uint32_t a) {
+  unsigned v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint4 remote_load4(uint32_t a) {  // 16-byte aligned
+  uint4 v;
+  asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+  return v;
+}
+
+__global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, LongArgs a, const int32_t* __restrict__ cu_seqlens,
+                                                                  const int32_t* __restrict__ keep_counts, const uint8_t* __restrict__ protect,
+                                                                  const int32_t* __restrict__ q_idx, const int32_t* __restrict__ cu_qlens,
+                                                                  int32_t* __restrict__ keep_idx, int32_t* __restrict__ cu_keep, int32_t* device_status) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  LongShared& sh = *reinterpret_cast<LongShared*>(smem_raw);
+  chain_begin_setup(s);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int blocks = a.blocks, b = (int)blockIdx.x / blocks, c = (int)cluster_rank();
+  unsigned* const keys = reinterpret_cast<unsigned*>(smem_raw + sizeof(LongShared));
+  unsigned* const totals = keys + a.slice_cap;
+  const int owned = owned_words(blocks);  // of an owner: a power of two, at least 256 words
+  auto clear_counts = [&] {
+    for (int i = tid; i < kBins / 8; i += kThreads) reinterpret_cast<uint4*>(sh.hist)[i] = make_uint4(0, 0, 0, 0);
+    for (int i = tid; i < owned / 4; i += kThreads) reinterpret_cast<uint4*>(totals)[i] = make_uint4(0, 0, 0, 0);
+  };
+  clear_counts();
+  if (tid < kSlice / 32) sh.prot_bits[tid] = 0u;
+  if (tid == 0) { sh.base = 0; sh.list_n = 0; }
+  cluster_arrive();  // this block runs and its totals are zero: waited for before the first remote access
+  chain_end_setup(s, cu_seqlens, keep_counts, protect, q_idx, cu_qlens);
+  if (warp == 0) {
+    const int32_t* word = lane < 2 ? cu_seqlens + b + lane : lane < 4 ? cu_qlens + b + lane - 2 : keep_counts + b;
+    if (lane < 5) sh.index[lane] = chain_load(word);
+  }
+  __syncthreads();
+  const Span seq = checked_words(sh.index[0], sh.index[1], s.total_tokens, s.max_seqlen);
+  const Span qrows = checked_words(sh.index[2], sh.index[3], s.total_q, s.max_qlen);
+  int k = sh.index[4];
+  const bool k_clamped = k < 0 || k > seq.count;
+  const int tok0 = seq.first, n = min(seq.count, a.slice_cap * blocks);
+  const int slice = slice_for(n, blocks), t0 = min(n, c * slice), m = min(n - t0, slice);
+  k = k < 0 ? 0 : (k > n ? n : k);
+  const bool lowest = (s.flags & FASTAV_SELECT_LOWEST) != 0;
+
+  pdl_wait();
+  const float* partial = a.partial;
+  pdl_acquire(partial);
+  if (tid == 0 && c == 0 && device_status) {
+    if (seq.bad || qrows.bad) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
+    if (k_clamped) atomicOr(device_status, FASTAV_DEV_K_CLAMPED);
+  }
+  {  // output offset: the clamped keep counts of the sequences before this one, 32 per warp
+    if (warp * 32 < b) {
+      int part = 0;
+#pragma unroll 1
+      for (int i = warp * 32 + lane; i < b; i += kThreads) {
+        const int ni = seq_span(s, cu_seqlens, i).count, ki = chain_load(keep_counts + i);
+        part += ki < 0 ? 0 : min(ki, ni);
+      }
+      part = __reduce_add_sync(0xFFFFFFFFu, part);
+      if (lane == 0 && part) atomicAdd(&sh.base, part);
+    }
+    if (s.flags & FASTAV_PROTECT_QUERY_ROWS)
+      for (int r = tid; r < qrows.count; r += kThreads) {
+        const int j = chain_load(q_idx + qrows.first + r) - t0;  // relative to this block's first token
+        if (j >= 0 && j < m) atomicOr(&sh.prot_bits[j >> 5], 1u << (j & 31));
+      }
+    if (protect)
+      for (int j0 = warp * 32; j0 < m; j0 += kThreads) {  // a warp covers 32 tokens: one word
+        const int j = j0 + lane;
+        const unsigned word = __ballot_sync(0xFFFFFFFFu, j < m && chain_load(protect + tok0 + t0 + j) != 0);
+        if (lane == 0 && word) atomicOr(&sh.prot_bits[j0 >> 5], word);
+      }
+  }
+  const float* const col = partial + tok0 + t0;
+  const int row_chunks = (qrows.count * s.group + a.rows_per_chunk - 1) / a.rows_per_chunk, terms = s.hkv * row_chunks;
+  const float inv = qrows.count > 0 ? 1.0f / ((float)s.hq * (float)qrows.count) : 0.f;
+  for (int j = tid; j < m; j += kThreads) {
+    // Partial i = (KV head, row chunk) in that order; sixteen loads in flight, one running sum in fixed order.
+    float total = 0.f;
+    int g = 0, rc = 0;  // (KV head, row chunk) of the next term, stepped along instead of divided out
+    for (int i0 = 0; i0 < terms; i0 += 16) {
+      float v[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        v[u] = i0 + u < terms ? chain_load(col + (long long)(g * a.row_chunks + rc) * s.total_tokens + j) : 0.f;
+        if (++rc == row_chunks) { rc = 0; ++g; }
+      }
+#pragma unroll
+      for (int u = 0; u < 16; ++u) total += v[u];
+    }
+    const float score = total * inv;
+    a.scores_out[tok0 + t0 + j] = score;
+    keys[j] = __float_as_uint(score);
+  }
+  __syncthreads();
+  const int base = sh.base;
+  if (c == 0 && tid == 0) {
+    cu_keep[b + 1] = base + k;
+    if (b == 0) cu_keep[0] = 0;
+  }
+  // Thread t owns the tokens 4 t .. 4 t + 3 of the slice.
+  const int mine = max(0, min(kPer, m - kPer * tid));
+  unsigned x[kPer];
+  {
+    uint4 v = make_uint4(0, 0, 0, 0);
+    if (mine > 0) v = *reinterpret_cast<const uint4*>(&keys[kPer * tid]);
+    const unsigned raw[kPer] = {v.x, v.y, v.z, v.w}, prot = sh.prot_bits[tid / (32 / kPer)] >> (kPer * (tid % (32 / kPer)));
+    bool any_protected = false;
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const float score = __uint_as_float(raw[u]);
+      x[u] = order_key(lowest ? -score : score);
+      if (x[u] == kProtectedKey) x[u] = kProtectedKey - 1;  // only a NaN pattern lands here
+      if ((prot >> u) & 1u) x[u] = kProtectedKey;
+      any_protected |= u < mine && x[u] == kProtectedKey;
+    }
+    if (k == 0 && any_protected && device_status) atomicOr(device_status, FASTAV_DEV_PROTECT_OVERFLOW);
+  }
+  cluster_wait();
+  if (k == 0) return;  // nothing is kept, protected or not (uniform for the cluster; nothing remote has been touched)
+
+  unsigned prefix = 0u;  // the bits of the k-th largest key fixed so far
+  int remaining = k, bits_left = 32;
+#pragma unroll 1
+  while (bits_left > 0) {
+    const int shift = max(0, bits_left - kDigitBits);
+    const unsigned above_want = __funnelshift_rc(prefix, 0u, bits_left);  // prefix >> bits_left, 0 for 32
+    if (bits_left < 32) {
+      cluster_sync();  // everybody has read the totals
+      clear_counts();
+      cluster_sync();
+    }
+    {
+      unsigned run_digit = kBins, run_len = 0u;  // equal digits of consecutive tokens (typically zeros): one update
+#pragma unroll
+      for (int u = 0; u < kPer; ++u) {
+        if (u < mine && __funnelshift_rc(x[u], 0u, bits_left) == above_want) {
+          const unsigned digit = (x[u] >> shift) & (kBins - 1);
+          if (digit != run_digit) {
+            if (run_len) atomicAdd(&sh.hist[run_digit >> 1], run_len << (16 * (run_digit & 1)));
+            run_digit = digit;
+            run_len = 0u;
+          }
+          ++run_len;
+        }
+      }
+      if (run_len) atomicAdd(&sh.hist[run_digit >> 1], run_len << (16 * (run_digit & 1)));
+    }
+    __syncthreads();
+    constexpr int kWords = kBinsPerThread / 2;
+    const int first_word = tid * kWords, owner = first_word / owned;
+    const uint32_t owner_at = remote(&totals[first_word & (owned - 1)], owner);
+#pragma unroll
+    for (int i = 0; i < kWords; i += 4) {
+      const uint4 v = *reinterpret_cast<const uint4*>(&sh.hist[first_word + i]);
+      if (v.x) remote_add(owner_at + 4 * i, v.x);
+      if (v.y) remote_add(owner_at + 4 * i + 4, v.y);
+      if (v.z) remote_add(owner_at + 4 * i + 8, v.z);
+      if (v.w) remote_add(owner_at + 4 * i + 12, v.w);
+    }
+    cluster_sync();
+    unsigned h[kBinsPerThread], own = 0;
+#pragma unroll
+    for (int i = 0; i < kWords; i += 4) {
+      const uint4 v = remote_load4(owner_at + 4 * i);
+      const unsigned w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        h[2 * (i + j)] = w[j] & 0xFFFFu;
+        h[2 * (i + j) + 1] = w[j] >> 16;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kBinsPerThread; ++i) own += h[i];
+    unsigned above = sum_above<kWarps>(own, sh.warp_a, lane, warp);
+    const unsigned rem = (unsigned)remaining;
+    if (above < rem && rem <= above + own) {  // exactly one thread: its bins from the top
+#pragma unroll
+      for (int i = kBinsPerThread - 1; i >= 0; --i) {
+        if (above < rem && rem <= above + h[i]) {
+          sh.prefix = prefix | ((unsigned)(2 * first_word + i) << shift);
+          sh.remaining = (int)(rem - above);
+          sh.bucket = (int)h[i];
+        }
+        above += h[i];
+      }
+    }
+    __syncthreads();
+    prefix = sh.prefix;
+    remaining = sh.remaining;
+    const int bucket = sh.bucket;
+    bits_left = shift;
+    if (bits_left > 0 && bucket <= kListMax) {  // few keys left in the cluster: everybody fetches them and finds their ranks by counting
+#pragma unroll
+      for (int u = 0; u < kPer; ++u)
+        if (u < mine && (x[u] >> bits_left) == (prefix >> bits_left)) sh.list[atomicAdd(&sh.list_n, 1)] = x[u];
+      __syncthreads();
+      if (tid < blocks) remote_store(remote(&sh.count_of[c], tid), (unsigned)sh.list_n);
+      cluster_sync();
+      if (tid < bucket) {
+        int at = tid, from = 0;
+        while (from < blocks - 1 && at >= (int)sh.count_of[from]) at -= (int)sh.count_of[from++];
+        sh.all[tid] = remote_load(remote(&sh.list[at & (kListMax - 1)], from));
+      }
+      __syncthreads();
+      rank_finish(sh.all, bucket, remaining, tid, &sh.threshold, &sh.need_eq);
+      __syncthreads();
+      prefix = sh.threshold;
+      remaining = sh.need_eq;
+      bits_left = 0;
+    }
+  }
+  const unsigned T = prefix;
+  const int need_eq = remaining;  // how many keys equal to T are kept: the lowest-index ones
+  unsigned both = 0;              // keys above the threshold in the low half, keys equal to it in the high half
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) both += u < mine ? (x[u] > T ? 1u : 0u) + (x[u] == T ? 0x10000u : 0u) : 0u;
+  const unsigned before = sum_before<kWarps>(both, sh.warp_b, lane, warp);
+  if (tid == kThreads - 1) sh.own = before + both;
+  __syncthreads();
+  if (tid < blocks) remote_store(remote(&sh.kept_of[c], tid), sh.own);
+  cluster_sync();  // the last remote access
+  const unsigned there = lane < blocks ? sh.kept_of[lane] : 0u, earlier = lane < c ? there : 0u;
+  int gt = (int)(before & 0xFFFFu) + (int)__reduce_add_sync(0xFFFFFFFFu, earlier & 0xFFFFu);
+  int eq = (int)(before >> 16) + (int)__reduce_add_sync(0xFFFFFFFFu, earlier >> 16);
+  if (c == 0 && warp == 0 && T == kProtectedKey) {
+    const int all_eq = (int)__reduce_add_sync(0xFFFFFFFFu, there >> 16);
+    if (lane == 0 && all_eq > need_eq && device_status) atomicOr(device_status, FASTAV_DEV_PROTECT_OVERFLOW);  // more protected tokens than k
+  }
+  const int offset = ((s.flags & FASTAV_KEEP_IDX_GLOBAL) ? tok0 : 0) + t0 + kPer * tid;
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    const bool is_gt = u < mine && x[u] > T, is_eq = u < mine && x[u] == T;
+    const int out = base + gt + min(eq, need_eq);
+    if ((is_gt || (is_eq && eq < need_eq)) && out < s.total_keep) keep_idx[out] = offset + u;
+    gt += is_gt;
+    eq += is_eq;
+  }
+}
+
+// Blocks per sequence, as many as run at once and have a slice worth it; 0 where the longest sequence does not fit.
+int blocks_for(const Shapes& s) {
+  const int blocks = cluster_blocks(s.batch, s.max_seqlen, kLeastSlice, s.cluster_limit);
+  return blocks >= 2 && slice_for(s.max_seqlen, blocks) <= kSlice ? blocks : 0;
+}
+
+}  // namespace
+
+bool long_select_applies(const Shapes& s) { return !cluster_select_applies(s) && blocks_for(s) > 0; }
+
+cudaError_t launch_long_partials(const Shapes& s, const float* partial, const ScoreLeft& left, float* scores_out, const SelectArgs& t, cudaStream_t stream) {
+  LongArgs a{};
+  a.partial = partial;
+  a.row_chunks = left.row_chunks;
+  a.rows_per_chunk = left.rows_per_chunk;
+  a.scores_out = scores_out;
+  a.blocks = blocks_for(s);
+  a.slice_cap = slice_for(s.max_seqlen, a.blocks);
+  cudaError_t e = once_per_context([] {
+    const cudaError_t f = cudaFuncSetAttribute(select_long_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)long_bytes(2, kSlice));
+    return f == cudaSuccess ? cudaFuncSetAttribute(select_long_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : f;
+  });
+  if (e != cudaSuccess) return e;
+  e = launch_chained_cluster(select_long_kernel, dim3(s.batch * a.blocks), dim3(kThreads), a.blocks, long_bytes(a.blocks, a.slice_cap), stream, s, a, t.cu_seqlens,
+                             t.keep_counts, t.protect, t.q_idx, t.cu_qlens, t.keep_idx, t.cu_keep, t.device_status);
+  count_launches(1);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+}  // namespace fastav

@@ -1,0 +1,30 @@
+"""Scores and selection of sequences beyond 2,048 tokens from the sweeps' partial sums by clusters (select_long.cu), against the
+oracle: ends of the range and of a block's slice, clusters of 16 to 2 and the paths next to them (too many sequences, too
+long), keys that share one bin of every pass, more protected tokens than are kept, empty and short sequences beside long ones."""
+import pytest
+import torch
+
+import parity
+from paper_2601_13143_b200 import fastav, workloads as W
+
+pytestmark = pytest.mark.gpu
+
+LENS = [[2049], [2050, 1, 0, 2111], [4097], [8191, 8193], [16384], [32768], [32769], [2600] * 7, [2600] * 8, [2051] * 15, [2051] * 16, [2500, 0, 1] * 11,
+        [2100] * 34, [4097] * 34, [2049] * 75]
+
+
+@pytest.mark.parametrize("lens", LENS, ids=lambda v: f"{len(v)}x{max(v)}")
+@pytest.mark.parametrize("equal", [False, True])
+def test_select_from_sums(lens, equal):
+    rows = [min(9, n) for n in lens]
+    shares = [0.4, 0.0, 1.0, 0.01, 0.9]
+    p = W.random_problem(seed=sum(lens), lens=lens, rows=rows, keeps=[min(n, int(round(shares[i % 5] * n))) for i, n in enumerate(lens)], num_q_heads=4,
+                         num_kv_heads=2, head_dim=64, hidden=64, duplicate_keys=2)
+    if equal:  # every token of a sequence that all its rows see has the same score
+        p.q.zero_()
+    protect = (torch.arange(p.total_tokens) % 31 == 5).to(torch.uint8) if len(lens) % 2 else None
+    buf = parity.to_device(p, protect=protect)
+    buf.prune()
+    torch.cuda.synchronize()
+    stats = parity.check_fused_against_oracle(p, buf, parity.oracle_prune(p, protect=protect), protect=protect, what=f"{lens} equal {equal}")
+    assert stats["device_status"] & ~fastav.FASTAV_DEV_PROTECT_OVERFLOW == 0
