@@ -17,8 +17,8 @@
 // Bound: latency.  Nothing here is long, so what counts is the number of dependent steps: every index array is asked for
 // at once, the keys before anything that is only needed later, every reduction is spread over as many lanes as keep its
 // order fixed, and nothing is computed by an owner that would have to publish it.  A prune call with one
-// scored row (28 / 4 heads of 128, hidden 3,584, 80 % kept), this kernel and the compaction against the five kernels it stands
-// for: 1 x 512 tokens 12.0 us instead of 20.7, 1 x 1,024 14.9 / 24.8, 1 x 2,048 18.3 / 28.8, 8 x 512 24.3 / 32.8.
+// scored row (28 / 4 heads of 128, hidden 3,584, 80 % kept), this kernel and the compaction as they were first against the five kernels
+// they stand for: 1 x 512 tokens 12.0 us instead of 20.7, 1 x 1,024 14.9 / 24.8, 1 x 2,048 18.3 / 28.8, 8 x 512 24.3 / 32.8.
 //
 // A sequence's scores depend on its length only, not on the cluster's size or the batch, and equal keys get bit-equal
 // scores: all sums have a fixed order.
