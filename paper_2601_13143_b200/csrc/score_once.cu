@@ -388,7 +388,7 @@ bool once_plan(const Shapes& s, bool lse_given, OncePlan* plan) {
   if (tiles > kMaxTiles) return false;
   const long long clusters = (long long)s.batch * s.hkv * plan->row_tiles;
   // Key tiles per block: the least time of all rounds (in quarters of a microsecond): a round of clusters that run at once takes
-  // some 6 us and 3.75 us per key tile of a block.  One round is always the better way (1 x 2,048 tokens, 32 rows, 28 / 4 heads:
+  // some 6 us and 3.75 us per key tile of a block (as fitted with exponentials in both passes; about 3.25 us since).  One round is always the better way (1 x 2,048 tokens, 32 rows, 28 / 4 heads:
   // 20.7 us with 2 key tiles per block in one round, 26.5 with 1 in two; the two sweeps 31.0).  Several rounds are compared with
   // the two sweeps: about 19 us, and per SM and key tile 2.25 us for every 128 rows of the first and 128 columns of the second.
   // Prune of 32 x 512 tokens, 32 rows: 60.0 against 71.1 us (32 / 8 heads: 66.8 against 83.4), 15 x 1,024: 57.9 / 64.5, but
