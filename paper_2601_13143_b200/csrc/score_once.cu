@@ -4,12 +4,12 @@
 // owns one tile of 128 query rows of one KV head, its blocks share out the keys, and a block's logits -- 128 rows x up to 512
 // keys in fp32 -- stay in its 256 KB of tensor memory.  So
 //
-//   S = Q K^T per key tile (tcgen05.mma, operands by TMA), read once for (max, sum 2^(z - max)) per row and key tile, and the
-//   2^(z - max) put back in its place; the blocks exchange the sums through distributed shared memory (one cluster barrier); each
-//   block then works out its rows' log2-sum-exp2 and reads again: 2^(z - max) 2^(max - lse), summed over the 128 rows of every
-//   key by a butterfly that leaves one key per lane -> partial[KV head, row tile][token], which the selecting kernel (prune_few.cu,
-//   select_long.cu) adds up.  (With exponentials in both passes, prune of 1 x 2,048 tokens, 64 rows: 23.4 us instead of 21.9; the error against
-//   64 bits is the same, 0.6 to 1.2e-7 in the 2-norm.)  Where the caller hands the log-sum-exp in, S itself is read in the second pass.
+//   S = Q K^T per key tile (tcgen05.mma, operands by TMA), read once for the sum of 2^(z - top) per row and group of 32 keys, with the
+//   2^(z - top) put back in its place; the blocks exchange the sums through distributed shared memory (one cluster barrier); each block
+//   then adds its rows' sums up and reads again: 2^(z - top) 2^(top - lse), summed over the 128 rows of every key by a butterfly that
+//   leaves one key per lane -> partial[KV head, row tile][token], which the selecting kernel (prune_few.cu, select_long.cu) adds up.
+//   (With exponentials in both passes, prune of 1 x 2,048 tokens, 64 rows: 23.4 us instead of 22.5; the error against 64 bits is the same
+//   on the whole, 0.6 to 1.8e-7 in the 2-norm.)  Where the caller hands the log-sum-exp in, S itself is read in the second pass.
 //
 // Two kernels (this and the selection) replace five (two sweeps, merge, per-token sums, selection).  Bound: latency, the
 // chip is far from full.  Prune calls against the two-sweep path (28 / 4 heads, half the tokens kept): 32 rows on 1 x 1,024
@@ -45,8 +45,9 @@ struct alignas(16) Control {
   int index[4];
   int limit[kTile];                            // last key each row may see (-1: no such row)
   float neg_lse[kTile];
-  float2 part[4][kBlockTiles][kTile];          // (max, sum) per column group, key tile, row
+  float2 part[4][kBlockTiles][kTile];          // (top, sum of 2^(z - top)) per column group, key tile, row
   float2 run[4][kTile];                        // ... per run of the sequence's key tiles
+  float2 fold[kTile];                          // per row: the second factor is 2^(top - x) y
   float2 stats[kMaxTiles][kTile];              // per key tile of the sequence: written by all blocks of the cluster
   float colsum[kBlockTiles][4][kTile];         // per key tile and 32-row quarter, the sums of every key
 };
@@ -80,6 +81,70 @@ __device__ __forceinline__ float transpose_sum(float (&v)[32], int lane) {
     }
   }
   return v[0];
+}
+
+// ---- 2^z in two factors ------------------------------------------------------------------------------
+// The first pass leaves 2^(z - top) of every key, the second multiplies by 2^(top - lse).  `top` differs from one group of 32 keys to
+// the next, and equal keys have to come out bit-equal all the same (with the group's own maximum taken off they differed by 1 to 3 units in the
+// last place).  So nothing but a power of two is taken off: z = n + f, n the nearest integer and f rounded once, neither of which
+// depends on `top`; 2^f has n - top added to its exponent; the row's factor is one over its sum with top - (the largest top) added; and
+// their product is rounded once, to the same value wherever the key stands.  `top` is even, so that n is rounded the same way with it and
+// without it, and above every z of its group, so that the first factor is at most 1.
+//   Small values: the first factor stops at 2^-125, the second is at most 4 kLift, and their product is flushed below 2^-126: whichever
+// factor would be too small, the key adds 0 in every group, as hidden keys do.  (kLift is undone in the partial sums.)
+//   The integer's part costs 0.5 us of the 22.5 at 1 x 2,048 tokens.  Without it as long as all logits of a group are within 2^+-63, 22.1,
+// and 24.2 to 25.2 where they are not.
+constexpr float kLift = 0.0625f;
+constexpr float kToInteger = 12582912.f;  // 1.5 x 2^23: the sum with it is rounded to an integer, which its low bits hold
+constexpr float kMostTop = 65536.f;       // |top| up to which the kernel's own form is exact
+
+__device__ __forceinline__ float top_of(float zmax) { return 2.f * floorf(0.5f * zmax) + 2.f; }
+
+// 2^d of an integer d <= 127, 0 below 2^-126 and for NaN (the sum's low bits are d + 127).
+__device__ __forceinline__ float power_of_two(float d) { return __int_as_float(__float_as_int(fmaxf(d, -127.f) + (kToInteger + 127.f)) << 23); }
+
+// 2^(v * scale - top) for any v and any top above: NaN where the logit is not a number or +infinity.
+__device__ __forceinline__ float exp_below(float v, float scale, float top) {
+  const float z = v * scale;
+  const bool exact = fabsf(z) < 4194304.f;  // (beyond, z is a multiple of 1/2)
+  const float n = exact ? __fmaf_rn(v, scale, kToInteger) - kToInteger : rintf(z);
+  const float f = exact ? __fmaf_rn(v, scale, -n) : z - n, d = n - top;
+  const float p = d >= -125.f ? ptx::ex2_approx(f) * power_of_two(d) : 0.f;
+  return z < INFINITY ? p : __int_as_float(0x7FFFFFFF);
+}
+
+// The first pass over a group of 32 keys where a row of the warp has logits that are far from 0, infinite or not a number: (top, sum).
+// Rare, and short code rather than fast.
+__device__ __forceinline__ float2 exponentials_far(uint32_t at, int bound, float scale) {
+  float m = -INFINITY;  // (what is not a number is left out)
+#pragma unroll 1
+  for (int j0 = 0; j0 < 32; j0 += 8) {
+    uint32_t v[8];
+    ptx::tmem_ld8(at + j0, v);
+    ptx::tmem_ld_wait_for(v);
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (j0 + j <= bound) m = fmaxf(m, __uint_as_float(v[j]));
+  }
+  const float top = m == -INFINITY ? 0.f : top_of(m * scale);
+  float2 sum = make_float2(0.f, 0.f);
+#pragma unroll 1
+  for (int j0 = 0; j0 < 32; j0 += 8) {
+    uint32_t v[8];
+    float p[8];
+    ptx::tmem_ld8(at + j0, v);
+    ptx::tmem_ld_wait_for(v);
+#pragma unroll
+    for (int j = 0; j < 8; j += 2) {
+      p[j] = j0 + j <= bound ? exp_below(__uint_as_float(v[j]), scale, top) : 0.f;
+      p[j + 1] = j0 + j + 1 <= bound ? exp_below(__uint_as_float(v[j + 1]), scale, top) : 0.f;
+      sum = __fadd2_rn(sum, make_float2(p[j], p[j + 1]));
+    }
+    __syncwarp();
+    ptx::tmem_st8(at + j0, p);
+  }
+  const float total = sum.x + sum.y;
+  return make_float2(m == -INFINITY && total == total ? -INFINITY : top, total);
 }
 
 template <int DIM>
@@ -195,6 +260,7 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
   uint32_t lane_addr = 0;
   const float scale = s.scale_log2;
   const float2 sc = make_float2(scale, scale);
+  const float inv_scale = 1.f / scale;
   bool ok = true;
   int limit = -1;
   if (warp >= 2) {
@@ -236,25 +302,32 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
           for (int j = 0; j < 32; ++j)
             if (j > bound) v[j] = 0xFF800000u;  // -inf
         }
-        float m0 = -INFINITY, m1 = -INFINITY;
+        float m0 = -INFINITY, m1 = -INFINITY;  // not a number if a logit is not
 #pragma unroll
         for (int j = 0; j < 32; j += 4) {
-          m0 = fmaxf(m0, fmaxf(__uint_as_float(v[j]), __uint_as_float(v[j + 1])));
-          m1 = fmaxf(m1, fmaxf(__uint_as_float(v[j + 2]), __uint_as_float(v[j + 3])));
+          m0 = ptx::max_nan(m0, __uint_as_float(v[j]), __uint_as_float(v[j + 1]));
+          m1 = ptx::max_nan(m1, __uint_as_float(v[j + 2]), __uint_as_float(v[j + 3]));
         }
-        const float m = fmaxf(m0, m1), shift = m == -INFINITY ? 0.f : -m * scale;
-        float2 sum = make_float2(0.f, 0.f);
-        float p[32];
+        const float m = ptx::max_nan(m0, m1, -INFINITY), top = m == -INFINITY ? 0.f : top_of(m * scale), least = (top - 125.f) * inv_scale;
+        if (__all_sync(0xFFFFFFFFu, m == -INFINITY || (fabsf(top) <= kMostTop && least < m))) {
+          const float2 shift = make_float2(kToInteger - top, kToInteger - top);
+          float2 sum = make_float2(0.f, 0.f);
+          float p[32];
 #pragma unroll
-        for (int j = 0; j < 32; j += 2) {
-          const float2 z = __ffma2_rn(make_float2(__uint_as_float(v[j]), __uint_as_float(v[j + 1])), sc, make_float2(shift, shift));
-          p[j] = ptx::ex2_approx(z.x);
-          p[j + 1] = ptx::ex2_approx(z.y);
-          sum = __fadd2_rn(sum, make_float2(p[j], p[j + 1]));
+          for (int j = 0; j < 32; j += 2) {
+            const float2 x = make_float2(fmaxf(__uint_as_float(v[j]), least), fmaxf(__uint_as_float(v[j + 1]), least));
+            const float2 to = __ffma2_rn(x, sc, shift);                                          // kToInteger + n - top
+            const float2 f = __ffma2_rn(x, sc, __ffma2_rn(to, make_float2(-1.f, -1.f), shift));  // z - n
+            p[j] = __uint_as_float(__float_as_uint(ptx::ex2_approx(f.x)) + (__float_as_uint(to.x) << 23));
+            p[j + 1] = __uint_as_float(__float_as_uint(ptx::ex2_approx(f.y)) + (__float_as_uint(to.y) << 23));
+            sum = __fadd2_rn(sum, make_float2(p[j], p[j + 1]));
+          }
+          ctl.part[cg][t][row_in] = make_float2(m == -INFINITY ? -INFINITY : top, sum.x + sum.y);
+          __syncwarp();  // rows differ in `bound`; the tcgen05 instructions need the whole warp
+          ptx::tmem_st32(lane_addr + t * kTile, p);  // in place of the logits: the second pass needs no exponentials
+        } else {
+          ctl.part[cg][t][row_in] = exponentials_far(lane_addr + t * kTile, bound, scale);
         }
-        ctl.part[cg][t][row_in] = make_float2(m * scale, sum.x + sum.y);
-        __syncwarp();  // rows differ in `bound`; the tcgen05 instructions that follow need the whole warp
-        ptx::tmem_st32(lane_addr + t * kTile, p);  // in place of the logits: the second pass needs no exponentials
       }
     }
   }
@@ -271,7 +344,7 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const float2 p = ctl.part[i][t][row];
-          if (p.x > -INFINITY) l += p.y * ptx::ex2_approx(p.x - m);
+          l += p.y * power_of_two(p.x - m);
         }
         for (int q = 0; q < blocks; ++q) remote_store2(remote(&ctl.stats[t0 + t][row], q), __float_as_uint(m), __float_as_uint(l));
       }
@@ -287,7 +360,7 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
       for (int t = j; t < tiles; t += 4) m = fmaxf(m, ctl.stats[t][row].x);
       for (int t = j; t < tiles; t += 4) {
         const float2 p = ctl.stats[t][row];
-        if (p.x > -INFINITY) l += p.y * ptx::ex2_approx(p.x - m);
+        l += p.y * power_of_two(p.x - m);
       }
       ctl.run[j][row] = make_float2(m, l);
       epilogue_sync();
@@ -298,14 +371,14 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const float2 p = ctl.run[i][ethread];
-          if (p.x > -INFINITY) total += p.y * ptx::ex2_approx(p.x - mm);
+          total += p.y * power_of_two(p.x - mm);
         }
-        ctl.neg_lse[ethread] = total > 0.f && ethread < rows_here ? -(mm + __log2f(total)) : -INFINITY;
+        ctl.fold[ethread] = make_float2(mm, total > 0.f && ethread < rows_here ? kLift * __frcp_rn(total) : 0.f);
       }
       epilogue_sync();
     }
     const float nl = ctl.neg_lse[row_in];
-    const float2 nl2 = make_float2(nl, nl);
+    const float2 nl2 = make_float2(nl, nl), fold = ctl.fold[row_in];
     __syncwarp();
     if (!lse_in) ptx::tmem_st_wait();
     for (int t = 0; t < mine; ++t) {
@@ -316,10 +389,9 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
       ptx::tmem_ld_wait_for(v);
       float p[32];
       if (!lse_in) {
-        const float m = ctl.part[cg][t][row_in].x;  // what the first pass took off; where a key is hidden it left 0
-        const float w = m > -INFINITY ? ptx::ex2_approx(m + nl) : 0.f;
+        const float w = fold.y * power_of_two(ctl.part[cg][t][row_in].x - fold.x);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) p[j] = __uint_as_float(v[j]) * w;
+        for (int j = 0; j < 32; ++j) p[j] = ptx::mul_ftz(__uint_as_float(v[j]), w);
       } else {
         const int bound = limit - ((t0 + t) * kTile + cg * 32);
 #pragma unroll
@@ -341,7 +413,7 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
     const int t = ethread >> 7, col = ethread & (kTile - 1), key = (t0 + t) * kTile + col;
     if (ok && t < mine && key < n)
       partial[(long long)(g * row_tiles + rt) * s.total_tokens + seq.first + key] =
-          (ctl.colsum[t][0][col] + ctl.colsum[t][1][col]) + (ctl.colsum[t][2][col] + ctl.colsum[t][3][col]);
+          ((ctl.colsum[t][0][col] + ctl.colsum[t][1][col]) + (ctl.colsum[t][2][col] + ctl.colsum[t][3][col])) * (lse_in ? 1.f : 1.f / kLift);
   }
 
   // ---- teardown: everybody meets here, whatever happened above ------------------------------------
