@@ -232,8 +232,12 @@ compact_rows_bulk_kernel(Shapes s, RowStreams t, const int32_t* __restrict__ kee
     }
     if (loaded & (1u << (i & 31))) {
       const uint32_t bar = ptx::smem_u32(&full[warp][i % kBulkStages]);
-      if (!ptx::mbar_wait_bounded(bar, (i / kBulkStages) & 1, &abort_flag)) {
+      // One answer for the warp: source_of needs all lanes, and a bound shuffled from one that had left would be any number.
+      if (!ptx::mbar_wait_warp(bar, (i / kBulkStages) & 1, &abort_flag)) {
         if (lane == 0 && device_status) atomicOr(device_status, FASTAV_DEV_WAIT_EXPIRED);
+        int never = 0;  // the copies in flight write into this block's shared memory: they are waited for before it may exit
+        for (int r = i; r <= min(next, my_rows - 1); ++r)
+          if (loaded & (1u << (r & 31))) ptx::mbar_wait_bounded(ptx::smem_u32(&full[warp][r % kBulkStages]), (r / kBulkStages) & 1, &never);
         break;
       }
       if (active) bulk_store(seg.out + (long long)(first + i * step) * seg.out_stride, ring + (i % kBulkStages) * row_bytes + seg.slot_off, seg.bytes);

@@ -1,0 +1,21 @@
+"""What can only be read off the kernels' sources: a wait that gives up needs half a second of a copy that never ends, which no test may
+bring about."""
+import os
+import re
+
+import pytest
+
+from paper_2601_13143_b200 import build
+
+# Kernels whose warps vote or shuffle after a bounded wait.  mbar_wait_bounded answers every lane for itself: lanes that leave on its
+# answer are missing in the next full-mask operation.
+WHOLE_WARP = ["compact.cu"]
+
+
+@pytest.mark.parametrize("name", WHOLE_WARP)
+def test_a_warp_that_votes_decides_on_one_answer(name):
+    with open(os.path.join(build.CSRC, name)) as f:
+        source = re.sub(r"//[^\n]*", "", f.read())
+    assert "_sync(0xFFFFFFFFu" in source and "mbar_wait_warp(" in source
+    for decision in re.findall(r"(?:if \(!?|= |while \(!?|&& !?)ptx::mbar_wait_bounded\(", source):
+        pytest.fail(f"{name} decides on the answer of a single lane: {decision}")
