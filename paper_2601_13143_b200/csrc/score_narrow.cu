@@ -93,9 +93,10 @@ score_narrow_logits_kernel(Shapes s, const uint16_t* __restrict__ q, const int32
     const int pieces_per_token = packed ? 1 : heads_per_block;
     const uint32_t piece_bytes = packed ? row_bytes : DIM * 2;
     bool ok = true;
-    for (int it = 0; it < passes * slots && ok; ++it) {
+    int it = 0;
+    for (; it < passes * slots; ++it) {
       const int stage = it % kStages;
-      ok = ptx::mbar_wait_bounded(ptx::smem_u32(&empty[stage]), ((it / kStages) & 1) ^ 1u, &abort_flag);
+      ok = ptx::mbar_wait_warp(ptx::smem_u32(&empty[stage]), ((it / kStages) & 1) ^ 1u, &abort_flag);
       if (!ok) break;
       const int key = key_begin + (it % slots) * kSlotKeys;
       const int tokens = min(kSlotKeys, key_end - key);
@@ -108,7 +109,11 @@ score_narrow_logits_kernel(Shapes s, const uint16_t* __restrict__ q, const int32
                   k + (long long)(tok0 + key + t) * s.k_st + (long long)(head0 + h) * s.k_sh, piece_bytes, bar);
       }
     }
-    if (!ok && lane == 0 && device_status) atomicOr(device_status, FASTAV_DEV_WAIT_EXPIRED);
+    if (!ok) {
+      if (lane == 0 && device_status) atomicOr(device_status, FASTAV_DEV_WAIT_EXPIRED);
+      int never = 0;  // the copies in flight write into this block's shared memory: they are waited for before it may exit
+      for (int t = max(0, it - kStages); t < it; ++t) ptx::mbar_wait_bounded(ptx::smem_u32(&full[t % kStages]), (t / kStages) & 1, &never);
+    }
     return;
   }
 
@@ -144,7 +149,7 @@ score_narrow_logits_kernel(Shapes s, const uint16_t* __restrict__ q, const int32
 
     for (int sl = 0; sl < slots; ++sl, ++it) {
       const int stage = it % kStages;
-      if (!ptx::mbar_wait_bounded(ptx::smem_u32(&full[stage]), (it / kStages) & 1, &abort_flag)) {
+      if (!ptx::mbar_wait_warp(ptx::smem_u32(&full[stage]), (it / kStages) & 1, &abort_flag)) {  // (one answer: the shuffles need all lanes)
         // the producer may have issued everything and left already: report here as well
         if ((threadIdx.x & 31) == 0 && device_status) atomicOr(device_status, FASTAV_DEV_WAIT_EXPIRED);
         return;

@@ -9,7 +9,7 @@ from paper_2601_13143_b200 import build
 
 # Kernels whose warps vote or shuffle after a bounded wait.  mbar_wait_bounded answers every lane for itself: lanes that leave on its
 # answer are missing in the next full-mask operation.
-WHOLE_WARP = ["compact.cu"]
+WHOLE_WARP = ["compact.cu", "score_narrow.cu"]
 
 
 @pytest.mark.parametrize("name", WHOLE_WARP)
