@@ -81,7 +81,8 @@ extern "C" {
 #define FASTAV_DEV_BAD_INDEX 8        /* fastav_compact met a keep_idx entry outside its sequence and skipped that row */
 #define FASTAV_DEV_SHAPE_MISMATCH 16  /* cu_seqlens / cu_qlens on the device disagree with the host scalars of params (a sequence
                                          longer than max_seqlen, a batch longer than total_tokens, more scored rows than max_qlen /
-                                         total_q, more work than the launch was sized for): the excess was left out */
+                                         total_q, more survivors than total_keep, more work than the launch was sized for): the
+                                         excess was left out */
 #define FASTAV_DEV_SLOW_PATH 32       /* informational: fastav_score could not describe q or k to the tensor-memory-accelerator
                                          (tensor-map encoding refused) and ran its CUDA-core tiles instead, much more slowly */
 

@@ -435,7 +435,9 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   if (c == 0 && tid == 0) {
     cu_keep[b + 1] = base + k;
     if (b == 0) cu_keep[0] = 0;
+    if (base + k > s.total_keep && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
   }
+  const int room = s.total_keep - base;  // of the caller's keep list, from this sequence on
   if (k == 0) {  // nothing is kept, protected or not (uniform for the cluster)
     if (c == 0 && device_status)
       for (int j = tid; j < n; j += kThreads)
@@ -491,7 +493,7 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
       int out = first + __popc(sh.kept[tid >> 5] & ((1u << lane) - 1u));
 #pragma unroll
       for (int w = 0; w < kCountSlice / 32; ++w) out += w < (tid >> 5) ? __popc(sh.kept[w]) : 0;
-      keep_idx[base + out] = (global_idx ? tok0 : 0) + t0 + tid;
+      if (out < room) keep_idx[base + out] = (global_idx ? tok0 : 0) + t0 + tid;
       picked[out & (kBins - 1)] = (unsigned)(t0 + tid);
     }
   } else {
@@ -583,7 +585,7 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
       const bool is_gt = x[u] > T, is_eq = x[u] == T;
       if (u < mine && (is_gt || (is_eq && eq < need_eq))) {
         const int out = gt + min(eq, need_eq), j = kPer * tid + u;
-        keep_idx[base + out] = (global_idx ? tok0 : 0) + j;
+        if (out < room) keep_idx[base + out] = (global_idx ? tok0 : 0) + j;
         picked[out & (kBins - 1)] = (unsigned)j;
       }
       gt += is_gt;
@@ -601,7 +603,7 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   // ---- gather: this block's survivors, 16-byte chunks of all their rows dealt over the threads ---------------------
   __syncthreads();
   const RowShape shape(s, a.rows);
-  count = min(count, s.total_keep - base - first);
+  count = min(count, room - first);
   if (a.rows.pos_in)
     for (int i = tid; i < count; i += kThreads)
       a.rows.pos_out[base + first + i] = chain_load(a.rows.pos_in + tok0 + picked[(first + i) & (kBins - 1)]);

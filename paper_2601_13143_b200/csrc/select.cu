@@ -140,6 +140,7 @@ __global__ void __launch_bounds__(kThreads) select_topk_kernel(Shapes s, const f
   if (tid == 0) {
     cu_keep[b + 1] = base + k;
     if (b == 0) cu_keep[0] = 0;
+    if (base + k > s.total_keep && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
     if (n_protected > k && device_status) atomicOr(device_status, FASTAV_DEV_PROTECT_OVERFLOW);
   }
   if (k == 0 || n == 0) return;
@@ -295,8 +296,8 @@ __global__ void __launch_bounds__(kThreads) select_topk_kernel(Shapes s, const f
     const unsigned key = keys[slot<kKeysInShared>(j)];
     const bool gt = key > T, eq = key == T;
     if (gt || (eq && (int)eq_before < need_eq)) {
-      const int out = (int)gt_before + min((int)eq_before, need_eq);
-      keep_idx[base + out] = global_idx ? tok0 + j : j;
+      const int out = base + (int)gt_before + min((int)eq_before, need_eq);
+      if (out < s.total_keep) keep_idx[out] = global_idx ? tok0 + j : j;
     }
     gt_before += gt;
     eq_before += eq;

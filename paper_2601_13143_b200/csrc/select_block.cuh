@@ -139,6 +139,7 @@ __device__ __forceinline__ void select_sequence_blocked(SelectBlockedShared<THRE
   if (tid == 0) {
     cu_keep[b + 1] = base + k;
     if (b == 0) cu_keep[0] = 0;
+    if (base + k > s.total_keep && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
     if (n_protected > k && device_status) atomicOr(device_status, FASTAV_DEV_PROTECT_OVERFLOW);
   }
   if (k == 0 || n == 0) return;  // uniform for the group
@@ -291,8 +292,8 @@ __device__ __forceinline__ void select_sequence_blocked(SelectBlockedShared<THRE
   for (int u = 0; u < mine; ++u) {
     const unsigned x = key[u];
     const bool gt = x > T, eq = x == T;
-    if (gt || (eq && (int)eq_before < need_eq))
-      keep_idx[base + (int)gt_before + min((int)eq_before, need_eq)] = global_idx ? tok0 + j_first + u : j_first + u;
+    const int out = base + (int)gt_before + min((int)eq_before, need_eq);
+    if ((gt || (eq && (int)eq_before < need_eq)) && out < s.total_keep) keep_idx[out] = global_idx ? tok0 + j_first + u : j_first + u;
     gt_before += gt;
     eq_before += eq;
   }

@@ -163,6 +163,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
   if (c == 0 && tid == 0) {
     cu_keep[b + 1] = base + k;
     if (b == 0) cu_keep[0] = 0;
+    if (base + k > s.total_keep && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
   }
   // Thread t owns the tokens 4 t .. 4 t + 3 of the slice.
   const int mine = max(0, min(kPer, m - kPer * tid));

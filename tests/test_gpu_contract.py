@@ -208,3 +208,30 @@ def test_a_key_that_is_not_a_number_shows_in_the_attention_map():
         fastav.fastav_rollout_begin(n, state)
         fastav.fastav_rollout_layer(p, q, bad, 0.5, 0, state, ws, map_out_opt=out)
         assert out[j:, j].isnan().all(), j
+
+
+# More survivors than total_keep says, on every path that writes a keep list: from the keys by counting and by digits, from partial
+# sums of short and of long sequences, after the sweeps of more sequences than clusters run at once, from scores (three layouts).
+@pytest.mark.parametrize("lens,rows", [([500, 40], 1), ([2048, 40], 1), ([1000, 40], 8), ([2600, 40], 9), ([40000, 40], 9), ([2600, 40], 1), ([40000, 40], 1),
+                                       ([60000, 40], 1)])
+@pytest.mark.parametrize("short", [1, 15, 60])  # of the second sequence's 30 survivors one, half, or all of them and some of the first's
+def test_survivors_beyond_the_capacity_are_left_out(lens, rows, short):
+    """The buffers hold all survivors, the parameters promise fewer: what lies beyond stays as it was, and the bit says so."""
+    p = W.random_problem(sum(lens) + rows, lens, [rows] * len(lens), [lens[0] // 2, 30], 4, 2, 64, 16)
+    buf = parity.to_device(p)
+    kept = sum(p.keep_counts.tolist())
+    buf.params.total_keep, buf.params.max_keep = kept - short, min(lens[0] // 2, kept - short)
+    outputs = ("keep_idx", "hidden_out", "pos_out", "k_out", "v_out")
+    for name in outputs:
+        getattr(buf, name).fill_(-7)
+    buf.prune()
+    torch.cuda.synchronize()
+    assert int(buf.device_status) == fastav.FASTAV_DEV_SHAPE_MISMATCH
+    idx, cu = oracle.select(buf.scores.cpu().numpy(), p.cu_seqlens.numpy(), p.keep_counts.numpy())
+    assert buf.cu_keep.cpu().tolist() == cu.tolist()
+    assert np.array_equal(buf.keep_idx.cpu().numpy()[:kept - short], idx[:kept - short])
+    rows_of = parity.gather_rows(p, idx, cu)
+    for name in outputs[1:]:
+        parity.assert_bits_equal(getattr(buf, name)[:kept - short], rows_of[name.removesuffix("_out")][:kept - short], name)
+    for name in outputs:
+        assert bool((getattr(buf, name)[kept - short:kept] == -7).all()), name
