@@ -71,7 +71,8 @@ struct FewArgs {
 // Short sequences are selected by counting: every block ranks its own slice's keys against all keys of the sequence, at most this
 // many comparisons and tokens per block.  In place of five block-wide steps, one with no barrier inside and another exchange over the
 // cluster; the comparisons grow with the square of the length.  From all keys to the keep list, by digits / by counting (time stamps):
-// 512 tokens 2.3 / 1.9 us, 744 2.3 / 2.1, 820 2.4 / 2.9, 1,024 2.7 / 3.2.
+// 512 tokens 2.3 / 1.9 us, 744 2.3 / 2.1, 820 2.4 / 2.9, 1,024 2.7 / 3.2 (by counting another 0.25 less from 513 to 768 since warps without
+// tokens leave the comparisons out).
 constexpr int kCountPairs = 36 << 10, kCountSlice = 256;
 
 struct alignas(16) FewShared {
@@ -457,8 +458,8 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
     const unsigned own = active ? sh.keys[at] : 0xFFFFFFFFu;
     const uint4* const quads = reinterpret_cast<const uint4*>(sh.keys);
     int rank = 0;
-    const int below = m > 0 ? t0 / 4 : 0, slice_end = min((t0 + m + 3) / 4, n / 4), whole = m > 0 ? n / 4 : 0;  // t0 is a multiple of 16
-    int i = part;
+    const int below = t0 / 4, slice_end = min((t0 + m + 3) / 4, n / 4), whole = n / 4;  // t0 is a multiple of 16
+    int i = (warp << tok_bits) < m ? part : n;  // a warp without tokens has nothing to rank: whole blocks of them from 257 to 480 and 513 to 720 tokens
 #pragma unroll 2
     for (; i < below; i += lanes) {  // tokens before the slice
       const uint4 v = quads[i];
@@ -577,7 +578,7 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   int gt = (int)(before & 0xFFFFu), eq = (int)(before >> 16);
   if (c == 0 && tid == kThreads - 1 && T == kProtectedKey && eq + (int)(both >> 16) > need_eq && device_status)
     atomicOr(device_status, FASTAV_DEV_PROTECT_OVERFLOW);  // more protected tokens than k
-  if (kPer * tid == t0) sh.first_out = gt + min(eq, need_eq);   // t0 is a multiple of 32
+  if (kPer * tid == t0) sh.first_out = gt + min(eq, need_eq);   // t0 is a multiple of 16
   if (kPer * tid == t0 + m) sh.end_out = gt + min(eq, need_eq); // so is the end of a slice, but for the last one's
   if (kPer * tid >= t0 && kPer * tid < t0 + m) {
 #pragma unroll
