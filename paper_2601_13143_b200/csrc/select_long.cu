@@ -29,8 +29,9 @@ constexpr int kBinsPerThread = kBins / kThreads;
 constexpr int kListMax = kThreads;           // keys of a bin that are ranked by counting
 constexpr int kLeastSlice = 256;             // tokens per block worth a block
 
-// Two counts to a word: a slice has at most 2,048 keys, a sequence at most 32,768.  In the 34 KB that the compaction's ring leaves, so that its
-// blocks are resident beside these when the selection ends.
+// Two counts to a word: a slice has at most 2,048 keys, a sequence at most 32,768.  With full slices a block takes 28 KB in clusters of 16,
+// 29 of 8, 31 of 4 and 35 of 2 (18.7 for this, 8 for the scores, 16 over the blocks for the totals): all but the last fit beside a compaction
+// ring of 192 KB, whose blocks are then resident when the selection ends.
 struct alignas(16) LongShared {
   union {
     unsigned hist[kBins / 2];  // of the block's slice

@@ -164,3 +164,37 @@ def check_fused_against_oracle(p, buf: fastav.PruneBuffers, ref: dict, hidden=No
         assert_bits_equal(buf.k_out, ref["k"], what + " k")
         assert_bits_equal(buf.v_out, ref["v"], what + " v")
     return {"max_rel_err": max_rel, "ambiguous_differing": differing, "device_status": status}
+
+
+def log_sum_exp(p) -> torch.Tensor:
+    """What an attention kernel reports for the scored rows: [total_q, Hq] fp32, natural logarithm."""
+    cu, cuq, groups = p.cu_seqlens.tolist(), p.cu_qlens.tolist(), p.q.shape[1] // p.k.shape[1]
+    out = torch.empty(p.q.shape[:2])
+    for b, a in enumerate(cu[:-1]):
+        k = p.k[a:cu[b + 1]].double().repeat_interleave(groups, dim=1)
+        z = torch.einsum("rhd,nhd->rhn", p.q[cuq[b]:cuq[b + 1]].double(), k) * p.softmax_scale
+        if p.causal:
+            z = z.masked_fill((torch.arange(z.shape[2])[None, :] > p.q_idx[cuq[b]:cuq[b + 1], None])[:, None, :], -np.inf)
+        out[cuq[b]:cuq[b + 1]] = torch.logsumexp(z, dim=2)
+    return out
+
+
+def check_prune_under_flags(p, lowest, global_idx, rows, lse, protect=None, what=""):
+    """A prune call under the flags that its selection reads: scores against the oracle's, and the keep list and survivors against
+    what the oracle's selector makes of the call's own scores."""
+    p.protect_rows = rows
+    buf = to_device(p, protect=protect, extra_flags=(fastav.FASTAV_SELECT_LOWEST if lowest else 0) | (fastav.FASTAV_KEEP_IDX_GLOBAL if global_idx else 0))
+    buf.prune(lse_opt=log_sum_exp(p).cuda() if lse else None)
+    torch.cuda.synchronize()
+    overflow = overflows(protected_mask(p, protect), p.cu_seqlens.tolist(), p.keep_counts.tolist())
+    assert int(buf.device_status) == (fastav.FASTAV_DEV_PROTECT_OVERFLOW if overflow else 0), what
+    assert_scores_close(buf.scores, oracle_scores(p), what)
+    scores = buf.scores.cpu().numpy()
+    args = (-scores if lowest else scores, p.cu_seqlens.numpy(), p.keep_counts.numpy(), None if protect is None else protect.numpy(), rows,
+            p.q_idx.numpy(), p.cu_qlens.numpy())
+    idx, cu = oracle.select(*args, global_idx)
+    assert buf.cu_keep.cpu().tolist() == cu.tolist(), what
+    assert np.array_equal(buf.keep_idx.cpu().numpy(), idx), what
+    mine = gather_rows(p, oracle.select(*args)[0], cu)
+    for name in ("hidden", "pos", "k", "v"):
+        assert_bits_equal(getattr(buf, name + "_out"), mine[name], f"{what} {name}")

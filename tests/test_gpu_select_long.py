@@ -28,3 +28,16 @@ def test_select_from_sums(lens, equal):
     torch.cuda.synchronize()
     stats = parity.check_fused_against_oracle(p, buf, parity.oracle_prune(p, protect=protect), protect=protect, what=f"{lens} equal {equal}")
     assert stats["device_status"] & ~fastav.FASTAV_DEV_PROTECT_OVERFLOW == 0
+
+
+@pytest.mark.parametrize("lens", [[2049], [8191, 8193], [2600] * 8, [2051, 40] * 8, [2100] * 34, [4097] * 46], ids=lambda v: f"{len(v)}x{max(v)}")
+@pytest.mark.parametrize("lowest,global_idx,by_rows,lse", [(True, False, False, False), (False, True, False, True), (False, False, True, False), (True, True, True, True)])
+def test_flags_of_the_selection(lens, lowest, global_idx, by_rows, lse):
+    """Scored rows lie on both sides of the borders that a block's slice has in clusters of 16, 8, 4 and 2."""
+    rows = [sorted({j for blocks in (16, 8, 4, 2) for j in ((n + blocks - 1) // blocks + 31 & ~31, ((n + blocks - 1) // blocks + 31 & ~31) - 1) if j < n} | {n - 1})
+            for n in lens]
+    p = W.random_problem(seed=sum(lens) + 1, lens=lens, rows=[len(r) for r in rows], keeps=[(i + 1) * n // (len(lens) + 1) for i, n in enumerate(lens)],
+                         num_q_heads=4, num_kv_heads=2, head_dim=64, hidden=64, duplicate_keys=2)
+    p.q_idx = torch.tensor([j for r in rows for j in r], dtype=torch.int32)
+    protect = (torch.arange(p.total_tokens) % 37 == 5).to(torch.uint8) if len(lens) % 4 else None
+    parity.check_prune_under_flags(p, lowest, global_idx, by_rows, lse, protect, f"{lens[0]} x {len(lens)}")

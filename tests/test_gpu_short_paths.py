@@ -103,3 +103,20 @@ def test_selection_by_counting(lens, equal):
 @pytest.mark.parametrize("batch,n", [(1, 40), (1, 592), (30, 50), (31, 50), (32, 50), (31, 1000), (33, 1000)])
 def test_gather_bounds_by_lane(batch, n):
     _check([n if b % 5 else 0 for b in range(1, batch)] + [n], 1, 4, 2, 64, hid=3584, keep=0.8)
+
+
+# The flags that the selection reads, from the keys (by counting and by digits) and from partial sums; scored rows around the borders of
+# a block's tokens.
+@pytest.mark.parametrize("lens", [[63], [512], [767], [2047], [300, 5] * 4, [1000] * 9, [140] * 35], ids=lambda v: f"{len(v)}x{max(v)}")
+@pytest.mark.parametrize("rows", [2, 9])
+@pytest.mark.parametrize("lowest,global_idx,by_rows,lse", [(True, False, False, False), (False, True, False, True), (False, False, True, False), (True, True, True, True)])
+def test_flags_of_the_selection(lens, rows, lowest, global_idx, by_rows, lse):
+    p = W.random_problem(seed=sum(lens) + rows, lens=lens, rows=[min(rows, n) for n in lens], keeps=[(i + 1) * n // (len(lens) + 1) for i, n in enumerate(lens)],
+                         num_q_heads=8, num_kv_heads=2, head_dim=64, hidden=64, duplicate_keys=2, trailing_rows=False)
+    cuq = p.cu_qlens.tolist()
+    for b, n in enumerate(lens):
+        edges = sorted({j for j in (31, 32, 47, 48, 255, 256) if j < n - 1})[-(cuq[b + 1] - cuq[b]) + 1:] + [n - 1]
+        p.q_idx[cuq[b + 1] - len(edges):cuq[b + 1]] = torch.tensor(edges, dtype=torch.int32)
+        p.q_idx[cuq[b]:cuq[b + 1]] = p.q_idx[cuq[b]:cuq[b + 1]].sort().values
+    protect = (torch.arange(p.total_tokens) % 29 == 3).to(torch.uint8) if len(lens) % 2 else None
+    parity.check_prune_under_flags(p, lowest, global_idx, by_rows, lse, protect, f"{lens[0]} x {len(lens)}, {rows} rows")
