@@ -226,6 +226,26 @@ __device__ __forceinline__ Span row_span(const Shapes& s, const int32_t* cu_qlen
   return checked_span<CACHED>(cu_qlens, b, s.total_q, s.max_qlen);
 }
 
+// One token's sum over its partials: (KV head, row chunk) in that order, `most_chunks` rows of `stride` floats per KV head of which
+// `chunks` hold something.  UNROLL loads in flight, one running sum: whoever adds them up gets the same bits.
+template <int UNROLL>
+__device__ __forceinline__ float sum_of_partials(const float* col, int hkv, int chunks, int most_chunks, int stride) {
+  const int terms = hkv * chunks;
+  float total = 0.f;
+  int g = 0, rc = 0;  // of the next term, stepped along instead of divided out
+  for (int i0 = 0; i0 < terms; i0 += UNROLL) {
+    float v[UNROLL];
+#pragma unroll
+    for (int u = 0; u < UNROLL; ++u) {
+      v[u] = i0 + u < terms ? chain_load(col + (long long)(g * most_chunks + rc) * stride) : 0.f;
+      if (++rc == chunks) { rc = 0; ++g; }
+    }
+#pragma unroll
+    for (int u = 0; u < UNROLL; ++u) total += v[u];
+  }
+  return total;
+}
+
 // Kernels read the caller's index arrays (cu_seqlens, cu_qlens, q_idx, keep_counts, protect) before their wait, and
 // those may be what earlier work on the stream wrote (the cu_keep of the call before).  So the FIRST kernel an entry
 // point launches waits at its very first instruction and lets its successor start only after that (chain_enter):

@@ -397,23 +397,10 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
     __syncthreads();
     const float* const col = in + tok0 + t0;
     if constexpr (FRONT == kPartials) {
-      const int row_chunks = (all_rows * s.group + a.rows_per_chunk - 1) / a.rows_per_chunk, terms = s.hkv * row_chunks;
+      const int row_chunks = (all_rows * s.group + a.rows_per_chunk - 1) / a.rows_per_chunk;
       const float inv = all_rows > 0 ? 1.0f / ((float)s.hq * (float)all_rows) : 0.f;
       for (int j = tid; j < m; j += kThreads) {
-        // Partial i = (KV head, row chunk) in that order; sixteen loads in flight, one running sum in fixed order.
-        float total = 0.f;
-        int g = 0, rc = 0;  // (KV head, row chunk) of the next term, stepped along instead of divided out
-        for (int i0 = 0; i0 < terms; i0 += 16) {
-          float v[16];
-#pragma unroll
-          for (int u = 0; u < 16; ++u) {
-            v[u] = i0 + u < terms ? chain_load(col + (long long)(g * a.row_chunks + rc) * s.total_tokens + j) : 0.f;
-            if (++rc == row_chunks) { rc = 0; ++g; }
-          }
-#pragma unroll
-          for (int u = 0; u < 16; ++u) total += v[u];
-        }
-        const float score = total * inv;
+        const float score = sum_of_partials<16>(col + j, s.hkv, row_chunks, a.row_chunks, s.total_tokens) * inv;
         a.scores_out[tok0 + t0 + j] = score;
         sh.keys[t0 + j] = key_of(j, score);
       }

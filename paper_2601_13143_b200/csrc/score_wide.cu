@@ -656,25 +656,7 @@ __global__ void __launch_bounds__(kFinalizeThreads) score_wide_finalize_kernel(S
   const float inv = rows > 0 ? 1.0f / ((float)s.hq * (float)rows) : 0.f;
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
-  // Partial i = (KV head, row chunk) in that order; eight loads in flight, one running sum in fixed order.
-  const int terms = s.hkv * row_chunks;
-  const float* col = partial + tok0 + j;
-  float total = 0.f;
-  int g = 0, rc = 0;  // (KV head, row chunk) of the next term, stepped along instead of divided out
-  for (int i0 = 0; i0 < terms; i0 += 8) {
-    float v[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      v[u] = i0 + u < terms ? chain_load(col + (long long)(g * rc_max + rc) * s.total_tokens) : 0.f;
-      if (++rc == row_chunks) {
-        rc = 0;
-        ++g;
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) total += v[u];
-  }
-  scores[tok0 + j] = total * inv;
+  scores[tok0 + j] = sum_of_partials<8>(partial + tok0 + j, s.hkv, row_chunks, rc_max, s.total_tokens) * inv;
 }
 
 // ---- host side -----------------------------------------------------------------------------------
