@@ -8,7 +8,7 @@
 //   2^(z - top) put back in its place; the blocks exchange the sums through distributed shared memory (one cluster barrier); each block
 //   then adds its rows' sums up and reads again: 2^(z - top) 2^(top - lse), summed over the 128 rows of every key by a butterfly that
 //   leaves one key per lane -> partial[KV head, row tile][token], which the selecting kernel (prune_few.cu, select_long.cu) adds up.
-//   (With exponentials in both passes, prune of 1 x 2,048 tokens, 64 rows: 23.4 us instead of 22.5; the error against 64 bits is the same
+//   (With exponentials in both passes, prune of 1 x 2,048 tokens, 64 rows: 23.4 us instead of 22.6; the error against 64 bits is the same
 //   on the whole, 0.6 to 1.8e-7 in the 2-norm.)  Where the caller hands the log-sum-exp in, S itself is read in the second pass.
 //
 // Two kernels (this and the selection) replace five (two sweeps, merge, per-token sums, selection).  Bound: latency, the
@@ -92,8 +92,8 @@ __device__ __forceinline__ float transpose_sum(float (&v)[32], int lane) {
 // without it, and above every z of its group, so that the first factor is at most 1.
 //   Small values: the first factor stops at 2^-125, the second is at most 4 kLift, and their product is flushed below 2^-126: whichever
 // factor would be too small, the key adds 0 in every group, as hidden keys do.  (kLift is undone in the partial sums.)
-//   The integer's part costs 0.5 us of the 22.5 at 1 x 2,048 tokens.  Without it as long as all logits of a group are within 2^+-63, 22.1,
-// and 24.2 to 25.2 where they are not.
+//   The integer's part costs 0.6 us of the 22.6 at 1 x 2,048 tokens.  Without it as long as all logits of a group are within 2^+-63, 22.1,
+// but 24.2 to 26.2 where they are not, instead of 21.8 to 23.6.
 constexpr float kLift = 0.0625f;
 constexpr float kToInteger = 12582912.f;  // 1.5 x 2^23: the sum with it is rounded to an integer, which its low bits hold
 constexpr float kMostTop = 65536.f;       // |top| up to which the kernel's own form is exact
@@ -460,7 +460,8 @@ bool once_plan(const Shapes& s, bool lse_given, OncePlan* plan) {
   if (tiles > kMaxTiles) return false;
   const long long clusters = (long long)s.batch * s.hkv * plan->row_tiles;
   // Key tiles per block: the least time of all rounds (in quarters of a microsecond): a round of clusters that run at once takes
-  // some 6 us and 3.75 us per key tile of a block (as fitted with exponentials in both passes; about 3.25 us since).  One round is always the better way (1 x 2,048 tokens, 32 rows, 28 / 4 heads:
+  // some 6 us and 3.75 us per key tile of a block (as fitted with exponentials in both passes; about 0.3 less since, so that a call near the
+  // border may still go to the two sweeps where this would be a little quicker).  One round is always the better way (1 x 2,048 tokens, 32 rows, 28 / 4 heads:
   // 20.7 us with 2 key tiles per block in one round, 26.5 with 1 in two; the two sweeps 31.0).  Several rounds are compared with
   // the two sweeps: about 19 us, and per SM and key tile 2.25 us for every 128 rows of the first and 128 columns of the second.
   // Prune of 32 x 512 tokens, 32 rows: 60.0 against 71.1 us (32 / 8 heads: 66.8 against 83.4), 15 x 1,024: 57.9 / 64.5, but
