@@ -348,6 +348,7 @@ cudaError_t enqueue_selection(const fastav_params& params, const void* q, const 
     *gathered = row_bytes > 0 && few_gathers(s, row_bytes);
     return launch_few(s, q, k, lse_opt, scores_out, true, *gathered ? rows : nullptr, t, st);
   }
+  if (left.kind == ScoreLeft::kLogits) return launch_long_logits(s, w, ws, lse_opt, scores_out, t, st);
   if (left.kind == ScoreLeft::kPartials && !cluster_select_applies(s))
     return launch_long_partials(s, reinterpret_cast<const float*>(ws + w.partial_off), left, scores_out, t, st);
   if (left.kind == ScoreLeft::kPartials) {

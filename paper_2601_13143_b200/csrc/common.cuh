@@ -31,8 +31,9 @@ struct ChainHead { int head_wait = 0; };
 
 // What a prune call still has to do after the scoring kernels, and from what.
 struct ScoreLeft {
-  enum Kind { kScores, kKeys, kPartials } kind = kScores;  // finished scores; nothing done: the kernel that selects starts from
-                                                            // the keys; sums per (KV head, chunk of query rows) and token
+  enum Kind { kScores, kKeys, kPartials, kLogits } kind = kScores;  // finished scores; nothing done: the kernel that selects starts
+                                                                     // from the keys; sums per (KV head, chunk of query rows) and
+                                                                     // token; logits and statistics of few rows
   int row_chunks = 0, rows_per_chunk = 0;                   // kPartials: most chunks of a KV head, query rows of a chunk
 };
 
@@ -87,9 +88,12 @@ cudaError_t launch_score_wide(const Shapes& s, const Workspace& w, const void* q
                               const int32_t* cu_qlens, const void* k, const int32_t* cu_seqlens, const float* lse_in,
                               float* scores_out, unsigned char* ws, int32_t* device_status, cudaStream_t stream, bool* used, ScoreLeft* left);
 
-cudaError_t launch_logits_wide(const Shapes& s, const void* q, const int32_t* q_idx, const int32_t* cu_qlens, const void* k,
-                               const int32_t* cu_seqlens, float* logits, int rq, int32_t* device_status, cudaStream_t stream,
-                               bool* used);
+// Few scored rows on longer sequences: logits and their statistics per 64 tokens (score_rows.cu); log-sum-exp per (row, head).
+// `*used` is false when it does not take the shapes; nothing was launched then.
+cudaError_t launch_rows(const Shapes& s, const Workspace& w, const void* q, const int32_t* q_idx, const int32_t* cu_qlens, const void* k,
+                        const int32_t* cu_seqlens, unsigned char* ws, int32_t* device_status, cudaStream_t stream, bool* used);
+cudaError_t launch_rows_lse(const Shapes& s, const Workspace& w, const int32_t* cu_qlens, const int32_t* cu_seqlens, unsigned char* ws,
+                            cudaStream_t stream);
 
 // The kernel that selects, a thread-block cluster per sequence (prune_few.cu): from the keys themselves (few scored rows, short
 // sequences), from partial sums or from finished scores, to the keep list, or to the gathered rows.
@@ -111,9 +115,11 @@ cudaError_t launch_select_partials(const Shapes& s, const float* partial, const 
                                    const SelectArgs& t, cudaStream_t stream);
 cudaError_t launch_select_scores(const Shapes& s, const float* scores, const SelectArgs& t, cudaStream_t stream);
 
-// ... and of longer sequences, a slice of the tokens per block (select_long.cu), from partial sums.
+// ... and of longer sequences, a slice of the tokens per block (select_long.cu), from partial sums or from logits.
 bool long_select_applies(const Shapes& s);
 cudaError_t launch_long_partials(const Shapes& s, const float* partial, const ScoreLeft& left, float* scores_out, const SelectArgs& t, cudaStream_t stream);
+cudaError_t launch_long_logits(const Shapes& s, const Workspace& w, const unsigned char* ws, const float* lse_in, float* scores_out, const SelectArgs& t,
+                               cudaStream_t stream);
 
 // Most blocks of a cluster that the current context can place: 16, or the portable 8.
 int cluster_limit();
@@ -159,6 +165,9 @@ void count_launches(int n);
 
 // The driver's tensor-map encoder (cuTensorMapEncodeTiled), looked up once through the runtime; nullptr if absent.
 void* tensor_map_encode_entry();
+// A [rows, heads, d] bf16 tensor with element strides (st, sh, 1) as a rank-3 tensor map (d, heads, rows) with the 128-byte swizzle; a
+// box is a 64-element (128-byte) column block of `box_heads` heads of `box_rows` consecutive rows.  `map`: a CUtensorMap.
+bool encode_rows_map(const void* ptr, int dim, int heads, long long rows, long long st, long long sh, int box_heads, int box_rows, void* map);
 
 // A number for the calling thread's current context, never given to another one in this process; 0 if there is none (yet).
 unsigned long long current_context();
@@ -226,24 +235,35 @@ __device__ __forceinline__ Span row_span(const Shapes& s, const int32_t* cu_qlen
   return checked_span<CACHED>(cu_qlens, b, s.total_q, s.max_qlen);
 }
 
-// One token's sum over its partials: (KV head, row chunk) in that order, `most_chunks` rows of `stride` floats per KV head of which
-// `chunks` hold something.  UNROLL loads in flight, one running sum: whoever adds them up gets the same bits.
-template <int UNROLL>
-__device__ __forceinline__ float sum_of_partials(const float* col, int hkv, int chunks, int most_chunks, int stride) {
+// The sums over the partials of TOKENS tokens `step` apart of which `have` exist: (KV head, row chunk) in that order, `most_chunks` rows
+// of `stride` floats per KV head of which `chunks` hold something.  UNROLL loads in flight per token, one running sum: whoever adds them up
+// gets the same bits.
+template <int UNROLL, int TOKENS>
+__device__ __forceinline__ void sum_of_partials(const float* col, int step, int have, int hkv, int chunks, int most_chunks, int stride, float (&total)[TOKENS]) {
   const int terms = hkv * chunks;
-  float total = 0.f;
+#pragma unroll
+  for (int t = 0; t < TOKENS; ++t) total[t] = 0.f;
   int g = 0, rc = 0;  // of the next term, stepped along instead of divided out
   for (int i0 = 0; i0 < terms; i0 += UNROLL) {
-    float v[UNROLL];
+    float v[UNROLL][TOKENS];
 #pragma unroll
     for (int u = 0; u < UNROLL; ++u) {
-      v[u] = i0 + u < terms ? chain_load(col + (long long)(g * most_chunks + rc) * stride) : 0.f;
+      const float* const row = col + (long long)(g * most_chunks + rc) * stride;
+#pragma unroll
+      for (int t = 0; t < TOKENS; ++t) v[u][t] = i0 + u < terms && t < have ? chain_load(row + t * step) : 0.f;
       if (++rc == chunks) { rc = 0; ++g; }
     }
 #pragma unroll
-    for (int u = 0; u < UNROLL; ++u) total += v[u];
+    for (int u = 0; u < UNROLL; ++u)
+#pragma unroll
+      for (int t = 0; t < TOKENS; ++t) total[t] += v[u][t];
   }
-  return total;
+}
+template <int UNROLL>
+__device__ __forceinline__ float sum_of_partials(const float* col, int hkv, int chunks, int most_chunks, int stride) {
+  float total[1];
+  sum_of_partials<UNROLL>(col, 0, 1, hkv, chunks, most_chunks, stride, total);
+  return total[0];
 }
 
 // Kernels read the caller's index arrays (cu_seqlens, cu_qlens, q_idx, keep_counts, protect) before their wait, and

@@ -1,12 +1,13 @@
 // Importance score, Eq. 4 (Section 2.2), for FEW scored rows per sequence -- the shape the paper
 // itself uses in the fine-pruning stage: Q_last is one row per head, so Q K^T is a matrix-vector
-// product and the step is bound by reading K once from HBM.
+// product and the step is bound by reading K once from HBM.  The dispatch, and the CUDA-core kernels that a caller can ask for
+// and that take what the others do not (prune_few.cu: up to 2,048 tokens; score_rows.cu: longer).
 //
 //   logits   : K streams through a ring of shared-memory slots filled by bulk asynchronous copies; every
 //              16-byte piece of a key row is read once by one lane and multiplied with up to eight query
 //              rows held in registers (the rows and heads of one KV group); a butterfly
 //              of shuffles that halves the row set at each step leaves one finished logit per lane.
-//              Logits [Hq, R, N] (base-2 units, -inf where the causal mask hides the key) go to the
+//              Logits [Hq, R, N] (R: the sequence's own rows; base-2 units, -inf where the causal mask hides the key) go to the
 //              workspace: R * Hq * 4 bytes per token next to the Hkv * d * 2 bytes of K read.
 //   stats    : one block per (sequence, head, row): max and sum 2^(z - max) -> log2-sum-exp2.
 //   finalize : per token, sum over heads and rows of 2^(z - lse) in a fixed order, times 1/(Hq R).
@@ -14,6 +15,7 @@
 // Every key goes through the same arithmetic in the same order, whatever its position, so equal
 // keys get bit-equal scores and runs are bit-reproducible.
 #include "common.cuh"
+#include "row_stats.cuh"
 #include "sm100_ptx.cuh"
 
 namespace fastav {
@@ -145,7 +147,7 @@ score_narrow_logits_kernel(Shapes s, const uint16_t* __restrict__ q, const int32
     const bool row_valid = f_mine < flat_rows;
     const int r_mine = row_valid ? f_mine / s.group : 0;
     const int limit = (causal && row_valid) ? q_idx[row0 + r_mine] : 0x7FFFFFFF;
-    float* out = logits + ((long long)(head * s.group + (row_valid ? f_mine % s.group : 0)) * rq + r_mine) * s.total_tokens + tok0;
+    float* out = logits + ((long long)(head * s.group + (row_valid ? f_mine % s.group : 0)) * rows + r_mine) * s.total_tokens + tok0;
 
     for (int sl = 0; sl < slots; ++sl, ++it) {
       const int stage = it % kStages;
@@ -220,7 +222,7 @@ __global__ void __launch_bounds__(256) score_narrow_stats_kernel(Shapes s, const
   const int row0 = qrows.first, rows = min(qrows.count, rq);
   const int tok0 = seq.first, n = seq.count;
   if (r >= rows) return;
-  const float* z = logits + ((long long)head * rq + r) * s.total_tokens + tok0;
+  const float* z = logits + ((long long)head * rows + r) * s.total_tokens + tok0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // One pass: every thread keeps a running (max, sum 2^(z - max)) over its strided share, sixteen loads at a time.
   float m = -INFINITY, l = 0.f;
@@ -266,13 +268,14 @@ constexpr int kFinalizeThreads = 64;  // small blocks: a few thousand tokens sti
 __global__ void __launch_bounds__(kFinalizeThreads) score_narrow_finalize_kernel(Shapes s, const int32_t* __restrict__ cu_qlens,
                                                                                  const int32_t* __restrict__ cu_seqlens,
                                                                                  const float* __restrict__ logits, int rq,
-                                                                                 const float* __restrict__ lse,
-                                                                                 float* __restrict__ scores) {
-  extern __shared__ float lse_sh[];  // [Hq][rows], then the term offsets
+                                                                                 const float* __restrict__ lse, const float2* __restrict__ pairs,
+                                                                                 int pair_stride, float* __restrict__ scores) {
+  extern __shared__ float2 weight[];  // [Hq][rows], from `pairs` (every pair_stride-th) where there are any, else from `lse`
   chain_enter(s);
   pdl_wait();
   pdl_acquire(logits);
   pdl_acquire(lse);
+  pdl_acquire(pairs);
   pdl_acquire(cu_qlens);
   pdl_acquire(cu_seqlens);
   const int b = blockIdx.y;
@@ -281,31 +284,20 @@ __global__ void __launch_bounds__(kFinalizeThreads) score_narrow_finalize_kernel
   const int row0 = qrows.first, all_rows = qrows.count, rows = min(all_rows, rq);
   const int terms = s.hq * rows;
   if ((int)(blockIdx.x * blockDim.x) >= n) return;
-  // where term i's logits start, in units of N floats: worked out once per block (no integer division per logit below)
-  int* term_row = reinterpret_cast<int*>(lse_sh + s.hq * rq);
   for (int i = threadIdx.x; i < terms; i += blockDim.x) {
-    const int head = i / rows, r = i % rows;
-    lse_sh[i] = chain_load(lse + (long long)(row0 + r) * s.hq + head);
-    term_row[i] = head * rq + r;
+    const long long at = (long long)(row0 + i % rows) * s.hq + i / rows;
+    weight[i] = pairs ? weight_from_pair(chain_load(pairs + at * pair_stride)) : weight_from_lse(chain_load(lse + at));
   }
   __syncthreads();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
-  // Term i = (head, row) in head-major order; sixteen loads in flight, one running sum in that fixed order.
-  const float* z = logits + tok0 + j;
-  float total = 0.f;
-  for (int i0 = 0; i0 < terms; i0 += 16) {
-    float v[16];
-#pragma unroll
-    for (int u = 0; u < 16; ++u) {
-      const int i = i0 + u;
-      v[u] = i < terms ? chain_load(z + (long long)term_row[i] * s.total_tokens) : -INFINITY;
-    }
-#pragma unroll
-    for (int u = 0; u < 16; ++u)
-      if (i0 + u < terms) total += exp2f(v[u] - lse_sh[i0 + u]);
+  float total[1] = {0.f};
+  Weights<1> w;
+  for (int i0 = 0; i0 < terms; i0 += Weights<1>::kUnroll) {
+    w.fetch(logits + tok0 + j, 0, 1, i0, terms, s.total_tokens);
+    w.add(weight, i0, terms, total);
   }
-  scores[tok0 + j] = all_rows > 0 ? total / ((float)s.hq * (float)all_rows) : 0.f;
+  scores[tok0 + j] = all_rows > 0 ? total[0] / ((float)s.hq * (float)all_rows) : 0.f;
 }
 
 template <int DIM, int ROWS>
@@ -341,13 +333,6 @@ cudaError_t launch_narrow_logits(const Shapes& s, const Workspace& w, const void
   const int rq = s.max_qlen;
   const bool four = s.max_qlen * s.group <= 4;
   cudaError_t e;
-  // The logits come from a skinny tensor-core MMA over TMA-streamed K tiles where that kernel takes the shapes
-  // (and the caller did not ask for the CUDA-core kernel); otherwise from the lane-group kernel above.
-  bool by_mma = false;
-  if ((s.flags & FASTAV_SCORE_PATH_MASK) != FASTAV_SCORE_PATH_NARROW && score_wide_applies(s)) {
-    e = launch_logits_wide(s, q, q_idx, cu_qlens, k, cu_seqlens, logits, rq, device_status, stream, &by_mma);
-    if (e != cudaSuccess || by_mma) return e;
-  }
   if (s.dim == 128) {
     e = four ? launch_logits<128, 4>(s, qq, q_idx, cu_qlens, kk, cu_seqlens, logits, rq, device_status, stream)
              : launch_logits<128, 8>(s, qq, q_idx, cu_qlens, kk, cu_seqlens, logits, rq, device_status, stream);
@@ -373,22 +358,30 @@ cudaError_t launch_score_narrow(const Shapes& s, const Workspace& w, const void*
     return launch_few(s, q, k, lse_in, scores_out, false, nullptr, SelectArgs{cu_seqlens, nullptr, nullptr, q_idx, cu_qlens, nullptr, nullptr, device_status},
                       stream);
   }
-  cudaError_t e = launch_narrow_logits(s, w, q, q_idx, cu_qlens, k, cu_seqlens, ws, device_status, stream);
+  bool by_mma = false;  // else the CUDA-core kernel above: on request, and where the other does not take the shapes
+  cudaError_t e = launch_rows(s, w, q, q_idx, cu_qlens, k, cu_seqlens, ws, device_status, stream, &by_mma);
+  if (e == cudaSuccess && !by_mma) e = launch_narrow_logits(s, w, q, q_idx, cu_qlens, k, cu_seqlens, ws, device_status, stream);
   if (e != cudaSuccess) return e;
+  if (by_mma && left && long_select_applies(s)) {  // the kernel that selects starts from the logits
+    left->kind = ScoreLeft::kLogits;
+    return cudaSuccess;
+  }
   if (lse_in) e = launch_lse_import(s, lse_in, lse, stream);
+  else if (by_mma) e = launch_rows_lse(s, w, cu_qlens, cu_seqlens, ws, stream);
   else e = launch_chained(score_narrow_stats_kernel, dim3(s.hq * rq, s.batch), dim3(256), 0, stream, s, cu_qlens, cu_seqlens,
                           (const float*)logits, rq, lse);
   if (e != cudaSuccess) return e;
   if (!scores_out) {  // only the statistics were asked for (fastav_lse)
-    count_launches(lse_in ? 0 : 1);
+    count_launches(lse_in || by_mma ? 0 : 1);
     return cudaGetLastError();
   }
   if ((e = launch_chained(score_narrow_finalize_kernel, dim3((s.max_seqlen + kFinalizeThreads - 1) / kFinalizeThreads, s.batch),
                           dim3(kFinalizeThreads),
-                          s.hq * rq * (sizeof(float) + sizeof(int)), stream, s, cu_qlens, cu_seqlens, (const float*)logits, rq, (const float*)lse,
-                          scores_out)) != cudaSuccess)
+                          s.hq * rq * sizeof(float2), stream, s, cu_qlens, cu_seqlens, (const float*)logits, rq, (const float*)lse,
+                          by_mma && !lse_in ? reinterpret_cast<const float2*>(ws + w.stats_off) : (const float2*)nullptr, w.stat_tiles, scores_out)) !=
+      cudaSuccess)
     return e;
-  count_launches((lse_in ? 0 : 1) + 1);  // the lse import counts itself
+  count_launches((lse_in || by_mma ? 0 : 1) + 1);  // the other two count themselves
   return cudaGetLastError();
 }
 

@@ -17,8 +17,7 @@
 // query rows, chunk of key tiles); the share is computed on the device from cu_seqlens.  Warp 0 streams
 // 128-key K tiles and the query tile with TMA (128-byte swizzle) through a 4-stage mbarrier ring, warp 1
 // issues the MMAs into double-buffered accumulators, warps 2-17 (four warpgroups) read the accumulators
-// back with tcgen05.ld and do the softmax arithmetic, part of the exponentials on the FMA pipe.  A third
-// mode of the same kernel only writes the scaled, masked logits (few scored rows: see score_narrow.cu).
+// back with tcgen05.ld and do the softmax arithmetic, part of the exponentials on the FMA pipe.
 // The per-key arithmetic does not depend on the key's position, so equal keys get bit-equal scores; all
 // sums have a fixed order, so runs are reproducible.  Every wait is bounded: a wait that expires makes the
 // block give up, wait for its own copies, free its tensor memory and set FASTAV_DEV_WAIT_EXPIRED.
@@ -124,7 +123,7 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
                   const int32_t* __restrict__ q_idx, const int32_t* __restrict__ cu_qlens,
                   const int32_t* __restrict__ cu_seqlens, int chunk_tiles, int stat_chunks, int rc_max, int rows_per_chunk,
                   float2* __restrict__ stats, const float* __restrict__ lse, float* __restrict__ partial,
-                  float* __restrict__ logits, int rq, int32_t* device_status) {
+                  int32_t* device_status) {
   using L = Layout<DIM>;
   extern __shared__ unsigned char smem_raw[];
   chain_enter(s, q_idx, cu_qlens, cu_seqlens);
@@ -463,52 +462,6 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
           stats[rh * stat_chunks + un.kc * 2 + h] = make_float2(zmax * s.scale_log2, sum2.x + sum2.y);
         }
       }
-    } else if constexpr (SWEEP == 0) {
-      // Logits only (few scored rows: the matrix-vector case done as a skinny MMA, bound by streaming K).
-      // Thread <-> key, warpgroup w owns the query-row columns [32 w, 32 w + 32) and writes their scaled,
-      // masked logits to the [Hq, rq, N] workspace; consecutive lanes write consecutive tokens.
-      int tile_no = 0;
-      bool ok = true;
-      int* slot_of = reinterpret_cast<int*>(ctl.neg_lse[warp - 2]);  // per column: head * rq + scored row
-      int* limit = ctl.limit[warp - 2];
-      for (int u = 0; u < n_units && ok; ++u) {
-        const Unit un = ctl.units[u];
-        const int key_begin = un.kc * chunk_keys;
-        const int tiles = (min(un.n - key_begin, chunk_keys) + kTileKeys - 1) / kTileKeys;
-        const int my_cols = max(0, min(32, un.rows_here - wg * 32));
-        if (un.new_q) {
-          __syncwarp();
-          const int f = un.rc * rows_per_chunk + wg * 32 + lane;
-          const int r = f / s.group;
-          slot_of[lane] = (un.g * s.group + f % s.group) * rq + r;
-          limit[lane] = (causal && lane < my_cols) ? chain_load_cached(q_idx + un.row0 + r) : INT_MAX;
-          __syncwarp();
-        }
-        float* out = logits + un.tok0;
-        for (int t = 0; t < tiles; ++t, ++tile_no) {
-          const int i = tile_no & 1;
-          ok = ptx::mbar_wait_warp(ptx::smem_u32(&ctl.tmem_full[i]), (tile_no >> 1) & 1, abort);
-          if (!ok) break;
-          ptx::tc_fence_after_sync();
-          const int key = key_begin + t * kTileKeys + my_lane;
-          if (my_cols > 0) {
-            uint32_t v[32];
-            ptx::tmem_ld32(lane_addr + i * 256 + wg * 32, v);
-            tmem_ld_wait_for(v);
-            ptx::tc_fence_before_sync();
-            ptx::mbar_arrive(ptx::smem_u32(&ctl.tmem_empty[i]));
-            if (key < un.n) {
-#pragma unroll
-              for (int c = 0; c < 32; ++c)
-                if (c < my_cols)
-                  out[(long long)slot_of[c] * s.total_tokens + key] = key <= limit[c] ? __uint_as_float(v[c]) * s.scale_log2 : -INFINITY;
-            }
-          } else {
-            ptx::tc_fence_before_sync();
-            ptx::mbar_arrive(ptx::smem_u32(&ctl.tmem_empty[i]));
-          }
-        }
-      }
     } else {
       // Every K tile is shared by the four warpgroups: thread <-> key, warpgroup w sums the query-row columns
       // [64 w, 64 w + 64); warpgroups 1-3 publish their sums in shared memory and warpgroup 0 adds them in a
@@ -667,21 +620,6 @@ using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t
 
 EncodeTiledFn encode_tiled_fn() { return reinterpret_cast<EncodeTiledFn>(tensor_map_encode_entry()); }
 
-// A [rows, heads, d] bf16 tensor with element strides (st, sh, 1) as a rank-3 tensor (d, heads, rows); a box
-// is a 64-element (128-byte) column block of `box_heads` heads of `box_rows` consecutive rows.
-bool make_map(const void* ptr, int dim, int heads, long long rows, long long st, long long sh, int box_heads, int box_rows,
-              CUtensorMap* map) {
-  EncodeTiledFn encode = encode_tiled_fn();
-  if (!encode || rows <= 0) return false;
-  const cuuint64_t dims[3] = {(cuuint64_t)dim, (cuuint64_t)heads, (cuuint64_t)rows};
-  const cuuint64_t strides[2] = {(cuuint64_t)sh * 2, (cuuint64_t)st * 2};
-  const cuuint32_t box[3] = {64, (cuuint32_t)box_heads, (cuuint32_t)box_rows};
-  const cuuint32_t elem[3] = {1, 1, 1};
-  return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, elem,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // Persistent grid and key chunk: one block per SM; chunks sized so that a block gets about a dozen units (fine
 // enough to balance, and never more than its table holds).  Batches of so many sequences that no chunk does that take more
 // blocks.
@@ -697,21 +635,6 @@ void plan_units(const Shapes& s, int rc_max, int* grid_out, int* chunk_tiles_out
   if ((units() + grid - 1) / grid + 1 > kMaxUnits) grid = (units() + kMaxUnits - 2) / (kMaxUnits - 1);
   *grid_out = (int)grid;
   *chunk_tiles_out = (int)chunk_tiles;
-}
-
-template <int DIM>
-cudaError_t run_logits(const Shapes& s, const CUtensorMap& k_map, const CUtensorMap& q_map, const int32_t* q_idx,
-                       const int32_t* cu_qlens, const int32_t* cu_seqlens, float* logits, int rq, int32_t* device_status,
-                       cudaStream_t stream) {
-  int grid, chunk_tiles;
-  plan_units(s, 1, &grid, &chunk_tiles);
-  const int smem = Layout<DIM>::kTotal;
-  cudaError_t e =
-      once_per_context([&] { return cudaFuncSetAttribute(score_wide_kernel<DIM, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
-  if (e != cudaSuccess) return e;
-  return launch_chained(score_wide_kernel<DIM, 0>, dim3(grid), dim3(kThreads), smem, stream, k_map, q_map, s, q_idx, cu_qlens,
-                        cu_seqlens, chunk_tiles, 0, 1, wide_rows_per_chunk(s.group), (float2*)nullptr, (const float*)nullptr,
-                        (float*)nullptr, logits, rq, device_status);
 }
 
 template <int DIM>
@@ -757,7 +680,7 @@ cudaError_t run(const Shapes& s, const Workspace& w, const CUtensorMap& k_map, c
   } else {
     if ((e = launch_chained(score_wide_kernel<DIM, 1>, dim3(grid), dim3(kThreads), smem, stream, k_map, q_map, s, q_idx, cu_qlens,
                             cu_seqlens, chunk_tiles, stat_chunks, rc_max, rows_per_chunk, stats, (const float*)nullptr,
-                            (float*)nullptr, (float*)nullptr, 0, device_status)) != cudaSuccess)
+                            (float*)nullptr, device_status)) != cudaSuccess)
       return e;
     const int warps = s.total_q * s.hq;
     if ((e = launch_chained(score_wide_merge_kernel, dim3((warps + 7) / 8), dim3(256), 0, stream, s, cu_qlens, cu_seqlens,
@@ -768,7 +691,7 @@ cudaError_t run(const Shapes& s, const Workspace& w, const CUtensorMap& k_map, c
   if (!scores_out) return cudaGetLastError();  // only the statistics were asked for (fastav_lse)
   if ((e = launch_chained(score_wide_kernel<DIM, 2>, dim3(grid), dim3(kThreads), smem, stream, k_map, q_map, s, q_idx, cu_qlens,
                           cu_seqlens, chunk_tiles, stat_chunks, rc_max, rows_per_chunk, (float2*)nullptr, (const float*)lse,
-                          partial, (float*)nullptr, 0, device_status)) != cudaSuccess)
+                          partial, device_status)) != cudaSuccess)
     return e;
   count_launches(1);
   if ((e = finish(rc_max, rows_per_chunk)) != cudaSuccess) return e;
@@ -789,6 +712,19 @@ void* tensor_map_encode_entry() {
   return entry;
 }
 
+bool encode_rows_map(const void* ptr, int dim, int heads, long long rows, long long st, long long sh, int box_heads, int box_rows,
+                     void* map) {
+  EncodeTiledFn encode = encode_tiled_fn();
+  if (!encode || rows <= 0) return false;
+  const cuuint64_t dims[3] = {(cuuint64_t)dim, (cuuint64_t)heads, (cuuint64_t)rows};
+  const cuuint64_t strides[2] = {(cuuint64_t)sh * 2, (cuuint64_t)st * 2};
+  const cuuint32_t box[3] = {64, (cuuint32_t)box_heads, (cuuint32_t)box_rows};
+  const cuuint32_t elem[3] = {1, 1, 1};
+  return encode(static_cast<CUtensorMap*>(map), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, elem,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Query rows per block: whole TMA boxes of 8 scored rows x G heads, as many as fit in 256 rows.
 int wide_rows_per_chunk(int group) { return group >= 1 && group <= 32 ? kRowsPerCta / (8 * group) * (8 * group) : 0; }
 
@@ -805,26 +741,13 @@ bool score_wide_applies(const Shapes& s) {
          ok_stride(s.k_st) && ok_stride(s.k_sh) && ok_stride(s.q_st) && ok_stride(s.q_sh);
 }
 
-// Logits [Hq, rq, N] of a batch with at most rq <= 4 scored rows per sequence, by the tensor-core kernel.
-cudaError_t launch_logits_wide(const Shapes& s, const void* q, const int32_t* q_idx, const int32_t* cu_qlens, const void* k,
-                               const int32_t* cu_seqlens, float* logits, int rq, int32_t* device_status, cudaStream_t stream,
-                               bool* used) {
-  CUtensorMap k_map, q_map;
-  *used = rq * s.group <= 128 && make_map(k, s.dim, s.hkv, s.total_tokens, s.k_st, s.k_sh, 1, kTileKeys, &k_map) &&
-          make_map(q, s.dim, s.hq, s.total_q, s.q_st, s.q_sh, s.group, 8, &q_map);
-  if (!*used) return cudaSuccess;
-  count_launches(1);
-  if (s.dim == 128) return run_logits<128>(s, k_map, q_map, q_idx, cu_qlens, cu_seqlens, logits, rq, device_status, stream);
-  return run_logits<64>(s, k_map, q_map, q_idx, cu_qlens, cu_seqlens, logits, rq, device_status, stream);
-}
-
 cudaError_t launch_score_wide(const Shapes& s, const Workspace& w, const void* q, const int32_t* q_idx,
                               const int32_t* cu_qlens, const void* k, const int32_t* cu_seqlens, const float* lse_in,
                               float* scores_out, unsigned char* ws, int32_t* device_status, cudaStream_t stream, bool* used,
                               ScoreLeft* left) {
   CUtensorMap k_map, q_map;
-  *used = make_map(k, s.dim, s.hkv, s.total_tokens, s.k_st, s.k_sh, 1, kTileKeys, &k_map) &&
-          make_map(q, s.dim, s.hq, s.total_q, s.q_st, s.q_sh, s.group, 8, &q_map);
+  *used = encode_rows_map(k, s.dim, s.hkv, s.total_tokens, s.k_st, s.k_sh, 1, kTileKeys, &k_map) &&
+          encode_rows_map(q, s.dim, s.hq, s.total_q, s.q_st, s.q_sh, s.group, 8, &q_map);
   if (!*used) return cudaSuccess;  // the caller falls back to the CUDA-core path
   if (s.dim == 128) return run<128>(s, w, k_map, q_map, q_idx, cu_qlens, cu_seqlens, lse_in, scores_out, ws, device_status, stream, left);
   return run<64>(s, w, k_map, q_map, q_idx, cu_qlens, cu_seqlens, lse_in, scores_out, ws, device_status, stream, left);

@@ -1,6 +1,7 @@
-// What follows the tensor-core sweeps on sequences of more than 2,048 tokens, in one kernel: their sums per (KV head, chunk of query
-// rows) and token become scores, in their fixed order, and the k highest are selected (Section 2.2; ties to the lower index,
-// protected tokens always).  One thread-block cluster per sequence, a slice of at most 2,048 tokens per block.
+// What follows the scoring kernels on sequences of more than 2,048 tokens, in one kernel: the tensor-core sweeps' sums per (KV head,
+// chunk of query rows) and token, or few rows' logits and statistics, become scores, in their fixed order, and the k highest
+// are selected (Section 2.2; ties to the lower index, protected tokens always).  One thread-block cluster per sequence, a slice of
+// at most 2,048 tokens per block.
 //
 // The keys stay where they are.  A pass takes 13 bits: each block counts its slice's digits, adds the bins it has to the block that
 // owns them (distributed shared memory), and after a cluster barrier each reads all totals and finds the bin of the k-th largest
@@ -9,11 +10,12 @@
 //
 // Bound: latency, a chain of a dozen steps of which four are cluster barriers.  It saves the kernel that added the sums up; against
 // that and a selection by one block: 3 x 8,001-9,001 tokens with the log-sum-exp given 74.0 -> 72.5 us, 1 to 3 % of a
-// call on a few thousand tokens, 0.3 % of one on 4 x 16,384.  Clusters of 4, 8 or 16 make no difference.  From finished scores
-// (the few-rows path, fastav_select) nothing is saved and one block stays quicker: 4 x 6,554 tokens, one row 109.8 us against 111.7, 32
-// ragged sequences 217.8 against 219.7.
+// call on a few thousand tokens, 0.3 % of one on 4 x 16,384.  From logits it saves two kernels (statistics, scores).  Clusters of 4, 8 or 16 make no
+// difference.  From finished scores (fastav_select) nothing is saved and one block stays quicker: 4 x 6,554 tokens 109.8 us against 111.7,
+// 32 ragged sequences 217.8 against 219.7 (of the calls that had finished scores then).
 #include "cluster.cuh"
 #include "common.cuh"
+#include "row_stats.cuh"
 #include "select_keys.cuh"
 
 namespace fastav {
@@ -27,6 +29,7 @@ constexpr int kDigitBits = 13;
 constexpr int kBins = 1 << kDigitBits;
 constexpr int kBinsPerThread = kBins / kThreads;
 constexpr int kListMax = kThreads;           // keys of a bin that are ranked by counting
+constexpr int kMaxTerms = 256 * kNarrowMaxRows;  // heads x scored rows of the few-rows path
 constexpr int kLeastSlice = 256;             // tokens per block worth a block
 
 // Two counts to a word: a slice has at most 2,048 keys, a sequence at most 32,768.  With full slices a block takes 28 KB in clusters of 16,
@@ -47,16 +50,28 @@ struct alignas(16) LongShared {
   unsigned prefix, threshold, own;
 };
 
+enum Front { kPartials, kLogits };
+
 struct LongArgs {
-  const float* partial;            // [Hkv * row_chunks][N]
-  int row_chunks, rows_per_chunk;
+  const float* in;                 // kPartials [Hkv * row_chunks][N]; kLogits [Hq * rq][N]
+  int row_chunks, rows_per_chunk;  // kPartials
+  const float2* stats;             // kLogits [total_q * Hq][stat_tiles]
+  const float* lse_in;             // kLogits, optional: the caller's natural-log log-sum-exp [total_q, Hq], in place of stats
+  int rq, stat_tiles;              // kLogits: most scored rows of a sequence
   float* scores_out;
   int blocks, slice_cap;           // blocks of a cluster; tokens of a block that the longest sequence needs
 };
 
 // After LongShared: the scores of the slice, then the totals of the bins this block owns, of the whole cluster.
 __host__ __device__ inline int owned_words(int blocks) { return kBins / 2 / blocks; }
-inline size_t long_bytes(int blocks, int slice_cap) { return sizeof(LongShared) + (size_t)(slice_cap + owned_words(blocks)) * sizeof(unsigned); }
+// ... and of kLogits what each term's weights are made with, at most `terms`.
+inline size_t long_bytes(int blocks, int slice_cap, int terms) {
+  return sizeof(LongShared) + (size_t)(slice_cap + owned_words(blocks) + 2 * terms) * sizeof(unsigned);
+}
+template <int N>
+struct Tokens {
+  static constexpr int value = N;
+};
 __host__ __device__ inline int slice_for(int n, int blocks) { return ((n + blocks - 1) / blocks + 31) & ~31; }
 
 __device__ __forceinline__ void remote_add(uint32_t a, unsigned v) {
@@ -73,6 +88,7 @@ __device__ __forceinline__ uint4 remote_load4(uint32_t a) {  // 16-byte aligned
   return v;
 }
 
+template <Front FRONT>
 __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, LongArgs a, const int32_t* __restrict__ cu_seqlens,
                                                                   const int32_t* __restrict__ keep_counts, const uint8_t* __restrict__ protect,
                                                                   const int32_t* __restrict__ q_idx, const int32_t* __restrict__ cu_qlens,
@@ -109,8 +125,8 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
   const bool lowest = (s.flags & FASTAV_SELECT_LOWEST) != 0;
 
   pdl_wait();
-  const float* partial = a.partial;
-  pdl_acquire(partial);
+  const float* in = a.in;
+  pdl_acquire(in);
   if (tid == 0 && c == 0 && device_status) {
     if (seq.bad || qrows.bad) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
     if (k_clamped) atomicOr(device_status, FASTAV_DEV_K_CLAMPED);
@@ -138,14 +154,71 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
         if (lane == 0 && word) atomicOr(&sh.prot_bits[j0 >> 5], word);
       }
   }
-  const float* const col = partial + tok0 + t0;
-  const int row_chunks = (qrows.count * s.group + a.rows_per_chunk - 1) / a.rows_per_chunk;
-  const float inv = qrows.count > 0 ? 1.0f / ((float)s.hq * (float)qrows.count) : 0.f;
-  for (int j = tid; j < m; j += kThreads) {
-    const float score = sum_of_partials<16>(col + j, s.hkv, row_chunks, a.row_chunks, s.total_tokens) * inv;
-    a.scores_out[tok0 + t0 + j] = score;
-    keys[j] = __float_as_uint(score);
-  }
+  const float* const col = in + tok0 + t0;
+  const int rows = FRONT == kLogits ? min(qrows.count, a.rq) : 0, terms = s.hq * rows;  // term i = (head i / rows, row i % rows)
+  float2* const weight = reinterpret_cast<float2*>(totals + owned);
+  const float2* stats = a.stats;
+  if constexpr (FRONT == kLogits) pdl_acquire(stats);
+  auto merge_stats = [&] {
+    if constexpr (FRONT == kLogits) {
+      const int l16 = lane & (kMergeLanes - 1), tiles = (n + kRowTileTokens - 1) / kRowTileTokens;
+#pragma unroll 1
+      for (int i0 = 0; i0 < terms; i0 += kThreads / kMergeLanes) {
+        const int i = i0 + tid / kMergeLanes, head = i / rows, r = i - head * rows;
+        const long long at = (long long)(qrows.first + r) * s.hq + head;
+        float2 w;
+        if (a.lse_in) {
+          const float v = i < terms ? chain_load(a.lse_in + at) : 0.f;
+          w = weight_from_lse((v == v && fabsf(v) != INFINITY) ? v * kLog2e : INFINITY);  // a row that sees no key adds 0
+        } else {
+          w = weight_from_pair(merge_row_stats(stats + at * a.stat_tiles, i < terms ? tiles : 0, l16));
+        }
+        if (l16 == 0 && i < terms) weight[i] = w;
+      }
+      __syncthreads();
+    }
+  };
+  // A thread's tokens lie kThreads apart; up to four of them are added up together.
+  auto add_up = [&](auto tokens) {
+    constexpr int kTokens = decltype(tokens)::value;
+    auto have_from = [&](int j0) { return min(kTokens, (m - j0 + kThreads - 1) / kThreads); };
+    Weights<kTokens> w;
+    if constexpr (FRONT == kLogits) {  // the first logits are on their way while the statistics are merged
+      w.fetch(col + tid, kThreads, have_from(tid), 0, terms, s.total_tokens);
+      merge_stats();
+    }
+#pragma unroll 1
+    for (int j0 = tid; j0 < m; j0 += kThreads * kTokens) {
+      const int have = have_from(j0);
+      float total[kTokens];
+      if constexpr (FRONT == kPartials) {
+        const int row_chunks = (qrows.count * s.group + a.rows_per_chunk - 1) / a.rows_per_chunk;
+        sum_of_partials<32 / kTokens>(col + j0, kThreads, have, s.hkv, row_chunks, a.row_chunks, s.total_tokens, total);
+        const float inv = qrows.count > 0 ? 1.0f / ((float)s.hq * (float)qrows.count) : 0.f;
+#pragma unroll
+        for (int t = 0; t < kTokens; ++t) total[t] *= inv;
+      } else {
+#pragma unroll
+        for (int t = 0; t < kTokens; ++t) total[t] = 0.f;
+#pragma unroll 1
+        for (int i0 = 0; i0 < terms; i0 += w.kUnroll) {
+          if (j0 != tid || i0 > 0) w.fetch(col + j0, kThreads, have, i0, terms, s.total_tokens);
+          w.add(weight, i0, terms, total);
+        }
+#pragma unroll
+        for (int t = 0; t < kTokens; ++t) total[t] = rows > 0 ? total[t] / ((float)s.hq * (float)qrows.count) : 0.f;
+      }
+#pragma unroll
+      for (int t = 0; t < kTokens; ++t)
+        if (t < have) {
+          a.scores_out[tok0 + t0 + j0 + t * kThreads] = total[t];
+          keys[j0 + t * kThreads] = __float_as_uint(total[t]);
+        }
+    }
+  };
+  if (m <= kThreads) add_up(Tokens<1>{});
+  else if (m <= 2 * kThreads) add_up(Tokens<2>{});
+  else add_up(Tokens<4>{});
   __syncthreads();
   const int base = sh.base;
   if (c == 0 && tid == 0) {
@@ -303,23 +376,45 @@ int blocks_for(const Shapes& s) {
 
 bool long_select_applies(const Shapes& s) { return !cluster_select_applies(s) && blocks_for(s) > 0; }
 
-cudaError_t launch_long_partials(const Shapes& s, const float* partial, const ScoreLeft& left, float* scores_out, const SelectArgs& t, cudaStream_t stream) {
-  LongArgs a{};
-  a.partial = partial;
-  a.row_chunks = left.row_chunks;
-  a.rows_per_chunk = left.rows_per_chunk;
+namespace {
+
+template <Front FRONT>
+cudaError_t launch(const Shapes& s, LongArgs a, float* scores_out, const SelectArgs& t, cudaStream_t stream) {
   a.scores_out = scores_out;
   a.blocks = blocks_for(s);
   a.slice_cap = slice_for(s.max_seqlen, a.blocks);
+  const int terms = FRONT == kLogits ? s.hq * a.rq : 0;
   cudaError_t e = once_per_context([] {
-    const cudaError_t f = cudaFuncSetAttribute(select_long_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)long_bytes(2, kSlice));
-    return f == cudaSuccess ? cudaFuncSetAttribute(select_long_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : f;
+    const cudaError_t f = cudaFuncSetAttribute(select_long_kernel<FRONT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)long_bytes(2, kSlice, FRONT == kLogits ? kMaxTerms : 0));
+    return f == cudaSuccess ? cudaFuncSetAttribute(select_long_kernel<FRONT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : f;
   });
   if (e != cudaSuccess) return e;
-  e = launch_chained_cluster(select_long_kernel, dim3(s.batch * a.blocks), dim3(kThreads), a.blocks, long_bytes(a.blocks, a.slice_cap), stream, s, a, t.cu_seqlens,
-                             t.keep_counts, t.protect, t.q_idx, t.cu_qlens, t.keep_idx, t.cu_keep, t.device_status);
+  e = launch_chained_cluster(select_long_kernel<FRONT>, dim3(s.batch * a.blocks), dim3(kThreads), a.blocks, long_bytes(a.blocks, a.slice_cap, terms), stream,
+                             s, a, t.cu_seqlens, t.keep_counts, t.protect, t.q_idx, t.cu_qlens, t.keep_idx, t.cu_keep, t.device_status);
   count_launches(1);
   return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_long_partials(const Shapes& s, const float* partial, const ScoreLeft& left, float* scores_out, const SelectArgs& t, cudaStream_t stream) {
+  LongArgs a{};
+  a.in = partial;
+  a.row_chunks = left.row_chunks;
+  a.rows_per_chunk = left.rows_per_chunk;
+  return launch<kPartials>(s, a, scores_out, t, stream);
+}
+
+cudaError_t launch_long_logits(const Shapes& s, const Workspace& w, const unsigned char* ws, const float* lse_in, float* scores_out, const SelectArgs& t,
+                               cudaStream_t stream) {
+  LongArgs a{};
+  a.in = reinterpret_cast<const float*>(ws + w.logits_off);
+  a.stats = reinterpret_cast<const float2*>(ws + w.stats_off);
+  a.lse_in = lse_in;
+  a.rq = s.max_qlen;
+  a.stat_tiles = w.stat_tiles;
+  return launch<kLogits>(s, a, scores_out, t, stream);
 }
 
 }  // namespace fastav

@@ -95,6 +95,12 @@ __device__ __forceinline__ void mbar_arrive_warp(uint32_t bar, int lane) {
   if (lane == 0) mbar_arrive(bar);
 }
 
+__device__ __forceinline__ uint4 ld_shared4(uint32_t at) {  // 16-byte aligned
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at) : "memory");
+  return v;
+}
+
 // ---- proxies and fences ------------------------------------------------------------------------
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }

@@ -1,0 +1,62 @@
+"""Few scored rows on sequences beyond 2,048 tokens (score_rows.cu, and the selection from its logits in select_long.cu): ends of tiles of
+64 tokens and of a block's slice, up to 32 sequences and more (the padded list of tiles), 1 to 128 query rows per KV head, empty
+sequences and ones without scored rows, head-major and packed keys.  Against the oracle, and the separate calls against the fused one."""
+import pytest
+import torch
+
+import parity
+from paper_2601_13143_b200 import fastav, workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _problem(lens, rows, hq, hkv, d, **more):
+    rows = [min(rows, n) if i % 5 != 3 else 0 for i, n in enumerate(lens)]
+    return W.random_problem(seed=sum(lens) + hq, lens=lens, rows=rows, keeps=[(i % 3 + 1) * n // 4 for i, n in enumerate(lens)], num_q_heads=hq,
+                            num_kv_heads=hkv, head_dim=d, hidden=64, duplicate_keys=2, **more)
+
+
+@pytest.mark.parametrize("lens,rows,hq,hkv,d", [
+    ([2049], 1, 28, 4, 128), ([2111, 64, 63, 65, 0, 1], 4, 8, 2, 64), ([4096, 4097], 2, 16, 16, 64), ([8257, 2050, 128], 3, 32, 4, 128), ([33000], 1, 8, 2, 64),
+    ([2500] * 3 + [300] * 5, 4, 32, 1, 64), ([2060] * 32, 1, 4, 2, 64), ([2060, 31, 0] * 11, 2, 4, 2, 128), ([2049] * 75, 1, 4, 2, 64), ([640] * 150, 1, 4, 1, 128),
+])
+@pytest.mark.parametrize("trailing", [True, False])
+def test_few_rows_of_long_sequences(lens, rows, hq, hkv, d, trailing):
+    p = _problem(lens, rows, hq, hkv, d, trailing_rows=trailing)
+    buf = parity.to_device(p)
+    buf.prune()
+    torch.cuda.synchronize()
+    stats = parity.check_fused_against_oracle(p, buf, parity.oracle_prune(p), what=f"{lens[0]} x {len(lens)}")
+    assert stats["device_status"] & ~fastav.FASTAV_DEV_PROTECT_OVERFLOW == 0
+    fused = buf.scores.clone()
+    buf.scores.fill_(-1.0)
+    buf.score()
+    torch.cuda.synchronize()
+    assert torch.equal(buf.scores.view(torch.int32), fused.view(torch.int32))
+    # The statistics by themselves: fp32 sums of up to 33,000 terms in a tree, and the logits' fp32 rounding (2^-24 of at most 128 products).
+    if p.q_idx.numel():
+        lse = torch.empty(p.q.shape[0], hq, device="cuda")
+        fastav.fastav_lse(buf.params, buf.q, buf.q_idx, buf.cu_qlens, buf.k, buf.cu_seqlens, lse, buf.workspace, buf.device_status)
+        torch.testing.assert_close(lse.cpu().double(), parity.log_sum_exp(p).double(), rtol=0, atol=2e-5)
+
+
+@pytest.mark.parametrize("layout", ["packed", "head_major"])
+def test_strided_keys(layout):
+    p = _problem([2300, 2100], 2, 8, 4, 64)
+    n, heads, d = p.k.shape
+    if layout == "packed":  # a view into a projection output that holds more than the keys
+        held = torch.zeros(n, heads + 3, d, dtype=p.k.dtype, device="cuda")
+        k = held[:, 2:2 + heads]
+    else:
+        held = torch.zeros(heads, n, d, dtype=p.k.dtype, device="cuda")
+        k = held.transpose(0, 1)
+    k.copy_(p.k)
+    plain = parity.to_device(p)
+    plain.prune()
+    buf = fastav.make_buffers(q=plain.q, q_idx=plain.q_idx, cu_qlens=plain.cu_qlens, k=k, v=plain.v, cu_seqlens=plain.cu_seqlens, keep_counts=plain.keep_counts,
+                              hidden=plain.hidden, pos=plain.pos, softmax_scale=p.softmax_scale, flags=parity.flags_of(p))
+    buf.prune()
+    torch.cuda.synchronize()
+    assert int(buf.device_status) == int(plain.device_status)
+    for name in ("scores", "keep_idx", "cu_keep", "hidden_out", "pos_out", "k_out", "v_out"):
+        assert torch.equal(getattr(buf, name), getattr(plain, name)), name
