@@ -176,8 +176,8 @@ __host__ __device__ inline size_t align_up(size_t x, size_t a) { return (x + a -
 
 // ---- programmatic dependent launch ----------------------------------------------------------------
 // The kernels of one prune call form a chain in which each reads what its predecessor wrote.  They
-// are launched with programmatic stream serialization: a kernel lets its successor start early
-// (pdl_trigger, first thing) so that the successor's set-up overlaps this kernel's tail, and every
+// are launched with programmatic stream serialization: a kernel lets its successor start before its own end
+// (pdl_trigger) so that the successor's launch and set-up overlap this kernel's tail, and every
 // block of the successor calls pdl_wait -- which returns once the predecessor has completed and its
 // writes are visible -- before it touches global memory another kernel may have written, or writes
 // global memory another kernel may still read.  Every block waits before it exits, so completion of a
@@ -286,18 +286,16 @@ __device__ __forceinline__ void chain_enter(const Head& head, P&... arrays) {
   (chain_acquire_one(arrays), ...);
   pdl_trigger();
 }
-// The same in two halves, for kernels with set-up work that touches no global memory: a call's first kernel does that work
-// ahead of its wait, the others let their successor start before anything else (a set-up of 0.2 us ahead of the trigger
-// shows as 0.2 us per launch in a chain of small calls).
-template <typename Head>
-__device__ __forceinline__ void chain_begin_setup(const Head& head) {
-  if (!head.head_wait) pdl_trigger();
-}
+// For kernels that let their successor start later (pdl_trigger in their own time): a call's first kernel does its set-up that touches no
+// global memory, then comes here.  A successor that is resident beside a kernel costs it more than its launch takes where
+// the kernel is a chain of short steps, or where its blocks end at different times and the successor's take the SMs in between: started
+// when the last loads have been issued, or some 3 us ahead of the end, 13 fine stages from 744 tokens take 148.8 us instead of 155.6,
+// 1 x 2,048 tokens 21.0 / 22.6, 4 x 16,384 288 / 292, 32 ragged sequences of up to 8,192 301 / 307.  (Later still costs launch latency:
+// the 13 stages 157 with the trigger behind the selection, 160 with the compaction's at its end.)
 template <typename Head, typename... P>
-__device__ __forceinline__ void chain_end_setup(const Head& head, P&... arrays) {
+__device__ __forceinline__ void chain_enter_late(const Head& head, P&... arrays) {
   if (head.head_wait) pdl_wait();
   (chain_acquire_one(arrays), ...);
-  if (head.head_wait) pdl_trigger();
 }
 inline thread_local bool g_chain_head = true;
 inline void chain_begin(uint32_t flags) { g_chain_head = (flags & FASTAV_CHAIN_CALLS) == 0; }

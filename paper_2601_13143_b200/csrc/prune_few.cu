@@ -119,7 +119,6 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
                                                                 int32_t* __restrict__ cu_keep, int32_t* device_status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   FewShared& sh = *reinterpret_cast<FewShared*>(smem_raw);
-  chain_begin_setup(s);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int blocks = (int)gridDim.x / s.batch;  // blocks per cluster
   const int b = blockIdx.x / blocks, c = (int)cluster_rank();
@@ -132,7 +131,7 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   if (tid < kMaxTokens / 32) sh.prot_bits[tid] = 0u;
   if (tid < kCountSlice / 32) sh.kept[tid] = 0u;
   if (tid == 32) { sh.base = 0; sh.list_n = 0; }
-  chain_end_setup(s, cu_seqlens, keep_counts, protect, q_idx, cu_qlens);
+  chain_enter_late(s, cu_seqlens, keep_counts, protect, q_idx, cu_qlens);
   // ---- the caller's index arrays: one warp asks for all of them at once (sixteen warps of sixteen blocks asking for the
   //      same words queue at one L2 slice: 2,500 cycles instead of 900) ----------------------------------------------------
   if (warp == 0) {
@@ -396,6 +395,7 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   if (!selecting) return;  // uniform for the cluster; nothing remote is outstanding
   cluster_sync();          // every block has all keys
 
+  pdl_trigger();
   const int base = sh.base;
   if (c == 0 && tid == 0) {
     cu_keep[b + 1] = base + k;

@@ -223,7 +223,7 @@ rollout_stats_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
   using Cfg = StatSmem<DIM>;
   constexpr int kStages = Cfg::kStages, kOperandBytes = Cfg::kOperandBytes;
   extern __shared__ unsigned char smem_raw[];
-  chain_enter(chain_head);
+  chain_enter_late(chain_head);
   const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t slots = base + kStages * kOperandBytes;
   AttnControl& ctl = *reinterpret_cast<AttnControl*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + 6 * kOperandBytes);
@@ -258,6 +258,7 @@ rollout_stats_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
         loads += load_q;
         x.advance();
       }
+      pdl_trigger();  // all loads have been issued
       if (*abort) drain_loads(ctl, it, kStages);
     }
   } else if (warp == 1) {
@@ -398,7 +399,7 @@ rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
   constexpr int kStages = Cfg::kStages, kOperandBytes = Cfg::kOperandBytes;
   constexpr int kStripCols = 32 * kMaxStripUnits;
   extern __shared__ unsigned char smem_raw[];
-  chain_enter(chain_head);
+  chain_enter_late(chain_head);
   const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t slots = base + kStages * kOperandBytes;
   AttnControl& ctl =
@@ -448,6 +449,7 @@ rollout_map_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
               ptx::tma_load_3d(slot + sub * Cfg::kStripSubBytes + u * 4096, &k_strip_map, sub * 64, it / group, (strip.unit + u) * 32, bar);
         }
       }
+      pdl_trigger();  // all loads have been issued
       if (*abort) drain_loads(ctl, it, kStages);
     }
   } else if (warp == 1) {
@@ -642,7 +644,7 @@ rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_
                     float* partials, int* counters, int32_t* device_status, ChainHead chain_head) {
   constexpr int kStages = kGemmStages, kStageBytes = kGemmStageBytes;
   extern __shared__ unsigned char smem_raw[];
-  chain_enter(chain_head);
+  chain_enter_late(chain_head);
   const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   PipeControl& ctl = *reinterpret_cast<PipeControl*>(smem_raw + (base - ptx::smem_u32(smem_raw)) + kStages * kStageBytes + kGemmStageOut);
   volatile int* abort = &ctl.abort;
@@ -673,6 +675,7 @@ rollout_gemm_kernel(const __grid_constant__ CUtensorMap rt_hi_map, const __grid_
           ptx::tma_load_2d(dst + 3 * kSubTileBytes, &a_lo_map, kb * 64, unit.nb * kTile, bar);
         }
       }
+      pdl_trigger();  // all loads have been issued
       if (*abort) drain_loads(ctl, it, kStages);
     }
   } else if (warp == 1) {

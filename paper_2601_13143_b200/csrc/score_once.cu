@@ -156,7 +156,6 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
   using L = Layout<DIM>;
   constexpr int kSubTiles = DIM / 64;
   extern __shared__ unsigned char smem_raw[];
-  chain_begin_setup(s);
   cluster_arrive();  // "this block runs": waited for before the first remote access
   const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t q_smem = base, k_smem = base + L::kOperandBytes;
@@ -186,7 +185,7 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
       asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(q_smem + i * 16), "r"(0) : "memory");
     ptx::fence_proxy_async_smem();  // ordered before the TMA writes that follow the barrier
   }
-  chain_end_setup(s, q_idx, cu_qlens, cu_seqlens);
+  chain_enter_late(s, q_idx, cu_qlens, cu_seqlens);
   if (warp == 0) {  // the sequence's bounds, asked for by one warp
     const int32_t* word = lane < 2 ? cu_seqlens + b + lane : cu_qlens + b + (lane & 1);
     if (lane < 4) ctl.index[lane] = chain_load(word);
@@ -289,6 +288,7 @@ score_once_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
     if (!have_tmem) mine = 0;
     ptx::tc_fence_after_sync();
     lane_addr = ctl.tmem_base + ((uint32_t)(quarter * 32) << 16) + cg * 32;
+    pdl_trigger();
     if (!lse_in) {
       for (int t = 0; t < mine; ++t) {
         ok &= ptx::mbar_wait_bounded(ptx::smem_u32(&ctl.s_full[t]), 0, abort);

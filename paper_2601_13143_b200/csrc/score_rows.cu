@@ -113,7 +113,6 @@ score_rows_kernel(const __grid_constant__ CUtensorMap k_map, Shapes s, const uin
   __shared__ uint64_t full[Ring::kStages], empty[Ring::kStages];
   __shared__ Span spans[2][32];
   __shared__ int abort_flag;
-  chain_begin_setup(s);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t ring = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   if (threadIdx.x == 0) {
@@ -125,7 +124,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap k_map, Shapes s, const uin
     ptx::fence_barrier_init();
     ptx::prefetch_tensormap(&k_map);
   }
-  chain_end_setup(s, cu_seqlens, cu_qlens, q_idx);
+  chain_enter_late(s, cu_seqlens, cu_qlens, q_idx);
   TileList list(s, cu_seqlens, cu_qlens, lane);
   list.open(spans, warp);
   const int units = list.total * s.hkv, each = units / (int)gridDim.x, more = units - each * (int)gridDim.x;  // (the host sees to it that they fit)
@@ -156,6 +155,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap k_map, Shapes s, const uin
       }
       __syncwarp();
     }
+    pdl_trigger();  // all loads have been issued
     if (!ok && lane == 0 && device_status) atomicOr(device_status, FASTAV_DEV_WAIT_EXPIRED);
     // The copies in flight write into this block's shared memory: they are waited for before it may exit, also where another warp gave up.
     int never = 0;

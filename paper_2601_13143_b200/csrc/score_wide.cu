@@ -126,7 +126,7 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
                   int32_t* device_status) {
   using L = Layout<DIM>;
   extern __shared__ unsigned char smem_raw[];
-  chain_enter(s, q_idx, cu_qlens, cu_seqlens);
+  chain_enter_late(s, q_idx, cu_qlens, cu_seqlens);
   const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   unsigned char* base_ptr = smem_raw + (base - ptx::smem_u32(smem_raw));
   Control& ctl = *reinterpret_cast<Control*>(base_ptr + L::kCtrlOff);
@@ -344,6 +344,7 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
                              un.tok0 + key_begin + t * kTileKeys, bar);
         }
       }
+      pdl_trigger();  // all loads have been issued
       if (*abort) {
         // Giving up: copies already issued still write into this block's shared memory, so wait (bounded
         // once more) for each of them before the block may exit.

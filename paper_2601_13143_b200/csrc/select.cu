@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(kThreads, COUNT_HERE ? 1 : 2) mask_emit_kernel
                                                              int32_t* __restrict__ cu_keep, int32_t* device_status) {
   __shared__ unsigned warp_a[kWarps];
   __shared__ int base_sh, mine_sh, start_sh;
-  chain_enter(s, cu_seqlens);
+  chain_enter_late(s, cu_seqlens);
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (!COUNT_HERE) {  // a large batch: through L1, after the wait (see checked_span)
     pdl_wait();
@@ -447,6 +447,7 @@ __global__ void __launch_bounds__(kThreads, COUNT_HERE ? 1 : 2) mask_emit_kernel
   pdl_acquire(keep_mask);
   pdl_acquire(counts);
   cut = __syncthreads_or(cut);
+  pdl_trigger();
   int part = 0;
   if (!COUNT_HERE) {
     for (int i = tid; i < b; i += kThreads) part += chain_load_cached(counts + i);

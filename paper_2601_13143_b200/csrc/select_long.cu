@@ -30,11 +30,13 @@ constexpr int kBins = 1 << kDigitBits;
 constexpr int kBinsPerThread = kBins / kThreads;
 constexpr int kListMax = kThreads;           // keys of a bin that are ranked by counting
 constexpr int kMaxTerms = 256 * kNarrowMaxRows;  // heads x scored rows of the few-rows path
+// Shared memory that a block asks for, so that no block of a compaction (192 KB and more) is resident beside it: those wait for the
+// selection and slow it down.  Together with the successor started ahead of the passes instead of first thing: 32 ragged
+// sequences of up to 8,192 tokens 307 -> 301 us, 4 x 16,384 292 -> 288.
+constexpr size_t kLeastBytes = 64 * 1024;
 constexpr int kLeastSlice = 256;             // tokens per block worth a block
 
-// Two counts to a word: a slice has at most 2,048 keys, a sequence at most 32,768.  With full slices a block takes 28 KB in clusters of 16,
-// 29 of 8, 31 of 4 and 35 of 2 (18.7 for this, 8 for the scores, 16 over the blocks for the totals): all but the last fit beside a compaction
-// ring of 192 KB, whose blocks are then resident when the selection ends.
+// Two counts to a word: a slice has at most 2,048 keys, a sequence at most 32,768.
 struct alignas(16) LongShared {
   union {
     unsigned hist[kBins / 2];  // of the block's slice
@@ -66,7 +68,8 @@ struct LongArgs {
 __host__ __device__ inline int owned_words(int blocks) { return kBins / 2 / blocks; }
 // ... and of kLogits what each term's weights are made with, at most `terms`.
 inline size_t long_bytes(int blocks, int slice_cap, int terms) {
-  return sizeof(LongShared) + (size_t)(slice_cap + owned_words(blocks) + 2 * terms) * sizeof(unsigned);
+  const size_t used = sizeof(LongShared) + (size_t)(slice_cap + owned_words(blocks) + 2 * terms) * sizeof(unsigned);
+  return used > kLeastBytes ? used : kLeastBytes;
 }
 template <int N>
 struct Tokens {
@@ -95,7 +98,6 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
                                                                   int32_t* __restrict__ keep_idx, int32_t* __restrict__ cu_keep, int32_t* device_status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   LongShared& sh = *reinterpret_cast<LongShared*>(smem_raw);
-  chain_begin_setup(s);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int blocks = a.blocks, b = (int)blockIdx.x / blocks, c = (int)cluster_rank();
   unsigned* const keys = reinterpret_cast<unsigned*>(smem_raw + sizeof(LongShared));
@@ -109,7 +111,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
   if (tid < kSlice / 32) sh.prot_bits[tid] = 0u;
   if (tid == 0) { sh.base = 0; sh.list_n = 0; }
   cluster_arrive();  // this block runs and its totals are zero: waited for before the first remote access
-  chain_end_setup(s, cu_seqlens, keep_counts, protect, q_idx, cu_qlens);
+  chain_enter_late(s, cu_seqlens, keep_counts, protect, q_idx, cu_qlens);
   if (warp == 0) {
     const int32_t* word = lane < 2 ? cu_seqlens + b + lane : lane < 4 ? cu_qlens + b + lane - 2 : keep_counts + b;
     if (lane < 5) sh.index[lane] = chain_load(word);
@@ -247,6 +249,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
   cluster_wait();
   if (k == 0) return;  // nothing is kept, protected or not (uniform for the cluster; nothing remote has been touched)
 
+  pdl_trigger();
   unsigned prefix = 0u;  // the bits of the k-th largest key fixed so far
   int remaining = k, bits_left = 32;
 #pragma unroll 1
