@@ -3,16 +3,18 @@
 // are selected (Section 2.2; ties to the lower index, protected tokens always).  One thread-block cluster per sequence, a slice of
 // at most 2,048 tokens per block.
 //
-// The keys stay where they are.  A pass takes 13 bits: each block counts its slice's digits, adds the bins it has to the block that
+// The keys stay where they are.  A pass takes 11 bits: each block counts its slice's digits, adds the bins it has to the block that
 // owns them (distributed shared memory), and after a cluster barrier each reads all totals and finds the bin of the k-th largest
-// for itself.  Where that bin holds at most 512 keys every block fetches them and ranks them by counting, else the next pass
-// follows.  Then the blocks tell one another how many of theirs lie above and on the threshold, and write their survivors.
+// for itself.  Where that bin holds at most 512 keys the blocks send one another theirs and how many they have above the bin, and each
+// ranks them all by counting, else the next pass follows.  From that each block also knows what the blocks before it keep.
 //
-// Bound: latency, a chain of a dozen steps of which four are cluster barriers.  It saves the kernel that added the sums up; against
-// that and a selection by one block: 3 x 8,001-9,001 tokens with the log-sum-exp given 74.0 -> 72.5 us, 1 to 3 % of a
-// call on a few thousand tokens, 0.3 % of one on 4 x 16,384.  From logits it saves two kernels (statistics, scores).  Clusters of 4, 8 or 16 make no
-// difference.  From finished scores (fastav_select) nothing is saved and one block stays quicker: 4 x 6,554 tokens 109.8 us against 111.7,
-// 32 ragged sequences 217.8 against 219.7 (of the calls that had finished scores then).
+// Bound: latency, a chain of a dozen steps of which three are cluster barriers; from the wait to the end 8.3 us (3 x 8,001-9,001 tokens) to 9.2
+// (4 x 16,384), of that 1 to 2.5 for the sums, 1.3 for the bins' exchange, 1.1 for the lists'.  13 bits from the first one on put 16
+// bins on an octave instead of 32 (lists of 300 keys, 3.1 us to rank) and had four barriers: 12.5 us and 13; 13 bits of the window
+// spread over more bins than their exchange pays for (2.2 to 3.3 us).  In calls, us: 3 x 8,001-9,001 tokens, log-sum-exp given 72.6 -> 69.2, 4 x 6,554 96.5 -> 95.1.
+// It saves the kernel that added the sums up, and from logits those for statistics and scores.  Clusters of 4, 8 or 16 make no
+// difference.  From finished scores (fastav_select) nothing is saved, and one block was quicker: 4 x 6,554 tokens 109.8 us against 111.7, 32
+// ragged sequences 217.8 against 219.7 (calls that had finished scores then).
 #include "cluster.cuh"
 #include "common.cuh"
 #include "row_stats.cuh"
@@ -25,31 +27,33 @@ constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr int kPer = 4;                      // keys per thread
 constexpr int kSlice = kPer * kThreads;      // most tokens of a block
-constexpr int kDigitBits = 13;
+constexpr int kDigitBits = 11;
 constexpr int kBins = 1 << kDigitBits;
-constexpr int kBinsPerThread = kBins / kThreads;
+constexpr int kBinsPerThread = kBins / kThreads;  // two words of two counts
 constexpr int kListMax = kThreads;           // keys of a bin that are ranked by counting
 constexpr int kMaxTerms = 256 * kNarrowMaxRows;  // heads x scored rows of the few-rows path
 // Shared memory that a block asks for, so that no block of a compaction (192 KB and more) is resident beside it: those wait for the
 // selection and slow it down.  Together with the successor started ahead of the passes instead of first thing: 32 ragged
 // sequences of up to 8,192 tokens 307 -> 301 us, 4 x 16,384 292 -> 288.
 constexpr size_t kLeastBytes = 64 * 1024;
+constexpr int kSent = 32;                    // keys that a block sends to the others
 constexpr int kLeastSlice = 256;             // tokens per block worth a block
 
 // Two counts to a word: a slice has at most 2,048 keys, a sequence at most 32,768.
 struct alignas(16) LongShared {
   union {
-    unsigned hist[kBins / 2];  // of the block's slice
-    unsigned all[kListMax];    // the cluster's list
+    unsigned hist[kBins / 2];          // of the block's slice
+    unsigned sent[kMaxCluster][kSent]; // what the cluster's blocks have in their lists
+    unsigned all[kListMax];            // ... fetched from where it lies
   };
   unsigned prot_bits[kSlice / 32];
   unsigned list[kListMax];
   unsigned warp_a[kWarps], warp_b[kWarps];
-  unsigned count_of[kMaxCluster];  // keys in each block's list
+  unsigned count_of[kMaxCluster];  // keys in each block's list (low half), keys above the list's bin (high half)
   unsigned kept_of[kMaxCluster];   // keys above the threshold (low half) and on it (high half)
   int index[8];
   int base, list_n, remaining, bucket, need_eq;
-  unsigned prefix, threshold, own;
+  unsigned prefix, threshold, own, above_n, earlier;
 };
 
 enum Front { kPartials, kLogits };
@@ -85,10 +89,36 @@ __device__ __forceinline__ unsigned remote_load(uint32_t a) {
   asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
   return v;
 }
-__device__ __forceinline__ uint4 remote_load4(uint32_t a) {  // 16-byte aligned
-  uint4 v;
-  asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+__device__ __forceinline__ uint2 remote_load2(uint32_t a) {  // 8-byte aligned
+  uint2 v;
+  asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a) : "memory");
   return v;
+}
+
+// rank_finish for a list that may be longer: lanes of a warp share a key where the block has more threads than there are keys, each
+// compares it with every so many quads (300 keys: 3.1 us one after the other).
+__device__ __forceinline__ void rank_list(const unsigned* list, int count, int remaining, int tid, unsigned* threshold, int* need_eq) {
+  const int log_lanes = min(5, 31 - __clz(kThreads) - (32 - __clz(count - 1))), lanes = 1 << log_lanes;  // lanes x count <= kThreads
+  const int at = tid >> log_lanes, part = tid & (lanes - 1), whole = count >> 2;
+  const bool active = at < count;
+  const unsigned mine = active ? list[at] : 0u;
+  int both = 0;  // keys above in the high half, equal ones in the low half
+  if (active) {
+#pragma unroll 2
+    for (int i = part; i < whole; i += lanes) {
+      const uint4 v = *reinterpret_cast<const uint4*>(list + 4 * i);
+      both += (v.x > mine ? 0x10000 : 0) + (v.y > mine ? 0x10000 : 0) + (v.z > mine ? 0x10000 : 0) + (v.w > mine ? 0x10000 : 0);
+      both += (v.x == mine) + (v.y == mine) + (v.z == mine) + (v.w == mine);
+    }
+    for (int i = 4 * whole + part; i < count; i += lanes) both += (list[i] > mine ? 0x10000 : 0) + (list[i] == mine);
+  }
+  __syncwarp();
+  for (int d = lanes / 2; d; d >>= 1) both += __shfl_xor_sync(0xFFFFFFFFu, both, d);
+  const int above = both >> 16, equal = both & 0xFFFF;
+  if (active && part == 0 && above < remaining && remaining <= above + equal) {
+    *threshold = mine;
+    *need_eq = remaining - above;
+  }
 }
 
 template <Front FRONT>
@@ -109,7 +139,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
   };
   clear_counts();
   if (tid < kSlice / 32) sh.prot_bits[tid] = 0u;
-  if (tid == 0) { sh.base = 0; sh.list_n = 0; }
+  if (tid == 0) { sh.base = 0; sh.list_n = 0; sh.above_n = 0u; sh.earlier = 0u; }
   cluster_arrive();  // this block runs and its totals are zero: waited for before the first remote access
   chain_enter_late(s, cu_seqlens, keep_counts, protect, q_idx, cu_qlens);
   if (warp == 0) {
@@ -126,14 +156,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
   k = k < 0 ? 0 : (k > n ? n : k);
   const bool lowest = (s.flags & FASTAV_SELECT_LOWEST) != 0;
 
-  pdl_wait();
-  const float* in = a.in;
-  pdl_acquire(in);
-  if (tid == 0 && c == 0 && device_status) {
-    if (seq.bad || qrows.bad) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
-    if (k_clamped) atomicOr(device_status, FASTAV_DEV_K_CLAMPED);
-  }
-  {  // output offset: the clamped keep counts of the sequences before this one, 32 per warp
+  {  // ahead of the wait: the output offset, the clamped keep counts of the sequences before this one, 32 per warp
     if (warp * 32 < b) {
       int part = 0;
 #pragma unroll 1
@@ -155,6 +178,13 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
         const unsigned word = __ballot_sync(0xFFFFFFFFu, j < m && chain_load(protect + tok0 + t0 + j) != 0);
         if (lane == 0 && word) atomicOr(&sh.prot_bits[j0 >> 5], word);
       }
+  }
+  pdl_wait();
+  const float* in = a.in;
+  pdl_acquire(in);
+  if (tid == 0 && c == 0 && device_status) {
+    if (seq.bad || qrows.bad) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
+    if (k_clamped) atomicOr(device_status, FASTAV_DEV_K_CLAMPED);
   }
   const float* const col = in + tok0 + t0;
   const int rows = FRONT == kLogits ? min(qrows.count, a.rq) : 0, terms = s.hq * rows;  // term i = (head i / rows, row i % rows)
@@ -250,13 +280,23 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
   if (k == 0) return;  // nothing is kept, protected or not (uniform for the cluster; nothing remote has been touched)
 
   pdl_trigger();
+  // The first pass looks at scores from 2^-63 up to 2 only: three leading bits are the same there, so that a bin is 1/32 of an octave
+  // wide instead of 1/4, and the bin of the k-th largest holds few keys.  Smaller scores share the lowest bin, larger ones
+  // (and protected tokens) the highest; where the k-th largest lies in one of these two the passes start again from the first bit.
+  constexpr int kWindowShift = 29 - kDigitBits;  // three leading bits, then the digit
+  const int window = lowest ? 2 << kDigitBits : 5 << kDigitBits;
+  bool windowed = true;
   unsigned prefix = 0u;  // the bits of the k-th largest key fixed so far
   int remaining = k, bits_left = 32;
+  bool listed = false;   // the threshold comes from the cluster's list
+  bool pulls = false;    // ... which was fetched
+  unsigned list_key = 0u;
+  int list_from = kMaxCluster;
 #pragma unroll 1
-  while (bits_left > 0) {
-    const int shift = max(0, bits_left - kDigitBits);
+  for (int pass = 0; bits_left > 0; ++pass) {
+    const int shift = windowed ? kWindowShift : max(0, bits_left - kDigitBits);
     const unsigned above_want = __funnelshift_rc(prefix, 0u, bits_left);  // prefix >> bits_left, 0 for 32
-    if (bits_left < 32) {
+    if (pass > 0) {
       cluster_sync();  // everybody has read the totals
       clear_counts();
       cluster_sync();
@@ -266,7 +306,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
 #pragma unroll
       for (int u = 0; u < kPer; ++u) {
         if (u < mine && __funnelshift_rc(x[u], 0u, bits_left) == above_want) {
-          const unsigned digit = (x[u] >> shift) & (kBins - 1);
+          const unsigned digit = windowed ? (unsigned)min(max((int)(x[u] >> kWindowShift) - window, 0), kBins - 1) : (x[u] >> shift) & (kBins - 1);
           if (digit != run_digit) {
             if (run_len) atomicAdd(&sh.hist[run_digit >> 1], run_len << (16 * (run_digit & 1)));
             run_digit = digit;
@@ -279,27 +319,22 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
     }
     __syncthreads();
     constexpr int kWords = kBinsPerThread / 2;
+    static_assert(kWords == 2);
     const int first_word = tid * kWords, owner = first_word / owned;
     const uint32_t owner_at = remote(&totals[first_word & (owned - 1)], owner);
-#pragma unroll
-    for (int i = 0; i < kWords; i += 4) {
-      const uint4 v = *reinterpret_cast<const uint4*>(&sh.hist[first_word + i]);
-      if (v.x) remote_add(owner_at + 4 * i, v.x);
-      if (v.y) remote_add(owner_at + 4 * i + 4, v.y);
-      if (v.z) remote_add(owner_at + 4 * i + 8, v.z);
-      if (v.w) remote_add(owner_at + 4 * i + 12, v.w);
+    {
+      const uint2 v = *reinterpret_cast<const uint2*>(&sh.hist[first_word]);
+      if (v.x) remote_add(owner_at, v.x);
+      if (v.y) remote_add(owner_at + 4, v.y);
     }
     cluster_sync();
     unsigned h[kBinsPerThread], own = 0;
-#pragma unroll
-    for (int i = 0; i < kWords; i += 4) {
-      const uint4 v = remote_load4(owner_at + 4 * i);
-      const unsigned w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        h[2 * (i + j)] = w[j] & 0xFFFFu;
-        h[2 * (i + j) + 1] = w[j] >> 16;
-      }
+    {
+      const uint2 v = remote_load2(owner_at);
+      h[0] = v.x & 0xFFFFu;
+      h[1] = v.x >> 16;
+      h[2] = v.y & 0xFFFFu;
+      h[3] = v.y >> 16;
     }
 #pragma unroll
     for (int i = 0; i < kBinsPerThread; ++i) own += h[i];
@@ -309,7 +344,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
 #pragma unroll
       for (int i = kBinsPerThread - 1; i >= 0; --i) {
         if (above < rem && rem <= above + h[i]) {
-          sh.prefix = prefix | ((unsigned)(2 * first_word + i) << shift);
+          sh.prefix = windowed ? (unsigned)(2 * first_word + i) : prefix | ((unsigned)(2 * first_word + i) << shift);
           sh.remaining = (int)(rem - above);
           sh.bucket = (int)h[i];
         }
@@ -317,28 +352,60 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
       }
     }
     __syncthreads();
-    prefix = sh.prefix;
-    remaining = sh.remaining;
+    const unsigned found = sh.prefix;
     const int bucket = sh.bucket;
+    if (windowed) {
+      windowed = false;
+      if (found == 0u || found == kBins - 1) continue;  // (prefix and remaining as they were)
+      prefix = ((unsigned)window + found) << kWindowShift;
+    } else {
+      prefix = found;
+    }
+    remaining = sh.remaining;
     bits_left = shift;
     if (bits_left > 0 && bucket <= kListMax) {  // few keys left in the cluster: everybody fetches them and finds their ranks by counting
+      unsigned over = 0u;
 #pragma unroll
-      for (int u = 0; u < kPer; ++u)
+      for (int u = 0; u < kPer; ++u) {
         if (u < mine && (x[u] >> bits_left) == (prefix >> bits_left)) sh.list[atomicAdd(&sh.list_n, 1)] = x[u];
+        over += u < mine && (x[u] >> bits_left) > (prefix >> bits_left);
+      }
+      over = __reduce_add_sync(0xFFFFFFFFu, over);
+      if (lane == 0 && over) atomicAdd(&sh.above_n, over);
       __syncthreads();
-      if (tid < blocks) remote_store(remote(&sh.count_of[c], tid), (unsigned)sh.list_n);
+      const int here = sh.list_n;
+      if (tid < blocks) remote_store(remote(&sh.count_of[c], tid), (unsigned)here | sh.above_n << 16);
+      if (here <= kSent)
+        for (int i = tid; i < here * blocks; i += kThreads) remote_store(remote(&sh.sent[c][i / blocks], i & (blocks - 1)), sh.list[i / blocks]);
       cluster_sync();
-      if (tid < bucket) {
-        int at = tid, from = 0;
-        while (from < blocks - 1 && at >= (int)sh.count_of[from]) at -= (int)sh.count_of[from++];
-        sh.all[tid] = remote_load(remote(&sh.list[at & (kListMax - 1)], from));
+      const int count = lane < blocks ? (int)(sh.count_of[lane] & 0xFFFFu) : 0;
+      const unsigned* ranked = sh.list;
+      pulls = __any_sync(0xFFFFFFFFu, count > kSent);  // (the same for the whole cluster)
+      if (!pulls) {  // warp w has block w's
+        const int start = (int)__reduce_add_sync(0xFFFFFFFFu, lane < warp ? count : 0), own = __shfl_sync(0xFFFFFFFFu, count, warp & 31);
+        if (lane < own) {
+          list_key = sh.sent[warp][lane];
+          list_from = warp;
+          sh.list[start + lane] = list_key;
+        }
+      } else {
+        if (tid < bucket) {
+          int at = tid, from = 0;
+          while (from < blocks - 1 && at >= (int)(sh.count_of[from] & 0xFFFFu)) at -= (int)(sh.count_of[from++] & 0xFFFFu);
+          list_key = remote_load(remote(&sh.list[at & (kListMax - 1)], from));
+          list_from = from;
+          sh.all[tid] = list_key;
+        }
+        cluster_arrive();  // nothing remote from here on: waited for before the block may exit
+        ranked = sh.all;
       }
       __syncthreads();
-      rank_finish(sh.all, bucket, remaining, tid, &sh.threshold, &sh.need_eq);
+      rank_list(ranked, bucket, remaining, tid, &sh.threshold, &sh.need_eq);
       __syncthreads();
       prefix = sh.threshold;
       remaining = sh.need_eq;
       bits_left = 0;
+      listed = true;
     }
   }
   const unsigned T = prefix;
@@ -346,17 +413,30 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
   unsigned both = 0;              // keys above the threshold in the low half, keys equal to it in the high half
 #pragma unroll
   for (int u = 0; u < kPer; ++u) both += u < mine ? (x[u] > T ? 1u : 0u) + (x[u] == T ? 0x10000u : 0u) : 0u;
+  // The blocks before this one: how many of theirs lie above and on the threshold.  From the list and the counts beside it every
+  // block works that out for itself; without a list they tell one another.
+  if (listed) {
+    unsigned part = list_from < c ? (list_key > T ? 1u : 0u) + (list_key == T ? 0x10000u : 0u) : 0u;
+    if (warp == 0 && lane < c) part += sh.count_of[lane] >> 16;
+    part = __reduce_add_sync(0xFFFFFFFFu, part);
+    if (lane == 0 && part) atomicAdd(&sh.earlier, part);
+  }
   const unsigned before = sum_before<kWarps>(both, sh.warp_b, lane, warp);
-  if (tid == kThreads - 1) sh.own = before + both;
-  __syncthreads();
-  if (tid < blocks) remote_store(remote(&sh.kept_of[c], tid), sh.own);
-  cluster_sync();  // the last remote access
-  const unsigned there = lane < blocks ? sh.kept_of[lane] : 0u, earlier = lane < c ? there : 0u;
-  int gt = (int)(before & 0xFFFFu) + (int)__reduce_add_sync(0xFFFFFFFFu, earlier & 0xFFFFu);
-  int eq = (int)(before >> 16) + (int)__reduce_add_sync(0xFFFFFFFFu, earlier >> 16);
-  if (c == 0 && warp == 0 && T == kProtectedKey) {
-    const int all_eq = (int)__reduce_add_sync(0xFFFFFFFFu, there >> 16);
-    if (lane == 0 && all_eq > need_eq && device_status) atomicOr(device_status, FASTAV_DEV_PROTECT_OVERFLOW);  // more protected tokens than k
+  unsigned earlier;
+  if (listed) {
+    earlier = sh.earlier;
+  } else {
+    if (tid == kThreads - 1) sh.own = before + both;
+    __syncthreads();
+    if (tid < blocks) remote_store(remote(&sh.kept_of[c], tid), sh.own);
+    cluster_sync();  // the last remote access
+    earlier = __reduce_add_sync(0xFFFFFFFFu, lane < c ? sh.kept_of[lane] : 0u);
+  }
+  int gt = (int)(before & 0xFFFFu) + (int)(earlier & 0xFFFFu);
+  int eq = (int)(before >> 16) + (int)(earlier >> 16);
+  if (T == kProtectedKey) {  // more protected tokens than k? (uniform for the block)
+    const int all_eq = listed ? __syncthreads_count(list_from < kMaxCluster && list_key == T) : sh.bucket;
+    if (c == 0 && tid == 0 && all_eq > need_eq && device_status) atomicOr(device_status, FASTAV_DEV_PROTECT_OVERFLOW);
   }
   const int offset = ((s.flags & FASTAV_KEEP_IDX_GLOBAL) ? tok0 : 0) + t0 + kPer * tid;
 #pragma unroll
@@ -367,6 +447,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
     gt += is_gt;
     eq += is_eq;
   }
+  if (pulls) cluster_wait();
 }
 
 // Blocks per sequence, as many as run at once and have a slice worth it; 0 where the longest sequence does not fit.

@@ -41,3 +41,42 @@ def test_flags_of_the_selection(lens, lowest, global_idx, by_rows, lse):
     p.q_idx = torch.tensor([j for r in rows for j in r], dtype=torch.int32)
     protect = (torch.arange(p.total_tokens) % 37 == 5).to(torch.uint8) if len(lens) % 4 else None
     parity.check_prune_under_flags(p, lowest, global_idx, by_rows, lse, protect, f"{lens[0]} x {len(lens)}")
+
+
+# The first pass looks at scores from 2^-63 to 2 in bins of 1/32 octave.  `crowd`: a hundred different scores within one or two bins and one
+# block's slice, the k-th largest among them (more than a block sends; some 40 per block where the bin has more); `small`: all scores but one
+# below 2^-63; `hidden`: most tokens behind the scored rows (score 0) and k beyond the others; `above`: the k-th largest is protected.
+@pytest.mark.parametrize("kind", ["crowd", "wide_crowd", "small", "hidden", "above"])
+@pytest.mark.parametrize("lens", [[2049], [5000, 2100], [17000]], ids=lambda v: f"{len(v)}x{max(v)}")
+@pytest.mark.parametrize("rows", [1, 9])
+@pytest.mark.parametrize("lowest", [False, True])
+def test_window_of_the_first_pass(kind, lens, rows, lowest):
+    p = W.random_problem(seed=sum(lens) + rows, lens=lens, rows=[rows] * len(lens), keeps=[n // 2 for n in lens], num_q_heads=2, num_kv_heads=1, head_dim=64,
+                         hidden=64)
+    gen = torch.Generator().manual_seed(rows)
+    p.softmax_scale = 1.0
+    p.q.zero_()
+    p.k.zero_()
+    p.q[..., 0], p.q[..., 1] = 8.0, 2.0 ** -13
+    protect, keeps, start = None, [], 0
+    for b, n in enumerate(lens):
+        z = (torch.rand(n, generator=gen) * 2 - 1).bfloat16()
+        tail = torch.zeros(n)
+        if kind == "crowd" or kind == "wide_crowd":
+            crowd = torch.arange(300, 400) if kind == "crowd" else torch.arange(100, n, 7)[:400]
+            z[crowd], tail[crowd] = 0.0, torch.arange(len(crowd)).float() % 128
+            above = int((z < 0).sum() if lowest else (z > 0).sum())
+            keeps.append(above + len(crowd) // 2)
+        elif kind == "small":
+            z[5] = 7.5
+            keeps.append(n // 3)
+        else:
+            keeps.append(n // 3)
+        if kind == "hidden":
+            p.q_idx[b * rows:(b + 1) * rows] = torch.arange(n // 5, n // 5 + rows)
+        p.k[start:start + n, 0, 0], p.k[start:start + n, 0, 1] = z, tail.bfloat16()
+        start += n
+    if kind == "above":
+        protect = (torch.arange(p.total_tokens) % 2).to(torch.uint8)
+    p.keep_counts = torch.tensor(keeps, dtype=torch.int32)
+    parity.check_prune_under_flags(p, lowest, False, True, False, protect, f"{kind} {lens[0]} x {len(lens)}")
