@@ -342,18 +342,20 @@ cudaError_t enqueue_selection(const fastav_params& params, const void* q, const 
   *gathered = false;
   if (s.total_tokens > 0) e = launch_score(s, w, q, q_idx, cu_qlens, k, cu_seqlens, lse_opt, scores_out, ws, device_status, st, &left);
   if (e != cudaSuccess) return e;
-  const SelectArgs t{cu_seqlens, keep_counts, protect_opt, q_idx, cu_qlens, keep_idx_out, cu_keep_out, device_status};
+  SelectArgs t{cu_seqlens, keep_counts, protect_opt, q_idx, cu_qlens, keep_idx_out, cu_keep_out, device_status};
   const int row_bytes = rows && s.total_keep > 0 ? row_bytes_of(s, *rows) : 0;
-  if (left.kind == ScoreLeft::kKeys) {
-    *gathered = row_bytes > 0 && few_gathers(s, row_bytes);
-    return launch_few(s, q, k, lse_opt, scores_out, true, *gathered ? rows : nullptr, t, st);
-  }
   if (left.kind == ScoreLeft::kLogits) return launch_long_logits(s, w, ws, lse_opt, scores_out, t, st);
   if (left.kind == ScoreLeft::kPartials && !cluster_select_applies(s))
     return launch_long_partials(s, reinterpret_cast<const float*>(ws + w.partial_off), left, scores_out, t, st);
-  if (left.kind == ScoreLeft::kPartials) {
-    *gathered = row_bytes > 0 && cluster_select_gathers(s, row_bytes);
-    return launch_select_partials(s, reinterpret_cast<const float*>(ws + w.partial_off), left, scores_out, *gathered ? rows : nullptr, t, st);
+  if (left.kind == ScoreLeft::kKeys || left.kind == ScoreLeft::kPartials) {  // a cluster per sequence, and the gather here or right behind
+    const bool from_keys = left.kind == ScoreLeft::kKeys;
+    const bool here = row_bytes > 0 && (from_keys ? few_gathers(s, row_bytes) : cluster_select_gathers(s, row_bytes));
+    const bool placed = from_keys && row_bytes > 0 && !here && placed_compact_applies(s, *rows);
+    *gathered = here || placed;
+    if (placed) t.place = reinterpret_cast<int32_t*>(ws + w.keys_off);
+    e = from_keys ? launch_few(s, q, k, lse_opt, scores_out, true, here ? rows : nullptr, t, st)
+                  : launch_select_partials(s, reinterpret_cast<const float*>(ws + w.partial_off), left, scores_out, here ? rows : nullptr, t, st);
+    return placed && e == cudaSuccess ? launch_compact_placed(s, *rows, t.place, cu_seqlens, device_status, st) : e;
   }
   return launch_select(s, w, scores_out, cu_seqlens, keep_counts, protect_opt, q_idx, cu_qlens, keep_idx_out, cu_keep_out, ws, device_status, st);
 }

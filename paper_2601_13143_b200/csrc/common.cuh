@@ -46,7 +46,7 @@ struct Workspace {
   size_t partial_off = 0;   // float  [Hkv * row chunks][N]        score partials per KV head and chunk of query rows
   size_t logits_off = 0;    // float  [Hq][max_qlen][N] (matrix-vector path only; 0 bytes otherwise)
   // select
-  size_t keys_off = 0;      // uint32 [N] (only when a sequence does not fit in shared memory)
+  size_t keys_off = 0;      // uint32 [N] (only when a sequence does not fit in shared memory); a prune call: a token's place among the survivors
   int stat_tiles = 0;
 };
 
@@ -103,6 +103,7 @@ struct SelectArgs {
   const uint8_t* protect;
   const int32_t *q_idx, *cu_qlens;
   int32_t *keep_idx, *cu_keep, *device_status;
+  int32_t* place = nullptr;  // launch_few, optional, [N]: where a token's row goes among the survivors, -1 if it is dropped
 };
 bool few_applies(const Shapes& s);              // from the keys
 bool cluster_select_applies(const Shapes& s);   // from partial sums or scores
@@ -148,6 +149,12 @@ cudaError_t launch_compact(const Shapes& s, const int32_t* keep_idx, const int32
                            const int32_t* cu_seqlens, const void* hidden_in, void* hidden_out, const int32_t* pos_in,
                            int32_t* pos_out, const void* k_in, void* k_out, const void* v_in, void* v_out,
                            int32_t* device_status, cudaStream_t stream);
+
+// The same for a call whose rows shared memory holds, behind launch_few: they are read while that kernel selects, which leaves every
+// token's place for it (SelectArgs::place).
+bool placed_compact_applies(const Shapes& s, const RowStreams& rows);
+cudaError_t launch_compact_placed(const Shapes& s, const RowStreams& rows, const int32_t* place, const int32_t* cu_seqlens, int32_t* device_status,
+                                  cudaStream_t stream);
 
 int32_t validate_prune(const fastav_params* params, const void* q, const int32_t* q_idx, const int32_t* cu_qlens, const void* k,
                        const void* v, const int32_t* cu_seqlens, const int32_t* keep_counts, const void* hidden_in,

@@ -248,6 +248,94 @@ compact_rows_bulk_kernel(Shapes s, RowStreams t, const int32_t* __restrict__ kee
   bulk_wait_all();  // the slots and the outputs are this kernel's until every store has landed
 }
 
+// ---- rows read ahead ----------------------------------------------------------------------------------
+// Where shared memory holds all rows of a call, survivors or not, they need not wait for the selection: every warp reads some tokens' rows
+// while the kernel before this one selects, and when that has ended asks for their places among the survivors and stores the rows that
+// have one.  (That kernel lets this one start after its own wait: the rows are complete by then.)
+// What it saves is a trip to memory for the list and one for the rows.  13 fine stages from 744 tokens 148.6 -> 138.5 us, three from
+// 1,024 37.9 -> 36.1, 11 from 576 with rows of 6 KB 125 -> 119.  Rows below 2 KB gain nothing (11 stages from 649, 1.5 KB: 104.6 -> 105.9), and
+// behind the selection from partial sums, which is shorter, dropped rows cost more than is saved (9 x 132 tokens 14.4 -> 14.9).
+constexpr int kPlacedMaxSequences = 31;  // bounds kept one per lane
+constexpr int kPlacedLeastRow = 2048;    // bytes
+__global__ void __launch_bounds__(kBulkMaxWarps * 32, 1)
+compact_placed_kernel(Shapes s, RowStreams t, const int32_t* __restrict__ place, const int32_t* __restrict__ cu_seqlens, int n_segments, int packed_k, int packed_v,
+                      int row_bytes, int slots, int32_t* device_status) {
+  extern __shared__ __align__(128) unsigned char bulk_smem[];
+  __shared__ uint64_t full[kBulkMaxWarps];
+  chain_enter(s, cu_seqlens);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+  const uint32_t ring = ptx::smem_u32(bulk_smem) + (uint32_t)warp * slots * row_bytes, bar = ptx::smem_u32(&full[warp]);
+  Segment seg{};
+  const bool active = lane < n_segments && make_segment(s, t, lane, packed_k != 0, packed_v != 0, seg);
+  if (lane == 0) {
+    ptx::mbar_init(bar, 1);
+    ptx::fence_barrier_init();
+  }
+  // Lane i has row i of the warp; it counts if it lies in a sequence as the selection sees it (a cut one's rest has no place).
+  const int seq_at = lane <= s.batch ? chain_load(cu_seqlens + lane) : 0;
+  const int row = blockIdx.x + gridDim.x * (warp + warps * lane);
+  bool there = false;
+  for (int b = 0; b < s.batch; ++b) {
+    const Span seq = checked_words(__shfl_sync(0xFFFFFFFFu, seq_at, b), __shfl_sync(0xFFFFFFFFu, seq_at, b + 1), s.total_tokens, s.max_seqlen);
+    there |= lane < slots && row >= seq.first && row < seq.first + seq.count;
+  }
+  const unsigned mine = __ballot_sync(0xFFFFFFFFu, there);
+  if (lane == 0 && mine) ptx::mbar_arrive_expect_tx(bar, __popc(mine) * row_bytes);
+  __syncwarp();
+  for (unsigned left = mine; left; left &= left - 1) {
+    const int i = __ffs(left) - 1;
+    const long long src = __shfl_sync(0xFFFFFFFFu, row, i);
+    if (active) bulk_load(ring + i * row_bytes + seg.slot_off, seg.in + src * seg.in_stride, seg.bytes, bar);
+  }
+  const int pos = there && t.pos_in ? chain_load(t.pos_in + row) : 0;
+  pdl_wait();
+  pdl_acquire(place);
+  const int at = there ? chain_load(place + row) : -1;
+  const unsigned kept = __ballot_sync(0xFFFFFFFFu, at >= 0 && at < s.total_keep);
+  if (((kept >> lane) & 1u) && t.pos_in) t.pos_out[at] = pos;
+  int abort_flag = 0;
+  if (mine && !ptx::mbar_wait_warp(bar, 0, &abort_flag)) {
+    if (lane == 0 && device_status) atomicOr(device_status, FASTAV_DEV_WAIT_EXPIRED);
+    int never = 0;  // the copies in flight write into this block's shared memory: waited for once more
+    ptx::mbar_wait_bounded(bar, 0, &never);
+    return;
+  }
+  for (unsigned left = kept; left; left &= left - 1) {
+    const int i = __ffs(left) - 1;
+    const long long dst = __shfl_sync(0xFFFFFFFFu, at, i);
+    if (active) bulk_store(seg.out + dst * seg.out_stride, ring + i * row_bytes + seg.slot_off, seg.bytes);
+  }
+  bulk_commit();
+  bulk_wait_all();
+}
+
+struct BulkPlan {
+  bool packed_k, packed_v;
+  int n_segments, row_bytes;
+};
+// Every segment must be 16-byte friendly (it is: rows and strides are multiples of 8 elements), and there may be at most one per lane.
+BulkPlan bulk_plan(const Shapes& s, const RowStreams& t) {
+  BulkPlan p;
+  p.packed_k = t.k_in && s.k_sh == s.dim && s.ko_sh == s.dim;
+  p.packed_v = t.v_in && s.v_sh == s.dim && s.vo_sh == s.dim;
+  p.n_segments = (t.hidden_in ? 1 : 0) + (t.k_in ? (p.packed_k ? 1 : s.hkv) : 0) + (t.v_in ? (p.packed_v ? 1 : s.hkv) : 0);
+  p.row_bytes = row_bytes_of(s, t);
+  return p;
+}
+
+struct PlacedPlan {
+  int warps, slots;
+};
+// As many blocks as SMs, but no block with less than 8 rows or 16 KB: SMs without one are left to the clusters that select (744 tokens, 13
+// stages: 144.3 us with 148 blocks, 138.5 with 124; at least 32 KB 137.3, but 123.6 instead of 121.5 for 13 stages from 126).
+PlacedPlan placed_plan(const Shapes& s, int row_bytes) {
+  const int least = row_bytes > 2048 ? 16384 / row_bytes : 8, even = (s.total_tokens + kNumSMs - 1) / kNumSMs, per_block = even > least ? even : least;
+  PlacedPlan p;
+  p.slots = (per_block + kBulkMaxWarps - 1) / kBulkMaxWarps;
+  p.warps = p.slots > 0 ? (per_block + p.slots - 1) / p.slots : 0;
+  return p;
+}
+
 }  // namespace
 
 cudaError_t launch_compact(const Shapes& s, const int32_t* keep_idx, const int32_t* cu_keep,
@@ -259,11 +347,8 @@ cudaError_t launch_compact(const Shapes& s, const int32_t* keep_idx, const int32
                static_cast<const uint16_t*>(k_in),      static_cast<uint16_t*>(k_out),
                static_cast<const uint16_t*>(v_in),      static_cast<uint16_t*>(v_out),
                pos_in,                                  pos_out};
-  // Bulk-copy path: every segment must be 16-byte friendly (it is: rows and strides are multiples of 8 elements),
-  // a row must fit a slot, and there may be at most one segment per lane.
-  const bool packed_k = k_in && s.k_sh == s.dim && s.ko_sh == s.dim, packed_v = v_in && s.v_sh == s.dim && s.vo_sh == s.dim;
-  const int n_segments = (hidden_in ? 1 : 0) + (k_in ? (packed_k ? 1 : s.hkv) : 0) + (v_in ? (packed_v ? 1 : s.hkv) : 0);
-  const int row_bytes = row_bytes_of(s, t);
+  const BulkPlan plan = bulk_plan(s, t);
+  const int n_segments = plan.n_segments, row_bytes = plan.row_bytes;
   const int forced = (s.flags & FASTAV_COMPACT_PATH_MASK);
   if (forced != FASTAV_COMPACT_PATH_LOADSTORE && n_segments >= 1 && n_segments <= 32 && row_bytes > 0 &&
       kBulkStages * row_bytes <= kBulkSmemBudget) {
@@ -279,7 +364,7 @@ cudaError_t launch_compact(const Shapes& s, const int32_t* keep_idx, const int32
     const int slots = rows_per_warp < kBulkStages ? rows_per_warp : kBulkStages;
     const size_t smem = (size_t)warps * slots * row_bytes;
     e = launch_chained(compact_rows_bulk_kernel, dim3(blocks), dim3(warps * 32), smem, stream, s, t, keep_idx, cu_keep, cu_seqlens,
-                       n_segments, (int)packed_k, (int)packed_v, row_bytes, slots, device_status);
+                       n_segments, (int)plan.packed_k, (int)plan.packed_v, row_bytes, slots, device_status);
     count_launches(1);
     return e != cudaSuccess ? e : cudaGetLastError();
   }
@@ -287,6 +372,26 @@ cudaError_t launch_compact(const Shapes& s, const int32_t* keep_idx, const int32
   if (blocks > s.total_keep) blocks = s.total_keep;
   const cudaError_t e = launch_chained(compact_rows_kernel, dim3(blocks), dim3(kThreads), 0, stream, s, t, keep_idx, cu_keep,
                                        cu_seqlens, device_status);
+  count_launches(1);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+bool placed_compact_applies(const Shapes& s, const RowStreams& rows) {
+  const BulkPlan plan = bulk_plan(s, rows);
+  if ((s.flags & FASTAV_COMPACT_PATH_MASK) != 0 || s.batch > kPlacedMaxSequences || s.total_keep <= 0 || plan.row_bytes < kPlacedLeastRow || plan.n_segments > 32) return false;
+  const PlacedPlan p = placed_plan(s, plan.row_bytes);
+  return p.slots <= 32 && (long long)p.warps * p.slots * plan.row_bytes <= kBulkSmemBudget;
+}
+
+cudaError_t launch_compact_placed(const Shapes& s, const RowStreams& rows, const int32_t* place, const int32_t* cu_seqlens, int32_t* device_status,
+                                  cudaStream_t stream) {
+  const BulkPlan plan = bulk_plan(s, rows);
+  const PlacedPlan p = placed_plan(s, plan.row_bytes);
+  cudaError_t e = once_per_context([] { return cudaFuncSetAttribute(compact_placed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBulkSmemBudget); });
+  if (e != cudaSuccess) return e;
+  const int per_block = p.warps * p.slots, blocks = (s.total_tokens + per_block - 1) / per_block;
+  e = launch_chained(compact_placed_kernel, dim3(blocks), dim3(p.warps * 32), (size_t)p.warps * p.slots * plan.row_bytes, stream, s, rows, place, cu_seqlens,
+                     plan.n_segments, (int)plan.packed_k, (int)plan.packed_v, plan.row_bytes, p.slots, device_status);
   count_launches(1);
   return e != cudaSuccess ? e : cudaGetLastError();
 }

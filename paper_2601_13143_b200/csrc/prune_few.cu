@@ -65,6 +65,7 @@ struct FewArgs {
   float* scores_out;    // [N] (not used by kScores)
   int do_select;        // 0: only the scores are wanted
   int do_gather;
+  int32_t* place;       // optional: see SelectArgs
   int slice_cap;        // tokens per block that shared memory was sized for
   RowStreams rows;      // do_gather
 };
@@ -111,7 +112,7 @@ __host__ __device__ inline FewLayout few_layout(int slice_cap, int terms, int di
   return l;
 }
 
-template <Front FRONT, int DIM>
+template <Front FRONT, int DIM, bool PLACED>
 __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArgs a, const int32_t* __restrict__ cu_seqlens,
                                                                 const int32_t* __restrict__ keep_counts,
                                                                 const uint8_t* __restrict__ protect, const int32_t* __restrict__ q_idx,
@@ -393,9 +394,10 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
     }
   }
   if (!selecting) return;  // uniform for the cluster; nothing remote is outstanding
+  if (PLACED) pdl_trigger();  // the gather reads its rows meanwhile: everything ahead of this kernel has ended
   cluster_sync();          // every block has all keys
 
-  pdl_trigger();
+  if (!PLACED) pdl_trigger();
   const int base = sh.base;
   if (c == 0 && tid == 0) {
     cu_keep[b + 1] = base + k;
@@ -404,6 +406,8 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   }
   const int room = s.total_keep - base;  // of the caller's keep list, from this sequence on
   if (k == 0) {  // nothing is kept, protected or not (uniform for the cluster)
+    if (PLACED)
+      for (int j = tid; j < m; j += kThreads) a.place[tok0 + t0 + j] = -1;
     if (c == 0 && device_status)
       for (int j = tid; j < n; j += kThreads)
         if (sh.keys[j] == kProtectedKey) atomicOr(device_status, FASTAV_DEV_PROTECT_OVERFLOW);
@@ -454,11 +458,14 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
     if (tid < blocks) remote_store(remote(&sh.kept_of[c], tid), (unsigned)count);
     cluster_sync();  // the last remote access
     first = (int)__reduce_add_sync(0xFFFFFFFFu, lane < c ? sh.kept_of[lane] : 0u);
-    if (tid < m && ((sh.kept[tid >> 5] >> lane) & 1u)) {
+    const bool kept = tid < m && ((sh.kept[tid >> 5] >> lane) & 1u);
+    if (tid < m && !kept && PLACED) a.place[tok0 + t0 + tid] = -1;
+    if (kept) {
       int out = first + __popc(sh.kept[tid >> 5] & ((1u << lane) - 1u));
 #pragma unroll
       for (int w = 0; w < kCountSlice / 32; ++w) out += w < (tid >> 5) ? __popc(sh.kept[w]) : 0;
       if (out < room) keep_idx[base + out] = (global_idx ? tok0 : 0) + t0 + tid;
+      if (PLACED) a.place[tok0 + t0 + tid] = out < room ? base + out : -1;
       picked[out & (kBins - 1)] = (unsigned)(t0 + tid);
     }
   } else {
@@ -548,10 +555,14 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
 #pragma unroll
     for (int u = 0; u < kPer; ++u) {
       const bool is_gt = x[u] > T, is_eq = x[u] == T;
+      const int j = kPer * tid + u;
       if (u < mine && (is_gt || (is_eq && eq < need_eq))) {
-        const int out = gt + min(eq, need_eq), j = kPer * tid + u;
+        const int out = gt + min(eq, need_eq);
         if (out < room) keep_idx[base + out] = (global_idx ? tok0 : 0) + j;
+        if (PLACED) a.place[tok0 + j] = out < room ? base + out : -1;
         picked[out & (kBins - 1)] = (unsigned)j;
+      } else if (u < mine && PLACED) {
+        a.place[tok0 + j] = -1;
       }
       gt += is_gt;
       eq += is_eq;
@@ -616,14 +627,9 @@ int cluster_keys(const Shapes& s) {
 }
 int cluster_select(const Shapes& s) { return cluster_blocks(s.batch, s.max_seqlen, kScoreSlice, s.cluster_limit); }
 
-template <Front FRONT, int DIM>
-cudaError_t launch(const Shapes& s, FewArgs a, int blocks, size_t smem, const RowStreams* rows, const SelectArgs& t, cudaStream_t stream) {
-  a.slice_cap = slice_of(s, blocks);
-  if (rows) {
-    a.do_gather = 1;
-    a.rows = *rows;
-  }
-  const auto kernel = prune_few_kernel<FRONT, DIM>;
+template <Front FRONT, int DIM, bool PLACED>
+cudaError_t launch_kernel(const Shapes& s, const FewArgs& a, int blocks, size_t smem, const SelectArgs& t, cudaStream_t stream) {
+  const auto kernel = prune_few_kernel<FRONT, DIM, PLACED>;
   cudaError_t e = once_per_context([&] {
     cudaError_t f = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamic);
     if (f == cudaSuccess) f = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -634,6 +640,19 @@ cudaError_t launch(const Shapes& s, FewArgs a, int blocks, size_t smem, const Ro
                              t.protect, t.q_idx, t.cu_qlens, t.keep_idx, t.cu_keep, t.device_status);
   count_launches(1);
   return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <Front FRONT, int DIM>
+cudaError_t launch(const Shapes& s, FewArgs a, int blocks, size_t smem, const RowStreams* rows, const SelectArgs& t, cudaStream_t stream) {
+  a.slice_cap = slice_of(s, blocks);
+  a.place = t.place;
+  if (rows) {
+    a.do_gather = 1;
+    a.rows = *rows;
+  }
+  if constexpr (FRONT == kKeys)
+    if (a.place) return launch_kernel<FRONT, DIM, true>(s, a, blocks, smem, t, stream);
+  return launch_kernel<FRONT, DIM, false>(s, a, blocks, smem, t, stream);
 }
 
 template <Front FRONT>
@@ -670,7 +689,7 @@ int cluster_limit() {
     const unsigned long long v = k.load(std::memory_order_acquire);
     if (context && v >> 1 == context) return v & 1 ? kMaxCluster : kPortableCluster;
   }
-  const auto kernel = prune_few_kernel<kKeys, 128>;
+  const auto kernel = prune_few_kernel<kKeys, 128, false>;
   int clusters = 0;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamic);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);

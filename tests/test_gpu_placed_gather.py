@@ -1,0 +1,91 @@
+"""Rows read ahead of the selection (compact_placed_kernel, behind the few-rows kernel): against the oracle, and bit for bit against the
+gather that starts from the keep list.  One token up to what shared memory holds, up to 31 sequences and 32, empty ones, nothing and
+everything kept, more protected tokens than are kept, selection by counting and by digits, keys and values packed and head-major, a call
+without values or positions, tokens ahead of the first sequence, and index arrays that promise less than they hold."""
+import pytest
+import torch
+
+import parity
+from paper_2601_13143_b200 import fastav, workloads as W
+
+pytestmark = pytest.mark.gpu
+
+OUT = ("keep_idx", "cu_keep", "hidden_out", "pos_out", "k_out", "v_out")
+
+
+def _problem(lens, keeps, hid=1024, hq=4, hkv=2, d=128, rows=1):
+    return W.random_problem(seed=sum(lens) + hid, lens=lens, rows=[min(rows, n) for n in lens], keeps=keeps, num_q_heads=hq, num_kv_heads=hkv, head_dim=d,
+                            hidden=hid, duplicate_keys=2)
+
+
+def _both(buf):
+    """The call as it is, and with the gather by loads and stores, which starts from the list."""
+    got = []
+    for flag in (0, fastav.FASTAV_COMPACT_PATH_LOADSTORE):
+        buf.params.flags = buf.params.flags & ~fastav.FASTAV_COMPACT_PATH_LOADSTORE | flag
+        for name in OUT:
+            if getattr(buf, name) is not None:
+                getattr(buf, name).view(torch.uint8).fill_(0x55)
+        buf.device_status.zero_()
+        buf.prune()
+        torch.cuda.synchronize()
+        got.append({name: getattr(buf, name).clone() for name in OUT if getattr(buf, name) is not None} | {"status": buf.device_status.clone()})
+    for name in got[0]:
+        assert torch.equal(got[0][name].view(torch.uint8), got[1][name].view(torch.uint8)), name
+    return got[0]
+
+
+@pytest.mark.parametrize("lens,keep,hid,hkv,d", [
+    ([1], 1.0, 1024, 2, 128), ([147, 1], 0.7, 3584, 4, 128), ([149], 0.8, 3584, 4, 128), ([744], 0.8, 3584, 4, 128), ([2048], 0.9, 4096, 8, 128),
+    ([2048, 300], 0.8, 2048, 2, 128), ([100] * 31, 0.8, 1024, 4, 64), ([100] * 32, 0.8, 1024, 4, 64), ([300, 0, 5] * 5, 0.9, 1024, 2, 128), ([1500], 0.9, 512, 2, 128),
+    ([1500], 0.9, 504, 2, 128),
+])
+def test_against_the_oracle(lens, keep, hid, hkv, d):
+    p = _problem(lens, [int(keep * n) if i % 4 else n * int(keep * 10) // 10 for i, n in enumerate(lens)], hid, 2 * hkv, hkv, d)
+    protect = (torch.arange(p.total_tokens) % 3 != 1).to(torch.uint8) if len(lens) % 3 == 0 else None
+    buf = parity.to_device(p, protect=protect)
+    buf.prune()
+    torch.cuda.synchronize()
+    parity.check_fused_against_oracle(p, buf, parity.oracle_prune(p, protect=protect), protect=protect, what=f"{lens}")
+    _both(buf)
+
+
+@pytest.mark.parametrize("keeps", [[0, 500], [700, 0], [700, 500], [1, 1]])
+@pytest.mark.parametrize("protected", [False, True])
+def test_nothing_and_everything_kept(keeps, protected):
+    p = _problem([700, 500], keeps)
+    _both(parity.to_device(p, protect=(torch.arange(1200) % 2).to(torch.uint8) if protected else None))
+
+
+@pytest.mark.parametrize("layout", ["head_major", "no_values", "no_positions", "no_hidden"])
+def test_layouts(layout):
+    p = _problem([600, 333], [500, 200], hkv=4, hq=4)
+    buf = parity.to_device(p)
+    if layout == "head_major":
+        k, v = (torch.empty(4, 933, 128, dtype=torch.bfloat16, device="cuda").transpose(0, 1) for _ in range(2))
+        k.copy_(buf.k), v.copy_(buf.v)
+        buf = fastav.make_buffers(q=buf.q, q_idx=buf.q_idx, cu_qlens=buf.cu_qlens, k=k, v=v, cu_seqlens=buf.cu_seqlens, keep_counts=buf.keep_counts, hidden=buf.hidden,
+                                  pos=buf.pos, softmax_scale=p.softmax_scale, flags=parity.flags_of(p))
+    elif layout == "no_values":
+        buf.v = buf.v_out = None
+    elif layout == "no_positions":
+        buf.pos = buf.pos_out = None
+    else:
+        buf.hidden = buf.hidden_out = None
+    _both(buf)
+
+
+def test_tokens_ahead_of_the_first_sequence():
+    p = _problem([400, 350], [300, 250])
+    buf = parity.to_device(p)
+    buf.cu_seqlens += torch.tensor([37, 0, 0], dtype=torch.int32, device="cuda")
+    _both(buf)
+
+
+def test_a_sequence_longer_than_promised_stays_inside_the_buffers():
+    """The excess is left out and reported; whatever the workspace held for those tokens moves no row."""
+    p = _problem([400, 350], [300, 250])
+    buf = parity.to_device(p)
+    buf.params.max_seqlen = 380
+    buf.workspace.fill_(1)  # a valid place for every token, were it read
+    assert int(_both(buf)["status"]) & fastav.FASTAV_DEV_SHAPE_MISMATCH
