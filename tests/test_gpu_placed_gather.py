@@ -89,3 +89,31 @@ def test_a_sequence_longer_than_promised_stays_inside_the_buffers():
     buf.params.max_seqlen = 380
     buf.workspace.fill_(1)  # a valid place for every token, were it read
     assert int(_both(buf)["status"]) & fastav.FASTAV_DEV_SHAPE_MISMATCH
+
+
+@pytest.mark.parametrize("layout", ["packed", "head_major", "no_values", "no_positions", "no_hidden"])
+@pytest.mark.parametrize("lens,rows", [([333, 0, 90], 1), ([700], 2), ([60] * 9, 9)])
+def test_rows_read_ahead_by_the_blocks_that_select(layout, lens, rows):
+    """Little per block: the slice's rows lie in shared memory before the selection is known (from the keys, and from partial sums)."""
+    p = W.random_problem(seed=sum(lens), lens=lens, rows=[min(rows, n) for n in lens], keeps=[n // 3 if i % 3 else n * 4 // 5 for i, n in enumerate(lens)],
+                         num_q_heads=4, num_kv_heads=2, head_dim=64, hidden=128)
+    buf = parity.to_device(p)
+    if layout == "head_major":
+        k, v = (torch.empty(2, p.total_tokens, 64, dtype=torch.bfloat16, device="cuda").transpose(0, 1) for _ in range(2))
+        k.copy_(buf.k), v.copy_(buf.v)
+        buf = fastav.make_buffers(q=buf.q, q_idx=buf.q_idx, cu_qlens=buf.cu_qlens, k=k, v=v, cu_seqlens=buf.cu_seqlens, keep_counts=buf.keep_counts, hidden=buf.hidden,
+                                  pos=buf.pos, softmax_scale=p.softmax_scale, flags=parity.flags_of(p))
+    for name in {"no_values": ("v",), "no_positions": ("pos",), "no_hidden": ("hidden",)}.get(layout, ()):
+        setattr(buf, name, None)
+        setattr(buf, name + "_out", None)
+    before = fastav.fastav_kernel_launches()
+    buf.prune()
+    torch.cuda.synchronize()
+    if rows <= 4 or len(lens) >= 8:
+        assert fastav.fastav_kernel_launches() - before == (1 if rows <= 4 else 2)  # no gather of its own
+    keep, cu = buf.keep_idx.cpu().numpy(), buf.cu_keep.cpu().numpy()
+    mine = parity.gather_rows(p, keep[:cu[-1]], cu)
+    assert int(buf.device_status) & ~fastav.FASTAV_DEV_PROTECT_OVERFLOW == 0
+    for name in ("hidden", "pos", "k", "v"):
+        if getattr(buf, name + "_out") is not None:
+            parity.assert_bits_equal(getattr(buf, name + "_out"), mine[name], f"{layout} {name}")
