@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap q_map, Shapes s,
                   const int32_t* __restrict__ q_idx, const int32_t* __restrict__ cu_qlens,
                   const int32_t* __restrict__ cu_seqlens, int chunk_tiles, int stat_chunks, int rc_max, int rows_per_chunk,
-                  float2* __restrict__ stats, const float* __restrict__ lse, float* __restrict__ partial,
+                  float2* __restrict__ stats, const float* __restrict__ lse, int lse_natural, float* __restrict__ partial,
                   int32_t* device_status) {
   using L = Layout<DIM>;
   extern __shared__ unsigned char smem_raw[];
@@ -306,9 +306,9 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
   if (warp == 0) {
     // ---- TMA producer: one elected lane streams query tiles and K tiles ---------------------------
     if (lane == 0) {
-      // q and k may be what the previous kernel in the stream wrote.  Sweep 2 is never the first kernel of a call,
-      // so it may fetch them ahead of its wait -- unless the call's first kernel was itself launched
-      // programmatically (FASTAV_CHAIN_CALLS): then the previous call's last kernel may still be running.
+      // q and k may be what the previous kernel in the stream wrote.  Sweep 2 may fetch them ahead of its wait: as a call's second
+      // kernel, or as its first, which has waited already -- unless calls are chained (FASTAV_CHAIN_CALLS): then the previous
+      // call's last kernel may still be running.
       if (SWEEP != 2 || (s.flags & FASTAV_CHAIN_CALLS)) pdl_wait();
       int tile_no = 0, q_gen = 0;  // K tiles / query tiles issued so far
       bool ok = true;
@@ -488,6 +488,7 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
             if (c < my_cols) {
               const int r = f / s.group;
               nl = -chain_load(lse + (long long)(un.row0 + r) * s.hq + un.g * s.group + f % s.group);
+              if (lse_natural) nl = nl == nl && fabsf(nl) != INFINITY ? nl * kLog2e : -INFINITY;  // a row that sees no key adds 0
               lim = causal ? chain_load_cached(q_idx + un.row0 + r) : INT_MAX;
               min_limit = min(min_limit, lim);
             }
@@ -677,11 +678,11 @@ cudaError_t run(const Shapes& s, const Workspace& w, const CUtensorMap& k_map, c
   if (e != cudaSuccess) return e;
   if (lse_in) {
     // The caller already has log-sum-exp per (row, head) (the layer's attention kernel returns it): one sweep.
-    if ((e = launch_lse_import(s, lse_in, lse, stream)) != cudaSuccess) return e;
+    // Sweep 2 reads it as it is (an import kernel first: 3 x 8,001-9,001 tokens 69.7 us instead of 68.7).
   } else {
     if ((e = launch_chained(score_wide_kernel<DIM, 1>, dim3(grid), dim3(kThreads), smem, stream, k_map, q_map, s, q_idx, cu_qlens,
                             cu_seqlens, chunk_tiles, stat_chunks, rc_max, rows_per_chunk, stats, (const float*)nullptr,
-                            (float*)nullptr, device_status)) != cudaSuccess)
+                            0, (float*)nullptr, device_status)) != cudaSuccess)
       return e;
     const int warps = s.total_q * s.hq;
     if ((e = launch_chained(score_wide_merge_kernel, dim3((warps + 7) / 8), dim3(256), 0, stream, s, cu_qlens, cu_seqlens,
@@ -691,8 +692,8 @@ cudaError_t run(const Shapes& s, const Workspace& w, const CUtensorMap& k_map, c
   }
   if (!scores_out) return cudaGetLastError();  // only the statistics were asked for (fastav_lse)
   if ((e = launch_chained(score_wide_kernel<DIM, 2>, dim3(grid), dim3(kThreads), smem, stream, k_map, q_map, s, q_idx, cu_qlens,
-                          cu_seqlens, chunk_tiles, stat_chunks, rc_max, rows_per_chunk, (float2*)nullptr, (const float*)lse,
-                          partial, device_status)) != cudaSuccess)
+                          cu_seqlens, chunk_tiles, stat_chunks, rc_max, rows_per_chunk, (float2*)nullptr,
+                          lse_in ? lse_in : (const float*)lse, lse_in ? 1 : 0, partial, device_status)) != cudaSuccess)
     return e;
   count_launches(1);
   if ((e = finish(rc_max, rows_per_chunk)) != cudaSuccess) return e;
