@@ -540,7 +540,12 @@ score_wide_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_consta
   if (threadIdx.x == 0 && ctl.abort && device_status) atomicOr(device_status, FASTAV_DEV_WAIT_EXPIRED);
 }
 
-// One warp per (scored row, head): fold the per-chunk (max, sum) pairs into log2-sum-exp2.
+// Fold the per-chunk (max, sum) pairs of a (scored row, head) into log2-sum-exp2.  Up to 32 pairs a row and 32 sequences: eight lanes per
+// row, four pairs each in flight, and each lane of the warp knows where one sequence starts.  Else a warp per row, which looks its
+// sequence up.  A call on 32 ragged sequences (28,672 rows) takes 295 us instead of 299 with a warp per row (the kernel took 9.2), on
+// 4 x 16,384 tokens (16,384 rows of 30 pairs) 262 instead of 263.6; with two pairs kept the latter stay with the warp.
+constexpr int kMergeKept = 4;
+template <int LANES>
 __global__ void __launch_bounds__(256) score_wide_merge_kernel(Shapes s, const int32_t* __restrict__ cu_qlens,
                                                                const int32_t* __restrict__ cu_seqlens,
                                                                const float2* __restrict__ stats, int stat_chunks,
@@ -550,46 +555,65 @@ __global__ void __launch_bounds__(256) score_wide_merge_kernel(Shapes s, const i
   pdl_acquire(stats);
   pdl_acquire(cu_qlens);
   pdl_acquire(cu_seqlens);
-  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (w >= s.total_q * s.hq) return;
+  const int w = (blockIdx.x * blockDim.x + threadIdx.x) / LANES, lane = threadIdx.x & 31, part = lane & (LANES - 1);
+  const bool there = w < s.total_q * s.hq;
+  if (LANES == 32 && !there) return;
   const int row = w / s.hq;
-  // The row's sequence is the last one that starts at or before it.  The whole warp looks, 32 starts at a time: at evenly spaced
-  // ones until at most 32 sequences are left, then at those (1,024 sequences: two rounds; one after the other 32 of them made a
-  // score call of 1,024 x 128 tokens 169 us instead of 98).
-  int lo = 0, left = s.batch;
-  while (left > 32) {
-    const int step = (left + 31) / 32, at = lo + lane * step;
-    const unsigned not_after = __ballot_sync(0xFFFFFFFFu, lane * step < left && chain_load_cached(cu_qlens + at) <= row);
-    const int skip = not_after ? (31 - __clz(not_after)) * step : 0;
-    lo += skip;
-    left = min(step, left - skip);
-  }
   int n = 0;
-  {
+  if constexpr (LANES < 32) {
+    const int b = min(lane, s.batch - 1), first = chain_load_cached(cu_qlens + b), count = seq_span<true>(s, cu_seqlens, b).count;
+#pragma unroll
+    for (int g = 0; g < 32 / LANES; ++g) {  // the last sequence that starts at or before the row of the warp's g-th entry
+      const int wanted = __shfl_sync(0xFFFFFFFFu, row, g * LANES);
+      const unsigned not_after = __ballot_sync(0xFFFFFFFFu, lane < s.batch && first <= wanted);
+      const int found = __shfl_sync(0xFFFFFFFFu, count, not_after ? 31 - __clz(not_after) : 0);
+      if (lane / LANES == g && not_after) n = found;
+    }
+  } else {
+    // The row's sequence is the last one that starts at or before it.  The whole warp looks, 32 starts at a time: at evenly spaced
+    // ones until at most 32 sequences are left, then at those (1,024 sequences: two rounds; one after the other 32 of them made a
+    // score call of 1,024 x 128 tokens 169 us instead of 98).
+    int lo = 0, left = s.batch;
+    while (left > 32) {
+      const int step = (left + 31) / 32, at = lo + lane * step;
+      const unsigned not_after = __ballot_sync(0xFFFFFFFFu, lane * step < left && chain_load_cached(cu_qlens + at) <= row);
+      const int skip = not_after ? (31 - __clz(not_after)) * step : 0;
+      lo += skip;
+      left = min(step, left - skip);
+    }
     const int b = min(lo + lane, s.batch - 1);
     const int first = chain_load_cached(cu_qlens + b), count = seq_span<true>(s, cu_seqlens, b).count;
     const unsigned not_after = __ballot_sync(0xFFFFFFFFu, lane < left && first <= row);
     if (not_after) n = __shfl_sync(0xFFFFFFFFu, count, 31 - __clz(not_after));
   }
-  const int chunks = 2 * ((n + chunk_keys - 1) / chunk_keys);  // one entry per 64-key half of every tile run
-  const float2* mine = stats + (long long)w * stat_chunks;
-  // the first 32 entries stay in a register (usually all of them); the rest, if any, is read twice
-  const float2 first = lane < chunks ? chain_load(mine + lane) : make_float2(-INFINITY, 0.f);
-  float m = first.x;
-  for (int t = lane + 32; t < chunks; t += 32) m = fmaxf(m, chain_load(mine + t).x);
+  const int chunks = there ? 2 * ((n + chunk_keys - 1) / chunk_keys) : 0;  // one entry per 64-key half of every tile run
+  const float2* mine = stats + (long long)(there ? w : 0) * stat_chunks;
+  // the first few entries of a lane stay in registers (usually all of them); the rest, if any, is read twice
+  constexpr int kKept = LANES < 32 ? kMergeKept : 1;
+  float2 kept[kKept];
 #pragma unroll
-  for (int d = 16; d; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
+  for (int u = 0; u < kKept; ++u) kept[u] = part + u * LANES < chunks ? chain_load(mine + part + u * LANES) : make_float2(-INFINITY, 0.f);
+  float m = kept[0].x;
+#pragma unroll
+  for (int u = 1; u < kKept; ++u) m = fmaxf(m, kept[u].x);
+  for (int t = part + kKept * LANES; t < chunks; t += LANES) m = fmaxf(m, chain_load(mine + t).x);
+  __syncwarp();
+#pragma unroll
+  for (int d = LANES / 2; d; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
   float l = 0.f;
   if (m > -INFINITY) {
-    if (first.x > -INFINITY) l = first.y * exp2f(first.x - m);
-    for (int t = lane + 32; t < chunks; t += 32) {
+#pragma unroll
+    for (int u = 0; u < kKept; ++u)
+      if (kept[u].x > -INFINITY) l += kept[u].y * exp2f(kept[u].x - m);
+    for (int t = part + kKept * LANES; t < chunks; t += LANES) {
       const float2 v = chain_load(mine + t);
       if (v.x > -INFINITY) l += v.y * exp2f(v.x - m);
     }
   }
+  __syncwarp();
 #pragma unroll
-  for (int d = 16; d; d >>= 1) l += __shfl_xor_sync(0xFFFFFFFFu, l, d);
-  if (lane == 0) lse[w] = (l > 0.f) ? m + log2f(l) : INFINITY;  // a row that sees no key contributes 0
+  for (int d = LANES / 2; d; d >>= 1) l += __shfl_xor_sync(0xFFFFFFFFu, l, d);
+  if (part == 0 && there) lse[w] = (l > 0.f) ? m + log2f(l) : INFINITY;  // a row that sees no key contributes 0
 }
 
 constexpr int kFinalizeThreads = 64;
@@ -684,9 +708,12 @@ cudaError_t run(const Shapes& s, const Workspace& w, const CUtensorMap& k_map, c
                             cu_seqlens, chunk_tiles, stat_chunks, rc_max, rows_per_chunk, stats, (const float*)nullptr,
                             0, (float*)nullptr, device_status)) != cudaSuccess)
       return e;
-    const int warps = s.total_q * s.hq;
-    if ((e = launch_chained(score_wide_merge_kernel, dim3((warps + 7) / 8), dim3(256), 0, stream, s, cu_qlens, cu_seqlens,
-                            (const float2*)stats, stat_chunks, chunk_keys, lse)) != cudaSuccess)
+    const int entries = s.total_q * s.hq;
+    const bool few_entries = s.batch <= 32 && stat_chunks <= 8 * kMergeKept;
+    const auto merge = few_entries ? score_wide_merge_kernel<8> : score_wide_merge_kernel<32>;
+    const int per_block = few_entries ? 32 : 8;
+    if ((e = launch_chained(merge, dim3((entries + per_block - 1) / per_block), dim3(256), 0, stream, s, cu_qlens, cu_seqlens, (const float2*)stats,
+                            stat_chunks, chunk_keys, lse)) != cudaSuccess)
       return e;
     count_launches(2);
   }
