@@ -519,13 +519,21 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
     const uint4 v = *reinterpret_cast<const uint4*>(&sh.keys[kPer * tid + u]);
     x[u] = v.x; x[u + 1] = v.y; x[u + 2] = v.z; x[u + 3] = v.w;
   }
+  // The first pass looks at scores from 2^-63 up to 2 only, whose three leading bits are the same: a bin is 1/64 of an octave wide
+  // instead of 1/8, and the bin of the k-th largest holds few keys to rank.  Smaller scores share the lowest bin, larger ones (and
+  // protected tokens) the highest; where the k-th largest lies in one of these two among many, the passes start again from the first bit.
+  // (From the keys only: three stages from 1,024 tokens 36.6 -> 36.3 us; from partial sums 1 x 2,048 tokens 21.5 -> 21.6.)
+  constexpr int kWindowShift = 29 - kDigitBits;
+  const int window = lowest ? 2 << kDigitBits : 5 << kDigitBits;
+  auto window_digit = [&](unsigned key) { return (unsigned)min(max((int)(key >> kWindowShift) - window, 0), kBins - 1); };
+  bool windowed = FRONT == kKeys;
   unsigned prefix = 0u;   // the bits of the k-th largest key fixed so far
   int remaining = k, bits_left = 32;
 #pragma unroll 1
-  while (bits_left > 0) {
-    const int shift = max(0, bits_left - kDigitBits);
+  for (int pass = 0; bits_left > 0; ++pass) {
+    const int shift = windowed ? kWindowShift : max(0, bits_left - kDigitBits);
     const unsigned above_want = __funnelshift_rc(prefix, 0u, bits_left);  // prefix >> bits_left, 0 for 32
-    if (bits_left < 32) {
+    if (pass > 0) {
       for (int i = tid; i < kBins / 4; i += kThreads) reinterpret_cast<uint4*>(sh.hist)[i] = make_uint4(0, 0, 0, 0);
       __syncthreads();
     }
@@ -534,7 +542,7 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
 #pragma unroll
       for (int u = 0; u < kPer; ++u) {
         if (u < mine && __funnelshift_rc(x[u], 0u, bits_left) == above_want) {
-          const unsigned digit = (x[u] >> shift) & (kBins - 1);
+          const unsigned digit = windowed ? window_digit(x[u]) : (x[u] >> shift) & (kBins - 1);
           if (digit != run_digit) {
             if (run_len) atomicAdd(&sh.hist[run_digit], run_len);
             run_digit = digit;
@@ -559,7 +567,7 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
 #pragma unroll
       for (int i = kBinsPerThread - 1; i >= 0; --i) {
         if (above < rem && rem <= above + h[i]) {
-          sh.prefix = prefix | ((unsigned)(tid * kBinsPerThread + i) << shift);
+          sh.prefix = windowed ? (unsigned)(tid * kBinsPerThread + i) : prefix | ((unsigned)(tid * kBinsPerThread + i) << shift);
           sh.remaining = (int)(rem - above);
           sh.bucket = (int)h[i];
         }
@@ -567,13 +575,21 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
       }
     }
     __syncthreads();
-    prefix = sh.prefix;
+    const unsigned found = sh.prefix;
+    const bool in_window = windowed;
+    if (windowed) {
+      windowed = false;
+      if ((found == 0u || found == kBins - 1) && sh.bucket > kDirectMax) continue;  // (prefix and remaining as they were)
+      prefix = ((unsigned)window + found) << kWindowShift;
+    } else {
+      prefix = found;
+    }
     remaining = sh.remaining;
     bits_left = shift;
     if (bits_left > 0 && sh.bucket <= kDirectMax) {  // few keys left: collect them, each finds its rank by counting
 #pragma unroll
       for (int u = 0; u < kPer; ++u)
-        if (u < mine && (x[u] >> bits_left) == (prefix >> bits_left)) sh.list[atomicAdd(&sh.list_n, 1)] = x[u];
+        if (u < mine && (in_window ? window_digit(x[u]) == found : (x[u] >> bits_left) == (prefix >> bits_left))) sh.list[atomicAdd(&sh.list_n, 1)] = x[u];
       __syncthreads();
       rank_finish(sh.list, sh.list_n, remaining, tid, &sh.threshold, &sh.need_eq);
       __syncthreads();

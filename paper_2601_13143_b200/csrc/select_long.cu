@@ -282,9 +282,10 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
   pdl_trigger();
   // The first pass looks at scores from 2^-63 up to 2 only: three leading bits are the same there, so that a bin is 1/32 of an octave
   // wide instead of 1/4, and the bin of the k-th largest holds few keys.  Smaller scores share the lowest bin, larger ones
-  // (and protected tokens) the highest; where the k-th largest lies in one of these two the passes start again from the first bit.
+  // (and protected tokens) the highest; where the k-th largest lies in one of these two among many, the passes start again from the first bit.
   constexpr int kWindowShift = 29 - kDigitBits;  // three leading bits, then the digit
   const int window = lowest ? 2 << kDigitBits : 5 << kDigitBits;
+  auto window_digit = [&](unsigned key) { return (unsigned)min(max((int)(key >> kWindowShift) - window, 0), kBins - 1); };
   bool windowed = true;
   unsigned prefix = 0u;  // the bits of the k-th largest key fixed so far
   int remaining = k, bits_left = 32;
@@ -306,7 +307,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
 #pragma unroll
       for (int u = 0; u < kPer; ++u) {
         if (u < mine && __funnelshift_rc(x[u], 0u, bits_left) == above_want) {
-          const unsigned digit = windowed ? (unsigned)min(max((int)(x[u] >> kWindowShift) - window, 0), kBins - 1) : (x[u] >> shift) & (kBins - 1);
+          const unsigned digit = windowed ? window_digit(x[u]) : (x[u] >> shift) & (kBins - 1);
           if (digit != run_digit) {
             if (run_len) atomicAdd(&sh.hist[run_digit >> 1], run_len << (16 * (run_digit & 1)));
             run_digit = digit;
@@ -354,9 +355,10 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
     __syncthreads();
     const unsigned found = sh.prefix;
     const int bucket = sh.bucket;
+    const bool in_window = windowed;
     if (windowed) {
       windowed = false;
-      if (found == 0u || found == kBins - 1) continue;  // (prefix and remaining as they were)
+      if ((found == 0u || found == kBins - 1) && bucket > kListMax) continue;  // (prefix and remaining as they were)
       prefix = ((unsigned)window + found) << kWindowShift;
     } else {
       prefix = found;
@@ -367,8 +369,9 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
       unsigned over = 0u;
 #pragma unroll
       for (int u = 0; u < kPer; ++u) {
-        if (u < mine && (x[u] >> bits_left) == (prefix >> bits_left)) sh.list[atomicAdd(&sh.list_n, 1)] = x[u];
-        over += u < mine && (x[u] >> bits_left) > (prefix >> bits_left);
+        const unsigned digit = in_window ? window_digit(x[u]) : x[u] >> bits_left, wanted = in_window ? found : prefix >> bits_left;
+        if (u < mine && digit == wanted) sh.list[atomicAdd(&sh.list_n, 1)] = x[u];
+        over += u < mine && digit > wanted;
       }
       over = __reduce_add_sync(0xFFFFFFFFu, over);
       if (lane == 0 && over) atomicAdd(&sh.above_n, over);

@@ -43,11 +43,11 @@ def test_flags_of_the_selection(lens, lowest, global_idx, by_rows, lse):
     parity.check_prune_under_flags(p, lowest, global_idx, by_rows, lse, protect, f"{lens[0]} x {len(lens)}")
 
 
-# The first pass looks at scores from 2^-63 to 2 in bins of 1/32 octave.  `crowd`: a hundred different scores within one or two bins and one
+# The first pass looks at scores from 2^-63 to 2 in bins of 1/32 octave (one scored row and up to 2,048 tokens, in the few-rows kernel: 1/64).  `crowd`: a hundred different scores within one or two bins and one
 # block's slice, the k-th largest among them (more than a block sends; some 40 per block where the bin has more); `small`: all scores but one
 # below 2^-63; `hidden`: most tokens behind the scored rows (score 0) and k beyond the others; `above`: the k-th largest is protected.
 @pytest.mark.parametrize("kind", ["crowd", "wide_crowd", "small", "hidden", "above"])
-@pytest.mark.parametrize("lens", [[2049], [5000, 2100], [17000]], ids=lambda v: f"{len(v)}x{max(v)}")
+@pytest.mark.parametrize("lens", [[1500], [2000, 900], [2049], [5000, 2100], [17000]], ids=lambda v: f"{len(v)}x{max(v)}")
 @pytest.mark.parametrize("rows", [1, 9])
 @pytest.mark.parametrize("lowest", [False, True])
 def test_window_of_the_first_pass(kind, lens, rows, lowest):
