@@ -41,6 +41,7 @@ def test_few_rows(lens, rows, hq, hkv, d):
 @pytest.mark.parametrize("lens,rows,hq,hkv,d", [
     ([5], 5, 2, 2, 64), ([127, 128, 129], 9, 8, 8, 64), ([1000, 3], 33, 28, 4, 128), ([4095], 8, 8, 2, 128), ([4096], 17, 16, 1, 64), ([4097], 8, 8, 2, 128),
     ([2048, 100], 130, 4, 2, 64), ([300], 12, 17, 1, 64), ([512] * 40, 32, 28, 4, 128), ([1024, 640, 999] * 5, 32, 8, 8, 64), ([256] * 24, 128, 16, 4, 64),
+    ([4200, 4097, 4150], 40, 32, 4, 64), ([5000, 4600], 9, 8, 2, 64), ([5000, 4900], 9, 8, 2, 64),  # chunks for about one length, and for ragged ones
 ])
 @pytest.mark.parametrize("trailing", [True, False])
 def test_many_rows(lens, rows, hq, hkv, d, trailing):
