@@ -444,6 +444,8 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
   auto rows_read = [&] {  // false: given up (one answer for the warp)
     if (m == 0 || ptx::mbar_wait_warp(rows_bar, 0, &sh.abort)) return true;
     if (lane == 0 && device_status) atomicOr(device_status, FASTAV_DEV_WAIT_EXPIRED);
+    int never = 0;  // the copies in flight write into this block's shared memory: waited for once more, whichever warp gave up
+    ptx::mbar_wait_bounded(rows_bar, 0, &never);
     return false;
   };
   if (k == 0) {  // nothing is kept, protected or not (uniform for the cluster)
