@@ -41,65 +41,106 @@ struct RowsRing {
   static_assert(kStages % kWarps == 0);
 };
 
-// The batch's tiles of 64 tokens in one list.  Up to 32 sequences: each lane knows one.  Larger batches: the tiles of the longest
-// sequence for each, those past a sequence's end empty.
+// The batch's tiles of 64 tokens in one list.  Shared memory has for every sequence its bounds and how many tiles come before it (of
+// batches beyond kTable for every `step`-th), and a warp finds a tile's sequence in two looks of 32 entries.  The list has to be exact, since every
+// block takes an equal run of it: with every sequence given as many tiles as the longest one has, the real ones of 64 sequences,
+// one of 20,000 tokens and 63 of 500, all fell to a few blocks (Mistral-7B shapes, one row: score call 49 us instead of 503, prune 205 instead of
+// 656; 100 of 300 to 3,000 tokens 72 / 131 and 482 / 532).  The spans in registers and shuffles for up to 32 sequences were no quicker (20 x
+// 3,000 tokens 32.3 / 32.0 us).
+constexpr int kTable = 1024;
+struct SharedList {
+  int4 bounds[kTable];              // first token, tokens, first scored row, scored rows (step 1)
+  int ahead[kTable + kTable / 32];  // entry e at e + e / 32: both looks are free of bank conflicts
+  int warp_sum[kWarps + 1];
+};
+
 struct TileList {
   const Shapes& s;
+  SharedList& sh;
   const int32_t *cu_seqlens, *cu_qlens;
-  int lane, padded;         // padded: tiles listed per sequence, 0 for up to 32 sequences
-  Span seq, rows;           // this lane's sequence
-  int upto;                 // tiles of the sequences up to and with this lane's
-  int total;
+  int lane;
+  int step, entries, total;
+  bool bad = false;         // a sequence that this thread has seen was cut
   // of the tile looked up last, in all lanes
-  int at = -1;
-  int b = 0, first = 0, tok0 = 0, tokens = 0, row0 = 0, row_count = 0;
-  __device__ TileList(const Shapes& s_, const int32_t* cu_seqlens_, const int32_t* cu_qlens_, int lane_)
-      : s(s_), cu_seqlens(cu_seqlens_), cu_qlens(cu_qlens_), lane(lane_), padded(0), seq{0, 0, false}, rows{0, 0, false}, upto(0) {}
-  // One warp per block asks for the sequences' bounds, the others read them from shared memory (all of them on a few lines of L2
-  // cost a microsecond).  All threads of the block.
-  __device__ void open(Span (&kept)[2][32], int warp) {
-    if (s.batch > 32) {
-      padded = (s.max_seqlen + kRowTileTokens - 1) / kRowTileTokens;
-      total = padded * s.batch;
-      __syncthreads();
-      return;
-    }
-    if (warp == 0) {
-      kept[0][lane] = lane < s.batch ? seq_span(s, cu_seqlens, lane) : Span{0, 0, false};
-      kept[1][lane] = lane < s.batch ? row_span(s, cu_qlens, lane) : Span{0, 0, false};
-    }
-    __syncthreads();
-    seq = kept[0][lane];
-    rows = kept[1][lane];
-    upto = (seq.count + kRowTileTokens - 1) / kRowTileTokens;
+  int first = 0, tok0 = 0, tokens = 0, row0 = 0, row_count = 0;
+  int begin = 0, end = 0;   // the tiles of its sequence
+  __device__ TileList(const Shapes& s_, SharedList& sh_, const int32_t* cu_seqlens_, const int32_t* cu_qlens_, int lane_)
+      : s(s_), sh(sh_), cu_seqlens(cu_seqlens_), cu_qlens(cu_qlens_), lane(lane_) {}
+  static __device__ int tiles_of(int count) { return (count + kRowTileTokens - 1) / kRowTileTokens; }
+  __device__ int sum_upto(int v) const {
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-      const int t = __shfl_up_sync(0xFFFFFFFFu, upto, d);
-      if (lane >= d) upto += t;
+      const int t = __shfl_up_sync(0xFFFFFFFFu, v, d);
+      if (lane >= d) v += t;
     }
-    total = __shfl_sync(0xFFFFFFFFu, upto, 31);
+    return v;
   }
-  __device__ void look_up(int t, int32_t* device_status) {  // the whole warp
-    if (t == at) return;
-    at = t;
-    if (padded) {
-      b = t / padded;
-      const Span q = seq_span<true>(s, cu_seqlens, b), r = row_span<true>(s, cu_qlens, b);
-      if ((q.bad || r.bad) && lane == 0 && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
-      tok0 = q.first;
-      tokens = q.count;
-      row0 = r.first;
-      row_count = r.count;
-      first = (t - b * padded) * kRowTileTokens;
-      return;
+  // All threads of the block.  Each bound is asked for by one thread of it (by all its warps: a microsecond on a few lines of L2).
+  // (Loops kept as loops: of a large call every line of code comes from memory again.)
+  __device__ void open(int warp) {
+    step = (s.batch + kTable - 1) / kTable;
+    entries = (s.batch + step - 1) / step;
+    const int each = (entries + kThreads - 1) / kThreads, e0 = min(entries, (int)threadIdx.x * each), e1 = min(entries, e0 + each);
+    int sum = 0;
+#pragma unroll 1
+    for (int e = e0; e < e1; ++e) {
+      sh.ahead[e + e / 32] = sum;
+#pragma unroll 1
+      for (int b = e * step; b < min(s.batch, (e + 1) * step); ++b) {
+        const Span q = seq_span(s, cu_seqlens, b), r = row_span(s, cu_qlens, b);
+        bad |= q.bad | r.bad;
+        sum += tiles_of(q.count);
+        sh.bounds[e] = make_int4(q.first, q.count, r.first, r.count);
+      }
     }
-    b = __ffs(__ballot_sync(0xFFFFFFFFu, upto > t)) - 1;
-    const int end = __shfl_sync(0xFFFFFFFFu, upto, b);
-    tok0 = __shfl_sync(0xFFFFFFFFu, seq.first, b);
-    tokens = __shfl_sync(0xFFFFFFFFu, seq.count, b);
-    row0 = __shfl_sync(0xFFFFFFFFu, rows.first, b);
-    row_count = __shfl_sync(0xFFFFFFFFu, rows.count, b);
-    first = (t - (end - (tokens + kRowTileTokens - 1) / kRowTileTokens)) * kRowTileTokens;
+    int before = sum_upto(sum) - sum;
+    if (lane == 31) sh.warp_sum[warp] = before + sum;
+    __syncthreads();
+    total = 0;
+#pragma unroll
+    for (int w = 0; w <= kWarps; ++w) {
+      before += w < warp ? sh.warp_sum[w] : 0;
+      total += sh.warp_sum[w];
+    }
+#pragma unroll 1
+    for (int e = e0; e < e1; ++e) sh.ahead[e + e / 32] += before;
+    __syncthreads();
+  }
+  __device__ void look_up(int t) {  // the whole warp; t < total
+    if (t < begin || t >= end) {    // another sequence: the last one that starts at or before it
+      const unsigned coarse = __ballot_sync(0xFFFFFFFFu, lane * 32 < entries && sh.ahead[lane * 33] <= t);
+      const int e0 = (31 - __clz(coarse)) * 32;
+      const unsigned fine = __ballot_sync(0xFFFFFFFFu, e0 + lane < entries && sh.ahead[e0 + lane + e0 / 32] <= t);
+      const int e = e0 + 31 - __clz(fine);
+      begin = sh.ahead[e + e / 32];
+      int4 v = sh.bounds[e];
+      if (step > 1) v = among(e, t);
+      tok0 = v.x;
+      tokens = v.y;
+      row0 = v.z;
+      row_count = v.w;
+      end = begin + tiles_of(tokens);
+    }
+    first = (t - begin) * kRowTileTokens;
+  }
+  // Beyond kTable sequences: tile t's among those of entry e, 32 of them at a time (after the kernel's wait).  Moves `begin` up to it.
+  __device__ int4 among(int e, int t) {
+    const int stop = min(s.batch, (e + 1) * step);
+#pragma unroll 1
+    for (int b0 = e * step; b0 < stop; b0 += 32) {
+      const int b = b0 + lane;
+      const Span q = b < stop ? seq_span<true>(s, cu_seqlens, b) : Span{0, 0, false}, r = b < stop ? row_span<true>(s, cu_qlens, b) : Span{0, 0, false};
+      const int own = tiles_of(q.count), with = begin + sum_upto(own);
+      const unsigned behind = __ballot_sync(0xFFFFFFFFu, with > t);
+      if (behind) {
+        const int from = __ffs(behind) - 1;
+        begin = __shfl_sync(0xFFFFFFFFu, with - own, from);
+        return make_int4(__shfl_sync(0xFFFFFFFFu, q.first, from), __shfl_sync(0xFFFFFFFFu, q.count, from), __shfl_sync(0xFFFFFFFFu, r.first, from),
+                         __shfl_sync(0xFFFFFFFFu, r.count, from));
+      }
+      begin = __shfl_sync(0xFFFFFFFFu, with, 31);
+    }
+    return make_int4(0, 0, 0, 0);
   }
 };
 
@@ -111,7 +152,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap k_map, Shapes s, const uin
   using Ring = RowsRing<DIM>;
   extern __shared__ unsigned char smem_raw[];
   __shared__ uint64_t full[Ring::kStages], empty[Ring::kStages];
-  __shared__ Span spans[2][32];
+  __shared__ SharedList listed;
   __shared__ int abort_flag;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t ring = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -125,33 +166,29 @@ score_rows_kernel(const __grid_constant__ CUtensorMap k_map, Shapes s, const uin
     ptx::prefetch_tensormap(&k_map);
   }
   chain_enter_late(s, cu_seqlens, cu_qlens, q_idx);
-  TileList list(s, cu_seqlens, cu_qlens, lane);
-  list.open(spans, warp);
+  TileList list(s, listed, cu_seqlens, cu_qlens, lane);
+  list.open(warp);
   const int units = list.total * s.hkv, each = units / (int)gridDim.x, more = units - each * (int)gridDim.x;  // (the host sees to it that they fit)
   const int begin = each * (int)blockIdx.x + min((int)blockIdx.x, more), count = each + ((int)blockIdx.x < more ? 1 : 0);
   pdl_wait();  // q and k may be what earlier work wrote; the logits may still be read by it
   pdl_acquire(q);
+  if (blockIdx.x == 0 && list.bad && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
 
   if (warp == kWarps) {
-    if (blockIdx.x == 0 && (list.seq.bad || list.rows.bad) && device_status) atomicOr(device_status, FASTAV_DEV_SHAPE_MISMATCH);
     int it = 0;
     bool ok = true;
     for (; it < count; ++it) {
       const int stage = it % Ring::kStages;
       const int u = begin + it, t = u / s.hkv;
-      list.look_up(t, device_status);
+      list.look_up(t);
       ok = ptx::mbar_wait_warp(ptx::smem_u32(&empty[stage]), ((it / Ring::kStages) & 1) ^ 1u, &abort_flag);
       if (!ok) break;
       if (lane == 0) {
         const uint32_t bar = ptx::smem_u32(&full[stage]);
-        if (list.first < list.tokens) {
-          ptx::mbar_arrive_expect_tx(bar, Ring::kUnitBytes);
+        ptx::mbar_arrive_expect_tx(bar, Ring::kUnitBytes);
 #pragma unroll
-          for (int sub = 0; sub < DIM / 64; ++sub)
-            ptx::tma_load_3d(ring + stage * Ring::kUnitBytes + sub * kSubBytes, &k_map, sub * 64, u - t * s.hkv, list.tok0 + list.first, bar);
-        } else {
-          ptx::mbar_arrive(bar);
-        }
+        for (int sub = 0; sub < DIM / 64; ++sub)
+          ptx::tma_load_3d(ring + stage * Ring::kUnitBytes + sub * kSubBytes, &k_map, sub * 64, u - t * s.hkv, list.tok0 + list.first, bar);
       }
       __syncwarp();
     }
@@ -170,8 +207,8 @@ score_rows_kernel(const __grid_constant__ CUtensorMap k_map, Shapes s, const uin
     const int stage = it % Ring::kStages;
     const int u = begin + it, t = u / s.hkv;
     const int head = u - t * s.hkv;
-    list.look_up(t, device_status);
-    const int m = min(list.tokens - list.first, kRowTileTokens), rows = min(list.row_count, rq), flat = m > 0 ? rows * s.group : 0;
+    list.look_up(t);
+    const int m = min(list.tokens - list.first, kRowTileTokens), rows = min(list.row_count, rq), flat = rows * s.group;
     // Query row f of the KV group: scored row f / G, head f % G.  A lane's 16-byte pieces of a query row, and of a key: elements 64
     // sub + 16 t4 + 8 i (any order of the contraction will do as long as both operands have it; this one reads the
     // swizzled tile free of bank conflicts).
@@ -278,7 +315,7 @@ __global__ void __launch_bounds__(256) score_rows_lse_kernel(Shapes s, const int
   }
 }
 
-// At least the batch's units; of larger batches as many as are listed.
+// At least the batch's units; of larger batches at least what is listed of arrays whose sequences overlap, too.
 long long most_units(const Shapes& s) {
   const long long tiles = s.batch > 32 ? (long long)((s.max_seqlen + kRowTileTokens - 1) / kRowTileTokens) * s.batch
                                        : (long long)s.total_tokens / kRowTileTokens + s.batch;

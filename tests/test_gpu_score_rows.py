@@ -60,3 +60,51 @@ def test_strided_keys(layout):
     assert int(buf.device_status) == int(plain.device_status)
     for name in ("scores", "keep_idx", "cu_keep", "hidden_out", "pos_out", "k_out", "v_out"):
         assert torch.equal(getattr(buf, name), getattr(plain, name)), name
+
+
+@pytest.mark.parametrize("lens", [
+    [2050] + [70] * 32, [64] * 40 + [0] * 3 + [2113, 1, 0, 65], [3, 130] * 500 + [2049] + [64] * 22, [2049] + [40] * 1024, [65, 0, 1] * 700 + [2300, 0, 0],
+    [5] * 33000 + [2049, 7],
+], ids=len)
+@pytest.mark.parametrize("rows", [1, 3])
+def test_many_sequences(lens, rows):
+    """The table of a block: 33 sequences, one entry per thread and several, its last entry, two and three sequences per entry, more than a warp."""
+    p = _problem(lens, rows, 2, 1, 64)
+    buf = parity.to_device(p)
+    buf.prune()
+    torch.cuda.synchronize()
+    parity.check_fused_against_oracle(p, buf, parity.oracle_prune(p), what=f"{len(lens)} sequences")
+
+
+def test_a_cut_sequence_among_many_is_reported():
+    p = _problem([2100] + [50] * 40, 1, 2, 1, 64)
+    buf = parity.to_device(p)
+    buf.params.max_seqlen = 2080
+    buf.prune()
+    torch.cuda.synchronize()
+    assert int(buf.device_status) & fastav.FASTAV_DEV_SHAPE_MISMATCH
+
+
+def _score_us(lens, rows):
+    """Best of five runs of 20 score calls, heads as in the benchmark's larger decoder."""
+    total, cu = sum(lens), lambda v: torch.tensor([0] + v, dtype=torch.int32).cumsum(0).to(torch.int32).cuda()
+    k = torch.randn(total, 8, 128, dtype=torch.bfloat16, device="cuda")
+    buf = fastav.make_buffers(q=torch.randn(sum(rows), 32, 128, dtype=torch.bfloat16, device="cuda"), q_idx=torch.tensor([n - 1 for n, r in zip(lens, rows) if r], dtype=torch.int32).cuda(),
+                              cu_qlens=cu(rows), k=k, v=None, cu_seqlens=cu(lens), keep_counts=torch.ones(len(lens), dtype=torch.int32).cuda(), lens=lens, rows=rows,
+                              keeps=[1] * len(lens))
+    best = float("inf")
+    for _ in range(6):
+        start, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        start.record()
+        for _ in range(20):
+            buf.score()
+        end.record()
+        torch.cuda.synchronize()
+        best = min(best, start.elapsed_time(end) * 50)
+    return best
+
+
+def test_a_long_sequence_among_many_is_shared_out():
+    """64 sequences against 32 with as many tokens and the same longest one: every block's share is as large.  Twice the time leaves room for
+    finding the sequences; two or three blocks with the long one to themselves took ten times as long."""
+    assert _score_us([20000] + [500] * 63, [1] * 64) < 2 * _score_us([20000] + [1016] * 30 + [1020], [1] * 32)
