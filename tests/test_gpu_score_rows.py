@@ -108,3 +108,8 @@ def test_a_long_sequence_among_many_is_shared_out():
     """64 sequences against 32 with as many tokens and the same longest one: every block's share is as large.  Twice the time leaves room for
     finding the sequences; two or three blocks with the long one to themselves took ten times as long."""
     assert _score_us([20000] + [500] * 63, [1] * 64) < 2 * _score_us([20000] + [1016] * 30 + [1020], [1] * 32)
+
+
+def test_keys_of_sequences_without_scored_rows_are_not_read():
+    """Half of the sequences without: the keys are what the call's time goes on, so it should take well below what it takes with all of them."""
+    assert _score_us([3000] * 40, [0, 1] * 20) < 0.8 * _score_us([3000] * 40, [1] * 40)
