@@ -146,7 +146,7 @@ struct TileList {
 };
 
 template <int DIM>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kThreads, 1)
 score_rows_kernel(const __grid_constant__ CUtensorMap k_map, Shapes s, const uint16_t* __restrict__ q, const int32_t* __restrict__ q_idx,
                   const int32_t* __restrict__ cu_qlens, const int32_t* __restrict__ cu_seqlens, float* __restrict__ logits,
                   float2* __restrict__ stats, int rq, int stat_tiles, int32_t* device_status) {
