@@ -96,16 +96,17 @@ struct TileList {
     }
     int before = sum_upto(sum) - sum;
     if (lane == 31) sh.warp_sum[warp] = before + sum;
-    __syncthreads();
-    total = 0;
-#pragma unroll
-    for (int w = 0; w <= kWarps; ++w) {
-      before += w < warp ? sh.warp_sum[w] : 0;
-      total += sh.warp_sum[w];
+    if (entries > 32) {  // (else all of them are the first warp's)
+      __syncthreads();
+#pragma unroll 1
+      for (int w = 0; w < warp; ++w) before += sh.warp_sum[w];
     }
 #pragma unroll 1
     for (int e = e0; e < e1; ++e) sh.ahead[e + e / 32] += before;
     __syncthreads();
+    total = 0;
+#pragma unroll
+    for (int w = 0; w <= kWarps; ++w) total += sh.warp_sum[w];
   }
   __device__ void look_up(int t) {  // the whole warp; t < total
     if (t < begin || t >= end) {    // another sequence: the last one that starts at or before it
