@@ -105,6 +105,7 @@ struct SelectArgs {
   int32_t *keep_idx, *cu_keep, *device_status;
   int32_t* place = nullptr;  // launch_few, optional, [N]: where a token's row goes among the survivors, -1 if it is dropped
 };
+int few_blocks(const Shapes& s);                // ... blocks of that kernel, each on an SM of its own as long as there are as many
 bool few_applies(const Shapes& s);              // from the keys
 bool cluster_select_applies(const Shapes& s);   // from partial sums or scores
 bool few_gathers(const Shapes& s, int row_bytes);

@@ -60,6 +60,13 @@ constexpr int kBulkStages = 4;          // row slots per warp
 constexpr int kAhead = kBulkStages - 2; // rows loaded ahead of the one being stored
 constexpr int kBulkMaxWarps = 8;
 constexpr int kBulkSmemBudget = 200 * 1024;
+// Shared memory that a block asks for at least: more than half of what an SM has, so that a kernel of few rows has one block per SM and no
+// block of the next call's first kernel comes to lie beside it.  That one's key loads want the L1 that is left where shared memory is split
+// for it alone; beside blocks of 25 to 64 KB it started early on an SM split for those, or not, as it happened.  us with what the rows
+// take / 64 KB / 116 KB: 8 x 120 rows of 6 KB, 70 % kept 22.6 / 18.5 / 18.3, 1 x 1,500 22.0 / 22.0 / 17.5, 16 x 120, half kept 24.6 / 20.8 / 19.7, 10 x 170 of
+// 9 KB 18.0 / 16.3 / 15.6.  (Of 400 shapes one lost: 12 x 90 rows of 12 KB, 30 % kept 16.1 / 16.1 / 16.8.)
+constexpr size_t kBulkLeastSmem = 116 * 1024;
+size_t least_smem(size_t used) { return used > kBulkLeastSmem ? used : kBulkLeastSmem; }
 
 __global__ void __launch_bounds__(kBulkMaxWarps * 32, 1)
 compact_rows_bulk_kernel(Shapes s, RowStreams t, const int32_t* __restrict__ keep_idx, const int32_t* __restrict__ cu_keep,
@@ -194,11 +201,11 @@ compact_rows_bulk_kernel(Shapes s, RowStreams t, const int32_t* __restrict__ kee
 // Where shared memory holds all rows of a call, survivors or not, they need not wait for the selection: every warp reads some tokens' rows
 // while the kernel before this one selects, and when that has ended asks for their places among the survivors and stores the rows that
 // have one.  (That kernel lets this one start after its own wait: the rows are complete by then.)
-// What it saves is a trip to memory for the list and one for the rows.  13 fine stages from 744 tokens 148.6 -> 138.5 us, three from
-// 1,024 37.9 -> 36.1, 11 from 576 with rows of 6 KB 125 -> 119.  Rows below 2 KB gain nothing (11 stages from 649, 1.5 KB: 104.6 -> 105.9), and
-// behind the selection from partial sums, which is shorter, dropped rows cost more than is saved (9 x 132 tokens 14.4 -> 14.9).
-constexpr int kPlacedMaxSequences = 31;  // bounds kept one per lane
-constexpr int kPlacedLeastRow = 2048;    // bytes
+// What it saves is a trip to memory for the list and one for the rows; what it costs is reading the dropped rows, beside a kernel that
+// reads keys.  So it is taken where most rows stay (placed_compact_applies).
+constexpr int kPlacedMaxSequences = 16;
+static_assert(kPlacedMaxSequences <= 31, "bounds are kept one per lane");
+constexpr int kPlacedLeastRow = 2048;  // bytes: shorter rows gain nothing (11 stages from 649 tokens, 1.5 KB: 104.6 -> 105.9 us)
 __global__ void __launch_bounds__(kBulkMaxWarps * 32, 1)
 compact_placed_kernel(Shapes s, RowStreams t, const int32_t* __restrict__ place, const int32_t* __restrict__ cu_seqlens, int n_segments, int packed_k, int packed_v,
                       int row_bytes, int slots, int32_t* device_status) {
@@ -253,14 +260,28 @@ compact_placed_kernel(Shapes s, RowStreams t, const int32_t* __restrict__ place,
 
 struct PlacedPlan {
   int warps, slots;
+  bool all_sms;
+  long long bytes(int row_bytes) const { return (long long)warps * slots * row_bytes; }
+  bool fits(int row_bytes) const { return slots <= 32 && bytes(row_bytes) <= kBulkSmemBudget; }
 };
-// As many blocks as SMs, but no block with less than 8 rows or 16 KB: SMs without one are left to the clusters that select (744 tokens, 13
-// stages: 144.3 us with 148 blocks, 138.5 with 124; at least 32 KB 137.3, but 123.6 instead of 121.5 for 13 stages from 126).
-PlacedPlan placed_plan(const Shapes& s, int row_bytes) {
-  const int least = row_bytes > 2048 ? 16384 / row_bytes : 8, even = (s.total_tokens + kNumSMs - 1) / kNumSMs, per_block = even > least ? even : least;
-  PlacedPlan p;
+PlacedPlan placed_on(const Shapes& s, int row_bytes, int sms) {
+  const int least = row_bytes > 2048 ? 16384 / row_bytes : 8;  // blocks of at least about 16 KB or 8 rows
+  const int even = (s.total_tokens + sms - 1) / sms, per_block = even > least ? even : least;
+  PlacedPlan p{};
   p.slots = (per_block + kBulkMaxWarps - 1) / kBulkMaxWarps;
   p.warps = p.slots > 0 ? (per_block + p.slots - 1) / p.slots : 0;
+  return p;
+}
+// A block per SM, and none on the SMs that select if the others hold all rows: a block that has to wait for such an SM starts reading when the
+// selection is over.  us on all SMs / on the others, 80 % kept: 1 x 1,700 rows of 12 KB 21.6 / 20.2, 2 x 800 18.2 / 17.7, 1 x 1,700 of 9 KB 17.3 /
+// 16.2, 8 x 120 of 6 KB 19.4 / 18.7.  From three sequences on the others are fewer, and rings of more than 150 KB there the slower way (3 x 500 rows of
+// 12 KB 16.7 / 17.2, 3 x 650 of 9 KB 15.5 / 16.1).
+PlacedPlan placed_plan(const Shapes& s, int row_bytes) {
+  const int others = kNumSMs - few_blocks(s);
+  PlacedPlan p = placed_on(s, row_bytes, others > 0 ? others : 1);
+  if (others >= kNumSMs / 2 && p.fits(row_bytes) && (s.batch <= 2 || p.bytes(row_bytes) <= kBulkSmemBudget * 3 / 4)) return p;
+  p = placed_on(s, row_bytes, kNumSMs);
+  p.all_sms = true;
   return p;
 }
 
@@ -287,10 +308,10 @@ cudaError_t launch_compact(const Shapes& s, const int32_t* keep_idx, const int32
     if (e != cudaSuccess) return e;
     int blocks = (s.total_keep + warps - 1) / warps;
     if (blocks > kNumSMs) blocks = kNumSMs;
-    // No deeper rings than a warp has rows: the next call's first kernel then fits beside this one on the same SMs.
+    // No deeper rings than a warp has rows.
     const int rows_per_warp = (s.total_keep + blocks * warps - 1) / (blocks * warps);
     const int slots = rows_per_warp < kBulkStages ? rows_per_warp : kBulkStages;
-    const size_t smem = (size_t)warps * slots * row_bytes;
+    const size_t smem = least_smem((size_t)warps * slots * row_bytes);
     e = launch_chained(compact_rows_bulk_kernel, dim3(blocks), dim3(warps * 32), smem, stream, s, t, keep_idx, cu_keep, cu_seqlens,
                        n_segments, (int)plan.packed_k, (int)plan.packed_v, row_bytes, slots, device_status);
     count_launches(1);
@@ -304,11 +325,20 @@ cudaError_t launch_compact(const Shapes& s, const int32_t* keep_idx, const int32
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+// The share kept from which reading all rows pays, us by the list / ahead: 4 x 200 rows of 9 KB 30 % kept 11.7 / 12.1, half 12.5 / 12.1, 80 % 13.9 / 12.5; 1 x
+// 1,000 half 13.9 / 12.9, 80 % 15.7 / 13.1; 8 x 120 half 14.8 / 14.7, 80 % 16.7 / 15.0.  One or two short sequences leave so much of the chip idle
+// that it pays from the first survivor on (330 rows, 10 % kept 10.1 / 9.3), up to 6 MB of dropped rows (2,000 rows of 12 KB, 10 % kept,
+// 22 MB: 17.3 / 21.0).  With more sequences the reads meet more of the selecting kernel's (8 x 230 rows of 12 KB, 30 % kept 15.5 / 18.1, 31 x 60, half
+// 16.5 / 20.2), and where blocks have to wait for an SM at all, it is the slower way from five sequences on (10 x 170 rows of 9 KB, 80 % kept 15.6 / 18.3).
 bool placed_compact_applies(const Shapes& s, const RowStreams& rows) {
   const BulkPlan plan = bulk_plan(s, rows);
   if ((s.flags & FASTAV_COMPACT_PATH_MASK) != 0 || s.batch > kPlacedMaxSequences || s.total_keep <= 0 || plan.row_bytes < kPlacedLeastRow || plan.n_segments > 32) return false;
   const PlacedPlan p = placed_plan(s, plan.row_bytes);
-  return p.slots <= 32 && (long long)p.warps * p.slots * plan.row_bytes <= kBulkSmemBudget;
+  if (!p.fits(plan.row_bytes)) return false;
+  const long long kept = s.total_keep, all = s.total_tokens;
+  if (p.all_sms && (s.batch > 4 || kept * 20 < all * 13)) return false;
+  if (s.batch <= 2 && (all - kept) * plan.row_bytes <= 6ll << 20) return true;
+  return s.batch <= 4 ? kept * 2 >= all : s.batch <= 8 ? kept * 5 >= all * 3 : kept * 4 >= all * 3;
 }
 
 cudaError_t launch_compact_placed(const Shapes& s, const RowStreams& rows, const int32_t* place, const int32_t* cu_seqlens, int32_t* device_status,
@@ -318,7 +348,7 @@ cudaError_t launch_compact_placed(const Shapes& s, const RowStreams& rows, const
   cudaError_t e = once_per_context([] { return cudaFuncSetAttribute(compact_placed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBulkSmemBudget); });
   if (e != cudaSuccess) return e;
   const int per_block = p.warps * p.slots, blocks = (s.total_tokens + per_block - 1) / per_block;
-  e = launch_chained(compact_placed_kernel, dim3(blocks), dim3(p.warps * 32), (size_t)p.warps * p.slots * plan.row_bytes, stream, s, rows, place, cu_seqlens,
+  e = launch_chained(compact_placed_kernel, dim3(blocks), dim3(p.warps * 32), least_smem((size_t)p.bytes(plan.row_bytes)), stream, s, rows, place, cu_seqlens,
                      plan.n_segments, (int)plan.packed_k, (int)plan.packed_v, plan.row_bytes, p.slots, device_status);
   count_launches(1);
   return e != cudaSuccess ? e : cudaGetLastError();

@@ -117,3 +117,24 @@ def test_rows_read_ahead_by_the_blocks_that_select(layout, lens, rows):
     for name in ("hidden", "pos", "k", "v"):
         if getattr(buf, name + "_out") is not None:
             parity.assert_bits_equal(getattr(buf, name + "_out"), mine[name], f"{layout} {name}")
+
+
+@pytest.mark.parametrize("lens,keep,hid,hkv,d,ahead", [
+    ([744], 0.8, 3584, 4, 128, True), ([330], 0.1, 3584, 4, 128, True), ([2000], 0.8, 3584, 4, 128, True), ([2000], 0.3, 3584, 4, 128, False),
+    ([2000], 0.1, 4096, 8, 128, False), ([250] * 4, 0.8, 3584, 4, 128, True), ([250] * 4, 0.3, 3584, 4, 128, False), ([480] * 4, 0.8, 3584, 4, 128, True),
+    ([480] * 4, 0.6, 3584, 4, 128, False), ([120] * 8, 0.75, 3584, 4, 128, True), ([120] * 8, 0.5, 3584, 4, 128, False), ([230] * 8, 0.9, 3584, 4, 128, False),
+    ([120, 0, 90, 33] * 2, 0.8, 1024, 16, 64, True), ([60] * 16, 0.8, 3584, 4, 128, True), ([60, 0, 7, 90] * 4, 0.9, 1024, 16, 64, True),
+    ([60] * 16, 0.5, 3584, 4, 128, False), ([60] * 17, 0.9, 3584, 4, 128, False), ([170] * 10, 0.8, 3584, 4, 128, False), ([1500], 0.9, 504, 2, 128, False),
+])
+def test_rows_are_read_ahead_where_most_of_them_stay(lens, keep, hid, hkv, d, ahead):
+    """The kernel that selects leaves every token's place in the workspace's last part for the gather that reads ahead, and nothing there for the other."""
+    p = _problem(lens, [int(keep * n) for n in lens], hid, 2 * hkv, hkv, d)
+    buf = parity.to_device(p)
+    size = -(-4 * p.total_tokens // 256) * 256
+    places = buf.workspace[fastav.fastav_workspace_bytes(buf.params) - size:].view(torch.int32)[:p.total_tokens]
+    places.fill_(0x77777777)
+    buf.prune()
+    torch.cuda.synchronize()
+    left = places != 0x77777777
+    assert bool(left.all()) if ahead else not bool(left.any())
+    _both(buf)
