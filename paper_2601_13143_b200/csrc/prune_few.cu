@@ -12,9 +12,9 @@
 //           many it keeps.  Beyond, each block runs the whole selection for itself: a histogram of the leading 12 bits,
 //           the keys of the bin that holds the k-th largest finished by counting ranks (further 12-bit passes only if it holds
 //           more than 256), one stable prefix sum in index order;
-//   gather  the survivors among a block's own tokens.  Where shared memory holds the rows of its whole slice, they are on their way from
-//           the beginning and only stored at the end (512 tokens of a small model 10.1 -> 9.8 us, 4 stages from 563 tokens with rows
-//           of 1.5 KB 37.9 -> 35.5).
+//   gather  the survivors among a block's own tokens.  From the keys, where shared memory holds the rows of its whole slice and at least half of
+//           the call's tokens stay, they are on their way from the beginning and only stored at the end (512 tokens of a small model
+//           10.1 -> 9.8 us, 4 stages from 563 tokens with rows of 1.5 KB 37.9 -> 35.5).
 //
 // Bound: latency.  Nothing here is long, so what counts is the number of dependent steps: every index array is asked for
 // at once, the keys before anything that is only needed later, every reduction is spread over as many lanes as keep its
@@ -405,7 +405,6 @@ __global__ void __launch_bounds__(kThreads, 1) prune_few_kernel(Shapes s, FewArg
     pdl_acquire(in);
     protect_rows(0, kThreads);
     selection_inputs();
-    read_ahead();
     cluster_wait();
     __syncthreads();
     const float* const col = in + tok0 + t0;
@@ -729,15 +728,15 @@ cudaError_t launch(const Shapes& s, FewArgs a, int blocks, size_t smem, const Ro
     a.rows = *rows;
     a.plan = bulk_plan(s, *rows);
     const size_t at = align_up(smem, 128), all = at + (size_t)a.slice_cap * (a.plan.row_bytes + sizeof(int));
-    if (a.plan.n_segments <= 32 && a.slice_cap <= kThreads && all <= kMaxDynamic) {
+    if (FRONT == kKeys && 2ll * s.total_keep >= s.total_tokens && a.plan.n_segments <= 32 && a.slice_cap <= kThreads && all <= kMaxDynamic) {
       a.ring = (int)at;
       smem = all;
     }
   }
-  if constexpr (FRONT == kKeys)
+  if constexpr (FRONT == kKeys) {
     if (a.place) return launch_kernel<FRONT, DIM, kPlaces>(s, a, blocks, smem, t, stream);
-  if constexpr (FRONT != kScores)
     if (a.ring) return launch_kernel<FRONT, DIM, kAhead>(s, a, blocks, smem, t, stream);
+  }
   return launch_kernel<FRONT, DIM, kByList>(s, a, blocks, smem, t, stream);
 }
 
