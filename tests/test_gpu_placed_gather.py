@@ -165,3 +165,20 @@ def test_few_survivors_take_no_longer_behind_partial_sums():
             times.append(start.elapsed_time(end))
         medians.append(sorted(times)[5])
     assert medians[0] < 1.05 * medians[1]
+
+
+def test_what_the_workspace_held_moves_no_row():
+    """Tokens cut off a sequence that is longer than promised have no place: were the stale one read, it would name an output row that no survivor has."""
+    p = _problem([400, 350], [300, 250])
+    buf = parity.to_device(p)
+    buf.params.max_seqlen = 380
+    buf.keep_counts -= 10
+    spare = buf.params.total_keep - 1
+    buf.workspace.view(torch.int32).fill_(spare)
+    for name in ("hidden_out", "pos_out", "k_out", "v_out"):
+        getattr(buf, name).view(torch.uint8).fill_(0x55)
+    buf.prune()
+    torch.cuda.synchronize()
+    assert int(buf.cu_keep[-1]) == spare - 19 and int(buf.device_status) & fastav.FASTAV_DEV_SHAPE_MISMATCH
+    for name in ("hidden_out", "pos_out", "k_out", "v_out"):
+        assert bool((getattr(buf, name)[spare - 19:].contiguous().view(torch.uint8) == 0x55).all()), name

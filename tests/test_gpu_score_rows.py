@@ -5,6 +5,7 @@ import pytest
 import torch
 
 import parity
+import test_gpu_equal_keys as equal_keys
 from paper_2601_13143_b200 import fastav, workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -113,3 +114,23 @@ def test_a_long_sequence_among_many_is_shared_out():
 def test_keys_of_sequences_without_scored_rows_are_not_read():
     """Half of the sequences without: the keys are what the call's time goes on, so it should take well below what it takes with all of them."""
     assert _score_us([3000] * 40, [0, 1] * 20) < 0.8 * _score_us([3000] * 40, [1] * 40)
+
+
+@pytest.mark.parametrize("lens,rows,hq,hkv,d", [([2049], 1, 28, 4, 128), ([5000, 2100, 70], 3, 8, 2, 64)])
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+def test_an_infinite_key_leaves_the_others_alone(lens, rows, hq, hkv, d, value):
+    """By the separate kernels and by the selection from the logits: +infinity for the even heads, -infinity for the odd ones, in two keys of each sequence."""
+    p, _ = equal_keys._problem(lens, rows, hq, hkv, d, 0.5)
+    p.q[:, ::2, 0], p.q[:, 1::2, 0] = 1, -1
+    for a, n in zip(p.cu_seqlens.tolist(), lens):
+        p.k[[a + n // 3, a + n // 2], :, 0] = value
+    want = equal_keys._reference(p)
+    there = ~want.isnan()
+    buf = parity.to_device(p)
+    for call in (buf.score, buf.prune):
+        buf.scores.fill_(-1.0)
+        call()
+        got = buf.scores.cpu().double()
+        assert torch.equal(got.isnan(), want.isnan()), f"{int(got.isnan().sum())} scores are NaN, {int(want.isnan().sum())} should be"
+        err = (got - want).abs()[there]
+        assert bool((err <= parity.SCORE_RTOL * want[there].abs() + parity.SCORE_ATOL).all()), float(err.max())

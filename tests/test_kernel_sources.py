@@ -34,3 +34,8 @@ def test_a_block_that_gives_up_waits_for_its_copies(name):
     for kernel in _kernels(name):
         if re.search(r"\b(?:bulk_load|tma_load_\w+)\(", kernel):
             assert re.search(r"mbar_wait_bounded\([^;]*&never\)", kernel) or "drain_loads(" in kernel, f"{name}: {kernel[:120]}"
+
+
+@pytest.mark.parametrize("name", ["score_rows.cu", "prune_few.cu"])
+def test_warps_that_shuffle_behind_a_bounded_wait_decide_on_one_answer(name):
+    test_a_warp_that_votes_decides_on_one_answer(name)
