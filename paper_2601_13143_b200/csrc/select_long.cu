@@ -5,7 +5,7 @@
 //
 // The keys stay where they are.  A pass takes 11 bits: each block counts its slice's digits, adds the bins it has to the block that
 // owns them (distributed shared memory), and after a cluster barrier each reads all totals and finds the bin of the k-th largest
-// for itself.  Where that bin holds at most 512 keys the blocks send one another theirs and how many they have above the bin, and each
+// for itself.  Where that bin holds at most 192 keys the blocks send one another theirs and how many they have above the bin, and each
 // ranks them all by counting, else the next pass follows.  From that each block also knows what the blocks before it keep.
 //
 // Bound: latency, a chain of a dozen steps of which three are cluster barriers; from the wait to the end 8.3 us (3 x 8,001-9,001 tokens) to 9.2
@@ -30,7 +30,10 @@ constexpr int kSlice = kPer * kThreads;      // most tokens of a block
 constexpr int kDigitBits = 11;
 constexpr int kBins = 1 << kDigitBits;
 constexpr int kBinsPerThread = kBins / kThreads;  // two words of two counts
-constexpr int kListMax = kThreads;           // keys of a bin that are ranked by counting
+// Keys of a bin that are ranked by counting.  Their comparisons grow with the square, another pass over the bits costs 2 us whatever its keys:
+// 1 x 3,633 tokens, 23 rows, some 240 / 300 / 400 keys in the bin with a limit of 512 22.1 / 24.9 / 28.1 us, with 192 21.8 (with 128 some more
+// calls pay the pass: 21.8 instead of 21.3 at 150 keys).
+constexpr int kListMax = 192;
 constexpr int kMaxTerms = 256 * kNarrowMaxRows;  // heads x scored rows of the few-rows path
 // Shared memory that a block asks for, so that no block of a compaction (192 KB and more) is resident beside it: those wait for the
 // selection and slow it down.  Together with the successor started ahead of the passes instead of first thing: 32 ragged
@@ -395,7 +398,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
         if (tid < bucket) {
           int at = tid, from = 0;
           while (from < blocks - 1 && at >= (int)(sh.count_of[from] & 0xFFFFu)) at -= (int)(sh.count_of[from++] & 0xFFFFu);
-          list_key = remote_load(remote(&sh.list[at & (kListMax - 1)], from));
+          list_key = remote_load(remote(&sh.list[min(at, kListMax - 1)], from));
           list_from = from;
           sh.all[tid] = list_key;
         }

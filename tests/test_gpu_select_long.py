@@ -80,3 +80,35 @@ def test_window_of_the_first_pass(kind, lens, rows, lowest):
         protect = (torch.arange(p.total_tokens) % 2).to(torch.uint8)
     p.keep_counts = torch.tensor(keeps, dtype=torch.int32)
     parity.check_prune_under_flags(p, lowest, False, True, False, protect, f"{kind} {lens[0]} x {len(lens)}")
+
+
+def test_scores_close_together_take_no_longer():
+    """1 x 3,633 tokens with scores from far apart to within a few percent: the threshold's first bin holds from some 60 keys to more than a
+    thousand.  Ranking them by counting up to 512 of them made one of these calls 1.3 times as long as another; another pass is a tenth."""
+    medians = []
+    for spread in (0.5, 1.0, 1.15, 1.3, 1.5, 1.75):
+        gen = torch.Generator(device="cuda").manual_seed(3)
+        normal = lambda *shape: torch.randn(shape, generator=gen, device="cuda", dtype=torch.bfloat16)
+        one = lambda *v: torch.tensor(v, dtype=torch.int32, device="cuda")
+        k = normal(3633, 4, 128)
+        buf = fastav.make_buffers(q=normal(23, 32, 128) * spread, q_idx=torch.arange(3610, 3633, dtype=torch.int32, device="cuda"), cu_qlens=one(0, 23), k=k, v=None,
+                                  cu_seqlens=one(0, 3633), keep_counts=one(1453), lens=[3633], rows=[23], keeps=[1453])
+        side = torch.cuda.Stream()
+        side.wait_stream(torch.cuda.current_stream())
+        for _ in range(3):
+            buf.prune(side)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side):
+            for _ in range(20):
+                buf.prune(side)
+        times = []
+        for _ in range(11):
+            start, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            start.record()
+            graph.replay()
+            end.record()
+            torch.cuda.synchronize()
+            times.append(start.elapsed_time(end))
+        medians.append(sorted(times)[5])
+    assert max(medians) < 1.12 * min(medians), medians
