@@ -722,7 +722,7 @@ cudaError_t launch(const Shapes& s, FewArgs a, int blocks, size_t smem, const Ro
   // Four sequences and more, and a gather of few rows behind: that is as short as the launch of the next call's first kernel, which it is to hide
   // and which waits for this trigger first.  From the start / behind the keys, us: 16 x 60 rows of 12 KB, 60 % kept 15.3 / 18.1, 16 x 120 of 6 KB 16.2 / 18.6, 8
   // x 230 of 12 KB, 30 % 15.6 / 17.7.  Up to three sequences start late by 0.1 sooner.
-  a.early = FRONT == kKeys && a.do_select && !rows && !a.place && s.batch >= 4;
+  a.early = FRONT == kKeys && (!a.do_select || (!rows && !a.place && s.batch >= 4));
   if (rows) {
     a.do_gather = 1;
     a.rows = *rows;

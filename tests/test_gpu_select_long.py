@@ -5,6 +5,7 @@ import pytest
 import torch
 
 import parity
+import timing
 from paper_2601_13143_b200 import fastav, workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -93,22 +94,5 @@ def test_scores_close_together_take_no_longer():
         k = normal(3633, 4, 128)
         buf = fastav.make_buffers(q=normal(23, 32, 128) * spread, q_idx=torch.arange(3610, 3633, dtype=torch.int32, device="cuda"), cu_qlens=one(0, 23), k=k, v=None,
                                   cu_seqlens=one(0, 3633), keep_counts=one(1453), lens=[3633], rows=[23], keeps=[1453])
-        side = torch.cuda.Stream()
-        side.wait_stream(torch.cuda.current_stream())
-        for _ in range(3):
-            buf.prune(side)
-        torch.cuda.synchronize()
-        graph = torch.cuda.CUDAGraph()
-        with torch.cuda.graph(graph, stream=side):
-            for _ in range(20):
-                buf.prune(side)
-        times = []
-        for _ in range(11):
-            start, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
-            start.record()
-            graph.replay()
-            end.record()
-            torch.cuda.synchronize()
-            times.append(start.elapsed_time(end))
-        medians.append(sorted(times)[5])
+        medians.append(timing.us_per_call(buf.prune))
     assert max(medians) < 1.12 * min(medians), medians

@@ -8,6 +8,7 @@ import torch
 
 import oracle
 import parity
+import timing
 from paper_2601_13143_b200 import fastav, workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -121,3 +122,9 @@ def test_flags_of_the_selection(lens, rows, lowest, global_idx, by_rows, lse):
         p.q_idx[cuq[b]:cuq[b + 1]] = p.q_idx[cuq[b]:cuq[b + 1]].sort().values
     protect = (torch.arange(p.total_tokens) % 29 == 3).to(torch.uint8) if len(lens) % 2 else None
     parity.check_prune_under_flags(p, lowest, global_idx, by_rows, lse, protect, f"{lens[0]} x {len(lens)}, {rows} rows")
+
+
+def test_the_scores_of_a_short_sequence_alone():
+    """300 tokens of a small model: without a selection and a gather behind, by far less than with them (the next call's launch is hidden)."""
+    buf = parity.to_device(W.random_problem(seed=2, lens=[300], rows=[1], keeps=[150], num_q_heads=8, num_kv_heads=2, head_dim=64, hidden=512))
+    assert timing.us_per_call(buf.score) < 0.6 * timing.us_per_call(buf.prune)
