@@ -362,7 +362,13 @@ cudaError_t launch_score_narrow(const Shapes& s, const Workspace& w, const void*
   cudaError_t e = launch_rows(s, w, q, q_idx, cu_qlens, k, cu_seqlens, ws, device_status, stream, &by_mma);
   if (e == cudaSuccess && !by_mma) e = launch_narrow_logits(s, w, q, q_idx, cu_qlens, k, cu_seqlens, ws, device_status, stream);
   if (e != cudaSuccess) return e;
-  if (by_mma && left && long_select_applies(s)) {  // the kernel that selects starts from the logits
+  // The kernel that selects starts from the logits: two launches less, but its few blocks merge the statistics and add the terms (heads x rows) up, where
+  // the kernels of their own have the whole chip.  us in a prune call, 70 % kept, from the logits / by kernels of their own: 28 terms 1 x 2,500 tokens 24.5 /
+  // 27.9, 56 29.8 / 26.9, 112 39.8 / 34.2, 8 x 3,000 90.0 / 83.6.  One block per sequence selects then, which costs more than that with many
+  // sequences (32 ragged ones, 112 terms 201 / 207) and with long ones (1 x 20,000, 56 terms 78.0 / 80.6, 112 97.0 / 91.1).
+  const int terms = s.hq * s.max_qlen;
+  const bool from_logits = terms <= 40 || s.batch >= 24 || (terms <= 64 && s.max_seqlen > 16384);
+  if (by_mma && left && from_logits && long_select_applies(s)) {
     left->kind = ScoreLeft::kLogits;
     return cudaSuccess;
   }

@@ -6,6 +6,7 @@ import torch
 
 import parity
 import test_gpu_equal_keys as equal_keys
+import timing
 from paper_2601_13143_b200 import fastav, workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -87,22 +88,13 @@ def test_a_cut_sequence_among_many_is_reported():
 
 
 def _score_us(lens, rows):
-    """Best of five runs of 20 score calls, heads as in the benchmark's larger decoder."""
+    """A score call, heads as in the benchmark's larger decoder."""
     total, cu = sum(lens), lambda v: torch.tensor([0] + v, dtype=torch.int32).cumsum(0).to(torch.int32).cuda()
     k = torch.randn(total, 8, 128, dtype=torch.bfloat16, device="cuda")
     buf = fastav.make_buffers(q=torch.randn(sum(rows), 32, 128, dtype=torch.bfloat16, device="cuda"), q_idx=torch.tensor([n - 1 for n, r in zip(lens, rows) if r], dtype=torch.int32).cuda(),
                               cu_qlens=cu(rows), k=k, v=None, cu_seqlens=cu(lens), keep_counts=torch.ones(len(lens), dtype=torch.int32).cuda(), lens=lens, rows=rows,
                               keeps=[1] * len(lens))
-    best = float("inf")
-    for _ in range(6):
-        start, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
-        start.record()
-        for _ in range(20):
-            buf.score()
-        end.record()
-        torch.cuda.synchronize()
-        best = min(best, start.elapsed_time(end) * 50)
-    return best
+    return timing.us_per_call(buf.score)
 
 
 def test_a_long_sequence_among_many_is_shared_out():
@@ -134,3 +126,17 @@ def test_an_infinite_key_leaves_the_others_alone(lens, rows, hq, hkv, d, value):
         assert torch.equal(got.isnan(), want.isnan()), f"{int(got.isnan().sum())} scores are NaN, {int(want.isnan().sum())} should be"
         err = (got - want).abs()[there]
         assert bool((err <= parity.SCORE_RTOL * want[there].abs() + parity.SCORE_ATOL).all()), float(err.max())
+
+
+@pytest.mark.parametrize("hq,hkv,rows", [(28, 4, 4), (32, 8, 4), (32, 8, 2)])
+def test_a_prune_call_takes_no_longer_than_its_parts(hq, hkv, rows):
+    """1 x 2,500 tokens: the selection from the logits against score, select and compact one after the other."""
+    p = W.random_problem(seed=4, lens=[2500], rows=[rows], keeps=[1750], num_q_heads=hq, num_kv_heads=hkv, head_dim=128, hidden=3584)
+    buf = parity.to_device(p)
+
+    def parts(stream):
+        buf.score(stream)
+        buf.select(stream)
+        buf.compact(stream)
+
+    assert timing.us_per_call(buf.prune) < 1.05 * timing.us_per_call(parts)
