@@ -79,8 +79,8 @@ struct TileList {
   // All threads of the block.  Each bound is asked for by one thread of it (by all its warps: a microsecond on a few lines of L2).
   // (Loops kept as loops: of a large call every line of code comes from memory again.)
   __device__ void open(int warp) {
-    step = (s.batch + kTable - 1) / kTable;
-    entries = (s.batch + step - 1) / step;
+    step = s.batch <= kTable ? 1 : (s.batch + kTable - 1) / kTable;
+    entries = step == 1 ? s.batch : (s.batch + step - 1) / step;
     const int each = (entries + kThreads - 1) / kThreads, e0 = min(entries, (int)threadIdx.x * each), e1 = min(entries, e0 + each);
     int sum = 0;
 #pragma unroll 1
