@@ -136,10 +136,6 @@ bool once_plan(const Shapes& s, bool lse_given, OncePlan* plan);
 cudaError_t launch_score_once(const Shapes& s, const void* k_map, const void* q_map, const int32_t* q_idx, const int32_t* cu_qlens,
                               const int32_t* cu_seqlens, const float* lse_in, const OncePlan& plan, float* partial, int32_t* device_status,
                               cudaStream_t stream);
-// Only the logits [Hq, max_qlen, N] of the few-rows path, into the workspace.
-cudaError_t launch_narrow_logits(const Shapes& s, const Workspace& w, const void* q, const int32_t* q_idx,
-                                 const int32_t* cu_qlens, const void* k, const int32_t* cu_seqlens, unsigned char* ws,
-                                 int32_t* device_status, cudaStream_t stream);
 
 cudaError_t launch_select(const Shapes& s, const Workspace& w, const float* scores, const int32_t* cu_seqlens,
                           const int32_t* keep_counts, const uint8_t* protect, const int32_t* q_idx,

@@ -15,6 +15,7 @@
 // Every key goes through the same arithmetic in the same order, whatever its position, so equal
 // keys get bit-equal scores and runs are bit-reproducible.
 #include "common.cuh"
+#include "gather.cuh"
 #include "row_stats.cuh"
 #include "sm100_ptx.cuh"
 
@@ -31,12 +32,6 @@ __device__ __forceinline__ void unpack8(const uint4& v, float2 (&out)[4]) {
   out[1] = make_float2(__uint_as_float(v.y << 16), __uint_as_float(v.y & 0xFFFF0000u));
   out[2] = make_float2(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xFFFF0000u));
   out[3] = make_float2(__uint_as_float(v.w << 16), __uint_as_float(v.w & 0xFFFF0000u));
-}
-
-__device__ __forceinline__ void bulk_load(uint32_t dst_smem, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst_smem),
-               "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(bar)
-               : "memory");
 }
 
 // DIM: head_dim; ROWS: query rows handled per pass (4 or 8).  One block covers `heads_per_block` KV heads
@@ -320,10 +315,7 @@ cudaError_t launch_logits(const Shapes& s, const uint16_t* q, const int32_t* q_i
                         logits, rq, hb, (int)chunk, device_status);
 }
 
-}  // namespace
-
-bool score_narrow_applies(const Shapes& s) { return s.max_qlen >= 1 && s.max_qlen <= kNarrowMaxRows && s.hq <= 256; }
-
+// Only the logits, into the workspace.
 cudaError_t launch_narrow_logits(const Shapes& s, const Workspace& w, const void* q, const int32_t* q_idx,
                                  const int32_t* cu_qlens, const void* k, const int32_t* cu_seqlens, unsigned char* ws,
                                  int32_t* device_status, cudaStream_t stream) {
@@ -343,6 +335,10 @@ cudaError_t launch_narrow_logits(const Shapes& s, const Workspace& w, const void
   count_launches(1);
   return e;
 }
+
+}  // namespace
+
+bool score_narrow_applies(const Shapes& s) { return s.max_qlen >= 1 && s.max_qlen <= kNarrowMaxRows && s.hq <= 256; }
 
 cudaError_t launch_score_narrow(const Shapes& s, const Workspace& w, const void* q, const int32_t* q_idx,
                                 const int32_t* cu_qlens, const void* k, const int32_t* cu_seqlens, const float* lse_in,

@@ -7,11 +7,11 @@
 //              instruction; the query rows come from L1).  Logits [Hq, R, N] (R: the sequence's own rows; base-2 units, -inf where the
 //              causal mask hides the key) go to the workspace, and with them (max, sum 2^(z - max)) of every row over the unit's tokens.
 //   the rest : log-sum-exp per row from those pairs, and per token the fixed-order sum over heads and rows -- by the kernel that
-//              selects (select_long.cu), or by two small kernels where the scores alone are wanted.
+//              selects (select_long.cu), or by two small kernels where the scores alone are wanted or the terms are many.
 //
-// A prune call with one row on 4 x 6,554 tokens (Mistral-7B shapes, 70 % kept) takes 97.4 us instead of 109.4 with a tcgen05 kernel
+// A prune call with one row on 4 x 6,554 tokens (Mistral-7B shapes, 70 % kept) takes 95.5 us instead of 109.4 with a tcgen05 kernel
 // for the logits and one each for statistics, scores and selection (its logits 23.5 us, the keys' floor 8.3), 32 ragged sequences of
-// 512 to 4,096 tokens 205 instead of 217.5.  Of the 12 us from the start to the last unit 1.9 are the sequences' bounds (cold), about
+// 512 to 4,096 tokens 204 instead of 217.5.  Of the 12 us from the start to the last unit 1.9 are the sequences' bounds (cold), about
 // 9 the keys.  Taken and put back: fragments straight from global memory, a block per tile (27 us: not enough bytes in flight);
 // four warps (14 us: they are the bound); the first 8 or 16 units prefetched into L2 ahead of the bounds (97.5 -> 97.9, 98.6).
 //

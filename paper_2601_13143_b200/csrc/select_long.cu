@@ -35,8 +35,8 @@ constexpr int kBinsPerThread = kBins / kThreads;  // two words of two counts
 // calls pay the pass: 21.8 instead of 21.3 at 150 keys).
 constexpr int kListMax = 192;
 constexpr int kMaxTerms = 256 * kNarrowMaxRows;  // heads x scored rows of the few-rows path
-// Shared memory that a block asks for, so that no block of a compaction (192 KB and more) is resident beside it: those wait for the
-// selection and slow it down.  Together with the successor started ahead of the passes instead of first thing: 32 ragged
+// Shared memory that a block asks for, so that no block of a compaction with full rings (192 KB; fewer survivors make shorter ones) is resident
+// beside it: those wait for the selection and slow it down.  Together with the successor started ahead of the passes instead of first thing: 32 ragged
 // sequences of up to 8,192 tokens 307 -> 301 us, 4 x 16,384 292 -> 288.
 constexpr size_t kLeastBytes = 64 * 1024;
 constexpr int kSent = 32;                    // keys that a block sends to the others
@@ -73,6 +73,7 @@ struct LongArgs {
 
 // After LongShared: the scores of the slice, then the totals of the bins this block owns, of the whole cluster.
 __host__ __device__ inline int owned_words(int blocks) { return kBins / 2 / blocks; }
+static_assert(kBins / 2 / kMaxCluster % 4 == 0, "cleared 16 bytes at a time");
 // ... and of kLogits what each term's weights are made with, at most `terms`.
 inline size_t long_bytes(int blocks, int slice_cap, int terms) {
   const size_t used = sizeof(LongShared) + (size_t)(slice_cap + owned_words(blocks) + 2 * terms) * sizeof(unsigned);
@@ -135,7 +136,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_long_kernel(Shapes s, Long
   const int blocks = a.blocks, b = (int)blockIdx.x / blocks, c = (int)cluster_rank();
   unsigned* const keys = reinterpret_cast<unsigned*>(smem_raw + sizeof(LongShared));
   unsigned* const totals = keys + a.slice_cap;
-  const int owned = owned_words(blocks);  // of an owner: a power of two, at least 256 words
+  const int owned = owned_words(blocks);  // of an owner: a power of two, at least 64 words
   auto clear_counts = [&] {
     for (int i = tid; i < kBins / 8; i += kThreads) reinterpret_cast<uint4*>(sh.hist)[i] = make_uint4(0, 0, 0, 0);
     for (int i = tid; i < owned / 4; i += kThreads) reinterpret_cast<uint4*>(totals)[i] = make_uint4(0, 0, 0, 0);
