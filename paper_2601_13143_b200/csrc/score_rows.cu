@@ -48,15 +48,22 @@ struct RowsRing {
 // 656; 100 of 300 to 3,000 tokens 72 / 131 and 482 / 532).  The spans in registers and shuffles for up to 32 sequences were no quicker (20 x
 // 3,000 tokens 32.3 / 32.0 us).
 constexpr int kTable = 1024;
+// Behind the ring, as large as the batch needs (all of it always there: 4 x 6,554 tokens 95.7 us instead of 95.6).
 struct SharedList {
-  int4 bounds[kTable];              // first token, tokens, first scored row, scored rows (step 1)
-  int ahead[kTable + kTable / 32];  // entry e at e + e / 32: both looks are free of bank conflicts
-  int warp_sum[kWarps + 1];
+  int4* bounds;  // [entries] first token, tokens, first scored row, scored rows (step 1)
+  int* ahead;    // entry e at e + e / 32: both looks are free of bank conflicts
+  int* warp_sum;
 };
+__host__ __device__ inline int table_entries(int batch) {
+  if (batch <= kTable) return batch;
+  const int step = (batch + kTable - 1) / kTable;
+  return (batch + step - 1) / step;
+}
+inline int table_bytes(int batch) { return table_entries(batch) * (int)(sizeof(int4) + sizeof(int)) + (table_entries(batch) / 32 + 1) * (int)sizeof(int); }
 
 struct TileList {
   const Shapes& s;
-  SharedList& sh;
+  const SharedList sh;
   const int32_t *cu_seqlens, *cu_qlens;
   int lane;
   int step, entries, total;
@@ -64,7 +71,7 @@ struct TileList {
   // of the tile looked up last, in all lanes
   int first = 0, tok0 = 0, tokens = 0, row0 = 0, row_count = 0;
   int begin = 0, end = 0;   // the tiles of its sequence
-  __device__ TileList(const Shapes& s_, SharedList& sh_, const int32_t* cu_seqlens_, const int32_t* cu_qlens_, int lane_)
+  __device__ TileList(const Shapes& s_, const SharedList& sh_, const int32_t* cu_seqlens_, const int32_t* cu_qlens_, int lane_)
       : s(s_), sh(sh_), cu_seqlens(cu_seqlens_), cu_qlens(cu_qlens_), lane(lane_) {}
   // A sequence without scored rows has none: nobody needs its keys (20 x 3,000 tokens, every second one without: 185 us instead of 196).
   static __device__ int tiles_of(int tokens, int rows) { return rows > 0 ? (tokens + kRowTileTokens - 1) / kRowTileTokens : 0; }
@@ -80,7 +87,7 @@ struct TileList {
   // (Loops kept as loops: of a large call every line of code comes from memory again.)
   __device__ void open(int warp) {
     step = s.batch <= kTable ? 1 : (s.batch + kTable - 1) / kTable;
-    entries = step == 1 ? s.batch : (s.batch + step - 1) / step;
+    entries = table_entries(s.batch);
     const int each = (entries + kThreads - 1) / kThreads, e0 = min(entries, (int)threadIdx.x * each), e1 = min(entries, e0 + each);
     int sum = 0;
 #pragma unroll 1
@@ -154,8 +161,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap k_map, Shapes s, const uin
   using Ring = RowsRing<DIM>;
   extern __shared__ unsigned char smem_raw[];
   __shared__ uint64_t full[Ring::kStages], empty[Ring::kStages];
-  __shared__ SharedList listed;
-  __shared__ int abort_flag;
+  __shared__ int warp_sum[kWarps + 1], abort_flag;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t ring = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   if (threadIdx.x == 0) {
@@ -168,7 +174,8 @@ score_rows_kernel(const __grid_constant__ CUtensorMap k_map, Shapes s, const uin
     ptx::prefetch_tensormap(&k_map);
   }
   chain_enter_late(s, cu_seqlens, cu_qlens, q_idx);
-  TileList list(s, listed, cu_seqlens, cu_qlens, lane);
+  int4* const table = reinterpret_cast<int4*>(smem_raw + (ring - ptx::smem_u32(smem_raw)) + kRingBytes);
+  TileList list(s, SharedList{table, reinterpret_cast<int*>(table + table_entries(s.batch)), warp_sum}, cu_seqlens, cu_qlens, lane);
   list.open(warp);
   const int units = list.total * s.hkv, each = units / (int)gridDim.x, more = units - each * (int)gridDim.x;  // (the host sees to it that they fit)
   const int begin = each * (int)blockIdx.x + min((int)blockIdx.x, more), count = each + ((int)blockIdx.x < more ? 1 : 0);
@@ -326,8 +333,10 @@ long long most_units(const Shapes& s) {
 template <int DIM>
 cudaError_t run(const Shapes& s, const CUtensorMap& k_map, const uint16_t* q, const int32_t* q_idx, const int32_t* cu_qlens, const int32_t* cu_seqlens,
                 float* logits, float2* stats, int stat_tiles, int32_t* device_status, cudaStream_t stream) {
-  constexpr int smem = kRingBytes + 1024;
-  cudaError_t e = once_per_context([] { return cudaFuncSetAttribute(score_rows_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
+  const int smem = kRingBytes + 1024 + table_bytes(s.batch);
+  cudaError_t e = once_per_context([] {
+    return cudaFuncSetAttribute(score_rows_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes + 1024 + table_bytes(kTable));
+  });
   if (e != cudaSuccess) return e;
   const long long units = most_units(s);
   count_launches(1);
