@@ -9,9 +9,9 @@
 //   the rest : log-sum-exp per row from those pairs, and per token the fixed-order sum over heads and rows -- by the kernel that
 //              selects (select_long.cu), or by two small kernels where the scores alone are wanted or the terms are many.
 //
-// A prune call with one row on 4 x 6,554 tokens (Mistral-7B shapes, 70 % kept) takes 95.5 us instead of 109.4 with a tcgen05 kernel
+// A prune call with one row on 4 x 6,554 tokens (Mistral-7B shapes, 70 % kept) takes 93.6 us instead of 109.4 with a tcgen05 kernel
 // for the logits and one each for statistics, scores and selection (its logits 23.5 us, the keys' floor 8.3), 32 ragged sequences of
-// 512 to 4,096 tokens 204 instead of 217.5.  Of the 12 us from the start to the last unit 1.9 are the sequences' bounds (cold), about
+// 512 to 4,096 tokens 203 instead of 217.5.  Of the 12 us from the start to the last unit 1.9 are the sequences' bounds (cold), about
 // 9 the keys.  Taken and put back: fragments straight from global memory, a block per tile (27 us: not enough bytes in flight);
 // four warps (14 us: they are the bound); the first 8 or 16 units prefetched into L2 ahead of the bounds (97.5 -> 97.9, 98.6).
 //
@@ -41,14 +41,14 @@ struct RowsRing {
   static_assert(kStages % kWarps == 0);
 };
 
-// The batch's tiles of 64 tokens in one list.  Shared memory has for every sequence its bounds and how many tiles come before it (of
-// batches beyond kTable for every `step`-th), and a warp finds a tile's sequence in two looks of 32 entries.  The list has to be exact, since every
-// block takes an equal run of it: with every sequence given as many tiles as the longest one has, the real ones of 64 sequences,
-// one of 20,000 tokens and 63 of 500, all fell to a few blocks (Mistral-7B shapes, one row: score call 49 us instead of 503, prune 205 instead of
-// 656; 100 of 300 to 3,000 tokens 72 / 131 and 482 / 532).  The spans in registers and shuffles for up to 32 sequences were no quicker (20 x
-// 3,000 tokens 32.3 / 32.0 us).
+// The batch's tiles of 64 tokens in one list.  Up to 32 sequences each lane of a warp knows one; beyond, shared memory has for every sequence its
+// bounds and how many tiles come before it (of batches beyond kTable for every `step`-th), and a warp finds a tile's sequence in two looks of 32
+// entries.  The list has to be exact, since every block takes an equal run of it: with every sequence given as many tiles as the longest one
+// has, the real ones of 64 sequences, one of 20,000 tokens and 63 of 500, all fell to a few blocks (Mistral-7B shapes, one row: score call 49 us
+// instead of 503, prune 205 instead of 656; 100 of 300 to 3,000 tokens 72 / 131 and 482 / 532).  Two kernels, since all of a large call's code comes
+// from memory again: 4 x 6,554 tokens 93.6 us, with the table for every batch 95.6, with both in one kernel 95.0.
 constexpr int kTable = 1024;
-// Behind the ring, as large as the batch needs (all of it always there: 4 x 6,554 tokens 95.7 us instead of 95.6).
+// Behind the ring, as large as the batch needs.
 struct SharedList {
   int4* bounds;  // [entries] first token, tokens, first scored row, scored rows (step 1)
   int* ahead;    // entry e at e + e / 32: both looks are free of bank conflicts
@@ -61,7 +61,55 @@ __host__ __device__ inline int table_entries(int batch) {
 }
 inline int table_bytes(int batch) { return table_entries(batch) * (int)(sizeof(int4) + sizeof(int)) + (table_entries(batch) / 32 + 1) * (int)sizeof(int); }
 
-struct TileList {
+// A sequence without scored rows has none: nobody needs its keys (20 x 3,000 tokens, every second one without: 185 us instead of 196).
+__device__ __forceinline__ int tiles_of(int tokens, int rows) { return rows > 0 ? (tokens + kRowTileTokens - 1) / kRowTileTokens : 0; }
+__device__ __forceinline__ int sum_upto(int lane, int v) {
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int t = __shfl_up_sync(0xFFFFFFFFu, v, d);
+    if (lane >= d) v += t;
+  }
+  return v;
+}
+
+// Up to 32 sequences: each lane knows one, and a vote of the warp finds a tile's.
+struct LaneList {
+  const Shapes& s;
+  const SharedList sh;
+  const int32_t *cu_seqlens, *cu_qlens;
+  int lane;
+  int4 mine{0, 0, 0, 0};  // this lane's sequence
+  int upto = 0, total;    // tiles of the sequences up to and with it
+  bool bad = false;
+  int at = -1, first = 0, tok0 = 0, tokens = 0, row0 = 0, row_count = 0;
+  __device__ LaneList(const Shapes& s_, const SharedList& sh_, const int32_t* cu_seqlens_, const int32_t* cu_qlens_, int lane_)
+      : s(s_), sh(sh_), cu_seqlens(cu_seqlens_), cu_qlens(cu_qlens_), lane(lane_) {}
+  // One warp per block asks for the bounds, the others read them from shared memory (all of them on a few lines of L2 cost a microsecond).
+  __device__ void open(int warp) {
+    if (warp == 0 && lane < s.batch) {
+      const Span q = seq_span(s, cu_seqlens, lane), r = row_span(s, cu_qlens, lane);
+      bad = q.bad || r.bad;
+      sh.bounds[lane] = make_int4(q.first, q.count, r.first, r.count);
+    }
+    __syncthreads();
+    if (lane < s.batch) mine = sh.bounds[lane];
+    upto = sum_upto(lane, tiles_of(mine.y, mine.w));
+    total = __shfl_sync(0xFFFFFFFFu, upto, 31);
+  }
+  __device__ void look_up(int t) {  // the whole warp; t < total
+    if (t == at) return;
+    at = t;
+    const int b = __ffs(__ballot_sync(0xFFFFFFFFu, upto > t)) - 1, end = __shfl_sync(0xFFFFFFFFu, upto, b);
+    tok0 = __shfl_sync(0xFFFFFFFFu, mine.x, b);
+    tokens = __shfl_sync(0xFFFFFFFFu, mine.y, b);
+    row0 = __shfl_sync(0xFFFFFFFFu, mine.z, b);
+    row_count = __shfl_sync(0xFFFFFFFFu, mine.w, b);
+    first = (t - (end - tiles_of(tokens, row_count))) * kRowTileTokens;
+  }
+};
+
+// More.
+struct TableList {
   const Shapes& s;
   const SharedList sh;
   const int32_t *cu_seqlens, *cu_qlens;
@@ -71,18 +119,8 @@ struct TileList {
   // of the tile looked up last, in all lanes
   int first = 0, tok0 = 0, tokens = 0, row0 = 0, row_count = 0;
   int begin = 0, end = 0;   // the tiles of its sequence
-  __device__ TileList(const Shapes& s_, const SharedList& sh_, const int32_t* cu_seqlens_, const int32_t* cu_qlens_, int lane_)
+  __device__ TableList(const Shapes& s_, const SharedList& sh_, const int32_t* cu_seqlens_, const int32_t* cu_qlens_, int lane_)
       : s(s_), sh(sh_), cu_seqlens(cu_seqlens_), cu_qlens(cu_qlens_), lane(lane_) {}
-  // A sequence without scored rows has none: nobody needs its keys (20 x 3,000 tokens, every second one without: 185 us instead of 196).
-  static __device__ int tiles_of(int tokens, int rows) { return rows > 0 ? (tokens + kRowTileTokens - 1) / kRowTileTokens : 0; }
-  __device__ int sum_upto(int v) const {
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const int t = __shfl_up_sync(0xFFFFFFFFu, v, d);
-      if (lane >= d) v += t;
-    }
-    return v;
-  }
   // All threads of the block.  Each bound is asked for by one thread of it (by all its warps: a microsecond on a few lines of L2).
   // (Loops kept as loops: of a large call every line of code comes from memory again.)
   __device__ void open(int warp) {
@@ -101,7 +139,7 @@ struct TileList {
         sh.bounds[e] = make_int4(q.first, q.count, r.first, r.count);
       }
     }
-    int before = sum_upto(sum) - sum;
+    int before = sum_upto(lane, sum) - sum;
     if (lane == 31) sh.warp_sum[warp] = before + sum;
     if (entries > 32) {  // (else all of them are the first warp's)
       __syncthreads();
@@ -139,7 +177,7 @@ struct TileList {
     for (int b0 = e * step; b0 < stop; b0 += 32) {
       const int b = b0 + lane;
       const Span q = b < stop ? seq_span<true>(s, cu_seqlens, b) : Span{0, 0, false}, r = b < stop ? row_span<true>(s, cu_qlens, b) : Span{0, 0, false};
-      const int own = tiles_of(q.count, r.count), with = begin + sum_upto(own);
+      const int own = tiles_of(q.count, r.count), with = begin + sum_upto(lane, own);
       const unsigned behind = __ballot_sync(0xFFFFFFFFu, with > t);
       if (behind) {
         const int from = __ffs(behind) - 1;
@@ -153,7 +191,7 @@ struct TileList {
   }
 };
 
-template <int DIM>
+template <int DIM, typename List>
 __global__ void __launch_bounds__(kThreads, 1)
 score_rows_kernel(const __grid_constant__ CUtensorMap k_map, Shapes s, const uint16_t* __restrict__ q, const int32_t* __restrict__ q_idx,
                   const int32_t* __restrict__ cu_qlens, const int32_t* __restrict__ cu_seqlens, float* __restrict__ logits,
@@ -175,7 +213,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap k_map, Shapes s, const uin
   }
   chain_enter_late(s, cu_seqlens, cu_qlens, q_idx);
   int4* const table = reinterpret_cast<int4*>(smem_raw + (ring - ptx::smem_u32(smem_raw)) + kRingBytes);
-  TileList list(s, SharedList{table, reinterpret_cast<int*>(table + table_entries(s.batch)), warp_sum}, cu_seqlens, cu_qlens, lane);
+  List list(s, SharedList{table, reinterpret_cast<int*>(table + table_entries(s.batch)), warp_sum}, cu_seqlens, cu_qlens, lane);
   list.open(warp);
   const int units = list.total * s.hkv, each = units / (int)gridDim.x, more = units - each * (int)gridDim.x;  // (the host sees to it that they fit)
   const int begin = each * (int)blockIdx.x + min((int)blockIdx.x, more), count = each + ((int)blockIdx.x < more ? 1 : 0);
@@ -330,18 +368,22 @@ long long most_units(const Shapes& s) {
   return tiles * s.hkv;
 }
 
-template <int DIM>
-cudaError_t run(const Shapes& s, const CUtensorMap& k_map, const uint16_t* q, const int32_t* q_idx, const int32_t* cu_qlens, const int32_t* cu_seqlens,
+template <int DIM, typename List>
+cudaError_t run_with(const Shapes& s, const CUtensorMap& k_map, const uint16_t* q, const int32_t* q_idx, const int32_t* cu_qlens, const int32_t* cu_seqlens,
                 float* logits, float2* stats, int stat_tiles, int32_t* device_status, cudaStream_t stream) {
   const int smem = kRingBytes + 1024 + table_bytes(s.batch);
   cudaError_t e = once_per_context([] {
-    return cudaFuncSetAttribute(score_rows_kernel<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes + 1024 + table_bytes(kTable));
+    return cudaFuncSetAttribute(score_rows_kernel<DIM, List>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes + 1024 + table_bytes(kTable));
   });
   if (e != cudaSuccess) return e;
   const long long units = most_units(s);
   count_launches(1);
-  return launch_chained(score_rows_kernel<DIM>, dim3((unsigned)(units < kNumSMs ? units : kNumSMs)), dim3(kThreads), smem, stream, k_map, s, q, q_idx,
+  return launch_chained(score_rows_kernel<DIM, List>, dim3((unsigned)(units < kNumSMs ? units : kNumSMs)), dim3(kThreads), smem, stream, k_map, s, q, q_idx,
                         cu_qlens, cu_seqlens, logits, stats, s.max_qlen, stat_tiles, device_status);
+}
+template <int DIM, typename... Args>
+cudaError_t run(const Shapes& s, Args... args) {
+  return s.batch <= 32 ? run_with<DIM, LaneList>(s, args...) : run_with<DIM, TableList>(s, args...);
 }
 
 }  // namespace
