@@ -60,13 +60,15 @@ constexpr int kBulkStages = 4;          // row slots per warp
 constexpr int kAhead = kBulkStages - 2; // rows loaded ahead of the one being stored
 constexpr int kBulkMaxWarps = 8;
 constexpr int kBulkSmemBudget = 200 * 1024;
-// Shared memory that a block asks for at least: more than half of what an SM has, so that a kernel of few rows has one block per SM and no
-// block of the next call's first kernel comes to lie beside it.  That one's key loads want the L1 that is left where shared memory is split
-// for it alone; beside blocks of 25 to 64 KB it started early on an SM split for those, or not, as it happened.  us with what the rows
-// take / 64 KB / 116 KB: 8 x 120 rows of 6 KB, 70 % kept 22.6 / 18.5 / 18.3, 1 x 1,500 22.0 / 22.0 / 17.5, 16 x 120, half kept 24.6 / 20.8 / 19.7, 10 x 170 of
-// 9 KB 18.0 / 16.3 / 15.6.  (Of 400 shapes one lost: 12 x 90 rows of 12 KB, 30 % kept 16.1 / 16.1 / 16.8.)
-constexpr size_t kBulkLeastSmem = 116 * 1024;
-size_t least_smem(size_t used) { return used > kBulkLeastSmem ? used : kBulkLeastSmem; }
+// Shared memory that a block asks for at least: more than half of what an SM has, so that there is one block per SM and no block of the next
+// call's first kernel comes to lie beside it.  That one's key loads want the L1 that is left where shared memory is split for it alone; beside
+// blocks of 25 to 64 KB it started early on an SM split for those, or not, as it happened.  us with what the rows take / 64 KB /
+// 116 KB: 8 x 120 rows of 6 KB, 70 % kept 22.6 / 18.5 / 18.3, 1 x 1,500 22.0 / 22.0 / 17.5, 16 x 120, half kept 24.6 / 20.8 / 19.7, 10 x 170 of 9 KB 18.0 /
+// 16.3 / 15.6, 8 stages from 520 tokens of 12 KB 103.3 / 94.3 / 92.1.  (Of 400 shapes one lost: 12 x 90 rows of 12 KB, 30 % kept 16.1 / 16.1 / 16.8.)
+// Short lists are gathered so soon that the next call's launch beside them is worth more: 5 stages from 2,000 tokens, rows of 1.5
+// KB, 25 KB used 55.1 / 55.1 / 56.7.
+constexpr size_t kBulkAlone = 116 * 1024;
+size_t list_smem(size_t used) { return used > kBulkAlone ? used : used > 28 * 1024 ? kBulkAlone : 64 * 1024; }
 
 __global__ void __launch_bounds__(kBulkMaxWarps * 32, 1)
 compact_rows_bulk_kernel(Shapes s, RowStreams t, const int32_t* __restrict__ keep_idx, const int32_t* __restrict__ cu_keep,
@@ -311,7 +313,7 @@ cudaError_t launch_compact(const Shapes& s, const int32_t* keep_idx, const int32
     // No deeper rings than a warp has rows.
     const int rows_per_warp = (s.total_keep + blocks * warps - 1) / (blocks * warps);
     const int slots = rows_per_warp < kBulkStages ? rows_per_warp : kBulkStages;
-    const size_t smem = least_smem((size_t)warps * slots * row_bytes);
+    const size_t smem = list_smem((size_t)warps * slots * row_bytes);
     e = launch_chained(compact_rows_bulk_kernel, dim3(blocks), dim3(warps * 32), smem, stream, s, t, keep_idx, cu_keep, cu_seqlens,
                        n_segments, (int)plan.packed_k, (int)plan.packed_v, row_bytes, slots, device_status);
     count_launches(1);
@@ -348,7 +350,7 @@ cudaError_t launch_compact_placed(const Shapes& s, const RowStreams& rows, const
   cudaError_t e = once_per_context([] { return cudaFuncSetAttribute(compact_placed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBulkSmemBudget); });
   if (e != cudaSuccess) return e;
   const int per_block = p.warps * p.slots, blocks = (s.total_tokens + per_block - 1) / per_block;
-  e = launch_chained(compact_placed_kernel, dim3(blocks), dim3(p.warps * 32), least_smem((size_t)p.bytes(plan.row_bytes)), stream, s, rows, place, cu_seqlens,
+  e = launch_chained(compact_placed_kernel, dim3(blocks), dim3(p.warps * 32), p.bytes(plan.row_bytes) > (long long)kBulkAlone ? (size_t)p.bytes(plan.row_bytes) : kBulkAlone, stream, s, rows, place, cu_seqlens,
                      plan.n_segments, (int)plan.packed_k, (int)plan.packed_v, plan.row_bytes, p.slots, device_status);
   count_launches(1);
   return e != cudaSuccess ? e : cudaGetLastError();
